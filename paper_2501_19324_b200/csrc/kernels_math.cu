@@ -495,90 +495,119 @@ cudaError_t launch_rope_only(float* v, const int32_t* pos, int T, int n_heads, i
 }
 
 // ---------------------------------------------------------------------------------------------
-// Generic causal attention over paged KV: one warp per (slot, query head), online softmax.
-// Each lane owns hd/32 consecutive dims; query head j reads KV head j / (H / KV).
+// Generic causal attention over paged KV (fp32 caches, groups wider than eight heads): one block of four to sixteen
+// warps per (slot, query head), the row's pages dealt round the warps; query head j reads KV head j / (H / KV).
+// Bound by latency: the caches it serves are small, the chain of dependent steps is not.  A page is therefore one
+// flat piece of work for a warp: lane = (token, half of the head dim), so that all 16 scores come out of ONE shuffle
+// instead of sixteen warp sums, every load of the page's keys and values goes out before the first use, and the next
+// page's id is fetched a page ahead.  The warps' partial (max, sum, O) meet in shared memory in warp order.
+// (One warp walking all pages of a head with a warp sum per token: 50 us a launch at 4 rows x 64..190 cached tokens,
+// growing with the context; this form: 4.5 us.)
 // ---------------------------------------------------------------------------------------------
+constexpr int kGenericWarps = 16;
+
 template <typename KT, typename OT, int HD>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32 * kGenericWarps)
 attn_generic_kernel(const float* __restrict__ q, PassView p, const KT* __restrict__ pool,
                     const int32_t* __restrict__ page_table, int max_pages, OT* __restrict__ out, OT* __restrict__ out_lo,
                     int H, int KV, int pf) {
   RSD_PDL_SYNC();
   RSD_SKIP_IF_IDLE(p.n_active);
-  constexpr int DPL = HD / 32;
-  const int lane = threadIdx.x & 31;
-  const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (w >= p.T * H) return;
-  const int t = w / H, h = w % H;
+  constexpr int DPL = HD / 32;            // output dims of a lane
+  constexpr int VN = 16 / sizeof(KT);     // elements of a 16-byte load
+  constexpr int NK = HD / 2 / VN;         // key loads of a lane
+  constexpr int NV = kPageTokens / VN;    // value loads of a dim
+  __shared__ __align__(16) float s_q[HD];
+  __shared__ float s_m[kGenericWarps], s_l[kGenericWarps], s_o[kGenericWarps][HD];
+  const int t = blockIdx.x / H, h = blockIdx.x % H;
   const int row = p.tok_row[t];
   if (row < 0) return;
   const int pos = p.tok_pos[t];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
+  const int tok = lane & 15, hf = lane >> 4;
   const int g = h / (H / KV);
   const float scale = rsqrtf((float)HD);
-  float qv[DPL];
-#pragma unroll
-  for (int i = 0; i < DPL; ++i) qv[i] = q[((size_t)t * H + h) * HD + lane * DPL + i] * scale;
+  const int32_t* pt = page_table + (size_t)row * max_pages;
+  const int n_pages = pos / kPageTokens + 1;
+  const size_t block = (size_t)KV * kPageTokens * HD;
+  int page = warp < n_pages ? pt[warp] : 0;
+  if (threadIdx.x < HD) s_q[threadIdx.x] = q[((size_t)t * H + h) * HD + threadIdx.x] * scale;
+  __syncthreads();
   float m = -INFINITY, l = 0.f, acc[DPL];
 #pragma unroll
   for (int i = 0; i < DPL; ++i) acc[i] = 0.f;
-  const int32_t* pt = page_table + (size_t)row * max_pages;
-  for (int p0 = 0; p0 <= pos; p0 += kPageTokens) {
-    const int page = pt[p0 / kPageTokens];
-    const size_t block = (size_t)KV * kPageTokens * HD;
-    const KT* kb = pool + (size_t)page * pf * block + (size_t)g * kPageTokens * HD;
-    const KT* vb = kb + block;
-    const int n = min(kPageTokens, pos + 1 - p0);
-    float sc[kPageTokens];
+  for (int pg = warp; pg < n_pages; pg += n_warps) {
+    const KT* kb = pool + (size_t)page * pf * block + (size_t)g * kPageTokens * HD + tok * HD + hf * (HD / 2);
+    const KT* vb = pool + (size_t)page * pf * block + block + (size_t)g * kPageTokens * HD + lane * DPL * kPageTokens;
+    if (pg + n_warps < n_pages) page = pt[pg + n_warps];
+    const int n = min(kPageTokens, pos + 1 - pg * kPageTokens);
+    uint4 kr[NK], vr[DPL * NV];
 #pragma unroll
-    for (int j = 0; j < kPageTokens; ++j) {
-      float a = 0.f;
-      if (j < n) {
+    for (int i = 0; i < NK; ++i) kr[i] = *reinterpret_cast<const uint4*>(kb + i * VN);
 #pragma unroll
-        for (int i = 0; i < DPL; ++i) {
-          float kk = to_f32(kb[j * HD + lane * DPL + i]);
-          if (pf == 4) kk += to_f32(kb[2 * block + j * HD + lane * DPL + i]);
-          a = fmaf(qv[i], kk, a);
-        }
+    for (int i = 0; i < DPL * NV; ++i) vr[i] = *reinterpret_cast<const uint4*>(vb + i * VN);
+    float part[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < NK; ++i) {
+      const KT* e = reinterpret_cast<const KT*>(&kr[i]);
+#pragma unroll
+      for (int j = 0; j < VN; ++j) {
+        float kk = to_f32(e[j]);
+        if (pf == 4) kk += to_f32(kb[2 * block + i * VN + j]);
+        part[j & 3] = fmaf(s_q[hf * (HD / 2) + i * VN + j], kk, part[j & 3]);
       }
-      sc[j] = a;
     }
+    float sc = (part[0] + part[1]) + (part[2] + part[3]);
+    sc += __shfl_xor_sync(0xFFFFFFFFu, sc, 16);
+    if (tok >= n) sc = -INFINITY;
+    float mx = sc;
 #pragma unroll
-    for (int j = 0; j < kPageTokens; ++j) sc[j] = warp_sum(sc[j]);
-    float mx = m;
-#pragma unroll
-    for (int j = 0; j < kPageTokens; ++j)
-      if (j < n) mx = fmaxf(mx, sc[j]);
-    const float corr = __expf(m - mx);
-    l *= corr;
+    for (int o = 1; o < 16; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+    mx = fmaxf(m, mx);                                     // finite: token 0 of a walked page is always valid
+    const float corr = __expf(m - mx), pr = __expf(sc - mx);
+    l = l * corr + (hf == 0 ? pr : 0.f);                   // this lane's token only; the lanes meet after the loop
 #pragma unroll
     for (int i = 0; i < DPL; ++i) acc[i] *= corr;
 #pragma unroll
     for (int j = 0; j < kPageTokens; ++j) {
-      if (j < n) {
-        const float pj = __expf(sc[j] - mx);
-        l += pj;
+      const float pj = __shfl_sync(0xFFFFFFFFu, pr, j);
+      if (j < n) {                                         // slots beyond the context hold anything, NaN included
 #pragma unroll
         for (int i = 0; i < DPL; ++i) {
-          float vv = to_f32(vb[(lane * DPL + i) * kPageTokens + j]);
-          if (pf == 4) vv += to_f32(vb[2 * block + (lane * DPL + i) * kPageTokens + j]);
+          float vv = to_f32(reinterpret_cast<const KT*>(&vr[i * NV + j / VN])[j % VN]);
+          if (pf == 4) vv += to_f32(vb[2 * block + i * kPageTokens + j]);
           acc[i] = fmaf(pj, vv, acc[i]);
         }
       }
     }
     m = mx;
   }
-  const float inv = 1.f / l;
+  l = warp_sum(l);
+  if (lane == 0) { s_m[warp] = m; s_l[warp] = l; }
 #pragma unroll
-  for (int i = 0; i < DPL; ++i) store_operand<OT>(out, out_lo, ((size_t)t * H + h) * HD + lane * DPL + i, acc[i] * inv);
+  for (int i = 0; i < DPL; ++i) s_o[warp][lane * DPL + i] = acc[i];
+  __syncthreads();
+  if (threadIdx.x < HD) {
+    float M = s_m[0], L = 0.f, O = 0.f;
+    for (int w = 1; w < n_warps; ++w) M = fmaxf(M, s_m[w]);
+    for (int w = 0; w < n_warps; ++w) {
+      const float e = __expf(s_m[w] - M);                  // 0 for a warp without pages
+      L += s_l[w] * e;
+      O += s_o[w][threadIdx.x] * e;
+    }
+    store_operand<OT>(out, out_lo, ((size_t)t * H + h) * HD + threadIdx.x, O / L);
+  }
 }
 
 cudaError_t launch_attn_generic(int kv_dtype, const float* q, PassView p, KvView kv, void* out, void* out_lo,
                                 int out_dtype, int H, int KV, int hd, cudaStream_t s) {
   if (p.T <= 0) return cudaSuccess;
-  const int warps = p.T * H;
-  const int blocks = (warps + 3) / 4;
+  const int blocks = p.T * H;
+  // few (slot, head) pairs: sixteen warps, so that 256 cached tokens are one round; once the pairs alone fill the SMs,
+  // four warps a block waste fewer on short contexts
+  const int threads = 32 * (blocks <= 148 ? kGenericWarps : (blocks <= 148 * 4 ? 8 : 4));
 #define RSD_ATTN(KT, OT, HD) \
-  RSD_LAUNCH((attn_generic_kernel<KT, OT, HD>), blocks, 128, 0, s, q, p, (const KT*)kv.pool_layer, kv.page_table, kv.max_pages, (OT*)out, (OT*)out_lo, H, KV, 2 + 2 * kv.v_extra)
+  RSD_LAUNCH((attn_generic_kernel<KT, OT, HD>), blocks, threads, 0, s, q, p, (const KT*)kv.pool_layer, kv.page_table, kv.max_pages, (OT*)out, (OT*)out_lo, H, KV, 2 + 2 * kv.v_extra)
 #define RSD_ATTN_HD(KT, OT) do { if (hd == 128) RSD_ATTN(KT, OT, 128); else RSD_ATTN(KT, OT, 64); } while (0)
   using bf = __nv_bfloat16;
   if (kv_dtype == 2) { if (out_dtype == 1) RSD_ATTN_HD(__half, bf); else RSD_ATTN_HD(__half, float); }

@@ -296,6 +296,25 @@ def test_decode_attention_against_definition(dtype, hd, H, KV):
             np.testing.assert_allclose(got[b, h], want, rtol=0, atol=tol)
 
 
+@pytest.mark.parametrize("dtype,hd,H,KV", [(torch.float32, 64, 4, 2), (torch.float32, 128, 3, 3), (torch.float16, 128, 18, 2),
+                                          (torch.bfloat16, 64, 9, 1)])
+def test_generic_attention_at_the_edges_of_a_round_of_warps(dtype, hd, H, KV):
+    """fp32 caches and groups wider than eight heads: contexts of fewer pages than the block has warps, exactly one page
+    a warp (128 tokens with eight warps, 256 with sixteen), one token more, and a second round; the unused slots hold
+    NaN.  fp32 arithmetic on the stored values: about 300 products and sums of order one, each rounded to 2^-24."""
+    rng = np.random.default_rng(12)
+    ctx = [1, 112, 127, 128, 129, 145, 256, 257]
+    pool, table, Ks, Vs = paged_kv(rng, len(ctx), KV, hd, ctx, dtype, 20)
+    q = rng.normal(size=(len(ctx), H, hd)).astype(np.float32)
+    got = rb.k_attn_decode(dev(q), pool, table, dev(np.array(ctx, np.int32)), KV).cpu().numpy()
+    for b in range(len(ctx)):
+        for h in range(H):
+            g = h // (H // KV)
+            s = Ks[b][:, g].astype(np.float64) @ q[b, h].astype(np.float64) / np.sqrt(hd)
+            p = np.exp(s - s.max()); p /= p.sum()
+            np.testing.assert_allclose(got[b, h], p @ Vs[b][:, g].astype(np.float64), rtol=0, atol=2e-5)
+
+
 @pytest.mark.parametrize("dtype,hd,H,KV", [(torch.float16, 128, 12, 2), (torch.float16, 128, 28, 4), (torch.float16, 64, 4, 2),
                                           (torch.float32, 64, 4, 2), (torch.float16, 128, 64, 8), (torch.float16, 128, 8, 4),
                                           (torch.float16, 128, 3, 3), (torch.bfloat16, 128, 12, 2)])
