@@ -371,9 +371,12 @@ cudaError_t launch_attn_decode(int kv_dtype, const float* q, const void* pool_la
   int32_t* pos = row + B;
   if (kv_dtype == 0 || G > 8) {
     // fp32 caches and wide groups take the generic kernel
-    RSD_LAUNCH((decode_slots_kernel), (B + 255) / 256, 256, 0, s, slot_row, len_or_pos, len_offset, row, pos, B);
-    launched(1);
-    PassView p{nullptr, row, pos, B, n_active};
+    PassView p{nullptr, slot_row, len_or_pos, B, n_active};
+    if (!slot_row || len_offset != 1) {        // else the slots are a pass's rows and positions already
+      RSD_LAUNCH((decode_slots_kernel), (B + 255) / 256, 256, 0, s, slot_row, len_or_pos, len_offset, row, pos, B);
+      launched(1);
+      p = PassView{nullptr, row, pos, B, nullptr};   // written a kernel ago: nothing to read ahead of the wait
+    }
     KvView kv{const_cast<void*>(pool_layer), page_table, max_pages, kv_dtype == 3 ? 1 : 0};
     return launch_attn_generic(kv_dtype == 3 ? 2 : kv_dtype, q, p, kv, out, out_lo, out_dtype, H, KV, hd, s);
   }

@@ -716,8 +716,7 @@ template <bool EXT>
 __global__ void __launch_bounds__(kThreads, 1)
 decode_mega_kernel(const MegaParams* __restrict__ Pp, const MegaLayer* __restrict__ layers, PassView pv,
                    const __nv_bfloat16* __restrict__ final_gain) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  RSD_PDL_SYNC_LATE();   // it stands in for the embedding kernel: its dependents read the pass lists ahead of their wait
   const MegaParams& P = *Pp;
   if (*pv.n_active == 0 || __ldcg(P.err) != 0) return;     // uniform over the grid
 

@@ -14,7 +14,7 @@ namespace rsd {
 // ---------------------------------------------------------------------------------------------
 template <typename WT>
 __global__ void embed_kernel(const WT* __restrict__ E, PassView p, float* __restrict__ x, int d) {
-  RSD_PDL_SYNC();
+  RSD_PDL_SYNC_LATE();
   RSD_SKIP_IF_IDLE(p.n_active);
   const int t = blockIdx.x;
   if (p.tok_row[t] < 0) return;
@@ -40,11 +40,9 @@ cudaError_t launch_embed(int dtype, const void* embed, PassView p, float* x, int
 // RMSNorm: out = x * gain / sqrt(mean(x^2) + eps), one block per token, x kept in registers
 // ---------------------------------------------------------------------------------------------
 template <typename OT, typename GT>
-__global__ void rmsnorm_kernel(float* __restrict__ x, const GT* __restrict__ gain, OT* __restrict__ out,
-                               OT* __restrict__ out_lo, int d, float eps, const int32_t* __restrict__ src,
-                               const int32_t* n_active, const float* __restrict__ partials, int splits, int T) {
-  RSD_PDL_SYNC();
-  RSD_SKIP_IF_IDLE(n_active);
+__global__ void rmsnorm_kernel(float* x, const GT* __restrict__ gain, OT* out, OT* out_lo, int d, float eps,
+                               const int32_t* src, const int32_t* n_active, const float* partials, int splits, int T) {
+  RSD_PDL_SYNC_UNLESS_IDLE(n_active);
   __shared__ float red[33];
   const int t = blockIdx.x;
   int st = t;
@@ -62,12 +60,12 @@ __global__ void rmsnorm_kernel(float* __restrict__ x, const GT* __restrict__ gai
       for (; sidx + 8 <= splits; sidx += 8) {
         float4 a[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) a[u] = __ldcg(reinterpret_cast<const float4*>(partials + ((size_t)(sidx + u) * T + st) * d + i));
+        for (int u = 0; u < 8; ++u) a[u] = ld_cg(reinterpret_cast<const float4*>(partials + ((size_t)(sidx + u) * T + st) * d + i));
 #pragma unroll
         for (int u = 0; u < 8; ++u) { v.x += a[u].x; v.y += a[u].y; v.z += a[u].z; v.w += a[u].w; }
       }
       for (; sidx < splits; ++sidx) {
-        const float4 a = __ldcg(reinterpret_cast<const float4*>(partials + ((size_t)sidx * T + st) * d + i));
+        const float4 a = ld_cg(reinterpret_cast<const float4*>(partials + ((size_t)sidx * T + st) * d + i));
         v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
       }
       *reinterpret_cast<float4*>(xr + i) = v;
@@ -185,13 +183,17 @@ cudaError_t launch_reduce_norm(const float* partials, int splits, float* x, cons
 // A block of 8 warps covers nb = 8/ks output columns; the ks warps of one column each stream a
 // strided share of the row with 16-byte loads and their partial sums meet in shared memory, in a
 // fixed order (deterministic).  Rows of x are taken MT at a time.
+// Bound by latency at the sizes it serves (the fp32 test models: 0.3-5 MB of weights a launch, resident in L2): in a
+// decode pass the first kGemvAhead weight vectors of a lane, and nearly always all of them, are requested before the
+// wait for the preceding kernels, and the old y before the products.
 // ---------------------------------------------------------------------------------------------
+constexpr int kGemvAhead = 4;
+
 template <typename WT, int MT>
 __global__ void __launch_bounds__(256)
-gemv_splitk_kernel(const WT* __restrict__ W, const WT* __restrict__ X, const WT* __restrict__ X_lo, float* __restrict__ Y,
-                   int M, int N, int K, int ks, int accumulate, const int32_t* n_active) {
-  RSD_PDL_SYNC();
-  RSD_SKIP_IF_IDLE(n_active);
+gemv_splitk_kernel(const WT* __restrict__ W, const WT* X, const WT* X_lo, float* Y, int M, int N, int K, int ks, int accumulate,
+                   const int32_t* n_active) {
+  RSD_PDL_TRIGGER();
   constexpr int VN = Vec16<WT>::N;
   __shared__ float part[8][MT];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -199,31 +201,48 @@ gemv_splitk_kernel(const WT* __restrict__ W, const WT* __restrict__ X, const WT*
   const int col = warp / ks, split = warp % ks;
   const int n = blockIdx.x * nb + col;
   const int m0 = blockIdx.y * MT;
+  const int nvec = n < N ? K / VN : 0, v0 = split * 32 + lane, step = ks * 32;
+  const WT* wrow = W + (size_t)n * K;
+  Vec16<WT> ahead[kGemvAhead];
+  if (n_active == nullptr) RSD_PDL_WAIT();   // outside a decode pass W may be an earlier kernel's output
+  const bool idle = n_active != nullptr && ld_cg(n_active) == 0;
+#pragma unroll
+  for (int i = 0; i < kGemvAhead; ++i)
+    if (v0 + i * step < nvec) ahead[i].load_stream(wrow + (size_t)(v0 + i * step) * VN);
+  RSD_PDL_WAIT();
+  if (idle) return;
+  // one thread per (column, m) finishes the sum and owns that element of y
+  const int oc = threadIdx.x / MT, om = threadIdx.x % MT, on = blockIdx.x * nb + oc;
+  const bool owner = threadIdx.x < nb * MT && on < N && m0 + om < M;
+  float* y = Y + (size_t)(m0 + om) * N + on;
+  const float old = owner && accumulate ? *y : 0.f;
   float acc[MT];
 #pragma unroll
   for (int m = 0; m < MT; ++m) acc[m] = 0.f;
-  if (n < N) {
-    const WT* wrow = W + (size_t)n * K;
-    const int nvec = K / VN;
-    for (int v = split * 32 + lane; v < nvec; v += ks * 32) {
-      Vec16<WT> w;
-      w.load_stream(wrow + (size_t)v * VN);
+  auto fold = [&](const Vec16<WT>& w, int v) {
 #pragma unroll
-      for (int m = 0; m < MT; ++m) {
-        if (m0 + m < M) {
-          Vec16<WT> xv;
-          xv.load(X + (size_t)(m0 + m) * K + (size_t)v * VN);
-          if (X_lo != nullptr) {
-            Vec16<WT> xl;
-            xl.load(X_lo + (size_t)(m0 + m) * K + (size_t)v * VN);
+    for (int m = 0; m < MT; ++m) {
+      if (m0 + m < M) {
+        Vec16<WT> xv;
+        xv.load(X + (size_t)(m0 + m) * K + (size_t)v * VN);
+        if (X_lo != nullptr) {
+          Vec16<WT> xl;
+          xl.load(X_lo + (size_t)(m0 + m) * K + (size_t)v * VN);
 #pragma unroll
-            for (int j = 0; j < VN; ++j) xv.v[j] += xl.v[j];
-          }
-#pragma unroll
-          for (int j = 0; j < VN; ++j) acc[m] = fmaf(w.v[j], xv.v[j], acc[m]);
+          for (int j = 0; j < VN; ++j) xv.v[j] += xl.v[j];
         }
+#pragma unroll
+        for (int j = 0; j < VN; ++j) acc[m] = fmaf(w.v[j], xv.v[j], acc[m]);
       }
     }
+  };
+#pragma unroll
+  for (int i = 0; i < kGemvAhead; ++i)
+    if (v0 + i * step < nvec) fold(ahead[i], v0 + i * step);
+  for (int v = v0 + kGemvAhead * step; v < nvec; v += step) {
+    Vec16<WT> w;
+    w.load_stream(wrow + (size_t)v * VN);
+    fold(w, v);
   }
 #pragma unroll
   for (int m = 0; m < MT; ++m) acc[m] = warp_sum(acc[m]);
@@ -232,32 +251,26 @@ gemv_splitk_kernel(const WT* __restrict__ W, const WT* __restrict__ X, const WT*
     for (int m = 0; m < MT; ++m) part[warp][m] = acc[m];
   }
   __syncthreads();
-  // one thread per (column, m): add the ks partial sums in split order
-  const int idx = threadIdx.x;
-  if (idx < nb * MT) {
-    const int c = idx / MT, m = idx % MT;
-    const int nn = blockIdx.x * nb + c;
-    if (nn < N && m0 + m < M) {
-      float sum = 0.f;
-      for (int sidx = 0; sidx < ks; ++sidx) sum += part[c * ks + sidx][m];
-      float* y = Y + (size_t)(m0 + m) * N + nn;
-      *y = accumulate ? (*y + sum) : sum;
-    }
+  if (owner) {
+    float sum = 0.f;
+    for (int sidx = 0; sidx < ks; ++sidx) sum += part[oc * ks + sidx][om];
+    *y = old + sum;
   }
 }
 
 cudaError_t launch_gemm_simt(int dtype, const void* W, const void* x, const void* x_lo, float* y, int M, int N, int K,
                              int accumulate, const int32_t* n_active, cudaStream_t s) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  // pick the split so that the grid covers the 148 SMs a few times over
+  // pick the split so that the grid covers the 148 SMs a few times over, as long as every lane has a vector
   int ks = 1;
-  while (ks < 8 && (long)N * ks / 8 < 148L * 4 && K / (ks * 2) >= 256) ks *= 2;
-  constexpr int MT = 8;
-  dim3 grid((N + (8 / ks) - 1) / (8 / ks), (M + MT - 1) / MT);
-  if (dtype == 1)
-    RSD_LAUNCH((gemv_splitk_kernel<__nv_bfloat16, MT>), grid, 256, 0, s, (const __nv_bfloat16*)W, (const __nv_bfloat16*)x, (const __nv_bfloat16*)x_lo, y, M, N, K, ks, accumulate, n_active);
-  else
-    RSD_LAUNCH((gemv_splitk_kernel<float, MT>), grid, 256, 0, s, (const float*)W, (const float*)x, nullptr, y, M, N, K, ks, accumulate, n_active);
+  const int per_warp = 32 * (dtype == 1 ? Vec16<__nv_bfloat16>::N : Vec16<float>::N);
+  while (ks < 8 && (long)N * ks / 8 < 148L * 4 && K / (ks * 2) >= per_warp) ks *= 2;
+  const int mt = M <= 4 ? 4 : 8;
+  dim3 grid((N + (8 / ks) - 1) / (8 / ks), (M + mt - 1) / mt);
+#define RSD_GEMV(WT, MT) RSD_LAUNCH((gemv_splitk_kernel<WT, MT>), grid, 256, 0, s, (const WT*)W, (const WT*)x, (const WT*)x_lo, y, M, N, K, ks, accumulate, n_active)
+  if (dtype == 1) { if (mt == 4) RSD_GEMV(__nv_bfloat16, 4); else RSD_GEMV(__nv_bfloat16, 8); }
+  else { x_lo = nullptr; if (mt == 4) RSD_GEMV(float, 4); else RSD_GEMV(float, 8); }
+#undef RSD_GEMV
   return launched(1);
 }
 
@@ -286,7 +299,7 @@ cudaError_t launch_rope_table(float2* table, int n_pos, int hd, float theta, cud
 // RoPE on q and k, KV page write.  One block per token slot; threads walk the (head, pair) grid.
 // Pair (i, i + hd/2) of a head turns by the angle of (position, i).
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ float split_sum(const float* __restrict__ direct, const float* __restrict__ partials, int splits,
+__device__ __forceinline__ float split_sum(const float* direct, const float* partials, int splits,
                                            size_t idx, size_t stride) {
   if (splits <= 1) return direct[idx];
   // loads go out twelve at a time (tail predicated) so their latencies overlap; the sums stay in split order
@@ -294,30 +307,35 @@ __device__ __forceinline__ float split_sum(const float* __restrict__ direct, con
   for (int s0 = 0; s0 < splits; s0 += 12) {
     float t[12];
 #pragma unroll
-    for (int u = 0; u < 12; ++u) t[u] = s0 + u < splits ? __ldcg(partials + (size_t)(s0 + u) * stride + idx) : 0.f;
+    for (int u = 0; u < 12; ++u) t[u] = s0 + u < splits ? ld_cg(partials + (size_t)(s0 + u) * stride + idx) : 0.f;
 #pragma unroll
     for (int u = 0; u < 12; ++u) v += t[u];
   }
   return v;
 }
 
+// The rotation, its roundings spelled out: every kernel that rotates gives the same bits, whatever the compiler would fuse.
+__device__ __forceinline__ float rotate_lo(float a, float b, float2 cs) { return fmaf(a, cs.x, -__fmul_rn(b, cs.y)); }
+__device__ __forceinline__ float rotate_hi(float a, float b, float2 cs) { return fmaf(b, cs.x, __fmul_rn(a, cs.y)); }
+
 template <typename KT>
-__global__ void rope_kv_kernel(const float* __restrict__ qkv, const float* __restrict__ partials, int splits,
-                               PassView p, float* __restrict__ q_out, KT* pool,
-                               const int32_t* __restrict__ page_table, int max_pages,
+__global__ void rope_kv_kernel(const float* qkv, const float* partials, int splits, PassView p, float* q_out, KT* pool,
+                               const int32_t* page_table, int max_pages,
                                const float2* __restrict__ rope, int H, int KV, int hd, int pf) {
-  RSD_PDL_SYNC();
-  RSD_SKIP_IF_IDLE(p.n_active);
+  RSD_PDL_TRIGGER();
+  if (p.n_active == nullptr) RSD_PDL_WAIT();   // a decode pass's lists may be read ahead of the wait, others not
   const int t = blockIdx.x;
-  const int row = p.tok_row[t];
-  if (row < 0) return;
-  const int pos = p.tok_pos[t];
+  const bool idle = p.n_active != nullptr && ld_cg(p.n_active) == 0;
+  const int row = ld_cg(p.tok_row + t), pos = ld_cg(p.tok_pos + t);
+  if (idle || row < 0) { RSD_PDL_WAIT(); return; }
   const int half = hd / 2;
   const int width = (H + 2 * KV) * hd;
   const size_t src0 = (size_t)t * width;                 // offset of this token's row in qkv / a partial
   const size_t sstride = (size_t)gridDim.x * width;      // one partial array = [T][width]
   const float2* cs = rope + (size_t)pos * half;
-  const int page = page_table[(size_t)row * max_pages + pos / kPageTokens];
+  const int page = ld_cg(page_table + (size_t)row * max_pages + pos / kPageTokens);
+  const float2 first = cs[min((int)threadIdx.x, half - 1)];   // this thread's first angle
+  RSD_PDL_WAIT();
   const int slot = pos % kPageTokens;
   // page = K block [KV][16][hd] followed by V block [KV][hd][16] (V transposed within the page)
   // (pf = 4: two more blocks hold the low halves of the keys and of the values)
@@ -330,8 +348,8 @@ __global__ void rope_kv_kernel(const float* __restrict__ qkv, const float* __res
     for (int i = threadIdx.x; i < half; i += blockDim.x) {
       const float a = split_sum(qkv, partials, splits, src0 + head * hd + i, sstride);
       const float b = split_sum(qkv, partials, splits, src0 + head * hd + i + half, sstride);
-      const float2 c = cs[i];
-      const float ra = a * c.x - b * c.y, rb = b * c.x + a * c.y;
+      const float2 c = i == (int)threadIdx.x ? first : cs[i];
+      const float ra = rotate_lo(a, b, c), rb = rotate_hi(a, b, c);
       if (head < H) {
         q_out[(size_t)t * H * hd + head * hd + i] = ra;
         q_out[(size_t)t * H * hd + head * hd + i + half] = rb;
@@ -403,7 +421,7 @@ rope_kv_long_kernel(const float* __restrict__ qkv, PassView p, float* __restrict
     const int t = t0 + tk, pos = s_pos[tk];
     const float a = qkv[(size_t)t * width + head * hd + i], b = qkv[(size_t)t * width + head * hd + i + half];
     const float2 c = rope[(size_t)pos * half + i];
-    const float ra = a * c.x - b * c.y, rb = b * c.x + a * c.y;
+    const float ra = rotate_lo(a, b, c), rb = rotate_hi(a, b, c);
     if (head < H) {
       q_out[(size_t)t * H * hd + head * hd + i] = ra;
       q_out[(size_t)t * H * hd + head * hd + i + half] = rb;
@@ -508,11 +526,9 @@ constexpr int kGenericWarps = 16;
 
 template <typename KT, typename OT, int HD>
 __global__ void __launch_bounds__(32 * kGenericWarps)
-attn_generic_kernel(const float* __restrict__ q, PassView p, const KT* __restrict__ pool,
-                    const int32_t* __restrict__ page_table, int max_pages, OT* __restrict__ out, OT* __restrict__ out_lo,
+attn_generic_kernel(const float* q, PassView p, const KT* pool, const int32_t* page_table, int max_pages, OT* out, OT* out_lo,
                     int H, int KV, int pf) {
-  RSD_PDL_SYNC();
-  RSD_SKIP_IF_IDLE(p.n_active);
+  RSD_PDL_TRIGGER();
   constexpr int DPL = HD / 32;            // output dims of a lane
   constexpr int VN = 16 / sizeof(KT);     // elements of a 16-byte load
   constexpr int NK = HD / 2 / VN;         // key loads of a lane
@@ -520,9 +536,10 @@ attn_generic_kernel(const float* __restrict__ q, PassView p, const KT* __restric
   __shared__ __align__(16) float s_q[HD];
   __shared__ float s_m[kGenericWarps], s_l[kGenericWarps], s_o[kGenericWarps][HD];
   const int t = blockIdx.x / H, h = blockIdx.x % H;
-  const int row = p.tok_row[t];
-  if (row < 0) return;
-  const int pos = p.tok_pos[t];
+  if (p.n_active == nullptr) RSD_PDL_WAIT();   // a decode pass's lists may be read ahead of the wait, others not
+  const bool idle = p.n_active != nullptr && ld_cg(p.n_active) == 0;
+  const int row = ld_cg(p.tok_row + t), pos = ld_cg(p.tok_pos + t);
+  if (idle || row < 0) { RSD_PDL_WAIT(); return; }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
   const int tok = lane & 15, hf = lane >> 4;
   const int g = h / (H / KV);
@@ -530,7 +547,8 @@ attn_generic_kernel(const float* __restrict__ q, PassView p, const KT* __restric
   const int32_t* pt = page_table + (size_t)row * max_pages;
   const int n_pages = pos / kPageTokens + 1;
   const size_t block = (size_t)KV * kPageTokens * HD;
-  int page = warp < n_pages ? pt[warp] : 0;
+  int page = warp < n_pages ? ld_cg(pt + warp) : 0;
+  RSD_PDL_WAIT();
   if (threadIdx.x < HD) s_q[threadIdx.x] = q[((size_t)t * H + h) * HD + threadIdx.x] * scale;
   __syncthreads();
   float m = -INFINITY, l = 0.f, acc[DPL];
@@ -539,7 +557,7 @@ attn_generic_kernel(const float* __restrict__ q, PassView p, const KT* __restric
   for (int pg = warp; pg < n_pages; pg += n_warps) {
     const KT* kb = pool + (size_t)page * pf * block + (size_t)g * kPageTokens * HD + tok * HD + hf * (HD / 2);
     const KT* vb = pool + (size_t)page * pf * block + block + (size_t)g * kPageTokens * HD + lane * DPL * kPageTokens;
-    if (pg + n_warps < n_pages) page = pt[pg + n_warps];
+    if (pg + n_warps < n_pages) page = ld_cg(pt + pg + n_warps);
     const int n = min(kPageTokens, pos + 1 - pg * kPageTokens);
     uint4 kr[NK], vr[DPL * NV];
 #pragma unroll
@@ -622,10 +640,8 @@ cudaError_t launch_attn_generic(int kv_dtype, const float* q, PassView p, KvView
 // SwiGLU: out[t, f] = silu(gu[t, f]) * gu[t, F + f]
 // ---------------------------------------------------------------------------------------------
 template <typename OT>
-__global__ void swiglu_kernel(const float* __restrict__ gu, const float* __restrict__ partials, int splits,
-                              OT* __restrict__ out, OT* __restrict__ out_lo, int T, int F, const int32_t* n_active) {
-  RSD_PDL_SYNC();
-  RSD_SKIP_IF_IDLE(n_active);
+__global__ void swiglu_kernel(const float* gu, const float* partials, int splits, OT* out, OT* out_lo, int T, int F, const int32_t* n_active) {
+  RSD_PDL_SYNC_UNLESS_IDLE(n_active);
   const size_t n = (size_t)T * F;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const size_t t = i / F, f = i % F;
@@ -666,8 +682,7 @@ __device__ __forceinline__ unsigned long long pack_best(float sc, int id) {
 // Grid (slots, chunks): every block scans one chunk of the vocabulary and folds its best candidate
 // into best[slot] with an atomic maximum (order-independent, hence deterministic).
 __global__ void __launch_bounds__(1024) sample_kernel(SampleArgs a) {
-  RSD_PDL_SYNC();
-  RSD_SKIP_IF_IDLE(a.n_active);
+  RSD_PDL_SYNC_UNLESS_IDLE(a.n_active);
   __shared__ float s_sc[32];
   __shared__ int s_ix[32];
   const int slot = blockIdx.x;
