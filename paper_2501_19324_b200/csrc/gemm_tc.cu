@@ -7,10 +7,11 @@
 // MT = 16..64 the same kernel is a bandwidth-bound skinny GEMM for decode (weights read once, MMA
 // cost hidden); with MT = 256 it is the dense GEMM of prefill / PRM scoring / catch-up.
 //
-// Roles inside a CTA of 6 warps: warps 0-3 read the accumulator out of TMEM (lane = output feature,
-// column = x row) and write y, warp 4 issues TMA loads through a ring of shared-memory stages,
-// warp 5 allocates TMEM and issues the MMAs.  Small problems are split along K across CTAs; the
-// partial tiles go to scratch and the last CTA to arrive adds them in split order (deterministic).
+// Roles inside a CTA of 7 warps: warps 0-3 read the accumulator out of TMEM (lane = output feature,
+// column = x row) and write y, warp 4 issues the TMA loads of the weights and warp 6 those of x through a ring
+// of shared-memory stages, warp 5 allocates TMEM and issues the MMAs.  Small problems are split along K across
+// CTAs; the partial tiles go to scratch and are added in split order by the consumer or a reduction kernel
+// (deterministic).
 // Every wait on an mbarrier is bounded; on expiry the CTA raises an error flag and leaves cleanly.
 #include <cuda.h>
 
@@ -42,6 +43,7 @@ constexpr int kUmmaK = 16;
 constexpr int kCounterBytes = 4096;
 constexpr int kMaxSplitTiles = kCounterBytes / 4;
 constexpr int kMaxSplitCtas = 640;
+constexpr int kTcThreads = 224;    // four epilogue warps, weight producer, MMA issuer, x producer
 
 // DEEP: a ring of eight (six for 128-row x tiles) stages for one CTA per SM, for grids that do not reach two CTAs per SM anyway (a lone
 // CTA needs about twice the bytes in flight to keep its share of the HBM stream going).
@@ -76,17 +78,19 @@ template <int MT, bool DEEP = false> struct TcCfg {
 // failure path -- error flag raised, epilogue warps released, tensor memory freed, clean return -- with nothing in
 // flight.  This is how the failure path is exercised without a fault or an endless wait.
 template <int MT, bool SPLIT, bool GU = false, bool DEEP = false, bool PROBE = false>
-__global__ void __launch_bounds__(192, TcCfg<MT, DEEP>::kCtasPerSm)
+__global__ void __launch_bounds__(kTcThreads, TcCfg<MT, DEEP>::kCtasPerSm)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
-               const __grid_constant__ CUtensorMap tm_x_lo, float* __restrict__ Y,
-               int M, int N, int K, int accumulate, int splits, int kb_per_split, float* __restrict__ partials,
-               int* __restrict__ err, const int32_t* __restrict__ n_active, RowScale rs,
-               __nv_bfloat16* __restrict__ act_hi = nullptr, __nv_bfloat16* __restrict__ act_lo = nullptr) {
+               const __grid_constant__ CUtensorMap tm_x_lo, float* Y,
+               int M, int N, int K, int accumulate, int splits, int kb_per_split, float* partials,
+               int* err, const int32_t* n_active, RowScale rs,
+               __nv_bfloat16* act_hi = nullptr, __nv_bfloat16* act_lo = nullptr) {
   // Programmatic dependent launch: the next kernel may be scheduled at once; this kernel sets itself
   // up and starts streaming its WEIGHT tiles (never written by any kernel) while its predecessors are
-  // still running, and only then waits for them (griddepcontrol.wait) before it touches activations,
-  // outputs or the idle flag.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // still running, and only then waits for them (griddepcontrol.wait) before it touches activations
+  // or outputs.  The idle flag is a constant of the decode pass (see RSD_PDL_SYNC_LATE): requested here, looked at
+  // after the first weight copies went out.  0: every row of the phase has finished.
+  RSD_PDL_TRIGGER();
+  const int active = n_active != nullptr ? ld_cg(n_active) : 1;
   using Cfg = TcCfg<MT, DEEP>;
   constexpr int kRows = SPLIT ? MT / 2 : MT;   // distinct x rows per tile
   extern __shared__ uint8_t smem_raw[];
@@ -119,11 +123,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
   const int kb1 = min(total_kb, kb0 + kb_per_split);
   const int n_kb = kb1 - kb0;   // >= 1 by construction of the grid
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < Cfg::kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+  if (threadIdx.x == 128) {                    // the weight producer's first lane
+    for (int s = 0; s < Cfg::kStages; ++s) { mbar_init(&full[s], 2); mbar_init(&empty[s], 1); }
     mbar_init(tmem_full, 1);
     flags[0] = 0; flags[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  } else if (threadIdx.x == 192) {             // the x producer's: its tensor maps are on their way under the wait
+    tma_prefetch_map(&tm_x);
+    if (SPLIT) tma_prefetch_map(&tm_x_lo);
   }
   if (warp == 5) tmem_alloc(tmem_slot, Cfg::kTmemCols);
   tc_fence_before();
@@ -131,65 +138,59 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  if (warp == 4) {
-    // ---------------- TMA producer ----------------
+  if (warp == 4 || warp == 6) {
+    // ---------------- TMA producers: warp 4 the weight tiles, warp 6 the x tiles ----------------
+    // Two threads, since one pays 100+ cycles for every box it issues: the weight stream runs ahead under the wait for
+    // the predecessors as far as the ring reaches, the x tiles follow after it.
     if (lane == 0 && !PROBE) {
+      const int pre = min(n_kb, Cfg::kStages);
+      int n_issue = n_kb;
+      if (warp == 4) {
+        if (active == 0) n_issue = pre;
+      } else {
+        RSD_PDL_WAIT();
+        if (active == 0) {                     // close the stages of the weight copies that went out
+          n_issue = 0;
+          for (int i = 0; i < pre; ++i) mbar_arrive(&full[i]);
+        }
+      }
       int issued = 0;
       bool ok = true;
-      // weight tiles of the first ring of stages go out before the predecessors have finished
-      const int pre = min(n_kb, Cfg::kStages);
-      for (int i = 0; i < pre; ++i) {
-        mbar_expect_tx(&full[i], Cfg::kStageBytes);
-        uint8_t* a = smem + (size_t)i * Cfg::kStageBytes;
-        if (GU) {
-          tma_load_2d(a, &tm_w, &full[i], (kb0 + i) * kTileK, n0);
-          tma_load_2d(a + Cfg::kABytes / 2, &tm_w, &full[i], (kb0 + i) * kTileK, N + n0);
-        } else {
-          tma_load_2d(a, &tm_w, &full[i], (kb0 + i) * kTileK, n0);
-        }
-      }
-      issued = pre;
-      asm volatile("griddepcontrol.wait;" ::: "memory");
-      // every row of the decode phase has finished: complete the copies that are in flight (their
-      // x halves are fetched too so that the stage barriers close), then leave without computing
-      const bool idle = n_active != nullptr && *n_active == 0;
-      if (idle) flags[0] = 2;
-      for (int i = 0; i < pre; ++i) {
-        uint8_t* a = smem + (size_t)i * Cfg::kStageBytes;
-        tma_load_2d(a + Cfg::kABytes, &tm_x, &full[i], (kb0 + i) * kTileK, m0);
-        if (SPLIT) tma_load_2d(a + Cfg::kABytes + kRows * kTileK * 2, &tm_x_lo, &full[i], (kb0 + i) * kTileK, m0);
-      }
-      if (idle) {
-        for (int i = 0; i < pre; ++i) mbar_wait(&full[i], 0);
-      } else {
-        for (int i = pre; i < n_kb && ok; ++i) {
-          const int s = i % Cfg::kStages;
+      for (int i = 0; i < n_issue; ++i) {
+        const int s = i % Cfg::kStages;
+        if (i >= Cfg::kStages) {
           ok = mbar_wait(&empty[s], ((i / Cfg::kStages) - 1) & 1);
           if (!ok || flags[0]) { ok = false; break; }
-          uint8_t* a = smem + (size_t)s * Cfg::kStageBytes;
-          mbar_expect_tx(&full[s], Cfg::kStageBytes);
-          if (GU) {
-            tma_load_2d(a, &tm_w, &full[s], (kb0 + i) * kTileK, n0);
-            tma_load_2d(a + Cfg::kABytes / 2, &tm_w, &full[s], (kb0 + i) * kTileK, N + n0);
-          } else {
-            tma_load_2d(a, &tm_w, &full[s], (kb0 + i) * kTileK, n0);
-          }
+        }
+        uint8_t* a = smem + (size_t)s * Cfg::kStageBytes;
+        if (warp == 4) {
+          mbar_expect_tx(&full[s], Cfg::kABytes);
+          tma_load_2d(a, &tm_w, &full[s], (kb0 + i) * kTileK, n0);
+          if (GU) tma_load_2d(a + Cfg::kABytes / 2, &tm_w, &full[s], (kb0 + i) * kTileK, N + n0);
+        } else {
+          mbar_expect_tx(&full[s], Cfg::kBBytes);
           tma_load_2d(a + Cfg::kABytes, &tm_x, &full[s], (kb0 + i) * kTileK, m0);
           if (SPLIT) tma_load_2d(a + Cfg::kABytes + kRows * kTileK * 2, &tm_x_lo, &full[s], (kb0 + i) * kTileK, m0);
-          issued = i + 1;
         }
-        if (!ok) {
-          if (err && flags[0] != 2) atomicCAS(err, 0, -5);
-          if (flags[0] == 0) flags[0] = 1;
-          // let the copies already in flight land before the CTA goes away
-          for (int i = max(0, issued - Cfg::kStages); i < issued; ++i)
-            mbar_wait(&full[i % Cfg::kStages], (i / Cfg::kStages) & 1);
+        issued = i + 1;
+      }
+      if (active == 0) {
+        for (int i = 0; i < issued; ++i) mbar_wait(&full[i], 0);
+      }
+      if (!ok) {
+        if (flags[0] == 0) {
+          if (err) atomicCAS(err, 0, -5);
+          flags[0] = 1;
         }
+        // let the copies already in flight land before the CTA goes away (a stage that only one producer has reached
+        // does not complete: the polls run out, long after the copy)
+        for (int i = max(0, issued - Cfg::kStages); i < issued; ++i)
+          mbar_wait(&full[i % Cfg::kStages], (i / Cfg::kStages) & 1, 1u << 16);
       }
     }
   } else if (warp == 5) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    if (lane == 0 && active != 0) {
       bool ok = true;
       for (int i = 0; i < n_kb; ++i) {
         const int s = i % Cfg::kStages;
@@ -214,25 +215,31 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
     }
   } else {
     // ---------------- epilogue: TMEM -> registers -> global ----------------
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // y and the partial sums belong to earlier kernels until now
-    if (rs.ssq != nullptr) {
-      // RMSNorm denominators of this tile's x rows, one per epilogue thread, while the MMAs run
-      const int r = threadIdx.x;
+    RSD_PDL_WAIT();                            // y and the partial sums belong to earlier kernels until now
+    if (rs.ssq != nullptr && active != 0) {
+      // RMSNorm denominators of this tile's x rows while the MMAs run: 128 / kRows threads per row, so that a row's
+      // chunk sums are one round of loads, or two, instead of a chain as long as the row is wide
+      constexpr int kLanes = kRows >= 128 ? 1 : (kRows >= 8 ? 128 / kRows : 16);
+      const int r = threadIdx.x / kLanes, sub = threadIdx.x % kLanes;
+      float sum = 0.f;
       if (r < kRows && m0 + r < M) {
-        float sum = 0.f;
-        for (int c = 0; c < rs.n_chunks; ++c) sum += rs.ssq[(size_t)(m0 + r) * rs.n_chunks + c];
-        row_scale[r] = rsqrtf(sum * rs.inv_d + rs.eps);
+        const float* src = rs.ssq + (size_t)(m0 + r) * rs.n_chunks;
+#pragma unroll 8
+        for (int c = sub; c < rs.n_chunks; c += kLanes) sum += src[c];
       }
+#pragma unroll
+      for (int o = kLanes / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+      if (sub == 0 && r < kRows) row_scale[r] = rsqrtf(sum * rs.inv_d + rs.eps);
       asm volatile("bar.sync 1, 128;" ::: "memory");   // the four epilogue warps only
     }
     // the four epilogue warps sleep in hardware between polls (about 1 us at most): busy polling by 128 threads
     // crowds the shared-memory pipe that the producer and the MMA issuer need for their own barriers
-    bool ok = mbar_try_wait(tmem_full, 0);
-    for (uint32_t i = 0; i < (1u << 21) && !ok; ++i) {
+    bool ok = active != 0 && mbar_try_wait(tmem_full, 0);
+    for (uint32_t i = 0; i < (1u << 21) && !ok && active != 0; ++i) {
       ok = mbar_try_wait_sleep(tmem_full, 0, 1000);
-      if (!ok && flags[0]) break;                        // the CTA was stopped (idle phase or an expired wait)
+      if (!ok && flags[0]) break;                        // the CTA was stopped (an expired wait)
     }
-    if (!ok && flags[0] == 0) {
+    if (!ok && active != 0 && flags[0] == 0) {
       if (err) atomicCAS(err, 0, -5);
       flags[0] = 1;
     }
@@ -701,7 +708,7 @@ cudaError_t launch_mt(const CUtensorMap& tw, const CUtensorMap& tx, const CUtens
     configured = true;
   }
   dim3 grid(p.n_tiles, p.m_tiles, p.splits);
-  RSD_LAUNCH((gemm_tc_kernel<MT, SPLIT, false, DEEP>), grid, 192, Cfg::kSmemBytes, s, tw, tx, txl, y, M, N, K, accumulate, p.splits,
+  RSD_LAUNCH((gemm_tc_kernel<MT, SPLIT, false, DEEP>), grid, kTcThreads, Cfg::kSmemBytes, s, tw, tx, txl, y, M, N, K, accumulate, p.splits,
                                                                      p.kb_per_split, partials, err, n_active, rs,
                                                                      (__nv_bfloat16*)nullptr, (__nv_bfloat16*)nullptr);
   if (p.splits > 1 && !defer_reduce) {
@@ -778,7 +785,7 @@ cudaError_t launch_gemm_wait_probe(const void* W, const void* x, float* y, void*
   }
   int* err = (int*)((char*)scratch + kCounterBytes);
   float* partials = (float*)((char*)scratch + kCounterBytes + 256);
-  RSD_LAUNCH((gemm_tc_kernel<16, false, false, false, true>), dim3(1, 1, 1), 192, TcCfg<16>::kSmemBytes, s, tw, tx, tx, y, 16, 128, 64, 0, 1, 1,
+  RSD_LAUNCH((gemm_tc_kernel<16, false, false, false, true>), dim3(1, 1, 1), kTcThreads, TcCfg<16>::kSmemBytes, s, tw, tx, tx, y, 16, 128, 64, 0, 1, 1,
              partials, err, (const int32_t*)nullptr, RowScale(), (__nv_bfloat16*)nullptr, (__nv_bfloat16*)nullptr);
   return launched(1);
 }
@@ -831,7 +838,7 @@ static cudaError_t launch_gu_mt(const CUtensorMap& tw, const CUtensorMap& tx, co
   }
   const int total_kb = (K + kTileK - 1) / kTileK;
   dim3 grid(F / 64, (M + rows - 1) / rows, 1);
-  RSD_LAUNCH((gemm_tc_kernel<MT, true, true, DEEP>), grid, 192, smem, s, tw, tx, txl, (float*)nullptr, M, F, K, 0, 1, total_kb,
+  RSD_LAUNCH((gemm_tc_kernel<MT, true, true, DEEP>), grid, kTcThreads, smem, s, tw, tx, txl, (float*)nullptr, M, F, K, 0, 1, total_kb,
              (float*)nullptr, err, n_active, rs, act_hi, act_lo);
   return launched(1);
 }
