@@ -127,44 +127,70 @@ cudaError_t launch_rmsnorm(int dtype, float* x, const void* gain, void* out, voi
 // over the chunk.  The next GEMM multiplies its result rows by rsqrt(sum_chunk ssq / d + eps)
 // (RowScale), which is RMSNorm applied after the product instead of before it.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(64)
-reduce_norm_kernel(const float* __restrict__ partials, int splits, float* __restrict__ x,
-                   const __nv_bfloat16* __restrict__ gain, __nv_bfloat16* __restrict__ hi,
-                   __nv_bfloat16* __restrict__ lo, float* __restrict__ ssq, int M, int d, int n_chunks,
-                   const int32_t* n_active) {
-  RSD_PDL_SYNC();
-  RSD_SKIP_IF_IDLE(n_active);
+// Bound by latency (a launch moves 1-5 MB, all of it in L2): the gain is fetched under the wait, and the partial sums are
+// dealt over kSumGroups groups of 64 threads, so that up to kSumGroups * kSumAhead = 24 splits, the rule, are one
+// round of loads.  The groups' sums meet in shared memory and are added in order.
+constexpr int kSumGroups = 4, kSumAhead = 6;
+
+__global__ void __launch_bounds__(64 * kSumGroups)
+reduce_norm_kernel(const float* partials, int splits, float* x, const __nv_bfloat16* __restrict__ gain, __nv_bfloat16* hi,
+                   __nv_bfloat16* lo, float* ssq, int M, int d, int n_chunks, const int32_t* n_active) {
+  RSD_PDL_TRIGGER();
   __shared__ float red[2];
+  __shared__ float4 s_part[kSumGroups - 1][64];
+  const bool idle = n_active != nullptr && ld_cg(n_active) == 0;
   const int m = blockIdx.y, c = blockIdx.x;
-  const int col = c * 256 + threadIdx.x * 4;
+  const int col = c * 256 + threadIdx.x * 4, grp = threadIdx.y;
+  const size_t o = (size_t)m * d + col, stride = (size_t)M * d;
+  float g[4] = {0.f, 0.f, 0.f, 0.f};
+  if (col < d && grp == 0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) g[i] = to_f32(gain[col + i]);
+  }
+  RSD_PDL_WAIT();
+  if (idle) return;
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (col < d) {
+    float4 old;
+    if (grp == 0) old = *reinterpret_cast<const float4*>(x + o);
+    if (splits > 1) {
+      const int per = (splits + kSumGroups - 1) / kSumGroups, s_end = min(splits, (grp + 1) * per);
+      for (int s0 = grp * per; s0 < s_end; s0 += kSumAhead) {
+        float4 a[kSumAhead];
+#pragma unroll
+        for (int u = 0; u < kSumAhead; ++u)
+          if (s0 + u < s_end) a[u] = ld_cg(reinterpret_cast<const float4*>(partials + (size_t)(s0 + u) * stride + o));
+#pragma unroll
+        for (int u = 0; u < kSumAhead; ++u)
+          if (s0 + u < s_end) { v.x += a[u].x; v.y += a[u].y; v.z += a[u].z; v.w += a[u].w; }
+      }
+      if (grp > 0) s_part[grp - 1][threadIdx.x] = v;
+    }
+    if (grp == 0) { v.x += old.x; v.y += old.y; v.z += old.z; v.w += old.w; }
+  }
+  if (splits > 1) __syncthreads();
+  if (grp > 0) return;
   float ss = 0.f;
   if (col < d) {
-    const size_t o = (size_t)m * d + col;
-    float4 v = *reinterpret_cast<const float4*>(x + o);
     if (splits > 1) {
-      const size_t stride = (size_t)M * d;
-      // twelve loads in flight at a time (tail predicated): each group is one L2 round trip, and 10-24 splits
-      // are the rule; the sums stay in split order
-      for (int s0 = 0; s0 < splits; s0 += 12) {
-        float4 a[12];
 #pragma unroll
-        for (int u = 0; u < 12; ++u)
-          a[u] = s0 + u < splits ? __ldcg(reinterpret_cast<const float4*>(partials + (size_t)(s0 + u) * stride + o))
-                                 : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int u = 0; u < 12; ++u) { v.x += a[u].x; v.y += a[u].y; v.z += a[u].z; v.w += a[u].w; }
+      for (int i = 0; i < kSumGroups - 1; ++i) {
+        const float4 a = s_part[i][threadIdx.x];
+        v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
       }
       *reinterpret_cast<float4*>(x + o) = v;
     }
     ss = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-    store_operand<__nv_bfloat16>(hi, lo, o, v.x * to_f32(gain[col]));
-    store_operand<__nv_bfloat16>(hi, lo, o + 1, v.y * to_f32(gain[col + 1]));
-    store_operand<__nv_bfloat16>(hi, lo, o + 2, v.z * to_f32(gain[col + 2]));
-    store_operand<__nv_bfloat16>(hi, lo, o + 3, v.w * to_f32(gain[col + 3]));
+    const float y[4] = {v.x * g[0], v.y * g[1], v.z * g[2], v.w * g[3]};
+    __align__(8) __nv_bfloat16 h4[4], l4[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) store_operand<__nv_bfloat16>(h4, l4, i, y[i]);
+    *reinterpret_cast<uint2*>(hi + o) = *reinterpret_cast<const uint2*>(h4);
+    *reinterpret_cast<uint2*>(lo + o) = *reinterpret_cast<const uint2*>(l4);
   }
   ss = warp_sum(ss);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-  __syncthreads();
+  asm volatile("bar.sync 1, 64;" ::: "memory");            // the two warps of group 0
   if (threadIdx.x == 0) ssq[(size_t)m * n_chunks + c] = red[0] + red[1];
 }
 
@@ -173,7 +199,7 @@ cudaError_t launch_reduce_norm(const float* partials, int splits, float* x, cons
   if (M <= 0) return cudaSuccess;
   if (d % 4 != 0) return cudaErrorInvalidValue;
   const int n_chunks = norm_chunks(d);
-  RSD_LAUNCH((reduce_norm_kernel), dim3(n_chunks, M), 64, 0, s, partials, splits, x, (const __nv_bfloat16*)gain,
+  RSD_LAUNCH((reduce_norm_kernel), dim3(n_chunks, M), dim3(64, splits > 1 ? kSumGroups : 1), 0, s, partials, splits, x, (const __nv_bfloat16*)gain,
              (__nv_bfloat16*)hi, (__nv_bfloat16*)lo, ssq, M, d, n_chunks, n_active);
   return launched(1);
 }
@@ -318,60 +344,83 @@ __device__ __forceinline__ float split_sum(const float* direct, const float* par
 __device__ __forceinline__ float rotate_lo(float a, float b, float2 cs) { return fmaf(a, cs.x, -__fmul_rn(b, cs.y)); }
 __device__ __forceinline__ float rotate_hi(float a, float b, float2 cs) { return fmaf(b, cs.x, __fmul_rn(a, cs.y)); }
 
+// Bound by latency like reduce_norm: lists, page and angle are fetched under the wait, and with K-split partial sums
+// kSumGroups groups of 64 threads share them out.
 template <typename KT>
-__global__ void rope_kv_kernel(const float* qkv, const float* partials, int splits, PassView p, float* q_out, KT* pool,
-                               const int32_t* page_table, int max_pages,
-                               const float2* __restrict__ rope, int H, int KV, int hd, int pf) {
+__global__ void __launch_bounds__(64 * kSumGroups)
+rope_kv_kernel(const float* qkv, const float* partials, int splits, PassView p, float* q_out, KT* pool, const int32_t* page_table,
+               int max_pages, const float2* __restrict__ rope, int H, int KV, int hd, int pf) {
   RSD_PDL_TRIGGER();
+  __shared__ float s_part[kSumGroups - 1][128];
   if (p.n_active == nullptr) RSD_PDL_WAIT();   // a decode pass's lists may be read ahead of the wait, others not
   const int t = blockIdx.x;
   const bool idle = p.n_active != nullptr && ld_cg(p.n_active) == 0;
   const int row = ld_cg(p.tok_row + t), pos = ld_cg(p.tok_pos + t);
   if (idle || row < 0) { RSD_PDL_WAIT(); return; }
-  const int half = hd / 2;
+  // one block per (token, head): query and key heads are rotated, value heads copied; a pair (i, i + hd/2) per thread
+  const int head = blockIdx.y, half = hd / 2, i = threadIdx.x, grp = threadIdx.y;
   const int width = (H + 2 * KV) * hd;
-  const size_t src0 = (size_t)t * width;                 // offset of this token's row in qkv / a partial
-  const size_t sstride = (size_t)gridDim.x * width;      // one partial array = [T][width]
-  const float2* cs = rope + (size_t)pos * half;
+  const size_t src = (size_t)t * width + (size_t)head * hd + i;   // of this thread's pair in qkv / a partial
+  const size_t sstride = (size_t)gridDim.x * width;               // one partial array = [T][width]
   const int page = ld_cg(page_table + (size_t)row * max_pages + pos / kPageTokens);
-  const float2 first = cs[min((int)threadIdx.x, half - 1)];   // this thread's first angle
-  RSD_PDL_WAIT();
   const int slot = pos % kPageTokens;
+  float2 cs = make_float2(1.f, 0.f);
+  if (i < half && head < H + KV && grp == 0) cs = rope[(size_t)pos * half + i];
+  RSD_PDL_WAIT();
+  float a = 0.f, b = 0.f;
+  if (i < half) {
+    if (splits <= 1) {
+      a = qkv[src]; b = qkv[src + half];
+    } else {
+      const int per = (splits + kSumGroups - 1) / kSumGroups, s_end = min(splits, (grp + 1) * per);
+      for (int s0 = grp * per; s0 < s_end; s0 += kSumAhead) {
+        float ta[kSumAhead], tb[kSumAhead];
+#pragma unroll
+        for (int u = 0; u < kSumAhead; ++u)
+          if (s0 + u < s_end) {
+            ta[u] = ld_cg(partials + (size_t)(s0 + u) * sstride + src);
+            tb[u] = ld_cg(partials + (size_t)(s0 + u) * sstride + src + half);
+          }
+#pragma unroll
+        for (int u = 0; u < kSumAhead; ++u)
+          if (s0 + u < s_end) { a += ta[u]; b += tb[u]; }
+      }
+      if (grp > 0) { s_part[grp - 1][i] = a; s_part[grp - 1][i + 64] = b; }
+    }
+  }
+  if (splits > 1) __syncthreads();
+  if (grp > 0 || i >= half) return;
+  if (splits > 1) {
+#pragma unroll
+    for (int u = 0; u < kSumGroups - 1; ++u) { a += s_part[u][i]; b += s_part[u][i + 64]; }
+  }
   // page = K block [KV][16][hd] followed by V block [KV][hd][16] (V transposed within the page)
   // (pf = 4: two more blocks hold the low halves of the keys and of the values)
   const size_t block = (size_t)KV * kPageTokens * hd;
   KT* kbase = pool + (size_t)page * pf * block;
-  KT* vbase = kbase + block;
-  // one block per (token, head): query and key heads are rotated, value heads copied
-  const int head = blockIdx.y;
+  KT* dst;                                     // where the pair's two elements go, `gap` elements apart
+  size_t gap;
   if (head < H + KV) {
-    for (int i = threadIdx.x; i < half; i += blockDim.x) {
-      const float a = split_sum(qkv, partials, splits, src0 + head * hd + i, sstride);
-      const float b = split_sum(qkv, partials, splits, src0 + head * hd + i + half, sstride);
-      const float2 c = i == (int)threadIdx.x ? first : cs[i];
-      const float ra = rotate_lo(a, b, c), rb = rotate_hi(a, b, c);
-      if (head < H) {
-        q_out[(size_t)t * H * hd + head * hd + i] = ra;
-        q_out[(size_t)t * H * hd + head * hd + i + half] = rb;
-      } else {
-        KT* k = kbase + ((size_t)(head - H) * kPageTokens + slot) * hd;
-        const KT ka = from_f32<KT>(ra), kb2 = from_f32<KT>(rb);
-        k[i] = ka;
-        k[i + half] = kb2;
-        if (pf == 4) {
-          k[2 * block + i] = from_f32<KT>(ra - to_f32(ka));
-          k[2 * block + i + half] = from_f32<KT>(rb - to_f32(kb2));
-        }
-      }
+    const float ra = rotate_lo(a, b, cs), rb = rotate_hi(a, b, cs);
+    a = ra; b = rb;
+    if (head < H) {
+      float* q = q_out + ((size_t)t * H + head) * hd + i;
+      q[0] = a;
+      q[half] = b;
+      return;
     }
+    dst = kbase + ((size_t)(head - H) * kPageTokens + slot) * hd + i;
+    gap = half;
   } else {
-    const int vh_idx = head - H - KV;
-    for (int i = threadIdx.x; i < hd; i += blockDim.x) {
-      const float v = split_sum(qkv, partials, splits, src0 + (size_t)head * hd + i, sstride);
-      const KT vh = from_f32<KT>(v);
-      vbase[((size_t)vh_idx * hd + i) * kPageTokens + slot] = vh;
-      if (pf == 4) vbase[2 * block + ((size_t)vh_idx * hd + i) * kPageTokens + slot] = from_f32<KT>(v - to_f32(vh));
-    }
+    dst = kbase + block + ((size_t)(head - H - KV) * hd + i) * kPageTokens + slot;
+    gap = (size_t)half * kPageTokens;
+  }
+  const KT ka = from_f32<KT>(a), kb = from_f32<KT>(b);
+  dst[0] = ka;
+  dst[gap] = kb;
+  if (pf == 4) {
+    dst[2 * block] = from_f32<KT>(a - to_f32(ka));
+    dst[2 * block + gap] = from_f32<KT>(b - to_f32(kb));
   }
 }
 
@@ -482,11 +531,11 @@ cudaError_t launch_rope_kv(int kv_dtype, const float* qkv, SplitSum pending, Pas
     return launched(1);
   }
   if (kv_dtype == 2 || kv_dtype == 3)
-    RSD_LAUNCH((rope_kv_kernel<__half>), dim3(p.T, H + 2 * KV), 64, 0, s, qkv, pending.partials, pending.splits, p, q_out, (__half*)kv.pool_layer, kv.page_table, kv.max_pages, rope, H, KV, hd, pf);
+    RSD_LAUNCH((rope_kv_kernel<__half>), dim3(p.T, H + 2 * KV), dim3(64, pending.splits > 1 ? kSumGroups : 1), 0, s, qkv, pending.partials, pending.splits, p, q_out, (__half*)kv.pool_layer, kv.page_table, kv.max_pages, rope, H, KV, hd, pf);
   else if (kv_dtype == 1)
-    RSD_LAUNCH((rope_kv_kernel<__nv_bfloat16>), dim3(p.T, H + 2 * KV), 64, 0, s, qkv, pending.partials, pending.splits, p, q_out, (__nv_bfloat16*)kv.pool_layer, kv.page_table, kv.max_pages, rope, H, KV, hd, pf);
+    RSD_LAUNCH((rope_kv_kernel<__nv_bfloat16>), dim3(p.T, H + 2 * KV), dim3(64, pending.splits > 1 ? kSumGroups : 1), 0, s, qkv, pending.partials, pending.splits, p, q_out, (__nv_bfloat16*)kv.pool_layer, kv.page_table, kv.max_pages, rope, H, KV, hd, pf);
   else
-    RSD_LAUNCH((rope_kv_kernel<float>), dim3(p.T, H + 2 * KV), 64, 0, s, qkv, pending.partials, pending.splits, p, q_out, (float*)kv.pool_layer, kv.page_table, kv.max_pages, rope, H, KV, hd, pf);
+    RSD_LAUNCH((rope_kv_kernel<float>), dim3(p.T, H + 2 * KV), dim3(64, pending.splits > 1 ? kSumGroups : 1), 0, s, qkv, pending.partials, pending.splits, p, q_out, (float*)kv.pool_layer, kv.page_table, kv.max_pages, rope, H, KV, hd, pf);
   return launched(1);
 }
 
