@@ -16,6 +16,9 @@
 // cluster barrier every CTA merges a slice of the G x HD outputs out of all the CTAs' shared memory (in split
 // order) and writes it: no second launch and no trip through global memory.  With more splits than a cluster
 // holds the CTA writes its partial to scratch and a second kernel merges them.
+//
+// In a decode pass the lists and page ids are read, and the pages of the first rounds of every warp asked into L2, before
+// the wait for the preceding kernels: the cache streams in while the qkv product and the rotation still run.
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -70,21 +73,20 @@ __device__ __forceinline__ void mma_16816<__half>(float& d0, float& d1, float& d
 // halves of its keys and values in two more blocks: the attention is accurate to about 2^-20.
 template <int HD, typename KT, typename OT, bool EXT, bool CL>
 __global__ void __launch_bounds__(128, EXT ? 2 : 4)
-attn_decode_kernel(const float* __restrict__ q, const KT* __restrict__ pool, const int32_t* __restrict__ page_table,
-                   int max_pages, const int32_t* __restrict__ slot_row, const int32_t* __restrict__ len_or_pos, int len_offset,
-                   OT* __restrict__ out, OT* __restrict__ out_lo, float* __restrict__ part_o, float* __restrict__ part_ml, int H, int KV, int n_splits,
-                   const int32_t* __restrict__ n_active) {
-  RSD_PDL_SYNC();
-  if (n_active != nullptr && *n_active == 0) return;
+attn_decode_kernel(const float* q, const KT* pool, const int32_t* page_table, int max_pages, const int32_t* slot_row,
+                   const int32_t* len_or_pos, int len_offset, OT* out, OT* out_lo, float* part_o, float* part_ml, int H, int KV,
+                   int n_splits, const int32_t* n_active) {
+  RSD_PDL_TRIGGER();
+  if (n_active == nullptr) RSD_PDL_WAIT();   // a decode pass's lists and old pages may be read ahead of the wait, others not
   constexpr int KB = HD / 32;    // 32-dim blocks of the head dimension
   constexpr int NT = HD / 8;     // 8-dim output tiles
   __shared__ float s_m[4][8], s_l[4][8];
   __shared__ float s_o[4][8][HD];
   const int kvh = blockIdx.x, slot = blockIdx.y, split = blockIdx.z;
-  const int row = slot_row ? slot_row[slot] : slot;
-  if (row < 0) return;
-  const int ctx = len_or_pos[slot] + len_offset;
-  if (ctx <= 0) return;
+  const bool idle = n_active != nullptr && ld_cg(n_active) == 0;
+  const int row = slot_row ? ld_cg(slot_row + slot) : slot;
+  const int ctx = ld_cg(len_or_pos + slot) + len_offset;
+  if (idle || row < 0 || ctx <= 0) { RSD_PDL_WAIT(); return; }
   const int G = H / KV, h0 = kvh * G;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
@@ -93,21 +95,47 @@ attn_decode_kernel(const float* __restrict__ q, const KT* __restrict__ pool, con
   const int n_pages = (ctx + kPageTokens - 1) / kPageTokens;
   const int pps = (n_pages + n_splits - 1) / n_splits;
   const int p_begin = split * pps, p_end = min(n_pages, p_begin + pps);
+  const int32_t* pt = page_table + (size_t)row * max_pages;
+  const int block_elems = KV * kPageTokens * HD, page_elems = (EXT ? 4 : 2) * block_elems;
+  // tokens whose keys this lane loads: tile 0 -> 4(g/2) + g%2, tile 1 -> that + 2
+  const int tok0 = 4 * (g >> 1) + (g & 1), tok1 = tok0 + 2;
+  const int first = p_begin + warp;
+  if (n_active != nullptr) {
+    // lane i fetches the id of the warp's i-th page, then all lanes ask for its 128-byte lines; a line that this pass
+    // still writes (the newest token's) is merely fetched, not read
+    constexpr int kAhead = 4, kLines = kPageTokens * HD * (int)sizeof(KT) / 128;    // lines of one block of a page
+    const int ahead = lane < kAhead && first + 4 * lane < p_end ? ld_cg(pt + first + 4 * lane) : -1;
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      const int pg = __shfl_sync(0xFFFFFFFFu, ahead, i);
+      if (pg < 0) break;
+      const char* base = reinterpret_cast<const char*>(pool + (size_t)pg * page_elems + (size_t)kvh * kPageTokens * HD);
+#pragma unroll
+      for (int bl = 0; bl < (EXT ? 4 : 2); ++bl)
+        if (lane < kLines) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + (size_t)bl * block_elems * sizeof(KT) + lane * 128));
+    }
+  }
+  int page = first < p_end ? ld_cg(pt + first) : 0;
+  RSD_PDL_WAIT();
 
+  // the group's queries, rounded once by the whole block: one coalesced round of loads
+  constexpr int kLd = HD + 32;                   // rows 64 bytes apart modulo 128: the fragment loads below do not collide
+  __shared__ __align__(16) KT s_q[EXT ? 2 : 1][8][kLd];
+#pragma unroll
+  for (int i = 0; i < 8 * HD / 128; ++i) {
+    const int idx = i * 128 + threadIdx.x, gg = idx / HD, dd = idx % HD;
+    const float v = gg < G ? q[((size_t)slot * H + h0 + gg) * HD + dd] : 0.f;
+    const KT hi = from_f32<KT>(v);
+    s_q[0][gg][dd] = hi;
+    if (EXT) s_q[EXT ? 1 : 0][gg][dd] = from_f32<KT>(v - to_f32(hi));
+  }
+  __syncthreads();
   // Q fragments (rows 8..15 of the tile are padding): dims 32j + 8t + e of head h0 + g
-  uint32_t qa[KB][2][2], ql[EXT ? KB : 1][2][2];
+  __align__(16) uint32_t qa[KB][2][2], ql[EXT ? KB : 1][2][2];
 #pragma unroll
   for (int j = 0; j < KB; ++j) {
-    float v[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = g < G ? q[((size_t)slot * H + h0 + g) * HD + 32 * j + 8 * t + e] : 0.f;
-    if (EXT) {
-      pack2_split<KT>(v[0], v[1], qa[j][0][0], ql[j][0][0]); pack2_split<KT>(v[2], v[3], qa[j][0][1], ql[j][0][1]);
-      pack2_split<KT>(v[4], v[5], qa[j][1][0], ql[j][1][0]); pack2_split<KT>(v[6], v[7], qa[j][1][1], ql[j][1][1]);
-    } else {
-      qa[j][0][0] = pack2<KT>(v[0], v[1]); qa[j][0][1] = pack2<KT>(v[2], v[3]);
-      qa[j][1][0] = pack2<KT>(v[4], v[5]); qa[j][1][1] = pack2<KT>(v[6], v[7]);
-    }
+    *reinterpret_cast<uint4*>(qa[j]) = *reinterpret_cast<const uint4*>(&s_q[0][g][32 * j + 8 * t]);
+    if (EXT) *reinterpret_cast<uint4*>(ql[EXT ? j : 0]) = *reinterpret_cast<const uint4*>(&s_q[EXT ? 1 : 0][g][32 * j + 8 * t]);
   }
   // Rows 8..15 of every MMA tile are padding (their A rows are zero), so all tiles share two dump
   // registers for those rows instead of carrying 2 x (NT + 2) dead accumulators.
@@ -117,16 +145,10 @@ attn_decode_kernel(const float* __restrict__ q, const KT* __restrict__ pool, con
   float dump0 = 0.f, dump1 = 0.f;
   float m_run = -INFINITY, l_run = 0.f;
 
-  const int32_t* pt = page_table + (size_t)row * max_pages;
-  const size_t block_elems = (size_t)KV * kPageTokens * HD;
-  const size_t page_elems = (EXT ? 4 : 2) * block_elems;
-  // tokens whose keys this lane loads: tile 0 -> 4(g/2) + g%2, tile 1 -> that + 2
-  const int tok0 = 4 * (g >> 1) + (g & 1), tok1 = tok0 + 2;
-  int page = (p_begin + warp < p_end) ? pt[p_begin + warp] : 0;
-  for (int p = p_begin + warp; p < p_end; p += 4) {
+  for (int p = first; p < p_end; p += 4) {
     const KT* kb = pool + (size_t)page * page_elems + (size_t)kvh * kPageTokens * HD;
-    const KT* vb = pool + (size_t)page * page_elems + (size_t)KV * kPageTokens * HD + (size_t)kvh * HD * kPageTokens;
-    if (p + 4 < p_end) page = pt[p + 4];     // next page's index is fetched while this page is worked on
+    const KT* vb = kb + block_elems;
+    if (p + 4 < p_end) page = ld_cg(pt + p + 4);     // next page's index is fetched while this page is worked on
     // all of the page's keys and values are requested up front (8 KB per warp in flight)
     uint4 k0[KB], k1[KB];
     uint2 vv[NT], vl[EXT ? NT : 1];
@@ -136,10 +158,10 @@ attn_decode_kernel(const float* __restrict__ q, const KT* __restrict__ pool, con
       k1[j] = *reinterpret_cast<const uint4*>(kb + tok1 * HD + 32 * j + 8 * t);
     }
 #pragma unroll
-    for (int i = 0; i < NT; ++i) vv[i] = *reinterpret_cast<const uint2*>(vb + (size_t)(8 * i + g) * kPageTokens + 4 * t);
+    for (int i = 0; i < NT; ++i) vv[i] = *reinterpret_cast<const uint2*>(vb + (8 * i + g) * kPageTokens + 4 * t);
     if (EXT) {
 #pragma unroll
-      for (int i = 0; i < NT; ++i) vl[i] = *reinterpret_cast<const uint2*>(vb + 2 * block_elems + (size_t)(8 * i + g) * kPageTokens + 4 * t);
+      for (int i = 0; i < NT; ++i) vl[i] = *reinterpret_cast<const uint2*>(vb + 2 * block_elems + (8 * i + g) * kPageTokens + 4 * t);
     }
     float s0[2] = {0.f, 0.f}, s1[2] = {0.f, 0.f};
 #pragma unroll
@@ -320,14 +342,14 @@ __global__ void decode_slots_kernel(const int32_t* slot_row, const int32_t* len_
 constexpr int kClusterSplits = 8;   // the portable cluster size
 
 int pick_splits(int B, int KV, int max_ctx) {
-  const int ctas = B * KV;
+  const int ctas = B * KV, max_pages = max_ctx / kPageTokens;
   int splits = (4 * 148) / ctas;   // one wave of at most four CTAs per SM: a second, partial wave would double the time
-  const int max_by_ctx = std::max(1, (max_ctx / kPageTokens) / 4);   // at least 4 pages per split (one per warp)
+  const int max_by_ctx = std::max(1, max_pages / 4);   // at least 4 pages per split (one per warp)
   splits = std::min(splits, max_by_ctx);
   splits = std::max(1, std::min(splits, kMaxSplits));
-  // a few splits more than a cluster holds are not worth the second launch: 8 splits of 16 or more (slot, KV head)
-  // pairs already put a CTA on most SMs
-  if (splits > kClusterSplits && ctas * kClusterSplits >= 128) splits = kClusterSplits;
+  // more splits than a cluster holds cost a second launch: not worth it when 8 splits of 16 or more (slot, KV head)
+  // pairs already put a CTA on most SMs, nor when 8 splits leave a warp at most six pages
+  if (splits > kClusterSplits && (ctas * kClusterSplits >= 128 || max_pages <= kClusterSplits * 24)) splits = kClusterSplits;
   return splits;
 }
 
