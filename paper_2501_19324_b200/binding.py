@@ -365,7 +365,7 @@ def k_attn_decode(q, kv_pool, page_table, ctx_len, KV, ext=False):
     max_pages = page_table.shape[1]
     out = torch.empty_like(q)
     nbytes = lib().rsd_k_attn_decode_scratch_bytes(B, H, hd, max_pages * 16)
-    scratch = torch.zeros(nbytes, dtype=torch.uint8, device=q.device)
+    scratch = torch.empty(nbytes, dtype=torch.uint8, device=q.device)
     dt = {torch.bfloat16: RSD_BF16, torch.float16: 2, torch.float32: RSD_F32}[kv_pool.dtype]
     if ext:
         dt = 3

@@ -108,6 +108,7 @@ struct rsd_ctx {
   uint64_t dec_graph_kernels[16] = {};
   int sd_k = 0, slots_max = 0;
 
+  int pass_width = 1;          // consecutive positions of a row that a decode pass writes (a speculative round: sd_k)
   int attn_rows_hint = 0;      // rows expected to be active in the running decode phase (0: all slots)
   bool time_this_iter = false, in_decode = false;
   // per-phase timing of rsd_step (rsd_debug_phase_ms)
@@ -522,7 +523,7 @@ int forward_pass(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
       // decode pass: one query per row slot
       CU(launch_attn_decode(M.kv_dtype, c->q, kv.pool_layer, kv.page_table, kv.max_pages, p.tok_row, p.tok_pos, 1,
                             c->attn, attn_lo, m.dtype, T, H, KV, hd, c->S, c->attn_scratch, c->attn_scratch_bytes,
-                            p.n_active, s, c->attn_rows_hint));
+                            p.n_active, s, c->attn_rows_hint, c->pass_width));
     } else {
       CU(launch_attn_chunk(M.kv_dtype, c->q, p, kv, c->attn, attn_lo, m.dtype, H, KV, hd, s,
                            (int*)((char*)c->gemm_scratch + 4096)));
@@ -574,7 +575,7 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
     CU(launch_rope_kv(M.kv_dtype, c->qkv, qkv_pending, p, c->q, kv, M.rope, H, KV, hd, s));
     CU(launch_attn_decode(M.kv_dtype, c->q, kv.pool_layer, kv.page_table, kv.max_pages, p.tok_row, p.tok_pos, 1,
                           c->attn, c->attn_lo, m.dtype, T, H, KV, hd, c->S, c->attn_scratch, c->attn_scratch_bytes,
-                          p.n_active, s, c->attn_rows_hint));
+                          p.n_active, s, c->attn_rows_hint, c->pass_width));
     rc = gemm(c, M, M.wo[l], c->attn, c->attn_lo, c->x, T, d, H * hd, 1, p.n_active, &x_pending, s);
     if (rc) return rc;
     CU(launch_reduce_norm(x_pending.partials, x_pending.splits, c->x, M.norm2[l], c->h, c->h_lo, c->norm_ssq, T, d,
@@ -751,7 +752,9 @@ int sd_verify_pass(rsd_ctx* c, int n_slots, cudaStream_t s) {
   CU(launch_sd_verify_prepare(c->st, n_slots, s));
   const int T = n_slots * c->sd_k;
   PassView p{c->st.pass_tok_id, c->st.pass_tok_row, c->st.pass_tok_pos, T, c->st.n_active};
+  c->pass_width = c->sd_k;
   int rc = model_logits(c, RSD_TARGET, p, false, s);
+  c->pass_width = 1;
   if (rc) return rc;
   if (c->dbg_logits[1]) {
     RSD_LAUNCH((scatter_logits_sd_kernel), T, 256, 0, s, c->logits, c->st.pass_tok_row, c->st.sd_out_idx, c->dbg_logits[1],

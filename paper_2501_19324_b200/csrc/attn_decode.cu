@@ -2,10 +2,10 @@
 //
 // A CTA of 4 warps serves one (row slot, KV head, context split): the G = H / KV query heads that
 // share the KV head are the rows of a 16-row MMA tile, so every key / value is read once from HBM for
-// the whole group.  Each warp walks its share of the 16-token pages:
-//   S  = Q K^T   with mma.sync m16n8k16 (bf16 in, fp32 out): keys stream from global memory straight
-//        into B fragments with 128-bit loads (the order of the head dims inside a 32-dim block is
-//        permuted identically for Q and K, which a dot product does not see);
+// the whole group.  Each warp walks its share of the 16-token pages through a ring of page buffers of its own in shared
+// memory (16-byte cp.async, a page ahead):
+//   S  = Q K^T   with mma.sync m16n8k16 (16-bit in, fp32 out): a key fragment is one 128-bit load (the order of
+//        the head dims inside a 32-dim block is permuted identically for Q and K, which a dot product does not see);
 //   softmax statistics per head are kept on line (running max / sum), reduced over the 4 lanes that
 //        share a row with warp shuffles;
 //   O += P V     with the same MMA: values are stored transposed inside a page ([hd][16 tokens]), so a
@@ -17,8 +17,13 @@
 // order) and writes it: no second launch and no trip through global memory.  With more splits than a cluster
 // holds the CTA writes its partial to scratch and a second kernel merges them.
 //
-// In a decode pass the lists and page ids are read, and the pages of the first rounds of every warp asked into L2, before
-// the wait for the preceding kernels: the cache streams in while the qkv product and the rotation still run.
+//
+// In a decode pass only the pass's own tokens are written by the kernels just before: every page that ends ahead of the
+// pass's first new position is older than the pass.  Lists, page ids and each warp's first pages are therefore
+// requested before the wait for the preceding kernels and stream in while the qkv product and the rotation still run;
+// at the step loop's contexts (a page or two per warp) the cache has arrived when the query has.  (Fragments loaded from
+// global memory straight into registers had one page a warp in flight and none under the wait: 12.3 us a launch at 32
+// rows x 400 tokens, 12 / 2 heads, and 330 us for 64 rows x 4096-16384 tokens, 28 / 4 heads; now 9 us and 217 us.)
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -68,20 +73,38 @@ __device__ __forceinline__ void mma_16816<__half>(float& d0, float& d1, float& d
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+// Shared memory of a CTA: 4 warps x kStages page buffers; the warps' outputs take its place after the loop.  An extended
+// page (16 KB) gets one buffer a warp, a plain one (8 KB) two, so that three CTAs fit an SM either way.
+template <int HD, bool EXT> struct DecCfg {
+  static constexpr int kPageBytes = (EXT ? 4 : 2) * kPageTokens * HD * 2;
+  static constexpr int kStages = EXT ? 1 : 2;
+  static constexpr int kRingBytes = 4 * kStages * kPageBytes;
+  static_assert(kRingBytes >= 4 * 8 * HD * 4, "the outputs of the four warps alias the ring");
+};
+
 // part_o: [slot][head][split][HD] un-normalised outputs; part_ml: [slot][head][split][2] (max, sum).
 // EXT: queries and softmax weights enter the products as hi + lo pairs and every page carries the low
 // halves of its keys and values in two more blocks: the attention is accurate to about 2^-20.
+// new_tokens: how many of a row's last positions the pass itself writes.
 template <int HD, typename KT, typename OT, bool EXT, bool CL>
-__global__ void __launch_bounds__(128, EXT ? 2 : 4)
+__global__ void __launch_bounds__(128, 3)
 attn_decode_kernel(const float* q, const KT* pool, const int32_t* page_table, int max_pages, const int32_t* slot_row,
                    const int32_t* len_or_pos, int len_offset, OT* out, OT* out_lo, float* part_o, float* part_ml, int H, int KV,
-                   int n_splits, const int32_t* n_active) {
+                   int n_splits, const int32_t* n_active, int new_tokens) {
   RSD_PDL_TRIGGER();
   if (n_active == nullptr) RSD_PDL_WAIT();   // a decode pass's lists and old pages may be read ahead of the wait, others not
+  using Cfg = DecCfg<HD, EXT>;
   constexpr int KB = HD / 32;    // 32-dim blocks of the head dimension
   constexpr int NT = HD / 8;     // 8-dim output tiles
+  constexpr int kBlock = kPageTokens * HD;       // elements of one head's keys (or values) in a page
+  constexpr int kStages = Cfg::kStages, kParts = EXT ? 4 : 2;
+  extern __shared__ __align__(128) uint8_t ring_raw[];
   __shared__ float s_m[4][8], s_l[4][8];
-  __shared__ float s_o[4][8][HD];
+  auto s_o = reinterpret_cast<float(*)[8][HD]>(ring_raw);
   const int kvh = blockIdx.x, slot = blockIdx.y, split = blockIdx.z;
   const bool idle = n_active != nullptr && ld_cg(n_active) == 0;
   const int row = slot_row ? ld_cg(slot_row + slot) : slot;
@@ -96,27 +119,38 @@ attn_decode_kernel(const float* q, const KT* pool, const int32_t* page_table, in
   const int pps = (n_pages + n_splits - 1) / n_splits;
   const int p_begin = split * pps, p_end = min(n_pages, p_begin + pps);
   const int32_t* pt = page_table + (size_t)row * max_pages;
-  const int block_elems = KV * kPageTokens * HD, page_elems = (EXT ? 4 : 2) * block_elems;
-  // tokens whose keys this lane loads: tile 0 -> 4(g/2) + g%2, tile 1 -> that + 2
-  const int tok0 = 4 * (g >> 1) + (g & 1), tok1 = tok0 + 2;
-  const int first = p_begin + warp;
-  if (n_active != nullptr) {
-    // lane i fetches the id of the warp's i-th page, then all lanes ask for its 128-byte lines; a line that this pass
-    // still writes (the newest token's) is merely fetched, not read
-    constexpr int kAhead = 4, kLines = kPageTokens * HD * (int)sizeof(KT) / 128;    // lines of one block of a page
-    const int ahead = lane < kAhead && first + 4 * lane < p_end ? ld_cg(pt + first + 4 * lane) : -1;
+  const size_t page_elems = (size_t)kParts * KV * kBlock;
+  KT* ring = reinterpret_cast<KT*>(ring_raw) + (size_t)warp * kStages * kParts * kBlock;
+  // Keys of token t: 16-byte chunk c of its row sits at chunk c ^ 4 (t & 1), so that the two rows a quarter warp reads
+  // together fall on different banks.  Values as in the page.
+  auto fetch = [&](int page, int stage) {
+    const KT* src = pool + (size_t)page * page_elems + (size_t)kvh * kBlock + lane * 8;
+    KT* dst = ring + stage * kParts * kBlock;
+    constexpr int kChunks = kBlock / 8, kRow = HD / 8;
 #pragma unroll
-    for (int i = 0; i < kAhead; ++i) {
-      const int pg = __shfl_sync(0xFFFFFFFFu, ahead, i);
-      if (pg < 0) break;
-      const char* base = reinterpret_cast<const char*>(pool + (size_t)pg * page_elems + (size_t)kvh * kPageTokens * HD);
+    for (int part = 0; part < kParts; ++part) {
 #pragma unroll
-      for (int bl = 0; bl < (EXT ? 4 : 2); ++bl)
-        if (lane < kLines) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + (size_t)bl * block_elems * sizeof(KT) + lane * 128));
+      for (int i = 0; i < kChunks / 32; ++i) {
+        const int c = i * 32 + lane, d = (part & 1) ? c : (c ^ (((c / kRow) & 1) << 2));
+        cp_async16(dst + part * kBlock + d * 8, src + (size_t)part * KV * kBlock + i * 256);
+      }
     }
-  }
-  int page = first < p_end ? ld_cg(pt + first) : 0;
+  };
+  const int first = p_begin + warp, n_old = (ctx - new_tokens) / kPageTokens;   // pages [0, n_old) are older than the pass
+  int next = first;                              // the page whose turn it is to be fetched
+  int next_id = next < p_end ? ld_cg(pt + next) : 0;
+  auto fetch_next = [&](int stage) {
+    if (next < p_end) {
+      fetch(next_id, stage);
+      next += 4;
+      if (next < p_end) next_id = ld_cg(pt + next);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  int fetched = 0;
+  for (; fetched < kStages && next < min(p_end, n_old); ++fetched) fetch_next(fetched);
   RSD_PDL_WAIT();
+  for (; fetched < kStages; ++fetched) fetch_next(fetched);
 
   // the group's queries, rounded once by the whole block: one coalesced round of loads
   constexpr int kLd = HD + 32;                   // rows 64 bytes apart modulo 128: the fragment loads below do not collide
@@ -144,43 +178,37 @@ attn_decode_kernel(const float* q, const KT* pool, const int32_t* page_table, in
   for (int i = 0; i < NT; ++i) { o[i][0] = o[i][1] = 0.f; }
   float dump0 = 0.f, dump1 = 0.f;
   float m_run = -INFINITY, l_run = 0.f;
+  // tokens whose keys this lane loads: tile 0 -> 4(g/2) + g%2, tile 1 -> that + 2 (the same parity)
+  const int tok0 = 4 * (g >> 1) + (g & 1), tok1 = tok0 + 2;
+  const int key_off = ((t ^ ((g & 1) << 2))) * 8;
 
+  int stage = 0;
   for (int p = first; p < p_end; p += 4) {
-    const KT* kb = pool + (size_t)page * page_elems + (size_t)kvh * kPageTokens * HD;
-    const KT* vb = kb + block_elems;
-    if (p + 4 < p_end) page = ld_cg(pt + p + 4);     // next page's index is fetched while this page is worked on
-    // all of the page's keys and values are requested up front (8 KB per warp in flight)
-    uint4 k0[KB], k1[KB];
-    uint2 vv[NT], vl[EXT ? NT : 1];
-#pragma unroll
-    for (int j = 0; j < KB; ++j) {
-      k0[j] = *reinterpret_cast<const uint4*>(kb + tok0 * HD + 32 * j + 8 * t);
-      k1[j] = *reinterpret_cast<const uint4*>(kb + tok1 * HD + 32 * j + 8 * t);
-    }
-#pragma unroll
-    for (int i = 0; i < NT; ++i) vv[i] = *reinterpret_cast<const uint2*>(vb + (8 * i + g) * kPageTokens + 4 * t);
-    if (EXT) {
-#pragma unroll
-      for (int i = 0; i < NT; ++i) vl[i] = *reinterpret_cast<const uint2*>(vb + 2 * block_elems + (8 * i + g) * kPageTokens + 4 * t);
-    }
+    asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 1) : "memory");
+    __syncwarp();
+    const KT* kb = ring + stage * kParts * kBlock;
+    const KT* vb = kb + kBlock;
     float s0[2] = {0.f, 0.f}, s1[2] = {0.f, 0.f};
 #pragma unroll
     for (int j = 0; j < KB; ++j) {
-      mma_16816<KT>(s0[0], s0[1], dump0, dump1, qa[j][0][0], 0u, qa[j][0][1], 0u, k0[j].x, k0[j].y);
-      mma_16816<KT>(s0[0], s0[1], dump0, dump1, qa[j][1][0], 0u, qa[j][1][1], 0u, k0[j].z, k0[j].w);
-      mma_16816<KT>(s1[0], s1[1], dump0, dump1, qa[j][0][0], 0u, qa[j][0][1], 0u, k1[j].x, k1[j].y);
-      mma_16816<KT>(s1[0], s1[1], dump0, dump1, qa[j][1][0], 0u, qa[j][1][1], 0u, k1[j].z, k1[j].w);
+      const int off = (32 * j) ^ key_off;        // chunk 4j + t, swizzled
+      const uint4 k0 = *reinterpret_cast<const uint4*>(kb + tok0 * HD + off);
+      const uint4 k1 = *reinterpret_cast<const uint4*>(kb + tok1 * HD + off);
+      mma_16816<KT>(s0[0], s0[1], dump0, dump1, qa[j][0][0], 0u, qa[j][0][1], 0u, k0.x, k0.y);
+      mma_16816<KT>(s0[0], s0[1], dump0, dump1, qa[j][1][0], 0u, qa[j][1][1], 0u, k0.z, k0.w);
+      mma_16816<KT>(s1[0], s1[1], dump0, dump1, qa[j][0][0], 0u, qa[j][0][1], 0u, k1.x, k1.y);
+      mma_16816<KT>(s1[0], s1[1], dump0, dump1, qa[j][1][0], 0u, qa[j][1][1], 0u, k1.z, k1.w);
       if (EXT) {
-        const uint4 e0 = *reinterpret_cast<const uint4*>(kb + 2 * block_elems + tok0 * HD + 32 * j + 8 * t);
-        const uint4 e1 = *reinterpret_cast<const uint4*>(kb + 2 * block_elems + tok1 * HD + 32 * j + 8 * t);
+        const uint4 e0 = *reinterpret_cast<const uint4*>(kb + 2 * kBlock + tok0 * HD + off);
+        const uint4 e1 = *reinterpret_cast<const uint4*>(kb + 2 * kBlock + tok1 * HD + off);
         mma_16816<KT>(s0[0], s0[1], dump0, dump1, qa[j][0][0], 0u, qa[j][0][1], 0u, e0.x, e0.y);
         mma_16816<KT>(s0[0], s0[1], dump0, dump1, qa[j][1][0], 0u, qa[j][1][1], 0u, e0.z, e0.w);
         mma_16816<KT>(s1[0], s1[1], dump0, dump1, qa[j][0][0], 0u, qa[j][0][1], 0u, e1.x, e1.y);
         mma_16816<KT>(s1[0], s1[1], dump0, dump1, qa[j][1][0], 0u, qa[j][1][1], 0u, e1.z, e1.w);
-        mma_16816<KT>(s0[0], s0[1], dump0, dump1, ql[j][0][0], 0u, ql[j][0][1], 0u, k0[j].x, k0[j].y);
-        mma_16816<KT>(s0[0], s0[1], dump0, dump1, ql[j][1][0], 0u, ql[j][1][1], 0u, k0[j].z, k0[j].w);
-        mma_16816<KT>(s1[0], s1[1], dump0, dump1, ql[j][0][0], 0u, ql[j][0][1], 0u, k1[j].x, k1[j].y);
-        mma_16816<KT>(s1[0], s1[1], dump0, dump1, ql[j][1][0], 0u, ql[j][1][1], 0u, k1[j].z, k1[j].w);
+        mma_16816<KT>(s0[0], s0[1], dump0, dump1, ql[j][0][0], 0u, ql[j][0][1], 0u, k0.x, k0.y);
+        mma_16816<KT>(s0[0], s0[1], dump0, dump1, ql[j][1][0], 0u, ql[j][1][1], 0u, k0.z, k0.w);
+        mma_16816<KT>(s1[0], s1[1], dump0, dump1, ql[j][0][0], 0u, ql[j][0][1], 0u, k1.x, k1.y);
+        mma_16816<KT>(s1[0], s1[1], dump0, dump1, ql[j][1][0], 0u, ql[j][1][1], 0u, k1.z, k1.w);
       }
     }
     // this lane's scores of head g: tokens 4t, 4t+1 (tile 0) and 4t+2, 4t+3 (tile 1) of the page
@@ -210,14 +238,21 @@ attn_decode_kernel(const float* q, const KT* pool, const int32_t* page_table, in
     }
 #pragma unroll
     for (int i = 0; i < NT; ++i) {
+      const uint2 vv = *reinterpret_cast<const uint2*>(vb + (8 * i + g) * kPageTokens + 4 * t);
       o[i][0] *= corr; o[i][1] *= corr;
-      mma_16816<KT>(o[i][0], o[i][1], dump0, dump1, pa0, 0u, pa2, 0u, vv[i].x & mlo, vv[i].y & mhi);
+      mma_16816<KT>(o[i][0], o[i][1], dump0, dump1, pa0, 0u, pa2, 0u, vv.x & mlo, vv.y & mhi);
       if (EXT) {
-        mma_16816<KT>(o[i][0], o[i][1], dump0, dump1, pl0, 0u, pl2, 0u, vv[i].x & mlo, vv[i].y & mhi);
-        mma_16816<KT>(o[i][0], o[i][1], dump0, dump1, pa0, 0u, pa2, 0u, vl[i].x & mlo, vl[i].y & mhi);
+        const uint2 vl = *reinterpret_cast<const uint2*>(vb + 2 * kBlock + (8 * i + g) * kPageTokens + 4 * t);
+        mma_16816<KT>(o[i][0], o[i][1], dump0, dump1, pl0, 0u, pl2, 0u, vv.x & mlo, vv.y & mhi);
+        mma_16816<KT>(o[i][0], o[i][1], dump0, dump1, pa0, 0u, pa2, 0u, vl.x & mlo, vl.y & mhi);
       }
     }
+    __syncwarp();                                // every lane has read the buffer
+    fetch_next(stage);
+    stage = stage + 1 == kStages ? 0 : stage + 1;
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();                               // the ring is free: the outputs take its place
   // the 4 lanes of a row hold partial sums of l
   l_run += __shfl_xor_sync(0xFFFFFFFFu, l_run, 1);
   l_run += __shfl_xor_sync(0xFFFFFFFFu, l_run, 2);
@@ -341,12 +376,18 @@ __global__ void decode_slots_kernel(const int32_t* slot_row, const int32_t* len_
 
 constexpr int kClusterSplits = 8;   // the portable cluster size
 
+// Splits of a row's context.  One wave of at most three CTAs per SM when that leaves short splits: a second, partial wave
+// would double the time (16 rows x 1000-2048 tokens, 28 / 4 heads: 21 us in one wave, 29 us with eight splits).  Splits
+// of 64 pages and more are worth several waves instead, since rows of different lengths then even out (64 rows x
+// 4096-16384 tokens, 28 / 4 heads: 261 us in one wave, 217 us = 93 % of the copy bandwidth with eight splits).
 int pick_splits(int B, int KV, int max_ctx) {
   const int ctas = B * KV, max_pages = max_ctx / kPageTokens;
-  int splits = (4 * 148) / ctas;   // one wave of at most four CTAs per SM: a second, partial wave would double the time
-  const int max_by_ctx = std::max(1, max_pages / 4);   // at least 4 pages per split (one per warp)
-  splits = std::min(splits, max_by_ctx);
-  splits = std::max(1, std::min(splits, kMaxSplits));
+  int splits = (3 * 148) / ctas;
+  while (splits < kClusterSplits && max_pages / std::max(1, splits) >= 64) ++splits;
+  // at least 8 pages per split: two per warp, both on their way before the wait (4 and 8 pages: 714 and 706 ms for two
+  // steps of 32 rows with contexts of a few hundred tokens)
+  splits = std::max(1, std::min(splits, std::max(1, max_pages / 8)));
+  splits = std::min(splits, kMaxSplits);
   // more splits than a cluster holds cost a second launch: not worth it when 8 splits of 16 or more (slot, KV head)
   // pairs already put a CTA on most SMs, nor when 8 splits leave a warp at most six pages
   if (splits > kClusterSplits && (ctas * kClusterSplits >= 128 || max_pages <= kClusterSplits * 24)) splits = kClusterSplits;
@@ -355,11 +396,11 @@ int pick_splits(int B, int KV, int max_ctx) {
 
 // Launch with programmatic stream serialisation and, when cluster_z > 1, clusters of cluster_z CTAs along z.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_decode(void (*kernel)(KArgs...), dim3 grid, int cluster_z, cudaStream_t s, Args&&... args) {
+cudaError_t launch_decode(void (*kernel)(KArgs...), dim3 grid, int cluster_z, int smem, cudaStream_t s, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(128);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -385,7 +426,8 @@ size_t attn_decode_scratch_bytes(int B, int H, int hd, int max_ctx) {
 cudaError_t launch_attn_decode(int kv_dtype, const float* q, const void* pool_layer, const int32_t* page_table,
                                int max_pages, const int32_t* slot_row, const int32_t* len_or_pos, int len_offset,
                                void* out, void* out_lo, int out_dtype, int B, int H, int KV, int hd, int max_ctx,
-                               void* scratch, size_t scratch_bytes, const int32_t* n_active, cudaStream_t s, int active_rows) {
+                               void* scratch, size_t scratch_bytes, const int32_t* n_active, cudaStream_t s, int active_rows,
+                               int new_tokens) {
   if (B <= 0) return cudaSuccess;
   if (!scratch || scratch_bytes < attn_decode_scratch_bytes(B, H, hd, max_ctx)) return cudaErrorInvalidValue;
   const int G = H / KV;
@@ -410,12 +452,19 @@ cudaError_t launch_attn_decode(int kv_dtype, const float* q, const void* pool_la
   dim3 grid(KV, B, splits);
 #define RSD_DEC(HD, KT, OT, EXTV)                                                                                          \
   do {                                                                                                               \
+    static const cudaError_t set_ = [] {                                                                             \
+      cudaError_t e = cudaFuncSetAttribute(attn_decode_kernel<HD, KT, OT, EXTV, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                           DecCfg<HD, EXTV>::kRingBytes);                                            \
+      return e != cudaSuccess ? e : cudaFuncSetAttribute(attn_decode_kernel<HD, KT, OT, EXTV, false>,                \
+                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, DecCfg<HD, EXTV>::kRingBytes); \
+    }();                                                                                                             \
+    if (set_ != cudaSuccess) return set_;                                                                            \
     if (clustered)                                                                                                   \
-      (void)launch_decode(attn_decode_kernel<HD, KT, OT, EXTV, true>, grid, splits, s, q, (const KT*)pool_layer, page_table,       \
-                          max_pages, slot_row, len_or_pos, len_offset, (OT*)out, (OT*)out_lo, part_o, part_ml, H, KV, splits, n_active); \
+      (void)launch_decode(attn_decode_kernel<HD, KT, OT, EXTV, true>, grid, splits, DecCfg<HD, EXTV>::kRingBytes, s, q, (const KT*)pool_layer, page_table,       \
+                          max_pages, slot_row, len_or_pos, len_offset, (OT*)out, (OT*)out_lo, part_o, part_ml, H, KV, splits, n_active, new_tokens); \
     else                                                                                                             \
-      (void)launch_decode(attn_decode_kernel<HD, KT, OT, EXTV, false>, grid, 1, s, q, (const KT*)pool_layer, page_table,           \
-                          max_pages, slot_row, len_or_pos, len_offset, (OT*)out, (OT*)out_lo, part_o, part_ml, H, KV, splits, n_active); \
+      (void)launch_decode(attn_decode_kernel<HD, KT, OT, EXTV, false>, grid, 1, DecCfg<HD, EXTV>::kRingBytes, s, q, (const KT*)pool_layer, page_table,           \
+                          max_pages, slot_row, len_or_pos, len_offset, (OT*)out, (OT*)out_lo, part_o, part_ml, H, KV, splits, n_active, new_tokens); \
     if (splits > 1 && !clustered)                                                                                    \
       RSD_LAUNCH((attn_merge_kernel<HD, OT>), dim3(H, B), HD, 0, s, part_o, part_ml, slot_row, len_or_pos, len_offset, (OT*)out, \
                                                           (OT*)out_lo, H, splits, n_active);                         \

@@ -296,6 +296,27 @@ def test_decode_attention_against_definition(dtype, hd, H, KV):
             np.testing.assert_allclose(got[b, h], want, rtol=0, atol=tol)
 
 
+@pytest.mark.parametrize("hd,H,KV", [(128, 28, 4), (64, 4, 2)])
+@pytest.mark.parametrize("B,max_pages", [(1, 15), (2, 16), (1, 200), (70, 24), (3, 520)])
+def test_decode_attention_at_the_edges_of_the_split_rule(hd, H, KV, B, max_pages):
+    """One split, two, eight in a cluster, more than a cluster holds (merge launch), one per row, and splits of more pages
+    than the ring holds; the longest row fills its page table, others end at a page's edge, in its first token, or after
+    one token.  Tolerance: the query and the softmax weights are rounded to fp16 (2^-11 relative each)."""
+    rng = np.random.default_rng(B * 1000 + max_pages)
+    ctx = [max_pages * 16] + [int(c) for c in rng.integers(1, max_pages * 4, size=B - 1)]
+    if B > 2:
+        ctx[1], ctx[2] = 1, 33
+    pool, table, Ks, Vs = paged_kv(rng, B, KV, hd, ctx, torch.float16, max_pages)
+    q = rng.normal(size=(B, H, hd)).astype(np.float32)
+    got = rb.k_attn_decode(dev(q), pool, table, dev(np.array(ctx, np.int32)), KV).cpu().numpy()
+    for b in range(B):
+        for h in range(0, H, max(1, H // 4)):
+            g = h // (H // KV)
+            s = Ks[b][:, g].astype(np.float64) @ q[b, h].astype(np.float64) / np.sqrt(hd)
+            p = np.exp(s - s.max()); p /= p.sum()
+            np.testing.assert_allclose(got[b, h], p @ Vs[b][:, g].astype(np.float64), rtol=0, atol=2e-3)
+
+
 @pytest.mark.parametrize("dtype,hd,H,KV", [(torch.float32, 64, 4, 2), (torch.float32, 128, 3, 3), (torch.float16, 128, 18, 2),
                                           (torch.bfloat16, 64, 9, 1)])
 def test_generic_attention_at_the_edges_of_a_round_of_warps(dtype, hd, H, KV):
