@@ -238,8 +238,11 @@ decode_update_kernel(RowState st, int which, int phase, unsigned long long* best
   }
   const int n_ended = __syncthreads_count(ended);
   if (threadIdx.x == 0) {
-    st.n_active[0] -= n_ended;
+    const int left = st.n_active[0] - n_ended;
+    st.n_active[0] = left;
     st.iter[0] = iter + 1;
+    // the host follows the phase through this word of its own memory: (iterations done, rows left)
+    *(volatile unsigned long long*)st.progress = ((unsigned long long)(iter + 1) << 32) | (unsigned)left;
   }
 }
 
