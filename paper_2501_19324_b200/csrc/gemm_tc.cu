@@ -343,8 +343,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// Persistent form of the kernel above for the dense regime (more than 128 rows of x, split-precision operand, no
-// K split): a CTA per SM walks the output tiles (128 weight rows x 128 x rows, the same grouped order), the TMA
+// Persistent form of the kernel above for the dense regime (more than 128 rows of x, no K split) and, with pairs, for the
+// decode products of 65 to 128 rows that have more weight tiles than the chip has SMs (rs and n_active then as above; a
+// single row tile): a CTA per SM walks the output tiles (128 weight rows x 128 x rows, the same grouped order), the TMA
 // ring runs on from tile to tile, and the accumulator alternates between the two halves of tensor memory, so
 // the epilogue of one tile (TMEM -> registers -> global) overlaps the MMAs of the next instead of ending the CTA.
 // GU: gate/up tiles with the SwiGLU epilogue as above; the exchange buffers get shared memory of their own, since
@@ -359,7 +360,7 @@ template <bool SPLIT, bool GU> struct PersistCfg {
   // the exchange buffers of the plain gate/up tile (2 x 64 x 129 floats) leave room for three stages
   static constexpr int kStages = (GU && !SPLIT) ? 3 : 4;
   static constexpr int kABytes = kTileN * kTileK * 2, kBBytes = kMT * kTileK * 2, kStageBytes = kABytes + kBBytes;
-  static constexpr size_t kSmemBytes = 1024 + (size_t)kStages * kStageBytes + 256 + kXchBytes;
+  static constexpr size_t kSmemBytes = 1024 + (size_t)kStages * kStageBytes + 256 + 512 + kXchBytes;   // barriers, row scales
   static constexpr uint32_t kIdesc = TcCfg<256>::kIdesc;
   static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
 };
@@ -370,10 +371,14 @@ constexpr int kPersistEpiWarps = 8, kPersistThreads = 32 * (kPersistEpiWarps + 2
 template <bool GU, bool SPLIT>
 __global__ void __launch_bounds__(kPersistThreads, 1)
 gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
-                          const __grid_constant__ CUtensorMap tm_x_lo, float* __restrict__ Y, int M, int N, int K,
-                          int accumulate, int n_tiles_n, int n_tiles_m, int* __restrict__ err,
-                          __nv_bfloat16* __restrict__ act_hi, __nv_bfloat16* __restrict__ act_lo, int f16) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+                          const __grid_constant__ CUtensorMap tm_x_lo, float* Y, int M, int N, int K,
+                          int accumulate, int n_tiles_n, int n_tiles_m, int* err,
+                          __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, int f16, const int32_t* n_active, RowScale rs) {
+  RSD_PDL_TRIGGER();
+  if (n_active != nullptr && ld_cg(n_active) == 0) {      // every row of the decode phase has finished
+    RSD_PDL_WAIT();
+    return;
+  }
   using C = PersistCfg<SPLIT, GU>;
   // f16: both operands are fp16 (weights re-encoded at load, one fp16 activation operand); the MMA's operand-format
   // fields become 0 and a gate/up tile writes its activations as fp16.  Otherwise bf16 throughout.
@@ -386,7 +391,8 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
   uint64_t* acc_empty = acc_full + 2;
   uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
   volatile uint32_t* stop = tmem_slot + 1;
-  float* xch = (float*)(smem + (size_t)C::kStages * C::kStageBytes + 256);
+  float* row_scale = (float*)(smem + (size_t)C::kStages * C::kStageBytes + 256);   // [128]
+  float* xch = row_scale + 128;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int total_kb = (K + kTileK - 1) / kTileK, n_tiles = n_tiles_n * n_tiles_m;
   if (threadIdx.x == 0) {
@@ -400,7 +406,6 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   // tile t -> (row tile of x, tile of W): groups of eight row tiles, row tile fastest
   auto tile_of = [&](int t, int& tm, int& tn) {
     const int per_group = 8 * n_tiles_n, g0 = (t / per_group) * 8, rem = t % per_group, gsz = min(8, n_tiles_m - g0);
@@ -412,20 +417,32 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
   if (warp == kPersistEpiWarps) {
     if (lane == 0) {
       uint32_t it = 0;
+      auto load_w = [&](uint8_t* a, uint64_t* bar, int kb, int n0) {
+        tma_load_2d(a, &tm_w, bar, kb * kTileK, n0);
+        if (GU) tma_load_2d(a + C::kABytes / 2, &tm_w, bar, kb * kTileK, N + n0);
+      };
+      // the weight tiles of the first ring of stages go out before the predecessors have finished
+      uint32_t ahead = 0;
+      if (blockIdx.x < n_tiles) {
+        int tm, tn;
+        tile_of(blockIdx.x, tm, tn);
+        for (; ahead < (uint32_t)min(C::kStages, total_kb); ++ahead) {
+          mbar_expect_tx(&full[ahead], C::kStageBytes);
+          load_w(smem + (size_t)ahead * C::kStageBytes, &full[ahead], ahead, tn * (GU ? kTileN / 2 : kTileN));
+        }
+      }
+      RSD_PDL_WAIT();
       for (int t = blockIdx.x; t < n_tiles && !*stop; t += gridDim.x) {
         int tm, tn;
         tile_of(t, tm, tn);
         const int n0 = tn * (GU ? kTileN / 2 : kTileN), m0 = tm * C::kRows;
         for (int kb = 0; kb < total_kb; ++kb, ++it) {
           const uint32_t s = it % C::kStages;
-          if (!mbar_wait(&empty[s], ((it / C::kStages) & 1u) ^ 1u) || *stop) { fail(); break; }
           uint8_t* a = smem + (size_t)s * C::kStageBytes;
-          mbar_expect_tx(&full[s], C::kStageBytes);
-          if (GU) {
-            tma_load_2d(a, &tm_w, &full[s], kb * kTileK, n0);
-            tma_load_2d(a + C::kABytes / 2, &tm_w, &full[s], kb * kTileK, N + n0);
-          } else {
-            tma_load_2d(a, &tm_w, &full[s], kb * kTileK, n0);
+          if (it >= ahead) {
+            if (!mbar_wait(&empty[s], ((it / C::kStages) & 1u) ^ 1u) || *stop) { fail(); break; }
+            mbar_expect_tx(&full[s], C::kStageBytes);
+            load_w(a, &full[s], kb, n0);
           }
           tma_load_2d(a + C::kABytes, &tm_x, &full[s], kb * kTileK, m0);
           if (SPLIT) tma_load_2d(a + C::kABytes + C::kRows * kTileK * 2, &tm_x_lo, &full[s], kb * kTileK, m0);
@@ -468,6 +485,20 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
     const int quarter = warp & 3, col0 = (warp >> 2) * 16;
     constexpr int kColStep = 16 * (kPersistEpiWarps / 4);
     uint32_t n_acc = 0;
+    RSD_PDL_WAIT();                            // y, the activations' sums of squares and act belong to earlier kernels until now
+    const bool scaled = SPLIT && rs.ssq != nullptr;
+    if (scaled) {
+      // RMSNorm denominators of the single row tile, two threads per row
+      const int r = threadIdx.x >> 1, sub = threadIdx.x & 1;
+      float sum = 0.f;
+      if (r < M) {
+#pragma unroll 8
+        for (int c = sub; c < rs.n_chunks; c += 2) sum += rs.ssq[(size_t)r * rs.n_chunks + c];
+      }
+      sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 1);
+      if (sub == 0) row_scale[r] = rsqrtf(sum * rs.inv_d + rs.eps);
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * kPersistEpiWarps) : "memory");
+    }
     for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++n_acc) {
       int tm, tn;
       tile_of(t, tm, tn);
@@ -490,6 +521,10 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
               tmem_ld16(taddr + C::kRows + c, w);
 #pragma unroll
               for (int j = 0; j < 16; ++j) v[j] += w[j];
+            }
+            if (scaled) {
+#pragma unroll
+              for (int j = 0; j < 16; ++j) v[j] *= row_scale[(c + j) & 127];
             }
             if (n < N) {
               // all sixteen old values first, then the stores (see the one-tile kernel's epilogue)
@@ -548,7 +583,8 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
             for (int j = 0; j < 16; ++j) {
               const int r = own0 + c + j;
               if (r < m_valid) {
-                const float mine = v[j], other = recv[c + j];
+                const float sc = scaled ? row_scale[r & 127] : 1.f;
+                const float mine = v[j] * sc, other = recv[c + j] * sc;
                 const float gate = is_gate ? mine : other, up = is_gate ? other : mine;
                 const float a = gate / (1.f + expf(-gate)) * up;
                 const size_t o = (size_t)(m0 + r) * N + n0 + l;
@@ -684,9 +720,11 @@ TcPlan plan_tc(int M, int N, int K, bool split_operand) {
   const int tiles = p.n_tiles * p.m_tiles;
   const int total_kb = (K + kTileK - 1) / kTileK;
   int splits = 1;
-  if (tiles < 148 && tiles <= kMaxSplitTiles && p.rows <= 64 && N % 4 == 0) {
-    // aim at one wave of two CTAs per SM, each with at least two k-blocks
-    splits = std::max(1, (2 * 148) / tiles);
+  if (tiles < 148 && tiles <= kMaxSplitTiles && N % 4 == 0 && (p.rows <= 64 || (split_operand && M <= 128))) {
+    // aim at one wave of two CTAs per SM (one, where a tile takes the SM alone), each with at least two k-blocks.
+    // 65 to 128 rows with pairs are the decode passes of large batches: without the split the 12 tiles of a
+    // 1536 x 8960 product leave 136 SMs idle (58 us at 128 rows; 11 us with 12 splits).
+    splits = std::max(1, (p.rows <= 64 ? 2 * 148 : 148) / tiles);
     splits = std::min(splits, std::max(1, total_kb / 2));
     splits = std::min(splits, kMaxSplitCtas / tiles);
     splits = std::max(splits, 1);
@@ -803,11 +841,11 @@ static int sm_count() {
   return n;
 }
 
-// Dense regime (M > 128 rows, no K split, no row scale, no idle flag): persistent kernel.
+// Dense regime (M > 128 rows, no K split, no row scale, no idle flag) and wide decode products: persistent kernel.
 template <bool GU, bool SPLIT>
 static cudaError_t launch_persistent(const CUtensorMap& tw, const CUtensorMap& tx, const CUtensorMap& txl, float* y, int M, int N,
                                      int K, int accumulate, int* err, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, cudaStream_t s,
-                                     int f16 = 0) {
+                                     int f16 = 0, const int32_t* n_active = nullptr, RowScale rs = RowScale()) {
   using C = PersistCfg<SPLIT, GU>;
   constexpr size_t smem = C::kSmemBytes;
   static bool configured = false;
@@ -821,9 +859,13 @@ static cudaError_t launch_persistent(const CUtensorMap& tw, const CUtensorMap& t
   const int tiles_n = GU ? N / 64 : (N + kTileN - 1) / kTileN, tiles_m = (M + C::kRows - 1) / C::kRows;
   const int grid = std::min(tiles_n * tiles_m, n_sm);
   RSD_LAUNCH((gemm_tc_persistent_kernel<GU, SPLIT>), grid, kPersistThreads, smem, s, tw, tx, txl, y, M, N, K, accumulate, tiles_n,
-             tiles_m, err, act_hi, act_lo, f16);
+             tiles_m, err, act_hi, act_lo, f16, n_active, rs);
   return launched(1);
 }
+
+// 65 to 128 rows with pairs take an SM per tile: with more tiles than SMs the persistent kernel hides the epilogues and
+// evens out the last wave (the 1187 tiles of a 151936-row head at 128 rows: 140 us one CTA per tile, 93 us persistent).
+static bool wide_decode(int M, int n_tiles) { return M > 64 && M <= 128 && n_tiles > 148; }
 
 template <int MT, bool DEEP>
 static cudaError_t launch_gu_mt(const CUtensorMap& tw, const CUtensorMap& tx, const CUtensorMap& txl, int M, int F, int K, int rows,
@@ -872,6 +914,7 @@ cudaError_t launch_gemm_gu(const void* Wgu, const void* x, const void* x_lo, voi
     return launch_persistent<true, true>(tw, tx, txl, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act_hi, (__nv_bfloat16*)act_lo, s);
   auto* hi = (__nv_bfloat16*)act_hi;
   auto* lo = (__nv_bfloat16*)act_lo;
+  if (wide_decode(M, F / 64)) return launch_persistent<true, true>(tw, tx, txl, nullptr, M, F, K, 0, err, hi, lo, s, 0, n_active, rs);
   // fewer than ~1.5 CTAs per SM: one CTA per SM with a deep ring streams faster than a thin second wave
   const bool deep = (F / 64) * ((M + rows - 1) / rows) <= 222;
   switch (rows) {
@@ -887,11 +930,11 @@ cudaError_t launch_gemm_gu(const void* Wgu, const void* x, const void* x_lo, voi
 // flag region of 256 bytes, then split-K partial tiles.
 size_t gemm_scratch_bytes(int M) {
   const int rows = pick_rows(M, false);
-  const size_t part = rows <= 64 ? (size_t)kMaxSplitCtas * kTileN * std::min(64, std::max(rows, 16)) * 4 : 0;
+  const size_t part = rows <= 128 ? (size_t)kMaxSplitCtas * kTileN * std::min(64, std::max(rows, 16)) * 4 : 0;
   return kCounterBytes + 256 + part;
 }
 
-// Enough for any M (split-K is only used with tiles of at most 64 rows of x).
+// Enough for any M (split-K is only used with up to 128 rows of x, and beyond 64 with half as many CTAs).
 size_t gemm_scratch_bytes_any() { return gemm_scratch_bytes(64); }
 
 const float* gemm_partials(const void* scratch) { return (const float*)((const char*)scratch + kCounterBytes + 256); }
@@ -920,6 +963,8 @@ cudaError_t launch_gemm_tc(const void* W, const void* x, const void* x_lo, float
     if (split_operand) return launch_persistent<false, true>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s);
     return launch_persistent<false, false>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s);
   }
+  if (split_operand && p.splits == 1 && wide_decode(M, p.n_tiles))
+    return launch_persistent<false, true>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s, 0, n_active, rs);
 #define RSD_TC(MT, SP) return launch_mt<MT, SP>(tw, tx, txl, y, M, N, K, accumulate, p, partials, err, n_active, defer, rs, s)
   // a grid of at most one CTA per SM: the deep ring (a lone CTA needs more bytes in flight to keep its stream going)
   if (split_operand && p.n_tiles * p.m_tiles * p.splits <= 148 && p.mt <= 128) {

@@ -446,7 +446,8 @@ def test_dense_gemm_on_fp16_operands(M, N, K):
 
 
 @pytest.mark.parametrize("M,F,K", [(1, 64, 64), (5, 192, 512), (32, 1408, 512), (33, 128, 520), (70, 2048, 768),
-                                   (129, 704, 1408), (300, 320, 256), (32, 8960, 1536), (200, 128, 520), (2100, 640, 128)])
+                                   (129, 704, 1408), (300, 320, 256), (32, 8960, 1536), (200, 128, 520), (2100, 640, 128),
+                                   (65, 9536, 192), (128, 9472, 520)])
 def test_gate_up_gemm_with_swiglu_epilogue(M, F, K):
     """Gate/up projection with SwiGLU inside the GEMM epilogue (tile = 64 gate rows + the 64 matching up rows):
     against matmul + silu(g) * u written out in fp64.  Ragged M (all three tile heights and several x tiles), F of
@@ -469,6 +470,27 @@ def test_gate_up_gemm_with_swiglu_epilogue(M, F, K):
         np.abs(a_hi.float().cpu().numpy() - got).max() <= 2 ** -8 * scale
     again_hi, again_lo = rb.k_gemm_gu(dev(W, torch.bfloat16), hi, lo)
     assert torch.equal(again_hi, a_hi) and torch.equal(again_lo, a_lo)
+
+
+@pytest.mark.parametrize("M,N,K", [(65, 128, 64), (65, 1536, 8960), (128, 640, 520), (96, 18816, 128), (65, 18945, 192), (128, 19072, 520)])
+def test_paired_gemm_of_65_to_128_rows(M, N, K):
+    """The decode products of large batches: K split over the SMs (the smallest, a long K with many splits, a K tail), a
+    weight matrix of 147 tiles (one wave) and of more than 148 (persistent kernel, ragged last tile).  fp32 sums of K
+    products of N(0, 1) activations and N(0, 0.02) weights: about 2^-24 * K * 0.02, bounded as in the tests above."""
+    rng = np.random.default_rng(M * 11 + N)
+    W = ri.cpu_tensor(2, 9, N, K, True)
+    xf = dev(rng.normal(size=(M, K)).astype(np.float32))
+    hi = xf.to(torch.bfloat16)
+    lo = (xf - hi.float()).to(torch.bfloat16)
+    want = oracle.matmul(W, (hi.float() + lo.float()).cpu().numpy())
+    Wd = dev(W, torch.bfloat16)
+    got = rb.k_gemm(Wd, hi, impl=2, x_lo=lo).cpu().numpy()
+    tol = 3e-5 * np.sqrt(K)
+    np.testing.assert_allclose(got, want, rtol=0, atol=tol)
+    assert np.array_equal(rb.k_gemm(Wd, hi, impl=2, x_lo=lo).cpu().numpy(), got)
+    y0 = rng.normal(size=(M, N)).astype(np.float32)
+    acc = rb.k_gemm(Wd, hi, y=dev(y0), accumulate=True, impl=2, x_lo=lo).cpu().numpy()
+    np.testing.assert_allclose(acc, want + y0, rtol=0, atol=tol)
 
 
 def test_bounded_wait_runs_out_and_the_kernel_leaves_cleanly():

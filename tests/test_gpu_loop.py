@@ -436,3 +436,18 @@ def test_device_outputs_and_target_step_rewards():
             assert np.isnan(got).all()                                   # nothing the target wrote has been scored yet
     assert seen > 0
     a.close(); b.close()
+
+
+def test_batches_of_more_than_64_rows_and_wide_heads():
+    """65 to 128 rows: K-split products over the whole machine, and the persistent kernel for the gate/up and the head with
+    more weight tiles than SMs (RMSNorm denominators and idle flag included), against the oracle."""
+    from dataclasses import replace
+    d, t = (replace(s, vocab=19300, d_ffn=9600) for s in (MINI[0], MINI[2]))
+    prompts = ri.prompts(93, 100, 2, 6, d.vocab)
+    base = dict(max_step_tokens=2, max_steps=2, max_seq_tokens=16, step_end_id=3, step_end_mod=5, temperature=0.7, seed=9)
+    eng, loop = build_pair((d, d, t), bf16=True, prompts=prompts, loop_kwargs=base)
+    stats = {}
+    parity_step(eng, loop, 2.0, stats=stats, **TOL16)          # every row is rejected: the target decodes 100 rows too
+    assert stats["tokens_compared"] > 0.5 * stats["tokens"]
+    compare_counters(eng, loop)
+    eng.close()
