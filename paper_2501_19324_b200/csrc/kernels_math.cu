@@ -39,6 +39,44 @@ cudaError_t launch_embed(int dtype, const void* embed, PassView p, float* x, int
 // ---------------------------------------------------------------------------------------------
 // RMSNorm: out = x * gain / sqrt(mean(x^2) + eps), one block per token, x kept in registers
 // ---------------------------------------------------------------------------------------------
+// Bound by DRAM in the dense passes (8192 x 3584: 117 MB in, 59 MB out).
+constexpr int kNormVecs = 4;
+
+// The roundings spelled out: the sum does not depend on what the compiler would fuse.
+__device__ __forceinline__ float sum_squares(float4 v) { return fmaf(v.w, v.w, fmaf(v.z, v.z, fmaf(v.x, v.x, __fmul_rn(v.y, v.y)))); }
+
+// Four elements of a residual row; K-split partial sums that the producing GEMM left are folded in (and x written back).
+__device__ __forceinline__ float4 norm_load(float* xr, const float* partials, int splits, size_t row0, size_t stride, int i) {
+  float4 v = *reinterpret_cast<const float4*>(xr + i);
+  if (splits > 1) {
+    int sidx = 0;
+    for (; sidx + 8 <= splits; sidx += 8) {
+      float4 a[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) a[u] = ld_cg(reinterpret_cast<const float4*>(partials + (size_t)(sidx + u) * stride + row0 + i));
+#pragma unroll
+      for (int u = 0; u < 8; ++u) { v.x += a[u].x; v.y += a[u].y; v.z += a[u].z; v.w += a[u].w; }
+    }
+    for (; sidx < splits; ++sidx) {
+      const float4 a = ld_cg(reinterpret_cast<const float4*>(partials + (size_t)sidx * stride + row0 + i));
+      v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
+    }
+    *reinterpret_cast<float4*>(xr + i) = v;
+  }
+  return v;
+}
+
+template <typename OT, typename GT>
+__device__ __forceinline__ void norm_store(OT* out, OT* out_lo, size_t o, float4 v, float inv, const GT* gain) {
+  const float y[4] = {v.x * inv * to_f32(gain[0]), v.y * inv * to_f32(gain[1]), v.z * inv * to_f32(gain[2]), v.w * inv * to_f32(gain[3])};
+  if (((uintptr_t)out & 15) == 0) {
+    store_operand4<OT>(out, out_lo, o, y);
+  } else {                                     // a caller's buffer may start anywhere
+#pragma unroll
+    for (int k = 0; k < 4; ++k) store_operand<OT>(out, out_lo, o + k, y[k]);
+  }
+}
+
 template <typename OT, typename GT>
 __global__ void rmsnorm_kernel(float* x, const GT* __restrict__ gain, OT* out, OT* out_lo, int d, float eps,
                                const int32_t* src, const int32_t* n_active, const float* partials, int splits, int T) {
@@ -52,36 +90,32 @@ __global__ void rmsnorm_kernel(float* x, const GT* __restrict__ gain, OT* out, O
   }
   float* xr = x + (size_t)st * d;
   float ss = 0.f;
-  for (int i = threadIdx.x * 4; i < d; i += blockDim.x * 4) {
-    float4 v = *reinterpret_cast<const float4*>(xr + i);
-    if (splits > 1) {
-      // the producing GEMM left K-split partial sums: fold them into the residual stream here
-      int sidx = 0;
-      for (; sidx + 8 <= splits; sidx += 8) {
-        float4 a[8];
+  // the row stays in registers between the two halves (up to kNormVecs float4 a thread; wider rows are read again)
+  float4 keep[kNormVecs];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) a[u] = ld_cg(reinterpret_cast<const float4*>(partials + ((size_t)(sidx + u) * T + st) * d + i));
+  for (int k = 0; k < kNormVecs; ++k) {
+    const int i = (k * blockDim.x + threadIdx.x) * 4;
+    if (i < d) keep[k] = norm_load(xr, partials, splits, (size_t)st * d, (size_t)T * d, i);
+  }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) { v.x += a[u].x; v.y += a[u].y; v.z += a[u].z; v.w += a[u].w; }
-      }
-      for (; sidx < splits; ++sidx) {
-        const float4 a = ld_cg(reinterpret_cast<const float4*>(partials + ((size_t)sidx * T + st) * d + i));
-        v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
-      }
-      *reinterpret_cast<float4*>(xr + i) = v;
-    }
-    ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+  for (int k = 0; k < kNormVecs; ++k) {
+    const float4 v = keep[k];
+    if ((k * (int)blockDim.x + (int)threadIdx.x) * 4 < d) ss += sum_squares(v);
+  }
+  for (int i = (kNormVecs * blockDim.x + threadIdx.x) * 4; i < d; i += blockDim.x * 4) {
+    const float4 v = norm_load(xr, partials, splits, (size_t)st * d, (size_t)T * d, i);
+    ss += sum_squares(v);
   }
   ss = block_sum(ss, red);
   const float inv = rsqrtf(ss / (float)d + eps);
   const size_t o = (size_t)t * d;
-  for (int i = threadIdx.x * 4; i < d; i += blockDim.x * 4) {
-    float4 v = *reinterpret_cast<const float4*>(xr + i);
-    store_operand<OT>(out, out_lo, o + i, v.x * inv * to_f32(gain[i]));
-    store_operand<OT>(out, out_lo, o + i + 1, v.y * inv * to_f32(gain[i + 1]));
-    store_operand<OT>(out, out_lo, o + i + 2, v.z * inv * to_f32(gain[i + 2]));
-    store_operand<OT>(out, out_lo, o + i + 3, v.w * inv * to_f32(gain[i + 3]));
+#pragma unroll
+  for (int k = 0; k < kNormVecs; ++k) {
+    const int i = (k * blockDim.x + threadIdx.x) * 4;
+    if (i < d) norm_store<OT>(out, out_lo, o + i, keep[k], inv, gain + i);
   }
+  for (int i = (kNormVecs * blockDim.x + threadIdx.x) * 4; i < d; i += blockDim.x * 4)
+    norm_store<OT>(out, out_lo, o + i, *reinterpret_cast<const float4*>(xr + i), inv, gain + i);
 }
 
 // bf16 -> fp16, element by element (n a multiple of 8: weight matrices are).
@@ -429,7 +463,21 @@ rope_kv_kernel(const float* qkv, const float* partials, int splits, PassView p, 
 // data loads of all entries go out together instead of after a chain of three dependent loads per (token, head)
 // block; and when the entries are consecutive positions of one row inside one page (the rule in a long pass), a thread
 // writes the eight transposed value elements of a (head, dim) as ONE 16-byte store instead of eight 2-byte ones.
+// Bound by DRAM: a token's fp32 qkv row in, its fp32 queries and 16-bit keys and values out.
 constexpr int kRopeTokens = 8;
+
+// Four neighbouring cache elements (and their low halves) as one store.
+template <typename KT> __device__ __forceinline__ void store_cache4(KT* hi, KT* lo, const float* v) {
+  __align__(16) KT h[4], l[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { h[i] = from_f32<KT>(v[i]); l[i] = from_f32<KT>(v[i] - to_f32(h[i])); }
+  if (sizeof(KT) == 2) {
+    *reinterpret_cast<uint2*>(hi) = *reinterpret_cast<const uint2*>(h);
+    if (lo != nullptr) *reinterpret_cast<uint2*>(lo) = *reinterpret_cast<const uint2*>(l);
+  } else {
+    *reinterpret_cast<uint4*>(hi) = *reinterpret_cast<const uint4*>(h);
+  }
+}
 
 template <typename KT>
 __global__ void __launch_bounds__(256)
@@ -461,27 +509,32 @@ rope_kv_long_kernel(const float* __restrict__ qkv, PassView p, float* __restrict
   const int half = hd / 2;
   const int width = (H + 2 * KV) * hd;
   const size_t block = (size_t)KV * kPageTokens * hd;
-  const int n_rot = (H + KV) * half;            // rotated pairs of one token
-  // queries and keys: one (token, head, pair) per step
-  for (int idx = threadIdx.x; idx < n_tok * n_rot; idx += blockDim.x) {
-    const int tk = idx / n_rot, e = idx % n_rot;
-    if (s_row[tk] < 0) continue;
-    const int head = e / half, i = e % half;
-    const int t = t0 + tk, pos = s_pos[tk];
-    const float a = qkv[(size_t)t * width + head * hd + i], b = qkv[(size_t)t * width + head * hd + i + half];
-    const float2 c = rope[(size_t)pos * half + i];
-    const float ra = rotate_lo(a, b, c), rb = rotate_hi(a, b, c);
-    if (head < H) {
-      q_out[(size_t)t * H * hd + head * hd + i] = ra;
-      q_out[(size_t)t * H * hd + head * hd + i + half] = rb;
-    } else {
-      KT* k = pool + (size_t)s_page[tk] * pf * block + ((size_t)(head - H) * kPageTokens + pos % kPageTokens) * hd;
-      const KT ka = from_f32<KT>(ra), kb2 = from_f32<KT>(rb);
-      k[i] = ka;
-      k[i + half] = kb2;
-      if (pf == 4) {
-        k[2 * block + i] = from_f32<KT>(ra - to_f32(ka));
-        k[2 * block + i + half] = from_f32<KT>(rb - to_f32(kb2));
+  // queries and keys: a thread takes four neighbouring pairs of a head for all tokens of the block, all their loads in
+  // flight together
+  const int per_head = half / 4;                // 8 or 16
+  for (int e = threadIdx.x; e < (H + KV) * per_head; e += blockDim.x) {
+    const int head = e / per_head, i = (e % per_head) * 4;
+    const float* src = qkv + (size_t)t0 * width + head * hd + i;
+#pragma unroll 4
+    for (int tk = 0; tk < n_tok; ++tk) {
+      if (s_row[tk] < 0) continue;
+      const float4 a = *reinterpret_cast<const float4*>(src + (size_t)tk * width);
+      const float4 b = *reinterpret_cast<const float4*>(src + (size_t)tk * width + half);
+      const float4 c01 = *reinterpret_cast<const float4*>(rope + (size_t)s_pos[tk] * half + i);
+      const float4 c23 = *reinterpret_cast<const float4*>(rope + (size_t)s_pos[tk] * half + i + 2);
+      const float2 c[4] = {make_float2(c01.x, c01.y), make_float2(c01.z, c01.w), make_float2(c23.x, c23.y), make_float2(c23.z, c23.w)};
+      const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+      float ra[4], rb[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) { ra[k] = rotate_lo(av[k], bv[k], c[k]); rb[k] = rotate_hi(av[k], bv[k], c[k]); }
+      if (head < H) {
+        float* q = q_out + ((size_t)(t0 + tk) * H + head) * hd + i;
+        *reinterpret_cast<float4*>(q) = make_float4(ra[0], ra[1], ra[2], ra[3]);
+        *reinterpret_cast<float4*>(q + half) = make_float4(rb[0], rb[1], rb[2], rb[3]);
+      } else {
+        KT* k = pool + (size_t)s_page[tk] * pf * block + ((size_t)(head - H) * kPageTokens + s_pos[tk] % kPageTokens) * hd + i;
+        store_cache4<KT>(k, pf == 4 ? k + 2 * block : nullptr, ra);
+        store_cache4<KT>(k + half, pf == 4 ? k + 2 * block + half : nullptr, rb);
       }
     }
   }
@@ -730,35 +783,123 @@ __device__ __forceinline__ unsigned long long pack_best(float sc, int id) {
 
 // Grid (slots, chunks): every block scans one chunk of the vocabulary and folds its best candidate
 // into best[slot] with an atomic maximum (order-independent, hence deterministic).
+// Bound by the ALUs: ten Philox rounds per four ids and two logarithms per id.  So the scores are first taken with fast
+// logarithms, and only ids within kScoreMargin of the block's best get the exact ones; and as the noise lies in
+// (-2.82, 16.64), four ids whose logits stay 20 below the block's largest draw none at all.  The winner is the same.
+// (Gumbel-max of 151936 ids x 128 rows, one logit 43 above the rest: 87 us with exact noise for all.)
+constexpr int kSampleGroups = 4;            // groups of four ids a thread holds; the launcher cuts the chunks accordingly
+constexpr float kScoreMargin = 1e-3f;       // the fast score errs by less than 1e-4 (see fast_gumbel)
+constexpr float kNoiseRange = 20.f;
+
+// -log(-log u) for u = (2k + 1) / 2^24.  Near 1, where the large values come from, -log u is its series in 1 - u (exact
+// in fp32; 1 - u < 2^-6: three terms err by 1e-6 relative); elsewhere __logf errs by 2^-21.4 on -log u > 2^-6, that is
+// 2.3e-5 relative, and so much in the outer logarithm, whose own error is 3 ulp of at most 17.
+__device__ __forceinline__ float fast_gumbel(float u) {
+  const float d = 1.f - u;
+  const float y = d < 0.015625f ? d * (1.f + d * (0.5f + d * 0.33333333f)) : -__logf(u);
+  return -__logf(y);
+}
+
+__device__ __forceinline__ float block_max(float v, float* smem) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  __syncthreads();
+  if (lane == 0) smem[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = lane < nw ? smem[lane] : -INFINITY;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+  return v;
+}
+
 __global__ void __launch_bounds__(1024) sample_kernel(SampleArgs a) {
-  RSD_PDL_SYNC_UNLESS_IDLE(a.n_active);
+  RSD_PDL_TRIGGER();
+  if (a.n_active == nullptr) RSD_PDL_WAIT();   // a decode pass's lists may be read ahead of the wait, others not
+  const bool idle = a.n_active != nullptr && ld_cg(a.n_active) == 0;
   __shared__ float s_sc[32];
   __shared__ int s_ix[32];
   const int slot = blockIdx.x;
-  const int row = a.slot_row[slot];
-  if (row < 0) return;
+  const int row = ld_cg(a.slot_row + slot);
+  const uint32_t position = (uint32_t)(ld_cg(a.slot_pos + slot) + 1);
+  RSD_PDL_WAIT();
+  if (idle || row < 0) return;
   const float* lg = a.logits + (size_t)slot * a.V;
-  const uint32_t position = (uint32_t)(a.slot_pos[slot] + 1);
   const uint2 key = make_uint2((uint32_t)(a.seed & 0xFFFFFFFFull), (uint32_t)(a.seed >> 32));
-  const float inv_t = a.temperature > 0.f ? 1.f / a.temperature : 1.f;
+  const bool noisy = a.temperature > 0.f;
+  const float inv_t = noisy ? 1.f / a.temperature : 1.f;
   float bs = -INFINITY;
   int bi = 0x7FFFFFFF;
   const int n_v4 = (a.v_limit + 3) / 4;
   const int per_chunk = (n_v4 + gridDim.y - 1) / gridDim.y;
-  const int v4_end = min(n_v4, (int)(blockIdx.y + 1) * per_chunk);
-  for (int v4 = blockIdx.y * per_chunk + threadIdx.x; v4 < v4_end; v4 += blockDim.x) {
-    float g[4] = {0.f, 0.f, 0.f, 0.f};
-    if (a.temperature > 0.f) {
-      const uint4 r = philox4x32_10(make_uint4((uint32_t)v4, position, (uint32_t)row, (uint32_t)a.model_id), key);
-      const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+  const int v4_0 = blockIdx.y * per_chunk + threadIdx.x, v4_end = min(n_v4, (int)(blockIdx.y + 1) * per_chunk);
+  const bool vec = (a.V & 3) == 0 && ((uintptr_t)a.logits & 15) == 0;
+  float x[kSampleGroups][4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) g[j] = -logf(-logf(uniform_from_bits(w[j])));
-    }
+  for (int k = 0; k < kSampleGroups; ++k) {
+    const int v4 = v4_0 + k * blockDim.x;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int v = v4 * 4 + j;
-      if (v < a.v_limit) better(bs, bi, lg[v] * inv_t + g[j], v);
+    for (int j = 0; j < 4; ++j) x[k][j] = -INFINITY;
+    if (v4 < v4_end) {
+      if (vec && v4 * 4 + 3 < a.v_limit) {
+        const float4 f = *reinterpret_cast<const float4*>(lg + v4 * 4);
+        x[k][0] = f.x; x[k][1] = f.y; x[k][2] = f.z; x[k][3] = f.w;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (v4 * 4 + j < a.v_limit) x[k][j] = lg[v4 * 4 + j];
+      }
     }
+  }
+  auto block_of = [&](int v4) { return philox4x32_10(make_uint4((uint32_t)v4, position, (uint32_t)row, (uint32_t)a.model_id), key); };
+  if (!noisy) {
+#pragma unroll
+    for (int k = 0; k < kSampleGroups; ++k) {
+      const int v4 = v4_0 + k * blockDim.x;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (v4 < v4_end && v4 * 4 + j < a.v_limit) better(bs, bi, x[k][j], v4 * 4 + j);
+    }
+  } else {
+    float top[kSampleGroups], top_all = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < kSampleGroups; ++k) {
+      top[k] = fmaxf(fmaxf(x[k][0], x[k][1]), fmaxf(x[k][2], x[k][3])) * inv_t;
+      top_all = fmaxf(top_all, top[k]);
+    }
+    const float floor_ = block_max(top_all, s_sc) - kNoiseRange;
+    float s_max = -INFINITY;
+    float sc[kSampleGroups][4];
+#pragma unroll
+    for (int k = 0; k < kSampleGroups; ++k) {
+      const int v4 = v4_0 + k * blockDim.x;
+      const bool on = v4 < v4_end && !(top[k] < floor_);
+      uint32_t w[4] = {0, 0, 0, 0};
+      if (on) {
+        const uint4 r = block_of(v4);
+        w[0] = r.x; w[1] = r.y; w[2] = r.z; w[3] = r.w;
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        sc[k][j] = on && v4 * 4 + j < a.v_limit ? fmaf(x[k][j], inv_t, fast_gumbel(uniform_from_bits(w[j]))) : __int_as_float(0x7FC00000);
+        s_max = fmaxf(s_max, sc[k][j]);        // NaN (an id out of the race) never wins
+      }
+    }
+    s_max = block_max(s_max, s_sc);
+    const float need = s_max == INFINITY ? s_max : s_max - (kScoreMargin + fabsf(s_max) * 1e-6f);
+#pragma unroll
+    for (int k = 0; k < kSampleGroups; ++k) {
+      const bool any = sc[k][0] >= need || sc[k][1] >= need || sc[k][2] >= need || sc[k][3] >= need;
+      if (any) {
+        const int v4 = v4_0 + k * blockDim.x;
+        const uint4 r = block_of(v4);
+        const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (sc[k][j] >= need) better(bs, bi, fmaf(x[k][j], inv_t, -logf(-logf(uniform_from_bits(w[j])))), v4 * 4 + j);
+      }
+    }
+    __syncthreads();                           // s_sc is used again below
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -792,14 +933,18 @@ __global__ void sample_finalize_kernel(unsigned long long* best, const int32_t* 
   best[i] = 0ull;
 }
 
-int sample_chunks(int v_limit) { return v_limit >= 65536 ? 16 : (v_limit >= 8192 ? 4 : 1); }
+// Blocks per slot: enough of them to fill the machine at small batches, and no more ids per block than its threads hold.
+int sample_chunks(int v_limit, int threads) {
+  const int want = v_limit >= 65536 ? 16 : (v_limit >= 8192 ? 4 : 1), per_block = threads * kSampleGroups * 4;
+  return std::max(want, (v_limit + per_block - 1) / per_block);
+}
 
 // Leaves the winners packed in a.best (which must be zero on entry); when a.token is given a second
 // kernel unpacks them into a.token and clears a.best.
 cudaError_t launch_sample(const SampleArgs& a, cudaStream_t s) {
   if (a.n_slots <= 0) return cudaSuccess;
   const int threads = a.v_limit >= 16384 ? 1024 : 256;
-  RSD_LAUNCH((sample_kernel), dim3(a.n_slots, sample_chunks(a.v_limit)), threads, 0, s, a);
+  RSD_LAUNCH((sample_kernel), dim3(a.n_slots, sample_chunks(a.v_limit, threads)), threads, 0, s, a);
   if (a.token == nullptr) return launched(1);
   RSD_LAUNCH((sample_finalize_kernel), (a.n_slots + 255) / 256, 256, 0, s, a.best, a.slot_row, a.token, a.n_slots);
   return launched(2);

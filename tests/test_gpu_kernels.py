@@ -161,6 +161,32 @@ def test_sampling_matches_oracle(temperature):
         assert got[0] == 4
 
 
+@pytest.mark.parametrize("v_limit,scale,shift", [(1, 1.0, 0.0), (4095, 1.0, 0.0), (4097, 4.0, 0.0), (16385, 30.0, 0.0), (65535, 0.8, 0.0),
+                                                 (65537, 8.0, -50.0), (262145, 1.0, 2000.0)])
+def test_sampling_shortcuts_keep_the_winner(v_limit, scale, shift):
+    """Flat and peaked logits, a few large ones far above the rest, ids that the noise range rules out, large offsets (where
+    one ulp of a score exceeds the shortcut's margin), infinite and NaN logits; one block per slot and many, full and
+    ragged chunks, an odd row length (no 16-byte loads).  Against fp64 scores with the oracle's noise: the winner
+    must be the oracle's unless its two best scores are within a few fp32 roundings of each other."""
+    rng = np.random.default_rng(v_limit)
+    B, V = 6, v_limit + 3
+    logits = (rng.normal(size=(B, V)) * scale + shift).astype(np.float32)
+    logits[1, rng.integers(0, v_limit, size=3)] += 25.0
+    logits[2] = shift
+    logits[3, :v_limit // 2] = -np.inf
+    logits[4, rng.integers(0, v_limit, size=5)] = np.nan
+    logits[4, v_limit - 1] = shift
+    logits[:, v_limit:] = 1e9                                  # beyond the vocabulary limit: never chosen
+    row, pos = np.arange(B, dtype=np.int32), np.arange(B, dtype=np.int32) * 37 + 5
+    for temperature in (0.7, 0.0):
+        got = rb.k_sample(dev(logits), v_limit, temperature, 77, 1, dev(row), dev(pos)).cpu().numpy()
+        for b in range(B):
+            fin = np.where(np.isnan(logits[b, :v_limit]), -np.inf, logits[b, :v_limit].astype(np.float64))
+            want, margin = oracle.sample(np.concatenate([fin, np.full(3, -np.inf)]), v_limit, temperature, 77, 1, row[b], pos[b] + 1)
+            if v_limit == 1 or temperature == 0.0 or margin > 4e-6 * (abs(shift) + 30 * scale) / 0.7:
+                assert got[b] == want, (b, temperature, got[b], want, margin)
+
+
 def test_gate_compaction_all_masks_and_large():
     """Brute force (a serial loop over the rows) against the ballot / prefix path: EVERY accept mask of 12 rows, one
     call per mask as the step loop calls it, and every mask of 16 rows laid end to end in one call of 2^20 rows."""
