@@ -368,6 +368,112 @@ template <bool SPLIT, bool GU> struct PersistCfg {
 // warps 0..7: epilogue, warp 8: TMA producer, warp 9: MMA issuer and owner of the tensor-memory allocation
 constexpr int kPersistEpiWarps = 8, kPersistThreads = 32 * (kPersistEpiWarps + 2);
 
+// One output tile out of tensor memory, by the eight epilogue warps of a persistent kernel: warp w reads the lanes of
+// quarter w % 4 (the hardware's rule), the two warps of a quarter take alternate groups of sixteen columns, which halves
+// the time an accumulator stays occupied.  release() hands the accumulator back; it is called by one lane of every warp.
+template <bool GU, bool SPLIT, typename Release>
+__device__ __forceinline__ void persist_epilogue(uint32_t taddr, bool ok, int quarter, int lane, int col0, int n0, int m0, int M, int N,
+                                                 float* Y, int accumulate, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, int f16,
+                                                 float* xch, const float* row_scale, Release release) {
+  using C = PersistCfg<SPLIT, GU>;
+  constexpr int kColStep = 16 * (kPersistEpiWarps / 4);
+  const int m_valid = min(C::kRows, M - m0);
+  if (!GU) {
+    const int n = n0 + quarter * 32 + lane;
+    if (ok) {
+      for (int c = col0; c < m_valid; c += kColStep) {
+        float v[16];
+        tmem_ld16(taddr + c, v);
+        if (SPLIT) {
+          float w[16];
+          tmem_ld16(taddr + C::kRows + c, w);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] += w[j];
+        }
+        if (row_scale != nullptr) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] *= row_scale[(c + j) & 127];
+        }
+        if (n < N) {
+          // all sixteen old values first, then the stores (see the one-tile kernel's epilogue)
+          if (accumulate) {
+            float old[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) old[j] = c + j < m_valid ? Y[(size_t)(m0 + c + j) * N + n] : 0.f;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] += old[j];
+          }
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            if (c + j < m_valid) Y[(size_t)(m0 + c + j) * N + n] = v[j];
+          }
+        }
+      }
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) release();
+  } else {
+    const bool is_gate = quarter < 2;
+    const int l = (quarter & 1) * 32 + lane;
+    float* send = xch + (is_gate ? 64 * C::kLd : 0) + l * C::kLd;
+    const float* recv = xch + (is_gate ? 0 : 64 * C::kLd) + l * C::kLd;
+    const int send0 = is_gate ? C::kHalf : 0, own0 = is_gate ? 0 : C::kHalf;
+    if (ok) {
+#pragma unroll 1
+      for (int c = col0; c < C::kHalf; c += kColStep) {
+        float v[16];
+        tmem_ld16(taddr + send0 + c, v);
+        if (SPLIT) {
+          float w[16];
+          tmem_ld16(taddr + C::kRows + send0 + c, w);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] += w[j];
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) send[c + j] = v[j];
+      }
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * kPersistEpiWarps) : "memory");
+    if (ok && n0 + l < N) {
+#pragma unroll 1
+      for (int c = col0; c < C::kHalf; c += kColStep) {
+        if (own0 + c >= m_valid) break;
+        float v[16];
+        tmem_ld16(taddr + own0 + c, v);
+        if (SPLIT) {
+          float w[16];
+          tmem_ld16(taddr + C::kRows + own0 + c, w);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] += w[j];
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const int r = own0 + c + j;
+          if (r < m_valid) {
+            const float sc = row_scale != nullptr ? row_scale[r & 127] : 1.f;
+            const float mine = v[j] * sc, other = recv[c + j] * sc;
+            const float gate = is_gate ? mine : other, up = is_gate ? other : mine;
+            const float a = gate / (1.f + expf(-gate)) * up;
+            const size_t o = (size_t)(m0 + r) * N + n0 + l;
+            if (!SPLIT && f16) {
+              reinterpret_cast<__half*>(act_hi)[o] = __float2half_rn(a);
+            } else {
+              const __nv_bfloat16 h = __float2bfloat16_rn(a);
+              act_hi[o] = h;
+              if (SPLIT) act_lo[o] = __float2bfloat16_rn(a - __bfloat162float(h));
+            }
+          }
+        }
+      }
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) release();
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * kPersistEpiWarps) : "memory");   // the exchange buffers are free for the next tile
+  }
+}
+
 template <bool GU, bool SPLIT>
 __global__ void __launch_bounds__(kPersistThreads, 1)
 gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
@@ -480,10 +586,7 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
     }
   } else {
     // ---------------- epilogue warps ----------------
-    // eight of them: warp w reads the tensor-memory lanes of quarter w % 4 (the hardware's rule), the two warps of a
-    // quarter take alternate groups of sixteen columns, which halves the time an accumulator stays occupied
     const int quarter = warp & 3, col0 = (warp >> 2) * 16;
-    constexpr int kColStep = 16 * (kPersistEpiWarps / 4);
     uint32_t n_acc = 0;
     RSD_PDL_WAIT();                            // y, the activations' sums of squares and act belong to earlier kernels until now
     const bool scaled = SPLIT && rs.ssq != nullptr;
@@ -509,101 +612,8 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
       if (!ok) fail();
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + b * (uint32_t)C::kMT;
-      const int m_valid = min(C::kRows, M - m0);
-      if (!GU) {
-        const int n = n0 + quarter * 32 + lane;
-        if (ok) {
-          for (int c = col0; c < m_valid; c += kColStep) {
-            float v[16];
-            tmem_ld16(taddr + c, v);
-            if (SPLIT) {
-              float w[16];
-              tmem_ld16(taddr + C::kRows + c, w);
-#pragma unroll
-              for (int j = 0; j < 16; ++j) v[j] += w[j];
-            }
-            if (scaled) {
-#pragma unroll
-              for (int j = 0; j < 16; ++j) v[j] *= row_scale[(c + j) & 127];
-            }
-            if (n < N) {
-              // all sixteen old values first, then the stores (see the one-tile kernel's epilogue)
-              if (accumulate) {
-                float old[16];
-#pragma unroll
-                for (int j = 0; j < 16; ++j) old[j] = c + j < m_valid ? Y[(size_t)(m0 + c + j) * N + n] : 0.f;
-#pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] += old[j];
-              }
-#pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                if (c + j < m_valid) Y[(size_t)(m0 + c + j) * N + n] = v[j];
-              }
-            }
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[b]);
-      } else {
-        const bool is_gate = quarter < 2;
-        const int l = (quarter & 1) * 32 + lane;
-        float* send = xch + (is_gate ? 64 * C::kLd : 0) + l * C::kLd;
-        const float* recv = xch + (is_gate ? 0 : 64 * C::kLd) + l * C::kLd;
-        const int send0 = is_gate ? C::kHalf : 0, own0 = is_gate ? 0 : C::kHalf;
-        if (ok) {
-#pragma unroll 1
-          for (int c = col0; c < C::kHalf; c += kColStep) {
-            float v[16];
-            tmem_ld16(taddr + send0 + c, v);
-            if (SPLIT) {
-              float w[16];
-              tmem_ld16(taddr + C::kRows + send0 + c, w);
-#pragma unroll
-              for (int j = 0; j < 16; ++j) v[j] += w[j];
-            }
-#pragma unroll
-            for (int j = 0; j < 16; ++j) send[c + j] = v[j];
-          }
-        }
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * kPersistEpiWarps) : "memory");
-        if (ok && n0 + l < N) {
-#pragma unroll 1
-          for (int c = col0; c < C::kHalf; c += kColStep) {
-            if (own0 + c >= m_valid) break;
-            float v[16];
-            tmem_ld16(taddr + own0 + c, v);
-            if (SPLIT) {
-              float w[16];
-              tmem_ld16(taddr + C::kRows + own0 + c, w);
-#pragma unroll
-              for (int j = 0; j < 16; ++j) v[j] += w[j];
-            }
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int r = own0 + c + j;
-              if (r < m_valid) {
-                const float sc = scaled ? row_scale[r & 127] : 1.f;
-                const float mine = v[j] * sc, other = recv[c + j] * sc;
-                const float gate = is_gate ? mine : other, up = is_gate ? other : mine;
-                const float a = gate / (1.f + expf(-gate)) * up;
-                const size_t o = (size_t)(m0 + r) * N + n0 + l;
-                if (!SPLIT && f16) {
-                  reinterpret_cast<__half*>(act_hi)[o] = __float2half_rn(a);
-                } else {
-                  const __nv_bfloat16 h = __float2bfloat16_rn(a);
-                  act_hi[o] = h;
-                  if (SPLIT) act_lo[o] = __float2bfloat16_rn(a - __bfloat162float(h));
-                }
-              }
-            }
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[b]);
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * kPersistEpiWarps) : "memory");   // the exchange buffers are free for the next tile
-      }
+      persist_epilogue<GU, SPLIT>(taddr, ok, quarter, lane, col0, n0, m0, M, N, Y, accumulate, act_hi, act_lo, f16, xch,
+                                  scaled ? row_scale : nullptr, [&]() { mbar_arrive(&acc_empty[b]); });
     }
   }
   tc_fence_before();
@@ -612,6 +622,165 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
     __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem_base, 512);
+  }
+}
+
+// ---------------------------------------------------------------------------------------------------------
+// The persistent kernel for pairs of CTAs (cta_group::2): two neighbouring SMs share one tile of 256 weight rows x 256
+// operand rows (256 plain rows of x, or 128 rows as hi | lo).  Each holds its 128 weight rows and HALF of the operand rows,
+// and one thread of the leading CTA issues 256 x 256 x 16 MMAs that read both halves from both shared memories.
+// Why: a lone CTA's 128 x 256 x 16 MMA takes 128 cycles and reads 12 KB, and the copies bring 48 KB every four MMAs:
+// together 192 bytes a cycle against the 128 that an SM's shared memory delivers.  In a pair each SM reads 8 KB and
+// receives 32 KB instead, 128 bytes a cycle, and L2 delivers two thirds of the bytes; the ring also gets deeper.
+// The accumulator, 256 columns in each SM's tensor memory (lanes = its own weight rows), alternates as above, and the
+// epilogues are those of the lone CTA, each SM finishing its own 128 weight rows (64 features in the gate/up mode).
+// Barriers: full[s] and acc_empty[b] of the leader count for both CTAs (the follower's copies and epilogue warps report
+// there), empty[s] and acc_full[b] are signalled in both by the MMAs' commits.  Every wait is bounded.
+// ---------------------------------------------------------------------------------------------------------
+template <bool SPLIT, bool GU> struct PairCfg {
+  using P = PersistCfg<SPLIT, GU>;
+  static constexpr int kStages = (GU && !SPLIT) ? 5 : 6;   // beside the exchange buffers of the plain gate/up tile: five
+  static constexpr int kABytes = kTileN * kTileK * 2, kBBytes = 128 * kTileK * 2, kStageBytes = kABytes + kBBytes;
+  static constexpr size_t kSmemBytes = 1024 + (size_t)kStages * kStageBytes + 256 + P::kXchBytes;
+  // as for the lone CTA, with M = 256
+  static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+  static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
+};
+
+template <bool GU, bool SPLIT>
+__global__ void __launch_bounds__(kPersistThreads, 1)
+gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
+                    const __grid_constant__ CUtensorMap tm_x_lo, float* Y, int M, int N, int K, int accumulate, int n_tiles_n,
+                    int n_tiles_m, int* err, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, int f16) {
+  RSD_PDL_TRIGGER();
+  using C = PairCfg<SPLIT, GU>;
+  constexpr int kRows = C::P::kRows;
+  const uint32_t idesc = f16 ? (C::kIdesc & ~((1u << 7) | (1u << 10))) : C::kIdesc;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = (uint64_t*)(smem + (size_t)C::kStages * C::kStageBytes);
+  uint64_t* empty = full + C::kStages;
+  uint64_t* acc_full = empty + C::kStages;
+  uint64_t* acc_empty = acc_full + 2;
+  uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
+  volatile uint32_t* stop = tmem_slot + 1;
+  float* xch = (float*)(smem + (size_t)C::kStages * C::kStageBytes + 256);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const int total_kb = (K + kTileK - 1) / kTileK, n_tiles = n_tiles_n * n_tiles_m;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < C::kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 2 * kPersistEpiWarps); }
+    *stop = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncwarp();
+  if (warp == kPersistEpiWarps + 1) tmem_alloc_pair(tmem_slot, 512);
+  tc_fence_before();
+  __syncwarp();
+  cluster_sync_all();                          // both CTAs' barriers and tensor memory are set up
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  // tile t -> (row tile of x, pair of weight tiles): groups of eight row tiles, row tile fastest
+  auto tile_of = [&](int t, int& tm, int& tn) {
+    const int per_group = 8 * n_tiles_n, g0 = (t / per_group) * 8, rem = t % per_group, gsz = min(8, n_tiles_m - g0);
+    tm = g0 + rem % gsz;
+    tn = rem / gsz;
+  };
+  constexpr int kFeat = GU ? kTileN / 2 : kTileN;          // output features of one CTA's tile
+  auto first_feature = [&](int tn) { return (2 * tn + (int)rank) * kFeat; };
+  auto fail = [&]() { if (*stop == 0) { if (err) atomicCAS(err, 0, -5); *stop = 1; } };
+
+  if (warp == kPersistEpiWarps) {
+    // ---------------- producer: this CTA's weight rows and its half of the operand rows ----------------
+    if (lane == 0) {
+      tma_prefetch_map(&tm_x);
+      uint32_t it = 0, ahead = 0;
+      auto load_w = [&](int s, int kb, int n0) {
+        uint8_t* a = smem + (size_t)s * C::kStageBytes;
+        const uint32_t bar = cluster_addr(&full[s], 0);
+        if (rank == 0) mbar_expect_tx(&full[s], 2 * C::kStageBytes);     // both CTAs' bytes
+        tma_load_2d_pair(a, &tm_w, bar, kb * kTileK, n0);
+        if (GU) tma_load_2d_pair(a + C::kABytes / 2, &tm_w, bar, kb * kTileK, N + n0);
+      };
+      // the weight tiles of the first ring of stages go out before the predecessors have finished
+      if (pair < n_tiles) {
+        int tm, tn;
+        tile_of(pair, tm, tn);
+        for (; ahead < (uint32_t)min(C::kStages, total_kb); ++ahead) load_w(ahead, ahead, first_feature(tn));
+      }
+      RSD_PDL_WAIT();
+      for (int t = pair; t < n_tiles && !*stop; t += n_pairs) {
+        int tm, tn;
+        tile_of(t, tm, tn);
+        const int n0 = first_feature(tn), m0 = tm * kRows;
+        for (int kb = 0; kb < total_kb; ++kb, ++it) {
+          const uint32_t s = it % C::kStages;
+          if (it >= ahead) {
+            if (!mbar_wait(&empty[s], ((it / C::kStages) & 1u) ^ 1u) || *stop) { fail(); break; }
+            load_w(s, kb, n0);
+          }
+          uint8_t* b = smem + (size_t)s * C::kStageBytes + C::kABytes;
+          const uint32_t bar = cluster_addr(&full[s], 0);
+          if (SPLIT) tma_load_2d_pair(b, rank == 0 ? &tm_x : &tm_x_lo, bar, kb * kTileK, m0);
+          else tma_load_2d_pair(b, &tm_x, bar, kb * kTileK, m0 + (int)rank * 128);
+        }
+      }
+      // the copies still in flight when a wait has run out report to the leader's barriers, which a follower cannot poll:
+      // a few milliseconds are far longer than any of them takes
+      if (*stop)
+        for (int i = 0; i < 4096; ++i) __nanosleep(1000);
+    }
+  } else if (warp == kPersistEpiWarps + 1) {
+    // ---------------- MMA issuer: one thread of the leading CTA ----------------
+    if (lane == 0 && rank == 0) {
+      uint32_t it = 0, n_acc = 0;
+      for (int t = pair; t < n_tiles && !*stop; t += n_pairs, ++n_acc) {
+        const uint32_t b = n_acc & 1u;
+        if (!mbar_wait(&acc_empty[b], ((n_acc >> 1) & 1u) ^ 1u) || *stop) { fail(); break; }
+        tc_fence_after();
+        const uint32_t d_tmem = tmem_base + b * 256u;
+        bool ok = true;
+        for (int kb = 0; kb < total_kb; ++kb, ++it) {
+          const uint32_t s = it % C::kStages;
+          if (!mbar_wait(&full[s], (it / C::kStages) & 1u) || *stop) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t a = smem_u32(smem + (size_t)s * C::kStageBytes), bb = a + C::kABytes;
+#pragma unroll
+          for (int k = 0; k < kTileK / kUmmaK; ++k)
+            umma_f16_pair(d_tmem, smem_desc_sw128(a + k * kUmmaK * 2), smem_desc_sw128(bb + k * kUmmaK * 2), idesc,
+                          (kb > 0 || k > 0) ? 1u : 0u);
+          umma_commit_pair(&empty[s]);
+        }
+        if (!ok) { fail(); break; }
+        umma_commit_pair(&acc_full[b]);
+      }
+    }
+  } else {
+    // ---------------- epilogue warps of both CTAs ----------------
+    const int quarter = warp & 3, col0 = (warp >> 2) * 16;
+    uint32_t n_acc = 0;
+    RSD_PDL_WAIT();                            // y and act belong to earlier kernels until now
+    for (int t = pair; t < n_tiles; t += n_pairs, ++n_acc) {
+      int tm, tn;
+      tile_of(t, tm, tn);
+      const uint32_t b = n_acc & 1u;
+      bool ok = mbar_try_wait(&acc_full[b], (n_acc >> 1) & 1u);
+      for (uint32_t i = 0; i < (1u << 21) && !ok && !*stop; ++i) ok = mbar_try_wait_sleep(&acc_full[b], (n_acc >> 1) & 1u, 1000);
+      if (!ok) fail();
+      tc_fence_after();
+      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + b * 256u;
+      persist_epilogue<GU, SPLIT>(taddr, ok, quarter, lane, col0, first_feature(tn), tm * kRows, M, N, Y, accumulate, act_hi, act_lo,
+                                  f16, xch, nullptr, [&]() { mbar_arrive_cluster(cluster_addr(&acc_empty[b], 0)); });
+    }
+  }
+  tc_fence_before();
+  __syncwarp();
+  cluster_sync_all();                          // nobody leaves while the other CTA may still signal its barriers
+  if (warp == kPersistEpiWarps + 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem_base, 512);
   }
 }
 
@@ -863,6 +1032,53 @@ static cudaError_t launch_persistent(const CUtensorMap& tw, const CUtensorMap& t
   return launched(1);
 }
 
+// Pairs of CTAs that fit the device at once.
+template <bool GU, bool SPLIT>
+static int max_pairs(size_t smem) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2048); cfg.blockDim = dim3(kPersistThreads); cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  int n = 0;
+  return cudaOccupancyMaxActiveClusters(&n, gemm_tc_pair_kernel<GU, SPLIT>, &cfg) == cudaSuccess ? n : 0;
+}
+
+// The map of x has a box of 128 rows.
+template <bool GU, bool SPLIT>
+static cudaError_t launch_pair(const CUtensorMap& tw, const CUtensorMap& tx, const CUtensorMap& txl, float* y, int M, int N, int K,
+                               int accumulate, int* err, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, cudaStream_t s, int f16) {
+  using C = PairCfg<SPLIT, GU>;
+  constexpr size_t smem = C::kSmemBytes;
+  static const int pairs = [] {
+    if (cudaFuncSetAttribute(gemm_tc_pair_kernel<GU, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+    return max_pairs<GU, SPLIT>(smem);
+  }();
+  if (pairs <= 0) return cudaErrorNotSupported;
+  const int feat = GU ? kTileN : 2 * kTileN, tiles_n = (N + feat - 1) / feat, tiles_m = (M + C::P::kRows - 1) / C::P::kRows;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * std::min(tiles_n * tiles_m, pairs)); cfg.blockDim = dim3(kPersistThreads); cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 2;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_tc_pair_kernel<GU, SPLIT>, tw, tx, txl, y, M, N, K, accumulate, tiles_n, tiles_m,
+                                           err, act_hi, act_lo, f16);
+  return e != cudaSuccess ? e : launched(1);
+}
+
+// Whether a dense product goes to pairs of CTAs: it has as many pair tiles as the chip has pairs, and a K long enough for
+// the main loop to matter beside the epilogues.  Lone CTAs / pairs, us: 8192 x 3584 x 18944 881 / 850, 8192 x 1536 x 8960
+// 182 / 170, gate/up 1000 x 18944 x 3584 228 / 203; but 4096 x 1536 x 1536 31.5 / 32.8.  (The paired gate/up tile of
+// hi + lo operands gains nothing, 3180 / 3160 at 8192 x 18944 x 3584, and keeps the lone CTAs.)
+static bool pair_pays(int M, int n_features, int K, int feat, int rows) {
+  return K >= 3072 && ((n_features + feat - 1) / feat) * ((M + rows - 1) / rows) >= 74;
+}
+
 // 65 to 128 rows with pairs take an SM per tile: with more tiles than SMs the persistent kernel hides the epilogues and
 // evens out the last wave (the 1187 tiles of a 151936-row head at 128 rows: 140 us one CTA per tile, 93 us persistent).
 static bool wide_decode(int M, int n_tiles) { return M > 64 && M <= 128 && n_tiles > 148; }
@@ -901,7 +1117,9 @@ cudaError_t launch_gemm_gu(const void* Wgu, const void* x, const void* x_lo, voi
   if (x_lo == nullptr) {
     // plain bf16 operand: the persistent kernel only (more than 128 rows, no row scale, no idle flag)
     if (!(M > 128 && rs.ssq == nullptr && n_active == nullptr)) return cudaErrorNotSupported;
-    if (!get_map(Wgu, 2 * F, K, kTileN / 2, &tw) || !get_map(x, M, K, 256, &tx)) return cudaErrorNotSupported;
+    const bool pair = pair_pays(M, F, K, kTileN, 256);
+    if (!get_map(Wgu, 2 * F, K, kTileN / 2, &tw) || !get_map(x, M, K, pair ? 128 : 256, &tx)) return cudaErrorNotSupported;
+    if (pair) return launch_pair<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act_hi, nullptr, s, 0);
     return launch_persistent<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act_hi, nullptr, s);
   }
   if (!act_lo) return cudaErrorNotSupported;
@@ -954,12 +1172,16 @@ cudaError_t launch_gemm_tc(const void* W, const void* x, const void* x_lo, float
   if (deferred_splits) *deferred_splits = p.splits;
   const bool defer = deferred_splits != nullptr;
   CUtensorMap tw, tx, txl;
-  if (!get_map(W, N, K, kTileN, &tw) || !get_map(x, M, K, p.rows, &tx)) return cudaErrorNotSupported;
+  const bool dense = M > 128 && p.splits == 1 && rs.ssq == nullptr && n_active == nullptr;
+  const bool pair = dense && pair_pays(M, N, K, 2 * kTileN, p.rows);
+  if (!get_map(W, N, K, kTileN, &tw) || !get_map(x, M, K, pair ? 128 : p.rows, &tx)) return cudaErrorNotSupported;
   if (split_operand) { if (!get_map(x_lo, M, K, p.rows, &txl)) return cudaErrorNotSupported; }
   else txl = tx;
   int* err = (int*)((char*)scratch + kCounterBytes);
   float* partials = (float*)((char*)scratch + kCounterBytes + 256);
-  if (M > 128 && p.splits == 1 && rs.ssq == nullptr && n_active == nullptr) {
+  if (dense) {
+    if (pair && split_operand) return launch_pair<false, true>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s, 0);
+    if (pair) return launch_pair<false, false>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s, 0);
     if (split_operand) return launch_persistent<false, true>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s);
     return launch_persistent<false, false>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s);
   }
@@ -1003,10 +1225,11 @@ cudaError_t launch_gemm_f16_dense(const void* W16, const void* x16, float* y, in
   if (M <= 128 || !gemm_tc_supported(1, M, N, K)) return cudaErrorNotSupported;
   if (!scratch || scratch_bytes < gemm_scratch_bytes(M)) return cudaErrorInvalidValue;
   if (((uintptr_t)W16 & 15) || ((uintptr_t)x16 & 15)) return cudaErrorMisalignedAddress;
-  TcPlan p = plan_tc(M, N, K, false);
+  const bool pair = pair_pays(M, N, K, 2 * kTileN, 256);
   CUtensorMap tw, tx;
-  if (!get_map(W16, N, K, kTileN, &tw) || !get_map(x16, M, K, p.rows, &tx)) return cudaErrorNotSupported;
+  if (!get_map(W16, N, K, kTileN, &tw) || !get_map(x16, M, K, pair ? 128 : 256, &tx)) return cudaErrorNotSupported;
   int* err = (int*)((char*)scratch + kCounterBytes);
+  if (pair) return launch_pair<false, false>(tw, tx, tx, y, M, N, K, accumulate, err, nullptr, nullptr, s, 1);
   return launch_persistent<false, false>(tw, tx, tx, y, M, N, K, accumulate, err, nullptr, nullptr, s, 1);
 }
 
@@ -1018,7 +1241,9 @@ cudaError_t launch_gemm_gu_f16_dense(const void* Wgu16, const void* x16, void* a
   if (((uintptr_t)Wgu16 & 15) || ((uintptr_t)x16 & 15)) return cudaErrorMisalignedAddress;
   int* err = (int*)((char*)scratch + kCounterBytes);
   CUtensorMap tw, tx;
-  if (!get_map(Wgu16, 2 * F, K, kTileN / 2, &tw) || !get_map(x16, M, K, 256, &tx)) return cudaErrorNotSupported;
+  const bool pair = pair_pays(M, F, K, kTileN, 256);
+  if (!get_map(Wgu16, 2 * F, K, kTileN / 2, &tw) || !get_map(x16, M, K, pair ? 128 : 256, &tx)) return cudaErrorNotSupported;
+  if (pair) return launch_pair<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act16, nullptr, s, 1);
   return launch_persistent<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act16, nullptr, s, 1);
 }
 

@@ -519,6 +519,45 @@ def test_paired_gemm_of_65_to_128_rows(M, N, K):
     np.testing.assert_allclose(acc, want + y0, rtol=0, atol=tol)
 
 
+@pytest.mark.parametrize("M,N,K", [(2100, 2304, 3072), (2049, 2305, 3080), (512, 18944, 3136), (300, 18817, 3072)])
+@pytest.mark.parametrize("kind", ["fp16", "bf16", "pairs"])
+def test_dense_gemm_on_pairs_of_ctas(M, N, K, kind):
+    """The paired kernel: one tile per pair and several, row and weight tiles that end ragged (also inside the leading CTA's
+    half), a K tail, accumulation into y.  Against an fp32 product of the stored operands: fp32 sums of K products of
+    N(0, 1) activations and N(0, 0.02) weights, bounded as in the tests above."""
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    W = torch.randn(N, K, generator=g, device="cuda") * 0.02
+    x = torch.randn(M, K, generator=g, device="cuda")
+    dt = torch.float16 if kind == "fp16" else torch.bfloat16
+    Wd, hi = W.to(dt), x.to(dt)
+    lo = (x - hi.float()).to(dt) if kind == "pairs" else None
+    want = (hi.double() + (lo.double() if lo is not None else 0)) @ Wd.double().t()
+    y = rb.k_gemm(Wd, hi, impl=4 if kind == "fp16" else 2, x_lo=lo)
+    tol = 3e-5 * K ** 0.5
+    assert (y.double() - want).abs().max().item() <= tol
+    y2 = rb.k_gemm(Wd, hi, y=y.clone(), accumulate=True, impl=4 if kind == "fp16" else 2, x_lo=lo)
+    assert (y2.double() - 2 * want).abs().max().item() <= 2 * tol
+
+
+@pytest.mark.parametrize("M,F,K", [(1100, 1920, 3080), (300, 5056, 3072)])
+def test_gate_up_gemm_on_pairs_of_ctas(M, F, K):
+    """Plain gate/up tiles of the paired kernel, the last pair with one CTA's features missing: silu(g) * u rounded to bf16
+    (2^-9 relative) after fp32 sums."""
+    g = torch.Generator(device="cuda").manual_seed(M + F)
+    W = (torch.randn(2 * F, K, generator=g, device="cuda") * 0.02).bfloat16()
+    x = torch.randn(M, K, generator=g, device="cuda").bfloat16()
+    act = torch.zeros(M, F, dtype=torch.bfloat16, device="cuda")
+    nbytes = rb.lib().rsd_k_gemm_scratch_bytes(M, 2 * F, K)
+    scratch = torch.zeros(nbytes, dtype=torch.uint8, device="cuda")
+    assert rb.lib().rsd_k_gemm_gu(W.data_ptr(), x.data_ptr(), None, act.data_ptr(), None, M, F, K, scratch.data_ptr(), nbytes,
+                                  torch.cuda.current_stream().cuda_stream) == 0
+    gu = x.double() @ W.double().t()
+    want = torch.nn.functional.silu(gu[:, :F]) * gu[:, F:]
+    err = (act.double() - want).abs()
+    assert (err <= 2 ** -8 * want.abs() + 3e-5 * K ** 0.5).all()
+    assert int(scratch[4096:4100].view(torch.int32).item()) == 0
+
+
 def test_bounded_wait_runs_out_and_the_kernel_leaves_cleanly():
     """RSD_ERR_TIMEOUT without a fault: one CTA of the tensor-core GEMM whose copies are never issued.  Its wait
     (a few thousand polls in this mode) expires, the error flag is raised and reported, tensor memory is freed: the
