@@ -39,22 +39,21 @@
 // flight, frees its tensor memory and leaves.
 #include <cuda.h>
 
+#include "attn_chunk_tc.cuh"
 #include "common.cuh"
 #include "kernels.cuh"
-#include "tc_ptx.cuh"
 
 namespace rsd {
 
 namespace {
 
 using namespace tc;
+using namespace chunk;
 
-constexpr int kHd = 128;
 constexpr int kKeys = 64;                           // keys per tile: four pages
 constexpr int kNS = 6;                              // ring stages (keys + values of one tile)
 constexpr int kKBytes = kKeys * kHd * 2;            // K tile: per page [2 token groups][2 dim halves][8 keys][64 dims]
 constexpr int kVBytes = kHd * kKeys * 2;            // V tile: four page buffers [128 dims][16 keys]
-constexpr int kBlockBytes = 4096;                   // keys (or values) of one page and KV head
 constexpr int kStageBytes = kKBytes + kVBytes;
 constexpr int kMetaBytes = 4096;                    // barriers, flags, the tile's entries, the row maxima and sums
 constexpr size_t kSmemBytes = 1024 + kNS * kStageBytes + kMetaBytes;
@@ -70,89 +69,6 @@ constexpr uint32_t kIdescO = (1u << 4) | ((uint32_t)(kHd >> 3) << 17) | ((uint32
 // Q 64 (fp16 pairs), P two buffers of 32 (fp16 pairs)
 constexpr int kSB = 4;
 constexpr uint32_t kColS = 0, kColO = 256, kColQ = 384, kColP = 448, kTmemCols = 512;
-constexpr uint32_t kProbeLimit = 1u << 18;          // polls of a bounded wait (a healthy wait ends within microseconds)
-
-// Writes of this thread to shared memory become visible to the tensor cores.
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
-// The box of a tensor map whose first block coordinate is `blk` (all inner coordinates 0).
-__device__ __forceinline__ void tma_load_block_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int blk) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %3, %4}], [%2];"
-      ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(0), "r"(blk) : "memory");
-}
-__device__ __forceinline__ void tma_load_block_5d(void* dst, const CUtensorMap* map, uint64_t* bar, int blk) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %3, %3, %3, %4}], [%2];"
-      ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(0), "r"(blk) : "memory");
-}
-
-// Shared-memory matrix descriptors of K-major operands (leading byte offset unused, version 1).  A later k-step or
-// half of the same tile is the descriptor plus its byte offset / 16: shared-memory addresses fit the 14-bit field.
-// 128-byte swizzle: rows of 128 bytes, groups of 8 rows `sbo` bytes apart.
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr, uint32_t sbo) {
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | (1ull << 16) | ((uint64_t)(sbo >> 4) << 32) | (1ull << 46) | (2ull << 61);
-}
-// 32-byte swizzle: rows of 32 bytes (one K = 16 step), groups of 8 rows 256 bytes apart.
-__device__ __forceinline__ uint64_t desc_sw32(uint32_t saddr) {
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | (1ull << 16) | ((uint64_t)(256 >> 4) << 32) | (1ull << 46) | (6ull << 61);
-}
-
-// D (tensor memory) (+)= A (tensor memory: 128 lanes x 8 columns of fp16 pairs, one K = 16 step) * B (shared memory)
-__device__ __forceinline__ void umma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
-}
-// 16 (32) registers of this thread into 16 (32) consecutive columns of its tensor-memory lane.
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
-}
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
-  tmem_st16(taddr, r);
-  tmem_st16(taddr + 16, r + 16);
-}
-__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
-  const __half2 h = __floats2half2_rn(lo, hi);         // .x (the low 16 bits) = lo: the element with the even index
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
-
-// 32 consecutive columns of this warp's tensor-memory lanes, one per register.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-// Bounded wait that leaves the issue slots to the warps with work: a short spin (most waits end within a few hundred
-// cycles), then suspended polls.
-__device__ __forceinline__ bool wait_sleep(uint64_t* bar, uint32_t parity, volatile uint32_t* stop) {
-  for (int i = 0; i < 64; ++i)
-    if (mbar_try_wait(bar, parity)) return true;
-  for (uint32_t i = 0; i < (1u << 19); ++i) {
-    if (mbar_try_wait_sleep(bar, parity, 1000)) return true;
-    if (*stop) return false;
-  }
-  return false;
-}
 
 struct Meta {
   uint64_t kv_full[kNS], kv_empty[kNS], s_full[kSB], s_empty[kSB], p_full[2], p_empty[2], o_full, o_empty;
@@ -163,51 +79,6 @@ struct Meta {
   float pmax[2][128], psum[2][128];
 };
 static_assert(sizeof(Meta) <= kMetaBytes, "metadata block");
-
-template <typename OT> __device__ __forceinline__ void store16(OT* hi, OT* lo, size_t o, const float* v);
-template <> __device__ __forceinline__ void store16<float>(float* hi, float*, size_t o, const float* v) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(hi + o + 4 * i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-}
-template <> __device__ __forceinline__ void store16<__half>(__half* hi, __half*, size_t o, const float* v) {
-  __align__(16) __half2 h[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) h[i] = __floats2half2_rn(v[2 * i], v[2 * i + 1]);
-  *reinterpret_cast<uint4*>(hi + o) = *reinterpret_cast<const uint4*>(h);
-  *reinterpret_cast<uint4*>(hi + o + 8) = *reinterpret_cast<const uint4*>(h + 4);
-}
-template <> __device__ __forceinline__ void store16<__nv_bfloat16>(__nv_bfloat16* hi, __nv_bfloat16* lo, size_t o, const float* v) {
-  __align__(16) __nv_bfloat16 h[16];
-  __align__(16) __nv_bfloat16 l[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    h[i] = __float2bfloat16_rn(v[i]);
-    l[i] = __float2bfloat16_rn(v[i] - __bfloat162float(h[i]));
-  }
-  *reinterpret_cast<uint4*>(hi + o) = *reinterpret_cast<const uint4*>(h);
-  *reinterpret_cast<uint4*>(hi + o + 8) = *reinterpret_cast<const uint4*>(h + 8);
-  if (lo != nullptr) {
-    *reinterpret_cast<uint4*>(lo + o) = *reinterpret_cast<const uint4*>(l);
-    *reinterpret_cast<uint4*>(lo + o + 8) = *reinterpret_cast<const uint4*>(l + 8);
-  }
-}
-
-// The values of a partly cached page (global: [128 dims][16 tokens]) into a page buffer of the value tile (rows of
-// 32 bytes under the 32-byte swizzle: the 16-byte halves of a row trade places when bit 2 of the row is set), the
-// tokens from `cached` on zeroed: their memory may hold anything, and 0 * NaN would poison the product.  One warp.
-__device__ __noinline__ void copy_partial_values(const __half* __restrict__ src, uint8_t* dst, int cached, int lane) {
-#pragma unroll 1
-  for (int j = 0; j < 8; ++j) {
-    const int d = lane + 32 * (j >> 1), c = j & 1;
-    __align__(16) __half hv[8];
-    *reinterpret_cast<uint4*>(hv) = *reinterpret_cast<const uint4*>(src + (size_t)d * kPageTokens + c * 8);
-#pragma unroll
-    for (int x = 0; x < 8; ++x)
-      if (c * 8 + x >= cached) hv[x] = __float2half_rn(0.f);
-    *reinterpret_cast<uint4*>(dst + d * 32 + ((c ^ ((d >> 2) & 1)) << 4)) = *reinterpret_cast<const uint4*>(hv);
-  }
-  fence_async_smem();
-}
 
 template <typename OT>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -558,6 +429,11 @@ attn_chunk_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
 
 }  // namespace
 
+// The one-pass kernel for long chunks (attn_chunk_long.cu) wants at least a few dozen CTAs of two query tiles each: from 1024
+// tokens on it wins (32 rows x 64 tokens over 300, 12 / 2 heads: 54 us here, 43 us there; 2 x 600 over 100, 28 / 4: 60 and 46),
+// below it leaves more of the chip idle than it saves (8 x 128 tokens: 25 and 33 us, 64 tokens: 24 and 29).
+static bool attn_chunk_long_pays(int T) { return T > 1024; }
+
 bool attn_chunk_tc_supported(int kv_dtype, int H, int KV, int hd, int T) {
   return kv_dtype == 2 && hd == kHd && KV >= 1 && H % KV == 0 && H / KV <= 8 && T >= 64;
 }
@@ -565,6 +441,7 @@ bool attn_chunk_tc_supported(int kv_dtype, int H, int KV, int hd, int T) {
 cudaError_t launch_attn_chunk_tc(const float* q, PassView p, KvView kv, void* out, void* out_lo, int out_dtype, int H, int KV,
                                  int* err, cudaStream_t s) {
   if (p.T <= 0) return cudaSuccess;
+  if (attn_chunk_long_pays(p.T)) return launch_attn_chunk_long(q, p, kv, out, out_lo, out_dtype, H, KV, err, s);
   const int G = H / KV, QT = 128 / G;
   dim3 grid((p.T + QT - 1) / QT, KV);
   CUtensorMap tm_k, tm_v;

@@ -118,6 +118,9 @@ cudaError_t launch_attn_chunk(int kv_dtype, const float* q, PassView p, KvView k
 bool attn_chunk_tc_supported(int kv_dtype, int H, int KV, int hd, int T);
 cudaError_t launch_attn_chunk_tc(const float* q, PassView p, KvView kv, void* out, void* out_lo, int out_dtype, int H, int KV,
                                  int* err, cudaStream_t s);
+// ... its one-pass form for long chunks, which launch_attn_chunk_tc picks by the chunk's length.
+cudaError_t launch_attn_chunk_long(const float* q, PassView p, KvView kv, void* out, void* out_lo, int out_dtype, int H, int KV,
+                                   int* err, cudaStream_t s);
 cudaError_t launch_swiglu(int dtype, const float* gu, SplitSum pending, void* out, void* out_lo, int T, int F,
                           const int32_t* n_active, cudaStream_t s);
 

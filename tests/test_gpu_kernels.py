@@ -395,6 +395,52 @@ def test_chunk_attention_against_definition(dtype, hd, H, KV):
             np.testing.assert_allclose(got[t, h], want, rtol=0, atol=tol)
 
 
+@pytest.mark.parametrize("H,KV", [(12, 2), (28, 4), (8, 1), (3, 3)])
+def test_long_chunk_attention_one_pass(H, KV):
+    """More than 1024 entries: rows of one token, rows that end inside a key tile, at its edge and one token on; tiles that
+    straddle rows, an idle entry, prefixes of several key tiles; scores that rise along the context so that the reference
+    maximum is raised again and again (keys scaled up with the position), and rows whose largest score comes first.  Against
+    brute-force softmax; the query and the weights are rounded to fp16 (2^-11 relative each), outputs are of order one."""
+    rng = np.random.default_rng(15)
+    ctx = [1, 128, 129, 700, 511, 260]
+    new = [1, 128, 100, 600, 250, 130]
+    max_pages = 48
+    pool, table, Ks, Vs = paged_kv(rng, len(ctx), KV, 128, ctx, torch.float16, max_pages)
+    raw = pool.float().cpu().numpy()
+    for b, grow in ((3, 1), (4, -1)):                  # scale the keys of row 3 up along the context, of row 4 down
+        for i in range((ctx[b] + 15) // 16):
+            f = 1 + (0.5 * i if grow > 0 else 0.5 * (31 - i))
+            raw[table[b, i].item(), 0] *= np.float32(f)
+    pool = torch.from_numpy(raw).cuda().to(torch.float16)
+    back = pool.float().cpu().numpy()
+    for b in (3, 4):
+        for i in range((ctx[b] + 15) // 16):
+            n = min(16, ctx[b] - 16 * i)
+            Ks[b][16 * i:16 * i + n] = back[table[b, i].item(), 0].reshape(KV, 16, 128)[:, :n].transpose(1, 0, 2)
+    rows, poss = [], []
+    for b in range(len(ctx)):
+        for p in range(ctx[b] - new[b], ctx[b]):
+            rows.append(b); poss.append(p)
+    rows.insert(45, -1); poss.insert(45, 0)
+    T = len(rows)
+    assert T > 1024
+    q = rng.normal(size=(T, H, 128)).astype(np.float32)
+    got = rb.k_attn_chunk(dev(q), pool, table, dev(np.array(rows, np.int32)), dev(np.array(poss, np.int32)), KV).cpu().numpy()
+    assert np.isfinite(got[np.array(rows) >= 0]).all()
+    # a score s enters as fp16(q) . K: it errs by |s| 2^-11 / sqrt(hd) or so, and the weights by as much in relative terms
+    for t in list(range(0, T, 17)) + [44, 46, T - 1]:
+        b, p = rows[t], poss[t]
+        if b < 0:
+            continue
+        for h in range(0, H, max(1, H // 4)):
+            g = h // (H // KV)
+            qh = q[t, h].astype(np.float64)
+            s = Ks[b][:p + 1, g].astype(np.float64) @ qh / np.sqrt(128)
+            w = np.exp(s - s.max()); w /= w.sum()
+            tol = 2e-3 + 2 ** -11 * np.abs(Ks[b][:p + 1, g]).max() * 4
+            np.testing.assert_allclose(got[t, h], w @ Vs[b][:p + 1, g].astype(np.float64), rtol=0, atol=tol)
+
+
 @pytest.mark.parametrize("H,KV", [(28, 4), (12, 2)])
 def test_chunk_attention_long_prefix(H, KV):
     """Prefixes of more than a hundred pages (the page ids of a row are fetched in batches of 32, several batches a
