@@ -144,7 +144,8 @@ cudaError_t launch_bf16_to_f16(const void* src, void* dst, size_t n, cudaStream_
 cudaError_t launch_rmsnorm(int dtype, float* x, const void* gain, void* out, void* out_lo, int T, int d, float eps,
                            const int32_t* src, const int32_t* n_active, SplitSum pending, cudaStream_t s, bool out_f16) {
   if (T <= 0) return cudaSuccess;
-  const int threads = d >= 2048 ? 512 : 256;
+  // as few threads as keep the row in registers: more rows are in flight on an SM
+  const int threads = d > 256 * 4 * kNormVecs ? 512 : 256;
   if (dtype == 1 && out_f16)
     RSD_LAUNCH((rmsnorm_kernel<__half, __nv_bfloat16>), T, threads, 0, s, x, (const __nv_bfloat16*)gain, (__half*)out, (__half*)nullptr, d, eps, src, n_active, pending.partials, pending.splits, T);
   else if (dtype == 1)
@@ -781,15 +782,22 @@ __device__ __forceinline__ unsigned long long pack_best(float sc, int id) {
   return ((unsigned long long)key << 32) | (uint32_t)(0xFFFFFFFFu - (uint32_t)id);
 }
 
-// Grid (slots, chunks): every block scans one chunk of the vocabulary and folds its best candidate
-// into best[slot] with an atomic maximum (order-independent, hence deterministic).
-// Bound by the ALUs: ten Philox rounds per four ids and two logarithms per id.  So the scores are first taken with fast
-// logarithms, and only ids within kScoreMargin of the block's best get the exact ones; and as the noise lies in
-// (-2.82, 16.64), four ids whose logits stay 20 below the block's largest draw none at all.  The winner is the same.
-// (Gumbel-max of 151936 ids x 128 rows, one logit 43 above the rest: 87 us with exact noise for all.)
-constexpr int kSampleGroups = 4;            // groups of four ids a thread holds; the launcher cuts the chunks accordingly
+__device__ __forceinline__ float unpack_score(unsigned long long packed) {
+  const uint32_t key = (uint32_t)(packed >> 32);
+  return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key);
+}
+
+// Grid (slots, chunks): every warp takes `steps` runs of 128 ids of a slot and folds its best candidate into best[slot] with
+// an atomic maximum (order-independent, hence deterministic).
+// Exact noise for every id -- ten Philox rounds per four ids and two logarithms per id -- kept the ALUs busy for 66 us at
+// 151936 ids x 128 rows, four times what the logits' 78 MB take.  So a warp first publishes the exact score of its largest
+// logit; then a score is first taken with fast logarithms, and only ids within kScoreMargin of the best so far (this warp's,
+// or what others have published) get exact ones; and as the noise lies below 16.64, ids whose logits stay kNoiseMax below
+// that best draw none at all.  The winner is the same.
+constexpr int kSampleThreads = 256;
+constexpr int kSampleSteps = 8;             // runs of 128 ids that a warp holds in registers at most
 constexpr float kScoreMargin = 1e-3f;       // the fast score errs by less than 1e-4 (see fast_gumbel)
-constexpr float kNoiseRange = 20.f;
+constexpr float kNoiseMax = 17.f;
 
 // -log(-log u) for u = (2k + 1) / 2^24.  Near 1, where the large values come from, -log u is its series in 1 - u (exact
 // in fp32; 1 - u < 2^-6: three terms err by 1e-6 relative); elsewhere __logf errs by 2^-21.4 on -log u > 2^-6, that is
@@ -800,25 +808,15 @@ __device__ __forceinline__ float fast_gumbel(float u) {
   return -__logf(y);
 }
 
-__device__ __forceinline__ float block_max(float v, float* smem) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  __syncthreads();
-  if (lane == 0) smem[threadIdx.x >> 5] = v;
-  __syncthreads();
-  v = lane < nw ? smem[lane] : -INFINITY;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-  return v;
+// What still can win against a best score of `run`.
+__device__ __forceinline__ float score_needed(float run) {
+  return run == INFINITY ? run : run - (kScoreMargin + fabsf(run) * 1e-6f);
 }
 
-__global__ void __launch_bounds__(1024) sample_kernel(SampleArgs a) {
+__global__ void __launch_bounds__(kSampleThreads) sample_kernel(SampleArgs a, int steps) {
   RSD_PDL_TRIGGER();
   if (a.n_active == nullptr) RSD_PDL_WAIT();   // a decode pass's lists may be read ahead of the wait, others not
   const bool idle = a.n_active != nullptr && ld_cg(a.n_active) == 0;
-  __shared__ float s_sc[32];
-  __shared__ int s_ix[32];
   const int slot = blockIdx.x;
   const int row = ld_cg(a.slot_row + slot);
   const uint32_t position = (uint32_t)(ld_cg(a.slot_pos + slot) + 1);
@@ -828,78 +826,80 @@ __global__ void __launch_bounds__(1024) sample_kernel(SampleArgs a) {
   const uint2 key = make_uint2((uint32_t)(a.seed & 0xFFFFFFFFull), (uint32_t)(a.seed >> 32));
   const bool noisy = a.temperature > 0.f;
   const float inv_t = noisy ? 1.f / a.temperature : 1.f;
-  float bs = -INFINITY;
-  int bi = 0x7FFFFFFF;
-  const int n_v4 = (a.v_limit + 3) / 4;
-  const int per_chunk = (n_v4 + gridDim.y - 1) / gridDim.y;
-  const int v4_0 = blockIdx.y * per_chunk + threadIdx.x, v4_end = min(n_v4, (int)(blockIdx.y + 1) * per_chunk);
+  const int lane = threadIdx.x & 31, n_v4 = (a.v_limit + 3) / 4;
+  const int v4_0 = ((blockIdx.y * (kSampleThreads / 32) + (threadIdx.x >> 5)) * steps) * 32 + lane;
   const bool vec = (a.V & 3) == 0 && ((uintptr_t)a.logits & 15) == 0;
-  float x[kSampleGroups][4];
+  const float out = __int_as_float(0x7FC00000);        // NaN: an id out of the race never wins a comparison
+  float x[kSampleSteps][4];
 #pragma unroll
-  for (int k = 0; k < kSampleGroups; ++k) {
-    const int v4 = v4_0 + k * blockDim.x;
+  for (int k = 0; k < kSampleSteps; ++k) {
+    const int v4 = v4_0 + k * 32;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) x[k][j] = -INFINITY;
-    if (v4 < v4_end) {
-      if (vec && v4 * 4 + 3 < a.v_limit) {
-        const float4 f = *reinterpret_cast<const float4*>(lg + v4 * 4);
-        x[k][0] = f.x; x[k][1] = f.y; x[k][2] = f.z; x[k][3] = f.w;
-      } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (v4 * 4 + j < a.v_limit) x[k][j] = lg[v4 * 4 + j];
-      }
-    }
-  }
-  auto block_of = [&](int v4) { return philox4x32_10(make_uint4((uint32_t)v4, position, (uint32_t)row, (uint32_t)a.model_id), key); };
-  if (!noisy) {
-#pragma unroll
-    for (int k = 0; k < kSampleGroups; ++k) {
-      const int v4 = v4_0 + k * blockDim.x;
+    for (int j = 0; j < 4; ++j) x[k][j] = out;
+    if (k < steps && vec && v4 * 4 + 3 < a.v_limit) {
+      const float4 t = *reinterpret_cast<const float4*>(lg + v4 * 4);
+      x[k][0] = t.x; x[k][1] = t.y; x[k][2] = t.z; x[k][3] = t.w;
+    } else if (k < steps && v4 < n_v4) {
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        if (v4 < v4_end && v4 * 4 + j < a.v_limit) better(bs, bi, x[k][j], v4 * 4 + j);
+        if (v4 * 4 + j < a.v_limit) x[k][j] = lg[v4 * 4 + j];
     }
+  }
+  auto noise_bits = [&](int v4, uint32_t (&w)[4]) {
+    const uint4 r = philox4x32_10(make_uint4((uint32_t)v4, position, (uint32_t)row, (uint32_t)a.model_id), key);
+    w[0] = r.x; w[1] = r.y; w[2] = r.z; w[3] = r.w;
+  };
+  auto exact = [&](float logit, uint32_t bits) { return fmaf(logit, inv_t, -logf(-logf(uniform_from_bits(bits)))); };
+  float bs = -INFINITY;
+  int bi = 0x7FFFFFFF;
+  // this lane's largest logit, then the warp's
+  float tx = -INFINITY;
+  int ti = 0x7FFFFFFF;
+#pragma unroll
+  for (int k = 0; k < kSampleSteps; ++k)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) better(tx, ti, x[k][j], (v4_0 + k * 32) * 4 + j);
+  if (!noisy) {
+    bs = tx; bi = ti;
   } else {
-    float top[kSampleGroups], top_all = -INFINITY;
+    float wx = tx;
 #pragma unroll
-    for (int k = 0; k < kSampleGroups; ++k) {
-      top[k] = fmaxf(fmaxf(x[k][0], x[k][1]), fmaxf(x[k][2], x[k][3])) * inv_t;
-      top_all = fmaxf(top_all, top[k]);
+    for (int o = 16; o > 0; o >>= 1) wx = fmaxf(wx, __shfl_xor_sync(0xFFFFFFFFu, wx, o));
+    float run = -INFINITY;
+    if (tx == wx && ti != 0x7FFFFFFF) {                // one lane, or a few that tie
+      uint32_t w[4];
+      noise_bits(ti >> 2, w);
+      const int j = ti & 3;
+      bs = exact(tx, j == 0 ? w[0] : j == 1 ? w[1] : j == 2 ? w[2] : w[3]);
+      bi = ti;
+      const unsigned long long mine = pack_best(bs, bi), seen = atomicMax(a.best + slot, mine);
+      run = unpack_score(seen > mine ? seen : mine);
     }
-    const float floor_ = block_max(top_all, s_sc) - kNoiseRange;
-    float s_max = -INFINITY;
-    float sc[kSampleGroups][4];
 #pragma unroll
-    for (int k = 0; k < kSampleGroups; ++k) {
-      const int v4 = v4_0 + k * blockDim.x;
-      const bool on = v4 < v4_end && !(top[k] < floor_);
-      uint32_t w[4] = {0, 0, 0, 0};
-      if (on) {
-        const uint4 r = block_of(v4);
-        w[0] = r.x; w[1] = r.y; w[2] = r.z; w[3] = r.w;
-      }
+    for (int o = 16; o > 0; o >>= 1) run = fmaxf(run, __shfl_xor_sync(0xFFFFFFFFu, run, o));
+#pragma unroll
+    for (int k = 0; k < kSampleSteps; ++k) {
+      if (k >= steps) break;
+      const int v4 = v4_0 + k * 32;
+      const float top = fmaxf(fmaxf(x[k][0], x[k][1]), fmaxf(x[k][2], x[k][3])) * inv_t;
+      if (!__any_sync(0xFFFFFFFFu, top >= run - kNoiseMax || run == -INFINITY)) continue;
+      uint32_t w[4];
+      noise_bits(v4, w);
+      float sc[4], wm = -INFINITY;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        sc[k][j] = on && v4 * 4 + j < a.v_limit ? fmaf(x[k][j], inv_t, fast_gumbel(uniform_from_bits(w[j]))) : __int_as_float(0x7FC00000);
-        s_max = fmaxf(s_max, sc[k][j]);        // NaN (an id out of the race) never wins
+        sc[j] = fmaf(x[k][j], inv_t, fast_gumbel(uniform_from_bits(w[j])));
+        wm = fmaxf(wm, sc[j]);
       }
-    }
-    s_max = block_max(s_max, s_sc);
-    const float need = s_max == INFINITY ? s_max : s_max - (kScoreMargin + fabsf(s_max) * 1e-6f);
+      const float need = score_needed(run);
+      if (!__any_sync(0xFFFFFFFFu, wm >= need)) continue;
 #pragma unroll
-    for (int k = 0; k < kSampleGroups; ++k) {
-      const bool any = sc[k][0] >= need || sc[k][1] >= need || sc[k][2] >= need || sc[k][3] >= need;
-      if (any) {
-        const int v4 = v4_0 + k * blockDim.x;
-        const uint4 r = block_of(v4);
-        const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+      for (int j = 0; j < 4; ++j)
+        if (sc[j] >= need) better(bs, bi, exact(x[k][j], w[j]), v4 * 4 + j);
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (sc[k][j] >= need) better(bs, bi, fmaf(x[k][j], inv_t, -logf(-logf(uniform_from_bits(w[j])))), v4 * 4 + j);
-      }
+      for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xFFFFFFFFu, wm, o));
+      run = fmaxf(run, wm);
     }
-    __syncthreads();                           // s_sc is used again below
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -907,21 +907,7 @@ __global__ void __launch_bounds__(1024) sample_kernel(SampleArgs a) {
     const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
     better(bs, bi, os, oi);
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) { s_sc[warp] = bs; s_ix[warp] = bi; }
-  __syncthreads();
-  if (warp == 0) {
-    const int nw = blockDim.x >> 5;
-    bs = lane < nw ? s_sc[lane] : -INFINITY;
-    bi = lane < nw ? s_ix[lane] : 0x7FFFFFFF;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float os = __shfl_xor_sync(0xFFFFFFFFu, bs, o);
-      const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
-      better(bs, bi, os, oi);
-    }
-    if (lane == 0 && bi != 0x7FFFFFFF) atomicMax(a.best + slot, pack_best(bs, bi));
-  }
+  if (lane == 0 && bi != 0x7FFFFFFF) atomicMax(a.best + slot, pack_best(bs, bi));
 }
 
 // token[slot] = id held in best[slot]; best is cleared for the next use.
@@ -933,18 +919,14 @@ __global__ void sample_finalize_kernel(unsigned long long* best, const int32_t* 
   best[i] = 0ull;
 }
 
-// Blocks per slot: enough of them to fill the machine at small batches, and no more ids per block than its threads hold.
-int sample_chunks(int v_limit, int threads) {
-  const int want = v_limit >= 65536 ? 16 : (v_limit >= 8192 ? 4 : 1), per_block = threads * kSampleGroups * 4;
-  return std::max(want, (v_limit + per_block - 1) / per_block);
-}
-
 // Leaves the winners packed in a.best (which must be zero on entry); when a.token is given a second
 // kernel unpacks them into a.token and clears a.best.
 cudaError_t launch_sample(const SampleArgs& a, cudaStream_t s) {
   if (a.n_slots <= 0) return cudaSuccess;
-  const int threads = a.v_limit >= 16384 ? 1024 : 256;
-  RSD_LAUNCH((sample_kernel), dim3(a.n_slots, sample_chunks(a.v_limit, threads)), threads, 0, s, a);
+  // runs of 128 ids per warp: as many as leave every SM its 24 warps or so, so that small batches stay wide
+  const int runs = (a.v_limit + 127) / 128, warps = kSampleThreads / 32;
+  const int steps = std::max(1, std::min(kSampleSteps, (int)((long)a.n_slots * runs / (148 * 24))));
+  RSD_LAUNCH((sample_kernel), dim3(a.n_slots, (runs + warps * steps - 1) / (warps * steps)), kSampleThreads, 0, s, a, steps);
   if (a.token == nullptr) return launched(1);
   RSD_LAUNCH((sample_finalize_kernel), (a.n_slots + 255) / 256, 256, 0, s, a.best, a.slot_row, a.token, a.n_slots);
   return launched(2);
