@@ -83,7 +83,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
                const __grid_constant__ CUtensorMap tm_x_lo, float* Y,
                int M, int N, int K, int accumulate, int splits, int kb_per_split, float* partials,
                int* err, const int32_t* n_active, RowScale rs,
-               __nv_bfloat16* act_hi = nullptr, __nv_bfloat16* act_lo = nullptr) {
+               __nv_bfloat16* act_hi = nullptr, __nv_bfloat16* act_lo = nullptr, int f16 = 0) {
   // Programmatic dependent launch: the next kernel may be scheduled at once; this kernel sets itself
   // up and starts streaming its WEIGHT tiles (never written by any kernel) while its predecessors are
   // still running, and only then waits for them (griddepcontrol.wait) before it touches activations
@@ -92,6 +92,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
   RSD_PDL_TRIGGER();
   const int active = n_active != nullptr ? ld_cg(n_active) : 1;
   using Cfg = TcCfg<MT, DEEP>;
+  const uint32_t idesc = f16 ? (Cfg::kIdesc & ~((1u << 7) | (1u << 10))) : Cfg::kIdesc;   // both operands fp16 instead of bf16
   constexpr int kRows = SPLIT ? MT / 2 : MT;   // distinct x rows per tile
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -201,7 +202,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
         const uint32_t b = a + Cfg::kABytes;
 #pragma unroll
         for (int k = 0; k < kTileK / kUmmaK; ++k) {
-          umma_bf16(tmem_base, smem_desc_sw128(a + k * kUmmaK * 2), smem_desc_sw128(b + k * kUmmaK * 2), Cfg::kIdesc,
+          umma_bf16(tmem_base, smem_desc_sw128(a + k * kUmmaK * 2), smem_desc_sw128(b + k * kUmmaK * 2), idesc,
                     (i > 0 || k > 0) ? 1u : 0u);
         }
         umma_commit(&empty[s]);   // frees the stage once these MMAs have read it
@@ -906,7 +907,7 @@ TcPlan plan_tc(int M, int N, int K, bool split_operand) {
 template <int MT, bool SPLIT, bool DEEP = false>
 cudaError_t launch_mt(const CUtensorMap& tw, const CUtensorMap& tx, const CUtensorMap& txl, float* y, int M, int N, int K,
                       int accumulate, const TcPlan& p, float* partials, int* err, const int32_t* n_active,
-                      bool defer_reduce, RowScale rs, cudaStream_t s) {
+                      bool defer_reduce, RowScale rs, cudaStream_t s, int f16 = 0) {
   using Cfg = TcCfg<MT, DEEP>;
   static bool configured = false;
   if (!configured) {
@@ -917,7 +918,7 @@ cudaError_t launch_mt(const CUtensorMap& tw, const CUtensorMap& tx, const CUtens
   dim3 grid(p.n_tiles, p.m_tiles, p.splits);
   RSD_LAUNCH((gemm_tc_kernel<MT, SPLIT, false, DEEP>), grid, kTcThreads, Cfg::kSmemBytes, s, tw, tx, txl, y, M, N, K, accumulate, p.splits,
                                                                      p.kb_per_split, partials, err, n_active, rs,
-                                                                     (__nv_bfloat16*)nullptr, (__nv_bfloat16*)nullptr);
+                                                                     (__nv_bfloat16*)nullptr, (__nv_bfloat16*)nullptr, f16);
   if (p.splits > 1 && !defer_reduce) {
     const size_t total4 = (size_t)M * N / 4;
     const int blocks = (int)std::min<size_t>((total4 + 255) / 256, 148 * 8);
@@ -993,7 +994,7 @@ cudaError_t launch_gemm_wait_probe(const void* W, const void* x, float* y, void*
   int* err = (int*)((char*)scratch + kCounterBytes);
   float* partials = (float*)((char*)scratch + kCounterBytes + 256);
   RSD_LAUNCH((gemm_tc_kernel<16, false, false, false, true>), dim3(1, 1, 1), kTcThreads, TcCfg<16>::kSmemBytes, s, tw, tx, tx, y, 16, 128, 64, 0, 1, 1,
-             partials, err, (const int32_t*)nullptr, RowScale(), (__nv_bfloat16*)nullptr, (__nv_bfloat16*)nullptr);
+             partials, err, (const int32_t*)nullptr, RowScale(), (__nv_bfloat16*)nullptr, (__nv_bfloat16*)nullptr, 0);
   return launched(1);
 }
 
@@ -1079,6 +1080,34 @@ static bool pair_pays(int M, int n_features, int K, int feat, int rows) {
   return K >= 3072 && ((n_features + feat - 1) / feat) * ((M + rows - 1) / rows) >= 74;
 }
 
+// Rows of x per tile for a dense product with one operand (bf16 or fp16): 256, or 128 or 64 while the tiles of the larger
+// size leave half of the SMs (of 256) or some (of 128) without one.  Every size sums along K in the same order: the
+// results are the same bits.  us at 256 / at the size taken, adding into y: 455 x 2048 x 1536 27.6 / 20.5 (64), 1000 x 1536 x 1536
+// 28.7 / 22.5 (64); 1000 x 3584 x 3584, 112 tiles of 256: 42 / 43.6 (128), kept at 256.
+static int dense_rows(int M, int N) {
+  const int n_tiles = (N + kTileN - 1) / kTileN;
+  int rows = 256;
+  while (rows > 64 && n_tiles * ((M + rows - 1) / rows) < (rows == 256 ? 74 : 148)) rows /= 2;
+  return rows;
+}
+
+// ... one tile per CTA; with at most one CTA per SM the deep ring (a lone CTA is bound by the latency of its stages).
+static cudaError_t launch_dense_small(const CUtensorMap& tw, const CUtensorMap& tx, float* y, int M, int N, int K, int accumulate,
+                                      int rows, int* err, cudaStream_t s, int f16) {
+  TcPlan p;
+  p.rows = p.mt = rows;
+  p.n_tiles = (N + kTileN - 1) / kTileN;
+  p.m_tiles = (M + rows - 1) / rows;
+  p.splits = 1;
+  p.kb_per_split = (K + kTileK - 1) / kTileK;
+  const bool deep = p.n_tiles * p.m_tiles <= 148;
+#define RSD_DENSE(MT, DEEP) return launch_mt<MT, false, DEEP>(tw, tx, tx, y, M, N, K, accumulate, p, nullptr, err, nullptr, false, RowScale(), s, f16)
+  if (rows == 64) { if (deep) RSD_DENSE(64, true); RSD_DENSE(64, false); }
+  if (deep) RSD_DENSE(128, true);
+  RSD_DENSE(128, false);
+#undef RSD_DENSE
+}
+
 // 65 to 128 rows with pairs take an SM per tile: with more tiles than SMs the persistent kernel hides the epilogues and
 // evens out the last wave (the 1187 tiles of a 151936-row head at 128 rows: 140 us one CTA per tile, 93 us persistent).
 static bool wide_decode(int M, int n_tiles) { return M > 64 && M <= 128 && n_tiles > 148; }
@@ -1097,7 +1126,7 @@ static cudaError_t launch_gu_mt(const CUtensorMap& tw, const CUtensorMap& tx, co
   const int total_kb = (K + kTileK - 1) / kTileK;
   dim3 grid(F / 64, (M + rows - 1) / rows, 1);
   RSD_LAUNCH((gemm_tc_kernel<MT, true, true, DEEP>), grid, kTcThreads, smem, s, tw, tx, txl, (float*)nullptr, M, F, K, 0, 1, total_kb,
-             (float*)nullptr, err, n_active, rs, act_hi, act_lo);
+             (float*)nullptr, err, n_active, rs, act_hi, act_lo, 0);
   return launched(1);
 }
 
@@ -1174,7 +1203,8 @@ cudaError_t launch_gemm_tc(const void* W, const void* x, const void* x_lo, float
   CUtensorMap tw, tx, txl;
   const bool dense = M > 128 && p.splits == 1 && rs.ssq == nullptr && n_active == nullptr;
   const bool pair = dense && pair_pays(M, N, K, 2 * kTileN, p.rows);
-  if (!get_map(W, N, K, kTileN, &tw) || !get_map(x, M, K, pair ? 128 : p.rows, &tx)) return cudaErrorNotSupported;
+  const int rows = dense && !split_operand && !pair && !no_k_split ? dense_rows(M, N) : p.rows;
+  if (!get_map(W, N, K, kTileN, &tw) || !get_map(x, M, K, pair ? 128 : rows, &tx)) return cudaErrorNotSupported;
   if (split_operand) { if (!get_map(x_lo, M, K, p.rows, &txl)) return cudaErrorNotSupported; }
   else txl = tx;
   int* err = (int*)((char*)scratch + kCounterBytes);
@@ -1182,6 +1212,7 @@ cudaError_t launch_gemm_tc(const void* W, const void* x, const void* x_lo, float
   if (dense) {
     if (pair && split_operand) return launch_pair<false, true>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s, 0);
     if (pair) return launch_pair<false, false>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s, 0);
+    if (rows < 256 && !split_operand) return launch_dense_small(tw, tx, y, M, N, K, accumulate, rows, err, s, 0);
     if (split_operand) return launch_persistent<false, true>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s);
     return launch_persistent<false, false>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s);
   }
@@ -1227,8 +1258,10 @@ cudaError_t launch_gemm_f16_dense(const void* W16, const void* x16, float* y, in
   if (((uintptr_t)W16 & 15) || ((uintptr_t)x16 & 15)) return cudaErrorMisalignedAddress;
   const bool pair = pair_pays(M, N, K, 2 * kTileN, 256);
   CUtensorMap tw, tx;
-  if (!get_map(W16, N, K, kTileN, &tw) || !get_map(x16, M, K, pair ? 128 : 256, &tx)) return cudaErrorNotSupported;
+  const int rows = pair ? 128 : dense_rows(M, N);
+  if (!get_map(W16, N, K, kTileN, &tw) || !get_map(x16, M, K, rows, &tx)) return cudaErrorNotSupported;
   int* err = (int*)((char*)scratch + kCounterBytes);
+  if (!pair && rows < 256) return launch_dense_small(tw, tx, y, M, N, K, accumulate, rows, err, s, 1);
   if (pair) return launch_pair<false, false>(tw, tx, tx, y, M, N, K, accumulate, err, nullptr, nullptr, s, 1);
   return launch_persistent<false, false>(tw, tx, tx, y, M, N, K, accumulate, err, nullptr, nullptr, s, 1);
 }
