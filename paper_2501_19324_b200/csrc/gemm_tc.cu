@@ -155,14 +155,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
           for (int i = 0; i < pre; ++i) mbar_arrive(&full[i]);
         }
       }
-      int issued = 0;
-      bool ok = true;
+      int issued = 0, s = 0;
+      uint32_t phase = 1;                      // of empty[s]: a fresh barrier passes for the parity before its first
+      bool ok = true, ready = true;
       for (int i = 0; i < n_issue; ++i) {
-        const int s = i % Cfg::kStages;
-        if (i >= Cfg::kStages) {
-          ok = mbar_wait(&empty[s], ((i / Cfg::kStages) - 1) & 1);
-          if (!ok || flags[0]) { ok = false; break; }
-        }
+        if (!ready && (!mbar_wait(&empty[s], phase) || flags[0])) { ok = false; break; }
         uint8_t* a = smem + (size_t)s * Cfg::kStageBytes;
         if (warp == 4) {
           mbar_expect_tx(&full[s], Cfg::kABytes);
@@ -174,6 +171,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
           if (SPLIT) tma_load_2d(a + Cfg::kABytes + kRows * kTileK * 2, &tm_x_lo, &full[s], (kb0 + i) * kTileK, m0);
         }
         issued = i + 1;
+        if (++s == Cfg::kStages) { s = 0; phase ^= 1u; }
+        ready = mbar_test(&empty[s], phase);
       }
       if (active == 0) {
         for (int i = 0; i < issued; ++i) mbar_wait(&full[i], 0);
@@ -192,12 +191,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
   } else if (warp == 5) {
     // ---------------- MMA issuer ----------------
     if (lane == 0 && active != 0) {
-      bool ok = true;
+      // The thread's own pace bounds a lone CTA: an MMA of 128 x N x 16 takes 64 cycles or more (it reads 4 KB of weights),
+      // four of them a k-block; the wait (127 cycles even when the data are there) and the commit (55) came on top, 440 cycles
+      // per k-block.  So the next stage is looked at before this one's MMAs, and the wait is entered only if it is late.
+      bool ok = true, ready = false;
+      int s = 0;
+      uint32_t phase = 0;
       for (int i = 0; i < n_kb; ++i) {
-        const int s = i % Cfg::kStages;
-        ok = mbar_wait(&full[s], (i / Cfg::kStages) & 1, PROBE ? 4096u : kWaitLimit);
-        if (!ok || flags[0]) { ok = false; break; }
+        if (!ready) {
+          ok = mbar_wait(&full[s], phase, PROBE ? 4096u : kWaitLimit);
+          if (!ok || flags[0]) { ok = false; break; }
+        }
         tc_fence_after();
+        const int s1 = s + 1 == Cfg::kStages ? 0 : s + 1;
+        const uint32_t phase1 = s1 == 0 ? phase ^ 1u : phase;
+        ready = i + 1 < n_kb && mbar_test(&full[s1], phase1);
         const uint32_t a = smem_u32(smem + (size_t)s * Cfg::kStageBytes);
         const uint32_t b = a + Cfg::kABytes;
 #pragma unroll
@@ -206,6 +214,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
                     (i > 0 || k > 0) ? 1u : 0u);
         }
         umma_commit(&empty[s]);   // frees the stage once these MMAs have read it
+        s = s1;
+        phase = phase1;
       }
       if (ok) {
         umma_commit(tmem_full);
@@ -736,23 +746,27 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_const
   } else if (warp == kPersistEpiWarps + 1) {
     // ---------------- MMA issuer: one thread of the leading CTA ----------------
     if (lane == 0 && rank == 0) {
-      uint32_t it = 0, n_acc = 0;
+      uint32_t s = 0, phase = 0, n_acc = 0;
+      bool ready = false;
       for (int t = pair; t < n_tiles && !*stop; t += n_pairs, ++n_acc) {
         const uint32_t b = n_acc & 1u;
         if (!mbar_wait(&acc_empty[b], ((n_acc >> 1) & 1u) ^ 1u) || *stop) { fail(); break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + b * 256u;
         bool ok = true;
-        for (int kb = 0; kb < total_kb; ++kb, ++it) {
-          const uint32_t s = it % C::kStages;
-          if (!mbar_wait(&full[s], (it / C::kStages) & 1u) || *stop) { ok = false; break; }
+        for (int kb = 0; kb < total_kb; ++kb) {
+          if (!ready && (!mbar_wait(&full[s], phase) || *stop)) { ok = false; break; }
           tc_fence_after();
+          const uint32_t s1 = s + 1 == (uint32_t)C::kStages ? 0u : s + 1, phase1 = s1 == 0 ? phase ^ 1u : phase;
+          ready = mbar_test(&full[s1], phase1);        // under this stage's MMAs (see the one-tile kernel)
           const uint32_t a = smem_u32(smem + (size_t)s * C::kStageBytes), bb = a + C::kABytes;
 #pragma unroll
           for (int k = 0; k < kTileK / kUmmaK; ++k)
             umma_f16_pair(d_tmem, smem_desc_sw128(a + k * kUmmaK * 2), smem_desc_sw128(bb + k * kUmmaK * 2), idesc,
                           (kb > 0 || k > 0) ? 1u : 0u);
           umma_commit_pair(&empty[s]);
+          s = s1;
+          phase = phase1;
         }
         if (!ok) { fail(); break; }
         umma_commit_pair(&acc_full[b]);
@@ -1072,12 +1086,13 @@ static cudaError_t launch_pair(const CUtensorMap& tw, const CUtensorMap& tx, con
   return e != cudaSuccess ? e : launched(1);
 }
 
-// Whether a dense product goes to pairs of CTAs: it has as many pair tiles as the chip has pairs, and a K long enough for
-// the main loop to matter beside the epilogues.  Lone CTAs / pairs, us: 8192 x 3584 x 18944 881 / 850, 8192 x 1536 x 8960
-// 182 / 170, gate/up 1000 x 18944 x 3584 228 / 203; but 4096 x 1536 x 1536 31.5 / 32.8.  (The paired gate/up tile of
-// hi + lo operands gains nothing, 3180 / 3160 at 8192 x 18944 x 3584, and keeps the lone CTAs.)
-static bool pair_pays(int M, int n_features, int K, int feat, int rows) {
-  return K >= 3072 && ((n_features + feat - 1) / feat) * ((M + rows - 1) / rows) >= 74;
+// Whether a dense product goes to pairs of CTAs: it has as many pair tiles as the chip has pairs, and where it adds into y a K
+// long enough for the main loop to matter beside the epilogues.  Lone CTAs / pairs, us: 8192 x 3584 x 18944 857 / 817,
+// 8192 x 1536 x 8960 182 / 158, 8192 x 2048 x 1536 55 / 51, gate/up 1000 x 18944 x 3584 226 / 193, 8192 x 18944 x 3584
+// 1636 / 1501; adding, 4096 x 1536 x 1536 41 / 43.  (The paired gate/up tile of hi + lo operands gains nothing, 3180 / 3160
+// at 8192 x 18944 x 3584, and keeps the lone CTAs.)
+static bool pair_pays(int M, int n_features, int K, int feat, int rows, bool adds) {
+  return K >= (adds ? 3072 : 1024) && ((n_features + feat - 1) / feat) * ((M + rows - 1) / rows) >= 74;
 }
 
 // Rows of x per tile for a dense product with one operand (bf16 or fp16): 256, or 128 or 64 while the tiles of the larger
@@ -1146,7 +1161,7 @@ cudaError_t launch_gemm_gu(const void* Wgu, const void* x, const void* x_lo, voi
   if (x_lo == nullptr) {
     // plain bf16 operand: the persistent kernel only (more than 128 rows, no row scale, no idle flag)
     if (!(M > 128 && rs.ssq == nullptr && n_active == nullptr)) return cudaErrorNotSupported;
-    const bool pair = pair_pays(M, F, K, kTileN, 256);
+    const bool pair = pair_pays(M, F, K, kTileN, 256, false);
     if (!get_map(Wgu, 2 * F, K, kTileN / 2, &tw) || !get_map(x, M, K, pair ? 128 : 256, &tx)) return cudaErrorNotSupported;
     if (pair) return launch_pair<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act_hi, nullptr, s, 0);
     return launch_persistent<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act_hi, nullptr, s);
@@ -1202,7 +1217,7 @@ cudaError_t launch_gemm_tc(const void* W, const void* x, const void* x_lo, float
   const bool defer = deferred_splits != nullptr;
   CUtensorMap tw, tx, txl;
   const bool dense = M > 128 && p.splits == 1 && rs.ssq == nullptr && n_active == nullptr;
-  const bool pair = dense && pair_pays(M, N, K, 2 * kTileN, p.rows);
+  const bool pair = dense && pair_pays(M, N, K, 2 * kTileN, p.rows, accumulate != 0);
   const int rows = dense && !split_operand && !pair && !no_k_split ? dense_rows(M, N) : p.rows;
   if (!get_map(W, N, K, kTileN, &tw) || !get_map(x, M, K, pair ? 128 : rows, &tx)) return cudaErrorNotSupported;
   if (split_operand) { if (!get_map(x_lo, M, K, p.rows, &txl)) return cudaErrorNotSupported; }
@@ -1256,7 +1271,7 @@ cudaError_t launch_gemm_f16_dense(const void* W16, const void* x16, float* y, in
   if (M <= 128 || !gemm_tc_supported(1, M, N, K)) return cudaErrorNotSupported;
   if (!scratch || scratch_bytes < gemm_scratch_bytes(M)) return cudaErrorInvalidValue;
   if (((uintptr_t)W16 & 15) || ((uintptr_t)x16 & 15)) return cudaErrorMisalignedAddress;
-  const bool pair = pair_pays(M, N, K, 2 * kTileN, 256);
+  const bool pair = pair_pays(M, N, K, 2 * kTileN, 256, accumulate != 0);
   CUtensorMap tw, tx;
   const int rows = pair ? 128 : dense_rows(M, N);
   if (!get_map(W16, N, K, kTileN, &tw) || !get_map(x16, M, K, rows, &tx)) return cudaErrorNotSupported;
@@ -1274,7 +1289,7 @@ cudaError_t launch_gemm_gu_f16_dense(const void* Wgu16, const void* x16, void* a
   if (((uintptr_t)Wgu16 & 15) || ((uintptr_t)x16 & 15)) return cudaErrorMisalignedAddress;
   int* err = (int*)((char*)scratch + kCounterBytes);
   CUtensorMap tw, tx;
-  const bool pair = pair_pays(M, F, K, kTileN, 256);
+  const bool pair = pair_pays(M, F, K, kTileN, 256, false);
   if (!get_map(Wgu16, 2 * F, K, kTileN / 2, &tw) || !get_map(x16, M, K, pair ? 128 : 256, &tx)) return cudaErrorNotSupported;
   if (pair) return launch_pair<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act16, nullptr, s, 1);
   return launch_persistent<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act16, nullptr, s, 1);

@@ -565,7 +565,7 @@ def test_paired_gemm_of_65_to_128_rows(M, N, K):
     np.testing.assert_allclose(acc, want + y0, rtol=0, atol=tol)
 
 
-@pytest.mark.parametrize("M,N,K", [(2100, 2304, 3072), (2049, 2305, 3080), (512, 18944, 3136), (300, 18817, 3072)])
+@pytest.mark.parametrize("M,N,K", [(2100, 2304, 3072), (2049, 2305, 3080), (512, 18944, 3136), (300, 18817, 3072), (4100, 1300, 1032)])
 @pytest.mark.parametrize("kind", ["fp16", "bf16", "pairs"])
 def test_dense_gemm_on_pairs_of_ctas(M, N, K, kind):
     """The paired kernel: one tile per pair and several, row and weight tiles that end ragged (also inside the leading CTA's
