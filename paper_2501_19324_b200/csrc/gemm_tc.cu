@@ -189,37 +189,40 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
       }
     }
   } else if (warp == 5) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0 && active != 0) {
-      // The thread's own pace bounds a lone CTA: an MMA of 128 x N x 16 takes 64 cycles or more (it reads 4 KB of weights),
-      // four of them a k-block; the wait (127 cycles even when the data are there) and the commit (55) came on top, 440 cycles
-      // per k-block.  So the next stage is looked at before this one's MMAs, and the wait is entered only if it is late.
+    // ---------------- MMA issuer: the whole warp walks the ring, one lane issues ----------------
+    // What a lone CTA gets through a second hangs on this loop.  Issued by a diverged thread, a narrow MMA took 140 cycles
+    // (its descriptors were moved into uniform registers one by one), the wait 127 even when the data were there: 0.32 us
+    // per k-block, 51 GB/s of weights a SM, whatever the ring's depth or the tile's width.  Converged and with the look ahead: 0.23 us.
+    if (active != 0) {
       bool ok = true, ready = false;
       int s = 0;
       uint32_t phase = 0;
+      const uint32_t on = elect_one();
       for (int i = 0; i < n_kb; ++i) {
         if (!ready) {
           ok = mbar_wait(&full[s], phase, PROBE ? 4096u : kWaitLimit);
-          if (!ok || flags[0]) { ok = false; break; }
+          ok = __all_sync(0xFFFFFFFFu, ok && !flags[0]);
+          if (!ok) break;
         }
         tc_fence_after();
         const int s1 = s + 1 == Cfg::kStages ? 0 : s + 1;
         const uint32_t phase1 = s1 == 0 ? phase ^ 1u : phase;
-        ready = i + 1 < n_kb && mbar_test(&full[s1], phase1);
+        // a look ahead at the next stage under this one's MMAs: even when the data are there, a wait takes 127 cycles
+        ready = __all_sync(0xFFFFFFFFu, i + 1 < n_kb && mbar_test(&full[s1], phase1));
         const uint32_t a = smem_u32(smem + (size_t)s * Cfg::kStageBytes);
         const uint32_t b = a + Cfg::kABytes;
 #pragma unroll
         for (int k = 0; k < kTileK / kUmmaK; ++k) {
-          umma_bf16(tmem_base, smem_desc_sw128(a + k * kUmmaK * 2), smem_desc_sw128(b + k * kUmmaK * 2), idesc,
-                    (i > 0 || k > 0) ? 1u : 0u);
+          umma_bf16_if(on, tmem_base, smem_desc_sw128(a + k * kUmmaK * 2), smem_desc_sw128(b + k * kUmmaK * 2), idesc,
+                       (i > 0 || k > 0) ? 1u : 0u);
         }
-        umma_commit(&empty[s]);   // frees the stage once these MMAs have read it
+        umma_commit_if(on, &empty[s]);   // frees the stage once these MMAs have read it
         s = s1;
         phase = phase1;
       }
       if (ok) {
-        umma_commit(tmem_full);
-      } else if (flags[0] == 0) {      // a wait of this thread expired (flags[0] != 0: someone else stopped the CTA)
+        umma_commit_if(on, tmem_full);
+      } else if (lane == 0 && flags[0] == 0) {      // a wait expired (flags[0] != 0: someone else stopped the CTA)
         if (err) atomicCAS(err, 0, -5);
         flags[0] = 1;
       }
@@ -532,69 +535,85 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
   auto fail = [&]() { if (*stop == 0) { if (err) atomicCAS(err, 0, -5); *stop = 1; } };
 
   if (warp == kPersistEpiWarps) {
-    if (lane == 0) {
-      uint32_t it = 0;
-      auto load_w = [&](uint8_t* a, uint64_t* bar, int kb, int n0) {
-        tma_load_2d(a, &tm_w, bar, kb * kTileK, n0);
-        if (GU) tma_load_2d(a + C::kABytes / 2, &tm_w, bar, kb * kTileK, N + n0);
-      };
-      // the weight tiles of the first ring of stages go out before the predecessors have finished
-      uint32_t ahead = 0;
-      if (blockIdx.x < n_tiles) {
-        int tm, tn;
-        tile_of(blockIdx.x, tm, tn);
-        for (; ahead < (uint32_t)min(C::kStages, total_kb); ++ahead) {
-          mbar_expect_tx(&full[ahead], C::kStageBytes);
-          load_w(smem + (size_t)ahead * C::kStageBytes, &full[ahead], ahead, tn * (GU ? kTileN / 2 : kTileN));
-        }
-      }
-      RSD_PDL_WAIT();
-      for (int t = blockIdx.x; t < n_tiles && !*stop; t += gridDim.x) {
-        int tm, tn;
-        tile_of(t, tm, tn);
-        const int n0 = tn * (GU ? kTileN / 2 : kTileN), m0 = tm * C::kRows;
-        for (int kb = 0; kb < total_kb; ++kb, ++it) {
-          const uint32_t s = it % C::kStages;
-          uint8_t* a = smem + (size_t)s * C::kStageBytes;
-          if (it >= ahead) {
-            if (!mbar_wait(&empty[s], ((it / C::kStages) & 1u) ^ 1u) || *stop) { fail(); break; }
-            mbar_expect_tx(&full[s], C::kStageBytes);
-            load_w(a, &full[s], kb, n0);
+    // ---------------- TMA producer: the whole warp walks the ring, one lane issues ----------------
+    const uint32_t on = elect_one();
+    uint32_t it = 0, s = 0, phase = 1;
+    bool ready = true;
+    auto load_w = [&](uint32_t st, int kb, int n0) {
+      uint8_t* a = smem + (size_t)st * C::kStageBytes;
+      mbar_expect_tx_if(on, &full[st], C::kStageBytes);
+      tma_load_2d_if(on, a, &tm_w, &full[st], kb * kTileK, n0);
+      if (GU) tma_load_2d_if(on, a + C::kABytes / 2, &tm_w, &full[st], kb * kTileK, N + n0);
+    };
+    // the weight tiles of the first ring of stages go out before the predecessors have finished
+    uint32_t ahead = 0;
+    if (blockIdx.x < n_tiles) {
+      int tm, tn;
+      tile_of(blockIdx.x, tm, tn);
+      for (; ahead < (uint32_t)min(C::kStages, total_kb); ++ahead) load_w(ahead, ahead, tn * (GU ? kTileN / 2 : kTileN));
+    }
+    RSD_PDL_WAIT();
+    bool ok = true;
+    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+      int tm, tn;
+      tile_of(t, tm, tn);
+      const int n0 = tn * (GU ? kTileN / 2 : kTileN), m0 = tm * C::kRows;
+      for (int kb = 0; kb < total_kb; ++kb, ++it) {
+        if (it >= ahead) {
+          if (!ready) {
+            ok = mbar_wait(&empty[s], phase);
+            ok = __all_sync(0xFFFFFFFFu, ok && !*stop);
+            if (!ok) break;
           }
-          tma_load_2d(a + C::kABytes, &tm_x, &full[s], kb * kTileK, m0);
-          if (SPLIT) tma_load_2d(a + C::kABytes + C::kRows * kTileK * 2, &tm_x_lo, &full[s], kb * kTileK, m0);
+          load_w(s, kb, n0);
         }
+        uint8_t* b = smem + (size_t)s * C::kStageBytes + C::kABytes;
+        tma_load_2d_if(on, b, &tm_x, &full[s], kb * kTileK, m0);
+        if (SPLIT) tma_load_2d_if(on, b + C::kRows * kTileK * 2, &tm_x_lo, &full[s], kb * kTileK, m0);
+        if (++s == (uint32_t)C::kStages) { s = 0; phase ^= 1u; }
+        ready = __all_sync(0xFFFFFFFFu, mbar_test(&empty[s], phase));
       }
-      if (*stop) {   // copies in flight must land before the CTA goes away
-        for (uint32_t i = (it > (uint32_t)C::kStages ? it - C::kStages : 0); i < it; ++i)
-          for (uint32_t k = 0; k < (1u << 16); ++k)
-            if (mbar_try_wait(&full[i % C::kStages], (i / C::kStages) & 1u)) break;
-      }
+    }
+    if (!ok) {
+      if (on) fail();
+      // copies in flight must land before the CTA goes away
+      for (uint32_t i = (it > (uint32_t)C::kStages ? it - C::kStages : 0); i < it; ++i)
+        for (uint32_t k = 0; k < (1u << 16); ++k)
+          if (mbar_try_wait(&full[i % C::kStages], (i / C::kStages) & 1u)) break;
     }
   } else if (warp == kPersistEpiWarps + 1) {
-    if (lane == 0) {
-      uint32_t it = 0, n_acc = 0;
-      for (int t = blockIdx.x; t < n_tiles && !*stop; t += gridDim.x, ++n_acc) {
-        const uint32_t b = n_acc & 1u;
-        if (!mbar_wait(&acc_empty[b], ((n_acc >> 1) & 1u) ^ 1u) || *stop) { fail(); break; }
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + b * (uint32_t)C::kMT;
-        bool ok = true;
-        for (int kb = 0; kb < total_kb; ++kb, ++it) {
-          const uint32_t s = it % C::kStages;
-          if (!mbar_wait(&full[s], (it / C::kStages) & 1u) || *stop) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t a = smem_u32(smem + (size_t)s * C::kStageBytes), bb = a + C::kABytes;
-#pragma unroll
-          for (int k = 0; k < kTileK / kUmmaK; ++k)
-            umma_bf16(d_tmem, smem_desc_sw128(a + k * kUmmaK * 2), smem_desc_sw128(bb + k * kUmmaK * 2), idesc,
-                      (kb > 0 || k > 0) ? 1u : 0u);
-          umma_commit(&empty[s]);
+    // ---------------- MMA issuer, likewise ----------------
+    const uint32_t on = elect_one();
+    uint32_t s = 0, phase = 0, n_acc = 0;
+    bool ok = true, ready = false;
+    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++n_acc) {
+      const uint32_t b = n_acc & 1u;
+      ok = mbar_wait(&acc_empty[b], ((n_acc >> 1) & 1u) ^ 1u);
+      ok = __all_sync(0xFFFFFFFFu, ok && !*stop);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + b * (uint32_t)C::kMT;
+      for (int kb = 0; kb < total_kb; ++kb) {
+        if (!ready) {
+          ok = mbar_wait(&full[s], phase);
+          ok = __all_sync(0xFFFFFFFFu, ok && !*stop);
+          if (!ok) break;
         }
-        if (!ok) { fail(); break; }
-        umma_commit(&acc_full[b]);
+        tc_fence_after();
+        const uint32_t s1 = s + 1 == (uint32_t)C::kStages ? 0u : s + 1, phase1 = s1 == 0 ? phase ^ 1u : phase;
+        ready = __all_sync(0xFFFFFFFFu, mbar_test(&full[s1], phase1));        // under this stage's MMAs
+        const uint32_t a = smem_u32(smem + (size_t)s * C::kStageBytes), bb = a + C::kABytes;
+#pragma unroll
+        for (int k = 0; k < kTileK / kUmmaK; ++k)
+          umma_bf16_if(on, d_tmem, smem_desc_sw128(a + k * kUmmaK * 2), smem_desc_sw128(bb + k * kUmmaK * 2), idesc,
+                       (kb > 0 || k > 0) ? 1u : 0u);
+        umma_commit_if(on, &empty[s]);
+        s = s1;
+        phase = phase1;
       }
+      if (ok) umma_commit_if(on, &acc_full[b]);
     }
+    if (!ok && on) fail();
   } else {
     // ---------------- epilogue warps ----------------
     const int quarter = warp & 3, col0 = (warp >> 2) * 16;
@@ -704,73 +723,86 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_const
   auto fail = [&]() { if (*stop == 0) { if (err) atomicCAS(err, 0, -5); *stop = 1; } };
 
   if (warp == kPersistEpiWarps) {
-    // ---------------- producer: this CTA's weight rows and its half of the operand rows ----------------
-    if (lane == 0) {
-      tma_prefetch_map(&tm_x);
-      uint32_t it = 0, ahead = 0;
-      auto load_w = [&](int s, int kb, int n0) {
-        uint8_t* a = smem + (size_t)s * C::kStageBytes;
-        const uint32_t bar = cluster_addr(&full[s], 0);
-        if (rank == 0) mbar_expect_tx(&full[s], 2 * C::kStageBytes);     // both CTAs' bytes
-        tma_load_2d_pair(a, &tm_w, bar, kb * kTileK, n0);
-        if (GU) tma_load_2d_pair(a + C::kABytes / 2, &tm_w, bar, kb * kTileK, N + n0);
-      };
-      // the weight tiles of the first ring of stages go out before the predecessors have finished
-      if (pair < n_tiles) {
-        int tm, tn;
-        tile_of(pair, tm, tn);
-        for (; ahead < (uint32_t)min(C::kStages, total_kb); ++ahead) load_w(ahead, ahead, first_feature(tn));
-      }
-      RSD_PDL_WAIT();
-      for (int t = pair; t < n_tiles && !*stop; t += n_pairs) {
-        int tm, tn;
-        tile_of(t, tm, tn);
-        const int n0 = first_feature(tn), m0 = tm * kRows;
-        for (int kb = 0; kb < total_kb; ++kb, ++it) {
-          const uint32_t s = it % C::kStages;
-          if (it >= ahead) {
-            if (!mbar_wait(&empty[s], ((it / C::kStages) & 1u) ^ 1u) || *stop) { fail(); break; }
-            load_w(s, kb, n0);
+    // ---------------- producer: this CTA's weight rows and its half of the operand rows; one lane issues ----------------
+    const uint32_t on = elect_one(), lead = on && rank == 0 ? 1u : 0u;
+    if (on) tma_prefetch_map(&tm_x);
+    uint32_t it = 0, s = 0, phase = 1, ahead = 0;
+    bool ready = true, ok = true;
+    auto load_w = [&](uint32_t st, int kb, int n0) {
+      uint8_t* a = smem + (size_t)st * C::kStageBytes;
+      const uint32_t bar = cluster_addr(&full[st], 0);
+      mbar_expect_tx_if(lead, &full[st], 2 * C::kStageBytes);     // both CTAs' bytes
+      tma_load_2d_pair_if(on, a, &tm_w, bar, kb * kTileK, n0);
+      if (GU) tma_load_2d_pair_if(on, a + C::kABytes / 2, &tm_w, bar, kb * kTileK, N + n0);
+    };
+    // the weight tiles of the first ring of stages go out before the predecessors have finished
+    if (pair < n_tiles) {
+      int tm, tn;
+      tile_of(pair, tm, tn);
+      for (; ahead < (uint32_t)min(C::kStages, total_kb); ++ahead) load_w(ahead, ahead, first_feature(tn));
+    }
+    RSD_PDL_WAIT();
+    for (int t = pair; t < n_tiles && ok; t += n_pairs) {
+      int tm, tn;
+      tile_of(t, tm, tn);
+      const int n0 = first_feature(tn), m0 = tm * kRows;
+      for (int kb = 0; kb < total_kb; ++kb, ++it) {
+        if (it >= ahead) {
+          if (!ready) {
+            ok = mbar_wait(&empty[s], phase);
+            ok = __all_sync(0xFFFFFFFFu, ok && !*stop);
+            if (!ok) break;
           }
-          uint8_t* b = smem + (size_t)s * C::kStageBytes + C::kABytes;
-          const uint32_t bar = cluster_addr(&full[s], 0);
-          if (SPLIT) tma_load_2d_pair(b, rank == 0 ? &tm_x : &tm_x_lo, bar, kb * kTileK, m0);
-          else tma_load_2d_pair(b, &tm_x, bar, kb * kTileK, m0 + (int)rank * 128);
+          load_w(s, kb, n0);
         }
+        uint8_t* b = smem + (size_t)s * C::kStageBytes + C::kABytes;
+        const uint32_t bar = cluster_addr(&full[s], 0);
+        if (SPLIT) tma_load_2d_pair_if(on, b, rank == 0 ? &tm_x : &tm_x_lo, bar, kb * kTileK, m0);
+        else tma_load_2d_pair_if(on, b, &tm_x, bar, kb * kTileK, m0 + (int)rank * 128);
+        if (++s == (uint32_t)C::kStages) { s = 0; phase ^= 1u; }
+        ready = __all_sync(0xFFFFFFFFu, mbar_test(&empty[s], phase));
       }
-      // the copies still in flight when a wait has run out report to the leader's barriers, which a follower cannot poll:
-      // a few milliseconds are far longer than any of them takes
-      if (*stop)
-        for (int i = 0; i < 4096; ++i) __nanosleep(1000);
+    }
+    if (!ok) {
+      if (on) fail();
+      // the copies still in flight report to the leader's barriers, which a follower cannot poll: a few milliseconds are far
+      // longer than any of them takes
+      for (int i = 0; i < 4096; ++i) __nanosleep(1000);
     }
   } else if (warp == kPersistEpiWarps + 1) {
-    // ---------------- MMA issuer: one thread of the leading CTA ----------------
-    if (lane == 0 && rank == 0) {
+    // ---------------- MMA issuer: one lane of the leading CTA ----------------
+    if (rank == 0) {
+      const uint32_t on = elect_one();
       uint32_t s = 0, phase = 0, n_acc = 0;
-      bool ready = false;
-      for (int t = pair; t < n_tiles && !*stop; t += n_pairs, ++n_acc) {
+      bool ok = true, ready = false;
+      for (int t = pair; t < n_tiles && ok; t += n_pairs, ++n_acc) {
         const uint32_t b = n_acc & 1u;
-        if (!mbar_wait(&acc_empty[b], ((n_acc >> 1) & 1u) ^ 1u) || *stop) { fail(); break; }
+        ok = mbar_wait(&acc_empty[b], ((n_acc >> 1) & 1u) ^ 1u);
+        ok = __all_sync(0xFFFFFFFFu, ok && !*stop);
+        if (!ok) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + b * 256u;
-        bool ok = true;
         for (int kb = 0; kb < total_kb; ++kb) {
-          if (!ready && (!mbar_wait(&full[s], phase) || *stop)) { ok = false; break; }
+          if (!ready) {
+            ok = mbar_wait(&full[s], phase);
+            ok = __all_sync(0xFFFFFFFFu, ok && !*stop);
+            if (!ok) break;
+          }
           tc_fence_after();
           const uint32_t s1 = s + 1 == (uint32_t)C::kStages ? 0u : s + 1, phase1 = s1 == 0 ? phase ^ 1u : phase;
-          ready = mbar_test(&full[s1], phase1);        // under this stage's MMAs (see the one-tile kernel)
+          ready = __all_sync(0xFFFFFFFFu, mbar_test(&full[s1], phase1));      // under this stage's MMAs
           const uint32_t a = smem_u32(smem + (size_t)s * C::kStageBytes), bb = a + C::kABytes;
 #pragma unroll
           for (int k = 0; k < kTileK / kUmmaK; ++k)
-            umma_f16_pair(d_tmem, smem_desc_sw128(a + k * kUmmaK * 2), smem_desc_sw128(bb + k * kUmmaK * 2), idesc,
-                          (kb > 0 || k > 0) ? 1u : 0u);
-          umma_commit_pair(&empty[s]);
+            umma_f16_pair_if(on, d_tmem, smem_desc_sw128(a + k * kUmmaK * 2), smem_desc_sw128(bb + k * kUmmaK * 2), idesc,
+                             (kb > 0 || k > 0) ? 1u : 0u);
+          umma_commit_pair_if(on, &empty[s]);
           s = s1;
           phase = phase1;
         }
-        if (!ok) { fail(); break; }
-        umma_commit_pair(&acc_full[b]);
+        if (ok) umma_commit_pair_if(on, &acc_full[b]);
       }
+      if (!ok && on) fail();
     }
   } else {
     // ---------------- epilogue warps of both CTAs ----------------
