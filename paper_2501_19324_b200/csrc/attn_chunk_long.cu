@@ -191,12 +191,16 @@ attn_chunk_long_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
       if (!ok) fail();
     }
   } else if (warp == kMmaWarp) {
-    // ---------------- the one MMA issuer ----------------
-    if (lane == 0) {
+    // ---------------- the one MMA issuer: a converged warp, one lane issues ----------------
+    {
+      const uint32_t on = elect_one();
       uint32_t it = 0, n_p[2] = {0, 0};
       bool ok = true;
       int seg = 0;
-      auto wait = [&](uint64_t* bar, uint32_t parity) { return mbar_wait(bar, parity, kProbeLimit) && !*stop; };
+      auto wait = [&](uint64_t* bar, uint32_t parity) {
+        const bool got = mbar_wait(bar, parity, kProbeLimit);
+        return __all_sync(0xFFFFFFFFu, got && !*stop) != 0;
+      };
       auto scores = [&](int j, uint32_t k_it) {
         const uint32_t a = smem_u32(smem + j * kQBytes);
         const uint64_t k_desc = desc_sw128(smem_u32(ring + (size_t)(k_it % kSlots) * kSlotBytes), 2048);
@@ -204,11 +208,11 @@ attn_chunk_long_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
         for (int hh = 0; hh < 2; ++hh)
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
-            umma_bf16(tmem_base + kColS + j * 128, smem_desc_sw128(a + hh * (kQBytes / 2) + kk * 32),
-                      k_desc + (uint64_t)((hh * 1024 + kk * 32) >> 4), kIdesc, (hh > 0 || kk > 0) ? 1u : 0u);
-        umma_commit(&mt->s_full[j]);
+            umma_bf16_if(on, tmem_base + kColS + j * 128, smem_desc_sw128(a + hh * (kQBytes / 2) + kk * 32),
+                         k_desc + (uint64_t)((hh * 1024 + kk * 32) >> 4), kIdesc, (hh > 0 || kk > 0) ? 1u : 0u);
+        umma_commit_if(on, &mt->s_full[j]);
       };
-      while (seg < n_ent && ok && !*stop) {
+      while (seg < n_ent && ok && !__any_sync(0xFFFFFFFFu, *stop)) {
         const Segment sg = segment_at(mt, seg, n_ent, QT);
         if (sg.row >= 0) {
           const int n_tiles = max(sg.n[0], sg.n[1]);
@@ -216,36 +220,38 @@ attn_chunk_long_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
           ok = wait(&mt->kv_full[it % kSlots], (it / kSlots) & 1u);
           if (!ok) break;
           tc_fence_after();
+#pragma unroll
           for (int j = 0; j < 2; ++j)
             if (sg.n[j] > 0) scores(j, it);
-          umma_commit(&mt->kv_empty[it % kSlots]);
+          umma_commit_if(on, &mt->kv_empty[it % kSlots]);
           for (int i = 0; i < n_tiles && ok; ++i) {
             const uint32_t v_it = it + 2 * i + 1, k_it = v_it + 1;
             ok = wait(&mt->kv_full[v_it % kSlots], (v_it / kSlots) & 1u);
             if (ok && i + 1 < n_tiles) ok = wait(&mt->kv_full[k_it % kSlots], (k_it / kSlots) & 1u);
-            for (int j = 0; j < 2 && ok; ++j) {
-              if (i >= sg.n[j]) continue;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+              if (!ok || i >= sg.n[j]) continue;
               ok = wait(&mt->p_full[j], n_p[j] & 1u);
-              if (!ok) break;
+              if (!ok) continue;
               ++n_p[j];
               tc_fence_after();
               const uint64_t v_desc = desc_sw32(smem_u32(ring + (size_t)(v_it % kSlots) * kSlotBytes));
 #pragma unroll
               for (int kk = 0; kk < kTilePages; ++kk)
-                umma_f16_ts(tmem_base + kColO + j * 128, tmem_base + kColS + j * 128 + kk * 8, v_desc + (uint64_t)((kk * kBlockBytes) >> 4),
-                            kIdesc, (i > 0 || kk > 0) ? 1u : 0u);
+                umma_f16_ts_if(on, tmem_base + kColO + j * 128, tmem_base + kColS + j * 128 + kk * 8,
+                               v_desc + (uint64_t)((kk * kBlockBytes) >> 4), kIdesc, (i > 0 || kk > 0) ? 1u : 0u);
               if (i + 1 < sg.n[j]) scores(j, k_it);
-              else umma_commit(&mt->o_full[j]);
+              else umma_commit_if(on, &mt->o_full[j]);
             }
             if (!ok) break;
-            umma_commit(&mt->kv_empty[v_it % kSlots]);
-            if (i + 1 < n_tiles) umma_commit(&mt->kv_empty[k_it % kSlots]);
+            umma_commit_if(on, &mt->kv_empty[v_it % kSlots]);
+            if (i + 1 < n_tiles) umma_commit_if(on, &mt->kv_empty[k_it % kSlots]);
           }
           it += 2 * n_tiles;
         }
         seg = sg.e;
       }
-      if (!ok) fail();
+      if (!ok && on) fail();
     }
   } else {
     // ---------------- softmax warps: thread = tile row = tensor-memory lane ----------------
