@@ -574,10 +574,12 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
     SplitSum qkv_pending, gu_pending, x_pending;
     int rc = gemm(c, M, M.wqkv[l], c->h, c->h_lo, c->qkv, T, (H + 2 * KV) * hd, d, 0, p.n_active, &qkv_pending, s, rs);
     if (rc) return rc;
-    CU(launch_rope_kv(M.kv_dtype, c->qkv, qkv_pending, p, c->q, kv, M.rope, H, KV, hd, s));
+    const QkvSource src{c->qkv, qkv_pending, M.rope};
+    const bool rotates = attn_decode_takes_qkv(M.kv_dtype, m.dtype, T, H, KV, c->S, c->attn_rows_hint, c->pass_width);
+    if (!rotates) CU(launch_rope_kv(M.kv_dtype, c->qkv, qkv_pending, p, c->q, kv, M.rope, H, KV, hd, s));
     CU(launch_attn_decode(M.kv_dtype, c->q, kv.pool_layer, kv.page_table, kv.max_pages, p.tok_row, p.tok_pos, 1,
                           c->attn, c->attn_lo, m.dtype, T, H, KV, hd, c->S, c->attn_scratch, c->attn_scratch_bytes,
-                          p.n_active, s, c->attn_rows_hint, c->pass_width));
+                          p.n_active, s, c->attn_rows_hint, c->pass_width, rotates ? &src : nullptr));
     rc = gemm(c, M, M.wo[l], c->attn, c->attn_lo, c->x, T, d, H * hd, 1, p.n_active, &x_pending, s);
     if (rc) return rc;
     CU(launch_reduce_norm(x_pending.partials, x_pending.splits, c->x, M.norm2[l], c->h, c->h_lo, c->norm_ssq, T, d,

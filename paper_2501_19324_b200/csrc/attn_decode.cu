@@ -12,18 +12,23 @@
 //        B fragment is one 64-bit load; the order of the tokens inside a page is permuted identically
 //        for P and V.
 // The warps' partial (max, sum, O) meet in shared memory.  With 2 to 8 context splits the splits of a (slot, KV
-// head) are the CTAs of one thread-block cluster: each leaves its partial in its own shared memory, and after a
-// cluster barrier every CTA merges a slice of the G x HD outputs out of all the CTAs' shared memory (in split
-// order) and writes it: no second launch and no trip through global memory.  With more splits than a cluster
-// holds the CTA writes its partial to scratch and a second kernel merges them.
-//
+// head) are the CTAs of one thread-block cluster: each sends every other CTA its partial of the slice of the G x HD outputs
+// that this one merges, and after a cluster barrier every CTA merges and writes its slice out of its own shared memory: no
+// second launch and no trip through global memory.  With more splits than a cluster holds the CTA writes its partial to
+// scratch and a second kernel merges them.
 //
 // In a decode pass only the pass's own tokens are written by the kernels just before: every page that ends ahead of the
 // pass's first new position is older than the pass.  Lists, page ids and each warp's first pages are therefore
 // requested before the wait for the preceding kernels and stream in while the qkv product and the rotation still run;
 // at the step loop's contexts (a page or two per warp) the cache has arrived when the query has.  (Fragments loaded from
 // global memory straight into registers had one page a warp in flight and none under the wait: 12.3 us a launch at 32
-// rows x 400 tokens, 12 / 2 heads, and 330 us for 64 rows x 4096-16384 tokens, 28 / 4 heads; now 9 us and 217 us.)
+// rows x 400 tokens, 12 / 2 heads, and 330 us for 64 rows x 4096-16384 tokens, 28 / 4 heads.)
+//
+// What is left after the wait is a chain of short steps.  Of the 5.8 us from the wait to the end at one row (12 / 2 heads,
+// a page per warp) 3.3 lay behind the last page: outputs stored with 8-way bank conflicts, one output dim a thread, loads
+// from the other CTAs' shared memory and a running maximum over them, a second cluster barrier; and the products of a page
+// formed one chain through the accumulators of the tile's padding rows.  As it stands: 3.8 us, 2.0 behind the last page;
+// 64 rows x 4096-16384 tokens: 201 us, the copy bandwidth.
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -33,7 +38,10 @@ namespace rsd {
 
 namespace {
 
+namespace cg = cooperative_groups;
+
 constexpr int kMaxSplits = 32;
+constexpr int kClusterSplits = 8;   // the portable cluster size
 
 // Two fp32 values rounded to the cache's 16-bit type and packed into one MMA operand register.
 template <typename KT> __device__ __forceinline__ uint32_t pack2(float lo, float hi);
@@ -53,24 +61,17 @@ template <typename KT> __device__ __forceinline__ void pack2_split(float a, floa
   lo = pack2<KT>(a - to_f32(ah), b - to_f32(bh));
 }
 
+// D += A B for a tile whose rows 8..15 are padding: their accumulators enter as zeros and what comes out is dropped, so
+// that no product waits for another one's padding.
 template <typename KT>
-__device__ __forceinline__ void mma_16816(float& d0, float& d1, float& d2, float& d3, uint32_t a0, uint32_t a1, uint32_t a2,
-                                          uint32_t a3, uint32_t b0, uint32_t b1);
-template <>
-__device__ __forceinline__ void mma_16816<__nv_bfloat16>(float& d0, float& d1, float& d2, float& d3, uint32_t a0, uint32_t a1,
-                                                         uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d0), "+f"(d1), "+f"(d2), "+f"(d3)
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-template <>
-__device__ __forceinline__ void mma_16816<__half>(float& d0, float& d1, float& d2, float& d3, uint32_t a0, uint32_t a1,
-                                                  uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d0), "+f"(d1), "+f"(d2), "+f"(d3)
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+__device__ __forceinline__ void mma_16816(float& d0, float& d1, uint32_t a0, uint32_t a2, uint32_t b0, uint32_t b1) {
+  float x, y;
+  if (std::is_same<KT, __half>::value)
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%8,%5,%8}, {%6,%7}, {%0,%1,%9,%9};"
+                 : "+f"(d0), "+f"(d1), "=f"(x), "=f"(y) : "r"(a0), "r"(a2), "r"(b0), "r"(b1), "r"(0u), "f"(0.f));
+  else
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%8,%5,%8}, {%6,%7}, {%0,%1,%9,%9};"
+                 : "+f"(d0), "+f"(d1), "=f"(x), "=f"(y) : "r"(a0), "r"(a2), "r"(b0), "r"(b1), "r"(0u), "f"(0.f));
 }
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -83,18 +84,20 @@ template <int HD, bool EXT> struct DecCfg {
   static constexpr int kPageBytes = (EXT ? 4 : 2) * kPageTokens * HD * 2;
   static constexpr int kStages = EXT ? 1 : 2;
   static constexpr int kRingBytes = 4 * kStages * kPageBytes;
-  static_assert(kRingBytes >= 4 * 8 * HD * 4, "the outputs of the four warps alias the ring");
+  static_assert(kRingBytes >= 4 * 8 * (HD + 8) * 4, "the outputs of the four warps alias the ring");
 };
 
 // part_o: [slot][head][split][HD] un-normalised outputs; part_ml: [slot][head][split][2] (max, sum).
 // EXT: queries and softmax weights enter the products as hi + lo pairs and every page carries the low
 // halves of its keys and values in two more blocks: the attention is accurate to about 2^-20.
 // new_tokens: how many of a row's last positions the pass itself writes.
-template <int HD, typename KT, typename OT, bool EXT, bool CL>
+// FUSE (one split; every row's only new position is its last): the kernel takes the qkv product itself, K-split partial sums or
+// not, adds them up, rotates, and writes the new key and value to the cache: see new_token below.
+template <int HD, typename KT, typename OT, bool EXT, bool CL, bool FUSE>
 __global__ void __launch_bounds__(128, 3)
-attn_decode_kernel(const float* q, const KT* pool, const int32_t* page_table, int max_pages, const int32_t* slot_row,
+attn_decode_kernel(const float* q, KT* pool, const int32_t* page_table, int max_pages, const int32_t* slot_row,
                    const int32_t* len_or_pos, int len_offset, OT* out, OT* out_lo, float* part_o, float* part_ml, int H, int KV,
-                   int n_splits, const int32_t* n_active, int new_tokens) {
+                   int n_splits, const int32_t* n_active, int new_tokens, const float* partials, int k_splits, const float2* rope) {
   RSD_PDL_TRIGGER();
   if (n_active == nullptr) RSD_PDL_WAIT();   // a decode pass's lists and old pages may be read ahead of the wait, others not
   using Cfg = DecCfg<HD, EXT>;
@@ -104,7 +107,7 @@ attn_decode_kernel(const float* q, const KT* pool, const int32_t* page_table, in
   constexpr int kStages = Cfg::kStages, kParts = EXT ? 4 : 2;
   extern __shared__ __align__(128) uint8_t ring_raw[];
   __shared__ float s_m[4][8], s_l[4][8];
-  auto s_o = reinterpret_cast<float(*)[8][HD]>(ring_raw);
+  auto s_o = reinterpret_cast<float(*)[8][HD + 8]>(ring_raw);   // rows 32 bytes apart modulo 128: the fragments' stores do not collide
   const int kvh = blockIdx.x, slot = blockIdx.y, split = blockIdx.z;
   const bool idle = n_active != nullptr && ld_cg(n_active) == 0;
   const int row = slot_row ? ld_cg(slot_row + slot) : slot;
@@ -136,7 +139,9 @@ attn_decode_kernel(const float* q, const KT* pool, const int32_t* page_table, in
       }
     }
   };
-  const int first = p_begin + warp, n_old = (ctx - new_tokens) / kPageTokens;   // pages [0, n_old) are older than the pass
+  // pages [0, n_old) may be read ahead of the wait: they are older than the pass, or (FUSE) all but the token that this
+  // kernel fills in itself
+  const int first = p_begin + warp, n_old = FUSE ? n_pages : (ctx - new_tokens) / kPageTokens;
   int next = first;                              // the page whose turn it is to be fetched
   int next_id = next < p_end ? ld_cg(pt + next) : 0;
   auto fetch_next = [&](int stage) {
@@ -149,19 +154,118 @@ attn_decode_kernel(const float* q, const KT* pool, const int32_t* page_table, in
   };
   int fetched = 0;
   for (; fetched < kStages && next < min(p_end, n_old); ++fetched) fetch_next(fetched);
+  for (; FUSE && fetched < kStages; ++fetched) fetch_next(fetched);
+  // every CTA of the cluster runs before the others write to its shared memory
+  if (CL) cg::this_cluster().barrier_arrive();
   RSD_PDL_WAIT();
   for (; fetched < kStages; ++fetched) fetch_next(fetched);
 
-  // the group's queries, rounded once by the whole block: one coalesced round of loads
+  // the group's queries, rounded once by the whole block
   constexpr int kLd = HD + 32;                   // rows 64 bytes apart modulo 128: the fragment loads below do not collide
   __shared__ __align__(16) KT s_q[EXT ? 2 : 1][8][kLd];
+  __shared__ __align__(16) KT s_new[FUSE ? kParts : 1][HD];   // the new token's key and value (and their low halves)
+  const int new_page = (ctx - 1) / kPageTokens, new_slot = (ctx - 1) % kPageTokens;
+  if (FUSE) {
+    // new_token.  A task is four neighbouring pairs (i, i + HD / 2) of a query head, of the key or of the value, with all
+    // its K splits in flight at once.
+    constexpr int NQ = HD / 8, kAhead = 3;
+    const int n_tasks = (G + 2) * NQ, width = (H + 2 * KV) * HD;
+    const size_t sstride = (size_t)gridDim.y * width;
+    const int per = (k_splits + kSumGroups - 1) / kSumGroups;
+    for (int idx = threadIdx.x; idx < (8 - G) * HD; idx += 128) {   // the tile's rows beyond the group
+      s_q[0][G + idx / HD][idx % HD] = from_f32<KT>(0.f);
+      if (EXT) s_q[EXT ? 1 : 0][G + idx / HD][idx % HD] = from_f32<KT>(0.f);
+    }
+    for (int task = threadIdx.x; task < n_tasks; task += 128) {
+      const bool is_q = task < G * NQ;
+      const int hh = is_q ? task / NQ : task / NQ - G, dd = 4 * (task % NQ);   // one of the group's heads, or 0 = the key, 1 = the value
+      const size_t src = (size_t)slot * width + (size_t)(is_q ? h0 + hh : H + hh * KV + kvh) * HD + dd;
+      float a[4] = {0.f, 0.f, 0.f, 0.f}, b[4] = {0.f, 0.f, 0.f, 0.f};
+      if (k_splits <= 1) {
+        *reinterpret_cast<float4*>(a) = ld_cg(reinterpret_cast<const float4*>(q + src));
+        *reinterpret_cast<float4*>(b) = ld_cg(reinterpret_cast<const float4*>(q + src + HD / 2));
+      } else {
+        // the order of the additions is rope_kv_kernel's: kSumGroups runs of splits, then their sums
+        float ga[kSumGroups][4], gb[kSumGroups][4];
 #pragma unroll
-  for (int i = 0; i < 8 * HD / 128; ++i) {
-    const int idx = i * 128 + threadIdx.x, gg = idx / HD, dd = idx % HD;
-    const float v = gg < G ? q[((size_t)slot * H + h0 + gg) * HD + dd] : 0.f;
-    const KT hi = from_f32<KT>(v);
-    s_q[0][gg][dd] = hi;
-    if (EXT) s_q[EXT ? 1 : 0][gg][dd] = from_f32<KT>(v - to_f32(hi));
+        for (int r = 0; r < kSumGroups; ++r)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) ga[r][i] = gb[r][i] = 0.f;
+        for (int s0 = 0; s0 < per; s0 += kAhead) {
+          float4 ta[kSumGroups][kAhead], tb[kSumGroups][kAhead];
+#pragma unroll
+          for (int r = 0; r < kSumGroups; ++r)
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u)
+              if (s0 + u < per && r * per + s0 + u < k_splits) {
+                const float* at = partials + (size_t)(r * per + s0 + u) * sstride + src;
+                ta[r][u] = ld_cg(reinterpret_cast<const float4*>(at));
+                tb[r][u] = ld_cg(reinterpret_cast<const float4*>(at + HD / 2));
+              }
+#pragma unroll
+          for (int r = 0; r < kSumGroups; ++r)
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u)
+              if (s0 + u < per && r * per + s0 + u < k_splits) {
+                ga[r][0] += ta[r][u].x; ga[r][1] += ta[r][u].y; ga[r][2] += ta[r][u].z; ga[r][3] += ta[r][u].w;
+                gb[r][0] += tb[r][u].x; gb[r][1] += tb[r][u].y; gb[r][2] += tb[r][u].z; gb[r][3] += tb[r][u].w;
+              }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          a[i] = ((ga[0][i] + ga[1][i]) + ga[2][i]) + ga[3][i];
+          b[i] = ((gb[0][i] + gb[1][i]) + gb[2][i]) + gb[3][i];
+        }
+      }
+      if (is_q || hh == 0) {
+        const float2* cs = rope + (size_t)(ctx - 1) * (HD / 2) + dd;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float ra = rotate_lo(a[i], b[i], cs[i]), rb = rotate_hi(a[i], b[i], cs[i]);
+          a[i] = ra; b[i] = rb;
+        }
+      }
+      __align__(8) KT hi[2][4], lo[2][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        hi[0][i] = from_f32<KT>(a[i]); lo[0][i] = from_f32<KT>(a[i] - to_f32(hi[0][i]));
+        hi[1][i] = from_f32<KT>(b[i]); lo[1][i] = from_f32<KT>(b[i] - to_f32(hi[1][i]));
+      }
+      if (is_q) {
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          *reinterpret_cast<uint2*>(&s_q[0][hh][half * (HD / 2) + dd]) = *reinterpret_cast<const uint2*>(hi[half]);
+          if (EXT) *reinterpret_cast<uint2*>(&s_q[EXT ? 1 : 0][hh][half * (HD / 2) + dd]) = *reinterpret_cast<const uint2*>(lo[half]);
+        }
+      } else {
+        KT* blk = pool + (size_t)ld_cg(pt + new_page) * page_elems + (size_t)hh * KV * kBlock + (size_t)kvh * kBlock;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          const int d0 = half * (HD / 2) + dd;
+          *reinterpret_cast<uint2*>(&s_new[hh][d0]) = *reinterpret_cast<const uint2*>(hi[half]);
+          if (EXT) *reinterpret_cast<uint2*>(&s_new[EXT ? hh + 2 : 0][d0]) = *reinterpret_cast<const uint2*>(lo[half]);
+          if (hh == 0) {
+            *reinterpret_cast<uint2*>(blk + new_slot * HD + d0) = *reinterpret_cast<const uint2*>(hi[half]);
+            if (EXT) *reinterpret_cast<uint2*>(blk + (size_t)2 * KV * kBlock + new_slot * HD + d0) = *reinterpret_cast<const uint2*>(lo[half]);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              blk[(d0 + i) * kPageTokens + new_slot] = hi[half][i];
+              if (EXT) blk[(size_t)2 * KV * kBlock + (d0 + i) * kPageTokens + new_slot] = lo[half][i];
+            }
+          }
+        }
+      }
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8 * HD / 128; ++i) {     // one coalesced round of loads
+      const int idx = i * 128 + threadIdx.x, gg = idx / HD, dd = idx % HD;
+      const float v = gg < G ? q[((size_t)slot * H + h0 + gg) * HD + dd] : 0.f;
+      const KT hi = from_f32<KT>(v);
+      s_q[0][gg][dd] = hi;
+      if (EXT) s_q[EXT ? 1 : 0][gg][dd] = from_f32<KT>(v - to_f32(hi));
+    }
   }
   __syncthreads();
   // Q fragments (rows 8..15 of the tile are padding): dims 32j + 8t + e of head h0 + g
@@ -171,12 +275,9 @@ attn_decode_kernel(const float* q, const KT* pool, const int32_t* page_table, in
     *reinterpret_cast<uint4*>(qa[j]) = *reinterpret_cast<const uint4*>(&s_q[0][g][32 * j + 8 * t]);
     if (EXT) *reinterpret_cast<uint4*>(ql[EXT ? j : 0]) = *reinterpret_cast<const uint4*>(&s_q[EXT ? 1 : 0][g][32 * j + 8 * t]);
   }
-  // Rows 8..15 of every MMA tile are padding (their A rows are zero), so all tiles share two dump
-  // registers for those rows instead of carrying 2 x (NT + 2) dead accumulators.
   float o[NT][2];
 #pragma unroll
   for (int i = 0; i < NT; ++i) { o[i][0] = o[i][1] = 0.f; }
-  float dump0 = 0.f, dump1 = 0.f;
   float m_run = -INFINITY, l_run = 0.f;
   // tokens whose keys this lane loads: tile 0 -> 4(g/2) + g%2, tile 1 -> that + 2 (the same parity)
   const int tok0 = 4 * (g >> 1) + (g & 1), tok1 = tok0 + 2;
@@ -186,29 +287,42 @@ attn_decode_kernel(const float* q, const KT* pool, const int32_t* page_table, in
   for (int p = first; p < p_end; p += 4) {
     asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 1) : "memory");
     __syncwarp();
-    const KT* kb = ring + stage * kParts * kBlock;
-    const KT* vb = kb + kBlock;
+    KT* kb = ring + stage * kParts * kBlock;
+    KT* vb = kb + kBlock;
+    if (FUSE && p == new_page) {
+      // the page was fetched before its last token was known
+#pragma unroll
+      for (int part = 0; part < kParts; part += 2) {
+        if (lane < HD / 8)
+          *reinterpret_cast<uint4*>(kb + part * kBlock + new_slot * HD + (lane ^ ((new_slot & 1) << 2)) * 8) =
+              *reinterpret_cast<const uint4*>(&s_new[part][lane * 8]);
+#pragma unroll
+        for (int i = 0; i < HD / 32; ++i)
+          vb[part * kBlock + (i * 32 + lane) * kPageTokens + new_slot] = s_new[FUSE ? part + 1 : 0][i * 32 + lane];
+      }
+      __syncwarp();
+    }
     float s0[2] = {0.f, 0.f}, s1[2] = {0.f, 0.f};
 #pragma unroll
     for (int j = 0; j < KB; ++j) {
       const int off = (32 * j) ^ key_off;        // chunk 4j + t, swizzled
       const uint4 k0 = *reinterpret_cast<const uint4*>(kb + tok0 * HD + off);
       const uint4 k1 = *reinterpret_cast<const uint4*>(kb + tok1 * HD + off);
-      mma_16816<KT>(s0[0], s0[1], dump0, dump1, qa[j][0][0], 0u, qa[j][0][1], 0u, k0.x, k0.y);
-      mma_16816<KT>(s0[0], s0[1], dump0, dump1, qa[j][1][0], 0u, qa[j][1][1], 0u, k0.z, k0.w);
-      mma_16816<KT>(s1[0], s1[1], dump0, dump1, qa[j][0][0], 0u, qa[j][0][1], 0u, k1.x, k1.y);
-      mma_16816<KT>(s1[0], s1[1], dump0, dump1, qa[j][1][0], 0u, qa[j][1][1], 0u, k1.z, k1.w);
+      mma_16816<KT>(s0[0], s0[1], qa[j][0][0], qa[j][0][1], k0.x, k0.y);
+      mma_16816<KT>(s0[0], s0[1], qa[j][1][0], qa[j][1][1], k0.z, k0.w);
+      mma_16816<KT>(s1[0], s1[1], qa[j][0][0], qa[j][0][1], k1.x, k1.y);
+      mma_16816<KT>(s1[0], s1[1], qa[j][1][0], qa[j][1][1], k1.z, k1.w);
       if (EXT) {
         const uint4 e0 = *reinterpret_cast<const uint4*>(kb + 2 * kBlock + tok0 * HD + off);
         const uint4 e1 = *reinterpret_cast<const uint4*>(kb + 2 * kBlock + tok1 * HD + off);
-        mma_16816<KT>(s0[0], s0[1], dump0, dump1, qa[j][0][0], 0u, qa[j][0][1], 0u, e0.x, e0.y);
-        mma_16816<KT>(s0[0], s0[1], dump0, dump1, qa[j][1][0], 0u, qa[j][1][1], 0u, e0.z, e0.w);
-        mma_16816<KT>(s1[0], s1[1], dump0, dump1, qa[j][0][0], 0u, qa[j][0][1], 0u, e1.x, e1.y);
-        mma_16816<KT>(s1[0], s1[1], dump0, dump1, qa[j][1][0], 0u, qa[j][1][1], 0u, e1.z, e1.w);
-        mma_16816<KT>(s0[0], s0[1], dump0, dump1, ql[j][0][0], 0u, ql[j][0][1], 0u, k0.x, k0.y);
-        mma_16816<KT>(s0[0], s0[1], dump0, dump1, ql[j][1][0], 0u, ql[j][1][1], 0u, k0.z, k0.w);
-        mma_16816<KT>(s1[0], s1[1], dump0, dump1, ql[j][0][0], 0u, ql[j][0][1], 0u, k1.x, k1.y);
-        mma_16816<KT>(s1[0], s1[1], dump0, dump1, ql[j][1][0], 0u, ql[j][1][1], 0u, k1.z, k1.w);
+        mma_16816<KT>(s0[0], s0[1], qa[j][0][0], qa[j][0][1], e0.x, e0.y);
+        mma_16816<KT>(s0[0], s0[1], qa[j][1][0], qa[j][1][1], e0.z, e0.w);
+        mma_16816<KT>(s1[0], s1[1], qa[j][0][0], qa[j][0][1], e1.x, e1.y);
+        mma_16816<KT>(s1[0], s1[1], qa[j][1][0], qa[j][1][1], e1.z, e1.w);
+        mma_16816<KT>(s0[0], s0[1], ql[j][0][0], ql[j][0][1], k0.x, k0.y);
+        mma_16816<KT>(s0[0], s0[1], ql[j][1][0], ql[j][1][1], k0.z, k0.w);
+        mma_16816<KT>(s1[0], s1[1], ql[j][0][0], ql[j][0][1], k1.x, k1.y);
+        mma_16816<KT>(s1[0], s1[1], ql[j][1][0], ql[j][1][1], k1.z, k1.w);
       }
     }
     // this lane's scores of head g: tokens 4t, 4t+1 (tile 0) and 4t+2, 4t+3 (tile 1) of the page
@@ -240,11 +354,11 @@ attn_decode_kernel(const float* q, const KT* pool, const int32_t* page_table, in
     for (int i = 0; i < NT; ++i) {
       const uint2 vv = *reinterpret_cast<const uint2*>(vb + (8 * i + g) * kPageTokens + 4 * t);
       o[i][0] *= corr; o[i][1] *= corr;
-      mma_16816<KT>(o[i][0], o[i][1], dump0, dump1, pa0, 0u, pa2, 0u, vv.x & mlo, vv.y & mhi);
+      mma_16816<KT>(o[i][0], o[i][1], pa0, pa2, vv.x & mlo, vv.y & mhi);
       if (EXT) {
         const uint2 vl = *reinterpret_cast<const uint2*>(vb + 2 * kBlock + (8 * i + g) * kPageTokens + 4 * t);
-        mma_16816<KT>(o[i][0], o[i][1], dump0, dump1, pl0, 0u, pl2, 0u, vv.x & mlo, vv.y & mhi);
-        mma_16816<KT>(o[i][0], o[i][1], dump0, dump1, pa0, 0u, pa2, 0u, vl.x & mlo, vl.y & mhi);
+        mma_16816<KT>(o[i][0], o[i][1], pl0, pl2, vv.x & mlo, vv.y & mhi);
+        mma_16816<KT>(o[i][0], o[i][1], pa0, pa2, vl.x & mlo, vl.y & mhi);
       }
     }
     __syncwarp();                                // every lane has read the buffer
@@ -258,73 +372,66 @@ attn_decode_kernel(const float* q, const KT* pool, const int32_t* page_table, in
   l_run += __shfl_xor_sync(0xFFFFFFFFu, l_run, 2);
   if (t == 0) { s_m[warp][g] = m_run; s_l[warp][g] = l_run; }
 #pragma unroll
-  for (int i = 0; i < NT; ++i) {
-    s_o[warp][g][8 * i + 2 * t] = o[i][0];
-    s_o[warp][g][8 * i + 2 * t + 1] = o[i][1];
-  }
+  for (int i = 0; i < NT; ++i) *reinterpret_cast<float2*>(&s_o[warp][g][8 * i + 2 * t]) = make_float2(o[i][0], o[i][1]);
+  // Cluster mode: rank r of n merges the outputs [r * per, r * per + per) of the G x HD; every CTA leaves its partial of
+  // them (and its max and sum per head) in r's shared memory, outside the ring, which r may still be reading pages from.
+  constexpr int kRecv = CL ? 8 * HD : 4;
+  __shared__ __align__(16) float r_o[kRecv + (CL ? 4 * kClusterSplits : 0)];
+  __shared__ float2 r_ml[CL ? kClusterSplits : 1][8];
+  const int n_rank = CL ? n_splits : 1, total = G * HD;
+  const int per = 4 * ((total / 4 + n_rank - 1) / n_rank);
+  if (CL) cg::this_cluster().barrier_wait();
   __syncthreads();
-  __shared__ float c_m[8], c_l[8];               // cluster mode: this CTA's (max, sum) per head; its O goes to s_o[0]
-  for (int idx = threadIdx.x; idx < G * HD; idx += blockDim.x) {
+  for (int idx = 4 * threadIdx.x; idx < total; idx += 4 * 128) {
     const int gg = idx / HD, dd = idx % HD;
-    float M = fmaxf(fmaxf(s_m[0][gg], s_m[1][gg]), fmaxf(s_m[2][gg], s_m[3][gg]));
-    float L = 0.f, O = 0.f;
+    const float M = fmaxf(fmaxf(s_m[0][gg], s_m[1][gg]), fmaxf(s_m[2][gg], s_m[3][gg]));
+    float L = 0.f, O[4] = {0.f, 0.f, 0.f, 0.f};
     if (M > -INFINITY) {
 #pragma unroll
       for (int w = 0; w < 4; ++w) {
         const float e = __expf(s_m[w][gg] - M);
+        const float4 v = *reinterpret_cast<const float4*>(&s_o[w][gg][dd]);
         L += s_l[w][gg] * e;
-        O += s_o[w][gg][dd] * e;
+        O[0] += v.x * e; O[1] += v.y * e; O[2] += v.z * e; O[3] += v.w * e;
       }
     }
     const int h = h0 + gg;
     if (CL) {
-      // (gg, dd) is this thread's alone: it has read the four warps' values and may overwrite the first
-      s_o[0][gg][dd] = O;
-      if (dd == 0) { c_m[gg] = M; c_l[gg] = L; }
+      const int r = idx / per;
+      *reinterpret_cast<float4*>(cg::this_cluster().map_shared_rank(r_o, r) + split * per + idx - r * per) = make_float4(O[0], O[1], O[2], O[3]);
+      if (dd < 4 * n_rank) *cg::this_cluster().map_shared_rank(&r_ml[split][gg], dd / 4) = make_float2(M, L);
     } else if (n_splits == 1) {
-      store_operand<OT>(out, out_lo, ((size_t)slot * H + h) * HD + dd, O / L);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) O[i] /= L;
+      store_operand4<OT>(out, out_lo, ((size_t)slot * H + h) * HD + dd, O);
     } else {
       const size_t base = ((size_t)slot * H + h) * n_splits + split;
-      part_o[base * HD + dd] = O;
+      *reinterpret_cast<float4*>(part_o + base * HD + dd) = make_float4(O[0], O[1], O[2], O[3]);
       if (dd == 0) { part_ml[base * 2] = M; part_ml[base * 2 + 1] = L; }
     }
   }
   if (CL) {
-    // Every CTA of the cluster gets here (the early returns above depend on the slot alone, which the cluster
-    // shares).  Rank = split.  A CTA merges the outputs [rank * per, rank * per + per) of the G x HD.
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    cluster.sync();
-    const int n_rank = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-    const int total = G * HD, per = (total + n_rank - 1) / n_rank;
-    const int end = min(total, (rank + 1) * per);
-    for (int idx = rank * per + threadIdx.x; idx < end; idx += blockDim.x) {
-      const int gg = idx / HD, dd = idx % HD;
-      float pm[8], pl[8], po[8];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        if (r < n_rank) {
-          pm[r] = *cluster.map_shared_rank(&c_m[gg], r);
-          pl[r] = *cluster.map_shared_rank(&c_l[gg], r);
-          po[r] = *cluster.map_shared_rank(&s_o[0][gg][dd], r);
-        } else {
-          pm[r] = -INFINITY; pl[r] = 0.f; po[r] = 0.f;
-        }
-      }
+    // Every CTA of the cluster gets here (the early returns above depend on the slot alone, which the cluster shares),
+    // and none touches another's shared memory after the barrier.
+    cg::this_cluster().sync();
+    const int idx = split * per + threadIdx.x, end = min(total, (split + 1) * per);
+    for (int k = idx; k < end; k += 128) {
+      const int gg = k / HD, dd = k % HD;
+      float2 ml[kClusterSplits];
       float M = -INFINITY, L = 0.f, O = 0.f;
 #pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        if (pm[r] > -INFINITY) {
-          const float Mn = fmaxf(M, pm[r]);
-          const float e_old = __expf(M - Mn), e_new = __expf(pm[r] - Mn);
-          L = L * e_old + pl[r] * e_new;
-          O = O * e_old + po[r] * e_new;
-          M = Mn;
-        }
+      for (int r = 0; r < kClusterSplits; ++r) {
+        ml[r] = r < n_rank ? r_ml[CL ? r : 0][gg] : make_float2(-INFINITY, 0.f);
+        M = fmaxf(M, ml[r].x);
+      }
+#pragma unroll
+      for (int r = 0; r < kClusterSplits; ++r) {
+        const float e = __expf(ml[r].x - M);     // a split without pages: max -inf, weight 0; split 0 always has some
+        L += ml[r].y * e;
+        O += (r < n_rank ? r_o[r * per + k - split * per] : 0.f) * e;
       }
       store_operand<OT>(out, out_lo, ((size_t)slot * H + h0 + gg) * HD + dd, O / L);
     }
-    cluster.sync();                              // nobody leaves while its shared memory may still be read
   }
 }
 
@@ -374,8 +481,6 @@ __global__ void decode_slots_kernel(const int32_t* slot_row, const int32_t* len_
   pos[i] = ctx - 1;
 }
 
-constexpr int kClusterSplits = 8;   // the portable cluster size
-
 // Splits of a row's context.  One wave of at most three CTAs per SM when that leaves short splits: a second, partial wave
 // would double the time (16 rows x 1000-2048 tokens, 28 / 4 heads: 21 us in one wave, 29 us with eight splits).  Splits
 // of 64 pages and more are worth several waves instead, since rows of different lengths then even out (64 rows x
@@ -423,16 +528,25 @@ size_t attn_decode_scratch_bytes(int B, int H, int hd, int max_ctx) {
   return sizeof(int32_t) * 2 * (size_t)B + 256 + partials;
 }
 
+bool attn_decode_takes_qkv(int kv_dtype, int out_dtype, int B, int H, int KV, int max_ctx, int active_rows, int new_tokens) {
+  // With the context split over a cluster every CTA would add up the query for itself, or wait for its share from the
+  // others: a rotation kernel ahead is faster there (iteration of 14 layers, 12 / 2 heads: 525 us at one row and 739 at 32
+  // against 583 and 794; at 128 rows, in one split, 1275 with the rotation kernel and 1206 without).
+  return kv_dtype >= 2 && H / KV <= 8 && out_dtype == 1 && new_tokens == 1 &&
+         pick_splits(active_rows > 0 ? std::min(active_rows, B) : B, KV, max_ctx) == 1;
+}
+
 cudaError_t launch_attn_decode(int kv_dtype, const float* q, const void* pool_layer, const int32_t* page_table,
                                int max_pages, const int32_t* slot_row, const int32_t* len_or_pos, int len_offset,
                                void* out, void* out_lo, int out_dtype, int B, int H, int KV, int hd, int max_ctx,
                                void* scratch, size_t scratch_bytes, const int32_t* n_active, cudaStream_t s, int active_rows,
-                               int new_tokens) {
+                               int new_tokens, const QkvSource* qkv) {
   if (B <= 0) return cudaSuccess;
   if (!scratch || scratch_bytes < attn_decode_scratch_bytes(B, H, hd, max_ctx)) return cudaErrorInvalidValue;
   const int G = H / KV;
   int32_t* row = (int32_t*)scratch;
   int32_t* pos = row + B;
+  if (qkv != nullptr && !attn_decode_takes_qkv(kv_dtype, out_dtype, B, H, KV, max_ctx, active_rows, new_tokens)) return cudaErrorInvalidValue;
   if (kv_dtype == 0 || G > 8) {
     // fp32 caches and wide groups take the generic kernel
     PassView p{nullptr, slot_row, len_or_pos, B, n_active};
@@ -450,31 +564,38 @@ cudaError_t launch_attn_decode(int kv_dtype, const float* q, const void* pool_la
   const int splits = pick_splits(active_rows > 0 ? std::min(active_rows, B) : B, KV, max_ctx);
   const bool clustered = splits >= 2 && splits <= kClusterSplits;
   dim3 grid(KV, B, splits);
-#define RSD_DEC(HD, KT, OT, EXTV)                                                                                          \
+#define RSD_DEC_K(HD, KT, OT, EXTV, CLV, FUSEV)                                                                        \
   do {                                                                                                               \
-    static const cudaError_t set_ = [] {                                                                             \
-      cudaError_t e = cudaFuncSetAttribute(attn_decode_kernel<HD, KT, OT, EXTV, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                           DecCfg<HD, EXTV>::kRingBytes);                                            \
-      return e != cudaSuccess ? e : cudaFuncSetAttribute(attn_decode_kernel<HD, KT, OT, EXTV, false>,                \
+    static const cudaError_t set_ = cudaFuncSetAttribute(attn_decode_kernel<HD, KT, OT, EXTV, CLV, FUSEV>,           \
                                                          cudaFuncAttributeMaxDynamicSharedMemorySize, DecCfg<HD, EXTV>::kRingBytes); \
-    }();                                                                                                             \
     if (set_ != cudaSuccess) return set_;                                                                            \
-    if (clustered)                                                                                                   \
-      (void)launch_decode(attn_decode_kernel<HD, KT, OT, EXTV, true>, grid, splits, DecCfg<HD, EXTV>::kRingBytes, s, q, (const KT*)pool_layer, page_table,       \
-                          max_pages, slot_row, len_or_pos, len_offset, (OT*)out, (OT*)out_lo, part_o, part_ml, H, KV, splits, n_active, new_tokens); \
-    else                                                                                                             \
-      (void)launch_decode(attn_decode_kernel<HD, KT, OT, EXTV, false>, grid, 1, DecCfg<HD, EXTV>::kRingBytes, s, q, (const KT*)pool_layer, page_table,           \
-                          max_pages, slot_row, len_or_pos, len_offset, (OT*)out, (OT*)out_lo, part_o, part_ml, H, KV, splits, n_active, new_tokens); \
+    (void)launch_decode(attn_decode_kernel<HD, KT, OT, EXTV, CLV, FUSEV>, grid, clustered ? splits : 1, DecCfg<HD, EXTV>::kRingBytes, s, \
+                        FUSEV ? qkv->qkv : q, (KT*)pool_layer, page_table, max_pages, slot_row, len_or_pos, len_offset, (OT*)out, \
+                        (OT*)out_lo, part_o, part_ml, H, KV, splits, n_active, new_tokens, FUSEV ? qkv->pending.partials : nullptr, \
+                        FUSEV ? qkv->pending.splits : 1, FUSEV ? qkv->rope : nullptr);                               \
+  } while (0)
+#define RSD_DEC(HD, KT, OT, EXTV, FUSEV)                                                                              \
+  do {                                                                                                               \
+    if (clustered) RSD_DEC_K(HD, KT, OT, EXTV, true, false);                                                          \
+    else RSD_DEC_K(HD, KT, OT, EXTV, false, FUSEV);                                                                   \
     if (splits > 1 && !clustered)                                                                                    \
       RSD_LAUNCH((attn_merge_kernel<HD, OT>), dim3(H, B), HD, 0, s, part_o, part_ml, slot_row, len_or_pos, len_offset, (OT*)out, \
                                                           (OT*)out_lo, H, splits, n_active);                         \
   } while (0)
-#define RSD_DEC_O(HD, KT, EXTV) do { if (out_dtype == 1) RSD_DEC(HD, KT, __nv_bfloat16, EXTV); else RSD_DEC(HD, KT, float, EXTV); } while (0)
+#define RSD_DEC_O(HD, KT, EXTV)                                                                                       \
+  do {                                                                                                               \
+    if (qkv != nullptr) RSD_DEC(HD, KT, __nv_bfloat16, EXTV, true);                                                   \
+    else if (out_dtype == 1) RSD_DEC(HD, KT, __nv_bfloat16, EXTV, false);                                             \
+    else RSD_DEC(HD, KT, float, EXTV, false);                                                                         \
+  } while (0)
+  // (a model of the engine has a 16-bit cache of fp16: bf16 caches come through the attention entry point alone)
   if (kv_dtype == 3) { if (hd == 128) RSD_DEC_O(128, __half, true); else RSD_DEC_O(64, __half, true); }
   else if (kv_dtype == 2) { if (hd == 128) RSD_DEC_O(128, __half, false); else RSD_DEC_O(64, __half, false); }
-  else { if (hd == 128) RSD_DEC_O(128, __nv_bfloat16, false); else RSD_DEC_O(64, __nv_bfloat16, false); }
+  else if (hd == 128) { if (out_dtype == 1) RSD_DEC(128, __nv_bfloat16, __nv_bfloat16, false, false); else RSD_DEC(128, __nv_bfloat16, float, false, false); }
+  else { if (out_dtype == 1) RSD_DEC(64, __nv_bfloat16, __nv_bfloat16, false, false); else RSD_DEC(64, __nv_bfloat16, float, false, false); }
 #undef RSD_DEC_O
 #undef RSD_DEC
+#undef RSD_DEC_K
   return launched(splits > 1 && !clustered ? 2 : 1);
 }
 

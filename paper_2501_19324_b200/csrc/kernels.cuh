@@ -124,6 +124,11 @@ cudaError_t launch_attn_chunk_long(const float* q, PassView p, KvView kv, void* 
 cudaError_t launch_swiglu(int dtype, const float* gu, SplitSum pending, void* out, void* out_lo, int T, int F,
                           const int32_t* n_active, cudaStream_t s);
 
+struct QkvSource {
+  const float* qkv;
+  SplitSum pending;      // splits > 1: the product is the sum of these instead
+  const float2* rope;
+};
 // Decode attention (one query per row) with split-KV partial results merged in a second pass.
 size_t attn_decode_scratch_bytes(int B, int H, int hd, int max_ctx);
 // Slot i attends positions [0, len_or_pos[i] + len_offset) of row slot_row[i] (slot i itself when
@@ -134,7 +139,10 @@ cudaError_t launch_attn_decode(int kv_dtype, const float* q, const void* pool_la
                                int max_pages, const int32_t* slot_row, const int32_t* len_or_pos, int len_offset,
                                void* out, void* out_lo, int out_dtype, int B, int H, int KV, int hd, int max_ctx, void* scratch,
                                size_t scratch_bytes, const int32_t* n_active, cudaStream_t s, int active_rows = 0,
-                               int new_tokens = 1);
+                               int new_tokens = 1, const QkvSource* qkv = nullptr);
+// qkv (nullable): the kernel takes the qkv product [B][(H + 2 KV) hd] instead of rotated queries, rotates by the table and
+// writes the new key and value to the cache, as launch_rope_kv would (the pool is written, q is not read).
+bool attn_decode_takes_qkv(int kv_dtype, int out_dtype, int B, int H, int KV, int max_ctx, int active_rows, int new_tokens);
 
 // ---- persistent decode kernel: the whole layer stack of one decode iteration in one launch -------------
 struct MegaShape {

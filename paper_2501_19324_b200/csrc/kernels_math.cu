@@ -165,7 +165,7 @@ cudaError_t launch_rmsnorm(int dtype, float* x, const void* gain, void* out, voi
 // Bound by latency (a launch moves 1-5 MB, all of it in L2): the gain is fetched under the wait, and the partial sums are
 // dealt over kSumGroups groups of 64 threads, so that up to kSumGroups * kSumAhead = 24 splits, the rule, are one
 // round of loads.  The groups' sums meet in shared memory and are added in order.
-constexpr int kSumGroups = 4, kSumAhead = 6;
+constexpr int kSumAhead = 6;
 
 __global__ void __launch_bounds__(64 * kSumGroups)
 reduce_norm_kernel(const float* partials, int splits, float* x, const __nv_bfloat16* __restrict__ gain, __nv_bfloat16* hi,
@@ -374,10 +374,6 @@ __device__ __forceinline__ float split_sum(const float* direct, const float* par
   }
   return v;
 }
-
-// The rotation, its roundings spelled out: every kernel that rotates gives the same bits, whatever the compiler would fuse.
-__device__ __forceinline__ float rotate_lo(float a, float b, float2 cs) { return fmaf(a, cs.x, -__fmul_rn(b, cs.y)); }
-__device__ __forceinline__ float rotate_hi(float a, float b, float2 cs) { return fmaf(b, cs.x, __fmul_rn(a, cs.y)); }
 
 // Bound by latency like reduce_norm: lists, page and angle are fetched under the wait, and with K-split partial sums
 // kSumGroups groups of 64 threads share them out.

@@ -451,3 +451,18 @@ def test_batches_of_more_than_64_rows_and_wide_heads():
     assert stats["tokens_compared"] > 0.5 * stats["tokens"]
     compare_counters(eng, loop)
     eng.close()
+
+
+@pytest.mark.parametrize("d,H,KV,hd,ext", [(128, 1, 1, 64, 0), (512, 7, 1, 128, 0), (2048, 8, 1, 64, 0), (512, 8, 2, 64, 1), (512, 8, 1, 128, 1)])
+def test_decode_attention_that_takes_the_qkv_product(d, H, KV, hd, ext):
+    """Contexts in one split: the attention adds up the product's K splits (1, 4 and 16 of them), rotates and writes the cache
+    itself; head groups of one to eight, both head sizes, a new token on the first and the last place of a page."""
+    sh = ri.ModelShape(2, d, H, KV, hd, 512, 1024)
+    prompts = ri.prompts(31 + H, 5, 13, 18, sh.vocab)
+    kw = dict(max_step_tokens=6, max_steps=2, max_seq_tokens=48, step_end_id=3, step_end_mod=7, temperature=0.7, seed=4)
+    eng, loop = build_pair((sh, sh, sh), bf16=True, prompts=prompts, loop_kwargs=kw, engine_kwargs=dict(kv_extended=ext))
+    stats = {}
+    for _ in range(2):
+        parity_step(eng, loop, 2.0, stats=stats, **TOL16)      # every row is rejected: draft and target decode
+    assert stats["tokens_compared"] > 0.5 * stats["tokens"]
+    eng.close()
