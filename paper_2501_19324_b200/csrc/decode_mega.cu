@@ -699,7 +699,7 @@ __device__ __forceinline__ void gemm_phase(const MegaParams& P, int which, const
             if (c + j < B) {
               const float sc = sh.row_scale[c + j];
               const float a = (v[j] + w[j]) * sc, u = xch[l * 65 + c + j] * sc;
-              store_operand<__nv_bfloat16>(P.act_hi, P.act_lo, (size_t)(c + j) * P.F + f, a / (1.f + expf(-a)) * u);
+              store_operand<__nv_bfloat16>(P.act_hi, P.act_lo, (size_t)(c + j) * P.F + f, swiglu(a, u));
             }
           }
         }

@@ -274,11 +274,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
       if (ok) {
 #pragma unroll 1
         for (int c = 0; c < kHalf; c += 16) {
-          float v[16], w[16];
-          tmem_ld16(taddr + send0 + c, v);
-          tmem_ld16(taddr + kRows + send0 + c, w);
+          float v[2][16];
+          tmem_ld16n<2>({taddr + send0 + c, taddr + kRows + send0 + c}, v);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) send[c + j] = v[j] + w[j];
+          for (int j = 0; j < 16; ++j) send[c + j] = v[0][j] + v[1][j];
         }
       }
       asm volatile("bar.sync 1, 128;" ::: "memory");
@@ -286,22 +285,23 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
 #pragma unroll 1
         for (int c = 0; c < kHalf; c += 16) {
           if (own0 + c >= m_valid) break;
-          float v[16], w[16];
-          tmem_ld16(taddr + own0 + c, v);
-          tmem_ld16(taddr + kRows + own0 + c, w);
+          float v[2][16];
+          tmem_ld16n<2>({taddr + own0 + c, taddr + kRows + own0 + c}, v);
+          // all sixteen, whether the row counts or not, and stores under predicates: a branch per row and a division per
+          // element kept the elements from overlapping (32 rows: 4250 cycles behind the exchange, now 1760)
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const int r = own0 + c + j;
-            if (r < m_valid) {
-              const float sc = rs.ssq != nullptr ? row_scale[r] : 1.f;
-              const float mine = (v[j] + w[j]) * sc, other = recv[c + j] * sc;
-              const float gate = is_gate ? mine : other, up = is_gate ? other : mine;
-              const float a = gate / (1.f + expf(-gate)) * up;
-              const size_t o = (size_t)(m0 + r) * N + n0 + l;
-              const __nv_bfloat16 h = __float2bfloat16_rn(a);
-              act_hi[o] = h;
-              act_lo[o] = __float2bfloat16_rn(a - __bfloat162float(h));
-            }
+            const float sc = rs.ssq != nullptr ? row_scale[own0 + c + j] : 1.f;
+            const float mine = (v[0][j] + v[1][j]) * sc, other = recv[c + j] * sc;
+            v[0][j] = swiglu(is_gate ? mine : other, is_gate ? other : mine);
+          }
+          const size_t o = (size_t)(m0 + own0 + c) * N + n0 + l;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            __nv_bfloat16 h, w;
+            store_operand<__nv_bfloat16>(&h, &w, 0, v[0][j]);
+            store_if(own0 + c + j < m_valid, act_hi + o + (size_t)j * N, h);
+            store_if(own0 + c + j < m_valid, act_lo + o + (size_t)j * N, w);
           }
         }
       }
@@ -309,40 +309,41 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
       // with several K-splits each CTA stores its partial sums as rows of a [split][M][N] array;
       // a reduction kernel adds the splits in order afterwards (deterministic)
       float* dst = splits == 1 ? Y : partials + (size_t)split * M * N;
-      for (int c = 0; c < m_valid; c += 16) {
-        float v[16];
-        tmem_ld16(taddr + c, v);
-        if (SPLIT) {
-          if (kRows == 8) {          // hi in columns 0..7, lo in columns 8..15 of the same load
+      constexpr int kC = kRows >= 32 ? 32 : 16;    // rows at a time
+      for (int c = 0; c < m_valid; c += kC) {
+        float v[kC];
+        if (SPLIT && kRows == 8) {                   // hi in columns 0..7, lo in columns 8..15 of the same load
+          tmem_ld16(taddr, v);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] += v[j + 8];
-          } else {
-            float w[16];
-            tmem_ld16(taddr + kRows + c, w);
+          for (int j = 0; j < 8; ++j) v[j] += v[j + 8];
+        } else {
+          constexpr int G = kC / 16 * (SPLIT ? 2 : 1);
+          float t[G][16];
+          uint32_t at[G];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] += w[j];
-          }
+          for (int g = 0; g < G; ++g) at[g] = taddr + c + (SPLIT ? (g & 1) * kRows + (g >> 1) * 16 : g * 16);
+          tmem_ld16n<G>(at, t);
+#pragma unroll
+          for (int j = 0; j < kC; ++j) v[j] = SPLIT ? t[j / 16 * 2][j % 16] + t[j / 16 * 2 + 1][j % 16] : t[j / 16][j % 16];
         }
         if (rs.ssq != nullptr) {
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (c + j < m_valid) v[j] *= row_scale[c + j];
+          for (int j = 0; j < kC; ++j) v[j] *= row_scale[(c + j) & 127];
         }
         if (n < N) {
-          // when adding into y, all sixteen old values are requested before the first store: written as
-          // "*y += v" row by row, every load would wait for the store before it (the compiler cannot rule out
-          // that two rows alias) and the epilogue would crawl at one memory round trip per element
+          float* to = dst + (size_t)(m0 + c) * N + n;
+          // when adding into y, all old values are requested before the first store: written as "*y += v" row by row,
+          // every load would wait for the store before it (the compiler cannot rule out that two rows alias) and the
+          // epilogue would crawl at one memory round trip per element
           if (accumulate && splits == 1) {
-            float old[16];
+            float old[kC];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) old[j] = c + j < m_valid ? dst[(size_t)(m0 + c + j) * N + n] : 0.f;
+            for (int j = 0; j < kC; ++j) old[j] = c + j < m_valid ? to[(size_t)j * N] : 0.f;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] += old[j];
+            for (int j = 0; j < kC; ++j) v[j] += old[j];
           }
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            if (c + j < m_valid) dst[(size_t)(m0 + c + j) * N + n] = v[j];
-          }
+          for (int j = 0; j < kC; ++j) store_if(c + j < m_valid, to + (size_t)j * N, v[j]);
         }
       }
     }
@@ -392,18 +393,22 @@ __device__ __forceinline__ void persist_epilogue(uint32_t taddr, bool ok, int qu
   using C = PersistCfg<SPLIT, GU>;
   constexpr int kColStep = 16 * (kPersistEpiWarps / 4);
   const int m_valid = min(C::kRows, M - m0);
+  auto ld = [&](int c, float (&v)[16]) {             // sixteen columns, the low halves' results added
+    if (SPLIT) {
+      float t[2][16];
+      tmem_ld16n<2>({taddr + c, taddr + C::kRows + c}, t);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] = t[0][j] + t[1][j];
+    } else {
+      tmem_ld16(taddr + c, v);
+    }
+  };
   if (!GU) {
     const int n = n0 + quarter * 32 + lane;
     if (ok) {
       for (int c = col0; c < m_valid; c += kColStep) {
         float v[16];
-        tmem_ld16(taddr + c, v);
-        if (SPLIT) {
-          float w[16];
-          tmem_ld16(taddr + C::kRows + c, w);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] += w[j];
-        }
+        ld(c, v);
         if (row_scale != nullptr) {
 #pragma unroll
           for (int j = 0; j < 16; ++j) v[j] *= row_scale[(c + j) & 127];
@@ -437,13 +442,7 @@ __device__ __forceinline__ void persist_epilogue(uint32_t taddr, bool ok, int qu
 #pragma unroll 1
       for (int c = col0; c < C::kHalf; c += kColStep) {
         float v[16];
-        tmem_ld16(taddr + send0 + c, v);
-        if (SPLIT) {
-          float w[16];
-          tmem_ld16(taddr + C::kRows + send0 + c, w);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] += w[j];
-        }
+        ld(send0 + c, v);
 #pragma unroll
         for (int j = 0; j < 16; ++j) send[c + j] = v[j];
       }
@@ -454,29 +453,20 @@ __device__ __forceinline__ void persist_epilogue(uint32_t taddr, bool ok, int qu
       for (int c = col0; c < C::kHalf; c += kColStep) {
         if (own0 + c >= m_valid) break;
         float v[16];
-        tmem_ld16(taddr + own0 + c, v);
-        if (SPLIT) {
-          float w[16];
-          tmem_ld16(taddr + C::kRows + own0 + c, w);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] += w[j];
-        }
+        ld(own0 + c, v);
+        // all sixteen, then the stores: see the one-tile kernel's epilogue
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          const int r = own0 + c + j;
-          if (r < m_valid) {
-            const float sc = row_scale != nullptr ? row_scale[r & 127] : 1.f;
-            const float mine = v[j] * sc, other = recv[c + j] * sc;
-            const float gate = is_gate ? mine : other, up = is_gate ? other : mine;
-            const float a = gate / (1.f + expf(-gate)) * up;
-            const size_t o = (size_t)(m0 + r) * N + n0 + l;
-            if (!SPLIT && f16) {
-              reinterpret_cast<__half*>(act_hi)[o] = __float2half_rn(a);
-            } else {
-              const __nv_bfloat16 h = __float2bfloat16_rn(a);
-              act_hi[o] = h;
-              if (SPLIT) act_lo[o] = __float2bfloat16_rn(a - __bfloat162float(h));
-            }
+          const float sc = row_scale != nullptr ? row_scale[(own0 + c + j) & 127] : 1.f;
+          const float mine = v[j] * sc, other = recv[c + j] * sc;
+          v[j] = swiglu(is_gate ? mine : other, is_gate ? other : mine);
+        }
+        const size_t o = (size_t)(m0 + own0 + c) * N + n0 + l;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          if (own0 + c + j < m_valid) {
+            if (!SPLIT && f16) store_operand<__half>(reinterpret_cast<__half*>(act_hi), nullptr, o + (size_t)j * N, v[j]);
+            else store_operand<__nv_bfloat16>(act_hi, SPLIT ? act_lo : nullptr, o + (size_t)j * N, v[j]);
           }
         }
       }

@@ -747,7 +747,7 @@ __global__ void swiglu_kernel(const float* gu, const float* partials, int splits
     const size_t sstride = (size_t)T * 2 * F;
     const float a = split_sum(gu, partials, splits, t * 2 * F + f, sstride);
     const float b = split_sum(gu, partials, splits, t * 2 * F + F + f, sstride);
-    store_operand<OT>(out, out_lo, i, a / (1.f + expf(-a)) * b);
+    store_operand<OT>(out, out_lo, i, swiglu(a, b));
   }
 }
 

@@ -130,6 +130,23 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// Several groups of sixteen columns with one wait: group g from taddr[g].
+template <int G> __device__ __forceinline__ void tmem_ld16n(const uint32_t (&taddr)[G], float (&v)[G][16]) {
+  uint32_t r[G][16];
+#pragma unroll
+  for (int g = 0; g < G; ++g)
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[g][0]), "=r"(r[g][1]), "=r"(r[g][2]), "=r"(r[g][3]), "=r"(r[g][4]), "=r"(r[g][5]), "=r"(r[g][6]), "=r"(r[g][7]),
+          "=r"(r[g][8]), "=r"(r[g][9]), "=r"(r[g][10]), "=r"(r[g][11]), "=r"(r[g][12]), "=r"(r[g][13]), "=r"(r[g][14]), "=r"(r[g][15])
+        : "r"(taddr[g]));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int g = 0; g < G; ++g)
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[g][i] = __uint_as_float(r[g][i]);
+}
+
 // ---- pairs of CTAs (a cluster of two on neighbouring SMs) --------------------------------------
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;

@@ -141,6 +141,17 @@ def test_rmsnorm_rope_swiglu():
     np.testing.assert_allclose(got, a / (1 + np.exp(-a)) * b, rtol=1e-6, atol=1e-6)
 
 
+@pytest.mark.parametrize("lo,hi", [(-1e-30, 1e-30), (-1.0, 1.0), (-30.0, 30.0), (-86.9, -80.0), (-120.0, -87.0), (80.0, 1e4)])
+def test_swiglu_over_its_range(lo, hi):
+    """The exponential is good to 2 ulp, sum, quotient and product to half an ulp each: 3.5 ulp = 3.5 * 2^-23, plus an ulp for the
+    step to the next binade.  Below -87 the exponential is held there: gate * e^-87 at most, 1e-36 or so, times up."""
+    rng = np.random.default_rng(12)
+    gu = np.concatenate([rng.uniform(lo, hi, (64, 512)), rng.normal(size=(64, 512))], axis=1).astype(np.float32)
+    got = rb.k_swiglu(dev(gu), torch.float32).cpu().numpy()
+    a, b = gu[:, :512].astype(np.float64), gu[:, 512:].astype(np.float64)
+    np.testing.assert_allclose(got, a / (1 + np.exp(-a)) * b, rtol=4.5 * 2.0 ** -23, atol=1e-34 if lo < -80 else 2.0 ** -149)
+
+
 @pytest.mark.parametrize("temperature", [0.0, 0.7])
 def test_sampling_matches_oracle(temperature):
     rng = np.random.default_rng(2)
