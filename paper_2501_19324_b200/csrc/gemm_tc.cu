@@ -927,10 +927,13 @@ TcPlan plan_tc(int M, int N, int K, bool split_operand) {
   const int total_kb = (K + kTileK - 1) / kTileK;
   int splits = 1;
   if (tiles < 148 && tiles <= kMaxSplitTiles && N % 4 == 0 && (p.rows <= 64 || (split_operand && M <= 128))) {
-    // aim at one wave of two CTAs per SM (one, where a tile takes the SM alone), each with at least two k-blocks.
+    // aim at one wave, each CTA with at least two k-blocks: of two CTAs per SM where the partial sums are small, of one where
+    // pairs of more than 16 rows make them larger than what a second CTA saves (an iteration of 14 layers, 1.5B / 7B shapes:
+    // 32 rows 726 / 1661 us with two, 710 / 1641 with one; 64 rows 905 / 1942 and 872 / 1900).  Plain rows keep two: the
+    // order of their sums shows in bf16 activations.
     // 65 to 128 rows with pairs are the decode passes of large batches: without the split the 12 tiles of a
     // 1536 x 8960 product leave 136 SMs idle (58 us at 128 rows; 11 us with 12 splits).
-    splits = std::max(1, (p.rows <= 64 ? 2 * 148 : 148) / tiles);
+    splits = std::max(1, (p.rows <= 16 || !split_operand ? 2 * 148 : 148) / tiles);
     splits = std::min(splits, std::max(1, total_kb / 2));
     splits = std::min(splits, kMaxSplitCtas / tiles);
     splits = std::max(splits, 1);
