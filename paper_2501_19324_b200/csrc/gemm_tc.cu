@@ -1123,11 +1123,14 @@ static bool pair_pays(int M, int n_features, int K, int feat, int rows, bool add
 // Rows of x per tile for a dense product with one operand (bf16 or fp16): 256, or 128 or 64 while the tiles of the larger
 // size leave half of the SMs (of 256) or some (of 128) without one.  Every size sums along K in the same order: the
 // results are the same bits.  us at 256 / at the size taken, adding into y: 455 x 2048 x 1536 27.6 / 20.5 (64), 1000 x 1536 x 1536
-// 28.7 / 22.5 (64); 1000 x 3584 x 3584, 112 tiles of 256: 42 / 43.6 (128), kept at 256.
-static int dense_rows(int M, int N) {
+// 28.7 / 22.5 (64); 1000 x 3584 x 3584, 112 tiles of 256: 42 / 43.6 (128), kept at 256.  Adding at a short K the epilogue is
+// most of a tile and one wave of 256-row tiles hides none of it, while two CTAs of 128 rows hide each other's: 2048 x 1536 x 1536,
+// 96 tiles, 28.7 / 24.6; 3000 x 1536 x 1536, 144 tiles, 30.7 / 26.6; from two waves on the persistent kernel does as well or
+// better (4096 x 1536 x 1536 43 / 43, 8192 x 1536 x 1536 57 / 64).
+static int dense_rows(int M, int N, int K, bool adds) {
   const int n_tiles = (N + kTileN - 1) / kTileN;
   int rows = 256;
-  while (rows > 64 && n_tiles * ((M + rows - 1) / rows) < (rows == 256 ? 74 : 148)) rows /= 2;
+  while (rows > 64 && n_tiles * ((M + rows - 1) / rows) < (rows == 256 && !(adds && K < 3072) ? 74 : 148)) rows /= 2;
   return rows;
 }
 
@@ -1243,7 +1246,7 @@ cudaError_t launch_gemm_tc(const void* W, const void* x, const void* x_lo, float
   CUtensorMap tw, tx, txl;
   const bool dense = M > 128 && p.splits == 1 && rs.ssq == nullptr && n_active == nullptr;
   const bool pair = dense && pair_pays(M, N, K, 2 * kTileN, p.rows, accumulate != 0);
-  const int rows = dense && !split_operand && !pair && !no_k_split ? dense_rows(M, N) : p.rows;
+  const int rows = dense && !split_operand && !pair && !no_k_split ? dense_rows(M, N, K, accumulate != 0) : p.rows;
   if (!get_map(W, N, K, kTileN, &tw) || !get_map(x, M, K, pair ? 128 : rows, &tx)) return cudaErrorNotSupported;
   if (split_operand) { if (!get_map(x_lo, M, K, p.rows, &txl)) return cudaErrorNotSupported; }
   else txl = tx;
@@ -1298,7 +1301,7 @@ cudaError_t launch_gemm_f16_dense(const void* W16, const void* x16, float* y, in
   if (((uintptr_t)W16 & 15) || ((uintptr_t)x16 & 15)) return cudaErrorMisalignedAddress;
   const bool pair = pair_pays(M, N, K, 2 * kTileN, 256, accumulate != 0);
   CUtensorMap tw, tx;
-  const int rows = pair ? 128 : dense_rows(M, N);
+  const int rows = pair ? 128 : dense_rows(M, N, K, accumulate != 0);
   if (!get_map(W16, N, K, kTileN, &tw) || !get_map(x16, M, K, rows, &tx)) return cudaErrorNotSupported;
   int* err = (int*)((char*)scratch + kCounterBytes);
   if (!pair && rows < 256) return launch_dense_small(tw, tx, y, M, N, K, accumulate, rows, err, s, 1);

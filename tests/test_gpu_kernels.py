@@ -528,6 +528,18 @@ def test_dense_gemm_on_fp16_operands(M, N, K):
         rb.k_gemm(Wd, xd[:128].contiguous(), impl=4)    # the form is for more than 128 rows
 
 
+@pytest.mark.parametrize("M", [1665, 2047, 3072, 3073])
+def test_dense_gemm_that_adds_over_a_short_k(M):
+    """Twelve weight tiles: up to 3072 rows make fewer 256-row tiles than SMs and are taken 128 rows at a time, one row more is not;
+    fp32 sums of K products of order 0.05."""
+    N, K = 1536, 136
+    rng = np.random.default_rng(M)
+    W = (rng.normal(size=(N, K)) * 0.05).astype(np.float16)
+    x, y0 = rng.normal(size=(M, K)).astype(np.float16), rng.normal(size=(M, N)).astype(np.float32)
+    got = rb.k_gemm(dev(W), dev(x), y=dev(y0.copy()), accumulate=True, impl=4).cpu().numpy()
+    np.testing.assert_allclose(got, x.astype(np.float64) @ W.astype(np.float64).T + y0, rtol=0, atol=2e-5 * np.sqrt(K) + 2e-6)
+
+
 @pytest.mark.parametrize("M,F,K", [(1, 64, 64), (5, 192, 512), (32, 1408, 512), (33, 128, 520), (70, 2048, 768),
                                    (129, 704, 1408), (300, 320, 256), (32, 8960, 1536), (200, 128, 520), (2100, 640, 128),
                                    (65, 9536, 192), (128, 9472, 520)])
