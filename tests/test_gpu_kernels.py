@@ -141,15 +141,30 @@ def test_rmsnorm_rope_swiglu():
     np.testing.assert_allclose(got, a / (1 + np.exp(-a)) * b, rtol=1e-6, atol=1e-6)
 
 
-@pytest.mark.parametrize("lo,hi", [(-1e-30, 1e-30), (-1.0, 1.0), (-30.0, 30.0), (-86.9, -80.0), (-120.0, -87.0), (80.0, 1e4)])
+@pytest.mark.parametrize("lo,hi", [(-1e-30, 1e-30), (-1.0, 1.0), (-30.0, 30.0), (-86.9, -80.0), (-88.7, -87.0), (-120.0, -87.0), (80.0, 1e4)])
 def test_swiglu_over_its_range(lo, hi):
     """The exponential is good to 2 ulp, sum, quotient and product to half an ulp each: 3.5 ulp = 3.5 * 2^-23, plus an ulp for the
-    step to the next binade.  Below -87 the exponential is held there: gate * e^-87 at most, 1e-36 or so, times up."""
+    step to the next binade.  Below -88.72 the exponential overflows and the result is zero: 2.7e-37 at most is lost, times up
+    (|up| < 5 here)."""
     rng = np.random.default_rng(12)
     gu = np.concatenate([rng.uniform(lo, hi, (64, 512)), rng.normal(size=(64, 512))], axis=1).astype(np.float32)
     got = rb.k_swiglu(dev(gu), torch.float32).cpu().numpy()
     a, b = gu[:, :512].astype(np.float64), gu[:, 512:].astype(np.float64)
-    np.testing.assert_allclose(got, a / (1 + np.exp(-a)) * b, rtol=4.5 * 2.0 ** -23, atol=1e-34 if lo < -80 else 2.0 ** -149)
+    np.testing.assert_allclose(got, a / (1 + np.exp(-a)) * b, rtol=4.5 * 2.0 ** -23, atol=5 * 2.7e-37 if lo < -88.72 else 2.0 ** -148)
+
+
+def test_swiglu_is_the_division():
+    """Every 61st float as the gate (all binades, both signs, infinities and NaNs among them) against gate / (1 + exp(-gate)) with
+    CUDA's own division: the same value; where gate or result is subnormal, within a subnormal step."""
+    gate = (torch.arange(0, 1 << 32, 61, device="cuda") - (1 << 31)).to(torch.int32).view(torch.float32)
+    ends = torch.tensor([np.inf, -np.inf, np.nan, 3.4028235e38, -3.4028235e38, -1e30, -1e10, -104.0, -90.0, -88.8, -88.7, -87.1], device="cuda")
+    gate = torch.cat([gate, ends])
+    got = rb.k_swiglu(torch.cat([gate, torch.ones_like(gate)]).view(1, -1), torch.float32)[0]
+    want = gate / (1 + torch.exp(-gate))
+    assert torch.equal(torch.isnan(got), torch.isnan(want))
+    tiny = (want.abs() < 2.0 ** -126) | (gate.abs() < 2.0 ** -124)
+    same = (got == want) | torch.isnan(want) | (tiny & ((got.double() - want.double()).abs() <= 2.0 ** -148))
+    assert bool(same.all()), (gate[~same][:8], got[~same][:8], want[~same][:8])
 
 
 @pytest.mark.parametrize("temperature", [0.0, 0.7])
