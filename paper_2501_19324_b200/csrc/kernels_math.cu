@@ -786,11 +786,12 @@ __device__ __forceinline__ float unpack_score(unsigned long long packed) {
 // Grid (slots, chunks): every warp takes `steps` runs of 128 ids of a slot and folds its best candidate into best[slot] with
 // an atomic maximum (order-independent, hence deterministic).
 // Exact noise for every id -- ten Philox rounds per four ids and two logarithms per id -- kept the ALUs busy for 66 us at
-// 151936 ids x 128 rows, four times what the logits' 78 MB take.  So a warp first publishes the exact score of its largest
-// logit; then a score is first taken with fast logarithms, and only ids within kScoreMargin of the best so far (this warp's,
-// or what others have published) get exact ones; and as the noise lies below 16.64, ids whose logits stay kNoiseMax below
-// that best draw none at all.  The winner is the same.
-constexpr int kSampleThreads = 256;
+// 151936 ids x 128 rows, four times what the logits' 78 MB take.  So with many ids in all (launch_sample draws the line) a warp
+// first publishes the exact score of its largest logit; then a score is first taken with fast logarithms, and only ids within
+// kScoreMargin of the best so far (this warp's, or what others have published) get exact ones; and as the noise lies below
+// 16.64, ids whose logits stay kNoiseMax below that best draw none at all.  The winner is the same.
+// DIRECT: few ids in all, exact noise for each of them.
+constexpr int kSampleThreads = 256, kSampleBlocks = 4;   // ... and blocks per SM
 constexpr int kSampleSteps = 8;             // runs of 128 ids that a warp holds in registers at most
 constexpr float kScoreMargin = 1e-3f;       // the fast score errs by less than 1e-4 (see fast_gumbel)
 constexpr float kNoiseMax = 17.f;
@@ -809,7 +810,8 @@ __device__ __forceinline__ float score_needed(float run) {
   return run == INFINITY ? run : run - (kScoreMargin + fabsf(run) * 1e-6f);
 }
 
-__global__ void __launch_bounds__(kSampleThreads) sample_kernel(SampleArgs a, int steps) {
+template <bool DIRECT>
+__global__ void __launch_bounds__(kSampleThreads, kSampleBlocks) sample_kernel(SampleArgs a, int steps) {
   RSD_PDL_TRIGGER();
   if (a.n_active == nullptr) RSD_PDL_WAIT();   // a decode pass's lists may be read ahead of the wait, others not
   const bool idle = a.n_active != nullptr && ld_cg(a.n_active) == 0;
@@ -848,53 +850,64 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(SampleArgs a, in
   auto exact = [&](float logit, uint32_t bits) { return fmaf(logit, inv_t, -logf(-logf(uniform_from_bits(bits)))); };
   float bs = -INFINITY;
   int bi = 0x7FFFFFFF;
-  // this lane's largest logit, then the warp's
-  float tx = -INFINITY;
-  int ti = 0x7FFFFFFF;
-#pragma unroll
-  for (int k = 0; k < kSampleSteps; ++k)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) better(tx, ti, x[k][j], (v4_0 + k * 32) * 4 + j);
-  if (!noisy) {
-    bs = tx; bi = ti;
-  } else {
-    float wx = tx;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) wx = fmaxf(wx, __shfl_xor_sync(0xFFFFFFFFu, wx, o));
-    float run = -INFINITY;
-    if (tx == wx && ti != 0x7FFFFFFF) {                // one lane, or a few that tie
-      uint32_t w[4];
-      noise_bits(ti >> 2, w);
-      const int j = ti & 3;
-      bs = exact(tx, j == 0 ? w[0] : j == 1 ? w[1] : j == 2 ? w[2] : w[3]);
-      bi = ti;
-      const unsigned long long mine = pack_best(bs, bi), seen = atomicMax(a.best + slot, mine);
-      run = unpack_score(seen > mine ? seen : mine);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) run = fmaxf(run, __shfl_xor_sync(0xFFFFFFFFu, run, o));
+  if (DIRECT && noisy) {
 #pragma unroll
     for (int k = 0; k < kSampleSteps; ++k) {
       if (k >= steps) break;
-      const int v4 = v4_0 + k * 32;
-      const float top = fmaxf(fmaxf(x[k][0], x[k][1]), fmaxf(x[k][2], x[k][3])) * inv_t;
-      if (!__any_sync(0xFFFFFFFFu, top >= run - kNoiseMax || run == -INFINITY)) continue;
       uint32_t w[4];
-      noise_bits(v4, w);
-      float sc[4], wm = -INFINITY;
+      noise_bits(v4_0 + k * 32, w);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        sc[j] = fmaf(x[k][j], inv_t, fast_gumbel(uniform_from_bits(w[j])));
-        wm = fmaxf(wm, sc[j]);
+      for (int j = 0; j < 4; ++j) better(bs, bi, exact(x[k][j], w[j]), (v4_0 + k * 32) * 4 + j);
+    }
+  } else {
+    // this lane's largest logit, then the warp's
+    float tx = -INFINITY;
+    int ti = 0x7FFFFFFF;
+#pragma unroll
+    for (int k = 0; k < kSampleSteps; ++k)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) better(tx, ti, x[k][j], (v4_0 + k * 32) * 4 + j);
+    if (!noisy) {
+      bs = tx; bi = ti;
+    } else {
+      float wx = tx;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) wx = fmaxf(wx, __shfl_xor_sync(0xFFFFFFFFu, wx, o));
+      float run = -INFINITY;
+      if (tx == wx && ti != 0x7FFFFFFF) {                // one lane, or a few that tie
+        uint32_t w[4];
+        noise_bits(ti >> 2, w);
+        const int j = ti & 3;
+        bs = exact(tx, j == 0 ? w[0] : j == 1 ? w[1] : j == 2 ? w[2] : w[3]);
+        bi = ti;
+        const unsigned long long mine = pack_best(bs, bi), seen = atomicMax(a.best + slot, mine);
+        run = unpack_score(seen > mine ? seen : mine);
       }
-      const float need = score_needed(run);
-      if (!__any_sync(0xFFFFFFFFu, wm >= need)) continue;
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (sc[j] >= need) better(bs, bi, exact(x[k][j], w[j]), v4 * 4 + j);
+      for (int o = 16; o > 0; o >>= 1) run = fmaxf(run, __shfl_xor_sync(0xFFFFFFFFu, run, o));
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xFFFFFFFFu, wm, o));
-      run = fmaxf(run, wm);
+      for (int k = 0; k < kSampleSteps; ++k) {
+        if (k >= steps) break;
+        const int v4 = v4_0 + k * 32;
+        const float top = fmaxf(fmaxf(x[k][0], x[k][1]), fmaxf(x[k][2], x[k][3])) * inv_t;
+        if (!__any_sync(0xFFFFFFFFu, top >= run - kNoiseMax || run == -INFINITY)) continue;
+        uint32_t w[4];
+        noise_bits(v4, w);
+        float sc[4], wm = -INFINITY;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          sc[j] = fmaf(x[k][j], inv_t, fast_gumbel(uniform_from_bits(w[j])));
+          wm = fmaxf(wm, sc[j]);
+        }
+        const float need = score_needed(run);
+        if (!__any_sync(0xFFFFFFFFu, wm >= need)) continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (sc[j] >= need) better(bs, bi, exact(x[k][j], w[j]), v4 * 4 + j);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xFFFFFFFFu, wm, o));
+        run = fmaxf(run, wm);
+      }
     }
   }
 #pragma unroll
@@ -902,6 +915,18 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(SampleArgs a, in
     const float os = __shfl_xor_sync(0xFFFFFFFFu, bs, o);
     const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
     better(bs, bi, os, oi);
+  }
+  if (DIRECT && (noisy || gridDim.y > 1)) {
+    // one atomic per block: with few slots the warps' own would queue up at a few addresses
+    __shared__ unsigned long long s_best[kSampleThreads / 32];
+    if (lane == 0) s_best[threadIdx.x >> 5] = bi != 0x7FFFFFFF ? pack_best(bs, bi) : 0ull;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    unsigned long long top = s_best[0];
+#pragma unroll
+    for (int w = 1; w < kSampleThreads / 32; ++w) top = s_best[w] > top ? s_best[w] : top;
+    if (top != 0ull) atomicMax(a.best + slot, top);
+    return;
   }
   if (lane == 0 && bi != 0x7FFFFFFF) atomicMax(a.best + slot, pack_best(bs, bi));
 }
@@ -919,10 +944,16 @@ __global__ void sample_finalize_kernel(unsigned long long* best, const int32_t* 
 // kernel unpacks them into a.token and clears a.best.
 cudaError_t launch_sample(const SampleArgs& a, cudaStream_t s) {
   if (a.n_slots <= 0) return cudaSuccess;
-  // runs of 128 ids per warp: as many as leave every SM its 24 warps or so, so that small batches stay wide
+  // Runs of 128 ids per warp: the fewest that leave one wave of kSampleBlocks blocks per SM (8 x 151936 ids, greedy, the call's
+  // other two nodes included: 600 blocks 10.4 us, 400 blocks 8.3).  Up to 1.5 million ids exact noise for all of them takes less
+  // than the shortcuts' two dependent rounds: shortcuts / all, 8 x 151936 ids 15.2 / 11.3 us, 3 x 151936 12.5 / 9.4, 8 x 1024
+  // 8.3 / 6.3; beyond it more, 32 x 151936 peaked logits 18.7 / 24.7.
   const int runs = (a.v_limit + 127) / 128, warps = kSampleThreads / 32;
-  const int steps = std::max(1, std::min(kSampleSteps, (int)((long)a.n_slots * runs / (148 * 24))));
-  RSD_LAUNCH((sample_kernel), dim3(a.n_slots, (runs + warps * steps - 1) / (warps * steps)), kSampleThreads, 0, s, a, steps);
+  int steps = 1;
+  while (steps < kSampleSteps && (long)a.n_slots * ((runs + warps * steps - 1) / (warps * steps)) > 148L * kSampleBlocks) ++steps;
+  const dim3 grid(a.n_slots, (runs + warps * steps - 1) / (warps * steps));
+  if ((long)a.n_slots * a.v_limit <= 1500000) RSD_LAUNCH((sample_kernel<true>), grid, kSampleThreads, 0, s, a, steps);
+  else RSD_LAUNCH((sample_kernel<false>), grid, kSampleThreads, 0, s, a, steps);
   if (a.token == nullptr) return launched(1);
   RSD_LAUNCH((sample_finalize_kernel), (a.n_slots + 255) / 256, 256, 0, s, a.best, a.slot_row, a.token, a.n_slots);
   return launched(2);

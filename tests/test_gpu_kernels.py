@@ -213,6 +213,26 @@ def test_sampling_shortcuts_keep_the_winner(v_limit, scale, shift):
                 assert got[b] == want, (b, temperature, got[b], want, margin)
 
 
+@pytest.mark.parametrize("v_limit,scale,shift", [(127, 1.0, 0.0), (1024, 8.0, 0.0), (4097, 4.0, 0.0), (16385, 30.0, 0.0), (65537, 8.0, -50.0), (151936, 1.0, 2000.0)])
+def test_sampling_forms_agree(v_limit, scale, shift):
+    """Few ids in all take exact noise at once, more than 1.5 million the shortcuts: a handful of rows alone and the same rows
+    repeated until the call is beyond that line must give the same ids (both forms compare the same exact scores)."""
+    rng = np.random.default_rng(v_limit + 1)
+    B, V = 5, v_limit + 2
+    logits = (rng.normal(size=(B, V)) * scale + shift).astype(np.float32)
+    logits[1, rng.integers(0, v_limit, size=3)] += 25.0
+    logits[2] = shift
+    logits[3, :v_limit // 2] = -np.inf
+    logits[4, rng.integers(0, v_limit, size=5)] = np.nan
+    row, pos = np.arange(B, dtype=np.int32), np.arange(B, dtype=np.int32) * 41 + 3
+    reps = 1500000 // (B * v_limit) + 1
+    for temperature in (0.7, 0.0):
+        few = rb.k_sample(dev(logits), v_limit, temperature, 91, 0, dev(row), dev(pos))
+        many = rb.k_sample(dev(logits).repeat(reps, 1), v_limit, temperature, 91, 0, dev(row).repeat(reps), dev(pos).repeat(reps))
+        assert B * v_limit <= 1500000 < reps * B * v_limit
+        assert torch.equal(many.view(reps, B), few.expand(reps, B)), temperature
+
+
 def test_gate_compaction_all_masks_and_large():
     """Brute force (a serial loop over the rows) against the ballot / prefix path: EVERY accept mask of 12 rows, one
     call per mask as the step loop calls it, and every mask of 16 rows laid end to end in one call of 2^20 rows."""
