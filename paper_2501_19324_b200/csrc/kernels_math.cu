@@ -250,7 +250,7 @@ cudaError_t launch_reduce_norm(const float* partials, int splits, float* x, cons
 // ---------------------------------------------------------------------------------------------
 constexpr int kGemvAhead = 4;
 
-template <typename WT, int MT>
+template <typename WT, int MT, int AHEAD>
 __global__ void __launch_bounds__(256)
 gemv_splitk_kernel(const WT* __restrict__ W, const WT* X, const WT* X_lo, float* Y, int M, int N, int K, int ks, int accumulate,
                    const int32_t* n_active) {
@@ -264,11 +264,11 @@ gemv_splitk_kernel(const WT* __restrict__ W, const WT* X, const WT* X_lo, float*
   const int m0 = blockIdx.y * MT;
   const int nvec = n < N ? K / VN : 0, v0 = split * 32 + lane, step = ks * 32;
   const WT* wrow = W + (size_t)n * K;
-  Vec16<WT> ahead[kGemvAhead];
+  Vec16<WT> ahead[AHEAD > 0 ? AHEAD : 1];
   if (n_active == nullptr) RSD_PDL_WAIT();   // outside a decode pass W may be an earlier kernel's output
   const bool idle = n_active != nullptr && ld_cg(n_active) == 0;
 #pragma unroll
-  for (int i = 0; i < kGemvAhead; ++i)
+  for (int i = 0; i < AHEAD; ++i)
     if (v0 + i * step < nvec) ahead[i].load_stream(wrow + (size_t)(v0 + i * step) * VN);
   RSD_PDL_WAIT();
   if (idle) return;
@@ -298,9 +298,9 @@ gemv_splitk_kernel(const WT* __restrict__ W, const WT* X, const WT* X_lo, float*
     }
   };
 #pragma unroll
-  for (int i = 0; i < kGemvAhead; ++i)
+  for (int i = 0; i < AHEAD; ++i)
     if (v0 + i * step < nvec) fold(ahead[i], v0 + i * step);
-  for (int v = v0 + kGemvAhead * step; v < nvec; v += step) {
+  for (int v = v0 + AHEAD * step; v < nvec; v += step) {
     Vec16<WT> w;
     w.load_stream(wrow + (size_t)v * VN);
     fold(w, v);
@@ -322,15 +322,20 @@ gemv_splitk_kernel(const WT* __restrict__ W, const WT* X, const WT* X_lo, float*
 cudaError_t launch_gemm_simt(int dtype, const void* W, const void* x, const void* x_lo, float* y, int M, int N, int K,
                              int accumulate, const int32_t* n_active, cudaStream_t s) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  // pick the split so that the grid covers the 148 SMs a few times over, as long as every lane has a vector
+  // Pick the split so that the grid covers the 148 SMs a few times over, as long as every lane has a vector (fp32, up to four
+  // rows) or two.  More rows are more blocks, each with its reductions: splitting them as finely, and holding weights ahead in
+  // registers where no wait is to be bridged, cost 256 x 512 x 1376 146 us instead of 84 and 60 x 512 x 256 12 instead of 5.6.
   int ks = 1;
-  const int per_warp = 32 * (dtype == 1 ? Vec16<__nv_bfloat16>::N : Vec16<float>::N);
+  const int per_warp = M <= 4 && dtype != 1 ? 128 : 256;
   while (ks < 8 && (long)N * ks / 8 < 148L * 4 && K / (ks * 2) >= per_warp) ks *= 2;
   const int mt = M <= 4 ? 4 : 8;
+  const bool ahead = M <= 4 || n_active != nullptr;
   dim3 grid((N + (8 / ks) - 1) / (8 / ks), (M + mt - 1) / mt);
-#define RSD_GEMV(WT, MT) RSD_LAUNCH((gemv_splitk_kernel<WT, MT>), grid, 256, 0, s, (const WT*)W, (const WT*)x, (const WT*)x_lo, y, M, N, K, ks, accumulate, n_active)
-  if (dtype == 1) { if (mt == 4) RSD_GEMV(__nv_bfloat16, 4); else RSD_GEMV(__nv_bfloat16, 8); }
-  else { x_lo = nullptr; if (mt == 4) RSD_GEMV(float, 4); else RSD_GEMV(float, 8); }
+#define RSD_GEMV(WT, MT, AHEAD) RSD_LAUNCH((gemv_splitk_kernel<WT, MT, AHEAD>), grid, 256, 0, s, (const WT*)W, (const WT*)x, (const WT*)x_lo, y, M, N, K, ks, accumulate, n_active)
+#define RSD_GEMV_M(WT) do { if (mt == 4) RSD_GEMV(WT, 4, kGemvAhead); else if (ahead) RSD_GEMV(WT, 8, kGemvAhead); else RSD_GEMV(WT, 8, 0); } while (0)
+  if (dtype == 1) RSD_GEMV_M(__nv_bfloat16);
+  else { x_lo = nullptr; RSD_GEMV_M(float); }
+#undef RSD_GEMV_M
 #undef RSD_GEMV
   return launched(1);
 }

@@ -68,7 +68,8 @@ def test_philox_matches_oracle_on_many_counters():
 
 
 @pytest.mark.parametrize("bf16", [False, True])
-@pytest.mark.parametrize("M,N,K", [(1, 1024, 256), (4, 688 * 2, 256), (7, 256, 688), (33, 1000, 512), (130, 257, 1024)])
+@pytest.mark.parametrize("M,N,K", [(1, 1024, 256), (4, 688 * 2, 256), (7, 256, 688), (33, 1000, 512), (130, 257, 1024),
+                                   (4, 40, 64), (5, 40, 64), (5, 512, 1376), (9, 2752, 512)])
 def test_gemm_simt(M, N, K, bf16):
     rng = np.random.default_rng(M * 1000 + N)
     W = ri.cpu_tensor(1, 77, N, K, bf16)
