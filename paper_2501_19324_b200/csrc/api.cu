@@ -470,14 +470,14 @@ int forward_pass_f16(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
   const int T = p.T;
   for (int l = 0; l < m.n_layers; ++l) {
     KvView kv{M.kv_pool + (size_t)l * M.layer_stride, c->st.page_table[which], c->max_pages, 0};
-    CU(launch_rmsnorm(m.dtype, c->x, M.norm1[l], c->h, nullptr, T, d, m.rms_eps, nullptr, nullptr, SplitSum(), s, true));
+    CU(launch_rmsnorm(m.dtype, c->x, M.norm1[l], c->h, nullptr, T, d, m.rms_eps, nullptr, s, true));
     int rc = gemm_f16(c, M.w16_of(l, 0), c->h, c->qkv, T, (H + 2 * KV) * hd, d, 0, s);
     if (rc) return rc;
     CU(launch_rope_kv(M.kv_dtype, c->qkv, SplitSum(), p, c->q, kv, M.rope, H, KV, hd, s));
     CU(launch_attn_chunk(M.kv_dtype, c->q, p, kv, c->attn, nullptr, 2, H, KV, hd, s, (int*)((char*)c->gemm_scratch + 4096)));
     rc = gemm_f16(c, M.w16_of(l, 1), c->attn, c->x, T, d, H * hd, 1, s);
     if (rc) return rc;
-    CU(launch_rmsnorm(m.dtype, c->x, M.norm2[l], c->h, nullptr, T, d, m.rms_eps, nullptr, nullptr, SplitSum(), s, true));
+    CU(launch_rmsnorm(m.dtype, c->x, M.norm2[l], c->h, nullptr, T, d, m.rms_eps, nullptr, s, true));
     {
       const bool pick = c->time_stride > 0 && (c->gemm_calls++ % (uint64_t)c->time_stride) == 0;
       const bool timed = pick && c->ev_used < c->ev_bytes.size();
@@ -509,18 +509,14 @@ int forward_pass(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
   void* h_lo = M.split ? c->h_lo : nullptr;
   void* attn_lo = M.split ? c->attn_lo : nullptr;
   void* act_lo = M.split ? c->act_lo : nullptr;
-  // K-split partial sums can be left for the consumer kernel to add up.  That pays where the
-  // consumer runs many blocks (SwiGLU); RMSNorm and RoPE run one block per token, too few to pull
-  // the partials in quickly, so those GEMMs reduce with their own kernel.
-  const bool defer_small = false;
-  SplitSum x_pending;   // partial sums of the last GEMM that adds into the residual stream
+  // K-split partial sums are left for the consumer kernel to add up where it runs many blocks (SwiGLU); RMSNorm and RoPE
+  // run one block per token, too few to pull the partials in quickly, so those GEMMs reduce with their own kernel.
   for (int l = 0; l < m.n_layers; ++l) {
     KvView kv{M.kv_pool + (size_t)l * M.layer_stride, c->st.page_table[which], c->max_pages, M.kv_dtype == 3 ? 1 : 0};
-    CU(launch_rmsnorm(m.dtype, c->x, M.norm1[l], c->h, h_lo, T, d, m.rms_eps, nullptr, p.n_active, x_pending, s));
-    SplitSum qkv_pending;
-    int rc = gemm(c, M, M.wqkv[l], c->h, h_lo, c->qkv, T, (H + 2 * KV) * hd, d, 0, p.n_active, defer_small ? &qkv_pending : nullptr, s);
+    CU(launch_rmsnorm(m.dtype, c->x, M.norm1[l], c->h, h_lo, T, d, m.rms_eps, p.n_active, s));
+    int rc = gemm(c, M, M.wqkv[l], c->h, h_lo, c->qkv, T, (H + 2 * KV) * hd, d, 0, p.n_active, nullptr, s);
     if (rc) return rc;
-    CU(launch_rope_kv(M.kv_dtype, c->qkv, qkv_pending, p, c->q, kv, M.rope, H, KV, hd, s));
+    CU(launch_rope_kv(M.kv_dtype, c->qkv, SplitSum(), p, c->q, kv, M.rope, H, KV, hd, s));
     if (p.n_active != nullptr) {
       // decode pass: one query per row slot
       CU(launch_attn_decode(M.kv_dtype, c->q, kv.pool_layer, kv.page_table, kv.max_pages, p.tok_row, p.tok_pos, 1,
@@ -530,9 +526,9 @@ int forward_pass(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
       CU(launch_attn_chunk(M.kv_dtype, c->q, p, kv, c->attn, attn_lo, m.dtype, H, KV, hd, s,
                            (int*)((char*)c->gemm_scratch + 4096)));
     }
-    rc = gemm(c, M, M.wo[l], c->attn, attn_lo, c->x, T, d, H * hd, 1, p.n_active, defer_small ? &x_pending : nullptr, s);
+    rc = gemm(c, M, M.wo[l], c->attn, attn_lo, c->x, T, d, H * hd, 1, p.n_active, nullptr, s);
     if (rc) return rc;
-    CU(launch_rmsnorm(m.dtype, c->x, M.norm2[l], c->h, h_lo, T, d, m.rms_eps, nullptr, p.n_active, x_pending, s));
+    CU(launch_rmsnorm(m.dtype, c->x, M.norm2[l], c->h, h_lo, T, d, m.rms_eps, p.n_active, s));
     // up to 128 rows: fused kernel; dense passes (no idle flag): the persistent kernel hides the SwiGLU epilogue
     // under the next tile's MMAs
     if (gu_fused_ok(M, T) || (T > 128 && p.n_active == nullptr && m.dtype == RSD_BF16 && gemm_gu_supported(1, T, F, d))) {
@@ -544,10 +540,7 @@ int forward_pass(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
       if (rc) return rc;
       CU(launch_swiglu(m.dtype, c->gu, gu_pending, c->act, act_lo, T, F, p.n_active, s));
     }
-    // the last layer's result must be complete in x when the pass ends
-    const bool last = l + 1 == m.n_layers;
-    x_pending = SplitSum();
-    rc = gemm(c, M, M.wdown[l], c->act, act_lo, c->x, T, d, F, 1, p.n_active, (last || !defer_small) ? nullptr : &x_pending, s);
+    rc = gemm(c, M, M.wdown[l], c->act, act_lo, c->x, T, d, F, 1, p.n_active, nullptr, s);
     if (rc) return rc;
   }
   return RSD_OK;
@@ -709,7 +702,7 @@ int model_logits(rsd_ctx* c, int which, PassView p, bool allow_mega, cudaStream_
   } else {
     if ((rc = forward_pass(c, which, p, s))) return rc;
     CU(launch_rmsnorm(m.dtype, c->x, m.final_norm, c->h, M.split ? c->h_lo : nullptr, T, m.d_model, m.rms_eps,
-                      nullptr, p.n_active, SplitSum(), s));
+                      p.n_active, s));
     rc = gemm(c, M, m.head, c->h, c->h_lo, c->logits, T, m.vocab, m.d_model, 0, p.n_active, nullptr, s);
   }
   return rc;
@@ -1541,7 +1534,7 @@ int rsd_k_gate_compact(const float* rewards, const uint8_t* live, float delta, u
 int rsd_k_rmsnorm(const float* x, const void* gain, void* out, int32_t T, int32_t d, float eps, int32_t dtype,
                   void* cuda_stream) {
   if (!x || !gain || !out || T < 0 || d < 4 || d % 4) return RSD_ERR_ARG;
-  KCU(launch_rmsnorm(dtype, const_cast<float*>(x), gain, out, nullptr, T, d, eps, nullptr, nullptr, SplitSum(), (cudaStream_t)cuda_stream));
+  KCU(launch_rmsnorm(dtype, x, gain, out, nullptr, T, d, eps, nullptr, (cudaStream_t)cuda_stream));
   return RSD_OK;
 }
 

@@ -55,11 +55,9 @@ struct KvView {
 
 cudaError_t launch_bf16_to_f16(const void* src, void* dst, size_t n, cudaStream_t s);
 cudaError_t launch_embed(int dtype, const void* embed, PassView p, float* x, int d, cudaStream_t s);
-// out[t] = rmsnorm(x[src ? src[t] : t]); rows with src[t] < 0 are skipped.
-// out (and out_lo when given, bf16 only: the low half of a split-precision operand)
-// pending (splits > 1): x[t] += sum of the partial sums [splits][T][d] first (x is written back).
-cudaError_t launch_rmsnorm(int dtype, float* x, const void* gain, void* out, void* out_lo, int T, int d, float eps,
-                           const int32_t* src, const int32_t* n_active, SplitSum pending, cudaStream_t s, bool out_f16 = false);
+// out[t] = rmsnorm(x[t]) (and out_lo when given, bf16 only: the low half of a split-precision operand)
+cudaError_t launch_rmsnorm(int dtype, const float* x, const void* gain, void* out, void* out_lo, int T, int d, float eps,
+                           const int32_t* n_active, cudaStream_t s, bool out_f16 = false);
 // x_lo (nullable, bf16 only): second operand matrix added to x (split-precision activations).
 cudaError_t launch_gemm_simt(int dtype, const void* W, const void* x, const void* x_lo, float* y, int M, int N, int K,
                              int accumulate, const int32_t* n_active, cudaStream_t s);

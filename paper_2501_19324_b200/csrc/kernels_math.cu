@@ -45,27 +45,6 @@ constexpr int kNormVecs = 4;
 // The roundings spelled out: the sum does not depend on what the compiler would fuse.
 __device__ __forceinline__ float sum_squares(float4 v) { return fmaf(v.w, v.w, fmaf(v.z, v.z, fmaf(v.x, v.x, __fmul_rn(v.y, v.y)))); }
 
-// Four elements of a residual row; K-split partial sums that the producing GEMM left are folded in (and x written back).
-__device__ __forceinline__ float4 norm_load(float* xr, const float* partials, int splits, size_t row0, size_t stride, int i) {
-  float4 v = *reinterpret_cast<const float4*>(xr + i);
-  if (splits > 1) {
-    int sidx = 0;
-    for (; sidx + 8 <= splits; sidx += 8) {
-      float4 a[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) a[u] = ld_cg(reinterpret_cast<const float4*>(partials + (size_t)(sidx + u) * stride + row0 + i));
-#pragma unroll
-      for (int u = 0; u < 8; ++u) { v.x += a[u].x; v.y += a[u].y; v.z += a[u].z; v.w += a[u].w; }
-    }
-    for (; sidx < splits; ++sidx) {
-      const float4 a = ld_cg(reinterpret_cast<const float4*>(partials + (size_t)sidx * stride + row0 + i));
-      v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
-    }
-    *reinterpret_cast<float4*>(xr + i) = v;
-  }
-  return v;
-}
-
 template <typename OT, typename GT>
 __device__ __forceinline__ void norm_store(OT* out, OT* out_lo, size_t o, float4 v, float inv, const GT* gain) {
   const float y[4] = {v.x * inv * to_f32(gain[0]), v.y * inv * to_f32(gain[1]), v.z * inv * to_f32(gain[2]), v.w * inv * to_f32(gain[3])};
@@ -78,24 +57,19 @@ __device__ __forceinline__ void norm_store(OT* out, OT* out_lo, size_t o, float4
 }
 
 template <typename OT, typename GT>
-__global__ void rmsnorm_kernel(float* x, const GT* __restrict__ gain, OT* out, OT* out_lo, int d, float eps,
-                               const int32_t* src, const int32_t* n_active, const float* partials, int splits, int T) {
+__global__ void rmsnorm_kernel(const float* x, const GT* __restrict__ gain, OT* out, OT* out_lo, int d, float eps,
+                               const int32_t* n_active) {
   RSD_PDL_SYNC_UNLESS_IDLE(n_active);
   __shared__ float red[33];
   const int t = blockIdx.x;
-  int st = t;
-  if (src != nullptr) {
-    st = src[t];
-    if (st < 0) return;
-  }
-  float* xr = x + (size_t)st * d;
+  const float* xr = x + (size_t)t * d;
   float ss = 0.f;
   // the row stays in registers between the two halves (up to kNormVecs float4 a thread; wider rows are read again)
   float4 keep[kNormVecs];
 #pragma unroll
   for (int k = 0; k < kNormVecs; ++k) {
     const int i = (k * blockDim.x + threadIdx.x) * 4;
-    if (i < d) keep[k] = norm_load(xr, partials, splits, (size_t)st * d, (size_t)T * d, i);
+    if (i < d) keep[k] = *reinterpret_cast<const float4*>(xr + i);
   }
 #pragma unroll
   for (int k = 0; k < kNormVecs; ++k) {
@@ -103,8 +77,7 @@ __global__ void rmsnorm_kernel(float* x, const GT* __restrict__ gain, OT* out, O
     if ((k * (int)blockDim.x + (int)threadIdx.x) * 4 < d) ss += sum_squares(v);
   }
   for (int i = (kNormVecs * blockDim.x + threadIdx.x) * 4; i < d; i += blockDim.x * 4) {
-    const float4 v = norm_load(xr, partials, splits, (size_t)st * d, (size_t)T * d, i);
-    ss += sum_squares(v);
+    ss += sum_squares(*reinterpret_cast<const float4*>(xr + i));
   }
   ss = block_sum(ss, red);
   const float inv = rsqrtf(ss / (float)d + eps);
@@ -141,17 +114,17 @@ cudaError_t launch_bf16_to_f16(const void* src, void* dst, size_t n, cudaStream_
   return launched(1);
 }
 
-cudaError_t launch_rmsnorm(int dtype, float* x, const void* gain, void* out, void* out_lo, int T, int d, float eps,
-                           const int32_t* src, const int32_t* n_active, SplitSum pending, cudaStream_t s, bool out_f16) {
+cudaError_t launch_rmsnorm(int dtype, const float* x, const void* gain, void* out, void* out_lo, int T, int d, float eps,
+                           const int32_t* n_active, cudaStream_t s, bool out_f16) {
   if (T <= 0) return cudaSuccess;
   // as few threads as keep the row in registers: more rows are in flight on an SM
   const int threads = d > 256 * 4 * kNormVecs ? 512 : 256;
   if (dtype == 1 && out_f16)
-    RSD_LAUNCH((rmsnorm_kernel<__half, __nv_bfloat16>), T, threads, 0, s, x, (const __nv_bfloat16*)gain, (__half*)out, (__half*)nullptr, d, eps, src, n_active, pending.partials, pending.splits, T);
+    RSD_LAUNCH((rmsnorm_kernel<__half, __nv_bfloat16>), T, threads, 0, s, x, (const __nv_bfloat16*)gain, (__half*)out, (__half*)nullptr, d, eps, n_active);
   else if (dtype == 1)
-    RSD_LAUNCH((rmsnorm_kernel<__nv_bfloat16, __nv_bfloat16>), T, threads, 0, s, x, (const __nv_bfloat16*)gain, (__nv_bfloat16*)out, (__nv_bfloat16*)out_lo, d, eps, src, n_active, pending.partials, pending.splits, T);
+    RSD_LAUNCH((rmsnorm_kernel<__nv_bfloat16, __nv_bfloat16>), T, threads, 0, s, x, (const __nv_bfloat16*)gain, (__nv_bfloat16*)out, (__nv_bfloat16*)out_lo, d, eps, n_active);
   else
-    RSD_LAUNCH((rmsnorm_kernel<float, float>), T, threads, 0, s, x, (const float*)gain, (float*)out, nullptr, d, eps, src, n_active, pending.partials, pending.splits, T);
+    RSD_LAUNCH((rmsnorm_kernel<float, float>), T, threads, 0, s, x, (const float*)gain, (float*)out, nullptr, d, eps, n_active);
   return launched(1);
 }
 
