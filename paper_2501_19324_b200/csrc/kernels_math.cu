@@ -39,8 +39,8 @@ cudaError_t launch_embed(int dtype, const void* embed, PassView p, float* x, int
 // ---------------------------------------------------------------------------------------------
 // RMSNorm: out = x * gain / sqrt(mean(x^2) + eps), one block per token, x kept in registers
 // ---------------------------------------------------------------------------------------------
-// Bound by DRAM in the dense passes (8192 x 3584: 117 MB in, 59 MB out).
-constexpr int kNormVecs = 4;
+// Bound by DRAM in the dense passes (8192 x 3584: 117 MB in, 59 MB out: 29.5 us from and to L2).  A thread keeps VECS
+// vectors of four elements; the block has as many threads as that takes (launch_rmsnorm), so that narrow rows leave none idle.
 
 // The roundings spelled out: the sum does not depend on what the compiler would fuse.
 __device__ __forceinline__ float sum_squares(float4 v) { return fmaf(v.w, v.w, fmaf(v.z, v.z, fmaf(v.x, v.x, __fmul_rn(v.y, v.y)))); }
@@ -56,7 +56,7 @@ __device__ __forceinline__ void norm_store(OT* out, OT* out_lo, size_t o, float4
   }
 }
 
-template <typename OT, typename GT>
+template <typename OT, typename GT, int VECS>
 __global__ void rmsnorm_kernel(const float* x, const GT* __restrict__ gain, OT* out, OT* out_lo, int d, float eps,
                                const int32_t* n_active) {
   RSD_PDL_SYNC_UNLESS_IDLE(n_active);
@@ -64,30 +64,30 @@ __global__ void rmsnorm_kernel(const float* x, const GT* __restrict__ gain, OT* 
   const int t = blockIdx.x;
   const float* xr = x + (size_t)t * d;
   float ss = 0.f;
-  // the row stays in registers between the two halves (up to kNormVecs float4 a thread; wider rows are read again)
-  float4 keep[kNormVecs];
+  // the row stays in registers between the two halves (wider ones are read again)
+  float4 keep[VECS];
 #pragma unroll
-  for (int k = 0; k < kNormVecs; ++k) {
+  for (int k = 0; k < VECS; ++k) {
     const int i = (k * blockDim.x + threadIdx.x) * 4;
     if (i < d) keep[k] = *reinterpret_cast<const float4*>(xr + i);
   }
 #pragma unroll
-  for (int k = 0; k < kNormVecs; ++k) {
+  for (int k = 0; k < VECS; ++k) {
     const float4 v = keep[k];
     if ((k * (int)blockDim.x + (int)threadIdx.x) * 4 < d) ss += sum_squares(v);
   }
-  for (int i = (kNormVecs * blockDim.x + threadIdx.x) * 4; i < d; i += blockDim.x * 4) {
+  for (int i = (VECS * blockDim.x + threadIdx.x) * 4; i < d; i += blockDim.x * 4) {
     ss += sum_squares(*reinterpret_cast<const float4*>(xr + i));
   }
   ss = block_sum(ss, red);
   const float inv = rsqrtf(ss / (float)d + eps);
   const size_t o = (size_t)t * d;
 #pragma unroll
-  for (int k = 0; k < kNormVecs; ++k) {
+  for (int k = 0; k < VECS; ++k) {
     const int i = (k * blockDim.x + threadIdx.x) * 4;
     if (i < d) norm_store<OT>(out, out_lo, o + i, keep[k], inv, gain + i);
   }
-  for (int i = (kNormVecs * blockDim.x + threadIdx.x) * 4; i < d; i += blockDim.x * 4)
+  for (int i = (VECS * blockDim.x + threadIdx.x) * 4; i < d; i += blockDim.x * 4)
     norm_store<OT>(out, out_lo, o + i, *reinterpret_cast<const float4*>(xr + i), inv, gain + i);
 }
 
@@ -117,14 +117,21 @@ cudaError_t launch_bf16_to_f16(const void* src, void* dst, size_t n, cudaStream_
 cudaError_t launch_rmsnorm(int dtype, const float* x, const void* gain, void* out, void* out_lo, int T, int d, float eps,
                            const int32_t* n_active, cudaStream_t s, bool out_f16) {
   if (T <= 0) return cudaSuccess;
-  // as few threads as keep the row in registers: more rows are in flight on an SM
-  const int threads = d > 256 * 4 * kNormVecs ? 512 : 256;
-  if (dtype == 1 && out_f16)
-    RSD_LAUNCH((rmsnorm_kernel<__half, __nv_bfloat16>), T, threads, 0, s, x, (const __nv_bfloat16*)gain, (__half*)out, (__half*)nullptr, d, eps, n_active);
-  else if (dtype == 1)
-    RSD_LAUNCH((rmsnorm_kernel<__nv_bfloat16, __nv_bfloat16>), T, threads, 0, s, x, (const __nv_bfloat16*)gain, (__nv_bfloat16*)out, (__nv_bfloat16*)out_lo, d, eps, n_active);
-  else
-    RSD_LAUNCH((rmsnorm_kernel<float, float>), T, threads, 0, s, x, (const float*)gain, (float*)out, nullptr, d, eps, n_active);
+  // As few threads as keep the row in registers: more rows are in flight on an SM.  Up to 1024 columns a vector a thread (64 to
+  // 256 threads), up to 4096 two or four and 256 threads, beyond 512 threads: 8192 x 256, bf16, 11.9 us with 256 threads and four
+  // vectors, 9.0 with 64 and one; 2048 x 512 4.2 / 3.3, 8192 x 1536 16.0 / 13.2.
+#define RSD_NORM(OT, GT, VECS, threads, lo) RSD_LAUNCH((rmsnorm_kernel<OT, GT, VECS>), T, threads, 0, s, x, (const GT*)gain, (OT*)out, lo, d, eps, n_active)
+#define RSD_NORM_D(OT, GT, lo)                                       \
+  do {                                                               \
+    if (d <= 1024) RSD_NORM(OT, GT, 1, d <= 256 ? 64 : (d <= 512 ? 128 : 256), lo); \
+    else if (d <= 2048) RSD_NORM(OT, GT, 2, 256, lo);                \
+    else RSD_NORM(OT, GT, 4, d <= 4096 ? 256 : 512, lo);             \
+  } while (0)
+  if (dtype == 1 && out_f16) RSD_NORM_D(__half, __nv_bfloat16, (__half*)nullptr);
+  else if (dtype == 1) RSD_NORM_D(__nv_bfloat16, __nv_bfloat16, (__nv_bfloat16*)out_lo);
+  else RSD_NORM_D(float, float, (float*)nullptr);
+#undef RSD_NORM_D
+#undef RSD_NORM
   return launched(1);
 }
 

@@ -142,6 +142,26 @@ def test_rmsnorm_rope_swiglu():
     np.testing.assert_allclose(got, a / (1 + np.exp(-a)) * b, rtol=1e-6, atol=1e-6)
 
 
+@pytest.mark.parametrize("d", [4, 252, 256, 260, 512, 516, 1024, 1028, 2048, 2052, 4096, 4100, 8192, 8196, 12288])
+def test_rmsnorm_widths(d):
+    """Both sides of every width at which the block or the vectors a thread keeps change, rows that are read again, and an output
+    that starts off a 16-byte boundary.  A thread adds at most 24 squares, warps and block ten partial sums: 34 roundings of the
+    sum, half of that in the root, and five more in root, quotient and products: 22 * 2^-24."""
+    rng = np.random.default_rng(d)
+    T = 3
+    x = (rng.normal(size=(T, d)) * 3).astype(np.float32)
+    g = (1 + 0.1 * rng.normal(size=d)).astype(np.float32)
+    xd = x.astype(np.float64)
+    root = np.sqrt((xd * xd).mean(axis=1, keepdims=True) + 1e-6)
+    np.testing.assert_allclose(rb.k_rmsnorm(dev(x), dev(g), 1e-6).cpu().numpy(), xd * g / root, rtol=22 * 2.0 ** -24, atol=0)
+    g16 = dev(g, torch.bfloat16)
+    want16 = xd * g16.double().cpu().numpy() / root
+    np.testing.assert_allclose(rb.k_rmsnorm(dev(x), g16, 1e-6).float().cpu().numpy(), want16, rtol=2 ** -8, atol=0)
+    x_d, off = dev(x), torch.zeros(T * d + 8, dtype=torch.bfloat16, device="cuda")
+    assert rb.lib().rsd_k_rmsnorm(x_d.data_ptr(), g16.data_ptr(), off.data_ptr() + 2, T, d, 1e-6, 1, torch.cuda.current_stream().cuda_stream) == 0
+    np.testing.assert_allclose(off[1:T * d + 1].view(T, d).float().cpu().numpy(), want16, rtol=2 ** -8, atol=0)
+
+
 @pytest.mark.parametrize("lo,hi", [(-1e-30, 1e-30), (-1.0, 1.0), (-30.0, 30.0), (-86.9, -80.0), (-88.7, -87.0), (-120.0, -87.0), (80.0, 1e4)])
 def test_swiglu_over_its_range(lo, hi):
     """The exponential is good to 2 ulp, sum, quotient and product to half an ulp each: 3.5 ulp = 3.5 * 2^-23, plus an ulp for the
