@@ -595,11 +595,12 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
   return RSD_OK;
 }
 
-// Multi-token pass over the flat list built by launch_build_pass, `chunk` tokens at a time.
-int run_ingest(rsd_ctx* c, int which, int n_total, bool want_reward, cudaStream_t s) {
+// Multi-token pass over the flat list of `rows` sequences at most built by launch_build_pass, `chunk` tokens at a time.
+int run_ingest(rsd_ctx* c, int which, int n_total, int rows, bool want_reward, cudaStream_t s) {
   for (int c0 = 0; c0 < n_total; c0 += c->chunk) {
     const int Tc = std::min(c->chunk, n_total - c0);
-    PassView p{c->st.pass_tok_id + c0, c->st.pass_tok_row + c0, c->st.pass_tok_pos + c0, Tc, nullptr};
+    PassView p{c->st.pass_tok_id + c0, c->st.pass_tok_row + c0, c->st.pass_tok_pos + c0, Tc, nullptr,
+               (int)(((long)rows * Tc + n_total - 1) / n_total)};
     int rc = forward_pass(c, which, p, s);
     if (rc) return rc;
     if (want_reward) {
@@ -1114,14 +1115,14 @@ int rsd_prefill(rsd_ctx* c, const int32_t* tokens, const int32_t* offsets, int32
   CU(launch_build_pass(c->st, RSD_DRAFT, kPassIngestDraft, 1, s));
   rc = read_scalars(c, s, &sc);
   if (rc) return rc;
-  rc = run_ingest(c, RSD_DRAFT, sc.n_tok, false, s);
+  rc = run_ingest(c, RSD_DRAFT, sc.n_tok, c->st.B, false, s);
   if (rc) return rc;
   c->ctr.ingest_tokens[RSD_DRAFT] += sc.n_tok;
   if (!merged) {
     CU(launch_build_pass(c->st, RSD_PRM, kPassScorePrm, 1, s));
     rc = read_scalars(c, s, &sc);
     if (rc) return rc;
-    rc = run_ingest(c, RSD_PRM, sc.n_tok, false, s);
+    rc = run_ingest(c, RSD_PRM, sc.n_tok, c->st.B, false, s);
     if (rc) return rc;
     c->ctr.ingest_tokens[RSD_PRM] += sc.n_tok;
   }
@@ -1170,7 +1171,7 @@ static int step_impl(rsd_ctx* c, float delta, int min_target_rows, void* cuda_st
   CU(launch_build_pass(c->st, RSD_DRAFT, kPassIngestDraft, 1, s));
   if ((rc = read_scalars(c, s, &sc))) return rc;
   const int n_sync = sc.n_tok;
-  if ((rc = run_ingest(c, RSD_DRAFT, n_sync, false, s))) return rc;
+  if ((rc = run_ingest(c, RSD_DRAFT, n_sync, B, false, s))) return rc;
   PHASE(1);
   if ((rc = decode_phase(c, RSD_DRAFT, 0, B, s))) return rc;
   PHASE(2);
@@ -1184,7 +1185,7 @@ static int step_impl(rsd_ctx* c, float delta, int min_target_rows, void* cuda_st
     CU(launch_build_pass(c->st, RSD_PRM, kPassScorePrm, 1, s));
     if ((rc = read_scalars(c, s, &sc))) return rc;
     n_prm = sc.n_tok;
-    if ((rc = run_ingest(c, RSD_PRM, n_prm, true, s))) return rc;
+    if ((rc = run_ingest(c, RSD_PRM, n_prm, B, true, s))) return rc;
   }
   PHASE(3);
   // gate, compaction of the waiting rows; once enough of them wait: target catch-up and decode
@@ -1196,7 +1197,7 @@ static int step_impl(rsd_ctx* c, float delta, int min_target_rows, void* cuda_st
   const bool target_runs = target_pass_due(n_rej, sc.n_live, min_target_rows);
   c->last_n_rej = n_rej;
   PHASE(4);
-  if (target_runs && (rc = run_ingest(c, RSD_TARGET, n_catch, false, s))) return rc;
+  if (target_runs && (rc = run_ingest(c, RSD_TARGET, n_catch, n_rej, false, s))) return rc;
   PHASE(5);
   if (target_runs && (rc = c->sd_k > 0 ? decode_phase_sd(c, n_rej, s) : decode_phase(c, RSD_TARGET, 1, n_rej, s))) return rc;
   PHASE(6);

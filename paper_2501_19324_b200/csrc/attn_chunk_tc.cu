@@ -429,10 +429,20 @@ attn_chunk_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
 
 }  // namespace
 
-// The one-pass kernel for long chunks (attn_chunk_long.cu) wants at least a few dozen CTAs of two query tiles each: from 1024
-// tokens on it wins (32 rows x 64 tokens over 300, 12 / 2 heads: 54 us here, 43 us there; 2 x 600 over 100, 28 / 4: 60 and 46),
-// below it leaves more of the chip idle than it saves (8 x 128 tokens: 25 and 33 us, 64 tokens: 24 and 29).
-static bool attn_chunk_long_pays(int T) { return T > 1024; }
+// Whether a chunk of more than 1024 tokens goes to the one-pass kernel (attn_chunk_long.cu).  Its CTAs hold two query tiles each
+// and take 0.95 (long prefixes) to 2 times (a few tokens over a few hundred keys) as long as the CTAs here, of which there are
+// twice as many: it pays by the waves it saves.  One wave either way, up to 74 of its CTAs, it loses: 64 x 20 tokens over 300 keys,
+// 12 / 2 heads, 25.9 us here, 40.2 there; 16 x 65 over 300 26.9 / 32.6; 128 x 8 over 300, 8 / 4 heads, 16.7 / 31.  One wave
+// against two it wins: 32 x 64 over 300, 12 / 2 heads, 44.9 / 33.1; 2 x 600 over 100, 28 / 4, 49.3 / 35.0; three waves against
+// five and the like as well, 0.5 to 1.0 of the time but for runs of eight tokens over 300 keys (1.1).  Two waves against three the
+// length of the rows' runs decides: 76 x 20 over 300, 28 / 4 heads, 1.09, 38 x 40 over 300 0.90, 12 x 128 over 300 0.88 of the time.
+static bool attn_chunk_long_pays(int T, int H, int KV, int rows) {
+  if (T <= 1024) return false;
+  const int QT = 128 / (H / KV);
+  const int here = ((T + QT - 1) / QT * KV + 147) / 148, there = ((T + 2 * QT - 1) / (2 * QT) * KV + 147) / 148;
+  if (here * 2 == there * 3) return rows <= 0 || T / rows >= 32;
+  return here * 5 >= there * 8;
+}
 
 bool attn_chunk_tc_supported(int kv_dtype, int H, int KV, int hd, int T) {
   return kv_dtype == 2 && hd == kHd && KV >= 1 && H % KV == 0 && H / KV <= 8 && T >= 64;
@@ -441,7 +451,7 @@ bool attn_chunk_tc_supported(int kv_dtype, int H, int KV, int hd, int T) {
 cudaError_t launch_attn_chunk_tc(const float* q, PassView p, KvView kv, void* out, void* out_lo, int out_dtype, int H, int KV,
                                  int* err, cudaStream_t s) {
   if (p.T <= 0) return cudaSuccess;
-  if (attn_chunk_long_pays(p.T)) return launch_attn_chunk_long(q, p, kv, out, out_lo, out_dtype, H, KV, err, s);
+  if (attn_chunk_long_pays(p.T, H, KV, p.rows)) return launch_attn_chunk_long(q, p, kv, out, out_lo, out_dtype, H, KV, err, s);
   const int G = H / KV, QT = 128 / G;
   dim3 grid((p.T + QT - 1) / QT, KV);
   CUtensorMap tm_k, tm_v;

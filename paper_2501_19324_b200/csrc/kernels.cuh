@@ -41,6 +41,7 @@ struct PassView {
   const int32_t* tok_pos;
   int T;
   const int32_t* n_active;
+  int rows = 0;                // about how many sequences the list holds (0: not known); for choosing a kernel
 };
 
 // Where one model keeps keys and values: per layer a slab of pages, each page holding the keys

@@ -462,7 +462,7 @@ def test_chunk_attention_against_definition(dtype, hd, H, KV):
             np.testing.assert_allclose(got[t, h], want, rtol=0, atol=tol)
 
 
-@pytest.mark.parametrize("H,KV", [(12, 2), (28, 4), (8, 1), (3, 3)])
+@pytest.mark.parametrize("H,KV", [(12, 2), (28, 4), (8, 1), (3, 3), (18, 3), (64, 8), (24, 24)])
 def test_long_chunk_attention_one_pass(H, KV):
     """More than 1024 entries: rows of one token, rows that end inside a key tile, at its edge and one token on; tiles that
     straddle rows, an idle entry, prefixes of several key tiles; scores that rise along the context so that the reference
