@@ -403,10 +403,10 @@ attn_decode_kernel(const float* q, KT* pool, const int32_t* page_table, int max_
     } else if (n_splits == 1) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) O[i] /= L;
-      store_operand4<OT>(out, out_lo, ((size_t)slot * H + h) * HD + dd, O);
+      store_operand4_any<OT>(out, out_lo, ((size_t)slot * H + h) * HD + dd, O);
     } else {
       const size_t base = ((size_t)slot * H + h) * n_splits + split;
-      *reinterpret_cast<float4*>(part_o + base * HD + dd) = make_float4(O[0], O[1], O[2], O[3]);
+      store_operand4_any<float>(part_o, nullptr, base * HD + dd, O);     // the scratch is a caller's too
       if (dd == 0) { part_ml[base * 2] = M; part_ml[base * 2 + 1] = L; }
     }
   }

@@ -48,12 +48,7 @@ __device__ __forceinline__ float sum_squares(float4 v) { return fmaf(v.w, v.w, f
 template <typename OT, typename GT>
 __device__ __forceinline__ void norm_store(OT* out, OT* out_lo, size_t o, float4 v, float inv, const GT* gain) {
   const float y[4] = {v.x * inv * to_f32(gain[0]), v.y * inv * to_f32(gain[1]), v.z * inv * to_f32(gain[2]), v.w * inv * to_f32(gain[3])};
-  if (((uintptr_t)out & 15) == 0) {
-    store_operand4<OT>(out, out_lo, o, y);
-  } else {                                     // a caller's buffer may start anywhere
-#pragma unroll
-    for (int k = 0; k < 4; ++k) store_operand<OT>(out, out_lo, o + k, y[k]);
-  }
+  store_operand4_any<OT>(out, out_lo, o, y);
 }
 
 template <typename OT, typename GT, int VECS>

@@ -537,6 +537,25 @@ def test_chunk_attention_long_prefix(H, KV):
             np.testing.assert_allclose(got[t, h], want, rtol=0, atol=2e-3)
 
 
+@pytest.mark.parametrize("ctx", [[5, 100, 33], [700, 400, 3], [9000]])
+def test_decode_attention_buffers_may_start_anywhere(ctx):
+    """One split, a cluster of splits, more splits than a cluster: output at a 4-byte and scratch at an 8-byte boundary give the
+    results of aligned buffers."""
+    rng = np.random.default_rng(31)
+    H, KV, hd, B = 12, 2, 128, len(ctx)
+    max_pages = (max(ctx) + 15) // 16
+    pool, table, _, _ = paged_kv(rng, B, KV, hd, ctx, torch.float16, max_pages)
+    q, lens = dev(rng.normal(size=(B, H, hd)).astype(np.float32)), dev(np.array(ctx, np.int32))
+    want = rb.k_attn_decode(q, pool, table, lens, KV)
+    nbytes = rb.lib().rsd_k_attn_decode_scratch_bytes(B, H, hd, max_pages * 16)
+    out = torch.full((B * H * hd + 4,), np.nan, device="cuda")
+    scratch = torch.empty(nbytes + 16, dtype=torch.uint8, device="cuda")
+    assert rb.lib().rsd_k_attn_decode(q.data_ptr(), pool.data_ptr(), table.data_ptr(), lens.data_ptr(), out.data_ptr() + 4, B, H, KV, hd, max_pages,
+                                      2, scratch.data_ptr() + 8, nbytes, torch.cuda.current_stream().cuda_stream) == 0
+    assert torch.equal(out[1:B * H * hd + 1].view(B, H, hd), want)
+    assert bool(out[[0, -3, -2, -1]].isnan().all())
+
+
 @pytest.mark.parametrize("hd,H,KV", [(128, 12, 2), (128, 64, 8), (64, 4, 2), (128, 16, 1)])
 def test_extended_precision_attention(hd, H, KV):
     """fp16 cache with keys and values kept as hi + lo pairs, queries and softmax weights as hi + lo
