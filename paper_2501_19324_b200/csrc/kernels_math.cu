@@ -603,7 +603,8 @@ cudaError_t launch_rope_only(float* v, const int32_t* pos, int T, int n_heads, i
 // ---------------------------------------------------------------------------------------------
 constexpr int kGenericWarps = 16;
 
-template <typename KT, typename OT, int HD>
+// VEC: 16-byte loads; a caller's pool may start anywhere, and one off a 16-byte boundary is read element by element.
+template <typename KT, typename OT, int HD, bool VEC>
 __global__ void __launch_bounds__(32 * kGenericWarps)
 attn_generic_kernel(const float* q, PassView p, const KT* pool, const int32_t* page_table, int max_pages, OT* out, OT* out_lo,
                     int H, int KV, int pf) {
@@ -639,10 +640,17 @@ attn_generic_kernel(const float* q, PassView p, const KT* pool, const int32_t* p
     if (pg + n_warps < n_pages) page = ld_cg(pt + pg + n_warps);
     const int n = min(kPageTokens, pos + 1 - pg * kPageTokens);
     uint4 kr[NK], vr[DPL * NV];
+    if (VEC) {
 #pragma unroll
-    for (int i = 0; i < NK; ++i) kr[i] = *reinterpret_cast<const uint4*>(kb + i * VN);
+      for (int i = 0; i < NK; ++i) kr[i] = *reinterpret_cast<const uint4*>(kb + i * VN);
 #pragma unroll
-    for (int i = 0; i < DPL * NV; ++i) vr[i] = *reinterpret_cast<const uint4*>(vb + i * VN);
+      for (int i = 0; i < DPL * NV; ++i) vr[i] = *reinterpret_cast<const uint4*>(vb + i * VN);
+    } else {
+#pragma unroll
+      for (int i = 0; i < NK * VN; ++i) reinterpret_cast<KT*>(kr)[i] = kb[i];
+#pragma unroll
+      for (int i = 0; i < DPL * NV * VN; ++i) reinterpret_cast<KT*>(vr)[i] = vb[i];
+    }
     float part[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int i = 0; i < NK; ++i) {
@@ -704,7 +712,12 @@ cudaError_t launch_attn_generic(int kv_dtype, const float* q, PassView p, KvView
   // four warps a block waste fewer on short contexts
   const int threads = 32 * (blocks <= 148 ? kGenericWarps : (blocks <= 148 * 4 ? 8 : 4));
 #define RSD_ATTN(KT, OT, HD) \
-  RSD_LAUNCH((attn_generic_kernel<KT, OT, HD>), blocks, threads, 0, s, q, p, (const KT*)kv.pool_layer, kv.page_table, kv.max_pages, (OT*)out, (OT*)out_lo, H, KV, 2 + 2 * kv.v_extra)
+  do {                                                                                                                  \
+    if (((uintptr_t)kv.pool_layer & 15) == 0)                                                                           \
+      RSD_LAUNCH((attn_generic_kernel<KT, OT, HD, true>), blocks, threads, 0, s, q, p, (const KT*)kv.pool_layer, kv.page_table, kv.max_pages, (OT*)out, (OT*)out_lo, H, KV, 2 + 2 * kv.v_extra); \
+    else                                                                                                                \
+      RSD_LAUNCH((attn_generic_kernel<KT, OT, HD, false>), blocks, threads, 0, s, q, p, (const KT*)kv.pool_layer, kv.page_table, kv.max_pages, (OT*)out, (OT*)out_lo, H, KV, 2 + 2 * kv.v_extra); \
+  } while (0)
 #define RSD_ATTN_HD(KT, OT) do { if (hd == 128) RSD_ATTN(KT, OT, 128); else RSD_ATTN(KT, OT, 64); } while (0)
   using bf = __nv_bfloat16;
   if (kv_dtype == 2) { if (out_dtype == 1) RSD_ATTN_HD(__half, bf); else RSD_ATTN_HD(__half, float); }

@@ -556,6 +556,20 @@ def test_decode_attention_buffers_may_start_anywhere(ctx):
     assert bool(out[[0, -3, -2, -1]].isnan().all())
 
 
+@pytest.mark.parametrize("dtype,hd,H,KV", [(torch.float32, 64, 4, 2), (torch.float32, 128, 6, 3), (torch.float16, 64, 18, 1), (torch.bfloat16, 128, 16, 1)])
+def test_generic_attention_pool_may_start_anywhere(dtype, hd, H, KV):
+    """fp32 caches and groups of more than eight heads: a pool that starts one element off a 16-byte boundary."""
+    rng = np.random.default_rng(32)
+    ctx = [1, 16, 75, 300]
+    pool, table, _, _ = paged_kv(rng, len(ctx), KV, hd, ctx, dtype, 20)
+    q, lens = dev(rng.normal(size=(len(ctx), H, hd)).astype(np.float32)), dev(np.array(ctx, np.int32))
+    want = rb.k_attn_decode(q, pool, table, lens, KV)
+    moved = torch.empty(pool.numel() + 1, dtype=dtype, device="cuda")[1:].view(pool.shape)
+    moved.copy_(pool)
+    assert moved.data_ptr() % 16 == dtype.itemsize
+    assert torch.equal(rb.k_attn_decode(q, moved, table, lens, KV), want)
+
+
 @pytest.mark.parametrize("hd,H,KV", [(128, 12, 2), (128, 64, 8), (64, 4, 2), (128, 16, 1)])
 def test_extended_precision_attention(hd, H, KV):
     """fp16 cache with keys and values kept as hi + lo pairs, queries and softmax weights as hi + lo
