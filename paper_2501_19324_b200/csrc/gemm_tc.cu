@@ -821,12 +821,22 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_const
   }
 }
 
-// y[m, n] (+)= sum over splits of partials[s][m][n], splits added in order; 4 columns per thread.
+// y[m, n] (+)= sum over splits of partials[s][m][n], splits added in order; 4 columns per thread, or one where a caller's y or
+// scratch does not start on a 16-byte boundary.
 __global__ void __launch_bounds__(256)
 splitk_reduce_kernel(const float* __restrict__ partials, float* __restrict__ Y, int M, int N, int splits, int accumulate,
                      const int32_t* __restrict__ n_active) {
   RSD_PDL_SYNC();
   if (n_active != nullptr && *n_active == 0) return;
+  if (((uintptr_t)Y | (uintptr_t)partials) & 15) {
+    const size_t total = (size_t)M * N;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+      float acc = accumulate ? Y[i] : 0.f;
+      for (int sidx = 0; sidx < splits; ++sidx) acc += __ldcg(partials + (size_t)sidx * total + i);
+      Y[i] = acc;
+    }
+    return;
+  }
   const size_t total4 = (size_t)M * N / 4, stride = (size_t)M * N / 4;
   const float4* p4 = reinterpret_cast<const float4*>(partials);
   float4* y4 = reinterpret_cast<float4*>(Y);

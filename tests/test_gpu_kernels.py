@@ -142,6 +142,28 @@ def test_rmsnorm_rope_swiglu():
     np.testing.assert_allclose(got, a / (1 + np.exp(-a)) * b, rtol=1e-6, atol=1e-6)
 
 
+@pytest.mark.parametrize("M,N,K", [(5, 256, 512), (40, 384, 1408), (100, 384, 1408), (128, 640, 768), (300, 384, 512)])
+def test_gemm_buffers_may_start_anywhere(M, N, K):
+    """Result at a 4-byte and scratch at an 8-byte boundary, with a K split (up to 128 rows) and without: the results of aligned
+    buffers, added to y or not."""
+    rng = np.random.default_rng(M)
+    W = dev(ri.cpu_tensor(2, 5, N, K, True), torch.bfloat16)
+    x = dev(rng.normal(size=(M, K)).astype(np.float32))
+    hi = x.to(torch.bfloat16)
+    lo = (x - hi.float()).to(torch.bfloat16)
+    y0 = dev(rng.normal(size=(M, N)).astype(np.float32))
+    nbytes = rb.lib().rsd_k_gemm_scratch_bytes(M, N, K)
+    for accumulate in (0, 1):
+        want = rb.k_gemm(W, hi, y=y0.clone(), accumulate=bool(accumulate), impl=2, x_lo=lo)
+        y = torch.full((M * N + 4,), np.nan, device="cuda")
+        y[1:M * N + 1] = y0.view(-1)
+        scratch = torch.zeros(nbytes + 16, dtype=torch.uint8, device="cuda")
+        assert rb.lib().rsd_k_gemm(W.data_ptr(), hi.data_ptr(), lo.data_ptr(), y.data_ptr() + 4, M, N, K, 1, accumulate, 2, scratch.data_ptr() + 8,
+                                   nbytes, torch.cuda.current_stream().cuda_stream) == 0
+        assert torch.equal(y[1:M * N + 1].view(M, N), want)
+        assert bool(y[[0, -3, -2, -1]].isnan().all())
+
+
 @pytest.mark.parametrize("d", [4, 252, 256, 260, 512, 516, 1024, 1028, 2048, 2052, 4096, 4100, 8192, 8196, 12288])
 def test_rmsnorm_widths(d):
     """Both sides of every width at which the block or the vectors a thread keeps change, rows that are read again, and an output
