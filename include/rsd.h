@@ -327,6 +327,14 @@ int rsd_k_attn_chunk(const float* q, const void* kv_pool, const int32_t* page_ta
                      const int32_t* tok_pos, float* out, int32_t T, int32_t H, int32_t KV, int32_t hd,
                      int32_t max_pages, int32_t dtype, void* cuda_stream);
 
+/* Failure path of the two tcgen05 chunk-attention kernels (one_pass 0 or 1) without a fault, as rsd_debug_gemm_wait_probe:
+ * one CTA over 16 entries of eight heads on one KV head whose page copies are never issued, so the MMA warp's bounded
+ * wait (cut to a few thousand polls) runs out.  Returns RSD_ERR_TIMEOUT (the expected outcome).  q [16, 8, 128] fp32 is
+ * read; kv_pool (one fp16 page, 16-byte aligned) and page_table [1] are mapped but not read; tok_row [16] = 0,
+ * tok_pos [16] in 0..15; out [16, 8, 128] is not written; flag: one DEVICE int.  Synchronises the stream.       */
+int rsd_debug_attn_wait_probe(int32_t one_pass, const float* q, const void* kv_pool, const int32_t* page_table,
+                              const int32_t* tok_row, const int32_t* tok_pos, float* out, int32_t* flag, void* cuda_stream);
+
 /* Gate + compaction (Table 1 binary step; Algorithm 1 else-branch batched over rows):
  * accept[b] = live[b] && rewards[b] >= delta; rej_idx [B] receives the ascending list of live
  * rejected rows, *n_rej (device) their count.  B up to 2^24.  scratch: 4 * ceil(B / 1024) bytes. */

@@ -1524,6 +1524,22 @@ int rsd_k_attn_chunk(const float* q, const void* kv_pool, const int32_t* page_ta
   return RSD_OK;
 }
 
+int rsd_debug_attn_wait_probe(int32_t one_pass, const float* q, const void* kv_pool, const int32_t* page_table, const int32_t* tok_row,
+                              const int32_t* tok_pos, float* out, int32_t* flag, void* cuda_stream) {
+  if (!q || !kv_pool || ((uintptr_t)kv_pool & 15) || ((uintptr_t)q & 15) || !page_table || !tok_row || !tok_pos || !out || !flag) return RSD_ERR_ARG;
+  cudaStream_t s = (cudaStream_t)cuda_stream;
+  PassView p{nullptr, tok_row, tok_pos, 16, nullptr};
+  KvView kv{const_cast<void*>(kv_pool), page_table, 1};
+  KCU(cudaMemsetAsync(flag, 0, sizeof(int32_t), s));
+  KCU(launch_attn_wait_probe(one_pass != 0, q, p, kv, out, flag, s));
+  int32_t raised = 0;
+  KCU(cudaMemcpyAsync(&raised, flag, sizeof(raised), cudaMemcpyDeviceToHost, s));
+  KCU(cudaStreamSynchronize(s));
+  if (raised == 0) return RSD_OK;                     // the wait did not run out: not what the probe is for
+  g_create_error = "a bounded wait inside the tensor-core chunk attention expired";
+  return RSD_ERR_TIMEOUT;
+}
+
 int rsd_k_gate_compact(const float* rewards, const uint8_t* live, float delta, uint8_t* accept, int32_t* rej_idx,
                        int32_t* n_rej, int32_t B, void* scratch, size_t scratch_bytes, void* cuda_stream) {
   if (!rewards || !live || !accept || !rej_idx || !n_rej || B < 1 || B > (1 << 24)) return RSD_ERR_ARG;

@@ -73,7 +73,7 @@ __device__ __forceinline__ Segment segment_at(const Meta* mt, int seg, int n_ent
   return s;
 }
 
-template <typename OT>
+template <typename OT, bool PROBE = false>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_chunk_long_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const float* q, PassView p,
                        const __half* pool, const int32_t* page_table, int max_pages, OT* out, OT* out_lo, int H, int KV, int QT,
@@ -141,7 +141,7 @@ attn_chunk_long_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     uint32_t it = 0;
     int seg = 0;
     bool ok = true;
-    while (seg < n_ent && ok) {
+    while (!PROBE && seg < n_ent && ok) {
       const Segment sg = segment_at(mt, seg, n_ent, QT);
       if (sg.row >= 0) {
         const int n_tiles = max(sg.n[0], sg.n[1]), n_pages = sg.pos_last / kPageTokens + 1;
@@ -198,7 +198,7 @@ attn_chunk_long_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
       bool ok = true;
       int seg = 0;
       auto wait = [&](uint64_t* bar, uint32_t parity) {
-        const bool got = mbar_wait(bar, parity, kProbeLimit);
+        const bool got = mbar_wait(bar, parity, PROBE ? kProbePolls : kProbeLimit);
         return __all_sync(0xFFFFFFFFu, got && !*stop) != 0;
       };
       auto scores = [&](int j, uint32_t k_it) {
@@ -268,7 +268,7 @@ attn_chunk_long_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
         const int pq = mine ? mt->pos[qi] : -1;              // last visible key position; -1: the row is not of this segment
         float m = -INFINITY, l = 0.f;
         for (int t = 0; t < n_tiles; ++t, ++n_s) {
-          ok = wait_sleep(&mt->s_full[wg], n_s & 1u, stop);
+          ok = wait_sleep_warp(&mt->s_full[wg], n_s & 1u, stop);
           if (!ok) break;
           tc_fence_after();
           float v[128];
@@ -319,7 +319,7 @@ attn_chunk_long_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
           if (lane == 0) mbar_arrive(&mt->p_full[wg]);
         }
         if (!ok) break;
-        ok = wait_sleep(&mt->o_full[wg], n_o & 1u, stop);
+        ok = wait_sleep_warp(&mt->o_full[wg], n_o & 1u, stop);
         if (!ok) break;
         ++n_o;
         tc_fence_after();
@@ -353,13 +353,13 @@ attn_chunk_long_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   }
 }
 
-template <typename OT>
+template <typename OT, bool PROBE = false>
 cudaError_t launch_long(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const float* q, PassView p, KvView kv, void* out, void* out_lo,
                         int H, int KV, int* err, cudaStream_t s) {
-  static const cudaError_t set = cudaFuncSetAttribute(attn_chunk_long_kernel<OT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+  static const cudaError_t set = cudaFuncSetAttribute(attn_chunk_long_kernel<OT, PROBE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
   if (set != cudaSuccess) return set;
   const int QT = 128 / (H / KV);
-  RSD_LAUNCH((attn_chunk_long_kernel<OT>), dim3((p.T + 2 * QT - 1) / (2 * QT), KV), kThreads, kSmemBytes, s, tm_k, tm_v, q, p,
+  RSD_LAUNCH((attn_chunk_long_kernel<OT, PROBE>), dim3((p.T + 2 * QT - 1) / (2 * QT), KV), kThreads, kSmemBytes, s, tm_k, tm_v, q, p,
              (const __half*)kv.pool_layer, kv.page_table, kv.max_pages, (OT*)out, (OT*)out_lo, H, KV, QT, err);
   return launched(1);
 }
@@ -367,10 +367,11 @@ cudaError_t launch_long(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const 
 }  // namespace
 
 cudaError_t launch_attn_chunk_long(const float* q, PassView p, KvView kv, void* out, void* out_lo, int out_dtype, int H, int KV, int* err,
-                                   cudaStream_t s) {
+                                   cudaStream_t s, bool probe) {
   if (p.T <= 0) return cudaSuccess;
   CUtensorMap tm_k, tm_v;
   if (!tc_tensor_map_kv(kv.pool_layer, 0, &tm_k) || !tc_tensor_map_kv(kv.pool_layer, 1, &tm_v)) return cudaErrorInvalidValue;
+  if (probe) return launch_long<float, true>(tm_k, tm_v, q, p, kv, out, nullptr, H, KV, err, s);
   if (out_dtype == 2) return launch_long<__half>(tm_k, tm_v, q, p, kv, out, nullptr, H, KV, err, s);
   if (out_dtype == 1) return launch_long<__nv_bfloat16>(tm_k, tm_v, q, p, kv, out, out_lo, H, KV, err, s);
   return launch_long<float>(tm_k, tm_v, q, p, kv, out, nullptr, H, KV, err, s);

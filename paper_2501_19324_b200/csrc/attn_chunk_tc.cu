@@ -80,13 +80,14 @@ struct Meta {
 };
 static_assert(sizeof(Meta) <= kMetaBytes, "metadata block");
 
-template <typename OT>
+template <typename OT, bool PROBE = false>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_chunk_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                      const float* __restrict__ q, PassView p, const __half* __restrict__ pool,
                      const int32_t* __restrict__ page_table, int max_pages, OT* __restrict__ out, OT* __restrict__ out_lo,
                      int H, int KV, int QT, int* __restrict__ err) {
   RSD_PDL_SYNC();
+  constexpr uint32_t kLimit = PROBE ? kProbePolls : kProbeLimit;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* ring = smem;
@@ -155,7 +156,7 @@ attn_chunk_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     uint32_t it = 0;
     int seg = 0;
     bool ok = true;
-    while (seg < n_ent && ok) {
+    while (!PROBE && seg < n_ent && ok) {
       const int row = mt->row[seg];
       int e = seg + 1;
       while (e < n_ent && mt->row[e] == row) ++e;
@@ -209,7 +210,7 @@ attn_chunk_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     // when nothing went wrong)
     if (lane == 0) {
       const uint32_t first = it > (uint32_t)kNS ? it - kNS : 0;
-      for (uint32_t j = first; j < it; ++j) mbar_wait(&mt->kv_full[j % kNS], (j / kNS) & 1u, kProbeLimit);
+      for (uint32_t j = first; j < it; ++j) mbar_wait(&mt->kv_full[j % kNS], (j / kNS) & 1u, kLimit);
       if (!ok) fail();
     }
   } else if (warp == kMmaWarp) {
@@ -229,8 +230,8 @@ attn_chunk_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             for (int t = 0; t < n_tiles; ++t, ++itk, ++its) {
               const int st = itk % kNS;
               const uint32_t b = its % kSB;
-              if (!mbar_wait(&mt->kv_full[st], (itk / kNS) & 1u, kProbeLimit) || *stop ||
-                  !mbar_wait(&mt->s_empty[b], ((its / kSB) & 1u) ^ 1u, kProbeLimit) || *stop) { ok = false; break; }
+              if (!mbar_wait(&mt->kv_full[st], (itk / kNS) & 1u, kLimit) || *stop ||
+                  !mbar_wait(&mt->s_empty[b], ((its / kSB) & 1u) ^ 1u, kLimit) || *stop) { ok = false; break; }
               tc_fence_after();
               const uint64_t k_desc = desc_sw128(smem_u32(ring + (size_t)st * kStageBytes), 2048);
 #pragma unroll
@@ -266,14 +267,14 @@ attn_chunk_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
           const int n_tiles = (pos_last / kPageTokens + 1 + 3) / 4;
           itk += n_tiles;                                  // the stages pass 1 went through
           // the output accumulator of the previous segment must have been read out
-          if (n_seg > 0) ok = mbar_wait(&mt->o_empty, (n_seg - 1) & 1u, kProbeLimit) && !*stop;
+          if (n_seg > 0) ok = mbar_wait(&mt->o_empty, (n_seg - 1) & 1u, kLimit) && !*stop;
           for (int t = 0; t < n_tiles && ok; ++t, ++itk, ++itp) {
             const int st = itk % kNS;
             const uint32_t pb = itp & 1u;
             // the weights imply the scores, and those the landed keys; the wait for the stage (over at once) makes
             // the landed values visible to this thread's MMAs
-            if (!mbar_wait(&mt->p_full[pb], (itp >> 1) & 1u, kProbeLimit) || *stop ||
-                !mbar_wait(&mt->kv_full[st], (itk / kNS) & 1u, kProbeLimit) || *stop) { ok = false; break; }
+            if (!mbar_wait(&mt->p_full[pb], (itp >> 1) & 1u, kLimit) || *stop ||
+                !mbar_wait(&mt->kv_full[st], (itk / kNS) & 1u, kLimit) || *stop) { ok = false; break; }
             tc_fence_after();
             const uint64_t v_desc = desc_sw32(smem_u32(ring + (size_t)st * kStageBytes + kKBytes));
 #pragma unroll
@@ -303,7 +304,7 @@ attn_chunk_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       slot[wg][r] = mine_half;
       __syncwarp();
       if (lane == 0) mbar_arrive(&mt->halves);
-      if (!wait_sleep(&mt->halves, n_x & 1u, stop)) return false;
+      if (!wait_sleep_warp(&mt->halves, n_x & 1u, stop)) return false;
       ++n_x;
       *a = slot[0][r]; *b = slot[1][r];
       return true;
@@ -321,7 +322,7 @@ attn_chunk_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         float m = -INFINITY;
         for (int t = 0; t < n_tiles && ok; ++t, ++its) {
           const uint32_t b = its % kSB;
-          ok = wait_sleep(&mt->s_full[b], (its / kSB) & 1u, stop);
+          ok = wait_sleep_warp(&mt->s_full[b], (its / kSB) & 1u, stop);
           if (!ok) break;
           tc_fence_after();
           {
@@ -352,7 +353,7 @@ attn_chunk_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         float l = 0.f;
         for (int t = 0; t < n_tiles && ok; ++t, ++its, ++itp) {
           const uint32_t b = its % kSB, pb = itp & 1u;
-          ok = wait_sleep(&mt->s_full[b], (its / kSB) & 1u, stop);
+          ok = wait_sleep_warp(&mt->s_full[b], (its / kSB) & 1u, stop);
           if (!ok) break;
           tc_fence_after();
           uint32_t pv[16];
@@ -377,7 +378,7 @@ attn_chunk_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
           __syncwarp();
           if (lane == 0) mbar_arrive(&mt->s_empty[b]);
           // the weight tile of two tiles ago must have been multiplied
-          ok = wait_sleep(&mt->p_empty[pb], ((itp >> 1) & 1u) ^ 1u, stop);
+          ok = wait_sleep_warp(&mt->p_empty[pb], ((itp >> 1) & 1u) ^ 1u, stop);
           if (!ok) break;
           tmem_st16(lane_base + kColP + pb * 32 + wg * 16, pv);
           tmem_st_wait();
@@ -393,7 +394,7 @@ attn_chunk_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
           if (!ok) break;
           l = la + lb;
         }
-        ok = wait_sleep(&mt->o_full, n_seg & 1u, stop);
+        ok = wait_sleep_warp(&mt->o_full, n_seg & 1u, stop);
         if (!ok) break;
         tc_fence_after();
         const float inv = l > 0.f ? 1.f / l : 0.f;
@@ -482,6 +483,19 @@ cudaError_t launch_attn_chunk_tc(const float* q, PassView p, KvView kv, void* ou
     RSD_LAUNCH((attn_chunk_tc_kernel<float>), grid, kThreads, kSmemBytes, s, tm_k, tm_v, q, p, (const __half*)kv.pool_layer,
                kv.page_table, kv.max_pages, (float*)out, (float*)nullptr, H, KV, QT, err);
   }
+  return launched(1);
+}
+
+// Launches the PROBE instantiation of the two-pass or of the one-pass kernel on 16 entries of eight heads over one KV head.
+cudaError_t launch_attn_wait_probe(bool one_pass, const float* q, PassView p, KvView kv, float* out, int* err, cudaStream_t s) {
+  if (one_pass) return launch_attn_chunk_long(q, p, kv, out, nullptr, 0, 8, 1, err, s, true);
+  CUtensorMap tm_k, tm_v;
+  if (!tc_tensor_map_kv(kv.pool_layer, 0, &tm_k) || !tc_tensor_map_kv(kv.pool_layer, 1, &tm_v)) return cudaErrorInvalidValue;
+  static const cudaError_t set =
+      cudaFuncSetAttribute(attn_chunk_tc_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+  if (set != cudaSuccess) return set;
+  RSD_LAUNCH((attn_chunk_tc_kernel<float, true>), dim3(1, 1), kThreads, kSmemBytes, s, tm_k, tm_v, q, p, (const __half*)kv.pool_layer,
+             kv.page_table, kv.max_pages, out, (float*)nullptr, 8, 1, 16, err);
   return launched(1);
 }
 

@@ -14,6 +14,10 @@ using namespace tc;
 constexpr int kHd = 128;
 constexpr int kBlockBytes = 4096;                   // keys (or values) of one page and KV head
 constexpr uint32_t kProbeLimit = 1u << 18;          // polls of a bounded wait (a healthy wait ends within microseconds)
+// PROBE (reached only through the wait-probe entry): the fetch warp issues NO copy, so that the first tile never comes; the MMA
+// warp's wait, cut to this many polls, runs out, and the kernel must take its failure path -- error flag raised, softmax warps
+// released, tensor memory freed, clean return -- with nothing in flight.
+constexpr uint32_t kProbePolls = 4096;
 
 // Writes of this thread to shared memory become visible to the tensor cores.
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -102,6 +106,13 @@ __device__ __forceinline__ bool wait_sleep(uint64_t* bar, uint32_t parity, volat
     if (*stop) return false;
   }
   return false;
+}
+
+// ... by a whole warp, with one answer for all lanes: what follows (tensor-memory loads and stores, votes) takes the warp together,
+// and a barrier that completes or a stop that is raised between two lanes' polls would part it.
+__device__ __forceinline__ bool wait_sleep_warp(uint64_t* bar, uint32_t parity, volatile uint32_t* stop) {
+  const bool ok = wait_sleep(bar, parity, stop);
+  return __all_sync(0xFFFFFFFFu, ok) != 0;
 }
 
 template <typename OT> __device__ __forceinline__ void store16(OT* hi, OT* lo, size_t o, const float* v);

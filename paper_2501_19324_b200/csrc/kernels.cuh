@@ -119,7 +119,9 @@ cudaError_t launch_attn_chunk_tc(const float* q, PassView p, KvView kv, void* ou
                                  int* err, cudaStream_t s);
 // ... its one-pass form for long chunks, which launch_attn_chunk_tc picks by the chunk's length.
 cudaError_t launch_attn_chunk_long(const float* q, PassView p, KvView kv, void* out, void* out_lo, int out_dtype, int H, int KV,
-                                   int* err, cudaStream_t s);
+                                   int* err, cudaStream_t s, bool probe = false);
+// The failure path of either: a launch over 16 entries of eight heads, one KV head, whose copies are never issued; *err becomes -5.
+cudaError_t launch_attn_wait_probe(bool one_pass, const float* q, PassView p, KvView kv, float* out, int* err, cudaStream_t s);
 cudaError_t launch_swiglu(int dtype, const float* gu, SplitSum pending, void* out, void* out_lo, int T, int F,
                           const int32_t* n_active, cudaStream_t s);
 

@@ -738,6 +738,40 @@ def test_gate_up_gemm_on_pairs_of_ctas(M, F, K):
     assert int(scratch[4096:4100].view(torch.int32).item()) == 0
 
 
+@pytest.mark.parametrize("one_pass", [0, 1])
+def test_chunk_attention_wait_runs_out_cleanly(one_pass):
+    """Failure path of the two tcgen05 chunk-attention kernels: no copy is issued, the bounded wait runs out, the flag is
+    raised, nothing is written and the kernel returns (its tensor memory freed: the same kernel runs many times afterwards)."""
+    rng = np.random.default_rng(41)
+    T, H, KV = 16, 8, 1
+    q = dev(rng.normal(size=(T, H, 128)).astype(np.float32))
+    pool = torch.zeros(2 * 16 * 128, dtype=torch.float16, device="cuda")
+    table = torch.zeros(1, dtype=torch.int32, device="cuda")
+    row, pos = torch.zeros(T, dtype=torch.int32, device="cuda"), torch.arange(T, dtype=torch.int32, device="cuda")
+    out = torch.full((T, H, 128), 7.0, device="cuda")
+    flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    for _ in range(3):
+        rc = rb.lib().rsd_debug_attn_wait_probe(one_pass, q.data_ptr(), pool.data_ptr(), table.data_ptr(), row.data_ptr(), pos.data_ptr(),
+                                                out.data_ptr(), flag.data_ptr(), stream)
+        assert rc == -5 and int(flag.item()) == -5
+        assert b"bounded wait" in rb.lib().rsd_last_error(None)
+        assert torch.all(out == 7.0)
+    ctx = [700, 900] if one_pass else [100]           # 1600 entries x 24 heads (one pass) or 100 entries (two passes)
+    H, KV = (24, 24) if one_pass else (8, 1)
+    pool, table, Ks, Vs = paged_kv(rng, len(ctx), KV, 128, ctx, torch.float16, 64)
+    rows = np.repeat(np.arange(len(ctx)), ctx).astype(np.int32)
+    poss = np.concatenate([np.arange(c) for c in ctx]).astype(np.int32)
+    qd = rng.normal(size=(len(rows), H, 128)).astype(np.float32)
+    for _ in range(4):
+        got = rb.k_attn_chunk(dev(qd), pool, table, dev(rows), dev(poss), KV).cpu().numpy()
+    for t in (0, 50, len(rows) - 1):
+        b, p = rows[t], poss[t]
+        s = Ks[b][:p + 1, 0].astype(np.float64) @ qd[t, 0].astype(np.float64) / np.sqrt(128)
+        w = np.exp(s - s.max()); w /= w.sum()
+        np.testing.assert_allclose(got[t, 0], w @ Vs[b][:p + 1, 0].astype(np.float64), rtol=0, atol=2e-3)
+
+
 def test_bounded_wait_runs_out_and_the_kernel_leaves_cleanly():
     """RSD_ERR_TIMEOUT without a fault: one CTA of the tensor-core GEMM whose copies are never issued.  Its wait
     (a few thousand polls in this mode) expires, the error flag is raised and reported, tensor memory is freed: the
