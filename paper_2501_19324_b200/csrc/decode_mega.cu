@@ -646,7 +646,7 @@ __device__ __forceinline__ void gemm_phase(const MegaParams& P, int which, const
   for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
     const Item im = item_of(g, it);
     const uint32_t b = ps.ae & 1u;
-    const bool ok = wait_bar(&sh.acc_full[b], (ps.ae >> 1) & 1u, sh, err);
+    const bool ok = __all_sync(0xFFFFFFFFu, wait_bar(&sh.acc_full[b], (ps.ae >> 1) & 1u, sh, err));   // one answer for the warp
     ++ps.ae;
     tc_fence_after();
     const uint32_t taddr = tmem_base + ((uint32_t)(warp * 32) << 16) + b * (uint32_t)mt;

@@ -253,6 +253,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
       ok = mbar_try_wait_sleep(tmem_full, 0, 1000);
       if (!ok && flags[0]) break;                        // the CTA was stopped (an expired wait)
     }
+    ok = __all_sync(0xFFFFFFFFu, ok);          // one answer for the warp: it goes on to tensor-memory loads together
     if (!ok && active != 0 && flags[0] == 0) {
       if (err) atomicCAS(err, 0, -5);
       flags[0] = 1;
@@ -629,6 +630,7 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
       const uint32_t b = n_acc & 1u;
       bool ok = mbar_try_wait(&acc_full[b], (n_acc >> 1) & 1u);
       for (uint32_t i = 0; i < (1u << 21) && !ok && !*stop; ++i) ok = mbar_try_wait_sleep(&acc_full[b], (n_acc >> 1) & 1u, 1000);
+      ok = __all_sync(0xFFFFFFFFu, ok);        // one answer for the warp
       if (!ok) fail();
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + b * (uint32_t)C::kMT;
@@ -805,6 +807,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_const
       const uint32_t b = n_acc & 1u;
       bool ok = mbar_try_wait(&acc_full[b], (n_acc >> 1) & 1u);
       for (uint32_t i = 0; i < (1u << 21) && !ok && !*stop; ++i) ok = mbar_try_wait_sleep(&acc_full[b], (n_acc >> 1) & 1u, 1000);
+      ok = __all_sync(0xFFFFFFFFu, ok);        // one answer for the warp
       if (!ok) fail();
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + b * 256u;
