@@ -297,15 +297,20 @@ gemv_splitk_kernel(const WT* __restrict__ W, const WT* X, const WT* X_lo, float*
 cudaError_t launch_gemm_simt(int dtype, const void* W, const void* x, const void* x_lo, float* y, int M, int N, int K,
                              int accumulate, const int32_t* n_active, cudaStream_t s) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  // Pick the split so that the grid covers the 148 SMs a few times over, as long as every lane has a vector (fp32, up to four
-  // rows) or two.  More rows are more blocks, each with its reductions: splitting them as finely, and holding weights ahead in
-  // registers where no wait is to be bridged, cost 256 x 512 x 1376 146 us instead of 84 and 60 x 512 x 256 12 instead of 5.6.
+  // Pick the split so that the grid covers the 148 SMs a few times over, as long as every lane has two vectors, or one (fp32) where
+  // there are up to four rows or few blocks.  More rows are more blocks, each with its reductions: splitting them as finely, and
+  // holding weights ahead in registers where no wait is to be bridged, cost 256 x 512 x 1376 146 us instead of 84 and 60 x 512 x
+  // 256 12 instead of 5.6; few blocks left whole, 8 x 512 x 256 4.6 us, halved 3.4.
   int ks = 1;
-  const int per_warp = M <= 4 && dtype != 1 ? 128 : 256;
-  while (ks < 8 && (long)N * ks / 8 < 148L * 4 && K / (ks * 2) >= per_warp) ks *= 2;
   const int mt = M <= 4 ? 4 : 8;
+  const long m_blocks = (M + mt - 1) / mt;
+  auto lanes_full = [&](int k) {
+    const long blocks = N * m_blocks * (k / 2) / 8;       // before the step to k
+    return K / k >= (dtype != 1 && (M <= 4 || blocks < 148 || (k == 2 && blocks < 296)) ? 128 : 256);
+  };
+  while (ks < 8 && (long)N * ks / 8 < 148L * 4 && lanes_full(2 * ks)) ks *= 2;
   const bool ahead = M <= 4 || n_active != nullptr;
-  dim3 grid((N + (8 / ks) - 1) / (8 / ks), (M + mt - 1) / mt);
+  dim3 grid((N + (8 / ks) - 1) / (8 / ks), (unsigned)m_blocks);
 #define RSD_GEMV(WT, MT, AHEAD) RSD_LAUNCH((gemv_splitk_kernel<WT, MT, AHEAD>), grid, 256, 0, s, (const WT*)W, (const WT*)x, (const WT*)x_lo, y, M, N, K, ks, accumulate, n_active)
 #define RSD_GEMV_M(WT) do { if (mt == 4) RSD_GEMV(WT, 4, kGemvAhead); else if (ahead) RSD_GEMV(WT, 8, kGemvAhead); else RSD_GEMV(WT, 8, 0); } while (0)
   if (dtype == 1) RSD_GEMV_M(__nv_bfloat16);
