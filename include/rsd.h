@@ -269,6 +269,10 @@ int rsd_debug_gemm_timing_dense(rsd_ctx*, double* ms, double* flops, uint64_t* l
 int rsd_debug_phase_ms(rsd_ctx*, int32_t enable, double* out);
 /* Number of kernels this library has enqueued in this process so far.                          */
 uint64_t rsd_debug_launch_count(void);
+/* Raises the error flag that an expired device-side wait would leave, from the host (a memset on the stream), ahead of
+ * iteration `iteration` of every decode phase from now on; -1 (the default) never.  For testing that a failing phase
+ * ends early with RSD_ERR_TIMEOUT.                                                              */
+int rsd_debug_fail_iteration(rsd_ctx*, int32_t iteration);
 /* Timeline of the last launch of the persistent decode kernel of model `which` (RSD_DRAFT or RSD_TARGET),
  * recorded by its first CTA when RSD_DEBUG_MEGA_PROFILE is set: stamps[0] = kernel start, then for every
  * grid barrier the global-timer value (ns) when the CTA's phase work was done and when the barrier let it

@@ -108,6 +108,7 @@ struct rsd_ctx {
   uint64_t dec_graph_kernels[16] = {};
   int sd_k = 0, slots_max = 0;
 
+  int fail_at = -1;            // rsd_debug_fail_iteration
   unsigned long long* progress = nullptr;   // pinned: how far the running decode phase is (RowState::progress)
   int pass_width = 1;          // consecutive positions of a row that a decode pass writes (a speculative round: sd_k)
   int attn_rows_hint = 0;      // rows expected to be active in the running decode phase (0: all slots)
@@ -320,6 +321,7 @@ size_t layout_workspace(const rsd_config& cfg, const rsd_model* const ms[3], rsd
 #undef TAKE
   if (c) {
     st.progress = c->progress;
+    st.wait_err = (const int32_t*)((char*)gscr + 4096);
     c->st = st; c->B_max = B; c->S = S; c->C = C; c->max_pages = max_pages; c->chunk = chunk; c->T_max = T;
     c->sd_k = sd_k; c->slots_max = slots;
     c->x = x; c->h = h; c->qkv = qkv; c->q = q; c->attn = attn; c->gu = gu; c->act = act; c->logits = logits;
@@ -811,6 +813,11 @@ int follow_phase(rsd_ctx* c, int launched, cudaStream_t s, bool* ended) {
   volatile unsigned long long* word = c->progress;
   for (uint32_t polls = 1;; ++polls) {
     const unsigned long long w = *word;
+    if (w >> 63) {
+      // a device-side wait has expired: the iterations to come would each run into their limits too
+      Scalars sc;
+      return read_scalars(c, s, &sc);
+    }
     const int done = (int)(w >> 32), left = (int)(w & 0xFFFFFFFFull);
     *ended = done > 0 && left == 0;
     if (*ended || done >= launched - kAhead) return RSD_OK;
@@ -844,6 +851,7 @@ int decode_phase(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t s) 
   bool ended = false;
   for (int j = 0; j < c->C && rc == RSD_OK && !ended; ++j) {
     const bool timed_iter = c->time_stride > 0 && (j % 16) == 5;
+    if (j == c->fail_at) CU(cudaMemsetAsync((char*)c->gemm_scratch + 4096, 0xFF, sizeof(int32_t), s));
     // the first iteration ever runs kernel by kernel (it also sets every kernel's attributes), then
     // the iteration is captured once and replayed
     const bool have_graph = graphs && c->dec_graph[g] && c->dec_graph_B[g] == c->st.B;
@@ -1419,6 +1427,12 @@ int rsd_debug_gemm_timing(rsd_ctx* c, int32_t stride, double* ms, double* bytes,
     c->ev_flops.assign(pairs, 0.0);
   }
   c->time_stride = stride;
+  return RSD_OK;
+}
+
+int rsd_debug_fail_iteration(rsd_ctx* c, int32_t iteration) {
+  if (!c || iteration < -1) return RSD_ERR_ARG;
+  c->fail_at = iteration;
   return RSD_OK;
 }
 

@@ -241,8 +241,9 @@ decode_update_kernel(RowState st, int which, int phase, unsigned long long* best
     const int left = st.n_active[0] - n_ended;
     st.n_active[0] = left;
     st.iter[0] = iter + 1;
-    // the host follows the phase through this word of its own memory: (iterations done, rows left)
-    *(volatile unsigned long long*)st.progress = ((unsigned long long)(iter + 1) << 32) | (unsigned)left;
+    // the host follows the phase through this word of its own memory: (an error was raised, iterations done, rows left)
+    const unsigned long long failed = ld_cg(st.wait_err) != 0 || ld_cg(st.err) != 0;
+    *(volatile unsigned long long*)st.progress = (failed << 63) | ((unsigned long long)(iter + 1) << 32) | (unsigned)left;
   }
 }
 

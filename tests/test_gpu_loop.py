@@ -466,3 +466,33 @@ def test_decode_attention_that_takes_the_qkv_product(d, H, KV, hd, ext):
         parity_step(eng, loop, 2.0, stats=stats, **TOL16)      # every row is rejected: draft and target decode
     assert stats["tokens_compared"] > 0.5 * stats["tokens"]
     eng.close()
+
+
+def _engine(prompts, **kw):
+    from paper_2501_19324_b200 import Engine, Model
+    heads = (ri.HEAD_LM, ri.HEAD_REWARD_SIGMOID, ri.HEAD_LM)
+    eng = Engine(*[Model(sh, ri.gpu_model_tensors(sh, slot, 0, True, hk), hk) for slot, (sh, hk) in enumerate(zip(MINI, heads))],
+                 max_batch=len(prompts[1]) - 1, **kw)
+    eng.prefill(*prompts)
+    return eng
+
+
+def test_a_failing_decode_phase_ends_early():
+    """The error flag of an expired wait, raised ahead of the fourth of 64 iterations: the call reports it after a few iterations
+    more, not after the whole phase, and the context refuses further work."""
+    from paper_2501_19324_b200.binding import RsdError, lib
+    prompts = ri.prompts(1, 3, 10, 20, MINI[0].vocab)
+    eng = _engine(prompts, max_seq_tokens=160, max_step_tokens=64, max_steps=3, step_end_id=-1, temperature=0.7, seed=1)
+    before = lib().rsd_debug_launch_count()
+    eng.step(0.0)                                       # 64 draft iterations, the target has nothing to do
+    whole = lib().rsd_debug_launch_count() - before
+    assert lib().rsd_debug_fail_iteration(eng.ctx, 3) == 0
+    before = lib().rsd_debug_launch_count()
+    with pytest.raises(RsdError) as e:
+        eng.step(0.0)
+    assert e.value.code == -5
+    assert lib().rsd_debug_launch_count() - before < whole / 4
+    with pytest.raises(RsdError) as e:
+        eng.step(0.0)
+    assert e.value.code == -2
+    eng.close()
