@@ -818,13 +818,13 @@ int follow_phase(rsd_ctx* c, int launched, cudaStream_t s, bool* ended) {
       Scalars sc;
       return read_scalars(c, s, &sc);
     }
-    const int done = (int)(w >> 32), left = (int)(w & 0xFFFFFFFFull);
-    *ended = done > 0 && left == 0;
+    const int done = (int)(w >> 32) - 1, left = (int)(w & 0xFFFFFFFFull);      // -1: the phase has not begun
+    *ended = done >= 0 && left == 0;
     if (*ended || done >= launched - kAhead) return RSD_OK;
     if ((polls & 0xFFFF) == 0) {
-      // a failed kernel never moves the word, and a phase without rows to decode leaves it alone
+      // a failed kernel never moves the word
       const cudaError_t e = cudaStreamQuery(s);
-      if (e == cudaSuccess) { *ended = (int)(*word >> 32) < launched || (*word & 0xFFFFFFFFull) == 0; return RSD_OK; }
+      if (e == cudaSuccess) { *ended = (int)(*word >> 32) - 1 < launched || (*word & 0xFFFFFFFFull) == 0; return RSD_OK; }
       if (e != cudaErrorNotReady) CU(e);
     }
   }
@@ -832,6 +832,7 @@ int follow_phase(rsd_ctx* c, int launched, cudaStream_t s, bool* ended) {
 
 // One decode phase: up to C iterations, fewer when every row ends before.
 int decode_phase(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t s) {
+  *c->progress = 0;            // the stream was synchronised since the last phase: no kernel that writes the word is in flight
   CU(launch_decode_begin(c->st, phase, s));
   if (n_slots <= 0) return RSD_OK;
   const bool graphs = !(c->cfg.debug_flags & RSD_DEBUG_NO_GRAPHS);
@@ -846,7 +847,6 @@ int decode_phase(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t s) 
   if (c->mega_B[which] == c->st.B) n_slots = c->st.B;
   else if (graphs) n_slots = rows_eff;
   c->in_decode = true;
-  *c->progress = 0;            // the stream was synchronised before the phase: no update kernel is in flight
   int rc = RSD_OK;
   bool ended = false;
   for (int j = 0; j < c->C && rc == RSD_OK && !ended; ++j) {

@@ -224,7 +224,7 @@ struct RowState {
   int32_t *n_live;             // live rows, counted by the gate
   int32_t *slot_row, *n_slots; // decode slots of the current phase
   int32_t *iter;               // iteration counter of the current decode phase
-  unsigned long long* progress;  // word of pinned host memory: error flag << 63 | iterations done << 32 | rows still decoding
+  unsigned long long* progress;  // word of pinned host memory: error flag << 63 | (1 + iterations done) << 32 | rows still decoding; 0: not begun
   const int32_t *wait_err;     // flag of the tensor-core kernels: a bounded wait has expired
   int32_t *last_idx;           // [B] flat index of each row's last token in the current pass
   int32_t *prev_idx;           // [B] PRM scoring pass: flat index of the row's last COMMITTED token when the pass

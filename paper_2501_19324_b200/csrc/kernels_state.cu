@@ -138,7 +138,10 @@ __global__ void __launch_bounds__(1024) decode_begin_kernel(RowState st, int pha
   }
   int total;
   block_exclusive_scan(part, scan, &total);
-  if (b == 0) { st.n_active[0] = total; st.iter[0] = 0; st.sd_stats[3] = 0; st.sd_stats[4] = 0; }
+  if (b == 0) {
+    st.n_active[0] = total; st.iter[0] = 0; st.sd_stats[3] = 0; st.sd_stats[4] = 0;
+    *(volatile unsigned long long*)st.progress = (1ull << 32) | (unsigned)total;   // begun, no iteration done (decode_update_kernel)
+  }
   const int n_slots = phase == 0 ? st.B : st.n_rej[0];
   if (b == 0) st.n_slots[0] = n_slots;
   if (b < st.B) st.slot_row[b] = phase == 0 ? b : (b < n_slots ? st.rej_idx[b] : -1);
@@ -243,7 +246,7 @@ decode_update_kernel(RowState st, int which, int phase, unsigned long long* best
     st.iter[0] = iter + 1;
     // the host follows the phase through this word of its own memory: (an error was raised, iterations done, rows left)
     const unsigned long long failed = ld_cg(st.wait_err) != 0 || ld_cg(st.err) != 0;
-    *(volatile unsigned long long*)st.progress = (failed << 63) | ((unsigned long long)(iter + 1) << 32) | (unsigned)left;
+    *(volatile unsigned long long*)st.progress = (failed << 63) | ((unsigned long long)(iter + 2) << 32) | (unsigned)left;
   }
 }
 

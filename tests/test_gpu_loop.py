@@ -496,3 +496,39 @@ def test_a_failing_decode_phase_ends_early():
         eng.step(0.0)
     assert e.value.code == -2
     eng.close()
+
+
+def test_a_phase_without_rows_does_not_wait_for_the_stream():
+    """No row has room for a step: the call returns although another thread keeps the caller's stream busy (for three seconds
+    at most), since the phase says itself that it has nothing to decode."""
+    import threading
+    import time
+    import torch
+    prompts = ri.prompts(1, 3, 40, 40, MINI[0].vocab)
+    eng = _engine(prompts, max_seq_tokens=64, max_step_tokens=32, max_steps=3, step_end_id=-1, temperature=0.0)
+    assert not eng.step(0.0)["live"].any()
+    stream, stop = torch.cuda.Stream(), threading.Event()
+
+    def feed():
+        end = time.monotonic() + 3.0
+        with torch.cuda.stream(stream):
+            pending = []
+            while time.monotonic() < end and not stop.is_set():
+                torch.cuda._sleep(2000000)               # about a millisecond
+                pending.append(torch.cuda.Event())
+                pending[-1].record()
+                if len(pending) > 8:
+                    pending.pop(0).synchronize()
+    t = threading.Thread(target=feed)
+    t.start()
+    time.sleep(0.2)
+    t0 = time.monotonic()
+    with torch.cuda.stream(stream):
+        out = eng.step(0.0)
+    took = time.monotonic() - t0
+    stop.set()
+    t.join()
+    torch.cuda.synchronize()
+    assert not out["live"].any() and (out["step_len"] == 0).all()
+    assert took < 1.5, took
+    eng.close()
