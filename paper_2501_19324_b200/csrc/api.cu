@@ -6,7 +6,9 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <chrono>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "common.cuh"
@@ -109,6 +111,7 @@ struct rsd_ctx {
   int sd_k = 0, slots_max = 0;
 
   int fail_at = -1;            // rsd_debug_fail_iteration
+  bool host_sleeps = false, host_yields = false;   // how this process waits for the device (cudaGetDeviceFlags)
   unsigned long long* progress = nullptr;   // pinned: how far the running decode phase is (RowState::progress)
   int pass_width = 1;          // consecutive positions of a row that a decode pass writes (a speculative round: sd_k)
   int attn_rows_hint = 0;      // rows expected to be active in the running decode phase (0: all slots)
@@ -803,14 +806,26 @@ int ensure_decode_graph(rsd_ctx* c, IterKind kind, int which, int phase, int g, 
   return RSD_OK;
 }
 
+// Tells the core that it is polling.
+inline void cpu_pause() {
+#if defined(__x86_64__)
+  __builtin_ia32_pause();
+#elif defined(__aarch64__)
+  asm volatile("yield");
+#endif
+}
+
 // Waits until all but kAhead of the `launched` iterations of the running decode phase are done, as the update kernel
 // notes in pinned host memory; *ended becomes true once no row is left.  Nothing is enqueued and the stream does not
 // drain: the device always has kAhead iterations before it, and at most so many are launched in vain after the last row
 // has ended (an idle iteration of a 28-layer model costs about 0.2 ms; looking once in 16 iterations, by a copy and a
-// synchronisation, left eight of them in vain on average: 4 steps of one question 8 % longer).
+// synchronisation, left eight of them in vain on average: 4 steps of one question 8 % longer).  How the thread waits is the
+// process's choice, as in a synchronisation: it sleeps between polls where blocking synchronisation was asked for
+// (cudaDeviceScheduleBlockingSync), and gives way to other threads now and then otherwise.
 int follow_phase(rsd_ctx* c, int launched, cudaStream_t s, bool* ended) {
   constexpr int kAhead = 2;
   volatile unsigned long long* word = c->progress;
+  const uint32_t query_every = c->host_sleeps ? 256 : 65536, yield_every = c->host_yields ? 1 : 1024;
   for (uint32_t polls = 1;; ++polls) {
     const unsigned long long w = *word;
     if (w >> 63) {
@@ -821,17 +836,24 @@ int follow_phase(rsd_ctx* c, int launched, cudaStream_t s, bool* ended) {
     const int done = (int)(w >> 32) - 1, left = (int)(w & 0xFFFFFFFFull);      // -1: the phase has not begun
     *ended = done >= 0 && left == 0;
     if (*ended || done >= launched - kAhead) return RSD_OK;
-    if ((polls & 0xFFFF) == 0) {
+    if (polls % query_every == 0) {
       // a failed kernel never moves the word
       const cudaError_t e = cudaStreamQuery(s);
       if (e == cudaSuccess) { *ended = (int)(*word >> 32) - 1 < launched || (*word & 0xFFFFFFFFull) == 0; return RSD_OK; }
       if (e != cudaErrorNotReady) CU(e);
     }
+    if (c->host_sleeps) std::this_thread::sleep_for(std::chrono::microseconds(20));
+    else if (polls % yield_every == 0) std::this_thread::yield();
+    else cpu_pause();
   }
 }
 
 // One decode phase: up to C iterations, fewer when every row ends before.
 int decode_phase(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t s) {
+  unsigned flags = 0;
+  if (cudaGetDeviceFlags(&flags) != cudaSuccess) { flags = 0; (void)cudaGetLastError(); }
+  c->host_sleeps = (flags & cudaDeviceScheduleMask) == cudaDeviceScheduleBlockingSync;
+  c->host_yields = (flags & cudaDeviceScheduleMask) == cudaDeviceScheduleYield;
   *c->progress = 0;            // the stream was synchronised since the last phase: no kernel that writes the word is in flight
   CU(launch_decode_begin(c->st, phase, s));
   if (n_slots <= 0) return RSD_OK;

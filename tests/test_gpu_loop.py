@@ -532,3 +532,35 @@ def test_a_phase_without_rows_does_not_wait_for_the_stream():
     assert not out["live"].any() and (out["step_len"] == 0).all()
     assert took < 1.5, took
     eng.close()
+
+
+_BLOCKING = """
+import ctypes, os, sys, time
+sys.path[:0] = [{root!r}, os.path.join({root!r}, "tests")]
+cuda = ctypes.CDLL("libcuda.so.1")
+assert cuda.cuInit(0) == 0
+if {blocking}:
+    assert cuda.cuDevicePrimaryCtxSetFlags(0, 4) == 0            # CU_CTX_SCHED_BLOCKING_SYNC, this process only
+import rsd_inputs as ri
+from test_gpu_loop import MINI, _engine
+eng = _engine(ri.prompts(1, 32, 40, 60, MINI[0].vocab), max_seq_tokens=600, max_step_tokens=120, max_steps=5, step_end_id=-1, temperature=0.7)
+eng.step(0.0)
+cpu, wall = time.thread_time(), time.perf_counter()
+for _ in range(2):
+    eng.step(0.0)
+print("SHARE", (time.thread_time() - cpu) / (time.perf_counter() - wall))
+"""
+
+
+def test_a_blocking_process_sleeps_through_a_decode_phase():
+    """A process that asked for blocking synchronisation has its thread asleep for much of a step; by default it polls."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    share = {}
+    for blocking in (True, False):
+        r = subprocess.run([sys.executable, "-c", _BLOCKING.format(root=root, blocking=blocking)], capture_output=True, text=True, timeout=240)
+        assert r.returncode == 0, r.stderr[-2000:]
+        share[blocking] = float(r.stdout.split("SHARE")[1])
+    assert share[True] < 0.7 and share[True] < share[False], share
