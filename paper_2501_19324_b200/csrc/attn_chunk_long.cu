@@ -356,7 +356,8 @@ attn_chunk_long_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
 template <typename OT, bool PROBE = false>
 cudaError_t launch_long(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const float* q, PassView p, KvView kv, void* out, void* out_lo,
                         int H, int KV, int* err, cudaStream_t s) {
-  static const cudaError_t set = cudaFuncSetAttribute(attn_chunk_long_kernel<OT, PROBE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+  static OncePerDevice configured;
+  const cudaError_t set = allow_smem(configured, attn_chunk_long_kernel<OT, PROBE>, kSmemBytes);
   if (set != cudaSuccess) return set;
   const int QT = 128 / (H / KV);
   RSD_LAUNCH((attn_chunk_long_kernel<OT, PROBE>), dim3((p.T + 2 * QT - 1) / (2 * QT), KV), kThreads, kSmemBytes, s, tm_k, tm_v, q, p,

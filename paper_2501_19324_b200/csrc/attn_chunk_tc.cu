@@ -457,32 +457,19 @@ cudaError_t launch_attn_chunk_tc(const float* q, PassView p, KvView kv, void* ou
   dim3 grid((p.T + QT - 1) / QT, KV);
   CUtensorMap tm_k, tm_v;
   if (!tc_tensor_map_kv(kv.pool_layer, 0, &tm_k) || !tc_tensor_map_kv(kv.pool_layer, 1, &tm_v)) return cudaErrorInvalidValue;
-  static bool configured[3] = {false, false, false};
-  if (out_dtype == 2) {      // one fp16 operand (out_lo unused)
-    if (!configured[2]) {
-      cudaError_t e = cudaFuncSetAttribute(attn_chunk_tc_kernel<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-      if (e != cudaSuccess) return e;
-      configured[2] = true;
-    }
-    RSD_LAUNCH((attn_chunk_tc_kernel<__half>), grid, kThreads, kSmemBytes, s, tm_k, tm_v, q, p, (const __half*)kv.pool_layer,
-               kv.page_table, kv.max_pages, (__half*)out, (__half*)nullptr, H, KV, QT, err);
-  } else if (out_dtype == 1) {
-    if (!configured[1]) {
-      cudaError_t e = cudaFuncSetAttribute(attn_chunk_tc_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-      if (e != cudaSuccess) return e;
-      configured[1] = true;
-    }
-    RSD_LAUNCH((attn_chunk_tc_kernel<__nv_bfloat16>), grid, kThreads, kSmemBytes, s, tm_k, tm_v, q, p, (const __half*)kv.pool_layer,
-               kv.page_table, kv.max_pages, (__nv_bfloat16*)out, (__nv_bfloat16*)out_lo, H, KV, QT, err);
-  } else {
-    if (!configured[0]) {
-      cudaError_t e = cudaFuncSetAttribute(attn_chunk_tc_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-      if (e != cudaSuccess) return e;
-      configured[0] = true;
-    }
-    RSD_LAUNCH((attn_chunk_tc_kernel<float>), grid, kThreads, kSmemBytes, s, tm_k, tm_v, q, p, (const __half*)kv.pool_layer,
-               kv.page_table, kv.max_pages, (float*)out, (float*)nullptr, H, KV, QT, err);
-  }
+  // out_dtype 2: one fp16 operand (out_lo unused)
+#define RSD_CHUNK(OT, lo)                                                                                              \
+  do {                                                                                                               \
+    static OncePerDevice configured;                                                                                 \
+    const cudaError_t set = allow_smem(configured, attn_chunk_tc_kernel<OT>, kSmemBytes);                            \
+    if (set != cudaSuccess) return set;                                                                              \
+    RSD_LAUNCH((attn_chunk_tc_kernel<OT>), grid, kThreads, kSmemBytes, s, tm_k, tm_v, q, p, (const __half*)kv.pool_layer, kv.page_table, \
+               kv.max_pages, (OT*)out, (OT*)(lo), H, KV, QT, err);                                                   \
+  } while (0)
+  if (out_dtype == 2) RSD_CHUNK(__half, nullptr);
+  else if (out_dtype == 1) RSD_CHUNK(__nv_bfloat16, out_lo);
+  else RSD_CHUNK(float, nullptr);
+#undef RSD_CHUNK
   return launched(1);
 }
 
@@ -491,8 +478,8 @@ cudaError_t launch_attn_wait_probe(bool one_pass, const float* q, PassView p, Kv
   if (one_pass) return launch_attn_chunk_long(q, p, kv, out, nullptr, 0, 8, 1, err, s, true);
   CUtensorMap tm_k, tm_v;
   if (!tc_tensor_map_kv(kv.pool_layer, 0, &tm_k) || !tc_tensor_map_kv(kv.pool_layer, 1, &tm_v)) return cudaErrorInvalidValue;
-  static const cudaError_t set =
-      cudaFuncSetAttribute(attn_chunk_tc_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+  static OncePerDevice configured;
+  const cudaError_t set = allow_smem(configured, attn_chunk_tc_kernel<float, true>, kSmemBytes);
   if (set != cudaSuccess) return set;
   RSD_LAUNCH((attn_chunk_tc_kernel<float, true>), dim3(1, 1), kThreads, kSmemBytes, s, tm_k, tm_v, q, p, (const __half*)kv.pool_layer,
              kv.page_table, kv.max_pages, out, (float*)nullptr, 8, 1, 16, err);

@@ -566,8 +566,8 @@ cudaError_t launch_attn_decode(int kv_dtype, const float* q, const void* pool_la
   dim3 grid(KV, B, splits);
 #define RSD_DEC_K(HD, KT, OT, EXTV, CLV, FUSEV)                                                                        \
   do {                                                                                                               \
-    static const cudaError_t set_ = cudaFuncSetAttribute(attn_decode_kernel<HD, KT, OT, EXTV, CLV, FUSEV>,           \
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, DecCfg<HD, EXTV>::kRingBytes); \
+    static OncePerDevice configured_;                                                                                \
+    const cudaError_t set_ = allow_smem(configured_, attn_decode_kernel<HD, KT, OT, EXTV, CLV, FUSEV>, DecCfg<HD, EXTV>::kRingBytes); \
     if (set_ != cudaSuccess) return set_;                                                                            \
     (void)launch_decode(attn_decode_kernel<HD, KT, OT, EXTV, CLV, FUSEV>, grid, clustered ? splits : 1, DecCfg<HD, EXTV>::kRingBytes, s, \
                         FUSEV ? qkv->qkv : q, (KT*)pool_layer, page_table, max_pages, slot_row, len_or_pos, len_offset, (OT*)out, \

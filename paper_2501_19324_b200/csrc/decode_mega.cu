@@ -893,7 +893,6 @@ Geometry geometry(int B) {
 }
 
 int g_sm_count = 0;
-size_t g_smem_set[2] = {0, 0};
 
 }  // namespace
 
@@ -978,12 +977,10 @@ cudaError_t launch_decode_mega(const void* dev_block, int B, int kv_extended, Pa
   if (n_ctas <= 0) return cudaErrorInvalidDevice;
   const size_t smem = geometry(B).smem;
   const int ext = kv_extended ? 1 : 0;
-  if (g_smem_set[ext] < smem) {
-    cudaError_t e = ext ? cudaFuncSetAttribute(decode_mega_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                        : cudaFuncSetAttribute(decode_mega_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    g_smem_set[ext] = smem;
-  }
+  // on every launch: the size depends on the batch, and the attribute belongs to the current device
+  const cudaError_t set = ext ? cudaFuncSetAttribute(decode_mega_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                              : cudaFuncSetAttribute(decode_mega_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (set != cudaSuccess) return set;
   const MegaParams* P = reinterpret_cast<const MegaParams*>(dev_block);
   const MegaLayer* Ls = reinterpret_cast<const MegaLayer*>((const uint8_t*)dev_block + sizeof(MegaParams));
   if (ext) RSD_LAUNCH((decode_mega_kernel<true>), n_ctas, kThreads, smem, s, P, Ls, p, (const __nv_bfloat16*)final_gain);

@@ -961,12 +961,9 @@ cudaError_t launch_mt(const CUtensorMap& tw, const CUtensorMap& tx, const CUtens
                       int accumulate, const TcPlan& p, float* partials, int* err, const int32_t* n_active,
                       bool defer_reduce, RowScale rs, cudaStream_t s, int f16 = 0) {
   using Cfg = TcCfg<MT, DEEP>;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<MT, SPLIT, false, DEEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static OncePerDevice configured;
+  const cudaError_t set = allow_smem(configured, gemm_tc_kernel<MT, SPLIT, false, DEEP>, Cfg::kSmemBytes);
+  if (set != cudaSuccess) return set;
   dim3 grid(p.n_tiles, p.m_tiles, p.splits);
   RSD_LAUNCH((gemm_tc_kernel<MT, SPLIT, false, DEEP>), grid, kTcThreads, Cfg::kSmemBytes, s, tw, tx, txl, y, M, N, K, accumulate, p.splits,
                                                                      p.kb_per_split, partials, err, n_active, rs,
@@ -1036,13 +1033,9 @@ cudaError_t launch_gemm_wait_probe(const void* W, const void* x, float* y, void*
   if (!scratch || scratch_bytes < gemm_scratch_bytes(16)) return cudaErrorInvalidValue;
   CUtensorMap tw, tx;
   if (!get_map(W, 128, 64, kTileN, &tw) || !get_map(x, 16, 64, 16, &tx)) return cudaErrorNotSupported;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<16, false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)TcCfg<16>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static OncePerDevice configured;
+  const cudaError_t set = allow_smem(configured, gemm_tc_kernel<16, false, false, false, true>, TcCfg<16>::kSmemBytes);
+  if (set != cudaSuccess) return set;
   int* err = (int*)((char*)scratch + kCounterBytes);
   float* partials = (float*)((char*)scratch + kCounterBytes + 256);
   RSD_LAUNCH((gemm_tc_kernel<16, false, false, false, true>), dim3(1, 1, 1), kTcThreads, TcCfg<16>::kSmemBytes, s, tw, tx, tx, y, 16, 128, 64, 0, 1, 1,
@@ -1070,12 +1063,9 @@ static cudaError_t launch_persistent(const CUtensorMap& tw, const CUtensorMap& t
                                      int f16 = 0, const int32_t* n_active = nullptr, RowScale rs = RowScale()) {
   using C = PersistCfg<SPLIT, GU>;
   constexpr size_t smem = C::kSmemBytes;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_persistent_kernel<GU, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static OncePerDevice configured;
+  const cudaError_t set = allow_smem(configured, gemm_tc_persistent_kernel<GU, SPLIT>, smem);
+  if (set != cudaSuccess) return set;
   const int n_sm = sm_count();
   if (n_sm <= 0) return cudaErrorInvalidDevice;
   const int tiles_n = GU ? N / 64 : (N + kTileN - 1) / kTileN, tiles_m = (M + C::kRows - 1) / C::kRows;
@@ -1104,10 +1094,10 @@ static cudaError_t launch_pair(const CUtensorMap& tw, const CUtensorMap& tx, con
                                int accumulate, int* err, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, cudaStream_t s, int f16) {
   using C = PairCfg<SPLIT, GU>;
   constexpr size_t smem = C::kSmemBytes;
-  static const int pairs = [] {
-    if (cudaFuncSetAttribute(gemm_tc_pair_kernel<GU, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
-    return max_pairs<GU, SPLIT>(smem);
-  }();
+  static OncePerDevice configured;
+  const cudaError_t set = allow_smem(configured, gemm_tc_pair_kernel<GU, SPLIT>, smem);
+  if (set != cudaSuccess) return set;
+  static const int pairs = max_pairs<GU, SPLIT>(smem);
   if (pairs <= 0) return cudaErrorNotSupported;
   const int feat = GU ? kTileN : 2 * kTileN, tiles_n = (N + feat - 1) / feat, tiles_m = (M + C::P::kRows - 1) / C::P::kRows;
   cudaLaunchConfig_t cfg = {};
@@ -1173,12 +1163,9 @@ static cudaError_t launch_gu_mt(const CUtensorMap& tw, const CUtensorMap& tx, co
                                 int* err, const int32_t* n_active, RowScale rs, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo,
                                 cudaStream_t s) {
   constexpr size_t smem = TcCfg<MT, DEEP>::kSmemBytes;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<MT, true, true, DEEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static OncePerDevice configured;
+  const cudaError_t set = allow_smem(configured, gemm_tc_kernel<MT, true, true, DEEP>, smem);
+  if (set != cudaSuccess) return set;
   const int total_kb = (K + kTileK - 1) / kTileK;
   dim3 grid(F / 64, (M + rows - 1) / rows, 1);
   RSD_LAUNCH((gemm_tc_kernel<MT, true, true, DEEP>), grid, kTcThreads, smem, s, tw, tx, txl, (float*)nullptr, M, F, K, 0, 1, total_kb,
