@@ -554,7 +554,7 @@ int forward_pass(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
 // Decode pass of a bf16 model with RMSNorm folded into its neighbours: the kernel that completes the
 // residual stream (reduce_norm) also writes the next GEMM's operand x * gain and the sums of squares, and
 // that GEMM scales its result rows by the RMSNorm denominator; the K-split sums of the qkv product are
-// added up by the RoPE kernel.  Ten kernels per layer instead of thirteen.  On return h / h_lo hold
+// added up by the RoPE kernel.  Eight kernels a layer, seven where the attention rotates for itself.  On return h / h_lo hold
 // x * final_gain and norm_ssq the sums of squares of the final residual stream.
 bool fused_decode_ok(const ModelHost& M) { return M.m.dtype == RSD_BF16 && M.split && M.m.d_model % 4 == 0; }
 

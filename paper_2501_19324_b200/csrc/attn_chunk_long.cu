@@ -16,7 +16,7 @@
 //
 // What bounds it: the exponentials (128 x 128 per tile and key tile take 1024 cycles of an SM's 16 per cycle) and the MMAs
 // (1024 cycles per query tile and key tile) are about even.  The older kernel (attn_chunk_tc.cu) walks the keys twice in
-// tiles of 64 and hands every tile through five roles; it stays for short passes, see attn_chunk_long_pays.  One row of 4096
+// tiles of 64 and hands every tile through five roles; it stays for short passes and few CTAs, see attn_chunk_long_pays.  One row of 4096
 // tokens over a prefix of 4000, 28 / 4 heads: 935 us (380 TFLOP/s algorithmic) there, 426 us (833) here; 16 rows of 256
 // over 3072: 627 us, 379 us.
 //

@@ -942,8 +942,9 @@ TcPlan plan_tc(int M, int N, int K, bool split_operand) {
   if (tiles < 148 && tiles <= kMaxSplitTiles && N % 4 == 0 && (p.rows <= 64 || (split_operand && M <= 128))) {
     // aim at one wave, each CTA with at least two k-blocks: of two CTAs per SM where the partial sums are small, of one where
     // pairs of more than 16 rows make them larger than what a second CTA saves (an iteration of 14 layers, 1.5B / 7B shapes:
-    // 32 rows 726 / 1661 us with two, 710 / 1641 with one; 64 rows 905 / 1942 and 872 / 1900).  Plain rows keep two: the
-    // order of their sums shows in bf16 activations.
+    // 32 rows 726 / 1661 us with two, 710 / 1641 with one; 64 rows 905 / 1942 and 872 / 1900).  Plain rows (in the step
+    // loop: short passes of the PRM) keep two: neither is better throughout (two / one, the reduction included: 32 x 1536 x 8960
+    // 8.3 / 7.1 us, 32 x 4608 x 3584 7.0 / 7.1, 64 x 3584 x 18944 28.1 / 30.3).
     // 65 to 128 rows with pairs are the decode passes of large batches: without the split the 12 tiles of a
     // 1536 x 8960 product leave 136 SMs idle (58 us at 128 rows; 11 us with 12 splits).
     splits = std::max(1, (p.rows <= 16 || !split_operand ? 2 * 148 : 148) / tiles);
@@ -1125,11 +1126,11 @@ static bool pair_pays(int M, int n_features, int K, int feat, int rows, bool add
 
 // Rows of x per tile for a dense product with one operand (bf16 or fp16): 256, or 128 or 64 while the tiles of the larger
 // size leave half of the SMs (of 256) or some (of 128) without one.  Every size sums along K in the same order: the
-// results are the same bits.  us at 256 / at the size taken, adding into y: 455 x 2048 x 1536 27.6 / 20.5 (64), 1000 x 1536 x 1536
-// 28.7 / 22.5 (64); 1000 x 3584 x 3584, 112 tiles of 256: 42 / 43.6 (128), kept at 256.  Adding at a short K the epilogue is
-// most of a tile and one wave of 256-row tiles hides none of it, while two CTAs of 128 rows hide each other's: 2048 x 1536 x 1536,
-// 96 tiles, 28.7 / 24.6; 3000 x 1536 x 1536, 144 tiles, 30.7 / 26.6; from two waves on the persistent kernel does as well or
-// better (4096 x 1536 x 1536 43 / 43, 8192 x 1536 x 1536 57 / 64).
+// results are the same bits.  us with 256 / 128 / 64 rows, adding into y (fp16, graph replays, operands in L2): 455 x 2048 x 1536
+// 18.7 / 11.1 / 9.1, 1000 x 1536 x 1536 18.8 / 11.5 / 11.8, 1000 x 3584 x 3584, 112 tiles of 256, 30.3 / 29.9 / 39.5.  Adding at a short K
+// the epilogue is most of a tile and one wave of 256-row tiles hides none of it, while two CTAs of 128 rows hide each other's:
+// 2048 x 1536 x 1536, 96 tiles, 19.8 / 17.0 / 19.6; 3000 x 1536 x 1536, 144 tiles, 20.0 / 17.4 / 23.4; from two waves on the
+// persistent kernel does as well or better (4096 x 1536 x 1536 30.2 / 28.9 / 33.1, 8192 x 1536 x 1536 47.4 / 52.2 / 66.6).
 static int dense_rows(int M, int N, int K, bool adds) {
   const int n_tiles = (N + kTileN - 1) / kTileN;
   int rows = 256;

@@ -117,7 +117,7 @@ cudaError_t launch_attn_chunk(int kv_dtype, const float* q, PassView p, KvView k
 bool attn_chunk_tc_supported(int kv_dtype, int H, int KV, int hd, int T);
 cudaError_t launch_attn_chunk_tc(const float* q, PassView p, KvView kv, void* out, void* out_lo, int out_dtype, int H, int KV,
                                  int* err, cudaStream_t s);
-// ... its one-pass form for long chunks, which launch_attn_chunk_tc picks by the chunk's length.
+// ... its one-pass form for long chunks, which launch_attn_chunk_tc picks where it saves waves.
 cudaError_t launch_attn_chunk_long(const float* q, PassView p, KvView kv, void* out, void* out_lo, int out_dtype, int H, int KV,
                                    int* err, cudaStream_t s, bool probe = false);
 // The failure path of either: a launch over 16 entries of eight heads, one KV head, whose copies are never issued; *err becomes -5.
