@@ -44,6 +44,11 @@ constexpr int kCounterBytes = 4096;
 constexpr int kMaxSplitTiles = kCounterBytes / 4;
 constexpr int kMaxSplitCtas = 640;
 constexpr int kTcThreads = 224;    // four epilogue warps, weight producer, MMA issuer, x producer
+// Ring stages of the decode pass's products into a fresh array (qkv, lm head), and of gate/up tiles of up to 16 rows: enough to keep a
+// stream going, and small enough that CTAs of the products after them (of three head tiles) find room beside these on an SM and
+// have their first weights there when their turn comes.  14-layer iterations, us, full rings / these: 1.5B shape at 1 row 538 / 514, at 8
+// 577 / 546; 7B shape 1391 / 1336 and 1418 / 1370.  Rings cut to the k-blocks of a CTA throughout spread the CTAs badly (16 rows 600 / 628).
+constexpr int kLightStages = 4, kGuStages = 6;
 
 // DEEP: a ring of eight (six for 128-row x tiles) stages for one CTA per SM, for grids that do not reach two CTAs per SM anyway (a lone
 // CTA needs about twice the bytes in flight to keep its share of the HBM stream going).
@@ -51,17 +56,18 @@ template <int MT, bool DEEP = false> struct TcCfg {
   // tiles of up to 128 x-rows leave room for two CTAs per SM (one streams while the other starts
   // up or drains); the 256-row tile of the dense regime takes the SM alone
   static constexpr int kCtasPerSm = DEEP ? 1 : (MT <= 128 ? 2 : 1);
-  static constexpr int kStages = DEEP ? (MT <= 64 ? 8 : 6) : (MT <= 32 ? 5 : (MT == 64 ? 4 : (MT == 128 ? 3 : 4)));
+  static constexpr int kStages = DEEP ? (MT <= 64 ? 8 : 6) : (MT == 16 ? 6 : (MT == 32 ? 5 : (MT == 64 ? 4 : (MT == 128 ? 3 : 4))));
   static constexpr int kABytes = kTileN * kTileK * 2;
   static constexpr int kBBytes = MT * kTileK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
   static constexpr int kTmemCols = MT < 32 ? 32 : MT;
-  static constexpr size_t kSmemBytes = 1024 + (size_t)kStages * kStageBytes + 256 + 512;   // barriers, row scales
+  static constexpr size_t smem_bytes(int stages) { return 1024 + (size_t)stages * kStageBytes + 256 + 512; }   // barriers, row scales
+  static constexpr size_t kSmemBytes = smem_bytes(kStages);
   // gate/up mode: two exchange buffers [64 features][MT / 4 rows + 1] between the gate and the up warps; they
   // reuse the pipeline stages once the last MMA has read them
   static constexpr size_t kXchBytes = 2 * 64 * (size_t)(MT / 4 + 1) * 4;
   static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
-  static_assert(kXchBytes <= (size_t)kStages * kStageBytes, "exchange buffers must fit in the stage ring");
+  static_assert(kXchBytes <= (size_t)(kStages < kGuStages ? kStages : kGuStages) * kStageBytes, "exchange buffers must fit in the stage ring");
   // instruction descriptor: fp32 accumulate, bf16 A and B, both K-major, N = MT, M = 128
   static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(MT >> 3) << 17) | ((uint32_t)(kTileN >> 4) << 24);
 };
@@ -82,7 +88,7 @@ __global__ void __launch_bounds__(kTcThreads, TcCfg<MT, DEEP>::kCtasPerSm)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                const __grid_constant__ CUtensorMap tm_x_lo, float* Y,
                int M, int N, int K, int accumulate, int splits, int kb_per_split, float* partials,
-               int* err, const int32_t* n_active, RowScale rs,
+               int* err, const int32_t* n_active, RowScale rs, int n_stages,
                __nv_bfloat16* act_hi = nullptr, __nv_bfloat16* act_lo = nullptr, int f16 = 0) {
   // Programmatic dependent launch: the next kernel may be scheduled at once; this kernel sets itself
   // up and starts streaming its WEIGHT tiles (never written by any kernel) while its predecessors are
@@ -96,12 +102,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
   constexpr int kRows = SPLIT ? MT / 2 : MT;   // distinct x rows per tile
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = (uint64_t*)(smem + (size_t)Cfg::kStages * Cfg::kStageBytes);
-  uint64_t* empty = full + Cfg::kStages;
-  uint64_t* tmem_full = empty + Cfg::kStages;
+  uint64_t* full = (uint64_t*)(smem + (size_t)n_stages * Cfg::kStageBytes);
+  uint64_t* empty = full + n_stages;
+  uint64_t* tmem_full = empty + n_stages;
   uint32_t* tmem_slot = (uint32_t*)(tmem_full + 1);
   volatile uint32_t* flags = tmem_slot + 1;   // [0] abort
-  float* row_scale = (float*)(smem + (size_t)Cfg::kStages * Cfg::kStageBytes + 256);   // [kRows <= 128]
+  float* row_scale = (float*)(smem + (size_t)n_stages * Cfg::kStageBytes + 256);   // [kRows <= 128]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // Tile order.  CTAs start in the order of their linear index; with n fastest, the CTAs in flight together would
@@ -125,7 +131,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
   const int n_kb = kb1 - kb0;   // >= 1 by construction of the grid
 
   if (threadIdx.x == 128) {                    // the weight producer's first lane
-    for (int s = 0; s < Cfg::kStages; ++s) { mbar_init(&full[s], 2); mbar_init(&empty[s], 1); }
+    for (int s = 0; s < n_stages; ++s) { mbar_init(&full[s], 2); mbar_init(&empty[s], 1); }
     mbar_init(tmem_full, 1);
     flags[0] = 0; flags[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -144,7 +150,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
     // Two threads, since one pays 100+ cycles for every box it issues: the weight stream runs ahead under the wait for
     // the predecessors as far as the ring reaches, the x tiles follow after it.
     if (lane == 0 && !PROBE) {
-      const int pre = min(n_kb, Cfg::kStages);
+      const int pre = min(n_kb, n_stages);
       int n_issue = n_kb;
       if (warp == 4) {
         if (active == 0) n_issue = pre;
@@ -171,7 +177,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
           if (SPLIT) tma_load_2d(a + Cfg::kABytes + kRows * kTileK * 2, &tm_x_lo, &full[s], (kb0 + i) * kTileK, m0);
         }
         issued = i + 1;
-        if (++s == Cfg::kStages) { s = 0; phase ^= 1u; }
+        if (++s == n_stages) { s = 0; phase ^= 1u; }
         ready = mbar_test(&empty[s], phase);
       }
       if (active == 0) {
@@ -184,8 +190,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
         }
         // let the copies already in flight land before the CTA goes away (a stage that only one producer has reached
         // does not complete: the polls run out, long after the copy)
-        for (int i = max(0, issued - Cfg::kStages); i < issued; ++i)
-          mbar_wait(&full[i % Cfg::kStages], (i / Cfg::kStages) & 1, 1u << 16);
+        for (int i = max(0, issued - n_stages); i < issued; ++i)
+          mbar_wait(&full[i % n_stages], (i / n_stages) & 1, 1u << 16);
       }
     }
   } else if (warp == 5) {
@@ -205,7 +211,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
           if (!ok) break;
         }
         tc_fence_after();
-        const int s1 = s + 1 == Cfg::kStages ? 0 : s + 1;
+        const int s1 = s + 1 == n_stages ? 0 : s + 1;
         const uint32_t phase1 = s1 == 0 ? phase ^ 1u : phase;
         // a look ahead at the next stage under this one's MMAs: even when the data are there, a wait takes 127 cycles
         ready = __all_sync(0xFFFFFFFFu, i + 1 < n_kb && mbar_test(&full[s1], phase1));
@@ -266,7 +272,26 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
     if (GU) {
       // SwiGLU epilogue.  Rows [0, half) of the tile are finished by the gate warps (they receive the up values
       // of those rows), rows [half, kRows) by the up warps (they receive the gate values).
-      constexpr int kHalf = kRows / 2, kLd = kHalf + 1;
+      constexpr int kHalf = kRows / 2, kLd = kHalf + 1, kCols = kHalf < 16 ? kHalf : 16;   // rows at a time
+      // hi + lo of rows [at, at + kCols) of the tile
+      auto rows_of = [&](int at, float (&v)[kCols]) {
+        if (kRows == 8) {                                      // hi in columns 0..7, lo in columns 8..15 of the same load
+          float w[16];
+          tmem_ld16(taddr, w);
+#pragma unroll
+          for (int j = 0; j < kCols; ++j) v[j] = at == 0 ? w[j] + w[(j + 8) & 15] : w[(j + 4) & 15] + w[(j + 12) & 15];
+        } else if (kRows == 16) {
+          float w[2][16];
+          tmem_ld16n<2>({taddr, taddr + 16}, w);
+#pragma unroll
+          for (int j = 0; j < kCols; ++j) v[j] = at == 0 ? w[0][j] + w[1][j] : w[0][(j + 8) & 15] + w[1][(j + 8) & 15];
+        } else {
+          float w[2][16];
+          tmem_ld16n<2>({taddr + at, taddr + kRows + at}, w);
+#pragma unroll
+          for (int j = 0; j < kCols; ++j) v[j] = w[0][j & 15] + w[1][j & 15];
+        }
+      };
       const bool is_gate = warp < 2;
       const int l = (warp & 1) * 32 + lane;                    // feature within the 64-row half
       float* send = xch + (is_gate ? 64 * kLd : 0) + l * kLd;  // [0]: up values of the low rows, [1]: gate values of the high rows
@@ -274,33 +299,33 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
       const int send0 = is_gate ? kHalf : 0, own0 = is_gate ? 0 : kHalf;
       if (ok) {
 #pragma unroll 1
-        for (int c = 0; c < kHalf; c += 16) {
-          float v[2][16];
-          tmem_ld16n<2>({taddr + send0 + c, taddr + kRows + send0 + c}, v);
+        for (int c = 0; c < kHalf; c += kCols) {
+          float v[kCols];
+          rows_of(send0 + c, v);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) send[c + j] = v[0][j] + v[1][j];
+          for (int j = 0; j < kCols; ++j) send[c + j] = v[j];
         }
       }
       asm volatile("bar.sync 1, 128;" ::: "memory");
       if (ok && n0 + l < N) {
 #pragma unroll 1
-        for (int c = 0; c < kHalf; c += 16) {
+        for (int c = 0; c < kHalf; c += kCols) {
           if (own0 + c >= m_valid) break;
-          float v[2][16];
-          tmem_ld16n<2>({taddr + own0 + c, taddr + kRows + own0 + c}, v);
+          float v[kCols];
+          rows_of(own0 + c, v);
           // all sixteen, whether the row counts or not, and stores under predicates: a branch per row and a division per
           // element kept the elements from overlapping (32 rows: 4250 cycles behind the exchange, now 1760)
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
+          for (int j = 0; j < kCols; ++j) {
             const float sc = rs.ssq != nullptr ? row_scale[own0 + c + j] : 1.f;
-            const float mine = (v[0][j] + v[1][j]) * sc, other = recv[c + j] * sc;
-            v[0][j] = swiglu(is_gate ? mine : other, is_gate ? other : mine);
+            const float mine = v[j] * sc, other = recv[c + j] * sc;
+            v[j] = swiglu(is_gate ? mine : other, is_gate ? other : mine);
           }
           const size_t o = (size_t)(m0 + own0 + c) * N + n0 + l;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
+          for (int j = 0; j < kCols; ++j) {
             __nv_bfloat16 h, w;
-            store_operand<__nv_bfloat16>(&h, &w, 0, v[0][j]);
+            store_operand<__nv_bfloat16>(&h, &w, 0, v[j]);
             store_if(own0 + c + j < m_valid, act_hi + o + (size_t)j * N, h);
             store_if(own0 + c + j < m_valid, act_lo + o + (size_t)j * N, w);
           }
@@ -930,7 +955,8 @@ int pick_rows(int M, bool split_operand) {
 
 struct TcPlan { int rows, mt, n_tiles, m_tiles, splits, kb_per_split; };
 
-TcPlan plan_tc(int M, int N, int K, bool split_operand) {
+// few_sums: the consumer adds the splits up in a step of few, latency-bound loads (the rotation of a qkv product).
+TcPlan plan_tc(int M, int N, int K, bool split_operand, bool few_sums = false) {
   TcPlan p;
   p.rows = pick_rows(M, split_operand);
   p.mt = split_operand ? 2 * p.rows : p.rows;
@@ -948,7 +974,9 @@ TcPlan plan_tc(int M, int N, int K, bool split_operand) {
     // 65 to 128 rows with pairs are the decode passes of large batches: without the split the 12 tiles of a
     // 1536 x 8960 product leave 136 SMs idle (58 us at 128 rows; 11 us with 12 splits).
     splits = std::max(1, (p.rows <= 16 || !split_operand ? 2 * 148 : 148) / tiles);
-    splits = std::min(splits, std::max(1, total_kb / 2));
+    // fewer and longer splits for the rotation, as long as they occupy half of the SMs (16 tiles, 24 k-blocks, 1 row: 12 / 6
+    // splits 522 / 514 us an iteration of 14 layers; but 8 tiles, 8 k-blocks: 51.6 / 54.6 an iteration of 2 with four / two)
+    splits = std::min(splits, std::max(1, few_sums && tiles * (total_kb / 4) >= 74 ? total_kb / 4 : total_kb / 2));
     splits = std::min(splits, kMaxSplitCtas / tiles);
     splits = std::max(splits, 1);
   }
@@ -966,8 +994,9 @@ cudaError_t launch_mt(const CUtensorMap& tw, const CUtensorMap& tx, const CUtens
   const cudaError_t set = allow_smem(configured, gemm_tc_kernel<MT, SPLIT, false, DEEP>, Cfg::kSmemBytes);
   if (set != cudaSuccess) return set;
   dim3 grid(p.n_tiles, p.m_tiles, p.splits);
-  RSD_LAUNCH((gemm_tc_kernel<MT, SPLIT, false, DEEP>), grid, kTcThreads, Cfg::kSmemBytes, s, tw, tx, txl, y, M, N, K, accumulate, p.splits,
-                                                                     p.kb_per_split, partials, err, n_active, rs,
+  const int stages = !accumulate && rs.ssq != nullptr ? std::min(Cfg::kStages, kLightStages) : Cfg::kStages;
+  RSD_LAUNCH((gemm_tc_kernel<MT, SPLIT, false, DEEP>), grid, kTcThreads, Cfg::smem_bytes(stages), s, tw, tx, txl, y, M, N, K, accumulate, p.splits,
+                                                                     p.kb_per_split, partials, err, n_active, rs, stages,
                                                                      (__nv_bfloat16*)nullptr, (__nv_bfloat16*)nullptr, f16);
   if (p.splits > 1 && !defer_reduce) {
     const size_t total4 = (size_t)M * N / 4;
@@ -1040,7 +1069,7 @@ cudaError_t launch_gemm_wait_probe(const void* W, const void* x, float* y, void*
   int* err = (int*)((char*)scratch + kCounterBytes);
   float* partials = (float*)((char*)scratch + kCounterBytes + 256);
   RSD_LAUNCH((gemm_tc_kernel<16, false, false, false, true>), dim3(1, 1, 1), kTcThreads, TcCfg<16>::kSmemBytes, s, tw, tx, tx, y, 16, 128, 64, 0, 1, 1,
-             partials, err, (const int32_t*)nullptr, RowScale(), (__nv_bfloat16*)nullptr, (__nv_bfloat16*)nullptr, 0);
+             partials, err, (const int32_t*)nullptr, RowScale(), TcCfg<16>::kStages, (__nv_bfloat16*)nullptr, (__nv_bfloat16*)nullptr, 0);
   return launched(1);
 }
 
@@ -1163,14 +1192,15 @@ template <int MT, bool DEEP>
 static cudaError_t launch_gu_mt(const CUtensorMap& tw, const CUtensorMap& tx, const CUtensorMap& txl, int M, int F, int K, int rows,
                                 int* err, const int32_t* n_active, RowScale rs, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo,
                                 cudaStream_t s) {
-  constexpr size_t smem = TcCfg<MT, DEEP>::kSmemBytes;
   static OncePerDevice configured;
-  const cudaError_t set = allow_smem(configured, gemm_tc_kernel<MT, true, true, DEEP>, smem);
+  const cudaError_t set = allow_smem(configured, gemm_tc_kernel<MT, true, true, DEEP>, TcCfg<MT, DEEP>::kSmemBytes);
   if (set != cudaSuccess) return set;
   const int total_kb = (K + kTileK - 1) / kTileK;
+  const int stages = MT <= 32 ? std::min(TcCfg<MT, DEEP>::kStages, kGuStages) : TcCfg<MT, DEEP>::kStages;
+  const size_t smem = TcCfg<MT, DEEP>::smem_bytes(stages);
   dim3 grid(F / 64, (M + rows - 1) / rows, 1);
   RSD_LAUNCH((gemm_tc_kernel<MT, true, true, DEEP>), grid, kTcThreads, smem, s, tw, tx, txl, (float*)nullptr, M, F, K, 0, 1, total_kb,
-             (float*)nullptr, err, n_active, rs, act_hi, act_lo, 0);
+             (float*)nullptr, err, n_active, rs, stages, act_hi, act_lo, 0);
   return launched(1);
 }
 
@@ -1196,8 +1226,8 @@ cudaError_t launch_gemm_gu(const void* Wgu, const void* x, const void* x_lo, voi
     return launch_persistent<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act_hi, nullptr, s);
   }
   if (!act_lo) return cudaErrorNotSupported;
-  // at least 32 x rows per tile: each warp pair finishes one half of them, 16 at a time
-  const int rows = M <= 32 ? 32 : (M <= 64 ? 64 : 128);
+  // each warp pair finishes one half of the rows, up to 16 at a time
+  const int rows = M <= 8 ? 8 : (M <= 16 ? 16 : (M <= 32 ? 32 : (M <= 64 ? 64 : 128)));
   if (rs.ssq != nullptr && rows > 128) return cudaErrorInvalidValue;
   if (!get_map(Wgu, 2 * F, K, kTileN / 2, &tw) || !get_map(x, M, K, rows, &tx) || !get_map(x_lo, M, K, rows, &txl))
     return cudaErrorNotSupported;
@@ -1209,6 +1239,10 @@ cudaError_t launch_gemm_gu(const void* Wgu, const void* x, const void* x_lo, voi
   // fewer than ~1.5 CTAs per SM: one CTA per SM with a deep ring streams faster than a thin second wave
   const bool deep = (F / 64) * ((M + rows - 1) / rows) <= 222;
   switch (rows) {
+    case 8: return deep ? launch_gu_mt<16, true>(tw, tx, txl, M, F, K, rows, err, n_active, rs, hi, lo, s)
+                        : launch_gu_mt<16, false>(tw, tx, txl, M, F, K, rows, err, n_active, rs, hi, lo, s);
+    case 16: return deep ? launch_gu_mt<32, true>(tw, tx, txl, M, F, K, rows, err, n_active, rs, hi, lo, s)
+                         : launch_gu_mt<32, false>(tw, tx, txl, M, F, K, rows, err, n_active, rs, hi, lo, s);
     case 32: return deep ? launch_gu_mt<64, true>(tw, tx, txl, M, F, K, rows, err, n_active, rs, hi, lo, s)
                          : launch_gu_mt<64, false>(tw, tx, txl, M, F, K, rows, err, n_active, rs, hi, lo, s);
     case 64: return deep ? launch_gu_mt<128, true>(tw, tx, txl, M, F, K, rows, err, n_active, rs, hi, lo, s)
@@ -1239,7 +1273,7 @@ cudaError_t launch_gemm_tc(const void* W, const void* x, const void* x_lo, float
   if (!scratch || scratch_bytes < gemm_scratch_bytes(M)) return cudaErrorInvalidValue;
   if (((uintptr_t)W & 15) || ((uintptr_t)x & 15) || ((uintptr_t)x_lo & 15)) return cudaErrorMisalignedAddress;
   const bool split_operand = x_lo != nullptr;
-  TcPlan p = plan_tc(M, N, K, split_operand);
+  TcPlan p = plan_tc(M, N, K, split_operand, rs.ssq != nullptr && !accumulate);
   if (no_k_split) { p.splits = 1; p.kb_per_split = (K + kTileK - 1) / kTileK; }
   if (rs.ssq != nullptr && p.rows > 128) return cudaErrorInvalidValue;   // one epilogue thread per x row of the tile
   if (deferred_splits) *deferred_splits = p.splits;

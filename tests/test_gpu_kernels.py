@@ -678,6 +678,12 @@ def test_gate_up_gemm_with_swiglu_epilogue(M, F, K):
     assert torch.equal(again_hi, a_hi) and torch.equal(again_lo, a_lo)
 
 
+@pytest.mark.parametrize("M,F,K", [(2, 1408, 512), (8, 192, 520), (9, 128, 768), (16, 18944, 256), (17, 64, 520)])
+def test_gate_up_tiles_of_few_rows(M, F, K):
+    """Tiles of 8, 16 and 32 rows at their edges: full, one row into the next, one or two CTAs per SM; the bound of the test above."""
+    test_gate_up_gemm_with_swiglu_epilogue(M, F, K)
+
+
 @pytest.mark.parametrize("M,N,K", [(65, 128, 64), (65, 1536, 8960), (128, 640, 520), (96, 18816, 128), (65, 18945, 192), (128, 19072, 520)])
 def test_paired_gemm_of_65_to_128_rows(M, N, K):
     """The decode products of large batches: K split over the SMs (the smallest, a long K with many splits, a K tail), a
