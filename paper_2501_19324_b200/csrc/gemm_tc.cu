@@ -44,10 +44,11 @@ constexpr int kCounterBytes = 4096;
 constexpr int kMaxSplitTiles = kCounterBytes / 4;
 constexpr int kMaxSplitCtas = 640;
 constexpr int kTcThreads = 224;    // four epilogue warps, weight producer, MMA issuer, x producer
-// Ring stages of the decode pass's products into a fresh array (qkv, lm head), and of gate/up tiles of up to 16 rows: enough to keep a
+// Ring stages of the decode pass's products of up to 16 rows into a fresh array (qkv, lm head), and of such gate/up tiles: enough to keep a
 // stream going, and small enough that CTAs of the products after them (of three head tiles) find room beside these on an SM and
 // have their first weights there when their turn comes.  14-layer iterations, us, full rings / these: 1.5B shape at 1 row 538 / 514, at 8
-// 577 / 546; 7B shape 1391 / 1336 and 1418 / 1370.  Rings cut to the k-blocks of a CTA throughout spread the CTAs badly (16 rows 600 / 628).
+// 577 / 546; 7B shape 1391 / 1336 and 1418 / 1370.  Rings cut to the k-blocks of a CTA throughout spread the CTAs badly (16 rows 600 / 628); at 32 rows
+// light rings cost the 7B shape's qkv product 8.4 -> 9.8 us.
 constexpr int kLightStages = 4, kGuStages = 6;
 
 // DEEP: a ring of eight (six for 128-row x tiles) stages for one CTA per SM, for grids that do not reach two CTAs per SM anyway (a lone
@@ -976,7 +977,7 @@ TcPlan plan_tc(int M, int N, int K, bool split_operand, bool few_sums = false) {
     splits = std::max(1, (p.rows <= 16 || !split_operand ? 2 * 148 : 148) / tiles);
     // fewer and longer splits for the rotation, as long as they occupy half of the SMs (16 tiles, 24 k-blocks, 1 row: 12 / 6
     // splits 522 / 514 us an iteration of 14 layers; but 8 tiles, 8 k-blocks: 51.6 / 54.6 an iteration of 2 with four / two)
-    splits = std::min(splits, std::max(1, few_sums && tiles * (total_kb / 4) >= 74 ? total_kb / 4 : total_kb / 2));
+    splits = std::min(splits, std::max(1, few_sums && p.rows <= 16 && tiles * (total_kb / 4) >= 74 ? total_kb / 4 : total_kb / 2));
     splits = std::min(splits, kMaxSplitCtas / tiles);
     splits = std::max(splits, 1);
   }
@@ -994,7 +995,7 @@ cudaError_t launch_mt(const CUtensorMap& tw, const CUtensorMap& tx, const CUtens
   const cudaError_t set = allow_smem(configured, gemm_tc_kernel<MT, SPLIT, false, DEEP>, Cfg::kSmemBytes);
   if (set != cudaSuccess) return set;
   dim3 grid(p.n_tiles, p.m_tiles, p.splits);
-  const int stages = !accumulate && rs.ssq != nullptr ? std::min(Cfg::kStages, kLightStages) : Cfg::kStages;
+  const int stages = MT <= 32 && !accumulate && rs.ssq != nullptr ? std::min(Cfg::kStages, kLightStages) : Cfg::kStages;
   RSD_LAUNCH((gemm_tc_kernel<MT, SPLIT, false, DEEP>), grid, kTcThreads, Cfg::smem_bytes(stages), s, tw, tx, txl, y, M, N, K, accumulate, p.splits,
                                                                      p.kb_per_split, partials, err, n_active, rs, stages,
                                                                      (__nv_bfloat16*)nullptr, (__nv_bfloat16*)nullptr, f16);
