@@ -407,6 +407,12 @@ template <bool SPLIT, bool GU> struct PersistCfg {
   static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
 };
 
+// An instruction descriptor with n columns, and the operand formats fp16 where asked for.
+__device__ __forceinline__ uint32_t tile_idesc(uint32_t idesc, int n, int f16) {
+  idesc = (idesc & ~(0x3Fu << 17)) | ((uint32_t)(n >> 3) << 17);
+  return f16 ? idesc & ~((1u << 7) | (1u << 10)) : idesc;
+}
+
 // warps 0..7: epilogue, warp 8: TMA producer, warp 9: MMA issuer and owner of the tensor-memory allocation
 constexpr int kPersistEpiWarps = 8, kPersistThreads = 32 * (kPersistEpiWarps + 2);
 
@@ -416,10 +422,10 @@ constexpr int kPersistEpiWarps = 8, kPersistThreads = 32 * (kPersistEpiWarps + 2
 template <bool GU, bool SPLIT, typename Release>
 __device__ __forceinline__ void persist_epilogue(uint32_t taddr, bool ok, int quarter, int lane, int col0, int n0, int m0, int M, int N,
                                                  float* Y, int accumulate, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, int f16,
-                                                 float* xch, const float* row_scale, Release release) {
+                                                 float* xch, const float* row_scale, int rows, Release release) {
   using C = PersistCfg<SPLIT, GU>;
   constexpr int kColStep = 16 * (kPersistEpiWarps / 4);
-  const int m_valid = min(C::kRows, M - m0);
+  const int m_valid = min(rows, M - m0);
   auto ld = [&](int c, float (&v)[16]) {             // sixteen columns, the low halves' results added
     if (SPLIT) {
       float t[2][16];
@@ -464,10 +470,10 @@ __device__ __forceinline__ void persist_epilogue(uint32_t taddr, bool ok, int qu
     const int l = (quarter & 1) * 32 + lane;
     float* send = xch + (is_gate ? 64 * C::kLd : 0) + l * C::kLd;
     const float* recv = xch + (is_gate ? 0 : 64 * C::kLd) + l * C::kLd;
-    const int send0 = is_gate ? C::kHalf : 0, own0 = is_gate ? 0 : C::kHalf;
+    const int half = rows / 2, send0 = is_gate ? half : 0, own0 = is_gate ? 0 : half;
     if (ok) {
 #pragma unroll 1
-      for (int c = col0; c < C::kHalf; c += kColStep) {
+      for (int c = col0; c < half; c += kColStep) {
         float v[16];
         ld(send0 + c, v);
 #pragma unroll
@@ -477,7 +483,7 @@ __device__ __forceinline__ void persist_epilogue(uint32_t taddr, bool ok, int qu
     asm volatile("bar.sync 1, %0;" ::"n"(32 * kPersistEpiWarps) : "memory");
     if (ok && n0 + l < N) {
 #pragma unroll 1
-      for (int c = col0; c < C::kHalf; c += kColStep) {
+      for (int c = col0; c < half; c += kColStep) {
         if (own0 + c >= m_valid) break;
         float v[16];
         ld(own0 + c, v);
@@ -510,7 +516,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
 gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                           const __grid_constant__ CUtensorMap tm_x_lo, float* Y, int M, int N, int K,
                           int accumulate, int n_tiles_n, int n_tiles_m, int* err,
-                          __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, int f16, const int32_t* n_active, RowScale rs) {
+                          __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, int f16, const int32_t* n_active, RowScale rs, int tile_rows) {
   RSD_PDL_TRIGGER();
   if (n_active != nullptr && ld_cg(n_active) == 0) {      // every row of the decode phase has finished
     RSD_PDL_WAIT();
@@ -519,7 +525,9 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
   using C = PersistCfg<SPLIT, GU>;
   // f16: both operands are fp16 (weights re-encoded at load, one fp16 activation operand); the MMA's operand-format
   // fields become 0 and a gate/up tile writes its activations as fp16.  Otherwise bf16 throughout.
-  const uint32_t idesc = f16 ? (C::kIdesc & ~((1u << 7) | (1u << 10))) : C::kIdesc;
+  const int rows = SPLIT ? C::kRows : tile_rows;           // x rows of a tile: of plain operands the launch's choice
+  const uint32_t idesc = tile_idesc(C::kIdesc, SPLIT ? C::kMT : rows, f16);
+  const uint32_t stage_bytes = C::kABytes + (SPLIT ? C::kMT : rows) * kTileK * 2;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(smem + (size_t)C::kStages * C::kStageBytes);
@@ -558,7 +566,7 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
     bool ready = true;
     auto load_w = [&](uint32_t st, int kb, int n0) {
       uint8_t* a = smem + (size_t)st * C::kStageBytes;
-      mbar_expect_tx_if(on, &full[st], C::kStageBytes);
+      mbar_expect_tx_if(on, &full[st], stage_bytes);
       tma_load_2d_if(on, a, &tm_w, &full[st], kb * kTileK, n0);
       if (GU) tma_load_2d_if(on, a + C::kABytes / 2, &tm_w, &full[st], kb * kTileK, N + n0);
     };
@@ -574,7 +582,7 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
     for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
       int tm, tn;
       tile_of(t, tm, tn);
-      const int n0 = tn * (GU ? kTileN / 2 : kTileN), m0 = tm * C::kRows;
+      const int n0 = tn * (GU ? kTileN / 2 : kTileN), m0 = tm * rows;
       for (int kb = 0; kb < total_kb; ++kb, ++it) {
         if (it >= ahead) {
           if (!ready) {
@@ -652,7 +660,7 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
     for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++n_acc) {
       int tm, tn;
       tile_of(t, tm, tn);
-      const int n0 = tn * (GU ? kTileN / 2 : kTileN), m0 = tm * C::kRows;
+      const int n0 = tn * (GU ? kTileN / 2 : kTileN), m0 = tm * rows;
       const uint32_t b = n_acc & 1u;
       bool ok = mbar_try_wait(&acc_full[b], (n_acc >> 1) & 1u);
       for (uint32_t i = 0; i < (1u << 21) && !ok && !*stop; ++i) ok = mbar_try_wait_sleep(&acc_full[b], (n_acc >> 1) & 1u, 1000);
@@ -661,7 +669,7 @@ gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + b * (uint32_t)C::kMT;
       persist_epilogue<GU, SPLIT>(taddr, ok, quarter, lane, col0, n0, m0, M, N, Y, accumulate, act_hi, act_lo, f16, xch,
-                                  scaled ? row_scale : nullptr, [&]() { mbar_arrive(&acc_empty[b]); });
+                                  scaled ? row_scale : nullptr, rows, [&]() { mbar_arrive(&acc_empty[b]); });
     }
   }
   tc_fence_before();
@@ -699,11 +707,12 @@ template <bool GU, bool SPLIT>
 __global__ void __launch_bounds__(kPersistThreads, 1)
 gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                     const __grid_constant__ CUtensorMap tm_x_lo, float* Y, int M, int N, int K, int accumulate, int n_tiles_n,
-                    int n_tiles_m, int* err, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, int f16) {
+                    int n_tiles_m, int* err, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, int f16, int tile_rows) {
   RSD_PDL_TRIGGER();
   using C = PairCfg<SPLIT, GU>;
-  constexpr int kRows = C::P::kRows;
-  const uint32_t idesc = f16 ? (C::kIdesc & ~((1u << 7) | (1u << 10))) : C::kIdesc;
+  const int rows = SPLIT ? C::P::kRows : tile_rows;        // x rows of a tile: of plain operands the launch's choice
+  const int half = SPLIT ? 128 : rows / 2;                 // operand rows of one CTA
+  const uint32_t idesc = tile_idesc(C::kIdesc, 2 * half, f16), stage_bytes = C::kABytes + half * kTileK * 2;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(smem + (size_t)C::kStages * C::kStageBytes);
@@ -749,7 +758,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_const
     auto load_w = [&](uint32_t st, int kb, int n0) {
       uint8_t* a = smem + (size_t)st * C::kStageBytes;
       const uint32_t bar = cluster_addr(&full[st], 0);
-      mbar_expect_tx_if(lead, &full[st], 2 * C::kStageBytes);     // both CTAs' bytes
+      mbar_expect_tx_if(lead, &full[st], 2 * stage_bytes);        // both CTAs' bytes
       tma_load_2d_pair_if(on, a, &tm_w, bar, kb * kTileK, n0);
       if (GU) tma_load_2d_pair_if(on, a + C::kABytes / 2, &tm_w, bar, kb * kTileK, N + n0);
     };
@@ -763,7 +772,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_const
     for (int t = pair; t < n_tiles && ok; t += n_pairs) {
       int tm, tn;
       tile_of(t, tm, tn);
-      const int n0 = first_feature(tn), m0 = tm * kRows;
+      const int n0 = first_feature(tn), m0 = tm * rows;
       for (int kb = 0; kb < total_kb; ++kb, ++it) {
         if (it >= ahead) {
           if (!ready) {
@@ -776,7 +785,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_const
         uint8_t* b = smem + (size_t)s * C::kStageBytes + C::kABytes;
         const uint32_t bar = cluster_addr(&full[s], 0);
         if (SPLIT) tma_load_2d_pair_if(on, b, rank == 0 ? &tm_x : &tm_x_lo, bar, kb * kTileK, m0);
-        else tma_load_2d_pair_if(on, b, &tm_x, bar, kb * kTileK, m0 + (int)rank * 128);
+        else tma_load_2d_pair_if(on, b, &tm_x, bar, kb * kTileK, m0 + (int)rank * half);
         if (++s == (uint32_t)C::kStages) { s = 0; phase ^= 1u; }
         ready = __all_sync(0xFFFFFFFFu, mbar_test(&empty[s], phase));
       }
@@ -837,8 +846,8 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_const
       if (!ok) fail();
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + b * 256u;
-      persist_epilogue<GU, SPLIT>(taddr, ok, quarter, lane, col0, first_feature(tn), tm * kRows, M, N, Y, accumulate, act_hi, act_lo,
-                                  f16, xch, nullptr, [&]() { mbar_arrive_cluster(cluster_addr(&acc_empty[b], 0)); });
+      persist_epilogue<GU, SPLIT>(taddr, ok, quarter, lane, col0, first_feature(tn), tm * rows, M, N, Y, accumulate, act_hi, act_lo,
+                                  f16, xch, nullptr, rows, [&]() { mbar_arrive_cluster(cluster_addr(&acc_empty[b], 0)); });
     }
   }
   tc_fence_before();
@@ -1091,7 +1100,7 @@ static int sm_count() {
 template <bool GU, bool SPLIT>
 static cudaError_t launch_persistent(const CUtensorMap& tw, const CUtensorMap& tx, const CUtensorMap& txl, float* y, int M, int N,
                                      int K, int accumulate, int* err, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, cudaStream_t s,
-                                     int f16 = 0, const int32_t* n_active = nullptr, RowScale rs = RowScale()) {
+                                     int f16 = 0, const int32_t* n_active = nullptr, RowScale rs = RowScale(), int rows = PersistCfg<SPLIT, GU>::kRows) {
   using C = PersistCfg<SPLIT, GU>;
   constexpr size_t smem = C::kSmemBytes;
   static OncePerDevice configured;
@@ -1099,10 +1108,10 @@ static cudaError_t launch_persistent(const CUtensorMap& tw, const CUtensorMap& t
   if (set != cudaSuccess) return set;
   const int n_sm = sm_count();
   if (n_sm <= 0) return cudaErrorInvalidDevice;
-  const int tiles_n = GU ? N / 64 : (N + kTileN - 1) / kTileN, tiles_m = (M + C::kRows - 1) / C::kRows;
+  const int tiles_n = GU ? N / 64 : (N + kTileN - 1) / kTileN, tiles_m = (M + rows - 1) / rows;
   const int grid = std::min(tiles_n * tiles_m, n_sm);
   RSD_LAUNCH((gemm_tc_persistent_kernel<GU, SPLIT>), grid, kPersistThreads, smem, s, tw, tx, txl, y, M, N, K, accumulate, tiles_n,
-             tiles_m, err, act_hi, act_lo, f16, n_active, rs);
+             tiles_m, err, act_hi, act_lo, f16, n_active, rs, rows);
   return launched(1);
 }
 
@@ -1119,10 +1128,10 @@ static int max_pairs(size_t smem) {
   return cudaOccupancyMaxActiveClusters(&n, gemm_tc_pair_kernel<GU, SPLIT>, &cfg) == cudaSuccess ? n : 0;
 }
 
-// The map of x has a box of 128 rows.
+// The map of x has a box of half the tile's operand rows.
 template <bool GU, bool SPLIT>
 static cudaError_t launch_pair(const CUtensorMap& tw, const CUtensorMap& tx, const CUtensorMap& txl, float* y, int M, int N, int K,
-                               int accumulate, int* err, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, cudaStream_t s, int f16) {
+                               int accumulate, int* err, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, cudaStream_t s, int f16, int rows) {
   using C = PairCfg<SPLIT, GU>;
   constexpr size_t smem = C::kSmemBytes;
   static OncePerDevice configured;
@@ -1130,7 +1139,7 @@ static cudaError_t launch_pair(const CUtensorMap& tw, const CUtensorMap& tx, con
   if (set != cudaSuccess) return set;
   static const int pairs = max_pairs<GU, SPLIT>(smem);
   if (pairs <= 0) return cudaErrorNotSupported;
-  const int feat = GU ? kTileN : 2 * kTileN, tiles_n = (N + feat - 1) / feat, tiles_m = (M + C::P::kRows - 1) / C::P::kRows;
+  const int feat = GU ? kTileN : 2 * kTileN, tiles_n = (N + feat - 1) / feat, tiles_m = (M + rows - 1) / rows;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * std::min(tiles_n * tiles_m, pairs)); cfg.blockDim = dim3(kPersistThreads); cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -1141,7 +1150,7 @@ static cudaError_t launch_pair(const CUtensorMap& tw, const CUtensorMap& tx, con
   attr[1].val.clusterDim.x = 2; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr; cfg.numAttrs = 2;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_tc_pair_kernel<GU, SPLIT>, tw, tx, txl, y, M, N, K, accumulate, tiles_n, tiles_m,
-                                           err, act_hi, act_lo, f16);
+                                           err, act_hi, act_lo, f16, rows);
   return e != cudaSuccess ? e : launched(1);
 }
 
@@ -1153,6 +1162,24 @@ static cudaError_t launch_pair(const CUtensorMap& tw, const CUtensorMap& tx, con
 static bool pair_pays(int M, int n_features, int K, int feat, int rows, bool adds) {
   return K >= (adds ? 3072 : 1024) && ((n_features + feat - 1) / feat) * ((M + rows - 1) / rows) >= 74;
 }
+
+// x rows of a tile for plain operands in the persistent kernels: 256, or fewer where the waves then cost less.  A smaller tile costs
+// more per row (the weight half of a stage is read as often): kCost, in 256-row units, fitted to 8192 x 18944 x 3584 (gate/up, full waves:
+// 1387 / 1460 / 1583 / 1826 us with 256 / 224 / 192 / 160 rows; 128 rows, 2355, never pay).  Where the last wave of 256-row tiles is
+// nearly empty (4096 x 3584: 224 tiles on 74 pairs of SMs) fewer rows win; us at 256 / 224 / 192 / 160: 4096 x 3584 x 18944 576 / 506 / 545 / 509,
+// 1300 x 3584 x 18944 260 / 229 / 204 / 192, 4096 x 1536 x 8960 140 / 125 / 113 / 144, 8192 x 1536 x 1536 (lone CTAs) 55.8 / 50.8 / 55.8 / 57.9,
+// 1300 x 4608 x 3584 55 / 50 / 45 / 54; and 4096 x 2048 x 1536, two full waves, stays at 256 (29.5 / 35.0 / 32.1 / 29.5).
+static int wave_rows(int M, int n_tiles, int slots) {
+  constexpr int kRows[4] = {256, 224, 192, 160}, kCost[4] = {256, 233, 217, 206};
+  int best = 0;
+  long cost = 0;
+  for (int i = 0; i < 4; ++i) {
+    const long c = (((long)n_tiles * ((M + kRows[i] - 1) / kRows[i]) + slots - 1) / slots) * kCost[i];
+    if (i == 0 || c < cost) { best = i; cost = c; }
+  }
+  return kRows[best];
+}
+static int pair_tiles(int n_features, int feat) { return (n_features + feat - 1) / feat; }
 
 // Rows of x per tile for a dense product with one operand (bf16 or fp16): 256, or 128 or 64 while the tiles of the larger
 // size leave half of the SMs (of 256) or some (of 128) without one.  Every size sums along K in the same order: the
@@ -1222,9 +1249,10 @@ cudaError_t launch_gemm_gu(const void* Wgu, const void* x, const void* x_lo, voi
     // plain bf16 operand: the persistent kernel only (more than 128 rows, no row scale, no idle flag)
     if (!(M > 128 && rs.ssq == nullptr && n_active == nullptr)) return cudaErrorNotSupported;
     const bool pair = pair_pays(M, F, K, kTileN, 256, false);
-    if (!get_map(Wgu, 2 * F, K, kTileN / 2, &tw) || !get_map(x, M, K, pair ? 128 : 256, &tx)) return cudaErrorNotSupported;
-    if (pair) return launch_pair<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act_hi, nullptr, s, 0);
-    return launch_persistent<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act_hi, nullptr, s);
+    const int tile_rows = pair ? wave_rows(M, pair_tiles(F, kTileN), 74) : wave_rows(M, F / 64, 148);
+    if (!get_map(Wgu, 2 * F, K, kTileN / 2, &tw) || !get_map(x, M, K, pair ? tile_rows / 2 : tile_rows, &tx)) return cudaErrorNotSupported;
+    if (pair) return launch_pair<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act_hi, nullptr, s, 0, tile_rows);
+    return launch_persistent<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act_hi, nullptr, s, 0, nullptr, RowScale(), tile_rows);
   }
   if (!act_lo) return cudaErrorNotSupported;
   // each warp pair finishes one half of the rows, up to 16 at a time
@@ -1282,18 +1310,20 @@ cudaError_t launch_gemm_tc(const void* W, const void* x, const void* x_lo, float
   CUtensorMap tw, tx, txl;
   const bool dense = M > 128 && p.splits == 1 && rs.ssq == nullptr && n_active == nullptr;
   const bool pair = dense && pair_pays(M, N, K, 2 * kTileN, p.rows, accumulate != 0);
-  const int rows = dense && !split_operand && !pair && !no_k_split ? dense_rows(M, N, K, accumulate != 0) : p.rows;
-  if (!get_map(W, N, K, kTileN, &tw) || !get_map(x, M, K, pair ? 128 : rows, &tx)) return cudaErrorNotSupported;
+  int rows = dense && !split_operand && !pair && !no_k_split ? dense_rows(M, N, K, accumulate != 0) : p.rows;
+  const bool small = dense && !pair && !split_operand && rows < 256;
+  if (dense && !split_operand && !small) rows = pair ? wave_rows(M, pair_tiles(N, 2 * kTileN), 74) : wave_rows(M, p.n_tiles, 148);
+  if (!get_map(W, N, K, kTileN, &tw) || !get_map(x, M, K, pair ? (split_operand ? 128 : rows / 2) : rows, &tx)) return cudaErrorNotSupported;
   if (split_operand) { if (!get_map(x_lo, M, K, p.rows, &txl)) return cudaErrorNotSupported; }
   else txl = tx;
   int* err = (int*)((char*)scratch + kCounterBytes);
   float* partials = (float*)((char*)scratch + kCounterBytes + 256);
   if (dense) {
-    if (pair && split_operand) return launch_pair<false, true>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s, 0);
-    if (pair) return launch_pair<false, false>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s, 0);
-    if (rows < 256 && !split_operand) return launch_dense_small(tw, tx, y, M, N, K, accumulate, rows, err, s, 0);
+    if (pair && split_operand) return launch_pair<false, true>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s, 0, p.rows);
+    if (pair) return launch_pair<false, false>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s, 0, rows);
+    if (small) return launch_dense_small(tw, tx, y, M, N, K, accumulate, rows, err, s, 0);
     if (split_operand) return launch_persistent<false, true>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s);
-    return launch_persistent<false, false>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s);
+    return launch_persistent<false, false>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s, 0, nullptr, RowScale(), rows);
   }
   if (split_operand && p.splits == 1 && wide_decode(M, p.n_tiles))
     return launch_persistent<false, true>(tw, tx, txl, y, M, N, K, accumulate, err, nullptr, nullptr, s, 0, n_active, rs);
@@ -1337,12 +1367,14 @@ cudaError_t launch_gemm_f16_dense(const void* W16, const void* x16, float* y, in
   if (((uintptr_t)W16 & 15) || ((uintptr_t)x16 & 15)) return cudaErrorMisalignedAddress;
   const bool pair = pair_pays(M, N, K, 2 * kTileN, 256, accumulate != 0);
   CUtensorMap tw, tx;
-  const int rows = pair ? 128 : dense_rows(M, N, K, accumulate != 0);
-  if (!get_map(W16, N, K, kTileN, &tw) || !get_map(x16, M, K, rows, &tx)) return cudaErrorNotSupported;
+  int rows = pair ? 256 : dense_rows(M, N, K, accumulate != 0);
+  const bool small = rows < 256;
+  if (!small) rows = pair ? wave_rows(M, pair_tiles(N, 2 * kTileN), 74) : wave_rows(M, (N + kTileN - 1) / kTileN, 148);
+  if (!get_map(W16, N, K, kTileN, &tw) || !get_map(x16, M, K, pair ? rows / 2 : rows, &tx)) return cudaErrorNotSupported;
   int* err = (int*)((char*)scratch + kCounterBytes);
-  if (!pair && rows < 256) return launch_dense_small(tw, tx, y, M, N, K, accumulate, rows, err, s, 1);
-  if (pair) return launch_pair<false, false>(tw, tx, tx, y, M, N, K, accumulate, err, nullptr, nullptr, s, 1);
-  return launch_persistent<false, false>(tw, tx, tx, y, M, N, K, accumulate, err, nullptr, nullptr, s, 1);
+  if (small) return launch_dense_small(tw, tx, y, M, N, K, accumulate, rows, err, s, 1);
+  if (pair) return launch_pair<false, false>(tw, tx, tx, y, M, N, K, accumulate, err, nullptr, nullptr, s, 1, rows);
+  return launch_persistent<false, false>(tw, tx, tx, y, M, N, K, accumulate, err, nullptr, nullptr, s, 1, nullptr, RowScale(), rows);
 }
 
 // act [M, F] fp16 = silu(g) * u with [g | u] = x [M, K] Wgu [2F, K]^T, fp16 operands, more than 128 rows.
@@ -1354,9 +1386,10 @@ cudaError_t launch_gemm_gu_f16_dense(const void* Wgu16, const void* x16, void* a
   int* err = (int*)((char*)scratch + kCounterBytes);
   CUtensorMap tw, tx;
   const bool pair = pair_pays(M, F, K, kTileN, 256, false);
-  if (!get_map(Wgu16, 2 * F, K, kTileN / 2, &tw) || !get_map(x16, M, K, pair ? 128 : 256, &tx)) return cudaErrorNotSupported;
-  if (pair) return launch_pair<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act16, nullptr, s, 1);
-  return launch_persistent<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act16, nullptr, s, 1);
+  const int rows = pair ? wave_rows(M, pair_tiles(F, kTileN), 74) : wave_rows(M, F / 64, 148);
+  if (!get_map(Wgu16, 2 * F, K, kTileN / 2, &tw) || !get_map(x16, M, K, pair ? rows / 2 : rows, &tx)) return cudaErrorNotSupported;
+  if (pair) return launch_pair<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act16, nullptr, s, 1, rows);
+  return launch_persistent<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act16, nullptr, s, 1, nullptr, RowScale(), rows);
 }
 
 cudaError_t launch_gemm(int dtype, const void* W, const void* x, const void* x_lo, float* y, int M, int N, int K,

@@ -744,6 +744,26 @@ def test_gate_up_gemm_on_pairs_of_ctas(M, F, K):
     assert int(scratch[4096:4100].view(torch.int32).item()) == 0
 
 
+@pytest.mark.parametrize("M,N,K,adds", [(1100, 4608, 1024, False), (1290, 4500, 1032, False), (3000, 3584, 3080, True),
+                                        (3200, 1536, 136, True), (4080, 1536, 136, True)])
+def test_dense_tiles_of_fewer_rows(M, N, K, adds):
+    """Products whose last wave of 256-row tiles would be nearly empty take tiles of 160, 192 and 224 rows, in pairs of CTAs (first three) and
+    lone; ragged last tiles of rows and features.  fp32 sums of K products of order 0.05, as above."""
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    W = (torch.randn(N, K, generator=g, device="cuda") * 0.05).half()
+    x = torch.randn(M, K, generator=g, device="cuda").half()
+    y0 = torch.randn(M, N, generator=g, device="cuda")
+    y = rb.k_gemm(W, x, y=y0.clone(), accumulate=True, impl=4) if adds else rb.k_gemm(W, x, impl=4)
+    want = x.double() @ W.double().t() + (y0 if adds else 0)
+    assert (y.double() - want).abs().max().item() <= 2e-5 * K ** 0.5 + 2e-6
+
+
+@pytest.mark.parametrize("M,F,K", [(300, 2048, 136), (1300, 18944, 1024)])
+def test_gate_up_tiles_of_fewer_rows(M, F, K):
+    """The same for gate/up products: 160-row tiles of lone CTAs, 224-row tiles of pairs; the bound of the paired test above."""
+    test_gate_up_gemm_on_pairs_of_ctas(M, F, K)
+
+
 @pytest.mark.parametrize("one_pass", [0, 1])
 def test_chunk_attention_wait_runs_out_cleanly(one_pass):
     """Failure path of the two tcgen05 chunk-attention kernels: no copy is issued, the bounded wait runs out, the flag is
