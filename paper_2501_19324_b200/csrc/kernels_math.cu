@@ -294,9 +294,99 @@ gemv_splitk_kernel(const WT* __restrict__ W, const WT* X, const WT* X_lo, float*
   }
 }
 
-cudaError_t launch_gemm_simt(int dtype, const void* W, const void* x, const void* x_lo, float* y, int M, int N, int K,
-                             int accumulate, const int32_t* n_active, cudaStream_t s) {
-  if (M <= 0 || N <= 0) return cudaSuccess;
+// fp32 products of more rows (prefill, scoring and catch-up of fp32 models): 32 rows of x by 32 of W a block, 32 values of K a stage, four
+// stages of 16-byte cp.async copies; four groups of 64 threads take eight of a stage's 32 values of K each, 4 x 4 results a thread, and
+// their sums meet at the end.  (Eight rows at a time, as above, the weights come from L2 once per eight rows and every one is used eight
+// times per load.)  Bound by shared-memory reads (two of 16 bytes per 16 multiply-adds) and by the latency of a stage, the blocks being
+// few: 0.5 us a stage
+// (tiles of 64 columns with 4 x 4 or 4 x 8 results a thread, 0.75 and 0.95).
+constexpr int kSgM = 32, kSgN = 32, kSgK = 32, kSgLd = kSgK + 4, kSgStages = 4, kSgGroups = 4;   // rows 16 bytes apart modulo 128: no bank conflicts
+constexpr int kSgStage = (kSgM + kSgN) * kSgLd, kSgThreads = 64 * kSgGroups;
+static_assert((kSgGroups - 1) * kSgM * kSgN <= kSgStages * kSgStage, "the groups' sums take the place of the stages");
+
+__global__ void __launch_bounds__(kSgThreads)
+sgemm_kernel(const float* __restrict__ W, const float* __restrict__ X, float* Y, int M, int N, int K, int accumulate) {
+  RSD_PDL_SYNC();
+  extern __shared__ __align__(16) float sg_smem[];
+  const int n0 = blockIdx.x * kSgN, m0 = blockIdx.y * kSgM, grp = threadIdx.x / 64, tid = threadIdx.x % 64;
+  const int steps = (K + kSgK - 1) / kSgK;
+  auto fetch = [&](int step) {
+    if (step < steps) {
+      float* dst = sg_smem + (step % kSgStages) * kSgStage;
+      for (int idx = threadIdx.x; idx < (kSgM + kSgN) * kSgK / 4; idx += kSgThreads) {
+        const int r = idx / (kSgK / 4), c = idx % (kSgK / 4) * 4, k = step * kSgK + c;
+        const bool is_x = r < kSgM;
+        const int row = is_x ? m0 + r : n0 + r - kSgM;
+        const bool in = k < K && row < (is_x ? M : N);
+        const float* src = (is_x ? X : W) + (in ? (size_t)row * K + k : 0);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst + r * kSgLd + c)),
+                     "l"(src), "r"(in ? 16 : 0) : "memory");          // beyond an edge: zeros
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int i = 0; i < kSgStages - 1; ++i) fetch(i);
+  const int tn = tid & 7, tm = tid >> 3;         // rows tm + 8 i of x, tn + 8 j of W
+  float acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  for (int step = 0; step < steps; ++step) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kSgStages - 2) : "memory");
+    __syncthreads();                             // the stage is there for all, and the one before it has been read by all
+    fetch(step + kSgStages - 1);
+    const float* xs = sg_smem + (step % kSgStages) * kSgStage;
+    const float* ws = xs + kSgM * kSgLd;
+#pragma unroll
+    for (int k = 0; k < kSgK / kSgGroups; k += 4) {
+      const int kk = grp * (kSgK / kSgGroups) + k;
+      float4 a[4], b[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(xs + (tm + 8 * i) * kSgLd + kk);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(ws + (tn + 8 * j) * kSgLd + kk);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          acc[i][j] = fmaf(a[i].w, b[j].w, fmaf(a[i].z, b[j].z, fmaf(a[i].y, b[j].y, fmaf(a[i].x, b[j].x, acc[i][j]))));
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  if (grp > 0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) sg_smem[((grp - 1) * kSgM + tm + 8 * i) * kSgN + tn + 8 * j] = acc[i][j];
+  }
+  __syncthreads();
+  if (grp > 0) return;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int m = m0 + tm + 8 * i;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int n = n0 + tn + 8 * j;
+      float v = acc[i][j];
+#pragma unroll
+      for (int r = 0; r < kSgGroups - 1; ++r) v += sg_smem[(r * kSgM + tm + 8 * i) * kSgN + tn + 8 * j];
+      if (m < M && n < N) {
+        float* y = Y + (size_t)m * N + n;
+        *y = accumulate ? *y + v : v;
+      }
+    }
+  }
+}
+
+// Both take as long along K, so that rows times columns decide.  us, eight rows at a time / tiled: 96 x 512 x 256 9.2 / 5.8, 64 x 512 x
+// 1376 24.4 / 23.2, 96 x 256 x 688 12.5 / 12.7, 17 x 2752 x 512 13.7 / 12.6, 48 x 512 x 512 9.3 / 9.9; 256 x 2752 x 512 153 / 32.
+static bool sgemm_pays(int M, int N) { return M > 16 && (long)M * N >= 32768; }
+
+// K splits over the warps of a block.
+static int simt_splits(int dtype, int M, int N, int K) {
   // Pick the split so that the grid covers the 148 SMs a few times over, as long as every lane has two vectors, or one (fp32) where
   // there are up to four rows or few blocks.  More rows are more blocks, each with its reductions: splitting them as finely, and
   // holding weights ahead in registers where no wait is to be bridged, cost 256 x 512 x 1376 146 us instead of 84 and 60 x 512 x
@@ -309,6 +399,22 @@ cudaError_t launch_gemm_simt(int dtype, const void* W, const void* x, const void
     return K / k >= (dtype != 1 && (M <= 4 || blocks < 148 || (k == 2 && blocks < 296)) ? 128 : 256);
   };
   while (ks < 8 && (long)N * ks / 8 < 148L * 4 && lanes_full(2 * ks)) ks *= 2;
+  return ks;
+}
+
+cudaError_t launch_gemm_simt(int dtype, const void* W, const void* x, const void* x_lo, float* y, int M, int N, int K,
+                             int accumulate, const int32_t* n_active, cudaStream_t s) {
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  if (dtype != 1 && n_active == nullptr && sgemm_pays(M, N)) {
+    static OncePerDevice configured;
+    constexpr size_t smem = kSgStages * kSgStage * sizeof(float);
+    const cudaError_t set = allow_smem(configured, sgemm_kernel, smem);
+    if (set != cudaSuccess) return set;
+    RSD_LAUNCH((sgemm_kernel), dim3((N + kSgN - 1) / kSgN, (M + kSgM - 1) / kSgM), kSgThreads, smem, s, (const float*)W, (const float*)x, y, M, N, K, accumulate);
+    return launched(1);
+  }
+  const int ks = simt_splits(dtype, M, N, K), mt = M <= 4 ? 4 : 8;
+  const long m_blocks = (M + mt - 1) / mt;
   const bool ahead = M <= 4 || n_active != nullptr;
   dim3 grid((N + (8 / ks) - 1) / (8 / ks), (unsigned)m_blocks);
 #define RSD_GEMV(WT, MT, AHEAD) RSD_LAUNCH((gemv_splitk_kernel<WT, MT, AHEAD>), grid, 256, 0, s, (const WT*)W, (const WT*)x, (const WT*)x_lo, y, M, N, K, ks, accumulate, n_active)

@@ -84,6 +84,12 @@ def test_gemm_simt(M, N, K, bf16):
     np.testing.assert_allclose(acc, want + y0, rtol=0, atol=2e-5 * np.sqrt(K))
 
 
+@pytest.mark.parametrize("M,N,K", [(17, 1928, 4), (33, 1000, 36), (97, 341, 688), (128, 256, 1376), (300, 130, 100)])
+def test_gemm_fp32_of_many_rows(M, N, K):
+    """The tiled fp32 product: less than a stage of K and many, ragged rows, columns and K; the bound of the test above."""
+    test_gemm_simt(M, N, K, False)
+
+
 @pytest.mark.parametrize("M,N,K", [(16, 128, 64), (5, 256, 512), (17, 1536, 1536), (32, 2048, 1536), (33, 1000, 520),
                                    (64, 1536, 8960), (100, 384, 1408), (128, 640, 768), (129, 256, 2048),
                                    (300, 4096, 512), (1000, 1280, 768), (8, 17920, 1536), (200, 384, 520), (2500, 1024, 192)])
