@@ -600,6 +600,32 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
   return RSD_OK;
 }
 
+// Decode pass of an fp32 model, five kernels a layer: RMSNorm goes into the products behind it, SwiGLU into the gate/up product, the
+// rotation and the page write into the attention.  On return x is the final residual stream.
+bool decode_f32_ok(const rsd_ctx* c, const ModelHost& M, PassView p) {
+  return M.m.dtype == RSD_F32 && M.kv_dtype == 0 && p.n_active != nullptr && c->pass_width == 1;
+}
+
+int forward_decode_f32(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
+  const ModelHost& M = c->mdl[which];
+  const rsd_model& m = M.m;
+  const int d = m.d_model, H = m.n_heads, KV = m.n_kv_heads, hd = m.head_dim, F = m.d_ffn, T = p.T;
+  if (T <= 0) return RSD_OK;
+  float *attn = (float*)c->attn, *act = (float*)c->act;
+  CU(launch_embed(m.dtype, m.tok_embed, p, c->x, d, s));
+  for (int l = 0; l < m.n_layers; ++l) {
+    KvView kv{M.kv_pool + (size_t)l * M.layer_stride, c->st.page_table[which], c->max_pages, 0};
+    CU(launch_gemv_norm((const float*)M.wqkv[l], (const float*)M.norm1[l], c->x, c->qkv, T, (H + 2 * KV) * hd, d, m.rms_eps, false, p.n_active, s));
+    CU(launch_attn_generic(0, c->qkv, p, kv, attn, nullptr, RSD_F32, H, KV, hd, s, M.rope));
+    int rc = gemm(c, M, M.wo[l], attn, nullptr, c->x, T, d, H * hd, 1, p.n_active, nullptr, s);
+    if (rc) return rc;
+    CU(launch_gemv_norm((const float*)M.wgu[l], (const float*)M.norm2[l], c->x, act, T, F, d, m.rms_eps, true, p.n_active, s));
+    rc = gemm(c, M, M.wdown[l], act, nullptr, c->x, T, d, F, 1, p.n_active, nullptr, s);
+    if (rc) return rc;
+  }
+  return RSD_OK;
+}
+
 // Multi-token pass over the flat list of `rows` sequences at most built by launch_build_pass, `chunk` tokens at a time.
 int run_ingest(rsd_ctx* c, int which, int n_total, int rows, bool want_reward, cudaStream_t s) {
   for (int c0 = 0; c0 < n_total; c0 += c->chunk) {
@@ -705,6 +731,9 @@ int model_logits(rsd_ctx* c, int which, PassView p, bool allow_mega, cudaStream_
     if ((rc = forward_decode_fused(c, which, p, m.final_norm, s))) return rc;
     const RowScale rs{c->norm_ssq, norm_chunks(m.d_model), 1.f / (float)m.d_model, m.rms_eps};
     rc = gemm(c, M, m.head, c->h, c->h_lo, c->logits, T, m.vocab, m.d_model, 0, p.n_active, nullptr, s, rs);
+  } else if (decode_f32_ok(c, M, p)) {
+    if ((rc = forward_decode_f32(c, which, p, s))) return rc;
+    CU(launch_gemv_norm((const float*)m.head, (const float*)m.final_norm, c->x, c->logits, T, m.vocab, m.d_model, m.rms_eps, false, p.n_active, s));
   } else {
     if ((rc = forward_pass(c, which, p, s))) return rc;
     CU(launch_rmsnorm(m.dtype, c->x, m.final_norm, c->h, M.split ? c->h_lo : nullptr, T, m.d_model, m.rms_eps,
@@ -1174,6 +1203,7 @@ static int score_with_draft_trunk(rsd_ctx* c, cudaStream_t s) {
   const bool was_in_decode = c->in_decode;
   c->in_decode = true;             // GEMM timing: treated like a decode iteration that is not sampled
   if (fused_decode_ok(D)) rc = forward_decode_fused(c, RSD_DRAFT, p, prm.final_norm, s);
+  else if (decode_f32_ok(c, D, p)) rc = forward_decode_f32(c, RSD_DRAFT, p, s);
   else rc = forward_pass(c, RSD_DRAFT, p, s);
   c->in_decode = was_in_decode;
   if (rc) return rc;

@@ -62,6 +62,9 @@ cudaError_t launch_rmsnorm(int dtype, const float* x, const void* gain, void* ou
 // x_lo (nullable, bf16 only): second operand matrix added to x (split-precision activations).
 cudaError_t launch_gemm_simt(int dtype, const void* W, const void* x, const void* x_lo, float* y, int M, int N, int K,
                              int accumulate, const int32_t* n_active, cudaStream_t s);
+// fp32 decode products with RMSNorm ahead: y [M, N] = rmsnorm(x) W^T, or (gate_up) silu(g) * u with [g | u] = rmsnorm(x) W^T, W of 2 N rows.
+cudaError_t launch_gemv_norm(const float* W, const float* gain, const float* x, float* y, int M, int N, int K, float eps, bool gate_up,
+                             const int32_t* n_active, cudaStream_t s);
 // tcgen05 / TMEM / TMA GEMM (bf16): same contract as launch_gemm_simt; `scratch` holds split-K
 // partial tiles and tile counters (the counters must be zero on entry and are left zero).
 bool gemm_tc_supported(int dtype, int M, int N, int K);
@@ -108,7 +111,8 @@ cudaError_t launch_rope_kv(int kv_dtype, const float* qkv, SplitSum pending, Pas
 cudaError_t launch_rope_only(float* v, const int32_t* pos, int T, int n_heads, int hd, float theta, cudaStream_t s);
 // Causal attention of every slot over positions [0, tok_pos] of its row, read from the pages.
 cudaError_t launch_attn_generic(int kv_dtype, const float* q, PassView p, KvView kv, void* out, void* out_lo,
-                                int out_dtype, int H, int KV, int hd, cudaStream_t s);
+                                int out_dtype, int H, int KV, int hd, cudaStream_t s, const float2* rope = nullptr);
+// (rope: fp32 caches, a decode pass: q is the qkv product; the kernel rotates and writes the cache as launch_rope_kv would.)
 // Tensor-core versions of the above for 16-bit caches with H / KV <= 8 (falls back otherwise): the tcgen05 kernel for
 // fp16 caches with head_dim 128 and at least 64 list entries (attn_chunk_tc.cu), else the mma.sync kernel.
 // err (nullable): raised to -5 when a bounded wait of the tcgen05 kernel expires.

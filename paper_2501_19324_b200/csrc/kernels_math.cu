@@ -294,6 +294,90 @@ gemv_splitk_kernel(const WT* __restrict__ W, const WT* X, const WT* X_lo, float*
   }
 }
 
+// The decode products of fp32 models with the small steps around them: RMSNorm ahead (the gain goes into the weights as they arrive,
+// the row's sum of squares is taken along with the products and its root divides the finished sum) and SwiGLU behind (GU: a warp
+// streams the gate row and the up row of its column).  Geometry, reads ahead and order of the sums are those of the kernel above.
+// Bound by latency like it; what this removes is a launch of 1.2-1.4 us for every norm and one for the SwiGLU.
+template <int MT, int AHEAD, bool GU>
+__global__ void __launch_bounds__(256)
+gemv_norm_kernel(const float* W, const float* __restrict__ gain, const float* X, float* Y, int M, int N, int K, int ks, float eps,
+                 const int32_t* n_active) {
+  RSD_PDL_TRIGGER();
+  constexpr int VN = 4, R = GU ? 2 : 1;
+  __shared__ float part[8][R + 1][MT];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nb = 8 / ks;
+  const int col = warp / ks, split = warp % ks;
+  const int n = blockIdx.x * nb + col;
+  const int m0 = blockIdx.y * MT;
+  const int nvec = n < N ? K / VN : 0, v0 = split * 32 + lane, step = ks * 32;
+  const float* wrow = W + (size_t)n * K;
+  Vec16<float> ahead[AHEAD][R];
+  if (n_active == nullptr) RSD_PDL_WAIT();   // outside a decode pass W may be an earlier kernel's output
+  const bool idle = n_active != nullptr && ld_cg(n_active) == 0;
+  auto weights = [&](Vec16<float> (&w)[R], int v) {
+    Vec16<float> g;
+    g.load(gain + (size_t)v * VN);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      w[r].load_stream(wrow + (size_t)r * N * K + (size_t)v * VN);
+#pragma unroll
+      for (int j = 0; j < VN; ++j) w[r].v[j] *= g.v[j];
+    }
+  };
+#pragma unroll
+  for (int i = 0; i < AHEAD; ++i)
+    if (v0 + i * step < nvec) weights(ahead[i], v0 + i * step);
+  RSD_PDL_WAIT();
+  if (idle) return;
+  float acc[R + 1][MT];                      // the last: sums of squares
+#pragma unroll
+  for (int r = 0; r <= R; ++r)
+#pragma unroll
+    for (int m = 0; m < MT; ++m) acc[r][m] = 0.f;
+  auto fold = [&](const Vec16<float> (&w)[R], int v) {
+#pragma unroll
+    for (int m = 0; m < MT; ++m) {
+      if (m0 + m < M) {
+        Vec16<float> xv;
+        xv.load(X + (size_t)(m0 + m) * K + (size_t)v * VN);
+#pragma unroll
+        for (int j = 0; j < VN; ++j) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) acc[r][m] = fmaf(w[r].v[j], xv.v[j], acc[r][m]);
+          acc[R][m] = fmaf(xv.v[j], xv.v[j], acc[R][m]);
+        }
+      }
+    }
+  };
+#pragma unroll
+  for (int i = 0; i < AHEAD; ++i)
+    if (v0 + i * step < nvec) fold(ahead[i], v0 + i * step);
+  for (int v = v0 + AHEAD * step; v < nvec; v += step) {
+    Vec16<float> w[R];
+    weights(w, v);
+    fold(w, v);
+  }
+#pragma unroll
+  for (int r = 0; r <= R; ++r)
+#pragma unroll
+    for (int m = 0; m < MT; ++m) {
+      const float t = warp_sum(acc[r][m]);
+      if (lane == 0) part[warp][r][m] = t;
+    }
+  __syncthreads();
+  const int oc = threadIdx.x / MT, om = threadIdx.x % MT, on = blockIdx.x * nb + oc;
+  if (!(threadIdx.x < nb * MT && on < N && m0 + om < M)) return;
+  float sum[R + 1];
+#pragma unroll
+  for (int r = 0; r <= R; ++r) {
+    sum[r] = 0.f;
+    for (int sidx = 0; sidx < ks; ++sidx) sum[r] += part[oc * ks + sidx][r][om];
+  }
+  const float inv = rsqrtf(sum[R] / (float)K + eps);
+  Y[(size_t)(m0 + om) * N + on] = GU ? swiglu(sum[0] * inv, sum[R - 1] * inv) : sum[0] * inv;
+}
+
 // fp32 products of more rows (prefill, scoring and catch-up of fp32 models): 32 rows of x by 32 of W a block, 32 values of K a stage, four
 // stages of 16-byte cp.async copies; four groups of 64 threads take eight of a stage's 32 values of K each, 4 x 4 results a thread, and
 // their sums meet at the end.  (Eight rows at a time, as above, the weights come from L2 once per eight rows and every one is used eight
@@ -400,6 +484,19 @@ static int simt_splits(int dtype, int M, int N, int K) {
   };
   while (ks < 8 && (long)N * ks / 8 < 148L * 4 && lanes_full(2 * ks)) ks *= 2;
   return ks;
+}
+
+// y = rmsnorm(x) W^T, or silu(g) * u with [g | u] = rmsnorm(x) W^T and W of 2 N rows.
+cudaError_t launch_gemv_norm(const float* W, const float* gain, const float* x, float* y, int M, int N, int K, float eps, bool gate_up,
+                             const int32_t* n_active, cudaStream_t s) {
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  const int ks = simt_splits(0, M, N, K), mt = M <= 4 ? 4 : 8;
+  const dim3 grid((N + (8 / ks) - 1) / (8 / ks), (unsigned)((M + mt - 1) / mt));
+#define RSD_GN(MT, GU) RSD_LAUNCH((gemv_norm_kernel<MT, GU ? 2 : kGemvAhead, GU>), grid, 256, 0, s, W, gain, x, y, M, N, K, ks, eps, n_active)
+  if (mt == 4) { if (gate_up) RSD_GN(4, true); else RSD_GN(4, false); }
+  else { if (gate_up) RSD_GN(8, true); else RSD_GN(8, false); }
+#undef RSD_GN
+  return launched(1);
 }
 
 cudaError_t launch_gemm_simt(int dtype, const void* W, const void* x, const void* x_lo, float* y, int M, int N, int K,
@@ -715,10 +812,13 @@ cudaError_t launch_rope_only(float* v, const int32_t* pos, int T, int n_heads, i
 constexpr int kGenericWarps = 16;
 
 // VEC: 16-byte loads; a caller's pool may start anywhere, and one off a 16-byte boundary is read element by element.
-template <typename KT, typename OT, int HD, bool VEC>
+// FUSE (a decode pass of an fp32 model; every row's only new position is its last): q is the qkv product [T][(H + 2 KV) HD]; the kernel
+// rotates by the table, keeps the new key and value in shared memory, and the first block of a group writes them to the cache.  Every page
+// is then older than the pass but for that one slot, so a warp's first page is on its way before the wait.
+template <typename KT, typename OT, int HD, bool VEC, bool FUSE>
 __global__ void __launch_bounds__(32 * kGenericWarps)
-attn_generic_kernel(const float* q, PassView p, const KT* pool, const int32_t* page_table, int max_pages, OT* out, OT* out_lo,
-                    int H, int KV, int pf) {
+attn_generic_kernel(const float* q, PassView p, KT* pool, const int32_t* page_table, int max_pages, OT* out, OT* out_lo,
+                    int H, int KV, int pf, const float2* __restrict__ rope) {
   RSD_PDL_TRIGGER();
   constexpr int DPL = HD / 32;            // output dims of a lane
   constexpr int VN = 16 / sizeof(KT);     // elements of a 16-byte load
@@ -726,6 +826,7 @@ attn_generic_kernel(const float* q, PassView p, const KT* pool, const int32_t* p
   constexpr int NV = kPageTokens / VN;    // value loads of a dim
   __shared__ __align__(16) float s_q[HD];
   __shared__ float s_m[kGenericWarps], s_l[kGenericWarps], s_o[kGenericWarps][HD];
+  __shared__ __align__(16) float s_kv[FUSE ? 2 : 1][HD];    // the new token's key and value
   const int t = blockIdx.x / H, h = blockIdx.x % H;
   if (p.n_active == nullptr) RSD_PDL_WAIT();   // a decode pass's lists may be read ahead of the wait, others not
   const bool idle = p.n_active != nullptr && ld_cg(p.n_active) == 0;
@@ -739,19 +840,54 @@ attn_generic_kernel(const float* q, PassView p, const KT* pool, const int32_t* p
   const int n_pages = pos / kPageTokens + 1;
   const size_t block = (size_t)KV * kPageTokens * HD;
   int page = warp < n_pages ? ld_cg(pt + warp) : 0;
+  uint4 kr[NK], vr[DPL * NV];
+  auto keys = [&](int id) { return pool + (size_t)id * pf * block + (size_t)g * kPageTokens * HD + tok * HD + hf * (HD / 2); };
+  auto values = [&](int id) { return pool + (size_t)id * pf * block + block + (size_t)g * kPageTokens * HD + lane * DPL * kPageTokens; };
+  float2 cs = make_float2(1.f, 0.f);
+  int new_page = 0;
+  if (FUSE) {
+    if (VEC && warp < n_pages) {
+#pragma unroll
+      for (int i = 0; i < NK; ++i) kr[i] = __ldcg(reinterpret_cast<const uint4*>(keys(page) + i * VN));
+#pragma unroll
+      for (int i = 0; i < DPL * NV; ++i) vr[i] = __ldcg(reinterpret_cast<const uint4*>(values(page) + i * VN));
+    }
+    cs = rope[(size_t)pos * (HD / 2) + threadIdx.x % (HD / 2)];        // HD divides the block
+    new_page = ld_cg(pt + n_pages - 1);
+  }
   RSD_PDL_WAIT();
-  if (threadIdx.x < HD) s_q[threadIdx.x] = q[((size_t)t * H + h) * HD + threadIdx.x] * scale;
+  if (FUSE) {
+    // HD threads each for the query, the key and the value; dim i < HD / 2 turns with i + HD / 2
+    const int dim = threadIdx.x % HD, pair = dim < HD / 2 ? dim + HD / 2 : dim - HD / 2;
+    for (int w = threadIdx.x / HD; w < 3; w += blockDim.x / HD) {
+      const float* src = q + (size_t)t * (H + 2 * KV) * HD + (size_t)(w == 0 ? h : H + (w - 1) * KV + g) * HD;
+      float a = src[dim];
+      if (w < 2) {
+        const float b = src[pair];
+        a = dim < HD / 2 ? rotate_lo(a, b, cs) : rotate_hi(b, a, cs);
+      }
+      if (w == 0) s_q[dim] = a * scale;
+      else s_kv[FUSE ? w - 1 : 0][dim] = a;
+      if (w > 0 && h % (H / KV) == 0) {
+        const int slot = pos % kPageTokens;
+        KT* at = pool + (size_t)new_page * pf * block + (w == 1 ? ((size_t)g * kPageTokens + slot) * HD + dim : block + ((size_t)g * HD + dim) * kPageTokens + slot);
+        *at = from_f32<KT>(a);
+      }
+    }
+  } else if (threadIdx.x < HD) {
+    s_q[threadIdx.x] = q[((size_t)t * H + h) * HD + threadIdx.x] * scale;
+  }
   __syncthreads();
   float m = -INFINITY, l = 0.f, acc[DPL];
 #pragma unroll
   for (int i = 0; i < DPL; ++i) acc[i] = 0.f;
   for (int pg = warp; pg < n_pages; pg += n_warps) {
-    const KT* kb = pool + (size_t)page * pf * block + (size_t)g * kPageTokens * HD + tok * HD + hf * (HD / 2);
-    const KT* vb = pool + (size_t)page * pf * block + block + (size_t)g * kPageTokens * HD + lane * DPL * kPageTokens;
+    const KT *kb = keys(page), *vb = values(page);
     if (pg + n_warps < n_pages) page = ld_cg(pt + pg + n_warps);
     const int n = min(kPageTokens, pos + 1 - pg * kPageTokens);
-    uint4 kr[NK], vr[DPL * NV];
-    if (VEC) {
+    const bool has_new = FUSE && pg == n_pages - 1;
+    if (FUSE && VEC && pg == warp) {                       // on its way since before the wait
+    } else if (VEC) {
 #pragma unroll
       for (int i = 0; i < NK; ++i) kr[i] = *reinterpret_cast<const uint4*>(kb + i * VN);
 #pragma unroll
@@ -761,6 +897,10 @@ attn_generic_kernel(const float* q, PassView p, const KT* pool, const int32_t* p
       for (int i = 0; i < NK * VN; ++i) reinterpret_cast<KT*>(kr)[i] = kb[i];
 #pragma unroll
       for (int i = 0; i < DPL * NV * VN; ++i) reinterpret_cast<KT*>(vr)[i] = vb[i];
+    }
+    if (has_new && tok == n - 1) {
+#pragma unroll
+      for (int i = 0; i < NK; ++i) kr[i] = *reinterpret_cast<const uint4*>(&s_kv[0][hf * (HD / 2) + i * VN]);
     }
     float part[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -791,6 +931,7 @@ attn_generic_kernel(const float* q, PassView p, const KT* pool, const int32_t* p
 #pragma unroll
         for (int i = 0; i < DPL; ++i) {
           float vv = to_f32(reinterpret_cast<const KT*>(&vr[i * NV + j / VN])[j % VN]);
+          if (FUSE && has_new && j == n - 1) vv = s_kv[FUSE ? 1 : 0][lane * DPL + i];
           if (pf == 4) vv += to_f32(vb[2 * block + i * kPageTokens + j]);
           acc[i] = fmaf(pj, vv, acc[i]);
         }
@@ -816,26 +957,27 @@ attn_generic_kernel(const float* q, PassView p, const KT* pool, const int32_t* p
 }
 
 cudaError_t launch_attn_generic(int kv_dtype, const float* q, PassView p, KvView kv, void* out, void* out_lo,
-                                int out_dtype, int H, int KV, int hd, cudaStream_t s) {
+                                int out_dtype, int H, int KV, int hd, cudaStream_t s, const float2* rope) {
   if (p.T <= 0) return cudaSuccess;
+  if (rope != nullptr && (kv_dtype != 0 || out_dtype != 0 || p.n_active == nullptr)) return cudaErrorInvalidValue;
   const int blocks = p.T * H;
   // few (slot, head) pairs: sixteen warps, so that 256 cached tokens are one round; once the pairs alone fill the SMs,
   // four warps a block waste fewer on short contexts
   const int threads = 32 * (blocks <= 148 ? kGenericWarps : (blocks <= 148 * 4 ? 8 : 4));
-#define RSD_ATTN(KT, OT, HD) \
-  do {                                                                                                                  \
-    if (((uintptr_t)kv.pool_layer & 15) == 0)                                                                           \
-      RSD_LAUNCH((attn_generic_kernel<KT, OT, HD, true>), blocks, threads, 0, s, q, p, (const KT*)kv.pool_layer, kv.page_table, kv.max_pages, (OT*)out, (OT*)out_lo, H, KV, 2 + 2 * kv.v_extra); \
-    else                                                                                                                \
-      RSD_LAUNCH((attn_generic_kernel<KT, OT, HD, false>), blocks, threads, 0, s, q, p, (const KT*)kv.pool_layer, kv.page_table, kv.max_pages, (OT*)out, (OT*)out_lo, H, KV, 2 + 2 * kv.v_extra); \
-  } while (0)
+#define RSD_ATTN_K(KT, OT, HD, VEC, FUSE)                                                                               \
+  RSD_LAUNCH((attn_generic_kernel<KT, OT, HD, VEC, FUSE>), blocks, threads, 0, s, q, p, (KT*)kv.pool_layer, kv.page_table, kv.max_pages, (OT*)out, (OT*)out_lo, H, KV, 2 + 2 * kv.v_extra, rope)
+#define RSD_ATTN_F(KT, OT, HD, FUSE) do { if (((uintptr_t)kv.pool_layer & 15) == 0) RSD_ATTN_K(KT, OT, HD, true, FUSE); else RSD_ATTN_K(KT, OT, HD, false, FUSE); } while (0)
+#define RSD_ATTN(KT, OT, HD) RSD_ATTN_F(KT, OT, HD, false)
 #define RSD_ATTN_HD(KT, OT) do { if (hd == 128) RSD_ATTN(KT, OT, 128); else RSD_ATTN(KT, OT, 64); } while (0)
   using bf = __nv_bfloat16;
   if (kv_dtype == 2) { if (out_dtype == 1) RSD_ATTN_HD(__half, bf); else RSD_ATTN_HD(__half, float); }
   else if (kv_dtype == 1) { if (out_dtype == 1) RSD_ATTN_HD(bf, bf); else RSD_ATTN_HD(bf, float); }
+  else if (rope != nullptr) { if (hd == 128) RSD_ATTN_F(float, float, 128, true); else RSD_ATTN_F(float, float, 64, true); }
   else RSD_ATTN_HD(float, float);
 #undef RSD_ATTN_HD
 #undef RSD_ATTN
+#undef RSD_ATTN_F
+#undef RSD_ATTN_K
   return launched(1);
 }
 

@@ -468,6 +468,22 @@ def test_decode_attention_that_takes_the_qkv_product(d, H, KV, hd, ext):
     eng.close()
 
 
+@pytest.mark.parametrize("d,H,KV,hd,rows,lo,hi", [(64, 1, 1, 64, 3, 13, 18), (260, 4, 2, 128, 9, 14, 33), (128, 10, 1, 64, 5, 252, 262)])
+def test_fp32_decode_with_the_small_steps_inside_the_products(d, H, KV, hd, rows, lo, hi):
+    """fp32 decode passes: norms and SwiGLU in the products, rotation and page write in the attention; one head group and groups of
+    ten, both head sizes, more rows than a block of the product takes, a new token on the first and last place of a page, more
+    pages than warps."""
+    sh = ri.ModelShape(2, d, H, KV, hd, 344, 1024)
+    prompts = ri.prompts(7 + d, rows, lo, hi, sh.vocab)
+    kw = dict(max_step_tokens=8, max_steps=2, max_seq_tokens=hi + 24, step_end_id=3, step_end_mod=9, temperature=0.7, seed=4)
+    eng, loop = build_pair((sh, sh, sh), bf16=False, prompts=prompts, loop_kwargs=kw)
+    stats = {}
+    for _ in range(2):
+        parity_step(eng, loop, 2.0, stats=stats, **TOL32)      # every row is rejected: draft and target decode
+    assert stats["tokens_compared"] > 0.9 * stats["tokens"]
+    eng.close()
+
+
 def _engine(prompts, **kw):
     from paper_2501_19324_b200 import Engine, Model
     heads = (ri.HEAD_LM, ri.HEAD_REWARD_SIGMOID, ri.HEAD_LM)
