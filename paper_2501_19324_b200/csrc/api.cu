@@ -743,10 +743,9 @@ int model_logits(rsd_ctx* c, int which, PassView p, bool allow_mega, cudaStream_
   return rc;
 }
 
-// Enqueues one decode iteration: (prepare, model pass, final norm, lm_head, sample, append).
+// Enqueues one decode iteration: model pass, final norm, lm_head, sample, append (and lay out the next one).
 int decode_iteration(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t s) {
   const rsd_model& m = c->mdl[which].m;
-  CU(launch_decode_prepare(c->st, which, n_slots, s));
   PassView p{c->st.pass_tok_id, c->st.pass_tok_row, c->st.pass_tok_pos, n_slots, c->st.n_active};
   int rc = model_logits(c, which, p, true, s);
   if (rc) return rc;
@@ -884,7 +883,7 @@ int decode_phase(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t s) 
   c->host_sleeps = (flags & cudaDeviceScheduleMask) == cudaDeviceScheduleBlockingSync;
   c->host_yields = (flags & cudaDeviceScheduleMask) == cudaDeviceScheduleYield;
   *c->progress = 0;            // the stream was synchronised since the last phase: no kernel that writes the word is in flight
-  CU(launch_decode_begin(c->st, phase, s));
+  CU(launch_decode_begin(c->st, which, phase, s));
   if (n_slots <= 0) return RSD_OK;
   const bool graphs = !(c->cfg.debug_flags & RSD_DEBUG_NO_GRAPHS);
   // The attention kernel splits every row's context over so many CTAs that the ACTIVE rows fill the machine; the
@@ -931,7 +930,7 @@ int decode_phase(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t s) 
 // there are at most C rounds; the host looks at the number of unfinished rows after each.  The first round runs
 // kernel by kernel, the following ones replay two captured graphs (proposal iteration, target pass) per bucket.
 int decode_phase_sd(rsd_ctx* c, int n_slots, cudaStream_t s) {
-  CU(launch_decode_begin(c->st, 1, s));
+  CU(launch_decode_begin(c->st, RSD_TARGET, 1, s));
   if (n_slots <= 0) return RSD_OK;
   const bool graphs = !(c->cfg.debug_flags & RSD_DEBUG_NO_GRAPHS);
   int bucket = 0, rows_eff = c->st.B;

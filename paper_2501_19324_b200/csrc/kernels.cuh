@@ -265,12 +265,11 @@ inline __host__ __device__ bool target_pass_due(int n_waiting, int n_live, int m
   const int want = min_target_rows < 1 ? 1 : min_target_rows;
   return n_waiting > 0 && n_waiting >= (want < n_live ? want : n_live);
 }
-cudaError_t launch_decode_begin(const RowState& st, int phase, cudaStream_t s);
+cudaError_t launch_decode_begin(const RowState& st, int which, int phase, cudaStream_t s);
 // Merged PRM: one slot per row that took a draft step, carrying the step's last token at the draft's
 // cursor (which stays where it is); n_active = number of such rows, last_idx[b] = b for them.
 cudaError_t launch_score_prepare(const RowState& st, cudaStream_t s);
-cudaError_t launch_decode_prepare(const RowState& st, int which, int n_slots, cudaStream_t s);
-// best: packed winners left by launch_sample (cleared here).
+// best: packed winners left by launch_sample (cleared here).  Writes the lists of the next iteration.
 cudaError_t launch_decode_update(const RowState& st, int which, int phase, unsigned long long* best,
                                  int n_slots, const LoopParams& lp, cudaStream_t s);
 cudaError_t launch_gate(const RowState& st, float delta, const LoopParams& lp, cudaStream_t s);

@@ -126,7 +126,14 @@ cudaError_t launch_build_pass(const RowState& st, int which, PassMode mode, int 
 // Decode-phase control.  Phase 0: the draft writes y^_i for every live row that is not waiting for
 // the target (slot b = row b).  Phase 1: the target writes y_i for the waiting rows (slot i = rej_idx[i]).
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) decode_begin_kernel(RowState st, int phase) {
+// A pass's lists are written ahead of it: the first one's by this kernel, every next one's by the update of the one before.
+__device__ __forceinline__ void pass_slot(const RowState& st, int i, int row, int pos, int token) {
+  st.pass_tok_id[i] = token;
+  st.pass_tok_pos[i] = pos;
+  st.pass_tok_row[i] = row;
+}
+
+__global__ void __launch_bounds__(1024) decode_begin_kernel(RowState st, int which, int phase) {
   RSD_PDL_SYNC();
   __shared__ int scan[33];
   const int b = threadIdx.x;
@@ -144,15 +151,22 @@ __global__ void __launch_bounds__(1024) decode_begin_kernel(RowState st, int pha
   }
   const int n_slots = phase == 0 ? st.B : st.n_rej[0];
   if (b == 0) st.n_slots[0] = n_slots;
-  if (b < st.B) st.slot_row[b] = phase == 0 ? b : (b < n_slots ? st.rej_idx[b] : -1);
+  if (b < st.B) {
+    const int row = phase == 0 ? b : (b < n_slots ? st.rej_idx[b] : -1);
+    st.slot_row[b] = row;
+    // (the scan above has ordered gen_active's writes before these reads)
+    const int pos = row >= 0 && st.gen_active[row] ? st.kv_len[which][row] : -1;
+    if (pos >= 0) pass_slot(st, b, row, pos, st.tok[(size_t)row * st.S + pos]);
+    else st.pass_tok_row[b] = -1;
+  }
   for (int i = threadIdx.x; i < st.B * st.C; i += blockDim.x) {
     st.gen_tok[phase][i] = 0;
     st.sampled[phase][i] = 0;
   }
 }
 
-cudaError_t launch_decode_begin(const RowState& st, int phase, cudaStream_t s) {
-  RSD_LAUNCH((decode_begin_kernel), 1, 1024, 0, s, st, phase);
+cudaError_t launch_decode_begin(const RowState& st, int which, int phase, cudaStream_t s) {
+  RSD_LAUNCH((decode_begin_kernel), 1, 1024, 0, s, st, which, phase);
   return launched(1);
 }
 
@@ -182,35 +196,13 @@ cudaError_t launch_score_prepare(const RowState& st, cudaStream_t s) {
   return launched(1);
 }
 
-__global__ void __launch_bounds__(1024) decode_prepare_kernel(RowState st, int which, int n_slots) {
-  RSD_PDL_SYNC();
-  if (st.n_active[0] == 0) return;
-  const int i = threadIdx.x;
-  if (i >= n_slots) return;
-  const int row = st.slot_row[i];
-  if (row >= 0 && st.gen_active[row]) {
-    const int pos = st.kv_len[which][row];
-    st.pass_tok_id[i] = st.tok[(size_t)row * st.S + pos];
-    st.pass_tok_pos[i] = pos;
-    st.pass_tok_row[i] = row;
-  } else {
-    st.pass_tok_row[i] = -1;
-  }
-}
-
-cudaError_t launch_decode_prepare(const RowState& st, int which, int n_slots, cudaStream_t s) {
-  if (n_slots <= 0) return cudaSuccess;
-  RSD_LAUNCH((decode_prepare_kernel), 1, 1024, 0, s, st, which, n_slots);
-  return launched(1);
-}
-
 __device__ __forceinline__ bool ends_step(int t, const LoopParams& lp) {
   if (lp.eos_id >= 0 && t == lp.eos_id) return true;
   if (lp.step_end_mod > 0) return (t % lp.step_end_mod) == (lp.step_end_id % lp.step_end_mod);
   return t == lp.step_end_id;
 }
 
-// Appends the current iteration's token of every active slot to its row and stops rows whose step ended.
+// Appends the current iteration's token of every active slot to its row, stops rows whose step ended and lays out the next iteration.
 __global__ void __launch_bounds__(1024)
 decode_update_kernel(RowState st, int which, int phase, unsigned long long* best, int n_slots, LoopParams lp) {
   RSD_PDL_SYNC();
@@ -237,6 +229,8 @@ decode_update_kernel(RowState st, int which, int phase, unsigned long long* best
         st.gen_active[row] = 0;
         ended = 1;
       }
+      if (ended) st.pass_tok_row[i] = -1;        // the lists of the next iteration
+      else pass_slot(st, i, row, pos + 1, t);
     }
   }
   const int n_ended = __syncthreads_count(ended);
