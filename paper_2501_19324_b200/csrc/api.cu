@@ -565,8 +565,7 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
   const int T = p.T;
   if (T <= 0) return RSD_OK;
   const RowScale rs{c->norm_ssq, norm_chunks(d), 1.f / (float)d, m.rms_eps};
-  CU(launch_embed(m.dtype, m.tok_embed, p, c->x, d, s));
-  CU(launch_reduce_norm(nullptr, 1, c->x, M.norm1[0], c->h, c->h_lo, c->norm_ssq, T, d, p.n_active, s));
+  CU(launch_embed_norm(m.tok_embed, p, c->x, M.norm1[0], c->h, c->h_lo, c->norm_ssq, d, s));
   for (int l = 0; l < m.n_layers; ++l) {
     KvView kv{M.kv_pool + (size_t)l * M.layer_stride, c->st.page_table[which], c->max_pages, M.kv_dtype == 3 ? 1 : 0};
     SplitSum qkv_pending, gu_pending, x_pending;

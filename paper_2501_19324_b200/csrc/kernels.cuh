@@ -56,6 +56,8 @@ struct KvView {
 
 cudaError_t launch_bf16_to_f16(const void* src, void* dst, size_t n, cudaStream_t s);
 cudaError_t launch_embed(int dtype, const void* embed, PassView p, float* x, int d, cudaStream_t s);
+// ... of bf16 tokens with what launch_reduce_norm would make of them: hi + lo = x * gain, ssq [T][ceil(d / 256)].
+cudaError_t launch_embed_norm(const void* embed, PassView p, float* x, const void* gain, void* hi, void* lo, float* ssq, int d, cudaStream_t s);
 // out[t] = rmsnorm(x[t]) (and out_lo when given, bf16 only: the low half of a split-precision operand)
 cudaError_t launch_rmsnorm(int dtype, const float* x, const void* gain, void* out, void* out_lo, int T, int d, float eps,
                            const int32_t* n_active, cudaStream_t s, bool out_f16 = false);

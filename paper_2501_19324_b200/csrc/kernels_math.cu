@@ -36,6 +36,46 @@ cudaError_t launch_embed(int dtype, const void* embed, PassView p, float* x, int
   return launched(1);
 }
 
+// ... of a decode pass of a bf16 model, with the first layer's un-normalised norm operand and sums of squares (see reduce_norm_kernel):
+// one block per (token, 256-column chunk).  A launch of 1.4-1.7 us less an iteration.
+__global__ void __launch_bounds__(64)
+embed_norm_kernel(const __nv_bfloat16* __restrict__ E, PassView p, float* __restrict__ x, const __nv_bfloat16* __restrict__ gain,
+                  __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo, float* __restrict__ ssq, int d) {
+  RSD_PDL_SYNC_LATE();
+  RSD_SKIP_IF_IDLE(p.n_active);
+  __shared__ float red[2];
+  const int t = blockIdx.y, col = blockIdx.x * 256 + threadIdx.x * 4;
+  if (p.tok_row[t] < 0) return;
+  float ss = 0.f;
+  if (col < d) {
+    float v[4], y[4];
+    __align__(8) __nv_bfloat16 e[4], g[4];
+    *reinterpret_cast<uint2*>(e) = *reinterpret_cast<const uint2*>(E + (size_t)p.tok_id[t] * d + col);
+    *reinterpret_cast<uint2*>(g) = *reinterpret_cast<const uint2*>(gain + col);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      v[i] = to_f32(e[i]);
+      y[i] = v[i] * to_f32(g[i]);
+    }
+    const size_t o = (size_t)t * d + col;
+    *reinterpret_cast<float4*>(x + o) = make_float4(v[0], v[1], v[2], v[3]);
+    store_operand4<__nv_bfloat16>(hi, lo, o, y);
+    ss = v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
+  }
+  ss = warp_sum(ss);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  if (threadIdx.x == 0) ssq[(size_t)t * gridDim.x + blockIdx.x] = red[0] + red[1];
+}
+
+cudaError_t launch_embed_norm(const void* embed, PassView p, float* x, const void* gain, void* hi, void* lo, float* ssq, int d, cudaStream_t s) {
+  if (p.T <= 0) return cudaSuccess;
+  if (d % 4 != 0) return cudaErrorInvalidValue;
+  RSD_LAUNCH((embed_norm_kernel), dim3(norm_chunks(d), p.T), 64, 0, s, (const __nv_bfloat16*)embed, p, x, (const __nv_bfloat16*)gain,
+             (__nv_bfloat16*)hi, (__nv_bfloat16*)lo, ssq, d);
+  return launched(1);
+}
+
 // ---------------------------------------------------------------------------------------------
 // RMSNorm: out = x * gain / sqrt(mean(x^2) + eps), one block per token, x kept in registers
 // ---------------------------------------------------------------------------------------------
