@@ -289,7 +289,7 @@ size_t layout_workspace(const rsd_config& cfg, const rsd_model* const ms[3], rsd
   void* act = TAKE(float, (size_t)T * dm.f);
   float* logits = TAKE(float, (size_t)slots * dm.v);
   unsigned long long* sample_best = TAKE(unsigned long long, slots);
-  float* norm_ssq = TAKE(float, (size_t)slots * 2 * norm_chunks(dm.d));   // room for 128-column chunks
+  float* norm_ssq = TAKE(float, std::max((size_t)slots * 2 * norm_chunks(dm.d), (size_t)std::min(slots, 8) * (dm.d / 8)));   // room for 128-column chunks, of few rows for 8
   void* mega_block[3] = {nullptr, nullptr, nullptr};
   for (int w = 0; w < 3; w += 2) mega_block[w] = TAKE(char, mega_block_bytes(ms[w]->n_layers));
   int32_t* mega_sync = TAKE(int32_t, 1024);
@@ -554,47 +554,69 @@ int forward_pass(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
 // Decode pass of a bf16 model with RMSNorm folded into its neighbours: the kernel that completes the
 // residual stream (reduce_norm) also writes the next GEMM's operand x * gain and the sums of squares, and
 // that GEMM scales its result rows by the RMSNorm denominator; the K-split sums of the qkv product are
-// added up by the RoPE kernel.  Eight kernels a layer, seven where the attention rotates for itself.  On return h / h_lo hold
+// added up by the RoPE kernel.  Eight kernels a layer, seven where the attention rotates for itself, five to seven for few rows
+// (gemm_rows.cu).  On return h / h_lo hold
 // x * final_gain and norm_ssq the sums of squares of the final residual stream.
 bool fused_decode_ok(const ModelHost& M) { return M.m.dtype == RSD_BF16 && M.split && M.m.d_model % 4 == 0; }
 
-int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_gain, cudaStream_t s) {
+int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_gain, cudaStream_t s, RowScale* final_rs) {
   const ModelHost& M = c->mdl[which];
   const rsd_model& m = M.m;
   const int d = m.d_model, H = m.n_heads, KV = m.n_kv_heads, hd = m.head_dim, F = m.d_ffn;
   const int T = p.T;
+  // few rows: products that take the step behind them along instead of a K split
+  const bool rows_qkv = (M.kv_dtype == 2 || M.kv_dtype == 3) && rows_gemm_pays(T, (H + 2 * KV) * hd, d, false);
+  const bool rows_wo = rows_gemm_pays(T, d, H * hd, false), rows_down = rows_gemm_pays(T, d, F, true);
+  auto scale = [&](int chunks) { return RowScale{c->norm_ssq, chunks, 1.f / (float)d, m.rms_eps}; };
+  const RowScale rs_mid = scale(rows_wo ? d / 8 : norm_chunks(d)), rs_end = scale(rows_down ? d / 8 : norm_chunks(d));
+  *final_rs = rs_end;
   if (T <= 0) return RSD_OK;
-  const RowScale rs{c->norm_ssq, norm_chunks(d), 1.f / (float)d, m.rms_eps};
   CU(launch_embed_norm(m.tok_embed, p, c->x, M.norm1[0], c->h, c->h_lo, c->norm_ssq, d, s));
   for (int l = 0; l < m.n_layers; ++l) {
     KvView kv{M.kv_pool + (size_t)l * M.layer_stride, c->st.page_table[which], c->max_pages, M.kv_dtype == 3 ? 1 : 0};
-    SplitSum qkv_pending, gu_pending, x_pending;
-    int rc = gemm(c, M, M.wqkv[l], c->h, c->h_lo, c->qkv, T, (H + 2 * KV) * hd, d, 0, p.n_active, &qkv_pending, s, rs);
-    if (rc) return rc;
-    const QkvSource src{c->qkv, qkv_pending, M.rope};
-    const bool rotates = attn_decode_takes_qkv(M.kv_dtype, m.dtype, T, H, KV, c->S, c->attn_rows_hint, c->pass_width);
-    if (!rotates) CU(launch_rope_kv(M.kv_dtype, c->qkv, qkv_pending, p, c->q, kv, M.rope, H, KV, hd, s));
+    const RowScale rs = l == 0 ? scale(norm_chunks(d)) : rs_end;
+    SplitSum gu_pending, x_pending;
+    QkvSource src{c->qkv, SplitSum(), M.rope};
+    bool rotates = false;
+    int rc;
+    if (rows_qkv) {
+      CU(launch_gemm_rows_qkv(M.wqkv[l], c->h, c->h_lo, rs, p, c->q, kv, M.rope, H, KV, hd, d, s));
+    } else {
+      rc = gemm(c, M, M.wqkv[l], c->h, c->h_lo, c->qkv, T, (H + 2 * KV) * hd, d, 0, p.n_active, &src.pending, s, rs);
+      if (rc) return rc;
+      rotates = attn_decode_takes_qkv(M.kv_dtype, m.dtype, T, H, KV, c->S, c->attn_rows_hint, c->pass_width);
+      if (!rotates) CU(launch_rope_kv(M.kv_dtype, c->qkv, src.pending, p, c->q, kv, M.rope, H, KV, hd, s));
+    }
     CU(launch_attn_decode(M.kv_dtype, c->q, kv.pool_layer, kv.page_table, kv.max_pages, p.tok_row, p.tok_pos, 1,
                           c->attn, c->attn_lo, m.dtype, T, H, KV, hd, c->S, c->attn_scratch, c->attn_scratch_bytes,
                           p.n_active, s, c->attn_rows_hint, c->pass_width, rotates ? &src : nullptr));
-    rc = gemm(c, M, M.wo[l], c->attn, c->attn_lo, c->x, T, d, H * hd, 1, p.n_active, &x_pending, s);
-    if (rc) return rc;
-    CU(launch_reduce_norm(x_pending.partials, x_pending.splits, c->x, M.norm2[l], c->h, c->h_lo, c->norm_ssq, T, d,
-                          p.n_active, s));
+    if (rows_wo) {
+      CU(launch_gemm_rows_residual(M.wo[l], c->attn, c->attn_lo, c->x, M.norm2[l], c->h, c->h_lo, c->norm_ssq, T, d, H * hd,
+                                   p.n_active, s));
+    } else {
+      rc = gemm(c, M, M.wo[l], c->attn, c->attn_lo, c->x, T, d, H * hd, 1, p.n_active, &x_pending, s);
+      if (rc) return rc;
+      CU(launch_reduce_norm(x_pending.partials, x_pending.splits, c->x, M.norm2[l], c->h, c->h_lo, c->norm_ssq, T, d,
+                            p.n_active, s));
+    }
     if (gu_fused_ok(M, T)) {
-      rc = gemm_gu(c, M, M.wgu[l], c->h, c->h_lo, c->act, c->act_lo, T, F, d, p.n_active, s, rs);
+      rc = gemm_gu(c, M, M.wgu[l], c->h, c->h_lo, c->act, c->act_lo, T, F, d, p.n_active, s, rs_mid);
       if (rc) return rc;
     } else {
-      rc = gemm(c, M, M.wgu[l], c->h, c->h_lo, c->gu, T, 2 * F, d, 0, p.n_active, &gu_pending, s, rs);
+      rc = gemm(c, M, M.wgu[l], c->h, c->h_lo, c->gu, T, 2 * F, d, 0, p.n_active, &gu_pending, s, rs_mid);
       if (rc) return rc;
       CU(launch_swiglu(m.dtype, c->gu, gu_pending, c->act, c->act_lo, T, F, p.n_active, s));
     }
-    x_pending = SplitSum();
-    rc = gemm(c, M, M.wdown[l], c->act, c->act_lo, c->x, T, d, F, 1, p.n_active, &x_pending, s);
-    if (rc) return rc;
     const void* next_gain = l + 1 < m.n_layers ? M.norm1[l + 1] : final_gain;
-    CU(launch_reduce_norm(x_pending.partials, x_pending.splits, c->x, next_gain, c->h, c->h_lo, c->norm_ssq, T, d,
-                          p.n_active, s));
+    if (rows_down) {
+      CU(launch_gemm_rows_residual(M.wdown[l], c->act, c->act_lo, c->x, next_gain, c->h, c->h_lo, c->norm_ssq, T, d, F, p.n_active, s));
+    } else {
+      x_pending = SplitSum();
+      rc = gemm(c, M, M.wdown[l], c->act, c->act_lo, c->x, T, d, F, 1, p.n_active, &x_pending, s);
+      if (rc) return rc;
+      CU(launch_reduce_norm(x_pending.partials, x_pending.splits, c->x, next_gain, c->h, c->h_lo, c->norm_ssq, T, d,
+                            p.n_active, s));
+    }
   }
   return RSD_OK;
 }
@@ -727,8 +749,8 @@ int model_logits(rsd_ctx* c, int which, PassView p, bool allow_mega, cudaStream_
     const RowScale rs{c->norm_ssq, m.d_model / 128, 1.f / (float)m.d_model, m.rms_eps};
     rc = gemm(c, M, m.head, c->h, c->h_lo, c->logits, T, m.vocab, m.d_model, 0, p.n_active, nullptr, s, rs);
   } else if (fused_decode_ok(M)) {
-    if ((rc = forward_decode_fused(c, which, p, m.final_norm, s))) return rc;
-    const RowScale rs{c->norm_ssq, norm_chunks(m.d_model), 1.f / (float)m.d_model, m.rms_eps};
+    RowScale rs;
+    if ((rc = forward_decode_fused(c, which, p, m.final_norm, s, &rs))) return rc;
     rc = gemm(c, M, m.head, c->h, c->h_lo, c->logits, T, m.vocab, m.d_model, 0, p.n_active, nullptr, s, rs);
   } else if (decode_f32_ok(c, M, p)) {
     if ((rc = forward_decode_f32(c, which, p, s))) return rc;
@@ -1200,7 +1222,8 @@ static int score_with_draft_trunk(rsd_ctx* c, cudaStream_t s) {
   int rc;
   const bool was_in_decode = c->in_decode;
   c->in_decode = true;             // GEMM timing: treated like a decode iteration that is not sampled
-  if (fused_decode_ok(D)) rc = forward_decode_fused(c, RSD_DRAFT, p, prm.final_norm, s);
+  RowScale rs;
+  if (fused_decode_ok(D)) rc = forward_decode_fused(c, RSD_DRAFT, p, prm.final_norm, s, &rs);
   else if (decode_f32_ok(c, D, p)) rc = forward_decode_f32(c, RSD_DRAFT, p, s);
   else rc = forward_pass(c, RSD_DRAFT, p, s);
   c->in_decode = was_in_decode;

@@ -238,19 +238,31 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
     // ---------------- epilogue: TMEM -> registers -> global ----------------
     RSD_PDL_WAIT();                            // y and the partial sums belong to earlier kernels until now
     if (rs.ssq != nullptr && active != 0) {
-      // RMSNorm denominators of this tile's x rows while the MMAs run: 128 / kRows threads per row, so that a row's
-      // chunk sums are one round of loads, or two, instead of a chain as long as the row is wide
-      constexpr int kLanes = kRows >= 128 ? 1 : (kRows >= 8 ? 128 / kRows : 16);
-      const int r = threadIdx.x / kLanes, sub = threadIdx.x % kLanes;
-      float sum = 0.f;
-      if (r < kRows && m0 + r < M) {
-        const float* src = rs.ssq + (size_t)(m0 + r) * rs.n_chunks;
+      if (rs.n_chunks > 32) {
+        // few rows in many chunks (gemm_rows.cu): a warp per row
+        for (int r = warp; r < kRows && m0 + r < M; r += 4) {
+          const float* src = rs.ssq + (size_t)(m0 + r) * rs.n_chunks;
+          float sum = 0.f;
 #pragma unroll 8
-        for (int c = sub; c < rs.n_chunks; c += kLanes) sum += src[c];
-      }
+          for (int c = lane; c < rs.n_chunks; c += 32) sum += src[c];
+          sum = warp_sum(sum);
+          if (lane == 0) row_scale[r] = rsqrtf(sum * rs.inv_d + rs.eps);
+        }
+      } else {
+        // RMSNorm denominators of this tile's x rows while the MMAs run: 128 / kRows threads per row, so that a row's
+        // chunk sums are one round of loads, or two, instead of a chain as long as the row is wide
+        constexpr int kLanes = kRows >= 128 ? 1 : (kRows >= 8 ? 128 / kRows : 16);
+        const int r = threadIdx.x / kLanes, sub = threadIdx.x % kLanes;
+        float sum = 0.f;
+        if (r < kRows && m0 + r < M) {
+          const float* src = rs.ssq + (size_t)(m0 + r) * rs.n_chunks;
+#pragma unroll 8
+          for (int c = sub; c < rs.n_chunks; c += kLanes) sum += src[c];
+        }
 #pragma unroll
-      for (int o = kLanes / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-      if (sub == 0 && r < kRows) row_scale[r] = rsqrtf(sum * rs.inv_d + rs.eps);
+        for (int o = kLanes / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+        if (sub == 0 && r < kRows) row_scale[r] = rsqrtf(sum * rs.inv_d + rs.eps);
+      }
       asm volatile("bar.sync 1, 128;" ::: "memory");   // the four epilogue warps only
     }
     // the four epilogue warps sleep in hardware between polls (about 1 us at most): busy polling by 128 threads

@@ -104,6 +104,15 @@ cudaError_t launch_gemm(int dtype, const void* W, const void* x, const void* x_l
 cudaError_t launch_reduce_norm(const float* partials, int splits, float* x, const void* gain, void* hi, void* lo,
                                float* ssq, int M, int d, const int32_t* n_active, cudaStream_t s);
 inline int norm_chunks(int d) { return (d + 255) / 256; }
+// Decode products of up to eight rows of hi + lo operands together with the small step behind them (gemm_rows.cu):
+// x += in W^T, hi + lo = x * gain, ssq [M][d / 8] as launch_reduce_norm's, per eight columns ...
+bool rows_gemm_supported(int M, int N, int K);
+bool rows_gemm_pays(int M, int N, int K, bool long_k);   // faster than a K split and its launch; long_k: the down projection
+cudaError_t launch_gemm_rows_residual(const void* W, const void* in, const void* in_lo, float* x, const void* gain, void* hi, void* lo,
+                                      float* ssq, int M, int d, int K, const int32_t* n_active, cudaStream_t s);
+// ... and qkv = rowscale * in W^T, rotated and written as by launch_rope_kv (fp16 cache).
+cudaError_t launch_gemm_rows_qkv(const void* W, const void* in, const void* in_lo, RowScale rs, PassView p, float* q_out, KvView kv,
+                                 const float2* rope, int H, int KV, int hd, int K, cudaStream_t s);
 cudaError_t launch_rope_table(float2* table, int n_pos, int hd, float theta, cudaStream_t s);
 // Splits qkv [T, (H+2KV)*hd] (fp32): rotated q -> q_out [T, H*hd] fp32; rotated k and v -> KV pages.
 // kv_dtype: element type of the cache: 0 fp32, 1 bf16, 2 fp16.

@@ -468,6 +468,23 @@ def test_decode_attention_that_takes_the_qkv_product(d, H, KV, hd, ext):
     eng.close()
 
 
+@pytest.mark.parametrize("d,H,KV,hd,F,rows,ext", [(64, 1, 1, 64, 64, 1, 0), (576, 7, 1, 128, 448, 8, 0), (576, 7, 1, 128, 448, 9, 0), (512, 4, 2, 64, 1408, 5, 1),
+                                                  (1536, 12, 2, 128, 1024, 4, 0), (1536, 12, 2, 128, 1024, 6, 0), (512, 8, 8, 128, 520, 2, 1)])
+def test_decode_products_of_few_rows(d, H, KV, hd, F, rows, ext):
+    """bf16 decode passes of one to eight rows and one more, products with their next step and (wide shapes, more rows; K off a multiple of
+    64) K splits side by side: sums of squares per 8 and per 256 columns, one chunk of K a warp and several, both head sizes,
+    both caches, a new token on the first and last place of a page."""
+    sh = ri.ModelShape(2, d, H, KV, hd, F, 1024)
+    prompts = ri.prompts(11 + d, rows, 14, 18, sh.vocab)
+    kw = dict(max_step_tokens=6, max_steps=2, max_seq_tokens=48, step_end_id=3, step_end_mod=7, temperature=0.7, seed=4)
+    eng, loop = build_pair((sh, sh, sh), bf16=True, prompts=prompts, loop_kwargs=kw, engine_kwargs=dict(kv_extended=ext))
+    stats = {}
+    for _ in range(2):
+        parity_step(eng, loop, 2.0, stats=stats, **TOL16)      # every row is rejected: draft and target decode
+    assert stats["tokens_compared"] > 0.4 * stats["tokens"]
+    eng.close()
+
+
 @pytest.mark.parametrize("d,H,KV,hd,rows,lo,hi", [(64, 1, 1, 64, 3, 13, 18), (260, 4, 2, 128, 9, 14, 33), (128, 10, 1, 64, 5, 252, 262)])
 def test_fp32_decode_with_the_small_steps_inside_the_products(d, H, KV, hd, rows, lo, hi):
     """fp32 decode passes: norms and SwiGLU in the products, rotation and page write in the attention; one head group and groups of
