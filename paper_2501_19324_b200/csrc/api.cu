@@ -468,7 +468,7 @@ int gemm_f16(rsd_ctx* c, const void* W16, const void* x16, float* y, int Mrows, 
 // The layer stack of a pass of more than 128 tokens on the fp16 copies of the weights: every GEMM operand (normed
 // residual, attention output, SwiGLU output) is written once, as fp16, by the kernel that produces it.  x holds the
 // embedded tokens on entry and the last layer's residual stream on exit, as in forward_pass.
-int forward_pass_f16(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
+int forward_pass_f16(rsd_ctx* c, int which, PassView p, bool cache_only, cudaStream_t s) {
   const ModelHost& M = c->mdl[which];
   const rsd_model& m = M.m;
   const int d = m.d_model, H = m.n_heads, KV = m.n_kv_heads, hd = m.head_dim, F = m.d_ffn;
@@ -479,6 +479,7 @@ int forward_pass_f16(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
     int rc = gemm_f16(c, M.w16_of(l, 0), c->h, c->qkv, T, (H + 2 * KV) * hd, d, 0, s);
     if (rc) return rc;
     CU(launch_rope_kv(M.kv_dtype, c->qkv, SplitSum(), p, c->q, kv, M.rope, H, KV, hd, s));
+    if (cache_only && l + 1 == m.n_layers) break;
     CU(launch_attn_chunk(M.kv_dtype, c->q, p, kv, c->attn, nullptr, 2, H, KV, hd, s, (int*)((char*)c->gemm_scratch + 4096)));
     rc = gemm_f16(c, M.w16_of(l, 1), c->attn, c->x, T, d, H * hd, 1, s);
     if (rc) return rc;
@@ -501,7 +502,9 @@ int forward_pass_f16(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
   return RSD_OK;
 }
 
-int forward_pass(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
+// cache_only: the pass is run for its keys and values alone; the last layer ends with them (what follows them there, the residual
+// stream, nobody reads: a 28th of such a pass, a 14th at half depth).
+int forward_pass(rsd_ctx* c, int which, PassView p, cudaStream_t s, bool cache_only = false) {
   const ModelHost& M = c->mdl[which];
   const rsd_model& m = M.m;
   const int d = m.d_model, H = m.n_heads, KV = m.n_kv_heads, hd = m.head_dim, F = m.d_ffn;
@@ -510,7 +513,7 @@ int forward_pass(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
   CU(launch_embed(m.dtype, m.tok_embed, p, c->x, d, s));
   // dense pass of a model with fp16 weight copies: one fp16 activation operand, no low halves
   const bool f16 = M.f16_dense && p.n_active == nullptr && T > 128 && gemm_gu_supported(1, T, F, d);
-  if (f16) return forward_pass_f16(c, which, p, s);
+  if (f16) return forward_pass_f16(c, which, p, cache_only, s);
   void* h_lo = M.split ? c->h_lo : nullptr;
   void* attn_lo = M.split ? c->attn_lo : nullptr;
   void* act_lo = M.split ? c->act_lo : nullptr;
@@ -522,6 +525,7 @@ int forward_pass(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
     int rc = gemm(c, M, M.wqkv[l], c->h, h_lo, c->qkv, T, (H + 2 * KV) * hd, d, 0, p.n_active, nullptr, s);
     if (rc) return rc;
     CU(launch_rope_kv(M.kv_dtype, c->qkv, SplitSum(), p, c->q, kv, M.rope, H, KV, hd, s));
+    if (cache_only && l + 1 == m.n_layers) break;
     if (p.n_active != nullptr) {
       // decode pass: one query per row slot
       CU(launch_attn_decode(M.kv_dtype, c->q, kv.pool_layer, kv.page_table, kv.max_pages, p.tok_row, p.tok_pos, 1,
@@ -653,7 +657,7 @@ int run_ingest(rsd_ctx* c, int which, int n_total, int rows, bool want_reward, c
     const int Tc = std::min(c->chunk, n_total - c0);
     PassView p{c->st.pass_tok_id + c0, c->st.pass_tok_row + c0, c->st.pass_tok_pos + c0, Tc, nullptr,
                (int)(((long)rows * Tc + n_total - 1) / n_total)};
-    int rc = forward_pass(c, which, p, s);
+    int rc = forward_pass(c, which, p, s, !want_reward);
     if (rc) return rc;
     if (want_reward) {
       const rsd_model& m = c->mdl[which].m;
