@@ -1,6 +1,6 @@
 // Paged-KV grouped-query decode attention (one query token per row), sm_100a.
 //
-// A CTA of 4 warps serves one (row slot, KV head, context split): the G = H / KV query heads that
+// A CTA of 4 warps (16 in one form) serves one (row slot, KV head, context split): the G = H / KV query heads that
 // share the KV head are the rows of a 16-row MMA tile, so every key / value is read once from HBM for
 // the whole group.  Each warp walks its share of the 16-token pages through a ring of page buffers of its own in shared
 // memory (16-byte cp.async, a page ahead):
@@ -78,13 +78,14 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
 
-// Shared memory of a CTA: 4 warps x kStages page buffers; the warps' outputs take its place after the loop.  An extended
-// page (16 KB) gets one buffer a warp, a plain one (8 KB) two, so that three CTAs fit an SM either way.
-template <int HD, bool EXT> struct DecCfg {
+// Shared memory of a CTA: NW warps x kStages page buffers; the warps' outputs take its place after the loop.  An extended
+// page (16 KB) gets one buffer a warp, a plain one (8 KB) two, so that three CTAs of four warps fit an SM either way; of sixteen warps
+// one buffer each, one CTA an SM.
+template <int HD, bool EXT, int NW> struct DecCfg {
   static constexpr int kPageBytes = (EXT ? 4 : 2) * kPageTokens * HD * 2;
-  static constexpr int kStages = EXT ? 1 : 2;
-  static constexpr int kRingBytes = 4 * kStages * kPageBytes;
-  static_assert(kRingBytes >= 4 * 8 * (HD + 8) * 4, "the outputs of the four warps alias the ring");
+  static constexpr int kStages = EXT || NW > 4 ? 1 : 2;
+  static constexpr int kOutBytes = NW * 8 * (HD + 8) * 4;
+  static constexpr int kRingBytes = NW * kStages * kPageBytes > kOutBytes ? NW * kStages * kPageBytes : kOutBytes;
 };
 
 // part_o: [slot][head][split][HD] un-normalised outputs; part_ml: [slot][head][split][2] (max, sum).
@@ -93,20 +94,22 @@ template <int HD, bool EXT> struct DecCfg {
 // new_tokens: how many of a row's last positions the pass itself writes.
 // FUSE (one split; every row's only new position is its last): the kernel takes the qkv product itself, K-split partial sums or
 // not, adds them up, rotates, and writes the new key and value to the cache: see new_token below.
-template <int HD, typename KT, typename OT, bool EXT, bool CL, bool FUSE>
-__global__ void __launch_bounds__(128, 3)
+// NW: warps, 4, or 16 where there is one CTA per SM at most (wide_ctas).
+template <int HD, typename KT, typename OT, bool EXT, bool CL, bool FUSE, int NW>
+__global__ void __launch_bounds__(32 * NW, NW == 4 ? 3 : 1)
 attn_decode_kernel(const float* q, KT* pool, const int32_t* page_table, int max_pages, const int32_t* slot_row,
                    const int32_t* len_or_pos, int len_offset, OT* out, OT* out_lo, float* part_o, float* part_ml, int H, int KV,
                    int n_splits, const int32_t* n_active, int new_tokens, const float* partials, int k_splits, const float2* rope) {
   RSD_PDL_TRIGGER();
   if (n_active == nullptr) RSD_PDL_WAIT();   // a decode pass's lists and old pages may be read ahead of the wait, others not
-  using Cfg = DecCfg<HD, EXT>;
+  using Cfg = DecCfg<HD, EXT, NW>;
+  constexpr int kThreads = 32 * NW;
   constexpr int KB = HD / 32;    // 32-dim blocks of the head dimension
   constexpr int NT = HD / 8;     // 8-dim output tiles
   constexpr int kBlock = kPageTokens * HD;       // elements of one head's keys (or values) in a page
   constexpr int kStages = Cfg::kStages, kParts = EXT ? 4 : 2;
   extern __shared__ __align__(128) uint8_t ring_raw[];
-  __shared__ float s_m[4][8], s_l[4][8];
+  __shared__ float s_m[NW][8], s_l[NW][8];
   auto s_o = reinterpret_cast<float(*)[8][HD + 8]>(ring_raw);   // rows 32 bytes apart modulo 128: the fragments' stores do not collide
   const int kvh = blockIdx.x, slot = blockIdx.y, split = blockIdx.z;
   const bool idle = n_active != nullptr && ld_cg(n_active) == 0;
@@ -147,7 +150,7 @@ attn_decode_kernel(const float* q, KT* pool, const int32_t* page_table, int max_
   auto fetch_next = [&](int stage) {
     if (next < p_end) {
       fetch(next_id, stage);
-      next += 4;
+      next += NW;
       if (next < p_end) next_id = ld_cg(pt + next);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -166,17 +169,19 @@ attn_decode_kernel(const float* q, KT* pool, const int32_t* page_table, int max_
   __shared__ __align__(16) KT s_new[FUSE ? kParts : 1][HD];   // the new token's key and value (and their low halves)
   const int new_page = (ctx - 1) / kPageTokens, new_slot = (ctx - 1) % kPageTokens;
   if (FUSE) {
-    // new_token.  A task is four neighbouring pairs (i, i + HD / 2) of a query head, of the key or of the value, with all
-    // its K splits in flight at once.
-    constexpr int NQ = HD / 8, kAhead = 3;
+    // new_token.  A task is four neighbouring pairs (i, i + HD / 2) of a query head, of the key or of the value; P lanes of a warp
+    // share its K splits, all of them in flight at once.
+    constexpr int NQ = HD / 8, kAhead = 3, P = NW == 16 ? 2 : 1, R = kSumGroups / P, kPerWarp = 32 / P;
     const int n_tasks = (G + 2) * NQ, width = (H + 2 * KV) * HD;
     const size_t sstride = (size_t)gridDim.y * width;
     const int per = (k_splits + kSumGroups - 1) / kSumGroups;
-    for (int idx = threadIdx.x; idx < (8 - G) * HD; idx += 128) {   // the tile's rows beyond the group
+    for (int idx = threadIdx.x; idx < (8 - G) * HD; idx += kThreads) {   // the tile's rows beyond the group
       s_q[0][G + idx / HD][idx % HD] = from_f32<KT>(0.f);
       if (EXT) s_q[EXT ? 1 : 0][G + idx / HD][idx % HD] = from_f32<KT>(0.f);
     }
-    for (int task = threadIdx.x; task < n_tasks; task += 128) {
+    const int part = lane / kPerWarp;              // of the K splits: runs [part R, part R + R)
+    for (int task0 = warp * kPerWarp; task0 < n_tasks; task0 += NW * kPerWarp) {
+      const int task = min(task0 + lane % kPerWarp, n_tasks - 1);          // whole warps: lanes beyond the last task repeat it
       const bool is_q = task < G * NQ;
       const int hh = is_q ? task / NQ : task / NQ - G, dd = 4 * (task % NQ);   // one of the group's heads, or 0 = the key, 1 = the value
       const size_t src = (size_t)slot * width + (size_t)(is_q ? h0 + hh : H + hh * KV + kvh) * HD + dd;
@@ -186,37 +191,46 @@ attn_decode_kernel(const float* q, KT* pool, const int32_t* page_table, int max_
         *reinterpret_cast<float4*>(b) = ld_cg(reinterpret_cast<const float4*>(q + src + HD / 2));
       } else {
         // the order of the additions is rope_kv_kernel's: kSumGroups runs of splits, then their sums
-        float ga[kSumGroups][4], gb[kSumGroups][4];
+        float ga[R][4], gb[R][4];
 #pragma unroll
-        for (int r = 0; r < kSumGroups; ++r)
+        for (int r = 0; r < R; ++r)
 #pragma unroll
           for (int i = 0; i < 4; ++i) ga[r][i] = gb[r][i] = 0.f;
         for (int s0 = 0; s0 < per; s0 += kAhead) {
-          float4 ta[kSumGroups][kAhead], tb[kSumGroups][kAhead];
+          float4 ta[R][kAhead], tb[R][kAhead];
 #pragma unroll
-          for (int r = 0; r < kSumGroups; ++r)
+          for (int r = 0; r < R; ++r)
 #pragma unroll
             for (int u = 0; u < kAhead; ++u)
-              if (s0 + u < per && r * per + s0 + u < k_splits) {
-                const float* at = partials + (size_t)(r * per + s0 + u) * sstride + src;
+              if (s0 + u < per && (part * R + r) * per + s0 + u < k_splits) {
+                const float* at = partials + (size_t)((part * R + r) * per + s0 + u) * sstride + src;
                 ta[r][u] = ld_cg(reinterpret_cast<const float4*>(at));
                 tb[r][u] = ld_cg(reinterpret_cast<const float4*>(at + HD / 2));
               }
 #pragma unroll
-          for (int r = 0; r < kSumGroups; ++r)
+          for (int r = 0; r < R; ++r)
 #pragma unroll
             for (int u = 0; u < kAhead; ++u)
-              if (s0 + u < per && r * per + s0 + u < k_splits) {
+              if (s0 + u < per && (part * R + r) * per + s0 + u < k_splits) {
                 ga[r][0] += ta[r][u].x; ga[r][1] += ta[r][u].y; ga[r][2] += ta[r][u].z; ga[r][3] += ta[r][u].w;
                 gb[r][0] += tb[r][u].x; gb[r][1] += tb[r][u].y; gb[r][2] += tb[r][u].z; gb[r][3] += tb[r][u].w;
               }
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          a[i] = ((ga[0][i] + ga[1][i]) + ga[2][i]) + ga[3][i];
-          b[i] = ((gb[0][i] + gb[1][i]) + gb[2][i]) + gb[3][i];
+          a[i] = ga[0][i]; b[i] = gb[0][i];
+#pragma unroll
+          for (int r = 1; r < R; ++r) { a[i] += ga[r][i]; b[i] += gb[r][i]; }
+          if (P == 2) {                            // the other lane's runs, one after the other
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              a[i] += __shfl_down_sync(0xFFFFFFFFu, ga[r][i], kPerWarp & 31);
+              b[i] += __shfl_down_sync(0xFFFFFFFFu, gb[r][i], kPerWarp & 31);
+            }
+          }
         }
       }
+      if (part > 0 || task0 + lane >= n_tasks) continue;
       if (is_q || hh == 0) {
         const float2* cs = rope + (size_t)(ctx - 1) * (HD / 2) + dd;
 #pragma unroll
@@ -259,8 +273,8 @@ attn_decode_kernel(const float* q, KT* pool, const int32_t* page_table, int max_
     }
   } else {
 #pragma unroll
-    for (int i = 0; i < 8 * HD / 128; ++i) {     // one coalesced round of loads
-      const int idx = i * 128 + threadIdx.x, gg = idx / HD, dd = idx % HD;
+    for (int i = 0; i < 8 * HD / kThreads; ++i) {     // one coalesced round of loads
+      const int idx = i * kThreads + threadIdx.x, gg = idx / HD, dd = idx % HD;
       const float v = gg < G ? q[((size_t)slot * H + h0 + gg) * HD + dd] : 0.f;
       const KT hi = from_f32<KT>(v);
       s_q[0][gg][dd] = hi;
@@ -284,7 +298,7 @@ attn_decode_kernel(const float* q, KT* pool, const int32_t* page_table, int max_
   const int key_off = ((t ^ ((g & 1) << 2))) * 8;
 
   int stage = 0;
-  for (int p = first; p < p_end; p += 4) {
+  for (int p = first; p < p_end; p += NW) {
     asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 1) : "memory");
     __syncwarp();
     KT* kb = ring + stage * kParts * kBlock;
@@ -382,13 +396,15 @@ attn_decode_kernel(const float* q, KT* pool, const int32_t* page_table, int max_
   const int per = 4 * ((total / 4 + n_rank - 1) / n_rank);
   if (CL) cg::this_cluster().barrier_wait();
   __syncthreads();
-  for (int idx = 4 * threadIdx.x; idx < total; idx += 4 * 128) {
+  for (int idx = 4 * threadIdx.x; idx < total; idx += 4 * kThreads) {
     const int gg = idx / HD, dd = idx % HD;
-    const float M = fmaxf(fmaxf(s_m[0][gg], s_m[1][gg]), fmaxf(s_m[2][gg], s_m[3][gg]));
+    float M = s_m[0][gg];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) M = fmaxf(M, s_m[w][gg]);
     float L = 0.f, O[4] = {0.f, 0.f, 0.f, 0.f};
     if (M > -INFINITY) {
 #pragma unroll
-      for (int w = 0; w < 4; ++w) {
+      for (int w = 0; w < NW; ++w) {
         const float e = __expf(s_m[w][gg] - M);
         const float4 v = *reinterpret_cast<const float4*>(&s_o[w][gg][dd]);
         L += s_l[w][gg] * e;
@@ -415,7 +431,7 @@ attn_decode_kernel(const float* q, KT* pool, const int32_t* page_table, int max_
     // and none touches another's shared memory after the barrier.
     cg::this_cluster().sync();
     const int idx = split * per + threadIdx.x, end = min(total, (split + 1) * per);
-    for (int k = idx; k < end; k += 128) {
+    for (int k = idx; k < end; k += kThreads) {
       const int gg = k / HD, dd = k % HD;
       float2 ml[kClusterSplits];
       float M = -INFINITY, L = 0.f, O = 0.f;
@@ -501,10 +517,10 @@ int pick_splits(int B, int KV, int max_ctx) {
 
 // Launch with programmatic stream serialisation and, when cluster_z > 1, clusters of cluster_z CTAs along z.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_decode(void (*kernel)(KArgs...), dim3 grid, int cluster_z, int smem, cudaStream_t s, Args&&... args) {
+cudaError_t launch_decode(void (*kernel)(KArgs...), dim3 grid, int threads, int cluster_z, int smem, cudaStream_t s, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(128);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
@@ -528,12 +544,22 @@ size_t attn_decode_scratch_bytes(int B, int H, int hd, int max_ctx) {
   return sizeof(int32_t) * 2 * (size_t)B + 256 + partials;
 }
 
+// Whether a pass that takes the qkv product runs one CTA of sixteen warps per (slot, KV head): 97 to 148 of them, one per SM and no cluster,
+// and few enough pages that a warp walks four at most.  14-layer iterations, us, split contexts with a rotation kernel ahead / so:
+// 64 rows, 12 / 2 heads, 256 cached tokens 849 / 773, 500 tokens 844 / 805; 32 rows, 28 / 4 heads 1631 / 1598 and 1748 / 1725; with
+// fewer (slot, KV head) pairs nothing or a loss (32 rows, 12 / 2 heads, 500 tokens 688 / 703), with more, four warps are better (64 rows, 28 / 4
+// heads 1951 / 2031).
+static bool wide_ctas(int kv_dtype, int rows, int KV, int max_ctx) {
+  return kv_dtype == 2 && rows * KV > 96 && rows * KV <= 148 && max_ctx <= 64 * kPageTokens;
+}
+
 bool attn_decode_takes_qkv(int kv_dtype, int out_dtype, int B, int H, int KV, int max_ctx, int active_rows, int new_tokens) {
   // With the context split over a cluster every CTA would add up the query for itself, or wait for its share from the
   // others: a rotation kernel ahead is faster there (iteration of 14 layers, 12 / 2 heads: 525 us at one row and 739 at 32
   // against 583 and 794; at 128 rows, in one split, 1275 with the rotation kernel and 1206 without).
+  const int rows = active_rows > 0 ? std::min(active_rows, B) : B;
   return kv_dtype >= 2 && H / KV <= 8 && out_dtype == 1 && new_tokens == 1 &&
-         pick_splits(active_rows > 0 ? std::min(active_rows, B) : B, KV, max_ctx) == 1;
+         (wide_ctas(kv_dtype, rows, KV, max_ctx) || pick_splits(rows, KV, max_ctx) == 1);
 }
 
 cudaError_t launch_attn_decode(int kv_dtype, const float* q, const void* pool_layer, const int32_t* page_table,
@@ -561,30 +587,34 @@ cudaError_t launch_attn_decode(int kv_dtype, const float* q, const void* pool_la
   const size_t head = ((sizeof(int32_t) * 2 * (size_t)B + 255) / 256) * 256;
   float* part_ml = (float*)((char*)scratch + head);
   float* part_o = part_ml + (size_t)B * H * kMaxSplits * 2;
-  const int splits = pick_splits(active_rows > 0 ? std::min(active_rows, B) : B, KV, max_ctx);
+  const int rows = active_rows > 0 ? std::min(active_rows, B) : B;
+  const bool wide = qkv != nullptr && wide_ctas(kv_dtype, rows, KV, max_ctx);
+  const int splits = wide ? 1 : pick_splits(rows, KV, max_ctx);
   const bool clustered = splits >= 2 && splits <= kClusterSplits;
   dim3 grid(KV, B, splits);
-#define RSD_DEC_K(HD, KT, OT, EXTV, CLV, FUSEV)                                                                        \
+#define RSD_DEC_K(HD, KT, OT, EXTV, CLV, FUSEV, NW)                                                                    \
   do {                                                                                                               \
     static OncePerDevice configured_;                                                                                \
-    const cudaError_t set_ = allow_smem(configured_, attn_decode_kernel<HD, KT, OT, EXTV, CLV, FUSEV>, DecCfg<HD, EXTV>::kRingBytes); \
+    constexpr int smem_ = DecCfg<HD, EXTV, NW>::kRingBytes;                                                          \
+    const cudaError_t set_ = allow_smem(configured_, attn_decode_kernel<HD, KT, OT, EXTV, CLV, FUSEV, NW>, smem_);    \
     if (set_ != cudaSuccess) return set_;                                                                            \
-    (void)launch_decode(attn_decode_kernel<HD, KT, OT, EXTV, CLV, FUSEV>, grid, clustered ? splits : 1, DecCfg<HD, EXTV>::kRingBytes, s, \
+    (void)launch_decode(attn_decode_kernel<HD, KT, OT, EXTV, CLV, FUSEV, NW>, grid, 32 * NW, clustered ? splits : 1, smem_, s, \
                         FUSEV ? qkv->qkv : q, (KT*)pool_layer, page_table, max_pages, slot_row, len_or_pos, len_offset, (OT*)out, \
                         (OT*)out_lo, part_o, part_ml, H, KV, splits, n_active, new_tokens, FUSEV ? qkv->pending.partials : nullptr, \
                         FUSEV ? qkv->pending.splits : 1, FUSEV ? qkv->rope : nullptr);                               \
   } while (0)
 #define RSD_DEC(HD, KT, OT, EXTV, FUSEV)                                                                              \
   do {                                                                                                               \
-    if (clustered) RSD_DEC_K(HD, KT, OT, EXTV, true, false);                                                          \
-    else RSD_DEC_K(HD, KT, OT, EXTV, false, FUSEV);                                                                   \
+    if (clustered) RSD_DEC_K(HD, KT, OT, EXTV, true, false, 4);                                                       \
+    else RSD_DEC_K(HD, KT, OT, EXTV, false, FUSEV, 4);                                                                \
     if (splits > 1 && !clustered)                                                                                    \
       RSD_LAUNCH((attn_merge_kernel<HD, OT>), dim3(H, B), HD, 0, s, part_o, part_ml, slot_row, len_or_pos, len_offset, (OT*)out, \
                                                           (OT*)out_lo, H, splits, n_active);                         \
   } while (0)
 #define RSD_DEC_O(HD, KT, EXTV)                                                                                       \
   do {                                                                                                               \
-    if (qkv != nullptr) RSD_DEC(HD, KT, __nv_bfloat16, EXTV, true);                                                   \
+    if (wide && !EXTV) RSD_DEC_K(HD, KT, __nv_bfloat16, false, false, true, 16);                                      \
+    else if (qkv != nullptr) RSD_DEC(HD, KT, __nv_bfloat16, EXTV, true);                                              \
     else if (out_dtype == 1) RSD_DEC(HD, KT, __nv_bfloat16, EXTV, false);                                             \
     else RSD_DEC(HD, KT, float, EXTV, false);                                                                         \
   } while (0)

@@ -501,6 +501,20 @@ def test_fp32_decode_with_the_small_steps_inside_the_products(d, H, KV, hd, rows
     eng.close()
 
 
+@pytest.mark.parametrize("rows,H,KV,hd,lo,hi", [(97, 1, 1, 64, 3, 18), (37, 16, 4, 128, 12, 33), (74, 14, 2, 128, 12, 20), (100, 8, 1, 128, 250, 262)])
+def test_decode_attention_of_sixteen_warps(rows, H, KV, hd, lo, hi):
+    """97 to 148 (slot, KV head) pairs: one CTA of sixteen warps each takes the qkv product; groups of one to eight heads, both head
+    sizes, fewer pages than warps and more."""
+    sh = ri.ModelShape(2, 512, H, KV, hd, 512, 1024)
+    prompts = ri.prompts(29 + H, rows, lo, hi, sh.vocab)
+    kw = dict(max_step_tokens=4, max_steps=1, max_seq_tokens=hi + 8, step_end_id=3, step_end_mod=7, temperature=0.7, seed=4)
+    eng, loop = build_pair((sh, sh, sh), bf16=True, prompts=prompts, loop_kwargs=kw)
+    stats = {}
+    parity_step(eng, loop, 2.0, stats=stats, **TOL16)          # every row is rejected: draft and target decode
+    assert stats["tokens_compared"] > 0.4 * stats["tokens"]
+    eng.close()
+
+
 def _engine(prompts, **kw):
     from paper_2501_19324_b200 import Engine, Model
     heads = (ri.HEAD_LM, ri.HEAD_REWARD_SIGMOID, ri.HEAD_LM)
