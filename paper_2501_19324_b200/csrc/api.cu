@@ -425,6 +425,22 @@ int gemm(rsd_ctx* c, const ModelHost& M, const void* W, const void* xin, const v
   return RSD_OK;
 }
 
+// A decode product that takes a neighbouring step along, timed like gemm(); bytes: its weights, input and output once.
+template <typename Launch> int timed_product(rsd_ctx* c, double bytes, cudaStream_t s, Launch launch) {
+  const bool pick = c->in_decode ? c->time_this_iter
+                                 : (c->time_stride > 0 && (c->gemm_calls++ % (uint64_t)c->time_stride) == 0);
+  const bool timed = pick && c->ev_used < c->ev_bytes.size();
+  if (timed) CU(cudaEventRecord(c->ev[2 * c->ev_used], s));
+  CU(launch());
+  if (timed) {
+    CU(cudaEventRecord(c->ev[2 * c->ev_used + 1], s));
+    c->ev_bytes[c->ev_used] = bytes;
+    c->ev_flops[c->ev_used] = 0.0;
+    ++c->ev_used;
+  }
+  return RSD_OK;
+}
+
 // Gate/up projection + SwiGLU in one kernel (bf16 models); timed like gemm().
 int gemm_gu(rsd_ctx* c, const ModelHost& M, const void* Wgu, const void* xin, const void* xin_lo, void* act, void* act_lo,
             int Mrows, int F, int K, const int32_t* n_active, cudaStream_t s, RowScale rs = RowScale()) {
@@ -574,6 +590,7 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
   auto scale = [&](int chunks) { return RowScale{c->norm_ssq, chunks, 1.f / (float)d, m.rms_eps}; };
   const RowScale rs_mid = scale(rows_wo ? d / 8 : norm_chunks(d)), rs_end = scale(rows_down ? d / 8 : norm_chunks(d));
   *final_rs = rs_end;
+  auto bytes = [&](double N, double K) { return (N * K + T * K) * M.elem + T * N * 4.0; };
   if (T <= 0) return RSD_OK;
   CU(launch_embed_norm(m.tok_embed, p, c->x, M.norm1[0], c->h, c->h_lo, c->norm_ssq, d, s));
   for (int l = 0; l < m.n_layers; ++l) {
@@ -584,7 +601,10 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
     bool rotates = false;
     int rc;
     if (rows_qkv) {
-      CU(launch_gemm_rows_qkv(M.wqkv[l], c->h, c->h_lo, rs, p, c->q, kv, M.rope, H, KV, hd, d, s));
+      rc = timed_product(c, bytes((H + 2 * KV) * hd, d), s, [&] {
+        return launch_gemm_rows_qkv(M.wqkv[l], c->h, c->h_lo, rs, p, c->q, kv, M.rope, H, KV, hd, d, s);
+      });
+      if (rc) return rc;
     } else {
       rc = gemm(c, M, M.wqkv[l], c->h, c->h_lo, c->qkv, T, (H + 2 * KV) * hd, d, 0, p.n_active, &src.pending, s, rs);
       if (rc) return rc;
@@ -595,8 +615,10 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
                           c->attn, c->attn_lo, m.dtype, T, H, KV, hd, c->S, c->attn_scratch, c->attn_scratch_bytes,
                           p.n_active, s, c->attn_rows_hint, c->pass_width, rotates ? &src : nullptr));
     if (rows_wo) {
-      CU(launch_gemm_rows_residual(M.wo[l], c->attn, c->attn_lo, c->x, M.norm2[l], c->h, c->h_lo, c->norm_ssq, T, d, H * hd,
-                                   p.n_active, s));
+      rc = timed_product(c, bytes(d, H * hd), s, [&] {
+        return launch_gemm_rows_residual(M.wo[l], c->attn, c->attn_lo, c->x, M.norm2[l], c->h, c->h_lo, c->norm_ssq, T, d, H * hd, p.n_active, s);
+      });
+      if (rc) return rc;
     } else {
       rc = gemm(c, M, M.wo[l], c->attn, c->attn_lo, c->x, T, d, H * hd, 1, p.n_active, &x_pending, s);
       if (rc) return rc;
@@ -613,7 +635,10 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
     }
     const void* next_gain = l + 1 < m.n_layers ? M.norm1[l + 1] : final_gain;
     if (rows_down) {
-      CU(launch_gemm_rows_residual(M.wdown[l], c->act, c->act_lo, c->x, next_gain, c->h, c->h_lo, c->norm_ssq, T, d, F, p.n_active, s));
+      rc = timed_product(c, bytes(d, F), s, [&] {
+        return launch_gemm_rows_residual(M.wdown[l], c->act, c->act_lo, c->x, next_gain, c->h, c->h_lo, c->norm_ssq, T, d, F, p.n_active, s);
+      });
+      if (rc) return rc;
     } else {
       x_pending = SplitSum();
       rc = gemm(c, M, M.wdown[l], c->act, c->act_lo, c->x, T, d, F, 1, p.n_active, &x_pending, s);
@@ -637,14 +662,21 @@ int forward_decode_f32(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
   const int d = m.d_model, H = m.n_heads, KV = m.n_kv_heads, hd = m.head_dim, F = m.d_ffn, T = p.T;
   if (T <= 0) return RSD_OK;
   float *attn = (float*)c->attn, *act = (float*)c->act;
+  auto bytes = [&](double N, double K) { return (N * K + T * K + T * N) * 4.0; };
   CU(launch_embed(m.dtype, m.tok_embed, p, c->x, d, s));
   for (int l = 0; l < m.n_layers; ++l) {
     KvView kv{M.kv_pool + (size_t)l * M.layer_stride, c->st.page_table[which], c->max_pages, 0};
-    CU(launch_gemv_norm((const float*)M.wqkv[l], (const float*)M.norm1[l], c->x, c->qkv, T, (H + 2 * KV) * hd, d, m.rms_eps, false, p.n_active, s));
-    CU(launch_attn_generic(0, c->qkv, p, kv, attn, nullptr, RSD_F32, H, KV, hd, s, M.rope));
-    int rc = gemm(c, M, M.wo[l], attn, nullptr, c->x, T, d, H * hd, 1, p.n_active, nullptr, s);
+    int rc = timed_product(c, bytes((H + 2 * KV) * hd, d), s, [&] {
+      return launch_gemv_norm((const float*)M.wqkv[l], (const float*)M.norm1[l], c->x, c->qkv, T, (H + 2 * KV) * hd, d, m.rms_eps, false, p.n_active, s);
+    });
     if (rc) return rc;
-    CU(launch_gemv_norm((const float*)M.wgu[l], (const float*)M.norm2[l], c->x, act, T, F, d, m.rms_eps, true, p.n_active, s));
+    CU(launch_attn_generic(0, c->qkv, p, kv, attn, nullptr, RSD_F32, H, KV, hd, s, M.rope));
+    rc = gemm(c, M, M.wo[l], attn, nullptr, c->x, T, d, H * hd, 1, p.n_active, nullptr, s);
+    if (rc) return rc;
+    rc = timed_product(c, bytes(2.0 * F, d), s, [&] {
+      return launch_gemv_norm((const float*)M.wgu[l], (const float*)M.norm2[l], c->x, act, T, F, d, m.rms_eps, true, p.n_active, s);
+    });
+    if (rc) return rc;
     rc = gemm(c, M, M.wdown[l], act, nullptr, c->x, T, d, F, 1, p.n_active, nullptr, s);
     if (rc) return rc;
   }
@@ -758,7 +790,9 @@ int model_logits(rsd_ctx* c, int which, PassView p, bool allow_mega, cudaStream_
     rc = gemm(c, M, m.head, c->h, c->h_lo, c->logits, T, m.vocab, m.d_model, 0, p.n_active, nullptr, s, rs);
   } else if (decode_f32_ok(c, M, p)) {
     if ((rc = forward_decode_f32(c, which, p, s))) return rc;
-    CU(launch_gemv_norm((const float*)m.head, (const float*)m.final_norm, c->x, c->logits, T, m.vocab, m.d_model, m.rms_eps, false, p.n_active, s));
+    rc = timed_product(c, ((double)m.vocab * m.d_model + (double)T * (m.vocab + m.d_model)) * 4.0, s, [&] {
+      return launch_gemv_norm((const float*)m.head, (const float*)m.final_norm, c->x, c->logits, T, m.vocab, m.d_model, m.rms_eps, false, p.n_active, s);
+    });
   } else {
     if ((rc = forward_pass(c, which, p, s))) return rc;
     CU(launch_rmsnorm(m.dtype, c->x, m.final_norm, c->h, M.split ? c->h_lo : nullptr, T, m.d_model, m.rms_eps,

@@ -49,13 +49,12 @@ embed_norm_kernel(const __nv_bfloat16* __restrict__ E, PassView p, float* __rest
   float ss = 0.f;
   if (col < d) {
     float v[4], y[4];
-    __align__(8) __nv_bfloat16 e[4], g[4];
+    __align__(8) __nv_bfloat16 e[4];
     *reinterpret_cast<uint2*>(e) = *reinterpret_cast<const uint2*>(E + (size_t)p.tok_id[t] * d + col);
-    *reinterpret_cast<uint2*>(g) = *reinterpret_cast<const uint2*>(gain + col);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       v[i] = to_f32(e[i]);
-      y[i] = v[i] * to_f32(g[i]);
+      y[i] = v[i] * to_f32(gain[col + i]);       // (a caller's gains may start anywhere)
     }
     const size_t o = (size_t)t * d + col;
     *reinterpret_cast<float4*>(x + o) = make_float4(v[0], v[1], v[2], v[3]);
@@ -356,13 +355,14 @@ gemv_norm_kernel(const float* W, const float* __restrict__ gain, const float* X,
   if (n_active == nullptr) RSD_PDL_WAIT();   // outside a decode pass W may be an earlier kernel's output
   const bool idle = n_active != nullptr && ld_cg(n_active) == 0;
   auto weights = [&](Vec16<float> (&w)[R], int v) {
-    Vec16<float> g;
-    g.load(gain + (size_t)v * VN);
+    float g[VN];                             // (a caller's gains may start anywhere)
+#pragma unroll
+    for (int j = 0; j < VN; ++j) g[j] = gain[(size_t)v * VN + j];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       w[r].load_stream(wrow + (size_t)r * N * K + (size_t)v * VN);
 #pragma unroll
-      for (int j = 0; j < VN; ++j) w[r].v[j] *= g.v[j];
+      for (int j = 0; j < VN; ++j) w[r].v[j] *= g[j];
     }
   };
 #pragma unroll

@@ -468,6 +468,32 @@ def test_decode_attention_that_takes_the_qkv_product(d, H, KV, hd, ext):
     eng.close()
 
 
+@pytest.mark.parametrize("bf16", [False, True])
+def test_norm_gains_may_start_anywhere(bf16):
+    """Norm gains one element off any wider boundary give the same step."""
+    import torch
+    from paper_2501_19324_b200 import Engine, Model
+    shapes = MINI if bf16 else TINY
+    heads = (ri.HEAD_LM, ri.HEAD_REWARD_SIGMOID, ri.HEAD_LM)
+
+    def off(g):
+        return torch.cat([g[:1], g])[1:]
+    out = []
+    for move in (lambda g: g, off):
+        models = []
+        for slot, (sh, hk) in enumerate(zip(shapes, heads)):
+            t = dict(ri.gpu_model_tensors(sh, slot, 0, bf16, hk))
+            t.update(final_norm=move(t["final_norm"]), norm1=[move(g) for g in t["norm1"]], norm2=[move(g) for g in t["norm2"]])
+            models.append(Model(sh, t, hk))
+        eng = Engine(*models, max_batch=3, max_seq_tokens=40, max_step_tokens=6, max_steps=2, step_end_id=3, temperature=0.7, seed=2)
+        eng.prefill(*ri.prompts(5, 3, 10, 20, shapes[0].vocab))
+        out.append([eng.step(2.0) for _ in range(2)])
+        eng.close()
+    for a, b in zip(*out):
+        for k in a:
+            np.testing.assert_array_equal(a[k], b[k])
+
+
 @pytest.mark.parametrize("d,H,KV,hd,F,rows,ext", [(64, 1, 1, 64, 64, 1, 0), (576, 7, 1, 128, 448, 8, 0), (576, 7, 1, 128, 448, 9, 0), (512, 4, 2, 64, 1408, 5, 1),
                                                   (1536, 12, 2, 128, 1024, 4, 0), (1536, 12, 2, 128, 1024, 6, 0), (512, 8, 8, 128, 520, 2, 1)])
 def test_decode_products_of_few_rows(d, H, KV, hd, F, rows, ext):
