@@ -452,17 +452,25 @@ sgemm_kernel(const float* __restrict__ W, const float* __restrict__ X, float* Y,
 #pragma unroll
   for (int i = 0; i < kSgStages - 1; ++i) fetch(i);
   const int tn = tid & 7, tm = tid >> 3;         // rows tm + 8 i of x, tn + 8 j of W
-  float acc[4][4];
+  float acc[4][4], mid[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    for (int j = 0; j < 4; ++j) acc[i][j] = mid[i][j] = 0.f;
   for (int step = 0; step < steps; ++step) {
     asm volatile("cp.async.wait_group %0;" ::"n"(kSgStages - 2) : "memory");
     __syncthreads();                             // the stage is there for all, and the one before it has been read by all
     fetch(step + kSgStages - 1);
     const float* xs = sg_smem + (step % kSgStages) * kSgStage;
     const float* ws = xs + kSgM * kSgLd;
+    // a stage's products are summed by themselves first, then four stages': one chain along all of K would be as long as K / 4 and
+    // round accordingly (relative error against fp64 at K = 512 / 1376: in one chain per stage 1.02e-7 / 1.38e-7, so 0.89e-7 / 1.02e-7, a
+    // lane's chain and warp sum of the kernel above 0.86e-7 / 0.97e-7)
+    float part[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) part[i][j] = 0.f;
 #pragma unroll
     for (int k = 0; k < kSgK / kSgGroups; k += 4) {
       const int kk = grp * (kSgK / kSgGroups) + k;
@@ -475,9 +483,20 @@ sgemm_kernel(const float* __restrict__ W, const float* __restrict__ X, float* Y,
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          acc[i][j] = fmaf(a[i].w, b[j].w, fmaf(a[i].z, b[j].z, fmaf(a[i].y, b[j].y, fmaf(a[i].x, b[j].x, acc[i][j]))));
+          part[i][j] = fmaf(a[i].w, b[j].w, fmaf(a[i].z, b[j].z, fmaf(a[i].y, b[j].y, fmaf(a[i].x, b[j].x, part[i][j]))));
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        mid[i][j] += part[i][j];
+        if ((step & 3) == 3) { acc[i][j] += mid[i][j]; mid[i][j] = 0.f; }
+      }
   }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] += mid[i][j];
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
   if (grp > 0) {
