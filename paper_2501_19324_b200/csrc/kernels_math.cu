@@ -421,14 +421,29 @@ gemv_norm_kernel(const float* W, const float* __restrict__ gain, const float* X,
 // fp32 products of more rows (prefill, scoring and catch-up of fp32 models): 32 rows of x by 32 of W a block, 32 values of K a stage, four
 // stages of 16-byte cp.async copies; four groups of 64 threads take eight of a stage's 32 values of K each, 4 x 4 results a thread, and
 // their sums meet at the end.  (Eight rows at a time, as above, the weights come from L2 once per eight rows and every one is used eight
-// times per load.)  Bound by shared-memory reads (two of 16 bytes per 16 multiply-adds) and by the latency of a stage, the blocks being
-// few: 0.5 us a stage
-// (tiles of 64 columns with 4 x 4 or 4 x 8 results a thread, 0.75 and 0.95).
+// times per load.)  Bound by shared memory (two reads of 16 bytes per 16 multiply-adds, the copies, the sums kept there), with few blocks by
+// the latency of a stage, 0.4 us (tiles of 64 columns with 4 x 4 or 4 x 8 results a thread took 1.5 and 1.9 times as long a stage).  Two products
+// at a time: 256 x 512 x 512, 256 x 512 x 1376 and 256 x 1024 x 4096 take 15.7, 37.9 and 112 us, with scalar ones and sums of less depth
+// 18.9, 47.0 and 154; with many blocks, 256 x 2752 x 512 and 1024 x 4096 x 1024, the depth of the sums costs 35.5 -> 38.9 and 354 -> 387.
 constexpr int kSgM = 32, kSgN = 32, kSgK = 32, kSgLd = kSgK + 4, kSgStages = 4, kSgGroups = 4;   // rows 16 bytes apart modulo 128: no bank conflicts
 constexpr int kSgStage = (kSgM + kSgN) * kSgLd, kSgThreads = 64 * kSgGroups;
 static_assert((kSgGroups - 1) * kSgM * kSgN <= kSgStages * kSgStage, "the groups' sums take the place of the stages");
+static_assert(kSgGroups == 4 && kSgK == 32, "the order of the sums below");
 
-__global__ void __launch_bounds__(kSgThreads)
+// Two fp32 products or sums at once, rounded as the scalar ones.
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float add_halves(uint64_t a) { return __uint_as_float((uint32_t)a) + __uint_as_float((uint32_t)(a >> 32)); }
+
+__global__ void __launch_bounds__(kSgThreads, 2)
 sgemm_kernel(const float* __restrict__ W, const float* __restrict__ X, float* Y, int M, int N, int K, int accumulate) {
   RSD_PDL_SYNC();
   extern __shared__ __align__(16) float sg_smem[];
@@ -452,58 +467,73 @@ sgemm_kernel(const float* __restrict__ W, const float* __restrict__ X, float* Y,
 #pragma unroll
   for (int i = 0; i < kSgStages - 1; ++i) fetch(i);
   const int tn = tid & 7, tm = tid >> 3;         // rows tm + 8 i of x, tn + 8 j of W
-  float acc[4][4], mid[4][4];
+  // Sums in a tree: two chains of four products a stage, pairs of stages, chains of four pairs, of four of those, and of these.  Along K it is
+  // then never deeper than a lane's chain, the warp's tree and the K splits of the kernel above (relative error against fp64, that kernel / this
+  // one, at K = 256, 512, 1376, 4096: 0.81 / 0.79, 0.85 / 0.83, 0.96 / 0.91, 1.10 / 0.99e-7).  The last two sums, touched every eighth and
+  // thirty-second stage, lie in shared memory: two blocks an SM instead of one.
+  float hold[4][4], eight[4][4];
+  float *acc = sg_smem + kSgStages * kSgStage + threadIdx.x, *top = acc + 16 * kSgThreads;
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = mid[i][j] = 0.f;
+    for (int j = 0; j < 4; ++j) acc[(4 * i + j) * kSgThreads] = top[(4 * i + j) * kSgThreads] = 0.f;
   for (int step = 0; step < steps; ++step) {
     asm volatile("cp.async.wait_group %0;" ::"n"(kSgStages - 2) : "memory");
     __syncthreads();                             // the stage is there for all, and the one before it has been read by all
     fetch(step + kSgStages - 1);
     const float* xs = sg_smem + (step % kSgStages) * kSgStage;
     const float* ws = xs + kSgM * kSgLd;
-    // a stage's products are summed by themselves first, then four stages': one chain along all of K would be as long as K / 4 and
-    // round accordingly (relative error against fp64 at K = 512 / 1376: in one chain per stage 1.02e-7 / 1.38e-7, so 0.89e-7 / 1.02e-7, a
-    // lane's chain and warp sum of the kernel above 0.86e-7 / 0.97e-7)
-    float part[4][4];
+    uint64_t part[4][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int k = 0; k < 2; ++k) {
+      const int kk = grp * (kSgK / kSgGroups) + 4 * k;
+      ulonglong2 a[4], b[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) part[i][j] = 0.f;
+      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const ulonglong2*>(xs + (tm + 8 * i) * kSgLd + kk);
 #pragma unroll
-    for (int k = 0; k < kSgK / kSgGroups; k += 4) {
-      const int kk = grp * (kSgK / kSgGroups) + k;
-      float4 a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(xs + (tm + 8 * i) * kSgLd + kk);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(ws + (tn + 8 * j) * kSgLd + kk);
+      for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const ulonglong2*>(ws + (tn + 8 * j) * kSgLd + kk);
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          part[i][j] = fmaf(a[i].w, b[j].w, fmaf(a[i].z, b[j].z, fmaf(a[i].y, b[j].y, fmaf(a[i].x, b[j].x, part[i][j]))));
+        for (int j = 0; j < 4; ++j) {
+          part[i][j] = k == 0 ? mul2(a[i].x, b[j].x) : fma2(a[i].x, b[j].x, part[i][j]);
+          part[i][j] = fma2(a[i].y, b[j].y, part[i][j]);
+        }
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        mid[i][j] += part[i][j];
-        if ((step & 3) == 3) { acc[i][j] += mid[i][j]; mid[i][j] = 0.f; }
+        const float p = add_halves(part[i][j]);
+        if ((step & 1) == 0) {
+          hold[i][j] = p;
+        } else if ((step & 7) == 1) {
+          eight[i][j] = hold[i][j] + p;
+        } else {
+          eight[i][j] += hold[i][j] + p;
+          if ((step & 7) == 7) {
+            float& u = acc[(4 * i + j) * kSgThreads];
+            const float v = u + eight[i][j];
+            u = (step & 31) == 31 ? 0.f : v;
+            if ((step & 31) == 31) top[(4 * i + j) * kSgThreads] += v;
+          }
+        }
       }
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] += mid[i][j];
+    for (int j = 0; j < 4; ++j) {
+      const float rest = (steps & 6 ? eight[i][j] : 0.f) + (steps & 1 ? hold[i][j] : 0.f);     // of the stages after the last eight
+      eight[i][j] = top[(4 * i + j) * kSgThreads] + (acc[(4 * i + j) * kSgThreads] + rest);
+    }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
   if (grp > 0) {
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) sg_smem[((grp - 1) * kSgM + tm + 8 * i) * kSgN + tn + 8 * j] = acc[i][j];
+      for (int j = 0; j < 4; ++j) sg_smem[((grp - 1) * kSgM + tm + 8 * i) * kSgN + tn + 8 * j] = eight[i][j];
   }
   __syncthreads();
   if (grp > 0) return;
@@ -513,9 +543,8 @@ sgemm_kernel(const float* __restrict__ W, const float* __restrict__ X, float* Y,
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int n = n0 + tn + 8 * j;
-      float v = acc[i][j];
-#pragma unroll
-      for (int r = 0; r < kSgGroups - 1; ++r) v += sg_smem[(r * kSgM + tm + 8 * i) * kSgN + tn + 8 * j];
+      const float* other = sg_smem + (tm + 8 * i) * kSgN + tn + 8 * j;
+      const float v = (eight[i][j] + other[0]) + (other[kSgM * kSgN] + other[2 * kSgM * kSgN]);
       if (m < M && n < N) {
         float* y = Y + (size_t)m * N + n;
         *y = accumulate ? *y + v : v;
@@ -563,7 +592,7 @@ cudaError_t launch_gemm_simt(int dtype, const void* W, const void* x, const void
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (dtype != 1 && n_active == nullptr && sgemm_pays(M, N)) {
     static OncePerDevice configured;
-    constexpr size_t smem = kSgStages * kSgStage * sizeof(float);
+    constexpr size_t smem = (kSgStages * kSgStage + 2 * 16 * kSgThreads) * sizeof(float);
     const cudaError_t set = allow_smem(configured, sgemm_kernel, smem);
     if (set != cudaSuccess) return set;
     RSD_LAUNCH((sgemm_kernel), dim3((N + kSgN - 1) / kSgN, (M + kSgM - 1) / kSgM), kSgThreads, smem, s, (const float*)W, (const float*)x, y, M, N, K, accumulate);
