@@ -1129,11 +1129,18 @@ static cudaError_t launch_persistent(const CUtensorMap& tw, const CUtensorMap& t
   return launched(1);
 }
 
+template <bool GU, bool SPLIT>
+static cudaError_t configure_pair() {
+  static OncePerDevice configured;
+  return allow_smem(configured, gemm_tc_pair_kernel<GU, SPLIT>, PairCfg<SPLIT, GU>::kSmemBytes);
+}
+
 // Pairs of CTAs that fit the device at once.
 template <bool GU, bool SPLIT>
-static int max_pairs(size_t smem) {
+static int query_pairs() {
+  if (configure_pair<GU, SPLIT>() != cudaSuccess) return 0;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2048); cfg.blockDim = dim3(kPersistThreads); cfg.dynamicSmemBytes = smem;
+  cfg.gridDim = dim3(2048); cfg.blockDim = dim3(kPersistThreads); cfg.dynamicSmemBytes = PairCfg<SPLIT, GU>::kSmemBytes;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
@@ -1141,17 +1148,20 @@ static int max_pairs(size_t smem) {
   int n = 0;
   return cudaOccupancyMaxActiveClusters(&n, gemm_tc_pair_kernel<GU, SPLIT>, &cfg) == cudaSuccess ? n : 0;
 }
+template <bool GU, bool SPLIT>
+static int max_pairs() {
+  static const int pairs = query_pairs<GU, SPLIT>();
+  return pairs;
+}
 
 // The map of x has a box of half the tile's operand rows.
 template <bool GU, bool SPLIT>
 static cudaError_t launch_pair(const CUtensorMap& tw, const CUtensorMap& tx, const CUtensorMap& txl, float* y, int M, int N, int K,
                                int accumulate, int* err, __nv_bfloat16* act_hi, __nv_bfloat16* act_lo, cudaStream_t s, int f16, int rows) {
-  using C = PairCfg<SPLIT, GU>;
-  constexpr size_t smem = C::kSmemBytes;
-  static OncePerDevice configured;
-  const cudaError_t set = allow_smem(configured, gemm_tc_pair_kernel<GU, SPLIT>, smem);
+  constexpr size_t smem = PairCfg<SPLIT, GU>::kSmemBytes;
+  const cudaError_t set = configure_pair<GU, SPLIT>();
   if (set != cudaSuccess) return set;
-  static const int pairs = max_pairs<GU, SPLIT>(smem);
+  const int pairs = max_pairs<GU, SPLIT>();
   if (pairs <= 0) return cudaErrorNotSupported;
   const int feat = GU ? kTileN : 2 * kTileN, tiles_n = (N + feat - 1) / feat, tiles_m = (M + rows - 1) / rows;
   cudaLaunchConfig_t cfg = {};
@@ -1183,7 +1193,9 @@ static bool pair_pays(int M, int n_features, int K, int feat, int rows, bool add
 // nearly empty (4096 x 3584: 224 tiles on 74 pairs of SMs) fewer rows win; us at 256 / 224 / 192 / 160: 4096 x 3584 x 18944 576 / 506 / 545 / 509,
 // 1300 x 3584 x 18944 260 / 229 / 204 / 192, 4096 x 1536 x 8960 140 / 125 / 113 / 144, 8192 x 1536 x 1536 (lone CTAs) 55.8 / 50.8 / 55.8 / 57.9,
 // 1300 x 4608 x 3584 55 / 50 / 45 / 54; and 4096 x 2048 x 1536, two full waves, stays at 256 (29.5 / 35.0 / 32.1 / 29.5).
+// slots: the pairs of CTAs, or CTAs, that the launch has at once.
 static int wave_rows(int M, int n_tiles, int slots) {
+  slots = std::max(slots, 1);              // (none: the launch reports it)
   constexpr int kRows[4] = {256, 224, 192, 160}, kCost[4] = {256, 233, 217, 206};
   int best = 0;
   long cost = 0;
@@ -1263,7 +1275,7 @@ cudaError_t launch_gemm_gu(const void* Wgu, const void* x, const void* x_lo, voi
     // plain bf16 operand: the persistent kernel only (more than 128 rows, no row scale, no idle flag)
     if (!(M > 128 && rs.ssq == nullptr && n_active == nullptr)) return cudaErrorNotSupported;
     const bool pair = pair_pays(M, F, K, kTileN, 256, false);
-    const int tile_rows = pair ? wave_rows(M, pair_tiles(F, kTileN), 74) : wave_rows(M, F / 64, 148);
+    const int tile_rows = pair ? wave_rows(M, pair_tiles(F, kTileN), max_pairs<true, false>()) : wave_rows(M, F / 64, sm_count());
     if (!get_map(Wgu, 2 * F, K, kTileN / 2, &tw) || !get_map(x, M, K, pair ? tile_rows / 2 : tile_rows, &tx)) return cudaErrorNotSupported;
     if (pair) return launch_pair<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act_hi, nullptr, s, 0, tile_rows);
     return launch_persistent<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act_hi, nullptr, s, 0, nullptr, RowScale(), tile_rows);
@@ -1326,7 +1338,7 @@ cudaError_t launch_gemm_tc(const void* W, const void* x, const void* x_lo, float
   const bool pair = dense && pair_pays(M, N, K, 2 * kTileN, p.rows, accumulate != 0);
   int rows = dense && !split_operand && !pair && !no_k_split ? dense_rows(M, N, K, accumulate != 0) : p.rows;
   const bool small = dense && !pair && !split_operand && rows < 256;
-  if (dense && !split_operand && !small) rows = pair ? wave_rows(M, pair_tiles(N, 2 * kTileN), 74) : wave_rows(M, p.n_tiles, 148);
+  if (dense && !split_operand && !small) rows = pair ? wave_rows(M, pair_tiles(N, 2 * kTileN), max_pairs<false, false>()) : wave_rows(M, p.n_tiles, sm_count());
   if (!get_map(W, N, K, kTileN, &tw) || !get_map(x, M, K, pair ? (split_operand ? 128 : rows / 2) : rows, &tx)) return cudaErrorNotSupported;
   if (split_operand) { if (!get_map(x_lo, M, K, p.rows, &txl)) return cudaErrorNotSupported; }
   else txl = tx;
@@ -1383,7 +1395,7 @@ cudaError_t launch_gemm_f16_dense(const void* W16, const void* x16, float* y, in
   CUtensorMap tw, tx;
   int rows = pair ? 256 : dense_rows(M, N, K, accumulate != 0);
   const bool small = rows < 256;
-  if (!small) rows = pair ? wave_rows(M, pair_tiles(N, 2 * kTileN), 74) : wave_rows(M, (N + kTileN - 1) / kTileN, 148);
+  if (!small) rows = pair ? wave_rows(M, pair_tiles(N, 2 * kTileN), max_pairs<false, false>()) : wave_rows(M, (N + kTileN - 1) / kTileN, sm_count());
   if (!get_map(W16, N, K, kTileN, &tw) || !get_map(x16, M, K, pair ? rows / 2 : rows, &tx)) return cudaErrorNotSupported;
   int* err = (int*)((char*)scratch + kCounterBytes);
   if (small) return launch_dense_small(tw, tx, y, M, N, K, accumulate, rows, err, s, 1);
@@ -1400,7 +1412,7 @@ cudaError_t launch_gemm_gu_f16_dense(const void* Wgu16, const void* x16, void* a
   int* err = (int*)((char*)scratch + kCounterBytes);
   CUtensorMap tw, tx;
   const bool pair = pair_pays(M, F, K, kTileN, 256, false);
-  const int rows = pair ? wave_rows(M, pair_tiles(F, kTileN), 74) : wave_rows(M, F / 64, 148);
+  const int rows = pair ? wave_rows(M, pair_tiles(F, kTileN), max_pairs<true, false>()) : wave_rows(M, F / 64, sm_count());
   if (!get_map(Wgu16, 2 * F, K, kTileN / 2, &tw) || !get_map(x16, M, K, pair ? rows / 2 : rows, &tx)) return cudaErrorNotSupported;
   if (pair) return launch_pair<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act16, nullptr, s, 1, rows);
   return launch_persistent<true, false>(tw, tx, tx, nullptr, M, F, K, 0, err, (__nv_bfloat16*)act16, nullptr, s, 1, nullptr, RowScale(), rows);

@@ -782,15 +782,16 @@ def test_gate_up_gemm_on_pairs_of_ctas(M, F, K):
 
 
 @pytest.mark.parametrize("M,N,K,adds", [(1100, 4608, 1024, False), (1290, 4500, 1032, False), (3000, 3584, 3080, True),
-                                        (3200, 1536, 136, True), (4080, 1536, 136, True)])
-def test_dense_tiles_of_fewer_rows(M, N, K, adds):
+                                        (3200, 1536, 136, True), (4080, 1536, 136, True), (8100, 1530, 136, True)])
+@pytest.mark.parametrize("dtype,impl", [(torch.float16, 4), (torch.bfloat16, 2)])
+def test_dense_tiles_of_fewer_rows(M, N, K, adds, dtype, impl):
     """Products whose last wave of 256-row tiles would be nearly empty take tiles of 160, 192 and 224 rows, in pairs of CTAs (first three) and
-    lone; ragged last tiles of rows and features.  fp32 sums of K products of order 0.05, as above."""
+    lone, of fp16 and of plain bf16 operands; ragged last tiles of rows and features.  fp32 sums of K products of order 0.05, as above."""
     g = torch.Generator(device="cuda").manual_seed(M + N)
-    W = (torch.randn(N, K, generator=g, device="cuda") * 0.05).half()
-    x = torch.randn(M, K, generator=g, device="cuda").half()
+    W = (torch.randn(N, K, generator=g, device="cuda") * 0.05).to(dtype)
+    x = torch.randn(M, K, generator=g, device="cuda").to(dtype)
     y0 = torch.randn(M, N, generator=g, device="cuda")
-    y = rb.k_gemm(W, x, y=y0.clone(), accumulate=True, impl=4) if adds else rb.k_gemm(W, x, impl=4)
+    y = rb.k_gemm(W, x, y=y0.clone(), accumulate=True, impl=impl) if adds else rb.k_gemm(W, x, impl=impl)
     want = x.double() @ W.double().t() + (y0 if adds else 0)
     assert (y.double() - want).abs().max().item() <= 2e-5 * K ** 0.5 + 2e-6
 
