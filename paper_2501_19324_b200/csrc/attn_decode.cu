@@ -180,8 +180,9 @@ attn_decode_kernel(const float* q, KT* pool, const int32_t* page_table, int max_
       if (EXT) s_q[EXT ? 1 : 0][G + idx / HD][idx % HD] = from_f32<KT>(0.f);
     }
     const int part = lane / kPerWarp;              // of the K splits: runs [part R, part R + R)
-    for (int task0 = warp * kPerWarp; task0 < n_tasks; task0 += NW * kPerWarp) {
-      const int task = min(task0 + lane % kPerWarp, n_tasks - 1);          // whole warps: lanes beyond the last task repeat it
+    // (P == 1: a task per thread; the loop over whole warps there cost registers, 80 bytes of spills instead of 48 with hi + lo caches)
+    for (int task0 = P == 1 ? threadIdx.x : warp * kPerWarp; task0 < n_tasks; task0 += NW * kPerWarp) {
+      const int task = P == 1 ? task0 : min(task0 + lane % kPerWarp, n_tasks - 1);   // whole warps: lanes beyond the last task repeat it
       const bool is_q = task < G * NQ;
       const int hh = is_q ? task / NQ : task / NQ - G, dd = 4 * (task % NQ);   // one of the group's heads, or 0 = the key, 1 = the value
       const size_t src = (size_t)slot * width + (size_t)(is_q ? h0 + hh : H + hh * KV + kvh) * HD + dd;
@@ -230,7 +231,7 @@ attn_decode_kernel(const float* q, KT* pool, const int32_t* page_table, int max_
           }
         }
       }
-      if (part > 0 || task0 + lane >= n_tasks) continue;
+      if (P > 1 && (part > 0 || task0 + lane >= n_tasks)) continue;
       if (is_q || hh == 0) {
         const float2* cs = rope + (size_t)(ctx - 1) * (HD / 2) + dd;
 #pragma unroll
