@@ -425,7 +425,12 @@ int gemm(rsd_ctx* c, const ModelHost& M, const void* W, const void* xin, const v
   return RSD_OK;
 }
 
-// A decode product that takes a neighbouring step along, timed like gemm(); bytes: its weights, input and output once.
+// A decode product that takes a neighbouring step along, timed like gemm() and with that function's bytes: W [N, K] and the input once, `out`
+// columns of output once, or twice when added to.
+struct ProductBytes {
+  double T, elem;
+  double operator()(double N, double K, double out, bool adds) const { return N * K * elem + T * K * elem + T * out * 4.0 * (adds ? 2.0 : 1.0); }
+};
 template <typename Launch> int timed_product(rsd_ctx* c, double bytes, cudaStream_t s, Launch launch) {
   const bool pick = c->in_decode ? c->time_this_iter
                                  : (c->time_stride > 0 && (c->gemm_calls++ % (uint64_t)c->time_stride) == 0);
@@ -590,7 +595,7 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
   auto scale = [&](int chunks) { return RowScale{c->norm_ssq, chunks, 1.f / (float)d, m.rms_eps}; };
   const RowScale rs_mid = scale(rows_wo ? d / 8 : norm_chunks(d)), rs_end = scale(rows_down ? d / 8 : norm_chunks(d));
   *final_rs = rs_end;
-  auto bytes = [&](double N, double K) { return (N * K + T * K) * M.elem + T * N * 4.0; };
+  const ProductBytes bytes{(double)T, (double)M.elem};
   if (T <= 0) return RSD_OK;
   CU(launch_embed_norm(m.tok_embed, p, c->x, M.norm1[0], c->h, c->h_lo, c->norm_ssq, d, s));
   for (int l = 0; l < m.n_layers; ++l) {
@@ -601,7 +606,7 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
     bool rotates = false;
     int rc;
     if (rows_qkv) {
-      rc = timed_product(c, bytes((H + 2 * KV) * hd, d), s, [&] {
+      rc = timed_product(c, bytes((H + 2 * KV) * hd, d, (H + 2 * KV) * hd, false), s, [&] {
         return launch_gemm_rows_qkv(M.wqkv[l], c->h, c->h_lo, rs, p, c->q, kv, M.rope, H, KV, hd, d, s);
       });
       if (rc) return rc;
@@ -615,7 +620,7 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
                           c->attn, c->attn_lo, m.dtype, T, H, KV, hd, c->S, c->attn_scratch, c->attn_scratch_bytes,
                           p.n_active, s, c->attn_rows_hint, c->pass_width, rotates ? &src : nullptr));
     if (rows_wo) {
-      rc = timed_product(c, bytes(d, H * hd), s, [&] {
+      rc = timed_product(c, bytes(d, H * hd, d, true), s, [&] {
         return launch_gemm_rows_residual(M.wo[l], c->attn, c->attn_lo, c->x, M.norm2[l], c->h, c->h_lo, c->norm_ssq, T, d, H * hd, p.n_active, s);
       });
       if (rc) return rc;
@@ -635,7 +640,7 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
     }
     const void* next_gain = l + 1 < m.n_layers ? M.norm1[l + 1] : final_gain;
     if (rows_down) {
-      rc = timed_product(c, bytes(d, F), s, [&] {
+      rc = timed_product(c, bytes(d, F, d, true), s, [&] {
         return launch_gemm_rows_residual(M.wdown[l], c->act, c->act_lo, c->x, next_gain, c->h, c->h_lo, c->norm_ssq, T, d, F, p.n_active, s);
       });
       if (rc) return rc;
@@ -662,18 +667,18 @@ int forward_decode_f32(rsd_ctx* c, int which, PassView p, cudaStream_t s) {
   const int d = m.d_model, H = m.n_heads, KV = m.n_kv_heads, hd = m.head_dim, F = m.d_ffn, T = p.T;
   if (T <= 0) return RSD_OK;
   float *attn = (float*)c->attn, *act = (float*)c->act;
-  auto bytes = [&](double N, double K) { return (N * K + T * K + T * N) * 4.0; };
+  const ProductBytes bytes{(double)T, 4.0};
   CU(launch_embed(m.dtype, m.tok_embed, p, c->x, d, s));
   for (int l = 0; l < m.n_layers; ++l) {
     KvView kv{M.kv_pool + (size_t)l * M.layer_stride, c->st.page_table[which], c->max_pages, 0};
-    int rc = timed_product(c, bytes((H + 2 * KV) * hd, d), s, [&] {
+    int rc = timed_product(c, bytes((H + 2 * KV) * hd, d, (H + 2 * KV) * hd, false), s, [&] {
       return launch_gemv_norm((const float*)M.wqkv[l], (const float*)M.norm1[l], c->x, c->qkv, T, (H + 2 * KV) * hd, d, m.rms_eps, false, p.n_active, s);
     });
     if (rc) return rc;
     CU(launch_attn_generic(0, c->qkv, p, kv, attn, nullptr, RSD_F32, H, KV, hd, s, M.rope));
     rc = gemm(c, M, M.wo[l], attn, nullptr, c->x, T, d, H * hd, 1, p.n_active, nullptr, s);
     if (rc) return rc;
-    rc = timed_product(c, bytes(2.0 * F, d), s, [&] {
+    rc = timed_product(c, bytes(2.0 * F, d, F, false), s, [&] {
       return launch_gemv_norm((const float*)M.wgu[l], (const float*)M.norm2[l], c->x, act, T, F, d, m.rms_eps, true, p.n_active, s);
     });
     if (rc) return rc;
@@ -790,7 +795,7 @@ int model_logits(rsd_ctx* c, int which, PassView p, bool allow_mega, cudaStream_
     rc = gemm(c, M, m.head, c->h, c->h_lo, c->logits, T, m.vocab, m.d_model, 0, p.n_active, nullptr, s, rs);
   } else if (decode_f32_ok(c, M, p)) {
     if ((rc = forward_decode_f32(c, which, p, s))) return rc;
-    rc = timed_product(c, ((double)m.vocab * m.d_model + (double)T * (m.vocab + m.d_model)) * 4.0, s, [&] {
+    rc = timed_product(c, ProductBytes{(double)T, 4.0}(m.vocab, m.d_model, m.vocab, false), s, [&] {
       return launch_gemv_norm((const float*)m.head, (const float*)m.final_norm, c->x, c->logits, T, m.vocab, m.d_model, m.rms_eps, false, p.n_active, s);
     });
   } else {

@@ -527,6 +527,32 @@ def test_fp32_decode_with_the_small_steps_inside_the_products(d, H, KV, hd, rows
     eng.close()
 
 
+@pytest.mark.parametrize("bf16,rows", [(False, 3), (True, 2), (True, 9)])
+def test_timed_decode_products_count_the_same_bytes(bf16, rows):
+    """The bytes reported with the timed products of a decode iteration are the algorithm's: weights and input once, output once or, added
+    to, twice.  They don't depend on the kernels that run (of few bf16 rows, of more, fp32); a fused gate/up writes F columns, in bf16
+    as pairs in and out."""
+    from paper_2501_19324_b200 import Engine, Model
+    sh = (MINI if bf16 else TINY)[0]
+    heads = (ri.HEAD_LM, ri.HEAD_REWARD_SIGMOID, ri.HEAD_LM)
+    models = [Model(sh, ri.gpu_model_tensors(sh, slot, 0, bf16, hk), hk, head_only=slot == 1) for slot, hk in enumerate(heads)]
+    eng = Engine(*models, max_batch=rows, max_seq_tokens=48, max_step_tokens=6, max_steps=2, step_end_id=-1, temperature=0.0, prm_shares_draft=1)
+    eng.prefill(*ri.prompts(3, rows, 10, 20, sh.vocab))
+    eng.gemm_timing(1 << 20)                  # of multi-token passes one in a million, of decode iterations the sixth
+    eng.step(-1.0)                            # every row is accepted: the draft alone decodes
+    got = eng.gemm_timing(0)
+    d, F, T, e = sh.d_model, sh.d_ffn, rows, 2 if bf16 else 4
+    width, wide = (sh.n_heads + 2 * sh.n_kv_heads) * sh.head_dim, sh.n_heads * sh.head_dim
+
+    def product(N, K, adds=False):
+        return (N + T) * K * e + T * N * (8 if adds else 4)
+    layer = product(width, d) + product(d, wide, True) + product(d, F, True)
+    layer += 2 * F * d * e + (2 * T * d * e + 2 * T * F * e if bf16 else T * (d + F) * e)
+    assert got["launches"] == 4 * sh.n_layers + 1
+    assert got["bytes"] == sh.n_layers * layer + product(sh.vocab, d)
+    eng.close()
+
+
 @pytest.mark.parametrize("rows,H,KV,hd,lo,hi", [(97, 1, 1, 64, 3, 18), (37, 16, 4, 128, 12, 33), (74, 14, 2, 128, 12, 20), (100, 8, 1, 128, 250, 262)])
 def test_decode_attention_of_sixteen_warps(rows, H, KV, hd, lo, hi):
     """97 to 148 (slot, KV head) pairs: one CTA of sixteen warps each takes the qkv product; groups of one to eight heads, both head
