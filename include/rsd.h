@@ -118,7 +118,8 @@ typedef struct {
                                  number of target passes changes.  The workspace grows with k (logits of k
                                  positions per row)                                                           */
   /* caller-allocated device memory, sizes as reported by rsd_query_sizes (or larger)        */
-  void* kv_pool[3];           /* RSD_DRAFT / RSD_PRM / RSD_TARGET                            */
+  void* kv_pool[3];           /* RSD_DRAFT / RSD_PRM / RSD_TARGET; 16-byte aligned for bf16 models with up to
+                                 eight query heads a KV head (rsd_load_models refuses others)     */
   size_t kv_bytes[3];
   void* workspace;
   size_t workspace_bytes;

@@ -1161,6 +1161,9 @@ int rsd_load_models(rsd_ctx* c, const rsd_model* draft, const rsd_model* prm, co
     M.w16_layer = layer_weight_elems(M.m);
     M.n_params = count_params(M.m);
     M.kv_pool = (char*)c->cfg.kv_pool[w];
+    // the generic attention (fp32 caches, wide groups) reads a pool off a 16-byte boundary element by element, the others copy 16 bytes at a time
+    if (M.kv_dtype != 0 && M.m.n_heads / M.m.n_kv_heads <= 8 && ((uintptr_t)M.kv_pool & 15))
+      return fail(c, RSD_ERR_ARG, "KV pool of a 16-bit cache must be 16-byte aligned%s");
     const size_t page_bytes = (size_t)(M.kv_dtype == 3 ? 4 : 2) * M.m.n_kv_heads * kPageTokens * M.m.head_dim * M.elem;
     int pages = (int)std::min<size_t>(c->cfg.kv_bytes[w] / (page_bytes * L), (size_t)c->B_max * max_pages);
     if (pages < 1) return fail(c, RSD_ERR_OOM_PAGES, "KV pool too small for a single page%s");

@@ -845,8 +845,8 @@ cudaError_t launch_rope_kv(int kv_dtype, const float* qkv, SplitSum pending, Pas
                            const float2* rope, int H, int KV, int hd, cudaStream_t s) {
   if (p.T <= 0) return cudaSuccess;
   const int pf = 2 + 2 * kv.v_extra;
-  if (pending.splits <= 1 && p.n_active == nullptr && p.T >= 64) {
-    // long pass: eight list entries per block
+  if (pending.splits <= 1 && p.n_active == nullptr && p.T >= 64 && ((uintptr_t)kv.pool_layer & 15) == 0) {
+    // long pass: eight list entries per block, keys and values in vectors (a caller's pool that starts off a 16-byte boundary: element by element below)
     const int blocks = (p.T + kRopeTokens - 1) / kRopeTokens;
     if (kv_dtype == 2 || kv_dtype == 3)
       RSD_LAUNCH((rope_kv_long_kernel<__half>), blocks, 256, 0, s, qkv, p, q_out, (__half*)kv.pool_layer, kv.page_table, kv.max_pages, rope, H, KV, hd, pf);

@@ -468,6 +468,49 @@ def test_decode_attention_that_takes_the_qkv_product(d, H, KV, hd, ext):
     eng.close()
 
 
+@pytest.mark.parametrize("d,H,KV,hd,lo,hi", [(256, 4, 2, 64, 10, 20), (512, 4, 1, 128, 250, 270)])
+def test_fp32_caches_may_start_anywhere(monkeypatch, d, H, KV, hd, lo, hi):
+    """fp32 pools that start 4 bytes off a 16-byte boundary, read element by element, give the same steps: the decode attention with the
+    rotation inside, a new token on the first and last place of a page, fewer pages than warps and more."""
+    import torch
+    from paper_2501_19324_b200 import Engine, Model
+    sh = ri.ModelShape(2, d, H, KV, hd, 344, 1024)
+    heads = (ri.HEAD_LM, ri.HEAD_REWARD_SIGMOID, ri.HEAD_LM)
+    models = [Model(sh, ri.gpu_model_tensors(sh, slot, 0, False, hk), hk) for slot, hk in enumerate(heads)]
+    empty, out = torch.empty, []
+    for off in (0, 4):
+        calls = []
+
+        def placed(*size, **kw):
+            calls.append(size)
+            if len(calls) > 3:                                  # the three pools come first, then the workspace
+                return empty(*size, **kw)
+            return empty(size[0] + 16, **kw)[off:off + size[0]]
+        monkeypatch.setattr(torch, "empty", placed)
+        eng = Engine(*models, max_batch=5, max_seq_tokens=hi + 24, max_step_tokens=8, max_steps=2, step_end_id=-1, temperature=0.7, seed=2)
+        monkeypatch.setattr(torch, "empty", empty)
+        assert all(eng.cfg.kv_pool[i] % 16 == off for i in range(3))
+        eng.prefill(*ri.prompts(5, 5, lo, hi, sh.vocab))
+        out.append([eng.step(2.0) for _ in range(2)])
+        eng.close()
+    for a, b in zip(*out):
+        for k in a:
+            np.testing.assert_array_equal(a[k], b[k])
+
+
+def test_16_bit_caches_off_a_boundary_are_refused(monkeypatch):
+    """The tensor-core attention copies 16 bytes at a time: a pool 4 bytes off a boundary is refused before anything runs on it."""
+    import torch
+    from paper_2501_19324_b200 import Engine, Model
+    from paper_2501_19324_b200.binding import RsdError
+    heads = (ri.HEAD_LM, ri.HEAD_REWARD_SIGMOID, ri.HEAD_LM)
+    models = [Model(sh, ri.gpu_model_tensors(sh, slot, 0, True, hk), hk) for slot, (sh, hk) in enumerate(zip(MINI, heads))]
+    empty = torch.empty
+    monkeypatch.setattr(torch, "empty", lambda *size, **kw: empty(size[0] + 512, **kw)[4:4 + size[0]] if kw["dtype"] == torch.uint8 and size[0] < (8 << 20) else empty(*size, **kw))
+    with pytest.raises(RsdError, match="16-byte aligned"):
+        Engine(*models, max_batch=2, max_seq_tokens=32, max_step_tokens=4, max_steps=2, step_end_id=3)
+
+
 @pytest.mark.parametrize("bf16", [False, True])
 def test_norm_gains_may_start_anywhere(bf16):
     """Norm gains one element off any wider boundary give the same step."""
