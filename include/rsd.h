@@ -312,7 +312,7 @@ int rsd_debug_gemm_wait_probe(const void* W, const void* x, float* y, void* scra
  * `dtype` (RSD_F32, RSD_BF16, RSD_F16 or RSD_F16_EXT, which adds the blocks keys_lo and values_lo after the
  * first two); page_table [B, max_pages]; ctx_len [B] (number of cached
  * positions attended; rows with ctx_len < 1 are skipped); out [B, H, hd] fp32.  16-bit caches with
- * H / KV <= 8 take the tensor-core split-context kernel, everything else a generic kernel.  The
+ * H / KV <= 8 take the tensor-core split-context kernel (kv_pool 16-byte aligned, else RSD_ERR_ARG), everything else a generic kernel.  The
  * step loop keeps fp16 caches for bf16 models (same bytes, three more mantissa bits).                                   */
 int rsd_k_attn_decode(const float* q, const void* kv_pool, const int32_t* page_table, const int32_t* ctx_len,
                       float* out, int32_t B, int32_t H, int32_t KV, int32_t hd, int32_t max_pages,
@@ -324,8 +324,8 @@ size_t rsd_k_attn_decode_scratch_bytes(int32_t B, int32_t H, int32_t hd, int32_t
  * skipped) and attends positions [0, tok_pos[t]] of that row, whose keys and values (those of the new
  * tokens included) are already in the pages.  q and out are [T, H, hd] fp32.  fp16 caches with
  * hd = 128, H / KV <= 8 and T >= 64 take the tcgen05 kernel (operands and accumulators in tensor
- * memory, pages fetched by TMA: kv_pool must be 16-byte aligned), other 16-bit caches with
- * H / KV <= 8 the mma.sync kernel, everything else the generic one.  (Inside rsd_prefill / rsd_step
+ * memory, pages fetched by TMA), other 16-bit caches with
+ * H / KV <= 8 the mma.sync kernel, both with kv_pool 16-byte aligned (else RSD_ERR_ARG), everything else the generic one.  (Inside rsd_prefill / rsd_step
  * a bounded device-side wait of the tcgen05 kernel that runs out makes the call return
  * RSD_ERR_TIMEOUT; this stand-alone entry has no error word to report it in.)                      */
 int rsd_k_attn_chunk(const float* q, const void* kv_pool, const int32_t* page_table, const int32_t* tok_row,

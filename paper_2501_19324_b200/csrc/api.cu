@@ -185,6 +185,9 @@ bool kv_extended_for(const rsd_model& m, int setting) {
   return setting == 1 || (setting == 0 && m.n_layers > 48);
 }
 
+// The generic attention (fp32 caches, wide groups) reads a pool off a 16-byte boundary element by element, the others copy 16 bytes at a time.
+bool kv_pool_ok(int kv_dtype, int H, int KV, const void* pool) { return kv_dtype == 0 || H / KV > 8 || ((uintptr_t)pool & 15) == 0; }
+
 size_t kv_pool_bytes(const rsd_model& m, int pages, int kv_extended) {
   const size_t elem = m.dtype == RSD_BF16 ? 2 : 4;
   const size_t blocks = kv_extended_for(m, kv_extended) ? 4 : 2;   // keys, values (, their low halves)
@@ -1161,8 +1164,7 @@ int rsd_load_models(rsd_ctx* c, const rsd_model* draft, const rsd_model* prm, co
     M.w16_layer = layer_weight_elems(M.m);
     M.n_params = count_params(M.m);
     M.kv_pool = (char*)c->cfg.kv_pool[w];
-    // the generic attention (fp32 caches, wide groups) reads a pool off a 16-byte boundary element by element, the others copy 16 bytes at a time
-    if (M.kv_dtype != 0 && M.m.n_heads / M.m.n_kv_heads <= 8 && ((uintptr_t)M.kv_pool & 15))
+    if (!kv_pool_ok(M.kv_dtype, M.m.n_heads, M.m.n_kv_heads, M.kv_pool))
       return fail(c, RSD_ERR_ARG, "KV pool of a 16-bit cache must be 16-byte aligned%s");
     const size_t page_bytes = (size_t)(M.kv_dtype == 3 ? 4 : 2) * M.m.n_kv_heads * kPageTokens * M.m.head_dim * M.elem;
     int pages = (int)std::min<size_t>(c->cfg.kv_bytes[w] / (page_bytes * L), (size_t)c->B_max * max_pages);
@@ -1639,6 +1641,7 @@ int rsd_k_attn_decode(const float* q, const void* kv_pool, const int32_t* page_t
   if (hd != 64 && hd != 128) return RSD_ERR_UNSUPPORTED;
   if (scratch_bytes < attn_decode_scratch_bytes(B, H, hd, max_pages * kPageTokens) || !scratch) return RSD_ERR_ARG;
   if (dtype < 0 || dtype > 3) return RSD_ERR_ARG;
+  if (!kv_pool_ok(dtype, H, KV, kv_pool)) return RSD_ERR_ARG;
   KCU(launch_attn_decode(dtype, q, kv_pool, page_table, max_pages, nullptr, ctx_len, 0, out, nullptr, RSD_F32, B, H, KV, hd,
                          max_pages * kPageTokens, scratch, scratch_bytes, nullptr, (cudaStream_t)cuda_stream));
   return RSD_OK;
@@ -1651,6 +1654,7 @@ int rsd_k_attn_chunk(const float* q, const void* kv_pool, const int32_t* page_ta
     return RSD_ERR_ARG;
   if (hd != 64 && hd != 128) return RSD_ERR_UNSUPPORTED;
   if (dtype < 0 || dtype > 3) return RSD_ERR_ARG;
+  if (!kv_pool_ok(dtype, H, KV, kv_pool)) return RSD_ERR_ARG;
   PassView p{nullptr, tok_row, tok_pos, T, nullptr};
   KvView kv{const_cast<void*>(kv_pool), page_table, max_pages};
   KCU(launch_attn_chunk(dtype, q, p, kv, out, nullptr, RSD_F32, H, KV, hd, (cudaStream_t)cuda_stream));

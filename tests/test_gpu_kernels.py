@@ -629,6 +629,21 @@ def test_generic_attention_pool_may_start_anywhere(dtype, hd, H, KV):
     assert torch.equal(rb.k_attn_decode(q, moved, table, lens, KV), want)
 
 
+@pytest.mark.parametrize("dtype,ext", [(torch.float16, False), (torch.bfloat16, False), (torch.float16, True)])
+def test_tensor_core_attention_refuses_pools_off_a_boundary(dtype, ext):
+    """These kernels copy 16 bytes at a time: a pool one element off is an argument error, before anything runs."""
+    H, KV, hd = 8, 2, 64
+    pool = torch.zeros(4 * KV * 16 * hd + 8, dtype=dtype, device="cuda")[1:]
+    q = torch.zeros(1, H, hd, device="cuda")
+    one = torch.ones(1, dtype=torch.int32, device="cuda")
+    table = torch.zeros(1, 1, dtype=torch.int32, device="cuda")
+    for call in (lambda: rb.k_attn_decode(q, pool, table, one, KV, ext=ext),
+                 lambda: rb.k_attn_chunk(q, pool, table, torch.zeros_like(one), one, KV, ext=ext)):
+        with pytest.raises(rb.RsdError) as e:
+            call()
+        assert e.value.code == -1
+
+
 @pytest.mark.parametrize("hd,H,KV", [(128, 12, 2), (128, 64, 8), (64, 4, 2), (128, 16, 1)])
 def test_extended_precision_attention(hd, H, KV):
     """fp16 cache with keys and values kept as hi + lo pairs, queries and softmax weights as hi + lo
