@@ -385,6 +385,19 @@ int rsd_k_swiglu(const float* gu, void* out, int32_t T, int32_t F, int32_t dtype
  * RSD_ERR_UNSUPPORTED for other shapes.                                                         */
 int rsd_k_gemm_gu(const void* Wgu, const void* x, const void* x_lo, void* act_hi, void* act_lo, int32_t M, int32_t F,
                   int32_t K, void* scratch, size_t scratch_bytes, void* cuda_stream);
+/* Products of decode passes of up to eight rows together with the small step behind them, as such passes run them (bf16 weights, operands
+ * as hi + lo pairs): y[M, N] += (x + x_lo)[M, K] * W[N, K]^T; hi = bf16(y * gain), lo = bf16(y * gain - hi), both [M, N]; ssq [M, N / 8] = sums of
+ * squares of y over eight columns.  gain [N] bf16.  1 <= M <= 8, N % 16 == 0, K % 64 == 0 (else RSD_ERR_UNSUPPORTED); W, x and x_lo 16-byte
+ * aligned, hi and lo not x and x_lo.                                                            */
+int rsd_k_gemm_rows(const void* W, const void* x, const void* x_lo, float* y, const void* gain, void* hi, void* lo, float* ssq,
+                    int32_t M, int32_t N, int32_t K, void* cuda_stream);
+/* ... and for queries, keys and values: qkv[M, (H + 2 KV) hd] = (x + x_lo) * W^T / sqrt(sum_c ssq[m, c] / K + eps), c < n_chunks; queries and keys
+ * rotated with rope [positions, hd / 2] (cos, sin) at tok_pos[m]; q [M, H, hd] fp32, the key and the value at that position of row
+ * tok_row[m] in its page of kv_pool (RSD_F16 pages, with ext RSD_F16_EXT).  tok_row[m] < 0: nothing is written for m.  hd 64 or 128. */
+int rsd_k_gemm_rows_qkv(const void* W, const void* x, const void* x_lo, const float* ssq, int32_t n_chunks, float eps,
+                        const int32_t* tok_row, const int32_t* tok_pos, const float* rope, float* q, void* kv_pool,
+                        const int32_t* page_table, int32_t M, int32_t H, int32_t KV, int32_t hd, int32_t K, int32_t max_pages,
+                        int32_t ext, void* cuda_stream);
 /* token[b] = argmax over v < v_limit of logits[b, v] / T + g, g = -log(-log u) with u the Philox
  * uniform of (seed; counter = (v / 4, pos[b] + 1, row[b], model_id), word v % 4), or the plain
  * argmax when temperature == 0; ties to the lowest id.  pos[b] is the position of the token fed to

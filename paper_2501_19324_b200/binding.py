@@ -58,7 +58,7 @@ EXPORTS = ["rsd_query_sizes", "rsd_create", "rsd_load_models", "rsd_prefill", "r
            "rsd_reset", "rsd_destroy", "rsd_last_error", "rsd_debug_force", "rsd_debug_force_sd", "rsd_debug_get_logits",
            "rsd_debug_get_sampled", "rsd_debug_get_state", "rsd_debug_gemm_timing", "rsd_debug_gemm_timing_dense", "rsd_debug_launch_count", "rsd_debug_fail_iteration", "rsd_debug_mega_profile", "rsd_debug_phase_ms", "rsd_k_gemm", "rsd_k_gemm_scratch_bytes", "rsd_debug_gemm_wait_probe", "rsd_debug_attn_wait_probe",
            "rsd_k_attn_decode", "rsd_k_attn_decode_scratch_bytes", "rsd_k_attn_chunk", "rsd_k_gate_compact", "rsd_k_gate_compact_static", "rsd_k_gate_compact_static_error", "rsd_k_rmsnorm",
-           "rsd_k_rope", "rsd_k_swiglu", "rsd_k_gemm_gu", "rsd_k_sample", "rsd_k_philox"]
+           "rsd_k_rope", "rsd_k_swiglu", "rsd_k_gemm_gu", "rsd_k_gemm_rows", "rsd_k_gemm_rows_qkv", "rsd_k_sample", "rsd_k_philox"]
 
 _lib = None
 
@@ -114,6 +114,8 @@ def lib():
         L.rsd_k_rope.argtypes = [vp, vp, c_int32, c_int32, c_int32, c_float, vp]
         L.rsd_k_swiglu.argtypes = [vp, vp, c_int32, c_int32, c_int32, vp]
         L.rsd_k_gemm_gu.argtypes = [vp, vp, vp, vp, vp, c_int32, c_int32, c_int32, vp, c_size_t, vp]
+        L.rsd_k_gemm_rows.argtypes = [vp] * 8 + [c_int32] * 3 + [vp]
+        L.rsd_k_gemm_rows_qkv.argtypes = [vp] * 4 + [c_int32, c_float] + [vp] * 6 + [c_int32] * 7 + [vp]
         L.rsd_k_sample.argtypes = [vp, c_int32, c_int32, c_int32, c_float, c_uint64, c_int32, vp, vp, vp, vp, c_size_t, vp]
         L.rsd_k_philox.argtypes = [vp, vp, vp, c_int32, vp]
         _lib = L
@@ -441,6 +443,28 @@ def k_gemm_gu(Wgu, x_hi, x_lo):
     scratch = torch.zeros(nbytes, dtype=torch.uint8, device=x_hi.device)
     _check(lib().rsd_k_gemm_gu(_ptr(Wgu), _ptr(x_hi), _ptr(x_lo), _ptr(hi), _ptr(lo), M, F, K, _ptr(scratch), nbytes, _stream()))
     return hi, lo
+
+
+def k_gemm_rows(W, x_hi, x_lo, y, gain):
+    """y += (x_hi + x_lo) W^T in place (fp32), up to eight rows: returns (hi, lo, ssq) of the next product's operand y * gain."""
+    import torch
+    M, K = x_hi.shape
+    N = W.shape[0]
+    hi, lo = (torch.zeros(M, N, dtype=torch.bfloat16, device=y.device) for _ in range(2))
+    ssq = torch.zeros(M, N // 8, dtype=torch.float32, device=y.device)
+    _check(lib().rsd_k_gemm_rows(_ptr(W), _ptr(x_hi), _ptr(x_lo), _ptr(y), _ptr(gain), _ptr(hi), _ptr(lo), _ptr(ssq), M, N, K, _stream()))
+    return hi, lo, ssq
+
+
+def k_gemm_rows_qkv(W, x_hi, x_lo, ssq, eps, tok_row, tok_pos, rope, kv_pool, page_table, H, KV, hd, ext=False):
+    """qkv product of up to eight rows with norm, rotation and page write: returns the queries [M, H, hd]; kv_pool is updated."""
+    import torch
+    M, K = x_hi.shape
+    q = torch.zeros(M, H, hd, dtype=torch.float32, device=x_hi.device)
+    _check(lib().rsd_k_gemm_rows_qkv(_ptr(W), _ptr(x_hi), _ptr(x_lo), _ptr(ssq), ssq.shape[1], eps, _ptr(tok_row), _ptr(tok_pos),
+                                     _ptr(rope), _ptr(q), _ptr(kv_pool), _ptr(page_table), M, H, KV, hd, K, page_table.shape[1],
+                                     int(ext), _stream()))
+    return q
 
 
 def k_sample(logits, v_limit, temperature, seed, model_id, row, pos):

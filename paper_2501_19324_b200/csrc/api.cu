@@ -1715,6 +1715,29 @@ int rsd_k_gemm_gu(const void* Wgu, const void* x, const void* x_lo, void* act_hi
   return RSD_OK;
 }
 
+int rsd_k_gemm_rows(const void* W, const void* x, const void* x_lo, float* y, const void* gain, void* hi, void* lo, float* ssq,
+                    int32_t M, int32_t N, int32_t K, void* cuda_stream) {
+  if (!W || !x || !x_lo || !y || !gain || !hi || !lo || !ssq) return RSD_ERR_ARG;
+  if (((uintptr_t)W | (uintptr_t)x | (uintptr_t)x_lo) & 15) return RSD_ERR_ARG;
+  if (!rows_gemm_supported(M, N, K)) return RSD_ERR_UNSUPPORTED;
+  KCU(launch_gemm_rows_residual(W, x, x_lo, y, gain, hi, lo, ssq, M, N, K, nullptr, (cudaStream_t)cuda_stream));
+  return RSD_OK;
+}
+
+int rsd_k_gemm_rows_qkv(const void* W, const void* x, const void* x_lo, const float* ssq, int32_t n_chunks, float eps,
+                        const int32_t* tok_row, const int32_t* tok_pos, const float* rope, float* q, void* kv_pool,
+                        const int32_t* page_table, int32_t M, int32_t H, int32_t KV, int32_t hd, int32_t K, int32_t max_pages,
+                        int32_t ext, void* cuda_stream) {
+  if (!W || !x || !x_lo || !ssq || !tok_row || !tok_pos || !rope || !q || !kv_pool || !page_table) return RSD_ERR_ARG;
+  if (((uintptr_t)W | (uintptr_t)x | (uintptr_t)x_lo) & 15 || ((uintptr_t)rope & 7)) return RSD_ERR_ARG;
+  if (n_chunks < 1 || H < 1 || KV < 1 || max_pages < 1 || (hd != 64 && hd != 128)) return RSD_ERR_ARG;
+  if (!rows_gemm_supported(M, (H + 2 * KV) * hd, K)) return RSD_ERR_UNSUPPORTED;
+  PassView p{nullptr, tok_row, tok_pos, M, nullptr};
+  KCU(launch_gemm_rows_qkv(W, x, x_lo, RowScale{ssq, n_chunks, 1.f / (float)K, eps}, p, q, KvView{kv_pool, page_table, max_pages, ext ? 1 : 0},
+                           (const float2*)rope, H, KV, hd, K, (cudaStream_t)cuda_stream));
+  return RSD_OK;
+}
+
 int rsd_k_sample(const float* logits, int32_t B, int32_t V, int32_t v_limit, float temperature, uint64_t seed,
                  int32_t model_id, const int32_t* row, const int32_t* pos, int32_t* token, void* scratch,
                  size_t scratch_bytes, void* cuda_stream) {

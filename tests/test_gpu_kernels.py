@@ -757,6 +757,78 @@ def test_paired_gemm_of_65_to_128_rows(M, N, K):
     np.testing.assert_allclose(acc, want + y0, rtol=0, atol=tol)
 
 
+def _operand_pair(rng, M, K):
+    x = dev(rng.normal(size=(M, K)).astype(np.float32))
+    hi = x.to(torch.bfloat16)
+    lo = (x - hi.float()).to(torch.bfloat16)
+    return hi, lo, (hi.double() + lo.double()).cpu().numpy()
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 16, 64), (8, 576, 448), (3, 1536, 1536), (8, 512, 1408), (5, 3584, 3584), (2, 32, 8960)])
+def test_rows_gemm_that_adds_into_the_residual(M, N, K):
+    """The decode product of few rows that completes the residual stream: one chunk of K a warp, fewer chunks than warps, more than the
+    ring's slots; the bound of the test above.  The operand and the sums of squares are exactly those of the y written."""
+    rng = np.random.default_rng(M * 5 + N)
+    W = ri.cpu_tensor(2, 9, N, K, True)
+    hi, lo, x = _operand_pair(rng, M, K)
+    y0 = rng.normal(size=(M, N)).astype(np.float32)
+    gain = dev((1 + 0.1 * rng.normal(size=N)).astype(np.float32), torch.bfloat16)
+    y = dev(y0)
+    out_hi, out_lo, ssq = rb.k_gemm_rows(dev(W, torch.bfloat16), hi, lo, y, gain)
+    np.testing.assert_allclose(y.cpu().numpy(), y0 + x @ W.astype(np.float64).T, rtol=0, atol=3e-5 * np.sqrt(K))
+    v = y * gain.float()
+    assert torch.equal(out_hi, v.to(torch.bfloat16)) and torch.equal(out_lo, (v - out_hi.float()).to(torch.bfloat16))
+    want = (y.double() ** 2).view(M, N // 8, 8).sum(2)
+    assert ((ssq.double() - want).abs() <= 8 * 2.0 ** -24 * want).all()          # eight roundings of positive terms
+
+
+@pytest.mark.parametrize("M,H,KV,hd,K,chunk,ext", [(1, 1, 1, 64, 64, 8, False), (8, 7, 1, 128, 576, 256, False), (3, 12, 2, 128, 1536, 8, True),
+                                                   (5, 8, 8, 64, 512, 8, True)])
+def test_rows_gemm_of_queries_keys_and_values(M, H, KV, hd, K, chunk, ext):
+    """... and the one that ends in queries and cache pages: sums of squares per 8 and per 256 columns, first, last and middle slots of a
+    page, one idle row, both caches.  The bound of the product grows by sqrt(2) where two values turn; keys and values carry fp16's rounding."""
+    rng = np.random.default_rng(M + K)
+    W = ri.cpu_tensor(2, 9, (H + 2 * KV) * hd, K, True)
+    hi, lo, x = _operand_pair(rng, M, K)
+    ssq = rng.uniform(0.5, 1.5, size=(M, -(-K // chunk))).astype(np.float32) * min(chunk, K)
+    eps = 1e-6
+    pos = np.array([15, 16, 40, 0, 33, 31, 7, 47][:M], np.int32)
+    row = np.arange(M, dtype=np.int32)
+    if M > 2:
+        row[1] = -1
+    table = rng.permutation(3 * M).reshape(M, 3).astype(np.int32)
+    parts = 4 if ext else 2
+    pool = torch.full((3 * M, parts, KV * 16 * hd), 7.0, dtype=torch.float16, device="cuda")
+    ang = np.arange(48)[:, None] * 1e4 ** (-2.0 * np.arange(hd // 2) / hd)
+    rope = np.stack([np.cos(ang), np.sin(ang)], -1).astype(np.float32)
+    q = rb.k_gemm_rows_qkv(dev(W, torch.bfloat16), hi, lo, dev(ssq), eps, dev(row), dev(pos), dev(rope), pool, dev(table), H, KV, hd, ext)
+    qkv = x @ W.astype(np.float64).T / np.sqrt(ssq.astype(np.float64).sum(1, keepdims=True) / K + eps)
+    qkv = qkv.reshape(M, H + 2 * KV, hd)
+    c, s = (rope[pos].astype(np.float64)[:, None, :, i] for i in (0, 1))
+    a, b = qkv[:, :H + KV, :hd // 2].copy(), qkv[:, :H + KV, hd // 2:].copy()
+    qkv[:, :H + KV, :hd // 2], qkv[:, :H + KV, hd // 2:] = a * c - b * s, b * c + a * s
+    tol = 3e-5 * np.sqrt(2 * K)
+    got = pool.cpu().numpy()
+    touched = np.zeros(got.shape, bool)
+    for m in range(M):
+        if row[m] < 0:
+            assert not q[m].any()
+            continue
+        np.testing.assert_allclose(q[m].cpu().numpy(), qkv[m, :H], rtol=0, atol=tol)
+        pg, slot = table[m, pos[m] // 16], pos[m] % 16
+        keys = [got[pg, i].reshape(KV, 16, hd)[:, slot].astype(np.float64) for i in range(0, parts, 2)]
+        vals = [got[pg, i].reshape(KV, hd, 16)[:, :, slot].astype(np.float64) for i in range(1, parts, 2)]
+        for i in range(parts):
+            t = touched[pg, i].reshape((KV, hd, 16) if i & 1 else (KV, 16, hd))
+            if i & 1:
+                t[:, :, slot] = True
+            else:
+                t[:, slot] = True
+        for have, want in ((sum(keys), qkv[m, H:H + KV]), (sum(vals), qkv[m, H + KV:])):
+            np.testing.assert_allclose(have, want, rtol=2.0 ** (-21 if ext else -11), atol=tol + 2.0 ** -24)
+    assert (got[~touched] == 7.0).all()
+
+
 @pytest.mark.parametrize("M,N,K", [(2100, 2304, 3072), (2049, 2305, 3080), (512, 18944, 3136), (300, 18817, 3072), (4100, 1300, 1032)])
 @pytest.mark.parametrize("kind", ["fp16", "bf16", "pairs"])
 def test_dense_gemm_on_pairs_of_ctas(M, N, K, kind):
