@@ -553,9 +553,10 @@ sgemm_kernel(const float* __restrict__ W, const float* __restrict__ X, float* Y,
   }
 }
 
-// Both take as long along K, so that rows times columns decide.  us, eight rows at a time / tiled: 96 x 512 x 256 9.2 / 5.8, 64 x 512 x
-// 1376 24.4 / 23.2, 96 x 256 x 688 12.5 / 12.7, 17 x 2752 x 512 13.7 / 12.6, 48 x 512 x 512 9.3 / 9.9; 256 x 2752 x 512 153 / 32.
-static bool sgemm_pays(int M, int N) { return M > 16 && (long)M * N >= 32768; }
+// Both take as long along K, so that rows times columns decide.  us, eight rows at a time / tiled: 128 x 256 x 256 5.6 / 6.3, 64 x 512 x 1376
+// 24.2 / 25.6, 72 x 512 x 1376 25.2 / 25.7, 80 x 512 x 1376 29.8 / 25.7, 160 x 256 x 688 18.2 / 13.9, 17 x 2752 x 512 13.7 / 14.7, 20 x 2752 x 512
+// 15.5 / 14.7, 48 x 1024 x 1024 24.1 / 24.8, 96 x 512 x 256 9.2 / 6.3, 256 x 2752 x 512 154 / 39.
+static bool sgemm_pays(int M, int N) { return M > 16 && (long)M * N >= 40000; }
 
 // K splits over the warps of a block.
 static int simt_splits(int dtype, int M, int N, int K) {
