@@ -205,7 +205,8 @@ int rsd_get_target_step_rewards(rsd_ctx*, float* out);
  * flops_paper follows Section 3.3: 2N per inference token of an N-parameter model (all
  * parameters, embedding and head included), counting every token the draft or the target
  * generated (discarded draft steps too) and every token the PRM processed.  flops_all_tokens
- * bills 2N for every token pushed through any model, prompts and catch-up included.         */
+ * bills 2N for every token pushed through any model, prompts and catch-up included: a convention, all of the model's
+ * parameters whether a pass needs them or not (passes run for their keys and values leave out head and most of the last layer). */
 typedef struct {
   uint64_t gen_tokens[3];
   uint64_t ingest_tokens[3];

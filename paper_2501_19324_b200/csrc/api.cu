@@ -526,8 +526,8 @@ int forward_pass_f16(rsd_ctx* c, int which, PassView p, bool cache_only, cudaStr
   return RSD_OK;
 }
 
-// cache_only: the pass is run for its keys and values alone; the last layer ends with them (what follows them there, the residual
-// stream, nobody reads: a 28th of such a pass, a 14th at half depth).
+// cache_only: the pass is run for its keys and values alone; the last layer ends with them: its norm, qkv product, rotation and page
+// write run, attention, wo and MLP, which is most of a layer, do not (nobody reads the residual stream behind them).
 int forward_pass(rsd_ctx* c, int which, PassView p, cudaStream_t s, bool cache_only = false) {
   const ModelHost& M = c->mdl[which];
   const rsd_model& m = M.m;

@@ -547,9 +547,12 @@ size_t attn_decode_scratch_bytes(int B, int H, int hd, int max_ctx) {
 
 // Whether a pass that takes the qkv product runs one CTA of sixteen warps per (slot, KV head): 97 to 148 of them, one per SM and no cluster,
 // and few enough pages that a warp walks four at most.  14-layer iterations, us, split contexts with a rotation kernel ahead / so:
-// 64 rows, 12 / 2 heads, 256 cached tokens 849 / 773, 500 tokens 844 / 805; 32 rows, 28 / 4 heads 1631 / 1598 and 1748 / 1725; with
+// 64 rows, 12 / 2 heads, 256 cached tokens 849 / 773, 500 tokens 844 / 805; 32 rows, 28 / 4 heads 1631 / 1598 and 1748 / 1725; near the lower
+// limit 49 rows, 12 / 2 heads, 100 and 256 tokens 747 / 730 and 829 / 787, 100 rows, 8 / 1 heads 597 / 544, 25 rows, 28 / 4 heads 1588 / 1589, 13 rows, 64 / 8
+// heads (8 layers) 2804 / 2740, 16 / 8 heads of 64 221 / 207.  Groups of one head mostly gain (8 layers: 37 rows, 4 / 4 heads, 420 tokens 282 / 245, 18
+// rows, 8 / 8, 160 tokens 239 / 228) but not all (13 rows, 8 / 8, 64, 320 and 480 tokens 209 / 210, 236 / 242 and 261 / 250; 50 rows, 2 / 2, 64 tokens 198 / 203).  With
 // fewer (slot, KV head) pairs nothing or a loss (32 rows, 12 / 2 heads, 500 tokens 688 / 703), with more, four warps are better (64 rows, 28 / 4
-// heads 1951 / 2031).
+// heads 1951 / 2031).  Heads of 128 dims spill 108 bytes at the 128 registers that 512 threads leave; in those times.
 static bool wide_ctas(int kv_dtype, int rows, int KV, int max_ctx) {
   return kv_dtype == 2 && rows * KV > 96 && rows * KV <= 148 && max_ctx <= 64 * kPageTokens;
 }
