@@ -783,6 +783,21 @@ def test_rows_gemm_that_adds_into_the_residual(M, N, K):
     assert ((ssq.double() - want).abs() <= 8 * 2.0 ** -24 * want).all()          # eight roundings of positive terms
 
 
+@pytest.mark.parametrize("M,N,K", [(8, 512, 1408), (1, 3584, 3584), (1, 512, 8960), (8, 16, 12288)])
+def test_rows_gemm_rounds_no_more_than_a_k_split(M, N, K):
+    """Against fp64 the product of few rows errs no more than the K split of the same operands.  An element's error varies, the norm over
+    128 and more of them by 1 / sqrt(256) = 6 % at most; twice that is allowed."""
+    rng = np.random.default_rng(K)
+    W = dev(ri.cpu_tensor(2, 9, N, K, True), torch.bfloat16)
+    hi, lo, x = _operand_pair(rng, M, K)
+    exact = x @ W.double().cpu().numpy().T
+    rows, split = torch.zeros(M, N, device="cuda"), torch.zeros(M, N, device="cuda")
+    rb.k_gemm_rows(W, hi, lo, rows, torch.ones(N, dtype=torch.bfloat16, device="cuda"))
+    rb.k_gemm(W, hi, y=split, accumulate=True, impl=2, x_lo=lo)
+    errs = [np.linalg.norm(y.cpu().numpy() - exact) for y in (rows, split)]
+    assert errs[0] <= 1.12 * errs[1], errs
+
+
 @pytest.mark.parametrize("M,H,KV,hd,K,chunk,ext", [(1, 1, 1, 64, 64, 8, False), (8, 7, 1, 128, 576, 256, False), (3, 12, 2, 128, 1536, 8, True),
                                                    (5, 8, 8, 64, 512, 8, True)])
 def test_rows_gemm_of_queries_keys_and_values(M, H, KV, hd, K, chunk, ext):
