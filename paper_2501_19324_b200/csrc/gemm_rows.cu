@@ -54,7 +54,13 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
 // products are not what the time goes to.)  The order of the 32 values of K inside a half chunk is permuted for both alike, so that a
 // lane's share of either is one 16-byte piece of a row; every lane copies the pieces that it multiplies itself, through slots of
 // shared memory of its own: nothing to synchronise, no bank conflicts.
-template <int EPI>
+// LONG: more than kFold chunks a warp.  The MMAs' own additions are not rounded to nearest, so a long chain of them drifts: every kFold chunks the
+// accumulators go into sums that are (relative error against fp64, K split / one chain / so: 2 x 512 x 8960 2.0 / 4.6 / 1.3e-7, 1 x 3584 x
+// 3584 2.8 / 1.7 / 1.0e-7; at 1536 one chain of three chunks, 1.1 / 0.8).  The short form is one chain: with the sums in its loop an iteration
+// of 14 layers of the 1.5B shape at one row took 485 us instead of 482.
+constexpr int kFold = 4;
+
+template <int EPI, bool LONG>
 __global__ void __launch_bounds__(32 * kRowsWarps)
 gemm_rows_kernel(const __nv_bfloat16* W, const __nv_bfloat16* in, const __nv_bfloat16* in_lo, int M, int K, int n_stages,
                  const int32_t* n_active, const __grid_constant__ RowsArgs a) {
@@ -136,9 +142,6 @@ gemm_rows_kernel(const __nv_bfloat16* W, const __nv_bfloat16* in, const __nv_bfl
 #pragma unroll
     for (int c = 0; c < 4; ++c) sq[c] = warp < M && c * 32 + lane < a.rs.n_chunks ? a.rs.ssq[(size_t)warp * a.rs.n_chunks + c * 32 + lane] : 0.f;
   }
-  // The MMAs' own additions are not rounded to nearest: a long chain of them drifts.  Every kFold chunks the accumulators go into sums that are
-  // (relative error against fp64 with the old values added in, K split / one chain / so: 2 x 512 x 8960 2.0 / 4.6 / @E8960e-7, 1 x 3584 x 3584 2.8 / 1.7 / @E3584e-7).
-  constexpr int kFold = 4;
   float acc[kGroups][2][4], sum[kGroups][2] = {};
 #pragma unroll
   for (int u = 0; u < kGroups; ++u)
@@ -180,7 +183,7 @@ gemm_rows_kernel(const __nv_bfloat16* W, const __nv_bfloat16* in, const __nv_bfl
     fetch_x(i + kRowsStages, stage);
     commit();
     stage = stage + 1 == kRowsStages ? 0 : stage + 1;
-    if (i % kFold == kFold - 1) fold();
+    if (LONG && i % kFold == kFold - 1) fold();
   }
   fold();
   asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -253,11 +256,18 @@ cudaError_t launch_rows(const void* W, const void* in, const void* in_lo, int M,
   if (((uintptr_t)W & 15) || ((uintptr_t)in & 15) || ((uintptr_t)in_lo & 15)) return cudaErrorMisalignedAddress;
   const int stages = std::min(kRowsStages, (K / kChunk + kRowsWarps - 1) / kRowsWarps);    // slots; the waits count kRowsStages groups
   const int smem = kRowsWarps * stages * (kGroups * 1024 + M * 256);
-  static OncePerDevice configured;
-  const cudaError_t set = allow_smem(configured, gemm_rows_kernel<EPI>, kRowsWarps * kRowsStages * (kGroups * 1024 + kRowsMax * 256));
-  if (set != cudaSuccess) return set;
-  RSD_LAUNCH((gemm_rows_kernel<EPI>), N / (8 * kGroups), 32 * kRowsWarps, smem, s, (const __nv_bfloat16*)W, (const __nv_bfloat16*)in,
-             (const __nv_bfloat16*)in_lo, M, K, stages, n_active, a);
+  constexpr int max_smem = kRowsWarps * kRowsStages * (kGroups * 1024 + kRowsMax * 256);
+#define RSD_ROWS(LONG)                                                                                                                          \
+  do {                                                                                                                                          \
+    static OncePerDevice configured;                                                                                                            \
+    const cudaError_t set = allow_smem(configured, gemm_rows_kernel<EPI, LONG>, max_smem);                                                       \
+    if (set != cudaSuccess) return set;                                                                                                         \
+    RSD_LAUNCH((gemm_rows_kernel<EPI, LONG>), N / (8 * kGroups), 32 * kRowsWarps, smem, s, (const __nv_bfloat16*)W, (const __nv_bfloat16*)in,    \
+               (const __nv_bfloat16*)in_lo, M, K, stages, n_active, a);                                                                          \
+  } while (0)
+  if (K > kFold * kRowsWarps * kChunk) RSD_ROWS(true);
+  else RSD_ROWS(false);
+#undef RSD_ROWS
   return launched(1);
 }
 
