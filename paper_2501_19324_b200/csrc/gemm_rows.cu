@@ -57,7 +57,7 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
 // LONG: more than kFold chunks a warp.  The MMAs' own additions are not rounded to nearest, so a long chain of them drifts: every kFold chunks the
 // accumulators go into sums that are (relative error against fp64, K split / one chain / so: 2 x 512 x 8960 2.0 / 4.6 / 1.3e-7, 1 x 3584 x
 // 3584 2.8 / 1.7 / 1.0e-7; at 1536 one chain of three chunks, 1.1 / 0.8).  The short form is one chain: with the sums in its loop an iteration
-// of 14 layers of the 1.5B shape at one row took 485 us instead of 482.
+// of 14 layers of the 1.5B shape at one row took 489 us instead of 487, of the small models at eight rows 68.0 instead of 67.5.
 constexpr int kFold = 4;
 
 template <int EPI, bool LONG>
@@ -142,24 +142,13 @@ gemm_rows_kernel(const __nv_bfloat16* W, const __nv_bfloat16* in, const __nv_bfl
 #pragma unroll
     for (int c = 0; c < 4; ++c) sq[c] = warp < M && c * 32 + lane < a.rs.n_chunks ? a.rs.ssq[(size_t)warp * a.rs.n_chunks + c * 32 + lane] : 0.f;
   }
-  float acc[kGroups][2][4], sum[kGroups][2] = {};
+  float acc[kGroups][2][4], sum[LONG ? kGroups : 1][2] = {};
 #pragma unroll
   for (int u = 0; u < kGroups; ++u)
 #pragma unroll
     for (int j = 0; j < 2; ++j)
 #pragma unroll
       for (int i = 0; i < 4; ++i) acc[u][j][i] = 0.f;
-  auto fold = [&]() {
-#pragma unroll
-    for (int u = 0; u < kGroups; ++u) {
-#pragma unroll
-      for (int i = 0; i < 2; ++i) sum[u][i] += (acc[u][0][i] + acc[u][1][i]) + (acc[u][0][i + 2] + acc[u][1][i + 2]);
-#pragma unroll
-      for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[u][j][i] = 0.f;
-    }
-  };
   int stage = 0;
   for (int i = 0; i < mine; ++i) {
     // groups in order: the weights of the first chunks, their operands, then one of both per chunk
@@ -183,12 +172,25 @@ gemm_rows_kernel(const __nv_bfloat16* W, const __nv_bfloat16* in, const __nv_bfl
     fetch_x(i + kRowsStages, stage);
     commit();
     stage = stage + 1 == kRowsStages ? 0 : stage + 1;
-    if (LONG && i % kFold == kFold - 1) fold();
+    if (LONG && i % kFold == kFold - 1) {
+#pragma unroll
+      for (int u = 0; u < kGroups; ++u) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) sum[LONG ? u : 0][k] += (acc[u][0][k] + acc[u][1][k]) + (acc[u][0][k + 2] + acc[u][1][k + 2]);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) acc[u][j][k] = 0.f;
+      }
+    }
   }
-  fold();
   asm volatile("cp.async.wait_group 0;" ::: "memory");
 #pragma unroll
-  for (int u = 0; u < kGroups; ++u) *reinterpret_cast<float2*>(&red[warp][u][g][2 * t]) = make_float2(sum[u][0], sum[u][1]);
+  for (int u = 0; u < kGroups; ++u) {
+    float2 v = make_float2((acc[u][0][0] + acc[u][1][0]) + (acc[u][0][2] + acc[u][1][2]), (acc[u][0][1] + acc[u][1][1]) + (acc[u][0][3] + acc[u][1][3]));
+    if (LONG) v = make_float2(sum[LONG ? u : 0][0] + v.x, sum[LONG ? u : 0][1] + v.y);
+    *reinterpret_cast<float2*>(&red[warp][u][g][2 * t]) = v;
+  }
   if (EPI == kQkv) {
     float s = (sq[0] + sq[1]) + (sq[2] + sq[3]);
     if (warp < M)
