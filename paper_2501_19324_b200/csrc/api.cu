@@ -407,7 +407,7 @@ int drain_gemm_events(rsd_ctx* c) {
 // `pending` (nullable): the caller's next kernel adds up K-split partial sums itself, so the GEMM may
 // leave them in the scratch; *pending then describes them (splits == 1: y is complete).
 int gemm(rsd_ctx* c, const ModelHost& M, const void* W, const void* xin, const void* xin_lo, float* y, int Mrows, int N,
-         int K, int accumulate, const int32_t* n_active, SplitSum* pending, cudaStream_t s, RowScale rs = RowScale(), bool few_sums = false) {
+         int K, int accumulate, const int32_t* n_active, SplitSum* pending, cudaStream_t s, RowScale rs = RowScale()) {
   // ragged passes: every stride-th GEMM; decode: every GEMM of the iterations chosen by decode_phase
   const bool pick = c->in_decode ? c->time_this_iter
                                  : (c->time_stride > 0 && (c->gemm_calls++ % (uint64_t)c->time_stride) == 0);
@@ -415,7 +415,7 @@ int gemm(rsd_ctx* c, const ModelHost& M, const void* W, const void* xin, const v
   if (timed) CU(cudaEventRecord(c->ev[2 * c->ev_used], s));
   int splits = 1;
   CU(launch_gemm(M.m.dtype, W, xin, M.split ? xin_lo : nullptr, y, Mrows, N, K, accumulate, 0, c->gemm_scratch,
-                 c->gemm_scratch_bytes, n_active, pending ? &splits : nullptr, s, rs, few_sums));
+                 c->gemm_scratch_bytes, n_active, pending ? &splits : nullptr, s, rs));
   if (pending) { pending->splits = splits; pending->partials = gemm_partials(c->gemm_scratch); }
   if (timed) {
     CU(cudaEventRecord(c->ev[2 * c->ev_used + 1], s));
@@ -614,7 +614,7 @@ int forward_decode_fused(rsd_ctx* c, int which, PassView p, const void* final_ga
       });
       if (rc) return rc;
     } else {
-      rc = gemm(c, M, M.wqkv[l], c->h, c->h_lo, c->qkv, T, (H + 2 * KV) * hd, d, 0, p.n_active, &src.pending, s, rs, true);
+      rc = gemm(c, M, M.wqkv[l], c->h, c->h_lo, c->qkv, T, (H + 2 * KV) * hd, d, 0, p.n_active, &src.pending, s, rs);
       if (rc) return rc;
       rotates = attn_decode_takes_qkv(M.kv_dtype, m.dtype, T, H, KV, c->S, c->attn_rows_hint, c->pass_width);
       if (!rotates) CU(launch_rope_kv(M.kv_dtype, c->qkv, src.pending, p, c->q, kv, M.rope, H, KV, hd, s));

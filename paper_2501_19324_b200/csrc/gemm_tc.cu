@@ -977,8 +977,7 @@ int pick_rows(int M, bool split_operand) {
 
 struct TcPlan { int rows, mt, n_tiles, m_tiles, splits, kb_per_split; };
 
-// few_sums: the consumer adds the splits up in a step of few, latency-bound loads (the rotation of a qkv product).
-TcPlan plan_tc(int M, int N, int K, bool split_operand, bool few_sums) {
+TcPlan plan_tc(int M, int N, int K, bool split_operand) {
   TcPlan p;
   p.rows = pick_rows(M, split_operand);
   p.mt = split_operand ? 2 * p.rows : p.rows;
@@ -996,11 +995,10 @@ TcPlan plan_tc(int M, int N, int K, bool split_operand, bool few_sums) {
     // 65 to 128 rows with pairs are the decode passes of large batches: without the split the 12 tiles of a
     // 1536 x 8960 product leave 136 SMs idle (58 us at 128 rows; 11 us with 12 splits).
     splits = std::max(1, (p.rows <= 16 || !split_operand ? 2 * 148 : 148) / tiles);
-    // fewer and longer splits for the rotation, as long as they occupy half of the SMs (16 tiles, 24 k-blocks, 1 row: 12 / 6
-    // splits 522 / 514 us an iteration of 14 layers; but 8 tiles, 8 k-blocks: 51.6 / 54.6 an iteration of 2 with four / two).  An lm
-    // head of few tiles keeps the many (us an iteration, many / few: 4096 x 768 at 1 / 8 / 16 rows 55.6 / 57.4, 67.0 / 67.2, 78.3 / 77.4; 4096 x
-    // 1024 259 / 261, 313 / 315, 364 / 365; 6144 x 512 63.4 / 64.0, 69.4 / 69.8, 94.8 / 95.2)
-    splits = std::min(splits, std::max(1, few_sums && p.rows <= 16 && tiles * (total_kb / 4) >= 74 ? total_kb / 4 : total_kb / 2));
+    // (Splits of four k-blocks instead of two for the qkv product of up to 16 rows, whose sums the rotation adds up: an iteration of 14 layers of the
+    // 1.5B shape at 4 / 6 / 8 / 12 / 16 rows 496 / 505 / 530 / 558 / 569 us, with two 496 / 508 / 532 / 558 / 567; and the sums' error against fp64
+    // grows with the chain of MMAs, 1.4 -> 2.4e-7.)
+    splits = std::min(splits, std::max(1, total_kb / 2));
     splits = std::min(splits, kMaxSplitCtas / tiles);
     splits = std::max(splits, 1);
   }
@@ -1321,14 +1319,14 @@ const float* gemm_partials(const void* scratch) { return (const float*)((const c
 
 cudaError_t launch_gemm_tc(const void* W, const void* x, const void* x_lo, float* y, int M, int N, int K, int accumulate,
                            void* scratch, size_t scratch_bytes, const int32_t* n_active, int* deferred_splits,
-                           cudaStream_t s, RowScale rs, bool no_k_split, bool few_sums) {
+                           cudaStream_t s, RowScale rs, bool no_k_split) {
   if (deferred_splits) *deferred_splits = 1;
   if (M <= 0) return cudaSuccess;
   if (rs.ssq != nullptr && accumulate) return cudaErrorInvalidValue;
   if (!scratch || scratch_bytes < gemm_scratch_bytes(M)) return cudaErrorInvalidValue;
   if (((uintptr_t)W & 15) || ((uintptr_t)x & 15) || ((uintptr_t)x_lo & 15)) return cudaErrorMisalignedAddress;
   const bool split_operand = x_lo != nullptr;
-  TcPlan p = plan_tc(M, N, K, split_operand, few_sums);
+  TcPlan p = plan_tc(M, N, K, split_operand);
   if (no_k_split) { p.splits = 1; p.kb_per_split = (K + kTileK - 1) / kTileK; }
   if (rs.ssq != nullptr && p.rows > 128) return cudaErrorInvalidValue;   // one epilogue thread per x row of the tile
   if (deferred_splits) *deferred_splits = p.splits;
@@ -1420,12 +1418,12 @@ cudaError_t launch_gemm_gu_f16_dense(const void* Wgu16, const void* x16, void* a
 
 cudaError_t launch_gemm(int dtype, const void* W, const void* x, const void* x_lo, float* y, int M, int N, int K,
                         int accumulate, int impl, void* scratch, size_t scratch_bytes, const int32_t* n_active,
-                        int* deferred_splits, cudaStream_t s, RowScale rs, bool few_sums) {
+                        int* deferred_splits, cudaStream_t s, RowScale rs) {
   if (deferred_splits) *deferred_splits = 1;
   const bool tc_ok = gemm_tc_supported(dtype, M, N, K) && scratch && scratch_bytes >= gemm_scratch_bytes(M);
   // the tensor-core path wins for every M (an M = 1 GEMV included: TMA streaming beats the SIMT loads)
   if (impl == 2 || impl == 3 || (impl == 0 && tc_ok))
-    return launch_gemm_tc(W, x, x_lo, y, M, N, K, accumulate, scratch, scratch_bytes, n_active, deferred_splits, s, rs, impl == 3, few_sums);
+    return launch_gemm_tc(W, x, x_lo, y, M, N, K, accumulate, scratch, scratch_bytes, n_active, deferred_splits, s, rs, impl == 3);
   if (rs.ssq != nullptr) return cudaErrorNotSupported;
   return launch_gemm_simt(dtype, W, x, dtype == 1 ? x_lo : nullptr, y, M, N, K, accumulate, n_active, s);
 }

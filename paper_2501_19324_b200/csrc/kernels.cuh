@@ -74,10 +74,10 @@ size_t gemm_scratch_bytes(int M);
 size_t gemm_scratch_bytes_any();
 // deferred_splits (nullable): when given, a K-split launch leaves its partial sums in the scratch as
 // [splits][M][N] (gemm_partials) for the consumer kernel to add up, and reports the split count;
-// 1 means y holds the finished result.  few_sums: that kernel would rather have few of them (the rotation of a qkv product).
+// 1 means y holds the finished result.
 cudaError_t launch_gemm_tc(const void* W, const void* x, const void* x_lo, float* y, int M, int N, int K, int accumulate,
                            void* scratch, size_t scratch_bytes, const int32_t* n_active, int* deferred_splits,
-                           cudaStream_t s, RowScale rs = RowScale(), bool no_k_split = false, bool few_sums = false);
+                           cudaStream_t s, RowScale rs = RowScale(), bool no_k_split = false);
 const float* gemm_partials(const void* scratch);
 // Failure-path probe of the tensor-core GEMM: one CTA whose copies are never issued; its bounded wait runs out and
 // the error flag at byte 4096 of the scratch becomes -5.  W [128, 64] and x [16, 64] bf16, y [16, 128] fp32 (untouched).
@@ -97,7 +97,7 @@ cudaError_t launch_gemm_gu(const void* Wgu, const void* x, const void* x_lo, voi
 // impl: 0 = by shape, 1 = SIMT split-K GEMV, 2 = tcgen05, 3 = tcgen05 without a K split.
 cudaError_t launch_gemm(int dtype, const void* W, const void* x, const void* x_lo, float* y, int M, int N, int K,
                         int accumulate, int impl, void* scratch, size_t scratch_bytes, const int32_t* n_active,
-                        int* deferred_splits, cudaStream_t s, RowScale rs = RowScale(), bool few_sums = false);
+                        int* deferred_splits, cudaStream_t s, RowScale rs = RowScale());
 // x (+)= sum of the K-split partial sums [splits][M][d] (splits == 1: x is complete already); then the
 // un-normalised RMSNorm operand of the next GEMM: hi + lo = x * gain as two bf16 arrays, and the sums of
 // squares of x per 256-column chunk, ssq [M][ceil(d / 256)], for that GEMM's RowScale.
