@@ -91,6 +91,12 @@ struct rsd_ctx {
   void* mega_block[3] = {nullptr, nullptr, nullptr};
   int mega_B[3] = {0, 0, 0};
   int32_t* mega_sync = nullptr;
+  // decode phases in one launch (decode_resident.cu): draft, target; on where the model is small enough
+  ResidentPlan resident_plan[3];
+  ResidentShape resident_shape[3] = {};
+  void* resident_block[3] = {nullptr, nullptr, nullptr};
+  uint32_t* resident_slots[3] = {nullptr, nullptr, nullptr};
+  bool resident[3] = {false, false, false};
   unsigned long long* mega_prof[3] = {nullptr, nullptr, nullptr};   // RSD_DEBUG_MEGA_PROFILE
   char* pinned = nullptr;
   size_t pinned_bytes = 0;
@@ -231,6 +237,10 @@ bool wants_f16_dense(const rsd_config& cfg, const rsd_model& m, int which) {
   return layer_weight_elems(m) * 2 * (size_t)m.n_layers <= ((size_t)20 << 30);
 }
 
+ResidentShape resident_shape_of(const rsd_model& m) {
+  return ResidentShape{m.n_layers, m.d_model, m.n_heads, m.n_kv_heads, m.head_dim, m.d_ffn, m.vocab, m.dtype == RSD_F32, m.rms_eps};
+}
+
 // Lays out the workspace; with c == nullptr only the size is computed.
 size_t layout_workspace(const rsd_config& cfg, const rsd_model* const ms[3], rsd_ctx* c) {
   Layout L;
@@ -299,6 +309,14 @@ size_t layout_workspace(const rsd_config& cfg, const rsd_model* const ms[3], rsd
   unsigned long long* mega_prof[3] = {nullptr, nullptr, nullptr};
   if (cfg.debug_flags & RSD_DEBUG_MEGA_PROFILE)
     for (int w = 0; w < 3; w += 2) mega_prof[w] = TAKE(unsigned long long, 1024);
+  void* resident_block[3] = {nullptr, nullptr, nullptr};
+  uint32_t* resident_slots[3] = {nullptr, nullptr, nullptr};
+  for (int w = 0; w < 3; w += 2) {
+    const ResidentShape rs = resident_shape_of(*ms[w]);
+    if (!resident_supported(rs)) continue;
+    resident_block[w] = TAKE(char, resident_block_bytes(rs.n_layers));
+    resident_slots[w] = TAKE(uint32_t, resident_slot_bytes(rs) / 4);
+  }
   float2* rope[3];
   for (int w = 0; w < 3; ++w) rope[w] = TAKE(float2, (size_t)S * (ms[w]->head_dim / 2));
   char* w16[3] = {nullptr, nullptr, nullptr};
@@ -339,6 +357,7 @@ size_t layout_workspace(const rsd_config& cfg, const rsd_model* const ms[3], rsd
     c->norm_ssq = norm_ssq;
     for (int w = 0; w < 3; ++w) { c->mega_block[w] = mega_block[w]; c->mega_B[w] = 0; }
     c->mega_sync = mega_sync;
+    for (int w = 0; w < 3; ++w) { c->resident_block[w] = resident_block[w]; c->resident_slots[w] = resident_slots[w]; }
     for (int w = 0; w < 3; ++w) c->mega_prof[w] = mega_prof[w];
     for (int w = 0; w < 3; ++w) c->mdl[w].rope = rope[w];
     for (int w = 0; w < 3; ++w) c->mdl[w].w16 = w16[w];
@@ -943,6 +962,13 @@ int follow_phase(rsd_ctx* c, int launched, cudaStream_t s, bool* ended) {
   }
 }
 
+// Whether the phase runs in one launch (decode_resident.cu).  Single kernels are timed, logits are kept, kernel by kernel.
+bool resident_wanted(const rsd_ctx* c, int which, int n_slots) {
+  const int flags = c->cfg.debug_flags;
+  return c->resident[which] && n_slots <= 8 && c->time_stride == 0 && !(flags & RSD_DEBUG_NO_GRAPHS) && c->mega_B[which] != c->st.B &&
+         (!(flags & RSD_DEBUG_KEEP_LOGITS) || (flags & RSD_DEBUG_RESIDENT_LOGITS));
+}
+
 // One decode phase: up to C iterations, fewer when every row ends before.
 int decode_phase(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t s) {
   unsigned flags = 0;
@@ -952,6 +978,12 @@ int decode_phase(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t s) 
   *c->progress = 0;            // the stream was synchronised since the last phase: no kernel that writes the word is in flight
   CU(launch_decode_begin(c->st, which, phase, s));
   if (n_slots <= 0) return RSD_OK;
+  if (resident_wanted(c, which, n_slots)) {
+    if (c->fail_at >= 0 && c->fail_at < c->C) CU(cudaMemsetAsync((char*)c->gemm_scratch + 4096, 0xFF, sizeof(int32_t), s));   // ahead of the first
+    CU(launch_decode_resident(c->resident_plan[which], c->resident_block[which], c->resident_shape[which], c->mdl[which].kv_dtype == 3, c->st, which,
+                              phase, n_slots, c->lp, s));
+    return RSD_OK;
+  }
   const bool graphs = !(c->cfg.debug_flags & RSD_DEBUG_NO_GRAPHS);
   // The attention kernel splits every row's context over so many CTAs that the ACTIVE rows fill the machine; the
   // rows of the phase are known here, so the iteration is captured once per power-of-two bucket of that number.
@@ -1186,6 +1218,22 @@ int rsd_load_models(rsd_ctx* c, const rsd_model* draft, const rsd_model* prm, co
       for (int k = 0; k < 4; ++k)
         CU(launch_bf16_to_f16(src[k], const_cast<void*>(M.w16_of(l, k)), M.w16_elems(k), s));
     }
+  }
+  for (int w = 0; w < 3; w += 2) {
+    const ModelHost& M = c->mdl[w];
+    c->resident[w] = false;
+    if (c->resident_block[w] == nullptr) continue;
+    ResidentBuild a{};
+    a.shape = c->resident_shape[w] = resident_shape_of(M.m);
+    a.max_pages = c->max_pages; a.v_limit = c->v_limit; a.model_id = w; a.temperature = c->cfg.temperature; a.seed = c->cfg.seed;
+    a.embed = M.m.tok_embed; a.head = M.m.head; a.final_norm = M.m.final_norm;
+    a.wqkv = M.m.wqkv; a.wo = M.m.wo; a.wgu = M.m.wgu; a.wdown = M.m.wdown; a.norm1 = M.m.norm1; a.norm2 = M.m.norm2;
+    a.kv_pool = M.kv_pool; a.layer_stride = M.layer_stride; a.rope = M.rope; a.page_table = c->st.page_table[w];
+    a.slots = c->resident_slots[w]; a.err = (int*)((char*)c->gemm_scratch + 4096); a.dbg_logits = c->dbg_logits[w == RSD_DRAFT ? 0 : 1];
+    const cudaError_t e = resident_build(&c->resident_plan[w], c->resident_block[w], a, s);
+    if (e == cudaErrorNotSupported) continue;
+    CU(e);
+    c->resident[w] = true;
   }
   CU(cudaMemsetAsync(c->d_scalars, 0, 16 * sizeof(int32_t), s));
   CU(cudaMemsetAsync(c->gemm_scratch, 0, c->gemm_scratch_bytes, s));

@@ -1036,6 +1036,25 @@ bool tc_tensor_map(const void* ptr, int rows, int cols, int box_rows, CUtensorMa
   return get_map(ptr, rows, cols, box_rows, out);
 }
 
+bool tc_tensor_map_rows(const void* ptr, bool f32, int rows, int cols, CUtensorMap* out) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn || ((uintptr_t)ptr & 15) || cols % (f32 ? 4 : kTileK) != 0) return false;
+  const cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r;
+  if (f32) {
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, strides[1] = {(cuuint64_t)cols * 4};
+    const cuuint32_t box[2] = {256, 8};
+    r = fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+           CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  } else {
+    const cuuint64_t dims[3] = {kTileK, (cuuint64_t)rows, (cuuint64_t)cols / kTileK}, strides[2] = {(cuuint64_t)cols * 2, kTileK * 2};
+    const cuuint32_t box[3] = {kTileK, 8, 8};
+    r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  }
+  return r == CUDA_SUCCESS;
+}
+
 // One layer's slab of fp16 KV pages as a tensor of 4096-byte blocks (per page: the keys of every KV head
 // [16 tokens][128 dims], then the values [128 dims][16 tokens]), one box per block:
 //   keys    (64 dims, 8 tokens, 2 dim halves, 2 token groups, block)   128-byte swizzle: lands as

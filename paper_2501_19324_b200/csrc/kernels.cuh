@@ -196,6 +196,34 @@ cudaError_t mega_build(void* dev_block, const MegaBuild& a, cudaStream_t s);
 cudaError_t launch_decode_mega(const void* dev_block, int B, int kv_extended, PassView p, const void* final_gain,
                                cudaStream_t s);
 
+// ---- a whole decode phase of a small model over up to eight rows in one launch (decode_resident.cu) ----
+struct ResidentShape {
+  int n_layers, d, H, KV, hd, F, vocab;
+  bool f32;
+  float eps;
+};
+struct ResidentBuild {
+  ResidentShape shape;
+  int max_pages, v_limit, model_id;
+  float temperature;
+  uint64_t seed;
+  const void *embed, *head, *final_norm;
+  const void* const *wqkv, *const *wo, *const *wgu, *const *wdown, *const *norm1, *const *norm2;
+  char* kv_pool;
+  size_t layer_stride;
+  const float2* rope;
+  const int32_t* page_table;
+  uint32_t* slots;             // resident_slot_bytes, 256-byte aligned
+  int* err;                    // raised to -5 when a bounded wait expires
+  float* dbg_logits;           // null, or [rows][C][vocab]: receives the logits
+};
+struct ResidentPlan { alignas(128) unsigned char bytes[512]; };   // the kernel's parameters
+bool resident_supported(const ResidentShape& m);
+size_t resident_block_bytes(int n_layers);
+size_t resident_slot_bytes(const ResidentShape& m);
+// Fills the plan, and dev_block (256-byte aligned) with the layers' tensor maps and pointers; cudaErrorNotSupported: weights or pools
+// that TMA or 16-byte loads cannot take.
+cudaError_t resident_build(ResidentPlan* plan, void* dev_block, const ResidentBuild& a, cudaStream_t s);
 struct SampleArgs {
   const float* logits;         // [n_slots, V]
   int n_slots, V, v_limit;
@@ -277,6 +305,9 @@ inline __host__ __device__ bool target_pass_due(int n_waiting, int n_live, int m
   return n_waiting > 0 && n_waiting >= (want < n_live ? want : n_live);
 }
 cudaError_t launch_decode_begin(const RowState& st, int which, int phase, cudaStream_t s);
+// Runs the decode phase that launch_decode_begin has opened, n_slots <= 8, to its end.
+cudaError_t launch_decode_resident(const ResidentPlan& plan, const void* dev_block, const ResidentShape& m, bool kv_extended, const RowState& st, int which,
+                                   int phase, int n_slots, const LoopParams& lp, cudaStream_t s);
 // Merged PRM: one slot per row that took a draft step, carrying the step's last token at the draft's
 // cursor (which stays where it is); n_active = number of such rows, last_idx[b] = b for them.
 cudaError_t launch_score_prepare(const RowState& st, cudaStream_t s);

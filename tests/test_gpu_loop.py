@@ -610,6 +610,71 @@ def test_decode_attention_of_sixteen_warps(rows, H, KV, hd, lo, hi):
     eng.close()
 
 
+# One launch per decode phase: the smallest and the widest models that it takes, columns that do not fill the last stage (512 / 256) or the
+# last unit of the head, groups of one to eight heads, contexts of one page to three rounds of the warps, one to eight rows.
+RESIDENT = [
+    # shape, bf16, rows, prompt tokens, extended cache
+    (ri.ModelShape(1, 64, 1, 1, 128, 64, 515), True, 1, (3, 3), 0),
+    (ri.ModelShape(3, 192, 3, 3, 128, 320, 1000), True, 5, (1, 40), 0),
+    (ri.ModelShape(2, 512, 4, 2, 128, 1408, 4096), True, 8, (120, 300), 0),
+    (ri.ModelShape(2, 512, 4, 2, 128, 1408, 4096), True, 3, (120, 300), 1),
+    (ri.ModelShape(2, 1024, 16, 2, 128, 2048, 1030), True, 7, (10, 150), 0),
+    (ri.ModelShape(1, 2048, 8, 8, 128, 1088, 1030), True, 4, (10, 50), 1),
+    (ri.ModelShape(1, 16, 1, 1, 64, 8, 100), False, 2, (1, 5), 0),
+    (ri.ModelShape(2, 336, 5, 5, 64, 200, 333), False, 8, (3, 70), 0),
+    (ri.ModelShape(2, 256, 4, 2, 64, 688, 1024), False, 4, (100, 300), 0),
+    (ri.ModelShape(1, 2048, 32, 2, 64, 2048, 520), False, 5, (10, 40), 0),
+]
+
+
+@pytest.mark.parametrize("sh,bf16,rows,ctx,ext", RESIDENT)
+def test_decode_phase_in_one_launch(sh, bf16, rows, ctx, ext):
+    from paper_2501_19324_b200 import lib, RSD_DEBUG_KEEP_LOGITS
+    from paper_2501_19324_b200.binding import RSD_DEBUG_RESIDENT_LOGITS
+    prompts = ri.prompts(61 + rows, rows, *ctx, sh.vocab)
+    kw = dict(max_step_tokens=7, max_steps=3, max_seq_tokens=ctx[1] + 32, step_end_id=2, step_end_mod=5, temperature=0.7, seed=6)
+    launches = []
+    for flags in (RSD_DEBUG_KEEP_LOGITS | RSD_DEBUG_RESIDENT_LOGITS, RSD_DEBUG_KEEP_LOGITS):
+        eng, loop = build_pair((sh, sh, sh), bf16=bf16, prompts=prompts, loop_kwargs=kw, engine_kwargs=dict(debug_flags=flags, kv_extended=ext))
+        stats = {}
+        before = lib().rsd_debug_launch_count()
+        for _ in range(2):
+            parity_step(eng, loop, 2.0, stats=stats, **(TOL16 if bf16 else TOL32))    # every row is rejected: draft and target decode
+        launches.append(lib().rsd_debug_launch_count() - before)
+        assert stats["tokens"] > 0
+        compare_counters(eng, loop)
+        eng.close()
+    assert launches[0] < launches[1]
+
+
+def test_decode_phases_in_one_launch_on_two_streams():
+    """Two contexts, a thread and a stream each: each phase takes the whole chip, and none may wait for a part of it."""
+    import threading
+    import torch
+    prompts = ri.prompts(3, 4, 10, 40, MINI[0].vocab)
+    kw = dict(max_seq_tokens=160, max_step_tokens=24, max_steps=4, step_end_id=3, step_end_mod=9, temperature=0.7, seed=1)
+    engines = [_engine(prompts, **kw) for _ in range(3)]
+    want = [engines[0].step(2.0)["step_tokens"].tolist() for _ in range(4)]
+    got, failed = [[], []], []
+
+    def run(i):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(4):
+                    got[i].append(engines[i + 1].step(2.0)["step_tokens"].tolist())
+        except Exception as e:                           # noqa: BLE001
+            failed.append(e)
+    threads = [threading.Thread(target=run, args=(i,)) for i in range(2)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not failed, failed
+    assert got[0] == want and got[1] == want
+    for e in engines:
+        e.close()
+
+
 def _engine(prompts, **kw):
     from paper_2501_19324_b200 import Engine, Model
     heads = (ri.HEAD_LM, ri.HEAD_REWARD_SIGMOID, ri.HEAD_LM)
