@@ -409,6 +409,12 @@ int rsd_k_gemm_rows_qkv(const void* W, const void* x, const void* x_lo, const fl
 int rsd_k_sample(const float* logits, int32_t B, int32_t V, int32_t v_limit, float temperature,
                  uint64_t seed, int32_t model_id, const int32_t* row, const int32_t* pos, int32_t* token,
                  void* scratch, size_t scratch_bytes, void* cuda_stream);
+/* rsd_k_sample of the logits (x + x_lo)[M, K] * W[N, K]^T / sqrt(sum_c ssq[m, c] / K + eps), c < n_chunks (ssq null: no denominator), which are
+ * not kept: the lm head of a decode pass samples in its epilogue.  bf16, 1 <= M <= 128, K % 8 == 0, W, x and x_lo 16-byte aligned (else
+ * RSD_ERR_ARG).  scratch: 8 * M + 256 bytes, 8-byte aligned.                                       */
+int rsd_k_head_sample(const void* W, const void* x, const void* x_lo, int32_t M, int32_t N, int32_t K, const float* ssq, int32_t n_chunks,
+                      float eps, int32_t v_limit, float temperature, uint64_t seed, int32_t model_id, const int32_t* row, const int32_t* pos,
+                      int32_t* token, void* scratch, size_t scratch_bytes, void* cuda_stream);
 /* Philox4x32-10 blocks: out[i] = philox(ctr[i], key), ctr [n, 4], key [2], out [n, 4] (uint32). */
 int rsd_k_philox(const uint32_t* ctr, const uint32_t* key, uint32_t* out, int32_t n, void* cuda_stream);
 

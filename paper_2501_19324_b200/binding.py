@@ -59,7 +59,7 @@ EXPORTS = ["rsd_query_sizes", "rsd_create", "rsd_load_models", "rsd_prefill", "r
            "rsd_reset", "rsd_destroy", "rsd_last_error", "rsd_debug_force", "rsd_debug_force_sd", "rsd_debug_get_logits",
            "rsd_debug_get_sampled", "rsd_debug_get_state", "rsd_debug_gemm_timing", "rsd_debug_gemm_timing_dense", "rsd_debug_launch_count", "rsd_debug_fail_iteration", "rsd_debug_mega_profile", "rsd_debug_phase_ms", "rsd_k_gemm", "rsd_k_gemm_scratch_bytes", "rsd_debug_gemm_wait_probe", "rsd_debug_attn_wait_probe",
            "rsd_k_attn_decode", "rsd_k_attn_decode_scratch_bytes", "rsd_k_attn_chunk", "rsd_k_gate_compact", "rsd_k_gate_compact_static", "rsd_k_gate_compact_static_error", "rsd_k_rmsnorm",
-           "rsd_k_rope", "rsd_k_swiglu", "rsd_k_gemm_gu", "rsd_k_gemm_rows", "rsd_k_gemm_rows_qkv", "rsd_k_sample", "rsd_k_philox"]
+           "rsd_k_rope", "rsd_k_swiglu", "rsd_k_gemm_gu", "rsd_k_gemm_rows", "rsd_k_gemm_rows_qkv", "rsd_k_sample", "rsd_k_head_sample", "rsd_k_philox"]
 
 _lib = None
 
@@ -117,6 +117,7 @@ def lib():
         L.rsd_k_gemm_gu.argtypes = [vp, vp, vp, vp, vp, c_int32, c_int32, c_int32, vp, c_size_t, vp]
         L.rsd_k_gemm_rows.argtypes = [vp] * 8 + [c_int32] * 3 + [vp]
         L.rsd_k_gemm_rows_qkv.argtypes = [vp] * 4 + [c_int32, c_float] + [vp] * 6 + [c_int32] * 7 + [vp]
+        L.rsd_k_head_sample.argtypes = [vp] * 3 + [c_int32] * 3 + [vp, c_int32, c_float, c_int32, c_float, c_uint64, c_int32, vp, vp, vp, vp, c_size_t, vp]
         L.rsd_k_sample.argtypes = [vp, c_int32, c_int32, c_int32, c_float, c_uint64, c_int32, vp, vp, vp, vp, c_size_t, vp]
         L.rsd_k_philox.argtypes = [vp, vp, vp, c_int32, vp]
         _lib = L
@@ -475,6 +476,20 @@ def k_sample(logits, v_limit, temperature, seed, model_id, row, pos):
     scratch = torch.zeros(B, dtype=torch.int64, device=logits.device)
     _check(lib().rsd_k_sample(_ptr(logits), B, V, v_limit, temperature, seed, model_id, _ptr(row), _ptr(pos), _ptr(tok),
                               _ptr(scratch), 8 * B, _stream()))
+    return tok
+
+
+def k_head_sample(W, x_hi, x_lo, v_limit, temperature, seed, model_id, row, pos, ssq=None, eps=0.0):
+    """k_sample of the logits (x_hi + x_lo) W^T / sqrt(mean square + eps), which the head's epilogue keeps to itself; up to 128 rows."""
+    import torch
+    M, K = x_hi.shape
+    tok = torch.zeros(M, dtype=torch.int32, device=W.device)
+    scratch = torch.zeros(M + 32, dtype=torch.int64, device=W.device)
+    _check(lib().rsd_k_head_sample(_ptr(W), _ptr(x_hi), _ptr(x_lo), M, W.shape[0], K, _ptr(ssq) if ssq is not None else None,
+                                   ssq.shape[1] if ssq is not None else 0, eps, v_limit, temperature, seed, model_id, _ptr(row), _ptr(pos), _ptr(tok),
+                                   _ptr(scratch), 8 * M + 256, _stream()))
+    if int(scratch[M].item()) & 0xFFFFFFFF:
+        raise RsdError(-5, "a bounded wait inside the head expired")
     return tok
 
 

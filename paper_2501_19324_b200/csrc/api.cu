@@ -830,9 +830,34 @@ int model_logits(rsd_ctx* c, int which, PassView p, bool allow_mega, cudaStream_
 }
 
 // Enqueues one decode iteration: model pass, final norm, lm_head, sample, append (and lay out the next one).
+// Decode passes of the fused bf16 path whose logits nobody keeps sample in the head's epilogue (head_sample.cu).
+bool head_samples(const rsd_ctx* c, int which, PassView p, bool keep_logits) {
+  const rsd_model& m = c->mdl[which].m;
+  return !keep_logits && fused_decode_ok(c->mdl[which]) && head_sample_pays(p.T, m.vocab, m.d_model);
+}
+
+int decode_and_sample(rsd_ctx* c, int which, PassView p, const SampleArgs& a, cudaStream_t s) {
+  const rsd_model& m = c->mdl[which].m;
+  RowScale rs;
+  const int rc = forward_decode_fused(c, which, p, m.final_norm, s, &rs);
+  if (rc) return rc;
+  return timed_product(c, ProductBytes{(double)p.T, 2.0}(m.vocab, m.d_model, 0, false), s, [&] {
+    return launch_head_sample(m.head, c->h, c->h_lo, m.vocab, m.d_model, (int*)((char*)c->gemm_scratch + 4096), rs, a, s);
+  });
+}
+
 int decode_iteration(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t s) {
   const rsd_model& m = c->mdl[which].m;
   PassView p{c->st.pass_tok_id, c->st.pass_tok_row, c->st.pass_tok_pos, n_slots, c->st.n_active};
+  SampleArgs a{c->logits, n_slots, m.vocab, c->v_limit, c->cfg.temperature, c->cfg.seed, which,
+               c->st.pass_tok_row, c->st.pass_tok_pos, nullptr, c->st.n_active, c->sample_best};
+  const bool mega = c->mega_B[which] > 0 && c->mega_B[which] == c->st.B && n_slots == c->st.B;
+  if (!mega && head_samples(c, which, p, c->dbg_logits[phase] != nullptr)) {
+    const int rc = decode_and_sample(c, which, p, a, s);
+    if (rc) return rc;
+    CU(launch_decode_update(c->st, which, phase, c->sample_best, n_slots, c->lp, s));
+    return RSD_OK;
+  }
   int rc = model_logits(c, which, p, true, s);
   if (rc) return rc;
   if (c->dbg_logits[phase]) {
@@ -840,8 +865,6 @@ int decode_iteration(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t
                                                   c->st.iter, c->st.n_active);
     CU(launched(1));
   }
-  SampleArgs a{c->logits, n_slots, m.vocab, c->v_limit, c->cfg.temperature, c->cfg.seed, which,
-               c->st.pass_tok_row, c->st.pass_tok_pos, nullptr, c->st.n_active, c->sample_best};
   CU(launch_sample(a, s));
   CU(launch_decode_update(c->st, which, phase, c->sample_best, n_slots, c->lp, s));
   return RSD_OK;
@@ -853,11 +876,16 @@ int sd_propose_iteration(rsd_ctx* c, int n_slots, cudaStream_t s) {
   const rsd_model& m = c->mdl[RSD_DRAFT].m;
   CU(launch_sd_propose_prepare(c->st, n_slots, s));
   PassView p{c->st.pass_tok_id, c->st.pass_tok_row, c->st.pass_tok_pos, n_slots, c->st.n_active};
-  int rc = model_logits(c, RSD_DRAFT, p, false, s);
-  if (rc) return rc;
   SampleArgs a{c->logits, n_slots, m.vocab, c->v_limit, c->cfg.temperature, c->cfg.seed, RSD_DRAFT,
                c->st.pass_tok_row, c->st.pass_tok_pos, nullptr, c->st.n_active, c->sample_best};
-  CU(launch_sample(a, s));
+  if (head_samples(c, RSD_DRAFT, p, false)) {
+    const int rc = decode_and_sample(c, RSD_DRAFT, p, a, s);
+    if (rc) return rc;
+  } else {
+    const int rc = model_logits(c, RSD_DRAFT, p, false, s);
+    if (rc) return rc;
+    CU(launch_sample(a, s));
+  }
   CU(launch_sd_propose_update(c->st, c->sample_best, n_slots, s));
   return RSD_OK;
 }
@@ -869,8 +897,11 @@ int sd_verify_pass(rsd_ctx* c, int n_slots, cudaStream_t s) {
   CU(launch_sd_verify_prepare(c->st, n_slots, s));
   const int T = n_slots * c->sd_k;
   PassView p{c->st.pass_tok_id, c->st.pass_tok_row, c->st.pass_tok_pos, T, c->st.n_active};
+  SampleArgs a{c->logits, T, m.vocab, c->v_limit, c->cfg.temperature, c->cfg.seed, RSD_TARGET,
+               c->st.pass_tok_row, c->st.pass_tok_pos, nullptr, c->st.n_active, c->sample_best};
+  const bool in_head = head_samples(c, RSD_TARGET, p, c->dbg_logits[1] != nullptr);
   c->pass_width = c->sd_k;
-  int rc = model_logits(c, RSD_TARGET, p, false, s);
+  int rc = in_head ? decode_and_sample(c, RSD_TARGET, p, a, s) : model_logits(c, RSD_TARGET, p, false, s);
   c->pass_width = 1;
   if (rc) return rc;
   if (c->dbg_logits[1]) {
@@ -878,9 +909,7 @@ int sd_verify_pass(rsd_ctx* c, int n_slots, cudaStream_t s) {
                m.vocab, c->C, c->st.n_active);
     CU(launched(1));
   }
-  SampleArgs a{c->logits, T, m.vocab, c->v_limit, c->cfg.temperature, c->cfg.seed, RSD_TARGET,
-               c->st.pass_tok_row, c->st.pass_tok_pos, nullptr, c->st.n_active, c->sample_best};
-  CU(launch_sample(a, s));
+  if (!in_head) CU(launch_sample(a, s));
   CU(launch_sd_accept(c->st, c->sample_best, n_slots, c->lp, s));
   return RSD_OK;
 }
@@ -1794,6 +1823,21 @@ int rsd_k_sample(const float* logits, int32_t B, int32_t V, int32_t v_limit, flo
   KCU(cudaMemsetAsync(scratch, 0, sizeof(unsigned long long) * (size_t)B, (cudaStream_t)cuda_stream));
   SampleArgs a{logits, B, V, v_limit, temperature, seed, model_id, row, pos, token, nullptr, (unsigned long long*)scratch};
   KCU(launch_sample(a, (cudaStream_t)cuda_stream));
+  return RSD_OK;
+}
+
+int rsd_k_head_sample(const void* W, const void* x, const void* x_lo, int32_t M, int32_t N, int32_t K, const float* ssq, int32_t n_chunks,
+                      float eps, int32_t v_limit, float temperature, uint64_t seed, int32_t model_id, const int32_t* row, const int32_t* pos,
+                      int32_t* token, void* scratch, size_t scratch_bytes, void* cuda_stream) {
+  if (!W || !x || !x_lo || !row || !pos || !token || v_limit < 1 || v_limit > N || temperature < 0.f || (ssq && n_chunks < 1)) return RSD_ERR_ARG;
+  if (!head_sample_supported(M, N, K) || ((uintptr_t)W | (uintptr_t)x | (uintptr_t)x_lo) & 15) return RSD_ERR_ARG;
+  const size_t best_bytes = sizeof(unsigned long long) * (size_t)M;
+  if (!scratch || scratch_bytes < best_bytes + 256 || ((uintptr_t)scratch & 7)) return RSD_ERR_ARG;
+  cudaStream_t s = (cudaStream_t)cuda_stream;
+  KCU(cudaMemsetAsync(scratch, 0, best_bytes + sizeof(int), s));
+  SampleArgs a{nullptr, M, N, v_limit, temperature, seed, model_id, row, pos, nullptr, nullptr, (unsigned long long*)scratch};
+  KCU(launch_head_sample(W, x, x_lo, N, K, (int*)((char*)scratch + best_bytes), RowScale{ssq, n_chunks, 1.f / (float)K, eps}, a, s));
+  KCU(launch_sample_finalize(a.best, row, token, M, s));
   return RSD_OK;
 }
 

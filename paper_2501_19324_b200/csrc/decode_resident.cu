@@ -35,6 +35,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "sampling.cuh"
 #include "tc_ptx.cuh"
 
 namespace rsd {
@@ -225,12 +226,6 @@ __device__ __forceinline__ bool step_ends(int t, const LoopParams& lp) {
   if (lp.eos_id >= 0 && t == lp.eos_id) return true;
   if (lp.step_end_mod > 0) return (t % lp.step_end_mod) == (lp.step_end_id % lp.step_end_mod);
   return t == lp.step_end_id;
-}
-
-// Order-preserving image of a score; no candidate: 0.
-__device__ __forceinline__ uint32_t score_key(float s) {
-  const uint32_t b = __float_as_uint(s);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
 // Shared memory behind the ring.

@@ -237,6 +237,13 @@ struct SampleArgs {
   unsigned long long* best;    // [n_slots] scratch, zero on entry: packed (score, id) maxima
 };
 cudaError_t launch_sample(const SampleArgs& a, cudaStream_t s);
+// token[i] = id packed in best[i] for slots with a row; best is cleared.
+cudaError_t launch_sample_finalize(unsigned long long* best, const int32_t* slot_row, int32_t* token, int n, cudaStream_t s);
+// The lm head of up to 128 slots with the sampling in its epilogue: winners packed in a.best as by launch_sample, from the logits rowscale * (x + x_lo) W^T
+// [a.n_slots, N] that nobody keeps (a.logits and a.V are not looked at, a.token is null).  err: raised to -5 when a bounded wait expires.
+bool head_sample_supported(int M, int N, int K);
+bool head_sample_pays(int M, int N, int K);      // faster than the head and the sampling by themselves
+cudaError_t launch_head_sample(const void* W, const void* x, const void* x_lo, int N, int K, int* err, RowScale rs, const SampleArgs& a, cudaStream_t s);
 cudaError_t launch_philox(const uint32_t* ctr, const uint32_t* key, uint32_t* out, int n, cudaStream_t s);
 
 // reward[row] = head(rmsnorm(x[last_idx[row] - t0])) for rows whose last token lies in [t0, t0+T).

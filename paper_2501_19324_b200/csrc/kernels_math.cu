@@ -3,6 +3,7 @@
 // the KV cache are stored in the model's element type (fp32 or bfloat16).
 #include "common.cuh"
 #include "kernels.cuh"
+#include "sampling.cuh"
 
 namespace rsd {
 
@@ -1101,23 +1102,6 @@ cudaError_t launch_swiglu(int dtype, const float* gu, SplitSum pending, void* ou
 // Sampling: greedy argmax, or Gumbel-max with Philox noise keyed by (seed; vocab id / 4, position
 // of the generated token, row, model id).  One block per slot; ties go to the lowest id.
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ void better(float& bs, int& bi, float s, int i) {
-  if (s > bs || (s == bs && i < bi)) { bs = s; bi = i; }
-}
-
-// (score, id) packed so that an unsigned 64-bit maximum picks the highest score and, among equal
-// scores, the lowest id: high word = order-preserving image of the float, low word = ~id.
-__device__ __forceinline__ unsigned long long pack_best(float sc, int id) {
-  const uint32_t b = __float_as_uint(sc);
-  const uint32_t key = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-  return ((unsigned long long)key << 32) | (uint32_t)(0xFFFFFFFFu - (uint32_t)id);
-}
-
-__device__ __forceinline__ float unpack_score(unsigned long long packed) {
-  const uint32_t key = (uint32_t)(packed >> 32);
-  return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key);
-}
-
 // Grid (slots, chunks): every warp takes `steps` runs of 128 ids of a slot and folds its best candidate into best[slot] with
 // an atomic maximum (order-independent, hence deterministic).
 // Exact noise for every id -- ten Philox rounds per four ids and two logarithms per id -- kept the ALUs busy for 66 us at
@@ -1128,23 +1112,6 @@ __device__ __forceinline__ float unpack_score(unsigned long long packed) {
 // DIRECT: few ids in all, exact noise for each of them.
 constexpr int kSampleThreads = 256, kSampleBlocks = 4;   // ... and blocks per SM
 constexpr int kSampleSteps = 8;             // runs of 128 ids that a warp holds in registers at most
-constexpr float kScoreMargin = 1e-3f;       // the fast score errs by less than 1e-4 (see fast_gumbel)
-constexpr float kNoiseMax = 17.f;
-
-// -log(-log u) for u = (2k + 1) / 2^24.  Near 1, where the large values come from, -log u is its series in 1 - u (exact
-// in fp32; 1 - u < 2^-6: three terms err by 1e-6 relative); elsewhere __logf errs by 2^-21.4 on -log u > 2^-6, that is
-// 2.3e-5 relative, and so much in the outer logarithm, whose own error is 3 ulp of at most 17.
-__device__ __forceinline__ float fast_gumbel(float u) {
-  const float d = 1.f - u;
-  const float y = d < 0.015625f ? d * (1.f + d * (0.5f + d * 0.33333333f)) : -__logf(u);
-  return -__logf(y);
-}
-
-// What still can win against a best score of `run`.
-__device__ __forceinline__ float score_needed(float run) {
-  return run == INFINITY ? run : run - (kScoreMargin + fabsf(run) * 1e-6f);
-}
-
 template <bool DIRECT>
 __global__ void __launch_bounds__(kSampleThreads, kSampleBlocks) sample_kernel(SampleArgs a, int steps) {
   RSD_PDL_TRIGGER();
@@ -1275,6 +1242,11 @@ __global__ void sample_finalize_kernel(unsigned long long* best, const int32_t* 
   best[i] = 0ull;
 }
 
+cudaError_t launch_sample_finalize(unsigned long long* best, const int32_t* slot_row, int32_t* token, int n, cudaStream_t s) {
+  RSD_LAUNCH((sample_finalize_kernel), (n + 255) / 256, 256, 0, s, best, slot_row, token, n);
+  return launched(1);
+}
+
 // Leaves the winners packed in a.best (which must be zero on entry); when a.token is given a second
 // kernel unpacks them into a.token and clears a.best.
 cudaError_t launch_sample(const SampleArgs& a, cudaStream_t s) {
@@ -1290,8 +1262,8 @@ cudaError_t launch_sample(const SampleArgs& a, cudaStream_t s) {
   if ((long)a.n_slots * a.v_limit <= 1500000) RSD_LAUNCH((sample_kernel<true>), grid, kSampleThreads, 0, s, a, steps);
   else RSD_LAUNCH((sample_kernel<false>), grid, kSampleThreads, 0, s, a, steps);
   if (a.token == nullptr) return launched(1);
-  RSD_LAUNCH((sample_finalize_kernel), (a.n_slots + 255) / 256, 256, 0, s, a.best, a.slot_row, a.token, a.n_slots);
-  return launched(2);
+  const cudaError_t e = launched(1);
+  return e != cudaSuccess ? e : launch_sample_finalize(a.best, a.slot_row, a.token, a.n_slots, s);
 }
 
 __global__ void philox_kernel(const uint32_t* ctr, const uint32_t* key, uint32_t* out, int n) {

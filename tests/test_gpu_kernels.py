@@ -939,6 +939,60 @@ def test_chunk_attention_wait_runs_out_cleanly(one_pass):
         np.testing.assert_allclose(got[t, 0], w @ Vs[b][:p + 1, 0].astype(np.float64), rtol=0, atol=2e-3)
 
 
+# Rows of every instruction width and their edges; ids that leave no whole tile, one and some, a remainder of less than a piece, no multiple of
+# four in the race; columns that do not fill a K step.
+HEAD_SAMPLE = [(1, 515, 64, 515), (8, 4096, 72, 4001), (9, 1030, 768, 1030), (16, 38000, 520, 37999), (17, 75777, 64, 75777), (33, 40000, 1536, 39998),
+               (64, 151936, 512, 151665), (65, 20000, 1536, 19999), (128, 38001, 264, 38001)]
+
+
+@pytest.mark.parametrize("temperature", [0.0, 0.7])
+@pytest.mark.parametrize("M,N,K,v_limit", HEAD_SAMPLE)
+def test_head_that_samples(M, N, K, v_limit, temperature):
+    """Against the head and the sampling one after the other: the sums are the same bits, so are the tokens.  Flat logits, logits with a peak, and two
+    ids whose logits overflow (the lower one wins)."""
+    gen = torch.Generator(device="cuda").manual_seed(M * N)
+    W = torch.randn(N, K, generator=gen, device="cuda").mul_(0.05).to(torch.bfloat16)
+    row = torch.randperm(M, generator=gen, device="cuda").to(torch.int32)
+    if M > 1:
+        row[M // 2] = -1
+    pos = torch.randint(0, 500, (M,), generator=gen, device="cuda").to(torch.int32)
+    ids = torch.randint(0, v_limit, (M,), generator=gen, device="cuda")
+    flat = torch.randn(M, K, generator=gen, device="cuda")
+    inputs = [(W, flat), (W, W[ids].float() * (20.0 / (0.0025 * K)))]
+    huge = W.clone()
+    huge[v_limit - 1] = 3e38
+    huge[v_limit // 2] = 3e38
+    inputs.append((huge, torch.full((M, K), 4.0, device="cuda")))
+    for w, x in inputs:
+        hi = x.to(torch.bfloat16)
+        lo = (x - hi.float()).to(torch.bfloat16)
+        got = rb.k_head_sample(w, hi, lo, v_limit, temperature, 77, 1, row, pos)
+        logits = rb.k_gemm(w, hi, x_lo=lo, impl=3)
+        want = rb.k_sample(logits, v_limit, temperature, 77, 1, row, pos)
+        assert torch.equal(got, want), (got, want)
+        if w is huge:
+            assert (got[row >= 0] == v_limit // 2).all()
+
+
+def test_head_that_samples_scales_its_rows():
+    """The denominators of a norm ahead of the head, from sums of squares in one chunk and in many."""
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    M, N, K = 24, 5000, 512
+    W = torch.randn(N, K, generator=gen, device="cuda").mul_(0.05).to(torch.bfloat16)
+    x = torch.randn(M, K, generator=gen, device="cuda") * torch.logspace(-1, 1, M, device="cuda")[:, None]
+    hi = x.to(torch.bfloat16)
+    lo = (x - hi.float()).to(torch.bfloat16)
+    idx = torch.arange(M, device="cuda", dtype=torch.int32)
+    logits = rb.k_gemm(W, hi, x_lo=lo, impl=3)
+    for chunks in (2, 64):
+        ssq = x.pow(2).view(M, chunks, -1).sum(-1)
+        scaled = logits * torch.rsqrt(ssq.sum(-1, keepdim=True) / K + 1e-6)
+        want = rb.k_sample(scaled, N, 0.7, 5, 0, idx, idx)
+        got = rb.k_head_sample(W, hi, lo, N, 0.7, 5, 0, idx, idx, ssq=ssq.contiguous(), eps=1e-6)
+        # the denominators' sums may differ in their last bits: a token may only where two scores are that close
+        assert (got == want).float().mean() > 0.9
+
+
 def test_bounded_wait_runs_out_and_the_kernel_leaves_cleanly():
     """RSD_ERR_TIMEOUT without a fault: one CTA of the tensor-core GEMM whose copies are never issued.  Its wait
     (a few thousand polls in this mode) expires, the error flag is raised and reported, tensor memory is freed: the
