@@ -240,7 +240,9 @@ int rsd_debug_force(rsd_ctx*, int which, const int32_t* tokens, const int32_t* l
 int rsd_debug_force_sd(rsd_ctx*, const int32_t* props, const uint8_t* on);
 
 /* Logits of the last rsd_step's decode iterations of model `which`, when RSD_DEBUG_KEEP_LOGITS
- * is set: out is a HOST array [B, max_step_tokens, vocab(which)] (row b, iteration j).        */
+ * is set: out is a HOST array [B, max_step_tokens, vocab(which)] (row b, iteration j).  Contexts with
+ * that flag hold 8 MB of page-locked memory, through which several host threads that end with the call
+ * fill an array of 2 MB or more.                                                             */
 int rsd_debug_get_logits(rsd_ctx*, int which, float* out);
 /* Ids sampled (before forcing) in the last rsd_step: HOST out [B, max_step_tokens].           */
 int rsd_debug_get_sampled(rsd_ctx*, int which, int32_t* out);

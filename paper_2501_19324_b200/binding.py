@@ -325,7 +325,7 @@ class Engine:
 
     def logits(self, which: int) -> np.ndarray:
         V = self.models[which].shape.vocab
-        out = np.zeros((self.B, self.C, V), np.float32)
+        out = np.empty((self.B, self.C, V), np.float32)
         _check(lib().rsd_debug_get_logits(self.ctx, which, out.ctypes.data), self.ctx)
         return out
 

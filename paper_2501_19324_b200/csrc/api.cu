@@ -100,6 +100,7 @@ struct rsd_ctx {
   unsigned long long* mega_prof[3] = {nullptr, nullptr, nullptr};   // RSD_DEBUG_MEGA_PROFILE
   char* pinned = nullptr;
   size_t pinned_bytes = 0;
+  char* copy_staging = nullptr;   // page-locked, for logits on their way to the caller (host_copy.cu)
   void* gemm_scratch = nullptr;
   size_t gemm_scratch_bytes = 0;
   void* attn_scratch = nullptr;
@@ -1163,6 +1164,10 @@ int rsd_create(const rsd_config* cfg, rsd_ctx** out) {
     delete c;
     return fail(nullptr, RSD_ERR_CUDA, "pinned host allocation failed%s");
   }
+  if ((cfg->debug_flags & RSD_DEBUG_KEEP_LOGITS) && cudaHostAlloc((void**)&c->copy_staging, host_copy_staging_bytes(), cudaHostAllocDefault) != cudaSuccess) {
+    (void)cudaGetLastError();                  // the copies go without
+    c->copy_staging = nullptr;
+  }
   c->progress = (unsigned long long*)(c->pinned + 192);
   c->lp.step_end_id = cfg->step_end_id; c->lp.eos_id = cfg->eos_id; c->lp.step_end_mod = cfg->step_end_mod;
   c->lp.max_steps = cfg->max_steps; c->lp.omega_kind = cfg->omega_kind; c->lp.omega_alpha = cfg->omega_alpha;
@@ -1514,6 +1519,7 @@ int rsd_destroy(rsd_ctx* c) {
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
 
   if (c->pinned) cudaFreeHost(c->pinned);
+  if (c->copy_staging) cudaFreeHost(c->copy_staging);
   delete c;
   return RSD_OK;
 }
@@ -1554,7 +1560,7 @@ int rsd_debug_get_logits(rsd_ctx* c, int which, float* out) {
   if (!c || !out) return RSD_ERR_ARG;
   const int p = which == RSD_DRAFT ? 0 : (which == RSD_TARGET ? 1 : -1);
   if (p < 0 || !c->dbg_logits[p]) return fail(c, RSD_ERR_STATE, "logits were not kept%s");
-  CU(cudaMemcpy(out, c->dbg_logits[p], sizeof(float) * (size_t)c->st.B * c->C * c->mdl[which].m.vocab, cudaMemcpyDeviceToHost));
+  CU(copy_to_host(out, c->dbg_logits[p], sizeof(float) * (size_t)c->st.B * c->C * c->mdl[which].m.vocab, c->copy_staging));
   return RSD_OK;
 }
 

@@ -196,6 +196,10 @@ cudaError_t mega_build(void* dev_block, const MegaBuild& a, cudaStream_t s);
 cudaError_t launch_decode_mega(const void* dev_block, int B, int kv_extended, PassView p, const void* final_gain,
                                cudaStream_t s);
 
+// ---- copies to the caller's pageable memory (host_copy.cu) ----
+size_t host_copy_staging_bytes();              // of page-locked memory; without any the driver copies
+cudaError_t copy_to_host(void* out, const void* src, size_t bytes, void* staging);
+
 // ---- a whole decode phase of a small model over up to eight rows in one launch (decode_resident.cu) ----
 struct ResidentShape {
   int n_layers, d, H, KV, hd, F, vocab;

@@ -771,3 +771,24 @@ def test_a_blocking_process_sleeps_through_a_decode_phase():
         assert r.returncode == 0, r.stderr[-2000:]
         share[blocking] = float(r.stdout.split("SHARE")[1])
     assert share[True] < 0.7 and share[True] < share[False], share
+
+
+@pytest.mark.parametrize("C", [160, 170, 171, 690, 1500])        # 12 300 bytes each: below and above the line, less and more than the staging
+def test_kept_logits_into_pageable_and_page_locked_memory(C):
+    """The same bytes whichever way they come."""
+    import torch
+    from dataclasses import replace
+    from paper_2501_19324_b200 import Engine, Model, lib, RSD_DEBUG_KEEP_LOGITS
+    sh = [replace(s, vocab=1025) for s in TINY]
+    models = [Model(s, ri.gpu_model_tensors(s, slot, 0, False, kind), kind) for slot, (s, kind) in enumerate(zip(sh, (ri.HEAD_LM, ri.HEAD_REWARD_SIGMOID, ri.HEAD_LM)))]
+    eng = Engine(*models, max_batch=3, max_seq_tokens=C + 16, max_step_tokens=C, max_steps=1, step_end_id=3, debug_flags=RSD_DEBUG_KEEP_LOGITS)
+    eng.prefill(*ri.prompts(1, 3, 5, 9, 1025))
+    torch.manual_seed(C)
+    eng._ws.random_(0, 256)                                            # the logits among them; nothing runs on it any more
+    torch.cuda.synchronize()
+    for which in (0, 2):
+        locked = torch.empty(3, C, 1025, pin_memory=True)
+        assert lib().rsd_debug_get_logits(eng.ctx, which, locked.data_ptr()) == 0
+        got = eng.logits(which)
+        assert got.shape == (3, C, 1025) and got.tobytes() == locked.numpy().tobytes()
+    eng.close()
