@@ -504,13 +504,26 @@ int pick_splits(int B, int KV, int max_ctx) {
   const int ctas = B * KV, max_pages = max_ctx / kPageTokens;
   int splits = (3 * 148) / ctas;
   while (splits < kClusterSplits && max_pages / std::max(1, splits) >= 64) ++splits;
-  // at least 8 pages per split: two per warp, both on their way before the wait (4 and 8 pages: 714 and 706 ms for two
-  // steps of 32 rows with contexts of a few hundred tokens)
-  splits = std::max(1, std::min(splits, std::max(1, max_pages / 8)));
+  // At least 8 pages per split: two per warp, both on their way before the wait (4 and 8 pages: 714 and 706 ms for two
+  // steps of 32 rows with contexts of a few hundred tokens).  Few CTAs leave the chip idle, and a warp that walks one page, or none, is done sooner:
+  // a page a split for up to eight (slot, KV head) pairs, three for up to 32.  14-layer iterations, 8 pages a split / so, us: 1.5B shape, two pairs,
+  // 80 / 140 / 250 / 700 tokens 470 / 475 / 483 / 486 -> 466 / 466 / 465 / 471, four, 250 490 / 469, eight, 250 490 / 476, 16, 170 / 250 / 500 517 / 526 / 544 ->
+  // 513 / 513 / 528; 7B shape, four pairs, 100 / 250 / 500 1271 / 1272 / 1265 -> 1257 / 1254 / 1256, eight, 250 1307 / 1284, 16, 170 / 250 1324 / 1315 ->
+  // 1301 / 1308, 32, 170 / 250 / 500 1328 / 1356 / 1362 -> 1326 / 1329 / 1365; 64 pairs no difference.  Below six pages, or 13, one split that takes the qkv product
+  // itself is the better: two pairs, five pages 468 / 473, 16 and 32 pairs, nine pages 513 / 518 and 1336 / 1347.
+  int in_cluster = max_pages / 8;
+  if (ctas <= 8 && max_pages >= 6) in_cluster = max_pages;
+  else if (ctas <= 32 && max_pages >= 13) in_cluster = max_pages / 3;
+  splits = std::max(1, std::min(splits, std::max(std::min(in_cluster, kClusterSplits), max_pages / 8)));
   splits = std::min(splits, kMaxSplits);
   // more splits than a cluster holds cost a second launch: not worth it when 8 splits of 16 or more (slot, KV head)
-  // pairs already put a CTA on most SMs, nor when 8 splits leave a warp at most six pages
+  // pairs already put a CTA on most SMs, nor when 8 splits leave a warp at most six pages (full at 3000 tokens 8 splits / more 528 / 517 us, but these are the most tokens that a
+  // row may come to: with 200 in that room 464 / 475)
   if (splits > kClusterSplits && (ctas * kClusterSplits >= 128 || max_pages <= kClusterSplits * 24)) splits = kClusterSplits;
+  if (splits <= kClusterSplits) {              // none without pages
+    const int pages = (max_pages + splits - 1) / splits;
+    splits = std::max(1, (max_pages + pages - 1) / std::max(1, pages));
+  }
   return splits;
 }
 

@@ -470,6 +470,13 @@ def test_decode_attention_at_the_edges_of_the_split_rule(hd, H, KV, B, max_pages
             np.testing.assert_allclose(got[b, h], p @ Vs[b][:, g].astype(np.float64), rtol=0, atol=2e-3)
 
 
+@pytest.mark.parametrize("hd,H,KV,B,max_pages", [(128, 28, 4, 1, 5), (128, 28, 4, 1, 6), (128, 28, 4, 2, 9), (64, 4, 2, 4, 31), (128, 12, 2, 5, 12), (128, 12, 2, 5, 13),
+                                                 (128, 28, 4, 8, 14), (128, 28, 4, 9, 15), (128, 12, 2, 1, 192), (128, 12, 2, 1, 193)])
+def test_decode_attention_of_few_rows_in_short_splits(hd, H, KV, B, max_pages):
+    """Either side of the lines between one split, a page a split, three pages a split and more splits than a cluster holds."""
+    test_decode_attention_at_the_edges_of_the_split_rule(hd, H, KV, B, max_pages)
+
+
 @pytest.mark.parametrize("dtype,hd,H,KV", [(torch.float32, 64, 4, 2), (torch.float32, 128, 3, 3), (torch.float16, 128, 18, 2),
                                           (torch.bfloat16, 64, 9, 1)])
 def test_generic_attention_at_the_edges_of_a_round_of_warps(dtype, hd, H, KV):
