@@ -546,7 +546,8 @@ decode_resident_kernel(const __grid_constant__ ResidentParams P, const ResidentL
         return true;
       };
       bool ok;
-      const int nv = (n_vec + 32 * PER - 1) / (32 * PER);
+      // (of Kp columns, not of K: the products take whole stages, and what lies beyond K must be zeros like the weights there)
+      const int nv = (Kp / 4 + 32 * PER - 1) / (32 * PER);
       if (nv <= 1) ok = gather(std::integral_constant<int, 1>());
       else if (nv <= 2) ok = gather(std::integral_constant<int, 2>());
       else if (nv <= 4) ok = gather(std::integral_constant<int, 4>());

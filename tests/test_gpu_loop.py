@@ -646,6 +646,36 @@ def test_decode_phase_in_one_launch(sh, bf16, rows, ctx, ext):
         eng.close()
     assert launches[0] < launches[1]
 
+def _shared_memory_full_of_nan():
+    """Every SM's shared memory, as far as the rings of the products reach, is left with NaN."""
+    import torch
+    from paper_2501_19324_b200.binding import k_gemm
+    W = torch.full((4 * 148 * 128, 2048), float("nan"), dtype=torch.bfloat16, device="cuda")
+    for rows in (32, 64, 128, 512):
+        k_gemm(W, W[:rows].clone(), x_lo=W[:rows].clone())
+    torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("rows", [4, 5, 8])
+@pytest.mark.parametrize("sh", [ri.ModelShape(2, 64, 1, 1, 64, 96, 300), ri.ModelShape(1, 128, 2, 2, 64, 128, 333), ri.ModelShape(2, 640, 2, 2, 64, 328, 300)],
+                         ids=["64", "128", "640"])
+def test_fp32_decode_phase_in_one_launch_reads_what_it_wrote(sh, rows):
+    """Products whose columns do not fill the last stage, after a kernel that left NaN in shared memory: the columns beyond the last meet weights of
+    zero, and zero times what lies there must be zero."""
+    from paper_2501_19324_b200 import RSD_DEBUG_KEEP_LOGITS
+    from paper_2501_19324_b200.binding import RSD_DEBUG_RESIDENT_LOGITS
+    prompts = ri.prompts(71 + rows, rows, 3, 20, sh.vocab)
+    kw = dict(max_step_tokens=5, max_steps=3, max_seq_tokens=52, step_end_id=2, step_end_mod=7, temperature=0.7, seed=8)
+    eng, loop = build_pair((sh, sh, sh), bf16=False, prompts=prompts, loop_kwargs=kw,
+                           engine_kwargs=dict(debug_flags=RSD_DEBUG_KEEP_LOGITS | RSD_DEBUG_RESIDENT_LOGITS))
+    for _ in range(2):
+        _shared_memory_full_of_nan()
+        _, o = parity_step(eng, loop, 2.0, **TOL32)
+        for b in range(rows):
+            n = len(o["draft_trace"][b]["sampled"])
+            assert np.isfinite(eng.logits(0)[b, :n]).all()
+    eng.close()
+
 
 def test_decode_phases_in_one_launch_on_two_streams():
     """Two contexts, a thread and a stream each: each phase takes the whole chip, and none may wait for a part of it."""
