@@ -247,14 +247,17 @@ head_sample_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
       for (int i = 0; i < kCols; i += 4) {
         if (c + i >= M) break;
         // step s of four: row c + i + (q ^ s), for which lane q ^ s of the four holds the block with this lane's word
-        float lg[4] = {v[i], v[i + 1], v[i + 2], v[i + 3]}, run[4], u[4];
+        // need: what a quick score has to reach.  Like sample_kernel's it leaves room for an ulp of the exact score, which is what decides: of two ids that
+        // round to the same score the lower one wins, whichever was found first
+        float lg[4] = {v[i], v[i + 1], v[i + 2], v[i + 3]}, need[4], u[4];
         by_lane(lg, q);
         bool near = false, first = false;
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
-          run[s] = s_run[c + i + (q ^ s)];
-          near = near || lg[s] * inv_t >= run[s] - kNoiseMax || run[s] == -INFINITY;
-          first = first || fabsf(run[s]) == INFINITY;
+          const float run = s_run[c + i + (q ^ s)];
+          need[s] = score_needed(run);
+          near = near || lg[s] * inv_t >= need[s] - kNoiseMax || run == -INFINITY;
+          first = first || fabsf(run) == INFINITY;
         }
         if (!__any_sync(0xFFFFFFFFu, near)) continue;
         const uint4 ph = philox4x32_10(make_uint4((uint32_t)id / 4u, (uint32_t)s_pos[c + i + q], (uint32_t)s_row[c + i + q], (uint32_t)a.model_id), key);
@@ -264,10 +267,11 @@ head_sample_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
         for (int s = 0; s < 4; ++s) u[s] = uniform_from_bits(__shfl_xor_sync(0xFFFFFFFFu, word[s], s));
         unsigned may = 0;
         if (!__any_sync(0xFFFFFFFFu, first)) {
-          // -log(-log u) + x >= run  <=>  u >= exp(-exp(x - run)): errs by less than 2e-6 of the bound, whose arguments lie below 17 where it matters
+          // -log(-log u) + x >= need  <=>  u >= exp(-exp(x - need)).  __expf errs by 2 + 1.173 |argument| ulp, and beyond 17 either way no u
+          // decides: 2.6e-6 of the bound, which the factor covers, and as much of the inner exponential, which is a shift of the score by 2.6e-6: need has 1e-3 of room
 #pragma unroll
           for (int s = 0; s < 4; ++s)
-            may |= u[s] >= __expf(-__expf(fmaf(lg[s], inv_t, -run[s]))) * (1.f - 4e-6f) ? 1u << s : 0u;
+            may |= u[s] >= __expf(-__expf(fmaf(lg[s], inv_t, -need[s]))) * (1.f - 4e-6f) ? 1u << s : 0u;
         } else {
           float sc[4], top[4];
 #pragma unroll
@@ -277,7 +281,7 @@ head_sample_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_consta
 #pragma unroll
             for (int s = 0; s < 4; ++s) top[s] = fmaxf(top[s], __shfl_xor_sync(0xFFFFFFFFu, top[s], x));   // of the eight lanes with the same row (a NaN drops out)
 #pragma unroll
-          for (int s = 0; s < 4; ++s) may |= (sc[s] >= score_needed(fmaxf(run[s], top[s])) && run[s] == run[s]) ? 1u << s : 0u;
+          for (int s = 0; s < 4; ++s) may |= (sc[s] >= fmaxf(need[s], score_needed(top[s])) && need[s] == need[s]) ? 1u << s : 0u;
         }
         while (may != 0u) {
           const int s = __ffs(may) - 1;

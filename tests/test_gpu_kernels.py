@@ -981,6 +981,33 @@ def test_head_that_samples(M, N, K, v_limit, temperature):
             assert (got[row >= 0] == v_limit // 2).all()
 
 
+@pytest.mark.parametrize("score", [60.0, 1e3, 1e5, 1e7])
+@pytest.mark.parametrize("M", [5, 16, 33, 128])
+def test_head_that_samples_among_scores_that_tie(M, score):
+    """Low temperatures: hundreds of ids share the largest logit and their scores differ by less than an ulp often, so the lowest of those that tie
+    must win, whichever CTA comes first.  Against the sampling of the same logits, many positions, each several times."""
+    gen = torch.Generator(device="cuda").manual_seed(M)
+    N, K, v_limit = 50000, 64, 49990
+    W = torch.zeros(N, K, device="cuda")
+    same = torch.randperm(v_limit, generator=gen, device="cuda")[:3000]
+    W[same, 0] = 4.0
+    W[:, 1] = torch.randn(N, generator=gen, device="cuda")
+    W = W.to(torch.bfloat16)
+    W[same, 1] = 0
+    hi = torch.zeros(M, K, dtype=torch.bfloat16, device="cuda")
+    hi[:, 0] = 8.0
+    hi[:, 1] = 0.5
+    lo = torch.zeros_like(hi)
+    row = torch.arange(M, dtype=torch.int32, device="cuda")
+    logits = rb.k_gemm(W, hi, x_lo=lo, impl=3)
+    for i in range(12):
+        pos = torch.randint(0, 100000, (M,), generator=gen, device="cuda").to(torch.int32)
+        want = rb.k_sample(logits, v_limit, 32.0 / score, 9, 2, row, pos)
+        for _ in range(3):
+            got = rb.k_head_sample(W, hi, lo, v_limit, 32.0 / score, 9, 2, row, pos)
+            assert torch.equal(got, want), (i, (got != want).nonzero().flatten().tolist())
+
+
 def test_head_that_samples_scales_its_rows():
     """The denominators of a norm ahead of the head, from sums of squares in one chunk and in many."""
     gen = torch.Generator(device="cuda").manual_seed(3)
