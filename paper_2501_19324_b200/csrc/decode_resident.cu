@@ -12,9 +12,10 @@
 //              until then, and who needs it polls the words themselves (kernel boundary 2.2-2.7 us; barrier by a counter and a load behind it 1.8-2.2;
 //              this 0.9-1.3 for 512-1536 columns, 148 CTAs).  Slots are written once an iteration and there are two sets of them:
 //              an iteration fills one and empties the other.  Everybody sends the ids that it has sampled to everybody else: who has them all
-//              knows that the set of this iteration has been read, and may empty it in the next; and since a fence stands between what a CTA empties
-//              and its ids, the slots are empty for all who poll them in the iteration after (polls are strong loads, past L1, issued after the
-//              ids have been seen).
+//              knows that the set of this iteration has been read, and may empty it in the next.  The ids are also what orders everything that is not
+//              polled itself: a CTA's ids are a release (behind a barrier, a fence by the lanes that send them), whoever has polled them acquires (a fence by the lanes
+//              that polled, ahead of a barrier).  So the slots that a CTA has emptied are empty for all who poll them in the iteration after, and the keys and
+//              values that it has put into pages are there for the CTAs that read them from then on (fp32: the other heads of the group).
 //   products   units of sixteen weight rows (two groups of eight) and all of K; which rows meet in a unit is what its epilogue needs together: the
 //              dims that rotate with one another, gate and up rows of the same features, sixteen features of the residual stream.
 //              bf16: hi + lo operand pairs, eight rows of each as the 16 rows of an mma.sync tile (as in gemm_rows.cu; tcgen05 has no tile this
@@ -94,6 +95,7 @@ __device__ __forceinline__ void st_word(uint32_t* p, uint2 a) { asm volatile("st
 __device__ __forceinline__ void st_word(uint32_t* p, uint4 a) {
   asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w) : "memory");
 }
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 __device__ __forceinline__ bool full(uint32_t v) { return v != kEmpty; }
 __device__ __forceinline__ bool full(uint4 v) { return v.x != kEmpty && v.y != kEmpty && v.z != kEmpty && v.w != kEmpty; }
 // an fp32 result as a word: arithmetic gives one NaN, moves may pass any
@@ -351,7 +353,7 @@ decode_resident_kernel(const __grid_constant__ ResidentParams P, const ResidentL
     feed(Cfg::kStages);
   }
   // Emptying, in iteration `it` >= 1: the set that iteration it - 1 has filled, which everybody has read once all ids of it - 1 are there, and of the four
-  // places of the ids the one of it - 2.  The steps go round the warps; a fence behind the next barrier makes it known ahead of the ids of `it`.
+  // places of the ids the one of it - 2.  The steps go round the warps; the ids of `it` make it known.
   auto empty_slots = [&](int it) {
     uint32_t* set = P.slots + ((it & 1) ? 0u : P.set_words);
     const uint2 e2 = make_uint2(kEmpty, kEmpty);
@@ -379,8 +381,6 @@ decode_resident_kernel(const __grid_constant__ ResidentParams P, const ResidentL
       if (it >= 2 && lane < 2 * kRows) st_word(P.slots + P.at_s + (((it - 2) & 3) * 160 + blockIdx.x) * 32 + lane, kEmpty);
     }
   };
-  bool fence_due = false;
-
   // ---------------- workers ----------------
   Wait wait{P.err, false};
   Ring ring{Cfg::kStages, 0, 0u};
@@ -471,11 +471,9 @@ decode_resident_kernel(const __grid_constant__ ResidentParams P, const ResidentL
     wait.dead = __any_sync(0xFFFFFFFFu, wait.dead);
   };
 
-  // Behind the barrier of a unit: its stages are free, and what the workers emptied ahead of it is made known.  Not by the warp of the epilogue.
+  // Behind the barrier of a unit: its stages are free.  Not by the warp of the epilogue.
   auto behind_unit = [&](int stages) {
     if (warp == ((turn + 4) & (kWarps - 1)) && lane == 0) feed(stages);
-    if (fence_due && warp == ((turn + 6) & (kWarps - 1))) __threadfence();
-    fence_due = false;
   };
 
   // One product: its operand, the CTA's units, their epilogues; false when a wait has expired.
@@ -1151,14 +1149,9 @@ decode_resident_kernel(const __grid_constant__ ResidentParams P, const ResidentL
         ok = product(sp);
       }
       // (behind the first step: whoever waits for it does not wait for this)
-      if (i == 0 && ok && round > 0) { empty_slots(round); fence_due = true; }
+      if (i == 0 && ok && round > 0) empty_slots(round);
     }
     if (!ok) break;
-    if (fence_due) {                             // no unit has come behind the emptying
-      if (sync_or(false)) break;
-      if (warp == 0) __threadfence();
-      fence_due = false;
-    }
     // this CTA's best id of every row, to all CTAs
     unsigned long long mine = best_id == 0x7FFFFFFF ? 0ull : (((unsigned long long)score_key(best_score) << 32) | (uint32_t)(0xFFFFFFFFu - (uint32_t)best_id));
 #pragma unroll
@@ -1177,7 +1170,9 @@ decode_resident_kernel(const __grid_constant__ ResidentParams P, const ResidentL
         v = __shfl_xor_sync(0xFFFFFFFFu, top, o);
         top = v > top ? v : top;
       }
-      // what this CTA has emptied in this iteration is empty for everybody who reads an id of it (behind_unit's fence).  (score, id + 1): neither is ever kEmpty, a score with those bits would be a NaN
+      // what this CTA has written in this iteration is there for everybody who reads an id of it
+      fence_gpu();
+      // (score, id + 1): neither is ever kEmpty, a score with those bits would be a NaN
       if (t == 0 && ((active >> g) & 1u))
         st_word(ids + blockIdx.x * 32 + g * 2, top == 0ull ? make_uint2(0u, 0u) : make_uint2((uint32_t)(top >> 32), 0xFFFFFFFFu - (uint32_t)top + 1u));
     }
@@ -1197,6 +1192,7 @@ decode_resident_kernel(const __grid_constant__ ResidentParams P, const ResidentL
         if (!(two & 1u)) x.x = x.y = 0u;         // rows that have ended publish nothing
         if (!(two & 2u)) x.z = x.w = 0u;
       });
+      fence_gpu();                               // and what the others had written ahead of their ids is seen from here on
       unsigned long long top[2] = {0ull, 0ull};
 #pragma unroll
       for (int i = 0; i < NP; ++i) {

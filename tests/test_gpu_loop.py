@@ -677,6 +677,23 @@ def test_fp32_decode_phase_in_one_launch_reads_what_it_wrote(sh, rows):
     eng.close()
 
 
+@pytest.mark.parametrize("H,KV", [(4, 2), (8, 1), (16, 2)])
+def test_fp32_decode_phase_in_one_launch_over_its_own_keys(H, KV):
+    """A group's new key and value are put into the page by the CTA of its first head and read by those of the others, iteration after iteration of one
+    launch: long steps behind short prompts, so that nearly all that is attended was written by the phase itself."""
+    from paper_2501_19324_b200 import RSD_DEBUG_KEEP_LOGITS
+    from paper_2501_19324_b200.binding import RSD_DEBUG_RESIDENT_LOGITS
+    sh = ri.ModelShape(3, 256, H, KV, 64, 344, 500)
+    prompts = ri.prompts(5, 3, 2, 4, sh.vocab)
+    kw = dict(max_step_tokens=70, max_steps=2, max_seq_tokens=150, step_end_id=-1, temperature=0.7, seed=3)
+    eng, loop = build_pair((sh, sh, sh), bf16=False, prompts=prompts, loop_kwargs=kw,
+                           engine_kwargs=dict(debug_flags=RSD_DEBUG_KEEP_LOGITS | RSD_DEBUG_RESIDENT_LOGITS))
+    stats = {}
+    parity_step(eng, loop, 2.0, stats=stats, **TOL32)
+    assert stats["tokens"] == 2 * 3 * 70
+    eng.close()
+
+
 def test_decode_phases_in_one_launch_on_two_streams():
     """Two contexts, a thread and a stream each: each phase takes the whole chip, and none may wait for a part of it."""
     import threading
