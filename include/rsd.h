@@ -279,6 +279,9 @@ uint64_t rsd_debug_launch_count(void);
  * iteration `iteration` of every decode phase from now on; -1 (the default) never.  For testing that a failing phase
  * ends early with RSD_ERR_TIMEOUT.                                                              */
 int rsd_debug_fail_iteration(rsd_ctx*, int32_t iteration);
+/* From now on launches whose CTAs wait for one another see at most `sms` SMs (0, the default: as many as the stream has).
+ * For testing that phases go on kernel by kernel where a stream has a part of the chip.         */
+int rsd_debug_sm_limit(rsd_ctx*, int32_t sms);
 /* Timeline of the last launch of the persistent decode kernel of model `which` (RSD_DRAFT or RSD_TARGET),
  * recorded by its first CTA when RSD_DEBUG_MEGA_PROFILE is set: stamps[0] = kernel start, then for every
  * grid barrier the global-timer value (ns) when the CTA's phase work was done and when the barrier let it

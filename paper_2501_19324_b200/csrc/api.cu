@@ -118,6 +118,7 @@ struct rsd_ctx {
   int sd_k = 0, slots_max = 0;
 
   int fail_at = -1;            // rsd_debug_fail_iteration
+  int sm_limit = 0;            // rsd_debug_sm_limit
   bool host_sleeps = false, host_yields = false;   // how this process waits for the device (cudaGetDeviceFlags)
   unsigned long long* progress = nullptr;   // pinned: how far the running decode phase is (RowState::progress)
   int pass_width = 1;          // consecutive positions of a row that a decode pass writes (a speculative round: sd_k)
@@ -830,7 +831,6 @@ int model_logits(rsd_ctx* c, int which, PassView p, bool allow_mega, cudaStream_
   return rc;
 }
 
-// Enqueues one decode iteration: model pass, final norm, lm_head, sample, append (and lay out the next one).
 // Decode passes of the fused bf16 path whose logits nobody keeps sample in the head's epilogue (head_sample.cu).
 bool head_samples(const rsd_ctx* c, int which, PassView p, bool keep_logits) {
   const rsd_model& m = c->mdl[which].m;
@@ -847,6 +847,7 @@ int decode_and_sample(rsd_ctx* c, int which, PassView p, const SampleArgs& a, cu
   });
 }
 
+// Enqueues one decode iteration: model pass, final norm, lm_head, sample, append (and lay out the next one).
 int decode_iteration(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t s) {
   const rsd_model& m = c->mdl[which].m;
   PassView p{c->st.pass_tok_id, c->st.pass_tok_row, c->st.pass_tok_pos, n_slots, c->st.n_active};
@@ -1010,9 +1011,12 @@ int decode_phase(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t s) 
   if (n_slots <= 0) return RSD_OK;
   if (resident_wanted(c, which, n_slots)) {
     if (c->fail_at >= 0 && c->fail_at < c->C) CU(cudaMemsetAsync((char*)c->gemm_scratch + 4096, 0xFF, sizeof(int32_t), s));   // ahead of the first
-    CU(launch_decode_resident(c->resident_plan[which], c->resident_block[which], c->resident_shape[which], c->mdl[which].kv_dtype == 3, c->st, which,
-                              phase, n_slots, c->lp, s));
-    return RSD_OK;
+    const cudaError_t e = launch_decode_resident(c->resident_plan[which], c->resident_block[which], c->resident_shape[which], c->mdl[which].kv_dtype == 3,
+                                                 c->st, which, phase, n_slots, c->lp, c->sm_limit, s);
+    if (e != cudaErrorCooperativeLaunchTooLarge) {
+      CU(e);
+      return RSD_OK;
+    }
   }
   const bool graphs = !(c->cfg.debug_flags & RSD_DEBUG_NO_GRAPHS);
   // The attention kernel splits every row's context over so many CTAs that the ACTIVE rows fill the machine; the
@@ -1637,6 +1641,12 @@ int rsd_debug_gemm_timing(rsd_ctx* c, int32_t stride, double* ms, double* bytes,
 int rsd_debug_fail_iteration(rsd_ctx* c, int32_t iteration) {
   if (!c || iteration < -1) return RSD_ERR_ARG;
   c->fail_at = iteration;
+  return RSD_OK;
+}
+
+int rsd_debug_sm_limit(rsd_ctx* c, int32_t sms) {
+  if (!c || sms < 0) return RSD_ERR_ARG;
+  c->sm_limit = sms;
   return RSD_OK;
 }
 

@@ -1278,6 +1278,41 @@ int device_sms() {
   return n;
 }
 
+template <typename F> void driver_entry(F& fn, const char* name) {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  fn = cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess ? (F)p : nullptr;
+  (void)cudaGetLastError();
+}
+
+// SMs that launches into `s` may come to: the device's, or those of the part of it that the stream's green context, or the current context, has.
+int stream_sms(cudaStream_t s) {
+  struct Driver {
+    decltype(&cuStreamGetGreenCtx) green_of;
+    decltype(&cuGreenCtxGetDevResource) of_green;
+    decltype(&cuCtxGetCurrent) current;
+    decltype(&cuCtxGetDevResource) of_ctx;
+    Driver() {
+      driver_entry(green_of, "cuStreamGetGreenCtx");
+      driver_entry(of_green, "cuGreenCtxGetDevResource");
+      driver_entry(current, "cuCtxGetCurrent");
+      driver_entry(of_ctx, "cuCtxGetDevResource");
+    }
+  };
+  static const Driver drv;
+  int n = device_sms();
+  CUdevResource r{};
+  CUgreenCtx green = nullptr;
+  CUcontext ctx = nullptr;
+  const bool named = s != nullptr && s != cudaStreamLegacy && s != cudaStreamPerThread;
+  if (named && drv.green_of && drv.of_green && drv.green_of((CUstream)s, &green) == CUDA_SUCCESS && green != nullptr) {
+    if (drv.of_green(green, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS) n = std::min(n, (int)r.sm.smCount);
+  } else if (drv.current && drv.of_ctx && drv.current(&ctx) == CUDA_SUCCESS && ctx != nullptr) {
+    if (drv.of_ctx(ctx, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS) n = std::min(n, (int)r.sm.smCount);
+  }
+  return n;
+}
+
 int grid_of(const ResidentShape& m, int sms) { return std::min(std::min(sms, m.F / 8), 160); }
 
 struct Words { uint32_t x, y, q, a, f, s, set, all; };
@@ -1315,6 +1350,8 @@ static_assert(sizeof(ResidentParams) <= sizeof(ResidentPlan) && alignof(Resident
 cudaError_t resident_build(ResidentPlan* plan, void* dev_block, const ResidentBuild& a, cudaStream_t s) {
   const ResidentShape& m = a.shape;
   const int grid = grid_of(m, device_sms());
+  int dev = 0, cooperative = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&cooperative, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !cooperative) return cudaErrorNotSupported;
   if (!resident_supported(m) || grid < 1 || (m.d / 16 + grid - 1) / grid > kOwn || (m.f32 && ((uintptr_t)a.kv_pool & 15))) return cudaErrorNotSupported;
   std::vector<uint8_t> host(resident_block_bytes(m.n_layers) + 128);
   uint8_t* hb = (uint8_t*)(((uintptr_t)host.data() + 127) & ~(uintptr_t)127);
@@ -1358,16 +1395,18 @@ cudaError_t launch_as(const ResidentPlan& plan, const void* dev_block, int grid,
   attr[0].val.cooperative = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, decode_resident_kernel<F32, EXT, MT>, P, Ls, st, which, phase, n_slots, lp);
+  if (e == cudaErrorCooperativeLaunchTooLarge) (void)cudaGetLastError();     // the caller has another way
   return e != cudaSuccess ? e : launched(1);
 }
 
 }  // namespace
 
 cudaError_t launch_decode_resident(const ResidentPlan& plan, const void* dev_block, const ResidentShape& m, bool kv_extended, const RowState& st, int which,
-                                   int phase, int n_slots, const LoopParams& lp, cudaStream_t s) {
+                                   int phase, int n_slots, const LoopParams& lp, int sm_limit, cudaStream_t s) {
   if (n_slots < 1 || n_slots > kRows) return cudaErrorNotSupported;
   const int sms = device_sms();
   if (sms <= 0) return cudaErrorInvalidDevice;
+  if (grid_of(m, sms) > (sm_limit > 0 ? std::min(sm_limit, stream_sms(s)) : stream_sms(s))) return cudaErrorCooperativeLaunchTooLarge;
   const cudaError_t e = cudaMemsetAsync(reinterpret_cast<const ResidentParams*>(plan.bytes)->slots, 0xFF, resident_slot_bytes(m), s);
   if (e != cudaSuccess) return e;
   const int grid = grid_of(m, sms);

@@ -228,6 +228,13 @@ size_t resident_slot_bytes(const ResidentShape& m);
 // Fills the plan, and dev_block (256-byte aligned) with the layers' tensor maps and pointers; cudaErrorNotSupported: weights or pools
 // that TMA or 16-byte loads cannot take.
 cudaError_t resident_build(ResidentPlan* plan, void* dev_block, const ResidentBuild& a, cudaStream_t s);
+struct RowState;
+struct LoopParams;
+// Runs the decode phase that launch_decode_begin has opened, n_slots <= 8, to its end.  cudaErrorCooperativeLaunchTooLarge, and nothing done: the stream has
+// fewer SMs than the launch has CTAs, which wait for one another (it belongs to a part of the chip); sm_limit > 0: as if it had no more than these.
+cudaError_t launch_decode_resident(const ResidentPlan& plan, const void* dev_block, const ResidentShape& m, bool kv_extended, const RowState& st, int which,
+                                   int phase, int n_slots, const LoopParams& lp, int sm_limit, cudaStream_t s);
+
 struct SampleArgs {
   const float* logits;         // [n_slots, V]
   int n_slots, V, v_limit;
@@ -316,9 +323,6 @@ inline __host__ __device__ bool target_pass_due(int n_waiting, int n_live, int m
   return n_waiting > 0 && n_waiting >= (want < n_live ? want : n_live);
 }
 cudaError_t launch_decode_begin(const RowState& st, int which, int phase, cudaStream_t s);
-// Runs the decode phase that launch_decode_begin has opened, n_slots <= 8, to its end.
-cudaError_t launch_decode_resident(const ResidentPlan& plan, const void* dev_block, const ResidentShape& m, bool kv_extended, const RowState& st, int which,
-                                   int phase, int n_slots, const LoopParams& lp, cudaStream_t s);
 // Merged PRM: one slot per row that took a draft step, carrying the step's last token at the draft's
 // cursor (which stays where it is); n_active = number of such rows, last_idx[b] = b for them.
 cudaError_t launch_score_prepare(const RowState& st, cudaStream_t s);

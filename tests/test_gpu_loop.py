@@ -694,6 +694,26 @@ def test_fp32_decode_phase_in_one_launch_over_its_own_keys(H, KV):
     eng.close()
 
 
+@pytest.mark.parametrize("sh,bf16", [(ri.ModelShape(2, 512, 4, 2, 128, 1408, 4096), True), (ri.ModelShape(2, 256, 4, 2, 64, 688, 1024), False)], ids=["bf16", "fp32"])
+def test_decode_phase_where_one_launch_does_not_fit(sh, bf16):
+    """A stream that belongs to a part of the chip cannot hold all the CTAs of the one launch at once: the phase runs kernel by kernel, not at all wrong
+    or refused, and in one launch again where there is room."""
+    from paper_2501_19324_b200 import lib, RSD_DEBUG_KEEP_LOGITS
+    from paper_2501_19324_b200.binding import RSD_DEBUG_RESIDENT_LOGITS
+    prompts = ri.prompts(12, 3, 10, 40, sh.vocab)
+    kw = dict(max_step_tokens=12, max_steps=4, max_seq_tokens=100, step_end_id=2, step_end_mod=50, temperature=0.7, seed=6)
+    eng, loop = build_pair((sh, sh, sh), bf16=bf16, prompts=prompts, loop_kwargs=kw,
+                           engine_kwargs=dict(debug_flags=RSD_DEBUG_KEEP_LOGITS | RSD_DEBUG_RESIDENT_LOGITS))
+    launches = []
+    for sms in (0, 40, 0):
+        assert lib().rsd_debug_sm_limit(eng.ctx, sms) == 0
+        before = lib().rsd_debug_launch_count()
+        parity_step(eng, loop, 2.0, **(TOL16 if bf16 else TOL32))
+        launches.append(lib().rsd_debug_launch_count() - before)
+    assert launches[1] > 2 * max(launches[0], launches[2])
+    eng.close()
+
+
 def test_decode_phases_in_one_launch_on_two_streams():
     """Two contexts, a thread and a stream each: each phase takes the whole chip, and none may wait for a part of it."""
     import threading
