@@ -21,6 +21,7 @@ RSD_DEBUG_PERSISTENT_DECODE = 4
 RSD_DEBUG_MEGA_PROFILE = 8
 RSD_DEBUG_NO_F16_DENSE = 16
 RSD_DEBUG_RESIDENT_LOGITS = 32
+RSD_DEBUG_LOGITS_AS_DECODED = 64
 ERRORS = {0: "RSD_OK", -1: "RSD_ERR_ARG", -2: "RSD_ERR_STATE", -3: "RSD_ERR_OOM_PAGES", -4: "RSD_ERR_CUDA",
           -5: "RSD_ERR_TIMEOUT", -6: "RSD_ERR_UNSUPPORTED"}
 

@@ -993,11 +993,11 @@ int follow_phase(rsd_ctx* c, int launched, cudaStream_t s, bool* ended) {
   }
 }
 
-// Whether the phase runs in one launch (decode_resident.cu).  Single kernels are timed, logits are kept, kernel by kernel.
+// Whether the phase runs in one launch (decode_resident.cu).  Single kernels are timed, and logits are kept, unless the caller says otherwise, kernel by kernel.
 bool resident_wanted(const rsd_ctx* c, int which, int n_slots) {
   const int flags = c->cfg.debug_flags;
   return c->resident[which] && n_slots <= 8 && c->time_stride == 0 && !(flags & RSD_DEBUG_NO_GRAPHS) && c->mega_B[which] != c->st.B &&
-         (!(flags & RSD_DEBUG_KEEP_LOGITS) || (flags & RSD_DEBUG_RESIDENT_LOGITS));
+         (!(flags & RSD_DEBUG_KEEP_LOGITS) || (flags & (RSD_DEBUG_RESIDENT_LOGITS | RSD_DEBUG_LOGITS_AS_DECODED)));
 }
 
 // One decode phase: up to C iterations, fewer when every row ends before.

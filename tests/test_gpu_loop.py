@@ -694,6 +694,34 @@ def test_fp32_decode_phase_in_one_launch_over_its_own_keys(H, KV):
     eng.close()
 
 
+@pytest.mark.parametrize("temperature", [0.0, 0.7])
+@pytest.mark.parametrize("sh,bf16", [(ri.ModelShape(2, 512, 4, 2, 128, 1408, 4096), True), (ri.ModelShape(4, 512, 8, 2, 64, 1376, 1024), False)], ids=["bf16", "fp32"])
+def test_kept_logits_are_those_of_the_tokens(sh, bf16, temperature):
+    """Logits kept with RSD_DEBUG_LOGITS_AS_DECODED change nothing: the steps and rewards of a small model are, bit by bit, those without them, and a greedy
+    token is the first of the largest logits."""
+    from paper_2501_19324_b200 import Engine, Model, RSD_DEBUG_KEEP_LOGITS, RSD_DEBUG_LOGITS_AS_DECODED
+    heads = (ri.HEAD_LM, ri.HEAD_REWARD_SIGMOID, ri.HEAD_LM)
+    models = [Model(sh, ri.gpu_model_tensors(sh, slot, 0, bf16, hk), hk) for slot, hk in enumerate(heads)]
+    tokens, offsets = ri.prompts(44, 5, 5, 60, sh.vocab)
+    got = []
+    for flags in (0, RSD_DEBUG_KEEP_LOGITS | RSD_DEBUG_LOGITS_AS_DECODED):
+        eng = Engine(*models, max_batch=5, max_seq_tokens=160, max_step_tokens=20, max_steps=4, step_end_id=1, step_end_mod=15,
+                     temperature=temperature, seed=2, debug_flags=flags)
+        eng.prefill(tokens, offsets)
+        steps = []
+        for delta, which in ((2.0, 2), (0.0, 0), (2.0, 2)):            # every row by the target, none, every row
+            r = eng.step(delta)
+            steps.append({k: v.tobytes() for k, v in r.items()})
+            if flags and temperature == 0.0:
+                kept = eng.logits(which)
+                for b in range(5):
+                    n = r["step_len"][b]
+                    assert (kept[b, :n].argmax(1) == r["step_tokens"][b, :n]).all()
+        got.append(steps)
+        eng.close()
+    assert got[0] == got[1]
+
+
 @pytest.mark.parametrize("sh,bf16", [(ri.ModelShape(2, 512, 4, 2, 128, 1408, 4096), True), (ri.ModelShape(2, 256, 4, 2, 64, 688, 1024), False)], ids=["bf16", "fp32"])
 def test_decode_phase_where_one_launch_does_not_fit(sh, bf16):
     """A stream that belongs to a part of the chip cannot hold all the CTAs of the one launch at once: the phase runs kernel by kernel, not at all wrong
