@@ -138,8 +138,8 @@ enum {
                                 (by default a bf16 model that uses the pairs gets fp16 copies of its layer
                                 matrices in the workspace, up to 20 GB a model, and those passes run on them
                                 with one fp16 activation operand: half the tensor-core work)             */
-  RSD_DEBUG_RESIDENT_LOGITS = 32, /* with RSD_DEBUG_KEEP_LOGITS: small models decode in one launch a phase all the same
-                                (by default logits are kept by the kernels of single iterations)         */
+  RSD_DEBUG_RESIDENT_LOGITS = 32, /* with RSD_DEBUG_KEEP_LOGITS: small models decode in one launch a phase wherever that works, faster or
+                                not (by default logits are kept by the kernels of single iterations)     */
   RSD_DEBUG_LOGITS_AS_DECODED = 64 /* with RSD_DEBUG_KEEP_LOGITS: logits are kept by whatever decodes without that flag; steps and rewards are the
                                 same bits as without it.  RSD_DEBUG_KEEP_LOGITS by itself, like RSD_DEBUG_NO_GRAPHS and
                                 rsd_debug_gemm_timing, means single kernels also where a phase would be one launch: sums are then rounded

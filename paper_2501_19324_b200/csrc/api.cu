@@ -117,6 +117,8 @@ struct rsd_ctx {
   uint64_t dec_graph_kernels[16] = {};
   int sd_k = 0, slots_max = 0;
 
+  std::vector<int> z_host;     // tokens of each row
+  int z_max = 0;               // the most that a row which goes on has
   int fail_at = -1;            // rsd_debug_fail_iteration
   int sm_limit = 0;            // rsd_debug_sm_limit
   bool host_sleeps = false, host_yields = false;   // how this process waits for the device (cudaGetDeviceFlags)
@@ -996,8 +998,12 @@ int follow_phase(rsd_ctx* c, int launched, cudaStream_t s, bool* ended) {
 // Whether the phase runs in one launch (decode_resident.cu).  Single kernels are timed, and logits are kept, unless the caller says otherwise, kernel by kernel.
 bool resident_wanted(const rsd_ctx* c, int which, int n_slots) {
   const int flags = c->cfg.debug_flags;
-  return c->resident[which] && n_slots <= 8 && c->time_stride == 0 && !(flags & RSD_DEBUG_NO_GRAPHS) && c->mega_B[which] != c->st.B &&
-         (!(flags & RSD_DEBUG_KEEP_LOGITS) || (flags & (RSD_DEBUG_RESIDENT_LOGITS | RSD_DEBUG_LOGITS_AS_DECODED)));
+  if (!c->resident[which] || n_slots > 8 || c->time_stride != 0 || (flags & RSD_DEBUG_NO_GRAPHS) || c->mega_B[which] == c->st.B) return false;
+  if (flags & RSD_DEBUG_KEEP_LOGITS) {
+    if (flags & RSD_DEBUG_RESIDENT_LOGITS) return true;
+    if (!(flags & RSD_DEBUG_LOGITS_AS_DECODED)) return false;
+  }
+  return resident_pays(c->resident_shape[which], n_slots, c->z_max + c->C);
 }
 
 // One decode phase: up to C iterations, fewer when every row ends before.
@@ -1314,6 +1320,9 @@ int rsd_prefill(rsd_ctx* c, const int32_t* tokens, const int32_t* offsets, int32
   int rc = rsd_reset(c);
   if (rc) return rc;
   c->st.B = B;
+  c->z_host.resize(B);
+  c->z_max = 0;
+  for (int b = 0; b < B; ++b) c->z_max = std::max(c->z_max, c->z_host[b] = offsets[b + 1] - offsets[b]);
   // stage the ragged prompt in the pass-list buffers, then scatter it into the row buffers
   CU(cudaMemcpyAsync(c->st.pass_tok_id, tokens, sizeof(int32_t) * total, cudaMemcpyHostToDevice, s));
   CU(cudaMemcpyAsync(c->st.pass_tok_row, offsets, sizeof(int32_t) * (B + 1), cudaMemcpyHostToDevice, s));
@@ -1452,6 +1461,11 @@ static int step_impl(rsd_ctx* c, float delta, int min_target_rows, void* cuda_st
       CU(cudaEventElapsedTime(&ms, c->ph_ev[i], c->ph_ev[i + 1]));
       c->ph_ms[i] += ms;
     }
+  }
+  c->z_max = 0;
+  for (int b = 0; b < B; ++b) {
+    c->z_host[b] += h_len[b];
+    if (h_live[b]) c->z_max = std::max(c->z_max, c->z_host[b]);
   }
   // counters (Section 3.3 accounting): draft tokens when they are generated, steps when they are committed
   uint64_t gen_d = 0, gen_t = 0, n_acc = 0, n_tgt = 0, discarded = 0, n_scored = 0;

@@ -1342,6 +1342,34 @@ bool resident_supported(const ResidentShape& m) {
   return m.hd == 128 && m.H / m.KV <= 8 && m.d % 64 == 0 && m.F % 64 == 0;
 }
 
+// Where the one launch is faster than graphs of the single kernels (kernels / here, us an iteration, two to 24 layers; each line where it stops):
+//   split       the grid is d_ffn / 8 CTAs at most.  With fewer than 80, fewer than columns / 8 (bf16: or than 148), more qkv units than CTAs or more pairs of the attention the
+//               CTAs take turns, while kernels choose another split: d_ffn 64 to 640 at 64 to 1792 columns 0.1-0.9, 16 heads of 128 for 256 columns 0.94.
+//               fp32 products of five to eight rows gain more than that (2048 columns, 192 units, 256 pairs, 1.27).  Where d_ffn is more than four times the
+//               columns, or the heads more than twice, the residual stream has few owners that work while all wait: 0.78-0.97.
+//   vocabulary  a head unit is 0.4 us and a barrier here, kernels stream: bf16, two layers of 512 columns, 4096 / 8192 / 16384 / 32000 / 151936 ids
+//               1.25 / 1.18 / 1.06 / 0.83 / 0.45; a layer makes up for 1000 ids (24 layers, 32000 ids 1.06).  fp32, whose kernels' head is slower, by columns:
+//               256 (88 CTAs), 8192 / 16384 / 50000 ids, one row 1.12 / 1.00 / 0.75, 8 rows, 32000 1.02; 512, 50000 / 100000 1.03 / 0.96; 1024, 100000 1.05.
+//   width       the weights come no faster here: bf16, one row, 1792 / 2048 columns 1.03 / 0.94; fp32, one / four rows (the products are for four), 1024 1.10 / 1.18,
+//               1280 0.90 / 1.05, 2048 0.85 / 0.99, five rows 1.07, and columns that do not fill their last stage, 384 to 1248, 0.82-0.96.
+//   context     one CTA walks all of a pair's, attn_decode.cu splits it: bf16, 512 columns, one / eight rows, 200 / 600 / 800 / 2000 / 12000 tokens
+//               1.21 / 1.03 / 0.96 / 0.74 / 0.27 and 1.26 / 1.10 / 1.01 / 0.79 / 0.32, 1024 columns, one row, 400 / 600 1.04 / 0.99; fp32, 256 columns,
+//               one / eight rows, 400 / 600 / 1000 1.01 / 0.98 / 0.92 and 1.17 / 1.11 / 1.03, 768, four rows, 400 / 600 1.02 / 0.95, 1024, one / two / four
+//               rows, 200 0.97 / 1.00 / 1.06, 400 0.92 / 0.93 / 0.99, 1536, eight rows, 400 / 600 1.07 / 0.99.  A layer gains less than head, sampling and update do, which one
+//               iteration has once: 22 layers of 512 columns, bf16, six rows, 600 0.86; 18 of 384, fp32, one row, 300 0.87.
+// 84 shapes, rows and contexts drawn at random from what is taken: 0.93-1.40, a tenth below 0.99, 1.11 in the middle.
+bool resident_pays(const ResidentShape& m, int rows, int tokens) {
+  const int grid = grid_of(m, 148), pairs = rows * (m.f32 ? m.H : m.KV);
+  const bool many = m.f32 && rows > 4;
+  if (grid < 80 || m.F < (m.f32 ? m.d : std::min(m.d, 1184)) || m.F > 4 * m.d || m.H * m.hd > 2 * m.d) return false;
+  if (((m.H + 2 * m.KV) * m.hd / 16 > grid && !(many && m.d >= 1536)) || pairs > (many ? 2 * grid : grid)) return false;
+  const auto walk = [&](int at_most, int a_layer, int once) { return tokens <= std::min(at_most, a_layer + once / m.n_layers); };
+  if (!m.f32) return m.vocab <= 1024 * (m.n_layers + 6) && m.d <= 1792 && walk(512 + 32 * rows, 320 + 16 * rows, 1200);
+  if (m.vocab > (many ? 128 : 64) * m.d * grid / 148 || (m.d > 256 && m.d % StageK<true>::value != 0)) return false;
+  if (many) return walk(m.d <= 512 ? 800 : 448, 400, 1200);
+  return m.d <= 1024 && walk(m.d <= 512 ? 448 : m.d <= 768 ? 320 : 64 * (rows + 1), 200, 750);
+}
+
 size_t resident_block_bytes(int n_layers) { return (size_t)n_layers * sizeof(ResidentLayer); }
 size_t resident_slot_bytes(const ResidentShape& m) { return (size_t)words_of(m).all * 4; }
 

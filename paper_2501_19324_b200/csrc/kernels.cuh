@@ -223,6 +223,7 @@ struct ResidentBuild {
 };
 struct ResidentPlan { alignas(128) unsigned char bytes[512]; };   // the kernel's parameters
 bool resident_supported(const ResidentShape& m);
+bool resident_pays(const ResidentShape& m, int rows, int tokens);      // faster than single kernels; tokens: the most that a row may come to in the phase
 size_t resident_block_bytes(int n_layers);
 size_t resident_slot_bytes(const ResidentShape& m);
 // Fills the plan, and dev_block (256-byte aligned) with the layers' tensor maps and pointers; cudaErrorNotSupported: weights or pools

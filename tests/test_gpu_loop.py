@@ -742,6 +742,37 @@ def test_decode_phase_where_one_launch_does_not_fit(sh, bf16):
     eng.close()
 
 
+@pytest.mark.parametrize("sh,bf16,prompt,one_launch", [
+    (ri.ModelShape(2, 512, 4, 2, 128, 1408, 4096), True, 520, [1, 1, 0]),         # bf16, one row: 544 tokens
+    (ri.ModelShape(2, 256, 4, 2, 64, 688, 1024), False, 424, [1, 1, 0]),          # fp32, one row: 448
+    (ri.ModelShape(1, 256, 2, 1, 128, 704, 7168), True, 20, [1]),                 # a vocabulary of 1024 ids a layer and 6144
+    (ri.ModelShape(1, 256, 2, 1, 128, 704, 7176), True, 20, [0]),
+    (ri.ModelShape(1, 160, 1, 1, 64, 640, 5535), False, 20, [1]),                 # 64 a column, by the CTAs' share of 148
+    (ri.ModelShape(1, 160, 1, 1, 64, 640, 5536), False, 20, [0]),
+    (ri.ModelShape(1, 1792, 2, 1, 128, 1216, 300), True, 20, [1]),                # columns
+    (ri.ModelShape(1, 1856, 2, 1, 128, 1216, 300), True, 20, [0]),
+    (ri.ModelShape(1, 1040, 2, 1, 64, 1200, 300), False, 20, [0]),
+    (ri.ModelShape(1, 256, 2, 1, 128, 576, 300), True, 20, [0]),                  # 72 CTAs
+    (ri.ModelShape(1, 768, 2, 1, 64, 760, 300), False, 20, [0]),                  # 95, fewer than columns / 8
+    (ri.ModelShape(1, 1024, 16, 2, 128, 1152, 300), True, 20, [0]),               # 160 units of qkv for 144
+    (ri.ModelShape(1, 192, 1, 1, 128, 768, 300), True, 20, [1]),                  # d_ffn, heads beside the columns
+    (ri.ModelShape(1, 192, 1, 1, 128, 832, 300), True, 20, [0]),
+    (ri.ModelShape(1, 256, 5, 1, 128, 704, 300), True, 20, [0]),
+], ids=["bf16-ctx", "fp32-ctx", "bf16-ids", "bf16-ids+", "fp32-ids", "fp32-ids+", "bf16-wide", "bf16-wide+", "fp32-wide+", "grid", "fp32-grid", "qkv", "ffn", "ffn+", "heads+"])
+def test_where_decode_phases_are_one_launch(sh, bf16, prompt, one_launch):
+    """On both sides of each line between the one launch and the single kernels, and across it as a row grows."""
+    from paper_2501_19324_b200 import lib, RSD_DEBUG_KEEP_LOGITS, RSD_DEBUG_LOGITS_AS_DECODED
+    prompts = ri.prompts(15, 1, prompt, prompt, sh.vocab)
+    kw = dict(max_step_tokens=12, max_steps=4, max_seq_tokens=prompt + 48, step_end_id=-1, temperature=0.7, seed=6)
+    eng, loop = build_pair((sh, sh, sh), bf16=bf16, prompts=prompts, loop_kwargs=kw,
+                           engine_kwargs=dict(debug_flags=RSD_DEBUG_KEEP_LOGITS | RSD_DEBUG_LOGITS_AS_DECODED))
+    for one in one_launch:
+        before = lib().rsd_debug_launch_count()
+        parity_step(eng, loop, 2.0, **(TOL16 if bf16 else TOL32))
+        assert (lib().rsd_debug_launch_count() - before < 100) == bool(one)       # two phases of 12 iterations, eight kernels or more each
+    eng.close()
+
+
 def test_decode_phases_in_one_launch_on_two_streams():
     """Two contexts, a thread and a stream each: each phase takes the whole chip, and none may wait for a part of it."""
     import threading
