@@ -286,6 +286,9 @@ int rsd_debug_fail_iteration(rsd_ctx*, int32_t iteration);
 /* From now on launches whose CTAs wait for one another see at most `sms` SMs (0, the default: as many as the stream has).
  * For testing that phases go on kernel by kernel where a stream has a part of the chip.         */
 int rsd_debug_sm_limit(rsd_ctx*, int32_t sms);
+/* From now on such launches leave room as if `n` step calls of this process were running on the device (0, the default: as many as are).
+ * For testing that the results do not depend on it.                                             */
+int rsd_debug_step_calls(rsd_ctx*, int32_t n);
 /* Timeline of the last launch of the persistent decode kernel of model `which` (RSD_DRAFT or RSD_TARGET),
  * recorded by its first CTA when RSD_DEBUG_MEGA_PROFILE is set: stamps[0] = kernel start, then for every
  * grid barrier the global-timer value (ns) when the CTA's phase work was done and when the barrier let it

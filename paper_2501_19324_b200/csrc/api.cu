@@ -6,6 +6,7 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <atomic>
 #include <chrono>
 #include <string>
 #include <thread>
@@ -120,7 +121,8 @@ struct rsd_ctx {
   std::vector<int> z_host;     // tokens of each row
   int z_max = 0;               // the most that a row which goes on has
   int fail_at = -1;            // rsd_debug_fail_iteration
-  int sm_limit = 0;            // rsd_debug_sm_limit
+  int sm_limit = 0, as_sharers = 0;   // rsd_debug_sm_limit, rsd_debug_step_calls
+  int device = 0;              // of the running step
   bool host_sleeps = false, host_yields = false;   // how this process waits for the device (cudaGetDeviceFlags)
   unsigned long long* progress = nullptr;   // pinned: how far the running decode phase is (RowState::progress)
   int pass_width = 1;          // consecutive positions of a row that a decode pass writes (a speculative round: sd_k)
@@ -995,6 +997,20 @@ int follow_phase(rsd_ctx* c, int launched, cudaStream_t s, bool* ended) {
   }
 }
 
+// Step calls of this process that are running, by device: how many callers there are to share its SMs among (decode_resident.cu; no result depends on it).
+std::atomic<int>& step_calls(int device) {
+  static std::atomic<int> running[64];
+  return running[device & 63];
+}
+
+struct StepCall {
+  int device;
+  explicit StepCall(int d) : device(d) { step_calls(device).fetch_add(1); }
+  ~StepCall() { step_calls(device).fetch_sub(1); }
+  StepCall(const StepCall&) = delete;
+  StepCall& operator=(const StepCall&) = delete;
+};
+
 // Whether the phase runs in one launch (decode_resident.cu).  Single kernels are timed, and logits are kept, unless the caller says otherwise, kernel by kernel.
 bool resident_wanted(const rsd_ctx* c, int which, int n_slots) {
   const int flags = c->cfg.debug_flags;
@@ -1018,7 +1034,7 @@ int decode_phase(rsd_ctx* c, int which, int phase, int n_slots, cudaStream_t s) 
   if (resident_wanted(c, which, n_slots)) {
     if (c->fail_at >= 0 && c->fail_at < c->C) CU(cudaMemsetAsync((char*)c->gemm_scratch + 4096, 0xFF, sizeof(int32_t), s));   // ahead of the first
     const cudaError_t e = launch_decode_resident(c->resident_plan[which], c->resident_block[which], c->resident_shape[which], c->mdl[which].kv_dtype == 3,
-                                                 c->st, which, phase, n_slots, c->lp, c->sm_limit, s);
+                                                 c->st, which, phase, n_slots, c->lp, c->as_sharers > 0 ? c->as_sharers : step_calls(c->device).load(), c->sm_limit, s);
     if (e != cudaErrorCooperativeLaunchTooLarge) {
       CU(e);
       return RSD_OK;
@@ -1387,6 +1403,8 @@ static int step_impl(rsd_ctx* c, float delta, int min_target_rows, void* cuda_st
   const int B = c->st.B;
   Scalars sc;
   int rc;
+  CU(cudaGetDevice(&c->device));
+  const StepCall running(c->device);
 #define PHASE(i) do { if (c->time_phases) CU(cudaEventRecord(c->ph_ev[i], s)); } while (0)
   PHASE(0);
   // draft: catch up on a step the target wrote last time, then decode y^_i (rows that wait for the
@@ -1661,6 +1679,12 @@ int rsd_debug_fail_iteration(rsd_ctx* c, int32_t iteration) {
 int rsd_debug_sm_limit(rsd_ctx* c, int32_t sms) {
   if (!c || sms < 0) return RSD_ERR_ARG;
   c->sm_limit = sms;
+  return RSD_OK;
+}
+
+int rsd_debug_step_calls(rsd_ctx* c, int32_t n) {
+  if (!c || n < 0) return RSD_ERR_ARG;
+  c->as_sharers = n;
   return RSD_OK;
 }
 

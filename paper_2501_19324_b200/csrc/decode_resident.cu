@@ -54,6 +54,7 @@ constexpr int kMaxK = 2048;
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;       // a NaN that no conversion or sum gives
 constexpr uint32_t kPolls = 1u << 21;          // of L2, half a microsecond or more each
 constexpr int kOwn = 4;                        // units of the residual stream that a CTA owns at most
+constexpr int kSharers = 4;                    // callers that share the SMs at most; more take turns
 
 struct alignas(128) ResidentLayer {
   CUtensorMap w[4];                            // qkv, wo, gate/up, down
@@ -1430,14 +1431,18 @@ cudaError_t launch_as(const ResidentPlan& plan, const void* dev_block, int grid,
 }  // namespace
 
 cudaError_t launch_decode_resident(const ResidentPlan& plan, const void* dev_block, const ResidentShape& m, bool kv_extended, const RowState& st, int which,
-                                   int phase, int n_slots, const LoopParams& lp, int sm_limit, cudaStream_t s) {
+                                   int phase, int n_slots, const LoopParams& lp, int sharers, int sm_limit, cudaStream_t s) {
   if (n_slots < 1 || n_slots > kRows) return cudaErrorNotSupported;
   const int sms = device_sms();
   if (sms <= 0) return cudaErrorInvalidDevice;
-  if (grid_of(m, sms) > (sm_limit > 0 ? std::min(sm_limit, stream_sms(s)) : stream_sms(s))) return cudaErrorCooperativeLaunchTooLarge;
+  // A CTA takes the shared memory of its SM, so two phases of as many CTAs as there are SMs take turns.  Which CTA does a unit changes no bit: callers that
+  // run at the same time get a part of the chip each, down to a quarter.  us an iteration of all, 1 / 2 / 4 callers of four rows each, graphs / all SMs each / so: bf16,
+  // 2 x 512 columns 44 / 36 / 36, 50 / 70 / 49, 60 / 136 / 66, 3 x 768 65 / 59 / 59, 85 / 115 / 87, 92 / 228 / 131; fp32, 2 x 256 49 / 44 / 45, 65 / 82 / 53,
+  // 73 / 164 / 69, 4 x 512 107 / 93 / 98, 142 / 183 / 138, 215 / 363 / 186.  (Graphs remain ahead for four and more callers of bf16 models: six, 66 / 87, 98 / 178.)
+  const int grid = grid_of(m, sms / std::max(1, std::min(sharers, kSharers)));
+  if (grid > (sm_limit > 0 ? std::min(sm_limit, stream_sms(s)) : stream_sms(s))) return cudaErrorCooperativeLaunchTooLarge;
   const cudaError_t e = cudaMemsetAsync(reinterpret_cast<const ResidentParams*>(plan.bytes)->slots, 0xFF, resident_slot_bytes(m), s);
   if (e != cudaSuccess) return e;
-  const int grid = grid_of(m, sms);
   if (m.f32) return n_slots <= 4 ? launch_as<true, false, 4>(plan, dev_block, grid, st, which, phase, n_slots, lp, s)
                                  : launch_as<true, false, 8>(plan, dev_block, grid, st, which, phase, n_slots, lp, s);
   return kv_extended ? launch_as<false, true, 8>(plan, dev_block, grid, st, which, phase, n_slots, lp, s)

@@ -233,8 +233,9 @@ struct RowState;
 struct LoopParams;
 // Runs the decode phase that launch_decode_begin has opened, n_slots <= 8, to its end.  cudaErrorCooperativeLaunchTooLarge, and nothing done: the stream has
 // fewer SMs than the launch has CTAs, which wait for one another (it belongs to a part of the chip); sm_limit > 0: as if it had no more than these.
+// sharers: callers that may be running such launches at this time, this one too; the results do not depend on it.
 cudaError_t launch_decode_resident(const ResidentPlan& plan, const void* dev_block, const ResidentShape& m, bool kv_extended, const RowState& st, int which,
-                                   int phase, int n_slots, const LoopParams& lp, int sm_limit, cudaStream_t s);
+                                   int phase, int n_slots, const LoopParams& lp, int sharers, int sm_limit, cudaStream_t s);
 
 struct SampleArgs {
   const float* logits;         // [n_slots, V]

@@ -801,6 +801,32 @@ def test_decode_phases_in_one_launch_on_two_streams():
         e.close()
 
 
+@pytest.mark.parametrize("sh,bf16,rows", [(ri.ModelShape(2, 512, 4, 2, 128, 1408, 4096), True, 8), (ri.ModelShape(1, 2048, 8, 8, 128, 1088, 1030), True, 5),
+                                          (ri.ModelShape(4, 512, 8, 2, 64, 1376, 1024), False, 3), (ri.ModelShape(1, 2048, 32, 2, 64, 2048, 520), False, 8)],
+                         ids=["bf16", "bf16-wide", "fp32", "fp32-wide"])
+def test_decode_phases_in_one_launch_share_the_chip(sh, bf16, rows):
+    """Callers that run at the same time get a part of the SMs each, and each CTA more units: the same bits."""
+    from paper_2501_19324_b200 import Engine, Model, lib, RSD_DEBUG_KEEP_LOGITS
+    from paper_2501_19324_b200.binding import RSD_DEBUG_RESIDENT_LOGITS
+    heads = (ri.HEAD_LM, ri.HEAD_REWARD_SIGMOID, ri.HEAD_LM)
+    models = [Model(sh, ri.gpu_model_tensors(sh, slot, 0, bf16, hk), hk) for slot, hk in enumerate(heads)]
+    prompts = ri.prompts(8, rows, 5, 60, sh.vocab)
+    got = []
+    for n in (1, 2, 3, 4, 9):
+        eng = Engine(*models, max_batch=rows, max_seq_tokens=120, max_step_tokens=9, max_steps=3, step_end_id=1, step_end_mod=30,
+                     temperature=0.7, seed=2, debug_flags=RSD_DEBUG_KEEP_LOGITS | RSD_DEBUG_RESIDENT_LOGITS)
+        eng.prefill(*prompts)
+        assert lib().rsd_debug_step_calls(eng.ctx, n) == 0
+        seen = []
+        for delta, which in ((2.0, 2), (0.0, 0)):
+            r = eng.step(delta)
+            kept = eng.logits(which)
+            seen.append([v.tobytes() for v in r.values()] + [kept[b, :r["step_len"][b]].tobytes() for b in range(rows)])
+        got.append(seen)
+        eng.close()
+    assert all(g == got[0] for g in got)
+
+
 def _engine(prompts, **kw):
     from paper_2501_19324_b200 import Engine, Model
     heads = (ri.HEAD_LM, ri.HEAD_REWARD_SIGMOID, ri.HEAD_LM)
