@@ -1436,9 +1436,10 @@ cudaError_t launch_decode_resident(const ResidentPlan& plan, const void* dev_blo
   const int sms = device_sms();
   if (sms <= 0) return cudaErrorInvalidDevice;
   // A CTA takes the shared memory of its SM, so two phases of as many CTAs as there are SMs take turns.  Which CTA does a unit changes no bit: callers that
-  // run at the same time get a part of the chip each, down to a quarter.  us an iteration of all, 1 / 2 / 4 callers of four rows each, graphs / all SMs each / so: bf16,
-  // 2 x 512 columns 44 / 36 / 36, 50 / 70 / 49, 60 / 136 / 66, 3 x 768 65 / 59 / 59, 85 / 115 / 87, 92 / 228 / 131; fp32, 2 x 256 49 / 44 / 45, 65 / 82 / 53,
-  // 73 / 164 / 69, 4 x 512 107 / 93 / 98, 142 / 183 / 138, 215 / 363 / 186.  (Graphs remain ahead for four and more callers of bf16 models: six, 66 / 87, 98 / 178.)
+  // run at the same time get a part of the chip each, down to a quarter.  us an iteration of all, 1 / 2 / 4 callers of four rows each, steps of 24 tokens and all that
+  // is around them, graphs -> so (all SMs each, two / four): bf16, 2 x 512 columns 49 / 55 / 68 -> 41 / 52 / 66 (70 / 136), 3 x 768 72 / 92 / 100 -> 63 / 85 / 128
+  // (115 / 228), 8 x 1536 210 / 251 / 347 -> 188 / 287 / 409; fp32, 2 x 256 49 / 66 / 73 -> 43 / 47 / 62 (82 / 164), 4 x 512 99 / 132 / 198 -> 86 / 123 / 161 (183 / 363).
+  // Graphs remain ahead for many callers of wide bf16 models, and for six of any (2 x 512 74 -> 91).
   const int grid = grid_of(m, sms / std::max(1, std::min(sharers, kSharers)));
   if (grid > (sm_limit > 0 ? std::min(sm_limit, stream_sms(s)) : stream_sms(s))) return cudaErrorCooperativeLaunchTooLarge;
   const cudaError_t e = cudaMemsetAsync(reinterpret_cast<const ResidentParams*>(plan.bytes)->slots, 0xFF, resident_slot_bytes(m), s);

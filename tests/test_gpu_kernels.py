@@ -1027,6 +1027,28 @@ def test_head_that_samples_scales_its_rows():
         assert (got == want).float().mean() > 0.9
 
 
+@pytest.mark.parametrize("chunks", [1, 3, 50, 129])
+@pytest.mark.parametrize("M", [5, 16, 33, 128])
+def test_head_that_samples_scales_its_rows_by_exact_denominators(M, chunks):
+    """Sums of squares that are exact in any order and add up to a power of four a column: the denominators are powers of two, and so the scores, and the
+    ids with them, are those of the scaled logits.  Chunks that the lanes of a row, 2 to 32 of them, do not share evenly."""
+    gen = torch.Generator(device="cuda").manual_seed(M + chunks)
+    N, K = 5000, 512
+    W = torch.randn(N, K, generator=gen, device="cuda").mul_(0.05).to(torch.bfloat16)
+    x = torch.randn(M, K, generator=gen, device="cuda")
+    hi = x.to(torch.bfloat16)
+    lo = (x - hi.float()).to(torch.bfloat16)
+    idx = torch.arange(M, device="cuda", dtype=torch.int32)
+    logits = rb.k_gemm(W, hi, x_lo=lo, impl=3)
+    power = torch.randint(-2, 3, (M,), generator=gen, device="cuda").float()
+    shares = torch.rand(M, chunks, generator=gen, device="cuda").mul_(900 / chunks).floor() + 1          # of 1024
+    shares[:, chunks // 2] += 1024 - shares.sum(1)
+    ssq = shares * (K / 1024) * torch.pow(4.0, power)[:, None]
+    want = rb.k_sample(logits * torch.pow(2.0, -power)[:, None], N, 0.7, 5, 0, idx, idx)
+    got = rb.k_head_sample(W, hi, lo, N, 0.7, 5, 0, idx, idx, ssq=ssq.contiguous(), eps=0.0)
+    assert torch.equal(got, want)
+
+
 def test_bounded_wait_runs_out_and_the_kernel_leaves_cleanly():
     """RSD_ERR_TIMEOUT without a fault: one CTA of the tensor-core GEMM whose copies are never issued.  Its wait
     (a few thousand polls in this mode) expires, the error flag is raised and reported, tensor memory is freed: the

@@ -857,6 +857,69 @@ def test_a_failing_decode_phase_ends_early():
     eng.close()
 
 
+def test_a_failing_decode_phase_of_single_kernels_ends_early():
+    """The same where the iterations are launched one by one (small models do that when logits are kept): the host follows the phase and launches a few
+    iterations more, not all 64."""
+    from paper_2501_19324_b200 import RSD_DEBUG_KEEP_LOGITS
+    from paper_2501_19324_b200.binding import RsdError, lib
+    prompts = ri.prompts(1, 3, 10, 20, MINI[0].vocab)
+    eng = _engine(prompts, max_seq_tokens=160, max_step_tokens=64, max_steps=3, step_end_id=-1, temperature=0.7, seed=1, debug_flags=RSD_DEBUG_KEEP_LOGITS)
+    before = lib().rsd_debug_launch_count()
+    eng.step(0.0)
+    whole = lib().rsd_debug_launch_count() - before
+    assert whole > 64 * 8
+    assert lib().rsd_debug_fail_iteration(eng.ctx, 3) == 0
+    before = lib().rsd_debug_launch_count()
+    with pytest.raises(RsdError) as e:
+        eng.step(0.0)
+    assert e.value.code == -5
+    assert lib().rsd_debug_launch_count() - before < whole / 4
+    with pytest.raises(RsdError) as e:
+        eng.step(0.0)
+    assert e.value.code == -2
+    eng.close()
+
+
+def test_a_failing_decode_phase_in_one_launch_ends_early():
+    """... and where the phase is one launch: the flag is up ahead of it, and it leaves with the first iteration, whose successors sample nothing."""
+    from paper_2501_19324_b200.binding import RsdError, lib
+    prompts = ri.prompts(1, 3, 10, 20, MINI[0].vocab)
+    eng = _engine(prompts, max_seq_tokens=160, max_step_tokens=64, max_steps=3, step_end_id=-1, temperature=0.7, seed=1)
+    before = lib().rsd_debug_launch_count()
+    eng.step(0.0)
+    assert lib().rsd_debug_launch_count() - before < 64 * 2
+    assert (eng.sampled(0) != 0).mean() > 0.9
+    assert lib().rsd_debug_fail_iteration(eng.ctx, 3) == 0
+    with pytest.raises(RsdError) as e:
+        eng.step(0.0)
+    assert e.value.code == -5
+    assert (eng.sampled(0)[:, 1:] == 0).all()
+    with pytest.raises(RsdError) as e:
+        eng.step(0.0)
+    assert e.value.code == -2
+    eng.close()
+
+
+@pytest.mark.parametrize("temperature", [0.0, 0.2, 0.7])
+def test_speculative_rounds_that_sample_in_the_head(temperature):
+    """From 65536 ids on proposals and the pass that verifies them sample in the head's epilogue, unless the target's logits are kept: the same tokens."""
+    from paper_2501_19324_b200 import Engine, Model, RSD_DEBUG_KEEP_LOGITS
+    sh = ri.ModelShape(2, 256, 2, 1, 128, 704, 65540)
+    heads = (ri.HEAD_LM, ri.HEAD_REWARD_SIGMOID, ri.HEAD_LM)
+    models = [Model(sh, ri.gpu_model_tensors(sh, slot, 0, True, hk), hk) for slot, hk in enumerate(heads)]
+    prompts = ri.prompts(9, 6, 5, 40, sh.vocab)
+    got = []
+    for flags in (0, RSD_DEBUG_KEEP_LOGITS):
+        eng = Engine(*models, max_batch=6, max_seq_tokens=100, max_step_tokens=12, max_steps=4, step_end_id=1, step_end_mod=20, temperature=temperature,
+                     seed=2, sd_tokens=4, debug_flags=flags)
+        eng.prefill(*prompts)
+        steps = [eng.step(delta) for delta in (2.0, 0.0, 2.0)]
+        got.append(([r["step_tokens"].tolist() for r in steps], eng.counters()))
+        eng.close()
+    assert got[0] == got[1]
+    assert got[0][1]["sd_rounds"] > 0
+
+
 def test_a_phase_without_rows_does_not_wait_for_the_stream():
     """No row has room for a step: the call returns although another thread keeps the caller's stream busy (for three seconds
     at most), since the phase says itself that it has nothing to decode."""
