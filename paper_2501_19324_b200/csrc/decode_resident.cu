@@ -225,12 +225,6 @@ __device__ __forceinline__ uint32_t attn_word(int f, int m) {               // b
 
 __device__ __forceinline__ float gumbel(uint32_t bits) { return -logf(-logf(uniform_from_bits(bits))); }
 
-__device__ __forceinline__ bool step_ends(int t, const LoopParams& lp) {
-  if (lp.eos_id >= 0 && t == lp.eos_id) return true;
-  if (lp.step_end_mod > 0) return (t % lp.step_end_mod) == (lp.step_end_id % lp.step_end_mod);
-  return t == lp.step_end_id;
-}
-
 // Shared memory behind the ring.
 template <bool F32, bool EXT> struct ResidentCfg {
   static constexpr int kPageBytes = (EXT ? 4 : 2) * kPageTokens * 128 * 2;
@@ -1229,7 +1223,7 @@ decode_resident_kernel(const __grid_constant__ ResidentParams P, const ResidentL
           sampled = top ? (int)(0xFFFFFFFFu - (uint32_t)(top & 0xFFFFFFFFull)) : 0;
           const int flen = s_flen[m];
           const int tk = flen > 0 ? st.forced_tok[phase][(size_t)s_row[m] * st.C + iter] : sampled;
-          ends = step_ends(tk, lp) || iter + 1 == st.C || (flen > 0 && iter + 1 == flen);
+          ends = ends_step(tk, lp) || iter + 1 == st.C || (flen > 0 && iter + 1 == flen);
           s_tok[m] = tk;
           s_pos[m] += 1;
         }

@@ -315,6 +315,12 @@ struct LoopParams {
   float omega_alpha;
   uint64_t seed;
 };
+// Whether token t ends its step.
+inline __device__ bool ends_step(int t, const LoopParams& lp) {
+  if (lp.eos_id >= 0 && t == lp.eos_id) return true;
+  if (lp.step_end_mod > 0) return (t % lp.step_end_mod) == (lp.step_end_id % lp.step_end_mod);
+  return t == lp.step_end_id;
+}
 
 // min_target_rows: the target serves the waiting rows only once that many wait, or every live row does
 // (target_pass_due); it matters to the target modes alone.

@@ -196,12 +196,6 @@ cudaError_t launch_score_prepare(const RowState& st, cudaStream_t s) {
   return launched(1);
 }
 
-__device__ __forceinline__ bool ends_step(int t, const LoopParams& lp) {
-  if (lp.eos_id >= 0 && t == lp.eos_id) return true;
-  if (lp.step_end_mod > 0) return (t % lp.step_end_mod) == (lp.step_end_id % lp.step_end_mod);
-  return t == lp.step_end_id;
-}
-
 // Appends the current iteration's token of every active slot to its row, stops rows whose step ended and lays out the next iteration.
 __global__ void __launch_bounds__(1024)
 decode_update_kernel(RowState st, int which, int phase, unsigned long long* best, int n_slots, LoopParams lp) {
