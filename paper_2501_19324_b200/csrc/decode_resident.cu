@@ -4,8 +4,8 @@
 // A model of a few dozen MB takes an iteration of 15 to 25 dependent steps, each of which is over in a microsecond once its input is
 // there.  As kernels they cost 2 to 5 us each, whatever they do (launch, wait, first loads, drain); here they are phases of
 // one cooperative launch, a CTA per SM, and a phase costs the way of its input through L2 and a few hundred instructions.  An iteration, us, kernels of
-// a graph / here: bf16, 2 x 512 and 3 x 768 columns, 8 rows 42 / 31 and 66 / 52, 1 row 39 / 29 and 55 / 50; fp32, 2 x 256 and 4 x 512 columns,
-// 4 rows 37 / 27 and 81 / 64, 8 rows 55 / 36 and 121 / 88; a phase has 10 us more to start.
+// a graph / here: bf16, 2 x 512 and 3 x 768 columns, 8 rows 42 / 32 and 67 / 54, 1 row 39 / 31 and 57 / 52; fp32, 2 x 256 and 4 x 512 columns,
+// 4 rows 37 / 29 and 85 / 66, 8 rows 55 / 38 and 124 / 93; a phase has 10 us more to start.
 //   weights    the CTA's weight rows of all phases, layers and iterations, in order, come by TMA into a ring of 16 KB stages, requested as soon as
 //              the stages are free.  Weights depend on nothing, so they are in shared memory before the phase that needs them.
 //   exchange   there is no barrier between phases.  A result goes to L2 as words that can never be kEmpty, into slots that are kEmpty

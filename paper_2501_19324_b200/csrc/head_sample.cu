@@ -3,13 +3,13 @@
 //
 // As two launches the head was one tile of 128 ids a CTA and the sampling read the logits back: in the step loop 151936 ids of 3584 columns took
 // 154-201 us at 8 to 64 rows for a weight stream of 149, of 1536 columns 67-115 at 8 to 128 for 64, and the sampling 11 us at 20 rows, 15-19 at 32 to
-// 40, 48 at 128.  Here both take 168-182 us at 16 to 64 rows, and 71 at 16, 79 at 40, 126 at 128.
+// 40, 48 at 128.  Here both take 168-185 us at 16 to 64 rows, and 71 at 16, 80 at 40, 128 at 128.
 //   - 1187 tiles are 8.02 for each of 148 SMs (4.01 rounds of two): the last round is nearly empty.  Here a CTA per SM walks the same number
 //     of whole tiles as every other and then one smaller tile, whose rows are the remainder shared out by sixteens.
 //   - Two tiles of 128 ids are multiplied at once with the same x tile (up to 64 rows): from 16 rows on the copies of x are what the head waits for,
 //     64 rows of 3584 columns are 0.92 MB a tile, as many bytes in all as the weights.
 //   - The ring runs on from tile to tile and the accumulators alternate, so the sampling of a tile runs beside the products of the next.
-// The sampling is sample_kernel's, exactly: ids whose logits cannot win against the best so far draw no noise, the others a quick one first, and only
+// The ids are sample_kernel's: ids whose logits cannot win against the best so far draw no noise, the others a quick one first, and only
 // what comes near the best an exact one.  A thread holds one id of sixteen rows; the four words of a Philox block belong to four neighbouring
 // ids, so four lanes take a block each of four rows and swap words.
 // What bounds it: the weights up to 64 rows; at 128 the copies of x (a tile at a time, 0.79 MB each of 1536 columns) and the noise beside them.
