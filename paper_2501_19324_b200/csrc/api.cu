@@ -1266,6 +1266,7 @@ int rsd_load_models(rsd_ctx* c, const rsd_model* draft, const rsd_model* prm, co
     c->st.pool_pages[w] = pages;
   }
   c->v_limit = std::min(std::min(draft->vocab, prm->vocab), target->vocab);
+  c->z_host.assign(c->B_max, 0);
   cudaStream_t s = 0;
   for (int w = 0; w < 3; ++w)
     CU(launch_rope_table(c->mdl[w].rope, c->S, c->mdl[w].m.head_dim, c->mdl[w].m.rope_theta, s));
@@ -1336,7 +1337,6 @@ int rsd_prefill(rsd_ctx* c, const int32_t* tokens, const int32_t* offsets, int32
   int rc = rsd_reset(c);
   if (rc) return rc;
   c->st.B = B;
-  c->z_host.resize(B);
   c->z_max = 0;
   for (int b = 0; b < B; ++b) c->z_max = std::max(c->z_max, c->z_host[b] = offsets[b + 1] - offsets[b]);
   // stage the ragged prompt in the pass-list buffers, then scatter it into the row buffers

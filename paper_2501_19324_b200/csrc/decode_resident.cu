@@ -30,9 +30,9 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <memory>
 #include <new>
 #include <type_traits>
-#include <vector>
 
 #include "common.cuh"
 #include "kernels.cuh"
@@ -1376,8 +1376,9 @@ cudaError_t resident_build(ResidentPlan* plan, void* dev_block, const ResidentBu
   int dev = 0, cooperative = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&cooperative, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !cooperative) return cudaErrorNotSupported;
   if (!resident_supported(m) || grid < 1 || (m.d / 16 + grid - 1) / grid > kOwn || (m.f32 && ((uintptr_t)a.kv_pool & 15))) return cudaErrorNotSupported;
-  std::vector<uint8_t> host(resident_block_bytes(m.n_layers) + 128);
-  uint8_t* hb = (uint8_t*)(((uintptr_t)host.data() + 127) & ~(uintptr_t)127);
+  const std::unique_ptr<uint8_t[]> host(new (std::nothrow) uint8_t[resident_block_bytes(m.n_layers) + 128]);
+  if (!host) return cudaErrorMemoryAllocation;
+  uint8_t* hb = (uint8_t*)(((uintptr_t)host.get() + 127) & ~(uintptr_t)127);
   ResidentParams* P = new (plan->bytes) ResidentParams();
   ResidentLayer* Ls = reinterpret_cast<ResidentLayer*>(hb);
   const int hq = m.H * m.hd, nq = (m.H + 2 * m.KV) * m.hd;
@@ -1398,7 +1399,7 @@ cudaError_t resident_build(ResidentPlan* plan, void* dev_block, const ResidentBu
   }
   const cudaError_t e = cudaMemcpyAsync(dev_block, hb, resident_block_bytes(m.n_layers), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
-  return cudaStreamSynchronize(s);             // the staging vector goes away
+  return cudaStreamSynchronize(s);             // the staging block goes away
 }
 
 namespace {
