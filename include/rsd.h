@@ -175,7 +175,10 @@ int rsd_prefill(rsd_ctx*, const int32_t* tokens, const int32_t* offsets, int32_t
 /* rsd_step(delta): one pass of the loop body of Algorithm 1 over all rows.  Outputs are HOST
  * arrays (any may be NULL): step_tokens [B, max_step_tokens] (y_i, zero padded), step_len [B],
  * rewards [B] (r_i of the draft step), accept [B] (1 = draft step kept), live [B] (row continues).
- * Rows that were already stopped report step_len 0, reward 0, accept 0.  Synchronises.       */
+ * Rows that were already stopped report step_len 0, reward 0, accept 0.  Synchronises.
+ * Decode phases of small models over up to eight rows are one cooperative launch that holds the shared memory of its SMs
+ * until the phase ends.  Step calls that run at the same time on a device (a context and a stream each) get a part of the
+ * SMs each; on a stream with fewer SMs than the launch needs (a green context's) the phase runs kernel by kernel.  */
 int rsd_step(rsd_ctx*, float delta, void* cuda_stream, int32_t* step_tokens, int32_t* step_len,
              float* rewards, uint8_t* accept, uint8_t* live);
 

@@ -801,6 +801,40 @@ def test_decode_phases_in_one_launch_on_two_streams():
         e.close()
 
 
+def test_decode_phases_on_a_part_of_the_chip():
+    """A stream of a green context with 40 SMs: its phases run kernel by kernel, the default stream's in one launch."""
+    import torch
+    from paper_2501_19324_b200 import lib, RSD_DEBUG_KEEP_LOGITS
+    from paper_2501_19324_b200.binding import RSD_DEBUG_RESIDENT_LOGITS
+    drv = pytest.importorskip("cuda.bindings.driver")
+
+    def ok(r):
+        assert int(r[0]) == 0, r
+        return r[1]
+    sm = drv.CUdevResourceType.CU_DEV_RESOURCE_TYPE_SM
+    sh = MINI[0]
+    prompts = ri.prompts(12, 3, 10, 40, sh.vocab)
+    kw = dict(max_step_tokens=12, max_steps=4, max_seq_tokens=100, step_end_id=2, step_end_mod=50, temperature=0.7, seed=6)
+    eng, loop = build_pair((sh, sh, sh), bf16=True, prompts=prompts, loop_kwargs=kw,
+                           engine_kwargs=dict(debug_flags=RSD_DEBUG_KEEP_LOGITS | RSD_DEBUG_RESIDENT_LOGITS))
+    dev = ok(drv.cuDeviceGet(torch.cuda.current_device()))
+    part = ok(drv.cuDevSmResourceSplitByCount(1, ok(drv.cuDeviceGetDevResource(dev, sm)), 0, 40))[0]
+    green = ok(drv.cuGreenCtxCreate(ok(drv.cuDevResourceGenerateDesc([part], 1)), dev, drv.CUgreenCtxCreate_flags.CU_GREEN_CTX_DEFAULT_STREAM))
+    stream = ok(drv.cuGreenCtxStreamCreate(green, drv.CUstream_flags.CU_STREAM_NON_BLOCKING, 0))
+    launches = []
+    for st in (torch.cuda.current_stream(), torch.cuda.ExternalStream(int(stream)), torch.cuda.current_stream()):
+        torch.cuda.synchronize()
+        before = lib().rsd_debug_launch_count()
+        with torch.cuda.stream(st):
+            parity_step(eng, loop, 2.0, **TOL16)
+        launches.append(lib().rsd_debug_launch_count() - before)
+    torch.cuda.synchronize()
+    assert launches[1] > 2 * max(launches[0], launches[2])
+    eng.close()
+    ok((drv.cuStreamDestroy(stream)[0], None))
+    ok((drv.cuGreenCtxDestroy(green)[0], None))
+
+
 @pytest.mark.parametrize("sh,bf16,rows", [(ri.ModelShape(2, 512, 4, 2, 128, 1408, 4096), True, 8), (ri.ModelShape(1, 2048, 8, 8, 128, 1088, 1030), True, 5),
                                           (ri.ModelShape(4, 512, 8, 2, 64, 1376, 1024), False, 3), (ri.ModelShape(1, 2048, 32, 2, 64, 2048, 520), False, 8)],
                          ids=["bf16", "bf16-wide", "fp32", "fp32-wide"])
