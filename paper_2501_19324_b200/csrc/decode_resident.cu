@@ -1435,7 +1435,8 @@ cudaError_t launch_decode_resident(const ResidentPlan& plan, const void* dev_blo
   // is around them, graphs -> so (all SMs each, two / four): bf16, 2 x 512 columns 49 / 55 / 68 -> 41 / 52 / 66 (70 / 136), 3 x 768 72 / 92 / 100 -> 63 / 85 / 128
   // (115 / 228), 8 x 1536 210 / 251 / 347 -> 188 / 287 / 409; fp32, 2 x 256 49 / 66 / 73 -> 43 / 47 / 62 (82 / 164), 4 x 512 99 / 132 / 198 -> 86 / 123 / 161 (183 / 363).
   // Graphs remain ahead for many callers of wide bf16 models, and for six of any (2 x 512 74 -> 91).
-  const int grid = grid_of(m, sms / std::max(1, std::min(sharers, kSharers)));
+  // (Never fewer CTAs than own the residual stream's units, kOwn each: the full grid has as many.)
+  const int grid = std::max(grid_of(m, sms / std::max(1, std::min(sharers, kSharers))), (m.d / 16 + kOwn - 1) / kOwn);
   if (grid > (sm_limit > 0 ? std::min(sm_limit, stream_sms(s)) : stream_sms(s))) return cudaErrorCooperativeLaunchTooLarge;
   const cudaError_t e = cudaMemsetAsync(reinterpret_cast<const ResidentParams*>(plan.bytes)->slots, 0xFF, resident_slot_bytes(m), s);
   if (e != cudaSuccess) return e;
